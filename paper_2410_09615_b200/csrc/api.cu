@@ -30,11 +30,6 @@ const DeviceInfo* device_info(slim_status_t* err) {
             if (cudaGetDeviceProperties(&prop, dev) != cudaSuccess) { *err = SLIM_ERR_CUDA; return nullptr; }
             di.cc_major = prop.major;
             di.sm_count = prop.multiProcessorCount;
-            if (prop.major == 10) {
-                di.decode_ctas_per_sm[0] = decode_query_residency(1);
-                di.decode_ctas_per_sm[1] = decode_query_residency(2);
-                di.decode_tiled_ok = decode_tiled_query_residency();
-            }
             g_info_ready[dev].store(true, std::memory_order_release);
         }
     }
@@ -65,22 +60,31 @@ static slim_status_t check_weight_shape(int d_out, int d_in) {
     return SLIM_OK;
 }
 
+// Small ragged problems (rows of d_in / 8 index bytes or 128-row tiles that do not come out even, less than one
+// 256-row tile and few multiply-adds) would occupy one cluster: the CUDA-core kernel spreads them.
+static bool small_and_ragged(int b, int d_out, int d_in) {
+    return (d_in % 128 != 0 || (d_out % 128 != 0 && b > 16)) && d_out < 256 && (long long)b * d_out * d_in < (1 << 24);
+}
+
+// The small-batch kernel's problems: one launch, up to 64 tokens.
+static bool runs_small(int b, int d_out, int d_in, int r) {
+    return small_supports(b, d_out, d_in, r) && !small_and_ragged(b, d_out, d_in);
+}
+
 static slim_kernel_t select_kernel(int b, int d_out, int d_in, int r) {
-    if (b <= 16 && decode_supports(b, d_out, d_in, r)) return SLIM_KERNEL_DECODE;
-    if (b > 16 && prefill_supports(b, d_out, d_in, r)) return SLIM_KERNEL_PREFILL;
+    if (b <= 16 && runs_small(b, d_out, d_in, r)) return SLIM_KERNEL_DECODE;
+    if (b > 16 && (runs_small(b, d_out, d_in, r) || prefill_supports(b, d_out, d_in, r))) return SLIM_KERNEL_PREFILL;
     return SLIM_KERNEL_SIMPLE;
 }
 
+// Sync words, then the region the small-batch kernel publishes T in (entries carry call numbers, so nothing else is
+// ever written there), then the other kernels' scratch.
 static size_t workspace_bytes(int b, int d_out, int d_in, int r) {
     size_t need = simple_workspace_bytes(b, d_out, d_in, r);
-    const size_t d = decode_workspace_bytes(b, d_out, d_in, r);
-    if (d > need) need = d;
     const size_t pf = prefill_workspace_bytes(b, d_out, d_in, r);
     if (pf > need) need = pf;
-    const size_t dt = b <= 16 ? decode_tiled_workspace_bytes(b, d_out, d_in, r) : 0;
-    if (dt > need) need = dt;
     need = (need + 255) / 256 * 256;
-    return SLIM_WORKSPACE_SYNC_BYTES + need;
+    return SLIM_WORKSPACE_SYNC_BYTES + kSmallTBytes + need;
 }
 
 }  // namespace slim
@@ -122,9 +126,9 @@ slim_status_t slim_workspace_reset(void* workspace, size_t workspace_bytes_, voi
 {
     if (!workspace || workspace_bytes_ < SLIM_WORKSPACE_SYNC_BYTES) return SLIM_ERR_WORKSPACE;
     cudaStream_t st = (cudaStream_t)cuda_stream;
-    // hand-over slots start "empty" (all-ones), the call counter at zero
-    if (cudaMemsetAsync(workspace, 0xFF, workspace_bytes_, st) != cudaSuccess) return SLIM_ERR_CUDA;
-    return cudaMemsetAsync(workspace, 0, SLIM_WORKSPACE_SYNC_BYTES, st) == cudaSuccess ? SLIM_OK : SLIM_ERR_CUDA;
+    // the call counter and the call numbers of T's entries start at zero (the first call is number one)
+    const size_t n = SLIM_WORKSPACE_SYNC_BYTES + kSmallTBytes;
+    return cudaMemsetAsync(workspace, 0, workspace_bytes_ < n ? workspace_bytes_ : n, st) == cudaSuccess ? SLIM_OK : SLIM_ERR_CUDA;
 }
 
 int slim_decode_layout_hint(int b, int d_out, int d_in, int r)
@@ -132,8 +136,7 @@ int slim_decode_layout_hint(int b, int d_out, int d_in, int r)
     if (b < 1 || b > (d_out >= d_in ? 4 : 2) || r < 0 || r % 16 != 0 || check_weight_shape(d_out, d_in) != SLIM_OK) return 0;
     if ((size_t)d_out * (size_t)d_in * 3 / 8 < ((size_t)64 << 20)) return 0;
     slim_status_t err;
-    const DeviceInfo* di = device_info(&err);
-    if (!di || !di->decode_tiled_ok || !decode_tiled_supports(b, d_out, d_in, r)) return 0;
+    if (!device_info(&err) || !small_supports(b, d_out, d_in, r) || slim_tiled_bytes(d_out, d_in, SLIM_LAYOUT_DECODE_TILED) == 0) return 0;
     return SLIM_LAYOUT_DECODE_TILED;
 }
 
@@ -161,7 +164,8 @@ slim_status_t slim_linear_fwd_ex(const void* X, int b, const uint8_t* vals, cons
     if (!workspace || workspace_bytes_ < workspace_bytes(b, d_out, d_in, r)) return SLIM_ERR_WORKSPACE;
     slim_status_t derr;
     if (!device_info(&derr)) return derr;
-    if (kernel == SLIM_KERNEL_AUTO) kernel = select_kernel(b, d_out, d_in, r);
+    const bool automatic = kernel == SLIM_KERNEL_AUTO;
+    if (automatic) kernel = select_kernel(b, d_out, d_in, r);
     const __nv_bfloat16* Xb = static_cast<const __nv_bfloat16*>(X);
     const __nv_bfloat16* Lb = static_cast<const __nv_bfloat16*>(L);
     const __nv_bfloat16* Rb = static_cast<const __nv_bfloat16*>(R);
@@ -171,9 +175,11 @@ slim_status_t slim_linear_fwd_ex(const void* X, int b, const uint8_t* vals, cons
     case SLIM_KERNEL_SIMPLE:
         return launch_simple(Xb, b, vals, meta, s, Lb, Rb, r, d_out, d_in, Yb, workspace, stream);
     case SLIM_KERNEL_DECODE:
-        if (b > 16 || !decode_supports(b, d_out, d_in, r)) return SLIM_ERR_UNSUPPORTED_SHAPE;
-        return launch_decode(Xb, b, vals, meta, s, Lb, Rb, r, d_out, d_in, Yb, workspace, status_dev, stream);
+        if (b > 16) return SLIM_ERR_UNSUPPORTED_SHAPE;
+        return launch_small(Xb, b, vals, meta, nullptr, s, Lb, Rb, nullptr, nullptr, r, d_out, d_in, Yb, workspace, status_dev, stream);
     case SLIM_KERNEL_PREFILL:
+        if (automatic && runs_small(b, d_out, d_in, r))            // up to 64 tokens: the small-batch kernel
+            return launch_small(Xb, b, vals, meta, nullptr, s, Lb, Rb, nullptr, nullptr, r, d_out, d_in, Yb, workspace, status_dev, stream);
         if (!prefill_supports(b, d_out, d_in, r)) return SLIM_ERR_UNSUPPORTED_SHAPE;
         return launch_prefill(Xb, b, vals, meta, s, Lb, Rb, r, d_out, d_in, Yb, workspace, status_dev, stream);
     case SLIM_KERNEL_PREFILL_PAIR:
@@ -270,16 +276,15 @@ slim_status_t slim_linear_fwd_q(const void* X, int b, const uint8_t* vals, const
     if (!workspace || workspace_bytes_ < need) return SLIM_ERR_WORKSPACE;
     const size_t base = align256(slim_workspace_bytes(b, d_out, d_in, r));
     cudaStream_t st = (cudaStream_t)cuda_stream;
-    // small batches: the decode kernel reads the codes and scales as they are
-    if (b <= 16 && decode_supports_q(b, d_out, d_in, r)) {
+    // small batches: the kernel reads the codes and scales as they are
+    if (runs_small(b, d_out, d_in, r)) {
         if (!X || !vals || !meta || !Y || !std::isfinite(s)) return SLIM_ERR_INVALID_ARG;
         if (!aligned16(X) || !aligned16(vals) || !aligned16(meta) || !aligned16(Y)) return SLIM_ERR_INVALID_ARG;
         if (status_dev && (reinterpret_cast<uintptr_t>(status_dev) & 3u)) return SLIM_ERR_INVALID_ARG;
         slim_status_t derr;
         if (!device_info(&derr)) return derr;
-        return launch_decode_q(static_cast<const __nv_bfloat16*>(X), b, vals, meta, s, Lq, static_cast<const __nv_bfloat16*>(Ls), Rq,
-                               static_cast<const __nv_bfloat16*>(Rs), r, d_out, d_in, static_cast<__nv_bfloat16*>(Y), workspace,
-                               status_dev, st);
+        return launch_small(static_cast<const __nv_bfloat16*>(X), b, vals, meta, nullptr, s, Lq, Rq, static_cast<const __nv_bfloat16*>(Ls),
+                            static_cast<const __nv_bfloat16*>(Rs), r, d_out, d_in, static_cast<__nv_bfloat16*>(Y), workspace, status_dev, st);
     }
     char* w = static_cast<char*>(workspace);
     __nv_bfloat16* Ld = reinterpret_cast<__nv_bfloat16*>(w + base);
@@ -323,11 +328,10 @@ slim_status_t slim_linear_fwd_tiled(const void* X, int b, const void* tiled, int
     if (status_dev && (reinterpret_cast<uintptr_t>(status_dev) & 3u)) return SLIM_ERR_INVALID_ARG;
     slim_status_t derr;
     if (!device_info(&derr)) return derr;
-    if (!decode_tiled_supports(b, d_out, d_in, r)) return SLIM_ERR_UNSUPPORTED_SHAPE;
+    if (!small_supports(b, d_out, d_in, r)) return SLIM_ERR_UNSUPPORTED_SHAPE;
     if (!workspace || workspace_bytes_ < workspace_bytes(b, d_out, d_in, r)) return SLIM_ERR_WORKSPACE;
-    return launch_decode_tiled(static_cast<const __nv_bfloat16*>(X), b, static_cast<const uint8_t*>(tiled), s,
-                               static_cast<const __nv_bfloat16*>(L), static_cast<const __nv_bfloat16*>(R), r, d_out, d_in,
-                               static_cast<__nv_bfloat16*>(Y), workspace, status_dev, (cudaStream_t)cuda_stream);
+    return launch_small(static_cast<const __nv_bfloat16*>(X), b, nullptr, nullptr, static_cast<const uint8_t*>(tiled), s, L, R, nullptr,
+                        nullptr, r, d_out, d_in, static_cast<__nv_bfloat16*>(Y), workspace, status_dev, (cudaStream_t)cuda_stream);
 }
 
 slim_status_t slim_linear_fwd_tiled_host(const void* X_host, int b, const void* tiled, int layout_id, float s,

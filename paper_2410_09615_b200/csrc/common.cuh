@@ -18,8 +18,6 @@ __host__ __device__ __forceinline__ int ceil_div(int a, int b) { return (a + b -
 struct DeviceInfo {
     int cc_major;
     int sm_count;
-    int decode_ctas_per_sm[2];   // cooperative residency of the decode kernel, NT = 1, 2
-    int decode_tiled_ok;         // every variant of the tiled decode kernel can be resident once per SM
 };
 const DeviceInfo* device_info(slim_status_t* err);
 
@@ -27,9 +25,11 @@ const DeviceInfo* device_info(slim_status_t* err);
 // nullptr when the driver does not have it.  Thread-safe.
 void* tensor_map_encoder();
 
-// The decode kernels keep the published T = X R^T at the start of the workspace, in a region of
-// this fixed size, so that calls of different shapes and kernels never read one kind of slot as another.
-constexpr size_t kDecodeTfinalBytes = 198656;
+// The small-batch kernel publishes T = X R^T in a region of this fixed size right after the sync words, whatever
+// the problem, and nothing else is kept there: calls of different shapes on one workspace never read one kind of
+// word as another.
+constexpr size_t kSmallTBytes = 512 << 10;
+constexpr int kSmallMaxRank = 3072;
 
 // Launch bookkeeping for slim_last_launch_count().
 void count_launch(int n);
@@ -47,24 +47,12 @@ slim_status_t launch_simple(const __nv_bfloat16* X, int b, const uint8_t* vals, 
                             float s, const __nv_bfloat16* L, const __nv_bfloat16* R, int r,
                             int d_out, int d_in, __nv_bfloat16* Y, void* ws, cudaStream_t st);
 
-bool decode_supports(int b, int d_out, int d_in, int r);
-size_t decode_workspace_bytes(int b, int d_out, int d_in, int r);
-slim_status_t launch_decode(const __nv_bfloat16* X, int b, const uint8_t* vals, const uint8_t* meta,
-                            float s, const __nv_bfloat16* L, const __nv_bfloat16* R, int r,
-                            int d_out, int d_in, __nv_bfloat16* Y, void* ws, uint32_t* status_dev,
-                            cudaStream_t st);
-bool decode_supports_q(int b, int d_out, int d_in, int r);
-slim_status_t launch_decode_q(const __nv_bfloat16* X, int b, const uint8_t* vals, const uint8_t* meta, float s,
-                              const uint8_t* Lq, const __nv_bfloat16* Ls, const uint8_t* Rq, const __nv_bfloat16* Rs, int r,
-                              int d_out, int d_in, __nv_bfloat16* Y, void* ws, uint32_t* status_dev, cudaStream_t st);
-int decode_query_residency(int nt);
-
-bool decode_tiled_supports(int b, int d_out, int d_in, int r);
-size_t decode_tiled_workspace_bytes(int b, int d_out, int d_in, int r);
-slim_status_t launch_decode_tiled(const __nv_bfloat16* X, int b, const uint8_t* W, float s, const __nv_bfloat16* L,
-                                  const __nv_bfloat16* R, int r, int d_out, int d_in, __nv_bfloat16* Y, void* ws,
-                                  uint32_t* status_dev, cudaStream_t st);
-int decode_tiled_query_residency();
+// Up to 64 tokens.  `tiled` (decode-tiled copy, up to 16 tokens) or vals / meta; Ls == nullptr: L and R are bf16
+// matrices, else the code bytes of quantized adapters.
+bool small_supports(int b, int d_out, int d_in, int r);
+slim_status_t launch_small(const __nv_bfloat16* X, int b, const uint8_t* vals, const uint8_t* meta, const uint8_t* tiled, float s,
+                           const void* L, const void* R, const __nv_bfloat16* Ls, const __nv_bfloat16* Rs, int r, int d_out, int d_in,
+                           __nv_bfloat16* Y, void* ws, uint32_t* status_dev, cudaStream_t st);
 
 slim_status_t launch_repack_tiled(const uint8_t* vals, const uint8_t* meta, int d_out, int d_in, uint8_t* out, cudaStream_t st);
 

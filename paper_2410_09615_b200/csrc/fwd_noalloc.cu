@@ -1,13 +1,13 @@
 // slim_linear_fwd_noalloc: the small-batch forward for callers that may not
 // allocate device memory.  Its scratch lives in this file's static device
-// array; everything else is the ordinary decode kernel.
+// array; everything else is the ordinary small-batch kernel.
 #include <mutex>
 #include "common.cuh"
 
 namespace slim {
 
-// Scratch shared by every call of slim_linear_fwd_noalloc on a device: split-K
-// partial slots plus, in its first SLIM_WORKSPACE_SYNC_BYTES, the call counter.  Each GPU that loads the library carries one copy until exit.
+// Scratch shared by every call of slim_linear_fwd_noalloc on a device: the call counter in its first
+// SLIM_WORKSPACE_SYNC_BYTES, then T.  Each GPU that loads the library carries one copy until exit.
 static __device__ __align__(256) unsigned char g_noalloc_scratch[SLIM_NOALLOC_SCRATCH_BYTES];
 
 // In host code `g_noalloc_scratch` is only a handle for the runtime, not an
@@ -28,6 +28,13 @@ static slim_status_t scratch_address(void** out) {
     return SLIM_OK;
 }
 
+// Size limit of the entry point: T, and one fp32 sum per output and 2048 columns (what a kernel that splits the
+// columns over the whole GPU needs), have to fit the array.  0: not a problem this entry point takes.
+static size_t noalloc_need(int b, int d_out, int d_in, int r) {
+    if (b < 1 || b > 16 || d_in % 256 != 0 || d_in > 32768 || !small_supports(b, d_out, d_in, r)) return 0;
+    return kSmallTBytes + (size_t)ceil_div(d_in, 2048) * d_out * (b <= 8 ? 8 : 16) * sizeof(float);
+}
+
 static bool is_aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 }  // namespace slim
@@ -37,7 +44,7 @@ using namespace slim;
 extern "C" size_t slim_noalloc_scratch_needed(int b, int d_out, int d_in, int r)
 {
     if (b < 1 || b > 16 || r < 0 || d_out < 1 || d_in < 1 || d_in % 64 != 0 || d_out % 16 != 0 || r % 16 != 0) return 0;
-    const size_t need = decode_workspace_bytes(b, d_out, d_in, r);
+    const size_t need = noalloc_need(b, d_out, d_in, r);
     return need ? SLIM_WORKSPACE_SYNC_BYTES + need : 0;
 }
 
@@ -54,23 +61,20 @@ extern "C" slim_status_t slim_linear_fwd_noalloc(const void* X, int b, const uin
         !is_aligned16(R))
         return SLIM_ERR_INVALID_ARG;
     if (status_dev && (reinterpret_cast<uintptr_t>(status_dev) & 3u)) return SLIM_ERR_INVALID_ARG;
-    // only problems the decode kernel takes, and only while its scratch fits the static array
-    const size_t need = decode_workspace_bytes(b, d_out, d_in, r);
+    // only while the scratch fits the static array
+    const size_t need = noalloc_need(b, d_out, d_in, r);
     if (b > 16 || need == 0) return SLIM_ERR_UNSUPPORTED_SHAPE;
     if (SLIM_WORKSPACE_SYNC_BYTES + need > (size_t)SLIM_NOALLOC_SCRATCH_BYTES) return SLIM_ERR_WORKSPACE;
     slim_status_t derr;
     if (!device_info(&derr)) return derr;
-    if (!decode_supports(b, d_out, d_in, r)) return SLIM_ERR_UNSUPPORTED_SHAPE;
     void* scratch = nullptr;
     slim_status_t st = scratch_address(&scratch);
     if (st != SLIM_OK) return st;
     cudaStream_t stream = (cudaStream_t)cuda_stream;
-    // the array keeps whatever the previous call left (possibly of another shape, possibly cut
-    // short by a timeout): mark this call's hand-over slots empty and restart the call counter
-    if (cudaMemsetAsync(static_cast<char*>(scratch) + SLIM_WORKSPACE_SYNC_BYTES, 0xFF, need, stream) != cudaSuccess ||
-        cudaMemsetAsync(scratch, 0, SLIM_WORKSPACE_SYNC_BYTES, stream) != cudaSuccess)
+    // the array keeps whatever the previous call left (possibly cut short by a timeout): restart the call counter and
+    // the call numbers of T's entries
+    if (cudaMemsetAsync(scratch, 0, SLIM_WORKSPACE_SYNC_BYTES + ((size_t)b * r * 4 + 255) / 256 * 256, stream) != cudaSuccess)
         return SLIM_ERR_CUDA;
-    return launch_decode(static_cast<const __nv_bfloat16*>(X), b, vals, meta, s,
-                         static_cast<const __nv_bfloat16*>(L), static_cast<const __nv_bfloat16*>(R), r, d_out,
-                         d_in, static_cast<__nv_bfloat16*>(Y), scratch, status_dev, stream);
+    return launch_small(static_cast<const __nv_bfloat16*>(X), b, vals, meta, nullptr, s, L, R, nullptr, nullptr, r, d_out, d_in,
+                        static_cast<__nv_bfloat16*>(Y), scratch, status_dev, stream);
 }

@@ -704,7 +704,7 @@ slim_status_t launch_prefill(const __nv_bfloat16* X, int b, const uint8_t* vals,
             return SLIM_ERR_CUDA;
         g_prefill_attr_set[dev].store(true, std::memory_order_release);
     }
-    __nv_bfloat16* Tq = reinterpret_cast<__nv_bfloat16*>(reinterpret_cast<char*>(ws) + SLIM_WORKSPACE_SYNC_BYTES);
+    __nv_bfloat16* Tq = reinterpret_cast<__nv_bfloat16*>(reinterpret_cast<char*>(ws) + SLIM_WORKSPACE_SYNC_BYTES + kSmallTBytes);
     const float s_eff = s != 0.f ? s : 1.f;       // with s == 0 only the adapter term remains
     // token tile: 256 when that gives a quarter of the SMs or more a tile, else 64 (measured: with 64 tiles of
     // 128 x 256 on 148 SMs the wide variant is a third faster than 256 tiles of 128 x 64; with 32 it is slower)
@@ -772,9 +772,6 @@ slim_status_t launch_prefill(const __nv_bfloat16* X, int b, const uint8_t* vals,
     else rc = pair ? launch_tile_kernel<256, true>(p, d_out, tmV, tmM, tmX, tmA2, tmB2, st, 1, dep)
                    : launch_tile_kernel<256, false>(p, d_out, tmV, tmM, tmX, tmA2, tmB2, st, 1, dep);
     if (rc != SLIM_OK) return rc;
-    // T' and the partial tiles were written where the decode kernels keep their hand-over slots
-    // (all ones = empty): leave the region as they expect it.
-    if (r > 0 && cudaMemsetAsync(Tq, 0xFF, prefill_workspace_bytes(b, d_out, d_in, r), st) != cudaSuccess) return SLIM_ERR_CUDA;
     return SLIM_OK;
 }
 

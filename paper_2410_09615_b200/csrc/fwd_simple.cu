@@ -79,7 +79,7 @@ slim_status_t launch_simple(const __nv_bfloat16* X, int b, const uint8_t* vals, 
     slim_status_t err;
     const DeviceInfo* di = device_info(&err);
     if (!di) return err;
-    float* T = reinterpret_cast<float*>(reinterpret_cast<char*>(ws) + SLIM_WORKSPACE_SYNC_BYTES);
+    float* T = reinterpret_cast<float*>(reinterpret_cast<char*>(ws) + SLIM_WORKSPACE_SYNC_BYTES + kSmallTBytes);
     const int cap = di->sm_count * 16;
     if (r > 0) {
         long long blocks = ((long long)b * r + 7) / 8;
@@ -91,8 +91,6 @@ slim_status_t launch_simple(const __nv_bfloat16* X, int b, const uint8_t* vals, 
                                                                       d_out, d_in, Y);
     count_launch(1);
     if (cudaGetLastError() != cudaSuccess) return SLIM_ERR_CUDA;
-    // The decode kernels read this region as hand-over slots (all ones = empty): leave it as they expect it.
-    if (r > 0 && cudaMemsetAsync(T, 0xFF, (size_t)b * r * sizeof(float), st) != cudaSuccess) return SLIM_ERR_CUDA;
     return SLIM_OK;
 }
 

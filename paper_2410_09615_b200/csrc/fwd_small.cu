@@ -1,0 +1,1019 @@
+// Small-batch forward (b <= 64): one launch of thread-block clusters that streams the weight and the
+// adapters exactly once.
+//
+// Work split.  A tile is 256 output rows; the C CTAs of a cluster (C = 1, 2, 4 or 8) cut d_in into C
+// ranges of whole 256-column units.  In a CTA eight consumer warps are 4 row blocks of 64 rows x 2
+// halves of every unit: a warp keeps the fp32 accumulators of its 64 rows x b tokens in registers
+// through the whole range (from 33 tokens on the two halves are token halves instead), so nothing is
+// summed across warps inside the stream; the partial tiles meet once, at the end, over distributed
+// shared memory.  C is the largest with which the clusters of all tiles are resident at once (two CTAs
+// per SM up to 16 tokens), so that a tile's stream is spread as widely as it can be.
+//   The first clusters make T = X R^T instead: 32 rows of R each, the same cut of d_in; their
+// CTAs exchange partial sums with asynchronous remote stores, round to bf16 and publish T as 8-byte words
+// {two columns, call number}.
+//   A tile's cluster streams the packed weight and the activations through a ring of stages by TMA
+// (256 rows x 64 value bytes, x 32 index bytes, b tokens x 512 bytes; two requesting warps, since one
+// thread starts a request every 220 cycles and the engine takes about one 32-64 byte row a cycle),
+// then the columns of L, waiting for just the words of T it multiplies, then writes
+// Y = s X Q^T + T L^T.
+//
+// Fragments of the sparse MMA.  Inside a 256-column unit the four 64-column regions are q = 2 a + h; step
+// j = 0..7 multiplies groups 2 j and 2 j + 1 of every region: thread t of a quad owns byte 2 j + (t & 1)
+// of region a = t / 2 (h = 0: registers 0 and 1, h = 1: registers 2 and 3).  Then
+//   - a row's 16 value bytes of a region are one thread pair's operand of eight steps: one 8-byte read
+//     per row and half serves four steps, and a register costs half a shift, one prmt, one lop3 and one
+//     bf16 subtraction;
+//   - the index bits a lane has to supply for a step are byte j of two regions of two rows: two prmt;
+//   - the activations of a step are 16 contiguous bytes per token and region: one ldmatrix.x4.
+// The decode-tiled copy holds registers and index words in the instruction's natural column order instead.
+// Alone on an SM (16 warps) a 16-row x 32-column step takes a scheduler 33 cycles at 8 tokens, 41 at 16
+// (20 of them the ALU pipe's), and 24 / 33 on the tiled copy.
+//
+// The hand-over of T is the only wait between clusters.  It goes from lower to higher cluster numbers only:
+// clusters that make T wait for nobody and are started first, so the wait ends whether or not the whole grid is
+// resident.  Every poll is bounded in time.  An entry carries the number of the call that wrote it, so
+// nothing has to be cleared between calls; the call number is (departures >> 16) + 1, and every call adds
+// 1 << 16 to that counter in all.
+// Reductions have a fixed order: results are bit-identical from run to run.
+#include <atomic>
+#include <mutex>
+#include <cuda.h>
+#include "decode_tile.cuh"
+
+namespace slim {
+
+namespace {
+
+using namespace dt;
+
+constexpr int kCW = 8;                          // consumer warps
+constexpr int kConsumers = kCW * 32;
+constexpr int kProdW = kCW, kProdX = kCW + 1;   // requests of the weight, R and L; of the activations and the index bytes
+constexpr int kFetchT = kCW + 2;                // from 17 tokens on: two warps that bring T into shared memory
+constexpr int kRows = 256;                      // output rows of a tile
+constexpr int kUnit = 256;                      // columns of a stage
+constexpr int kValsBytes = kRows * 64, kMetaBytes = kRows * 32;
+constexpr int kWBytes = kValsBytes + kMetaBytes;   // 24 KB, = four 6144-byte pieces of the tiled copy
+constexpr int kGroup = 32;                      // rows of R in one piece of the T product
+constexpr int kRedPitch = 260;                  // floats per token of a partial tile (conflict-free writes)
+constexpr unsigned long long kWaitNs = 500ull * 1000 * 1000;
+
+enum { FMT_PACKED = 0, FMT_PACKED_LD = 1, FMT_TILED = 2 };   // LD: index bytes by cp.async (rows no 16-byte multiples)
+
+struct SmallParams {
+    const __nv_bfloat16* X; const uint8_t* meta; const uint8_t* tiled;
+    const void* L; const void* R;                             // bf16, or int4 codes
+    const __nv_bfloat16* Ls; const __nv_bfloat16* Rs;         // scales of quantized adapters
+    __nv_bfloat16* Y;
+    unsigned long long* T;                                    // [b][r / 2] {bf16 pair, call number}
+    unsigned long long* departures;
+    uint32_t* status;
+    float s;
+    int b, r, d_out, d_in;
+    int tiles, units, groups;                                 // of 256 rows, 256 columns, 32 rows of R
+};
+
+template <int NT> struct Cfg {
+    static constexpr int kTok = NT * 8;
+    static constexpr int kThreads = (kCW + (NT >= 4 ? 4 : 2)) * 32;
+    static constexpr int kNW = NT < 4 ? NT : 4;               // n-tiles of a warp: with eight, two warps share the tokens of a row block
+    static constexpr int kTSlots = NT == 8 ? 6 : 8, kTSlot = kTok * 64;        // steps of T in shared memory: 32 columns in bf16
+    static constexpr int kXBytes = kTok * 512;                // activations of a unit
+    static constexpr int kStage = kWBytes + kXBytes;
+    static constexpr int kStages = NT == 4 ? 4 : 3;
+    static constexpr int kPiece = kTok * kGroup * 4;          // bytes of a piece of T
+    static constexpr int kOffPart = kStages * kStage;         // [4][kNW * 8][kGroup] floats, or the steps of T
+    static constexpr int kPartBytes = 4 * kNW * 8 * kGroup * 4 > (NT >= 4 ? kTSlots * kTSlot : 0) ? 4 * kNW * 8 * kGroup * 4 : kTSlots * kTSlot;
+    static constexpr int kOffRecv = kOffPart + kPartBytes;
+    static constexpr int kOffBars = kOffRecv + kPiece;
+    static constexpr int kSmem = kOffBars + 256;
+    static constexpr int kCtasPerSm = NT <= 2 ? 2 : 1;
+    static_assert((NT == 8 ? 1 : 2) * kTok * kRedPitch * 4 <= kStages * kStage, "partial tiles do not fit the ring");
+    static_assert(kSmem <= (NT <= 2 ? 113 : 227) * 1024, "shared memory");
+};
+
+__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" :: "r"(bar), "r"(count));
+}
+__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(bar) : "memory");
+}
+__device__ __forceinline__ void mbar_expect(uint32_t bar, uint32_t bytes) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" :: "r"(bar), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ uint32_t peer(uint32_t addr, uint32_t rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void mbar_arrive_peer(uint32_t bar) {
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" :: "r"(bar) : "memory");
+}
+__device__ __forceinline__ unsigned long long now_ns() {
+    unsigned long long t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+    return t;
+}
+// Waits for a phase, for kWaitNs at most (a try may suspend the thread, so the bound is on time).
+template <bool CLUSTER = false>
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
+    unsigned long long t0 = 0;
+    for (uint32_t it = 0;; ++it) {
+        uint32_t done;
+        if (CLUSTER)
+            asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                         : "=r"(done) : "r"(bar), "r"(parity) : "memory");
+        else
+            asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                         : "=r"(done) : "r"(bar), "r"(parity) : "memory");
+        if (done) return true;
+        if ((it & 63u) == 63u) {
+            const unsigned long long now = now_ns();
+            if (t0 == 0) t0 = now;
+            else if (now - t0 > kWaitNs) return false;
+        }
+    }
+}
+__device__ __forceinline__ void tma_tile(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar) {
+    asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
+                 :: "r"(dst), "l"(map), "r"(x), "r"(y), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void tma_tile3(uint32_t dst, const CUtensorMap* map, int y, int z, uint32_t bar) {
+    asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
+                 :: "r"(dst), "l"(map), "r"(0), "r"(y), "r"(z), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void bulk_copy(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 :: "r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void consumer_sync() { asm volatile("bar.sync 1, %0;" :: "n"(kConsumers) : "memory"); }
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ float4 ld_peer4(uint32_t addr) {
+    float4 v;
+    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr));
+    return v;
+}
+// Eight bytes into a peer's shared memory; its barrier counts them.
+__device__ __forceinline__ void st_peer2(uint32_t addr, float x, float y, uint32_t bar) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];" :: "r"(addr), "f"(x), "f"(y), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void sts_f(uint32_t addr, float v) { asm volatile("st.shared.f32 [%0], %1;" :: "r"(addr), "f"(v) : "memory"); }
+__device__ __forceinline__ void sts32(uint32_t addr, uint32_t v) { asm volatile("st.shared.u32 [%0], %1;" :: "r"(addr), "r"(v) : "memory"); }
+__device__ __forceinline__ float2 lds_f2(uint32_t addr) { float2 v; asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr)); return v; }
+__device__ __forceinline__ uint2 lds64(uint32_t addr) {
+    return *reinterpret_cast<const uint2*>(__cvta_shared_to_generic(addr));
+}
+// An entry of T is one 64-bit access: value and call number are seen together.
+__device__ __forceinline__ unsigned long long ld_gpu64(const unsigned long long* p) {
+    unsigned long long v;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_gpu64(unsigned long long* p, unsigned long long v) {
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" :: "l"(p), "l"(v) : "memory");
+}
+// Streamed once: keep it out of L1.
+__device__ __forceinline__ uint32_t ldg_stream32(const void* p) {
+    uint32_t v;
+    asm volatile("ld.global.nc.L1::no_allocate.u32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ void ldsm4(uint32_t addr, uint4& v) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr));
+}
+__device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
+    uint32_t d;
+    asm("prmt.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(sel));
+    return d;
+}
+// Eight int4 codes of a word give, shifted by 4 i, the pair (c_i, c_{i+4}); the other operand's eight
+// consecutive bf16 values are put in the same order.
+__device__ __forceinline__ uint4 pair_four_apart(const uint4& v) {
+    return make_uint4(prmt(v.x, v.z, 0x5410), prmt(v.x, v.z, 0x7632), prmt(v.y, v.w, 0x5410), prmt(v.y, v.w, 0x7632));
+}
+
+// ---------------------------------------------------------------- one stage of the weight
+struct Lane { int lane, g, t; };
+
+// Rows past d_out and columns past d_in arrive as zero bytes.  Zero values are what they should be, but zero index
+// bits name one position twice: before a ragged stage is multiplied every lane completes the index words it will
+// read itself (0x4: positions 0 and 1).
+__device__ __forceinline__ void complete_index(uint32_t stage, int rb, int kk, int mts, int cols_left, const Lane& ln)
+{
+    const int h = ln.t & 1, g = ln.g;
+    const uint32_t mrow = stage + kValsBytes + (uint32_t)(rb * 64 + g) * 32 + h * 8 + kk * 4, mx = (uint32_t)(g >> 2) & 1;
+    for (int i = 0; i < 8; ++i)                                   // rows g + 8 i; regions h and 2 + h
+#pragma unroll
+        for (int a = 0; a < 2; ++a)
+            if ((i >> 1) >= mts || 64 * (2 * a + h) >= cols_left) sts32(mrow + i * 256 + (((uint32_t)a ^ mx) << 4), 0x44444444u);
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the next use of the stage is written by TMA
+    __syncwarp();
+}
+
+// This warp's 64 rows x half a unit (four steps) of a packed-format stage, NB n-tiles from tile n0 on.
+// KS steps' activations are held at a time: four where the registers allow it, else two.
+template <int NT, int NB>
+__device__ __forceinline__ void weight_stage(float (&acc)[4][NB][4], uint32_t stage, int rb, int kk, int n0, const Lane& ln)
+{
+    constexpr int KS = NB <= 2 ? 4 : 2;
+    const int a = ln.t >> 1, h = ln.t & 1, g = ln.g;
+    // value bytes: 64-byte rows, 64-byte swizzle; index bytes: 32-byte rows, 32-byte swizzle
+    const uint32_t vrow = stage + (uint32_t)(rb * 64 + g) * 64 + kk * 8, vx = (uint32_t)(g >> 1) & 3;
+    const uint32_t v0 = vrow + (((uint32_t)(2 * a) ^ vx) << 4), v1 = vrow + (((uint32_t)(2 * a + 1) ^ vx) << 4);
+    const uint32_t mrow = stage + kValsBytes + (uint32_t)(rb * 64 + g) * 32 + h * 8 + kk * 4, mx = (uint32_t)(g >> 2) & 1;
+    const uint32_t m0 = mrow + (mx << 4), m1 = mrow + ((mx ^ 1) << 4);
+    // activations: 64-column sub-tiles of 128-byte token rows, 128-byte swizzle; lane l addresses row l & 7 of matrix l / 8
+    const int mat = ln.lane >> 3, tok = ln.lane & 7, q = 2 * (mat & 1) + (mat >> 1);
+    const uint32_t xrow = stage + kWBytes + (uint32_t)q * (NT * 1024) + (uint32_t)(n0 * 8 + tok) * 128;
+    const uint32_t sel_e = 0x4400u + (uint32_t)h * 0x1111u, sel_o = sel_e + 0x2222u;     // byte h (+ 2) of w and of w >> 4
+#pragma unroll
+    for (int s0 = 0; s0 < 4; s0 += KS) {
+        uint4 xb[KS][NB];
+#pragma unroll
+        for (int s = 0; s < KS; ++s)
+#pragma unroll
+            for (int n = 0; n < NB; ++n)
+                ldsm4(xrow + n * 1024 + ((((uint32_t)(kk * 4 + s0 + s)) ^ (uint32_t)tok) << 4), xb[s][n]);
+        // which two steps' index words this lane supplies: with four steps a quad's lanes share the work
+        const uint32_t S = KS == 4 ? (uint32_t)a : (uint32_t)(s0 >> 1);
+        const uint32_t msel = (2 * S) | ((4 + 2 * S) << 4) | ((2 * S + 1) << 8) | ((5 + 2 * S) << 12);
+#pragma unroll
+        for (int mt = 0; mt < 4; ++mt) {
+            const uint32_t vo = mt * 1024, mo = mt * 512;
+            uint32_t w[4][KS / 2];                            // (row g, h 0), (row g + 8, h 0), (row g, h 1), (row g + 8, h 1)
+            if (KS == 4) {
+                const uint2 x0 = lds64(v0 + vo), x1 = lds64(v0 + vo + 512), x2 = lds64(v1 + vo), x3 = lds64(v1 + vo + 512);
+                w[0][0] = x0.x; w[1][0] = x1.x; w[2][0] = x2.x; w[3][0] = x3.x;
+                w[0][KS / 2 - 1] = x0.y; w[1][KS / 2 - 1] = x1.y; w[2][KS / 2 - 1] = x2.y; w[3][KS / 2 - 1] = x3.y;
+            } else {
+                w[0][0] = lds32(v0 + vo + s0 * 2); w[1][0] = lds32(v0 + vo + 512 + s0 * 2);
+                w[2][0] = lds32(v1 + vo + s0 * 2); w[3][0] = lds32(v1 + vo + 512 + s0 * 2);
+            }
+            const uint32_t u = prmt(lds32(m0 + mo), lds32(m1 + mo), msel), v = prmt(lds32(m0 + mo + 256), lds32(m1 + mo + 256), msel);
+            const uint32_t e0 = prmt(u, v, 0x5410), e1 = prmt(u, v, 0x7632);
+#pragma unroll
+            for (int s = 0; s < KS; ++s) {
+                uint32_t ar[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const uint32_t ww = w[i][s >> 1];
+                    ar[i] = nibbles_to_bf16x2(prmt(ww, ww >> 4, (s & 1) ? sel_o : sel_e));
+                }
+#pragma unroll
+                for (int n = 0; n < NB; ++n) {
+                    if (s < 2) mma_sp_16832<0>(acc[mt][n], ar, xb[s][n], (s & 1) ? e1 : e0);
+                    else       mma_sp_16832<1>(acc[mt][n], ar, xb[s][n], (s & 1) ? e1 : e0);
+                }
+            }
+        }
+    }
+}
+
+// The same for a stage of the decode-tiled copy (its row groups are complete): registers and index words in the
+// instruction's column order.
+template <int NT>
+__device__ __forceinline__ void weight_stage_tiled(float (&acc)[4][NT][4], uint32_t stage, int rb, int kk, const Lane& ln)
+{
+    const int mat = ln.lane >> 3, tok = ln.lane & 7;
+    const uint32_t xrow = stage + kWBytes + (uint32_t)tok * 128;
+    const uint32_t piece0 = stage + (uint32_t)rb * 6144;
+    const uint32_t idx_lane = (uint32_t)(ln.g * 4 + 2 * kk + (ln.t & 1));       // the lane that holds this half's index words
+#pragma unroll
+    for (int s0 = 0; s0 < 4; s0 += 2) {
+        uint4 xb[2][NT];
+#pragma unroll
+        for (int s = 0; s < 2; ++s)
+#pragma unroll
+            for (int n = 0; n < NT; ++n)   // step j = 4 kk + s0 + s: columns 32 j + 8 mat, sub-tile j / 2
+                ldsm4(xrow + (uint32_t)(2 * kk + (s0 >> 1)) * (NT * 1024) + n * 1024 + ((uint32_t)((s * 4 + mat) ^ tok) << 4), xb[s][n]);
+        uint2 w[4], e[4];
+#pragma unroll
+        for (int mt = 0; mt < 4; ++mt) {
+            w[mt] = lds64(piece0 + mt * 1536 + kk * 512 + ln.lane * 16 + s0 * 4);
+            e[mt] = lds64(piece0 + mt * 1536 + 1024 + idx_lane * 16 + s0 * 4);
+        }
+#pragma unroll
+        for (int s = 0; s < 2; ++s)
+#pragma unroll
+            for (int mt = 0; mt < 4; ++mt) {
+                const uint32_t ww = s ? w[mt].y : w[mt].x;
+                uint32_t ar[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) ar[i] = nibbles_to_bf16x2(ww >> (4 * i));
+#pragma unroll
+                for (int n = 0; n < NT; ++n) mma_sp_16832<0>(acc[mt][n], ar, xb[s][n], s ? e[mt].y : e[mt].x);
+            }
+    }
+}
+
+// ---------------------------------------------------------------- one stage of R
+// 32 rows of R x 256 columns: warp = (16-row tile m, 64-column sub-tile kq).
+template <int NT>
+__device__ __forceinline__ void adapter_stage(float (&acc)[NT][4], uint32_t stage, int m, int kq, const Lane& ln)
+{
+    const int mat = ln.lane >> 3, r8 = ln.lane & 7;
+    const uint32_t arow = stage + (uint32_t)kq * 4096 + (uint32_t)(m * 16 + (mat & 1) * 8 + r8) * 128;
+    const uint32_t xrow = stage + kWBytes + (uint32_t)kq * (NT * 1024) + (uint32_t)r8 * 128;
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {                  // 32 columns
+        uint4 a0, a1;
+        ldsm4(arow + ((uint32_t)((4 * s + (mat >> 1)) ^ r8) << 4), a0);
+        ldsm4(arow + ((uint32_t)((4 * s + 2 + (mat >> 1)) ^ r8) << 4), a1);
+#pragma unroll
+        for (int n = 0; n < NT; ++n) {
+            uint4 x;
+            ldsm4(xrow + n * 1024 + ((uint32_t)((4 * s + mat) ^ r8) << 4), x);
+            mma_16816(acc[n], a0.x, a0.y, a0.z, a0.w, x.x, x.y);
+            mma_16816(acc[n], a1.x, a1.y, a1.z, a1.w, x.z, x.w);
+        }
+    }
+}
+// The same on int4 codes.  A word of a row is eight columns; the activations of a step are read as the thread's
+// own eight columns and paired four apart.  The 64 columns lie in one group: the integer products are scaled once.
+template <int NT>
+__device__ __forceinline__ void adapter_stage_q(float (&acc)[NT][4], uint32_t stage, int m, int kq, float sc0, float sc1, const Lane& ln)
+{
+    const uint32_t arow = stage + (uint32_t)(m * 16 + ln.g) * 128 + ln.t * 4;
+    const uint32_t xrow = stage + kWBytes + (uint32_t)kq * (NT * 1024) + (uint32_t)ln.g * 128;
+    float part[NT][4];
+#pragma unroll
+    for (int n = 0; n < NT; ++n)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) part[n][e] = 0.f;
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+        const uint32_t lo = lds32(arow + ((uint32_t)((2 * kq + s) ^ ln.g) << 4)), hi = lds32(arow + 1024 + ((uint32_t)((2 * kq + s) ^ ln.g) << 4));
+        uint32_t a[4], c[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) { a[i] = nibbles_to_bf16x2(lo >> (4 * i)); c[i] = nibbles_to_bf16x2(hi >> (4 * i)); }
+#pragma unroll
+        for (int n = 0; n < NT; ++n) {
+            const uint4 x = pair_four_apart(lds128(xrow + n * 1024 + ((uint32_t)((4 * s + ln.t) ^ ln.g) << 4)));
+            mma_16816(part[n], a[0], c[0], a[1], c[1], x.x, x.y);
+            mma_16816(part[n], a[2], c[2], a[3], c[3], x.z, x.w);
+        }
+    }
+#pragma unroll
+    for (int n = 0; n < NT; ++n) {
+        acc[n][0] = fmaf(part[n][0], sc0, acc[n][0]); acc[n][1] = fmaf(part[n][1], sc0, acc[n][1]);
+        acc[n][2] = fmaf(part[n][2], sc1, acc[n][2]); acc[n][3] = fmaf(part[n][3], sc1, acc[n][3]);
+    }
+}
+
+// The words of T that B fragments need (two columns each): asked for, then waited for.  No address: a padding token or
+// column, zero.
+template <int NE>
+__device__ __forceinline__ void ask_T(unsigned long long (&v)[NE], const unsigned long long* const (&at)[NE], uint32_t call)
+{
+#pragma unroll
+    for (int n = 0; n < NE; ++n) v[n] = at[n] ? ld_gpu64(at[n]) : (unsigned long long)call << 32;
+}
+template <int NE>
+__device__ __forceinline__ bool wait_T(unsigned long long (&v)[NE], const unsigned long long* const (&at)[NE], uint32_t call)
+{
+    unsigned long long t0 = 0;
+    for (uint32_t spin = 0;; ++spin) {
+        bool all = true;
+#pragma unroll
+        for (int n = 0; n < NE; ++n) all = all && (uint32_t)(v[n] >> 32) == call;
+        if (__all_sync(0xffffffffu, all)) return true;
+        if ((spin & 63u) == 63u) {
+            const unsigned long long now = now_ns();
+            bool late = false;
+            if (t0 == 0) t0 = now;
+            else late = now - t0 > kWaitNs;
+            if (__any_sync(0xffffffffu, late)) return false;
+        }
+        __nanosleep(40);
+        ask_T<NE>(v, at, call);
+    }
+}
+
+// Y of the rows this CTA finishes, 256 / C of the tile: the 2 C (eight n-tiles: C) partial tiles in a fixed order, four
+// rows of a token at a time.
+template <int NT, int C>
+__device__ __forceinline__ void finish(const SmallParams& p, uint32_t smem, int tile, int rank)
+{
+    constexpr int kHalves = NT == 8 ? 1 : 2, kQuads = kRows / C / 4;
+    constexpr int kUn = NT == 1 || NT < C ? 1 : NT / C;       // items in flight
+    const uint32_t half = (uint32_t)(NT * 8 * kRedPitch * 4);
+    for (int e0 = threadIdx.x; e0 < p.b * kQuads; e0 += kConsumers * kUn) {
+        float4 v[kUn][C][kHalves];
+#pragma unroll
+        for (int i = 0; i < kUn; ++i) {
+            const int e = min(e0 + i * kConsumers, p.b * kQuads - 1), tok = e / kQuads, row = rank * (kRows / C) + 4 * (e % kQuads);
+            const uint32_t at = smem + (uint32_t)(tok * kRedPitch + row) * 4;
+#pragma unroll
+            for (int c = 0; c < C; ++c)
+#pragma unroll
+                for (int h = 0; h < kHalves; ++h) v[i][c][h] = ld_peer4(peer(at + h * half, c));
+        }
+#pragma unroll
+        for (int i = 0; i < kUn; ++i) {
+            const int e = e0 + i * kConsumers, tok = e / kQuads, n = tile * kRows + rank * (kRows / C) + 4 * (e % kQuads);
+            if (e < p.b * kQuads && n < p.d_out) {
+                float4 y = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                for (int c = 0; c < C; ++c)
+#pragma unroll
+                    for (int h = 0; h < kHalves; ++h) { y.x += v[i][c][h].x; y.y += v[i][c][h].y; y.z += v[i][c][h].z; y.w += v[i][c][h].w; }
+                __nv_bfloat162 lo = __floats2bfloat162_rn(y.x, y.y), hi = __floats2bfloat162_rn(y.z, y.w);
+                *reinterpret_cast<uint2*>(p.Y + (size_t)tok * p.d_out + n) = make_uint2(*reinterpret_cast<uint32_t*>(&lo), *reinterpret_cast<uint32_t*>(&hi));
+            }
+        }
+    }
+}
+
+// ---------------------------------------------------------------- the kernel
+template <int NT, int FMT, bool QA>
+__global__ void __launch_bounds__(Cfg<NT>::kThreads, Cfg<NT>::kCtasPerSm)
+small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmM,
+             const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmR, const __grid_constant__ CUtensorMap tmL)
+{
+    using C_ = Cfg<NT>;
+    constexpr int kTok = C_::kTok, kNW = C_::kNW, kStages = C_::kStages, kStage = C_::kStage;
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    const uint32_t smem = smem_u32(smem_raw);
+    const uint32_t part = smem + C_::kOffPart, recv = smem + C_::kOffRecv, bars = smem + C_::kOffBars;
+    const uint32_t full = bars, empty = bars + 32, piece_bar = bars + 64, red_full = bars + 72, t_full = bars + 80, t_empty = bars + 144;
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    Lane ln; ln.lane = lane; ln.g = lane >> 2; ln.t = lane & 3;
+    uint32_t C, rank;
+    asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(C));
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+    const int logC = 31 - __clz((int)C);
+    // the first clusters make T, a piece each, and wait for nobody; the others wait for them
+    const int cluster = blockIdx.x >> logC;
+    const bool makes_T = cluster < p.groups;
+    const int piece = cluster, tile = cluster - p.groups;
+    const int u0 = (int)(rank * (unsigned)p.units) >> logC, u1 = (int)((rank + 1) * (unsigned)p.units) >> logC;
+    const int u_end = p.s != 0.f ? u1 : u0;                    // s == 0: the adapter term alone
+    const int l_steps = ceil_div(p.r, 32);
+
+    if (threadIdx.x == 0) {
+        // a stage's barrier counts both producers (and, with index bytes by cp.async, the lanes of one of them)
+        for (int i = 0; i < kStages; ++i) { mbar_init(full + 8 * i, FMT == FMT_PACKED_LD ? 34 : 2); mbar_init(empty + 8 * i, kCW); }
+        mbar_init(piece_bar, 1); mbar_init(red_full, C);
+        if (NT >= 4) for (int i = 0; i < C_::kTSlots; ++i) { mbar_init(t_full + 8 * i, 2); mbar_init(t_empty + 8 * i, kCW); }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        // every CTA of the cluster sends this one its share of the piece: 16 / C column pairs per token
+        mbar_expect(piece_bar, (uint32_t)p.b * 16 * 8);
+    }
+    __syncthreads();
+    cluster_arrive();                                          // waited for before the first access to a peer
+    bool ok = true;
+
+    int p_it = 0;                                              // producers: next stage
+    auto acquire = [&]() -> int {
+        const int st = p_it % kStages, use = p_it / kStages;
+        if (use > 0) ok = mbar_wait(empty + 8 * st, (use - 1) & 1) && ok;
+        ++p_it;
+        return st;
+    };
+    if (warp == kProdW) {
+        // ============================ the weight, R, L ============================
+        const int row0 = tile * kRows;
+        if (makes_T) {
+            for (int u = u0; u < u1; ++u) {
+                const int st = acquire();
+                const uint32_t bar = full + 8 * st;
+                if (lane == 0) {
+                    mbar_expect(bar, QA ? 4096 : 16384);
+                    if (QA) tma_tile(smem + st * kStage, &tmR, u * 128, piece * kGroup, bar);
+                    else tma_tile3(smem + st * kStage, &tmR, piece * kGroup, u * 4, bar);
+                }
+            }
+        } else {
+            const int groups = FMT == FMT_TILED ? min(4, ceil_div(p.d_out - row0, 64)) : 0;
+            for (int u = u0; u < u_end; ++u) {
+                const int st = acquire();
+                const uint32_t dst = smem + st * kStage, bar = full + 8 * st;
+                if (lane == 0) mbar_expect(bar, FMT == FMT_TILED ? groups * 6144 : kValsBytes);
+                if (FMT == FMT_TILED) {
+                    __syncwarp();
+                    if (lane < groups) bulk_copy(dst + lane * 6144, p.tiled + ((size_t)(tile * 4 + lane) * p.units + u) * 6144, 6144, bar);
+                } else if (lane == 0) {
+                    tma_tile(dst, &tmV, u * 64, row0, bar);
+                }
+            }
+            if (!QA)
+                for (int ls = (int)rank; ls < l_steps; ls += (int)C) {
+                    const int st = acquire();
+                    const uint32_t bar = full + 8 * st;
+                    if (lane == 0) {
+                        mbar_expect(bar, kRows * 64);
+                        mbar_arrive(bar);                       // in place of the other producer
+                        tma_tile(smem + st * kStage, &tmL, ls * 32, row0, bar);
+                    }
+                    if (FMT == FMT_PACKED_LD) mbar_arrive(bar);
+                }
+        }
+        cluster_wait();
+    } else if (warp == kProdX) {
+        // ============================ activations, index bytes ============================
+        const int row0 = tile * kRows;
+        if (makes_T) {
+            for (int u = u0; u < u1; ++u) {
+                const int st = acquire();
+                const uint32_t bar = full + 8 * st;
+                if (lane == 0) {
+                    mbar_expect(bar, C_::kXBytes);
+                    tma_tile3(smem + st * kStage + kWBytes, &tmX, 0, u * 4, bar);
+                }
+                if (FMT == FMT_PACKED_LD) mbar_arrive(bar);
+            }
+            // this CTA's share of the piece, once every CTA of the cluster has sent its sums
+            const uint32_t call = (uint32_t)(ld_gpu64(p.departures) >> 16) + 1u;
+            const int per = 16 >> logC;                        // column pairs of a token that this CTA adds up
+            ok = mbar_wait<true>(piece_bar, 0) && ok;
+            for (int e = lane; e < p.b * per; e += 32) {
+                const int tok = e / per, j = piece * kGroup + 2 * ((int)rank * per + e % per);
+                float2 s = lds_f2(recv + e * 8);
+#pragma unroll
+                for (int c = 1; c < 8; ++c)
+                    if (c < (int)C) {
+                        const float2 v = lds_f2(recv + (c * p.b * per + e) * 8);
+                        s.x += v.x; s.y += v.y;
+                    }
+                __nv_bfloat162 pr = __floats2bfloat162_rn(s.x, s.y);
+                if (j < p.r)
+                    st_gpu64(p.T + (size_t)tok * (p.r / 2) + (j >> 1), ((unsigned long long)call << 32) | *reinterpret_cast<uint32_t*>(&pr));
+            }
+        } else {
+            for (int u = u0; u < u_end; ++u) {
+                const int st = acquire();
+                const uint32_t dst = smem + st * kStage, bar = full + 8 * st;
+                if (lane == 0) mbar_expect(bar, C_::kXBytes + (FMT == FMT_PACKED ? kMetaBytes : 0));
+                __syncwarp();
+                if (lane == 0) tma_tile3(dst + kWBytes, &tmX, 0, u * 4, bar);
+                if (FMT == FMT_PACKED && lane == 1) tma_tile(dst + kValsBytes, &tmM, u * 32, row0, bar);
+                if (FMT == FMT_PACKED_LD) {
+                    // 256 rows x four 8-byte pieces (64 columns), stored as the TMA's 32-byte swizzle would
+                    const size_t pitch = (size_t)p.d_in / 8;
+                    const int q = lane & 3;
+                    const bool col_in = u * kUnit + q * 64 < p.d_in;
+#pragma unroll 4
+                    for (int r = lane >> 2; r < kRows; r += 8) {
+                        const bool in = col_in && row0 + r < p.d_out;
+                        const uint8_t* src = p.meta + (in ? (size_t)(row0 + r) * pitch + (size_t)u * 32 + q * 8 : 0);
+                        const uint32_t d = dst + kValsBytes + r * 32 + (((q >> 1) ^ ((r >> 2) & 1)) << 4) + (q & 1) * 8;
+                        asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" :: "r"(d), "l"(src), "r"(in ? 8 : 0) : "memory");
+                    }
+                    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" :: "r"(bar) : "memory");
+                }
+            }
+        }
+        cluster_wait();
+    } else if (NT >= 4 && warp >= kFetchT) {
+        // ============================ T into shared memory, step by step ============================
+        // [token][32 columns] bf16, 64-byte rows stored with the 64-byte swizzle; each of the two warps half of the tokens
+        if (!makes_T && p.r > 0) {
+            const uint32_t call = (uint32_t)(ld_gpu64(p.departures) >> 16) + 1u;
+            constexpr int kPer = NT * 2;                       // words a lane fetches
+            int it = 0;
+            for (int ls = (int)rank; ls < l_steps; ls += (int)C, ++it) {
+                const int st = it % C_::kTSlots, use = it / C_::kTSlots;
+                if (use > 0) ok = mbar_wait(t_empty + 8 * st, (use - 1) & 1) && ok;
+                unsigned long long v[kPer];
+                const unsigned long long* at[kPer];
+                const int pr = lane & 15, tok0 = (warp - kFetchT) * (kTok / 2) + (lane >> 4);
+#pragma unroll
+                for (int i = 0; i < kPer; ++i)
+                    at[i] = tok0 + 2 * i < p.b && ls * 32 + 2 * pr < p.r ? p.T + (size_t)(tok0 + 2 * i) * (p.r / 2) + ls * 16 + pr : nullptr;
+                ask_T<kPer>(v, at, call);
+                ok = wait_T<kPer>(v, at, call) && ok;
+#pragma unroll
+                for (int i = 0; i < kPer; ++i) {
+                    const int tok = tok0 + 2 * i;
+                    sts32(part + st * C_::kTSlot + tok * 64 + (((pr >> 2) ^ ((tok >> 1) & 3)) << 4) + (pr & 3) * 4, (uint32_t)v[i]);
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(t_full + 8 * st);
+            }
+        }
+        cluster_wait();
+    } else {
+        // ============================ consumer warps ============================
+        uint32_t call = 0;
+        if (p.r > 0) call = (uint32_t)(ld_gpu64(p.departures) >> 16) + 1u;
+        int it = 0;
+        auto wait_stage = [&]() -> uint32_t {
+            const int st = it % kStages;
+            ok = mbar_wait(full + 8 * st, (it / kStages) & 1) && ok;
+            return smem + st * kStage;
+        };
+        auto release = [&]() {
+            __syncwarp();
+            if (lane == 0) mbar_arrive(empty + 8 * (it % kStages));
+            ++it;
+        };
+        if (makes_T) {
+            // ---------------- a piece of T
+            const int m = warp & 1, kq = warp >> 1;
+            const bool valid = piece * kGroup + m * 16 < p.r;
+            float acc[NT][4];
+#pragma unroll
+            for (int n = 0; n < NT; ++n)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) acc[n][e] = 0.f;
+            for (int u = u0; u < u1; ++u) {
+                float sc0 = 0.f, sc1 = 0.f;
+                if (QA && valid && u * kUnit + 64 * kq < p.d_in) {
+                    const size_t per_row = (size_t)((p.d_in + 127) >> 7);
+                    const __nv_bfloat16* s = p.Rs + (size_t)(piece * kGroup + m * 16 + ln.g) * per_row + 2 * u + (kq >> 1);
+                    sc0 = __bfloat162float(s[0]); sc1 = __bfloat162float(s[8 * per_row]);
+                }
+                const uint32_t stage = wait_stage();
+                if (valid) {
+                    if (QA) adapter_stage_q<NT>(acc, stage, m, kq, sc0, sc1, ln);
+                    else adapter_stage<NT>(acc, stage, m, kq, ln);
+                }
+                release();
+            }
+            // four partial sums per element: added up in shared memory and sent to the CTA that owns the column pair.
+            // Element (token, column j) sits at token * 32 + (j ^ 8 * (token / 2 % 4)): conflict-free both ways.
+            const int per = 16 >> logC;
+#pragma unroll
+            for (int n0 = 0; n0 < NT; n0 += kNW) {
+                if (n0 > 0) consumer_sync();
+#pragma unroll
+                for (int n = 0; n < kNW; ++n)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e)
+                        sts_f(part + (uint32_t)((kq * kNW * 8 + n * 8 + 2 * ln.t + (e & 1)) * kGroup + ((m * 16 + ln.g + 8 * (e >> 1)) ^ (8 * ln.t))) * 4, acc[n0 + n][e]);
+                consumer_sync();
+                if (n0 == 0) cluster_wait();
+                for (int e = threadIdx.x; e < kNW * 8 * 16; e += kConsumers) {
+                    const int tok = e >> 4, pr = e & 15;
+                    const uint32_t at = part + (uint32_t)(tok * kGroup + ((2 * pr) ^ (8 * ((tok >> 1) & 3)))) * 4;
+                    float2 s = lds_f2(at);
+#pragma unroll
+                    for (int w = 1; w < 4; ++w) {
+                        const float2 v = lds_f2(at + w * kNW * 8 * kGroup * 4);
+                        s.x += v.x; s.y += v.y;
+                    }
+                    const int gt = n0 * 8 + tok, owner = pr >> (4 - logC);
+                    if (gt < p.b) {
+                        const uint32_t dst = recv + (uint32_t)(((int)rank * p.b + gt) * per + (pr & (per - 1))) * 8;
+                        st_peer2(peer(dst, owner), s.x, s.y, peer(piece_bar, owner));
+                    }
+                }
+            }
+        } else {
+            const int rb = warp & 3, kk = warp >> 2;
+            const int n_first = NT == 8 ? 4 * kk : 0;           // with eight n-tiles kk picks tokens, not columns
+            const int row0 = tile * kRows + rb * 64;
+            const int mts = max(0, min(4, (p.d_out - row0) / 16));          // valid 16-row tiles of this warp
+            float acc[4][kNW][4];
+#pragma unroll
+            for (int m = 0; m < 4; ++m)
+#pragma unroll
+                for (int n = 0; n < kNW; ++n)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) acc[m][n][e] = 0.f;
+            // ---------------- the weight
+            for (int u = u0; u < u_end; ++u) {
+                const uint32_t stage = wait_stage();
+                if (mts > 0) {
+                    const int left = p.d_in - u * kUnit;
+                    if constexpr (FMT == FMT_TILED) {
+                        weight_stage_tiled<NT>(acc, stage, rb, kk, ln);
+                    } else if constexpr (NT == 8) {
+#pragma unroll 1
+                        for (int h = 0; h < 2; ++h) {
+                            if (mts < 4 || left < kUnit) complete_index(stage, rb, h, mts, left, ln);
+                            weight_stage<NT, kNW>(acc, stage, rb, h, n_first, ln);
+                        }
+                    } else {
+                        if (mts < 4 || left < kUnit) complete_index(stage, rb, kk, mts, left, ln);
+                        weight_stage<NT, kNW>(acc, stage, rb, kk, 0, ln);
+                    }
+                }
+                release();
+            }
+#pragma unroll
+            for (int m = 0; m < 4; ++m)
+#pragma unroll
+                for (int n = 0; n < kNW; ++n)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) acc[m][n][e] *= p.s;
+            // ---------------- T L^T
+            if constexpr (NT >= 4) {
+                // T from shared memory.  bf16: with four n-tiles kk picks the step's MMA depth; codes: the row tiles
+                int lt = 0;
+                for (int ls = (int)rank; ls < l_steps; ls += (int)C, ++lt) {
+                    const int ts = lt % C_::kTSlots;
+                    const uint32_t tslot = part + ts * C_::kTSlot;
+                    const int c = ls * 32 + 8 * ln.t;               // codes: r is a multiple of 16, a thread's 8 columns exist or not
+                    uint32_t lc[8];
+                    float sc[8];
+                    uint32_t stage = 0;
+                    if (QA) {
+#pragma unroll
+                        for (int m = 0; m < 8; ++m) {
+                            const bool mine = (m >> 1) < mts && (NT == 8 || (m >> 2) == kk);
+                            const size_t row = (size_t)(row0 + ln.g + 8 * m);
+                            lc[m] = mine && c < p.r ? ldg_stream32(static_cast<const uint8_t*>(p.L) + row * (p.r / 2) + c / 2) : 0u;
+                            sc[m] = mine ? __bfloat162float(p.Ls[row * ((p.r + 127) >> 7) + (ls >> 2)]) : 0.f;
+                        }
+                    } else {
+                        stage = wait_stage();
+                    }
+                    ok = mbar_wait(t_full + 8 * ts, (lt / C_::kTSlots) & 1) && ok;
+                    if (mts > 0) {
+                        const int mat = lane >> 3, r8 = lane & 7;
+                        if (QA) {
+                            uint4 tb[kNW];
+#pragma unroll
+                            for (int n = 0; n < kNW; ++n)
+                                tb[n] = pair_four_apart(lds128(tslot + ((n_first + n) * 8 + ln.g) * 64 + ((ln.t ^ ((ln.g >> 1) & 3)) << 4)));
+#pragma unroll
+                            for (int m = 0; m < 4; ++m) {
+                                if (NT == 8 || (m >> 1) == kk) {
+                                    uint32_t a[4], d[4];
+#pragma unroll
+                                    for (int q = 0; q < 4; ++q) { a[q] = nibbles_to_bf16x2(lc[2 * m] >> (4 * q)); d[q] = nibbles_to_bf16x2(lc[2 * m + 1] >> (4 * q)); }
+#pragma unroll
+                                    for (int n = 0; n < kNW; ++n) {
+                                        float pt[4] = {0.f, 0.f, 0.f, 0.f};
+                                        mma_16816(pt, a[0], d[0], a[1], d[1], tb[n].x, tb[n].y);
+                                        mma_16816(pt, a[2], d[2], a[3], d[3], tb[n].z, tb[n].w);
+                                        acc[m][n][0] = fmaf(pt[0], sc[2 * m], acc[m][n][0]); acc[m][n][1] = fmaf(pt[1], sc[2 * m], acc[m][n][1]);
+                                        acc[m][n][2] = fmaf(pt[2], sc[2 * m + 1], acc[m][n][2]); acc[m][n][3] = fmaf(pt[3], sc[2 * m + 1], acc[m][n][3]);
+                                    }
+                                }
+                            }
+                        } else {
+#pragma unroll
+                            for (int h = 0; h < 2; ++h) {
+                                if ((NT == 8 || h == kk) && ls * 32 + 16 * h < p.r) {
+                                    uint4 tb[kNW / 2];              // two n-tiles of 8 tokens x two chunks of 8 columns
+#pragma unroll
+                                    for (int n = 0; n < kNW / 2; ++n)
+                                        ldsm4(tslot + ((n_first + 2 * n + (mat >> 1)) * 8 + r8) * 64 + ((uint32_t)((2 * h + (mat & 1)) ^ ((r8 >> 1) & 3)) << 4), tb[n]);
+#pragma unroll
+                                    for (int m = 0; m < 4; ++m) {
+                                        uint4 a;                    // 64-byte rows, 64-byte swizzle
+                                        ldsm4(stage + (rb * 64 + m * 16 + (mat & 1) * 8 + r8) * 64 + ((uint32_t)((2 * h + (mat >> 1)) ^ ((r8 >> 1) & 3)) << 4), a);
+#pragma unroll
+                                        for (int n = 0; n < kNW / 2; ++n) {
+                                            mma_16816(acc[m][2 * n], a.x, a.y, a.z, a.w, tb[n].x, tb[n].y);
+                                            mma_16816(acc[m][2 * n + 1], a.x, a.y, a.z, a.w, tb[n].z, tb[n].w);
+                                        }
+                                    }
+                                }
+                            }
+                        }
+                    }
+                    if (!QA) release();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(t_empty + 8 * ts);
+                }
+            } else if constexpr (!QA) {
+                // kk picks the MMA depth of 16 of a 32-column step; the words of T are asked for one step ahead
+                const int mat = lane >> 3, r8 = lane & 7;
+                unsigned long long v[2 * kNW];
+                const unsigned long long* at[2 * kNW];
+                auto ask = [&](int ls) {
+                    const int j = ls * 32 + 16 * kk;
+#pragma unroll
+                    for (int n = 0; n < kNW; ++n) {
+                        const int tok = n * 8 + ln.g;
+                        const unsigned long long* e = p.T + (size_t)tok * (p.r / 2) + (j >> 1) + ln.t;
+                        const bool in = tok < p.b && j < p.r;
+                        at[2 * n] = in ? e : nullptr;
+                        at[2 * n + 1] = in ? e + 4 : nullptr;
+                    }
+                    ask_T<2 * kNW>(v, at, call);
+                };
+                ask((int)rank);
+                for (int ls = (int)rank; ls < l_steps; ls += (int)C) {
+                    ok = wait_T<2 * kNW>(v, at, call) && ok;
+                    uint32_t tb[2 * kNW];
+#pragma unroll
+                    for (int q = 0; q < 2 * kNW; ++q) tb[q] = (uint32_t)v[q];
+                    ask(ls + (int)C);
+                    const uint32_t stage = wait_stage();
+                    if (ls * 32 + 16 * kk < p.r && mts > 0) {
+#pragma unroll
+                        for (int m = 0; m < 4; ++m) {
+                            uint4 a;                                // 64-byte rows, 64-byte swizzle
+                            const int row = rb * 64 + m * 16 + (mat & 1) * 8 + r8;
+                            ldsm4(stage + row * 64 + ((uint32_t)((2 * kk + (mat >> 1)) ^ ((r8 >> 1) & 3)) << 4), a);
+#pragma unroll
+                            for (int n = 0; n < kNW; ++n) mma_16816(acc[m][n], a.x, a.y, a.z, a.w, tb[2 * n], tb[2 * n + 1]);
+                        }
+                    }
+                    release();
+                }
+            } else if (mts > 0) {
+                // codes by plain loads (rows of r / 2 bytes need not be 16-byte multiples), one step ahead
+                const int stride = 2 * (int)C;
+                uint32_t lc[8];
+                auto load = [&](int ls) {
+                    const int c = ls * 32 + 8 * ln.t;               // r is a multiple of 16: a thread's 8 columns exist or not
+#pragma unroll
+                    for (int m = 0; m < 8; ++m)                     // rows g + 8 m of the warp's 64
+                        lc[m] = c < p.r && (m >> 1) < mts ? ldg_stream32(static_cast<const uint8_t*>(p.L) + (size_t)(row0 + ln.g + 8 * m) * (p.r / 2) + c / 2) : 0u;
+                };
+                const int ls0 = (int)rank * 2 + kk;
+                load(ls0);
+                for (int ls = ls0; ls < l_steps; ls += stride) {
+                    const int c = ls * 32 + 8 * ln.t;
+                    float sc[8];
+#pragma unroll
+                    for (int m = 0; m < 8; ++m)
+                        sc[m] = (m >> 1) < mts ? __bfloat162float(p.Ls[(size_t)(row0 + ln.g + 8 * m) * ((p.r + 127) >> 7) + (ls >> 2)]) : 0.f;
+                    uint4 tb[kNW];
+#pragma unroll
+                    for (int n = 0; n < kNW; ++n) {
+                        const int tok = n * 8 + ln.g;
+                        unsigned long long v[4];
+                        const unsigned long long* at[4];
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) at[q] = c < p.r && tok < p.b ? p.T + (size_t)tok * (p.r / 2) + (c >> 1) + q : nullptr;
+                        ask_T<4>(v, at, call);
+                        ok = wait_T<4>(v, at, call) && ok;
+                        tb[n] = pair_four_apart(make_uint4((uint32_t)v[0], (uint32_t)v[1], (uint32_t)v[2], (uint32_t)v[3]));
+                    }
+                    uint32_t now[8];
+#pragma unroll
+                    for (int m = 0; m < 8; ++m) now[m] = lc[m];
+                    load(ls + stride);
+#pragma unroll
+                    for (int m = 0; m < 4; ++m) {
+                        uint32_t a[4], d[4];
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) { a[q] = nibbles_to_bf16x2(now[2 * m] >> (4 * q)); d[q] = nibbles_to_bf16x2(now[2 * m + 1] >> (4 * q)); }
+#pragma unroll
+                        for (int n = 0; n < kNW; ++n) {
+                            float pt[4] = {0.f, 0.f, 0.f, 0.f};
+                            mma_16816(pt, a[0], d[0], a[1], d[1], tb[n].x, tb[n].y);
+                            mma_16816(pt, a[2], d[2], a[3], d[3], tb[n].z, tb[n].w);
+                            acc[m][n][0] = fmaf(pt[0], sc[2 * m], acc[m][n][0]); acc[m][n][1] = fmaf(pt[1], sc[2 * m], acc[m][n][1]);
+                            acc[m][n][2] = fmaf(pt[2], sc[2 * m + 1], acc[m][n][2]); acc[m][n][3] = fmaf(pt[3], sc[2 * m + 1], acc[m][n][3]);
+                        }
+                    }
+                }
+            }
+            // ---------------- partial tiles -> Y
+            consumer_sync();                                   // every warp is done with the ring
+#pragma unroll
+            for (int m = 0; m < 4; ++m)
+#pragma unroll
+                for (int n = 0; n < kNW; ++n)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e)
+                        sts_f(smem + (uint32_t)(((NT == 8 ? 0 : kk * kTok) + (n_first + n) * 8 + 2 * ln.t + (e & 1)) * kRedPitch + rb * 64 + m * 16 + ln.g + 8 * (e >> 1)) * 4, acc[m][n][e]);
+            consumer_sync();
+            cluster_wait();
+            if (warp == 0 && lane < (int)C) mbar_arrive_peer(peer(red_full, lane));
+            ok = mbar_wait<true>(red_full, 0) && ok;
+            if (logC == 3) finish<NT, 8>(p, smem, tile, (int)rank);
+            else if (logC == 2) finish<NT, 4>(p, smem, tile, (int)rank);
+            else if (logC == 1) finish<NT, 2>(p, smem, tile, (int)rank);
+            else finish<NT, 1>(p, smem, tile, (int)rank);
+        }
+    }
+    if (!ok && lane == 0) flag_error(p.status, SLIM_ERR_TIMEOUT);
+    __syncwarp();
+    // nobody leaves while a peer may still read its shared memory (the reads are over: no memory ordering is asked for)
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+    cluster_wait();
+    if (threadIdx.x == 0) atomicAdd(p.departures, blockIdx.x == 0 ? 65536ull - (gridDim.x - 1) : 1ull);
+}
+
+// ------------------------------------------------------------------ host side
+using KernelFn = void (*)(const SmallParams, const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap);
+
+template <int NT, int FMT> KernelFn pick_q(bool qa) { return qa ? small_kernel<NT, FMT, true> : small_kernel<NT, FMT, false>; }
+KernelFn pick(int nt, int fmt, bool qa) {
+    if (fmt == FMT_TILED) return nt == 1 ? small_kernel<1, FMT_TILED, false> : small_kernel<2, FMT_TILED, false>;
+    if (fmt == FMT_PACKED)
+        return nt == 1 ? pick_q<1, FMT_PACKED>(qa) : nt == 2 ? pick_q<2, FMT_PACKED>(qa) : nt == 4 ? pick_q<4, FMT_PACKED>(qa) : pick_q<8, FMT_PACKED>(qa);
+    return nt == 1 ? pick_q<1, FMT_PACKED_LD>(qa) : nt == 2 ? pick_q<2, FMT_PACKED_LD>(qa) : nt == 4 ? pick_q<4, FMT_PACKED_LD>(qa) : pick_q<8, FMT_PACKED_LD>(qa);
+}
+int smem_bytes(int nt) { return nt == 1 ? Cfg<1>::kSmem : nt == 2 ? Cfg<2>::kSmem : nt == 4 ? Cfg<4>::kSmem : Cfg<8>::kSmem; }
+int threads_of(int nt) { return nt >= 4 ? Cfg<4>::kThreads : Cfg<1>::kThreads; }
+int tiles_of(int b) { return b <= 8 ? 1 : b <= 16 ? 2 : b <= 32 ? 4 : 8; }
+
+// Clusters of 1, 2, 4, 8 CTAs of one kernel that the device holds at once; asked once per device and kernel.
+struct Residency { std::atomic<int> ready{0}; int clusters[4]; };
+Residency g_res[64][4][3][2];
+std::mutex g_res_mutex;
+
+const int* residency(int dev, int nt, int fmt, bool qa) {
+    const int ni = nt == 1 ? 0 : nt == 2 ? 1 : nt == 4 ? 2 : 3;
+    Residency& rs = g_res[dev][ni][fmt][qa ? 1 : 0];
+    if (rs.ready.load(std::memory_order_acquire)) return rs.clusters;
+    std::lock_guard<std::mutex> lock(g_res_mutex);
+    if (rs.ready.load(std::memory_order_relaxed)) return rs.clusters;
+    const void* fn = (const void*)pick(nt, fmt, qa);
+    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes(nt)) != cudaSuccess) return nullptr;
+    for (int i = 0; i < 4; ++i) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(1u << i); cfg.blockDim = dim3(threads_of(nt)); cfg.dynamicSmemBytes = smem_bytes(nt);
+        cudaLaunchAttribute a[1];
+        a[0].id = cudaLaunchAttributeClusterDimension;
+        a[0].val.clusterDim.x = 1u << i; a[0].val.clusterDim.y = 1; a[0].val.clusterDim.z = 1;
+        cfg.attrs = a; cfg.numAttrs = 1;
+        int n = 0;
+        if (cudaOccupancyMaxActiveClusters(&n, fn, &cfg) != cudaSuccess) { cudaGetLastError(); n = 0; }
+        rs.clusters[i] = n;
+    }
+    rs.ready.store(1, std::memory_order_release);
+    return rs.clusters;
+}
+
+typedef CUresult (*EncodeFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
+                             const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
+                             CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+
+bool make_map(CUtensorMap* map, const void* base, CUtensorMapDataType type, int esize, uint64_t cols, uint64_t rows,
+              int box_cols, int box_rows, CUtensorMapSwizzle swz) {
+    EncodeFn fn = reinterpret_cast<EncodeFn>(tensor_map_encoder());
+    if (!fn) return false;
+    cuuint64_t dims[2] = {cols, rows};
+    cuuint64_t strides[1] = {cols * (uint64_t)esize};
+    cuuint32_t box[2] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows};
+    cuuint32_t estr[2] = {1, 1};
+    return fn(map, type, 2, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, swz,
+              CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// bf16 rows as 64-column sub-tiles: one box of box_rows rows x 4 sub-tiles of 128 bytes, in that order.
+bool make_map3(CUtensorMap* map, const void* base, uint64_t cols, uint64_t rows, int box_rows) {
+    EncodeFn fn = reinterpret_cast<EncodeFn>(tensor_map_encoder());
+    if (!fn) return false;
+    cuuint64_t dims[3] = {64, rows, cols / 64};
+    cuuint64_t strides[2] = {cols * 2, 128};
+    cuuint32_t box[3] = {64, (cuuint32_t)box_rows, 4};
+    cuuint32_t estr[3] = {1, 1, 1};
+    return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+              CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// CTAs per cluster: the most (up to 8, and no more than there are units) with which the clusters of all tiles fit the
+// device at once, so that the stream of a tile is spread as widely as it can be; with more tiles than that, one.
+int cluster_size(const int* res, int tiles, int units) {
+    for (int i = 3; i > 0; --i)
+        if ((1 << i) <= units && tiles <= res[i]) return 1 << i;
+    return 1;
+}
+
+}  // namespace
+
+// Limits of the kernel: the region of the workspace that T lives in (and r <= 3072), and the call counter, which
+// takes 65536 CTAs.
+bool small_supports(int b, int d_out, int d_in, int r) {
+    return b >= 1 && b <= 64 && d_out >= 16 && d_out % 16 == 0 && d_in >= 64 && d_in % 64 == 0 && r >= 0 && r % 16 == 0 &&
+           r <= kSmallMaxRank && (size_t)b * r * 4 <= kSmallTBytes && ceil_div(d_out, kRows) < 32768;
+}
+
+slim_status_t launch_small(const __nv_bfloat16* X, int b, const uint8_t* vals, const uint8_t* meta, const uint8_t* tiled, float s,
+                           const void* L, const void* R, const __nv_bfloat16* Ls, const __nv_bfloat16* Rs, int r, int d_out, int d_in,
+                           __nv_bfloat16* Y, void* ws, uint32_t* status_dev, cudaStream_t st)
+{
+    slim_status_t err;
+    if (!device_info(&err)) return err;
+    if (!small_supports(b, d_out, d_in, r) || (tiled && (b > 16 || d_in % 256 != 0 || Ls))) return SLIM_ERR_UNSUPPORTED_SHAPE;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return SLIM_ERR_CUDA;
+    const int nt = tiles_of(b), fmt = tiled ? FMT_TILED : d_in % 128 == 0 ? FMT_PACKED : FMT_PACKED_LD;
+    const bool qa = Ls != nullptr;
+    const int* res = residency(dev, nt, fmt, qa);
+    if (!res) return SLIM_ERR_CUDA;
+    SmallParams p;
+    p.X = X; p.meta = meta; p.tiled = tiled; p.L = L; p.R = R; p.Ls = Ls; p.Rs = Rs; p.Y = Y;
+    p.departures = reinterpret_cast<unsigned long long*>(ws);
+    p.T = reinterpret_cast<unsigned long long*>(reinterpret_cast<char*>(ws) + SLIM_WORKSPACE_SYNC_BYTES);
+    p.status = status_dev; p.s = s; p.b = b; p.r = r; p.d_out = d_out; p.d_in = d_in;
+    p.tiles = ceil_div(d_out, kRows); p.units = ceil_div(d_in, kUnit); p.groups = ceil_div(r, kGroup);
+    const int C = cluster_size(res, p.tiles, p.units);
+    CUtensorMap tmV, tmM, tmX, tmR, tmL;
+    bool ok = make_map3(&tmX, X, (uint64_t)d_in, (uint64_t)b, nt * 8);
+    if (!tiled) ok = ok && make_map(&tmV, vals, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)d_in / 4, (uint64_t)d_out, 64, kRows, CU_TENSOR_MAP_SWIZZLE_64B);
+    else tmV = tmX;
+    if (fmt == FMT_PACKED) ok = ok && make_map(&tmM, meta, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)d_in / 8, (uint64_t)d_out, 32, kRows, CU_TENSOR_MAP_SWIZZLE_32B);
+    else tmM = tmX;
+    if (r > 0) ok = ok && (qa ? make_map(&tmR, R, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)d_in / 2, (uint64_t)r, 128, kGroup, CU_TENSOR_MAP_SWIZZLE_128B)
+                              : make_map3(&tmR, R, (uint64_t)d_in, (uint64_t)r, kGroup));
+    else tmR = tmX;
+    if (r > 0 && !qa) ok = ok && make_map(&tmL, L, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (uint64_t)r, (uint64_t)d_out, 32, kRows, CU_TENSOR_MAP_SWIZZLE_64B);
+    else tmL = tmX;
+    if (!ok) return SLIM_ERR_CUDA;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(C * (p.tiles + p.groups))); cfg.blockDim = dim3(threads_of(nt)); cfg.dynamicSmemBytes = smem_bytes(nt); cfg.stream = st;
+    cudaLaunchAttribute a[1];
+    a[0].id = cudaLaunchAttributeClusterDimension;
+    a[0].val.clusterDim.x = (unsigned)C; a[0].val.clusterDim.y = 1; a[0].val.clusterDim.z = 1;
+    cfg.attrs = a; cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, pick(nt, fmt, qa), p, tmV, tmM, tmX, tmR, tmL);
+    count_launch(1);
+    return e == cudaSuccess ? SLIM_OK : SLIM_ERR_CUDA;
+}
+
+}  // namespace slim
