@@ -1,13 +1,15 @@
-"""ctypes binding of ``libslim.so`` with the same names as ``include/slim.h``.
+"""Binding of ``libslim.so`` with the same names as ``include/slim.h``.
 
 Argument marshalling only: tensors are torch CUDA tensors (torch supplies device
 memory and streams), every step of the computation runs in the library's
-kernels.  If the library is missing or a call fails, a :class:`SlimError` is
-raised; there is no fallback path.
+kernels.  The forward entry points go through the compiled call path of
+``csrc/native.cpp``, everything else through ctypes.  If a library is missing or a
+call fails, a :class:`SlimError` is raised; there is no fallback path.
 """
 from __future__ import annotations
 
 import ctypes
+import importlib.util
 import os
 
 import numpy as np
@@ -15,6 +17,7 @@ import torch
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libslim.so")
+NATIVE_PATH = os.path.join(_HERE, "_slim_native.so")
 
 (SLIM_OK, SLIM_ERR_INVALID_ARG, SLIM_ERR_UNSUPPORTED_SHAPE, SLIM_ERR_BAD_MASK, SLIM_ERR_CODE_RANGE,
  SLIM_ERR_WORKSPACE, SLIM_ERR_CUDA, SLIM_ERR_TIMEOUT, SLIM_ERR_ARCH) = range(9)
@@ -79,6 +82,24 @@ def lib() -> ctypes.CDLL:
             fn.restype, fn.argtypes = res, args
         _lib = l
     return _lib
+
+
+_native = None
+
+
+def native():
+    """Load the compiled call path and point it at :func:`lib`'s library; raise if it is absent."""
+    global _native
+    if _native is None:
+        if not os.path.exists(NATIVE_PATH):
+            raise SlimError(-1, "load", f"{NATIVE_PATH} not found: run paper_2410_09615_b200/build.py")
+        spec = importlib.util.spec_from_file_location("_slim_native", NATIVE_PATH)
+        m = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(m)
+        m.bind(SlimError, *[ctypes.cast(getattr(lib(), name), ctypes.c_void_p).value for name in
+                            ("slim_linear_fwd_ex", "slim_linear_fwd_tiled", "slim_linear_fwd_q", "slim_tiled_bytes", "slim_strerror")])
+        _native = m
+    return _native
 
 
 def strerror(code: int) -> str:
@@ -192,25 +213,10 @@ def slim_workspace_reset(workspace: torch.Tensor):
 def slim_linear_fwd(X, vals, meta, s: float, L, R, Y=None, workspace=None, status=None,
                     kernel: int = KERNEL_AUTO):
     """Y = X (s Q)^T + (X R^T) L^T on the current stream.  Returns Y (bf16 [b, d_out])."""
-    _dev(X, torch.bfloat16, "X"), _dev(vals, torch.uint8, "vals"), _dev(meta, torch.uint8, "meta")
-    b, d_in = X.shape
-    d_out = vals.shape[0]
-    r = 0 if L is None else L.shape[1]
-    if r:
-        _dev(L, torch.bfloat16, "L"), _dev(R, torch.bfloat16, "R")
-        if tuple(L.shape) != (d_out, r) or tuple(R.shape) != (r, d_in):
-            raise ValueError("adapter shapes do not match the weight")
-    if vals.shape[1] * 4 != d_in or tuple(meta.shape) != (d_out, d_in // 8):
-        raise ValueError("packed weight does not match X")
-    if Y is None:
-        Y = torch.empty((b, d_out), dtype=torch.bfloat16, device=X.device)
     if workspace is None:
-        workspace = new_workspace(b, d_out, d_in, r, X.device)
-    fn = lib().slim_linear_fwd_ex
-    _check(fn(_ptr(X), b, _ptr(vals), _ptr(meta), float(s), _ptr(L) if r else None, _ptr(R) if r else None,
-              r, d_out, d_in, _ptr(Y), _ptr(workspace), workspace.numel(), _ptr(status), _stream(), int(kernel)),
-           "slim_linear_fwd")
-    return Y
+        _dev(X, torch.bfloat16, "X"), _dev(vals, torch.uint8, "vals")
+        workspace = new_workspace(X.shape[0], vals.shape[0], X.shape[1], 0 if L is None else L.shape[1], X.device)
+    return (_native or native()).linear_fwd(X, vals, meta, s, L, R, Y, workspace, status, kernel)
 
 
 def slim_tiled_bytes(d_out: int, d_in: int, layout: int = LAYOUT_DECODE_TILED) -> int:
@@ -233,23 +239,10 @@ def slim_repack_tiled(vals: torch.Tensor, meta: torch.Tensor, layout: int = LAYO
 def slim_linear_fwd_tiled(X, tiled, d_out: int, s: float, L, R, Y=None, workspace=None, status=None,
                           layout: int = LAYOUT_DECODE_TILED):
     """Small-batch forward on a decode-tiled weight.  Returns Y (bf16 [b, d_out])."""
-    _dev(X, torch.bfloat16, "X"), _dev(tiled, torch.uint8, "tiled")
-    b, d_in = X.shape
-    r = 0 if L is None else L.shape[1]
-    if r:
-        _dev(L, torch.bfloat16, "L"), _dev(R, torch.bfloat16, "R")
-        if tuple(L.shape) != (d_out, r) or tuple(R.shape) != (r, d_in):
-            raise ValueError("adapter shapes do not match the weight")
-    if tiled.numel() != slim_tiled_bytes(d_out, d_in, layout):
-        raise ValueError("tiled weight does not match the shape")
-    if Y is None:
-        Y = torch.empty((b, d_out), dtype=torch.bfloat16, device=X.device)
     if workspace is None:
-        workspace = new_workspace(b, d_out, d_in, r, X.device)
-    _check(lib().slim_linear_fwd_tiled(_ptr(X), b, _ptr(tiled), layout, float(s), _ptr(L) if r else None,
-                                       _ptr(R) if r else None, r, d_out, d_in, _ptr(Y), _ptr(workspace),
-                                       workspace.numel(), _ptr(status), _stream()), "slim_linear_fwd_tiled")
-    return Y
+        _dev(X, torch.bfloat16, "X")
+        workspace = new_workspace(X.shape[0], d_out, X.shape[1], 0 if L is None else L.shape[1], X.device)
+    return (_native or native()).linear_fwd_tiled(X, tiled, d_out, s, L, R, Y, workspace, status, layout)
 
 
 def slim_linear_fwd_tiled_host(X_host: torch.Tensor, tiled, d_out: int, s: float, L, R, Y_host: torch.Tensor,
@@ -327,26 +320,15 @@ def slim_workspace_bytes_q(b: int, d_out: int, d_in: int, r: int) -> int:
 
 def slim_linear_fwd_q(X, vals, meta, s: float, Lq, Ls, Rq, Rs, Y=None, workspace=None, status=None):
     """Layer forward with quantized adapters.  Returns Y (bf16 [b, d_out])."""
-    _dev(X, torch.bfloat16, "X"), _dev(vals, torch.uint8, "vals"), _dev(meta, torch.uint8, "meta")
-    for name, t, dt in (("Lq", Lq, torch.uint8), ("Ls", Ls, torch.bfloat16), ("Rq", Rq, torch.uint8), ("Rs", Rs, torch.bfloat16)):
-        _dev(t, dt, name)
-    b, d_in = X.shape
-    d_out, r = vals.shape[0], Lq.shape[1] * 2
-    if tuple(Lq.shape) != (d_out, r // 2) or tuple(Rq.shape) != (r, d_in // 2):
-        raise ValueError("adapter code shapes do not match the weight")
-    if Y is None:
-        Y = torch.empty((b, d_out), dtype=torch.bfloat16, device=X.device)
     if workspace is None:
-        n = slim_workspace_bytes_q(b, d_out, d_in, r)
+        _dev(X, torch.bfloat16, "X"), _dev(vals, torch.uint8, "vals"), _dev(Lq, torch.uint8, "Lq")
+        n = slim_workspace_bytes_q(X.shape[0], vals.shape[0], X.shape[1], Lq.shape[1] * 2)
         if n == 0:
             raise SlimError(SLIM_ERR_UNSUPPORTED_SHAPE, "slim_workspace_bytes_q", "illegal shape")
         workspace = torch.empty(n, dtype=torch.uint8, device=X.device)
         with torch.cuda.device(X.device):
             slim_workspace_reset(workspace)
-    _check(lib().slim_linear_fwd_q(_ptr(X), b, _ptr(vals), _ptr(meta), float(s), _ptr(Lq), _ptr(Ls), _ptr(Rq), _ptr(Rs), r,
-                                   d_out, d_in, _ptr(Y), _ptr(workspace), workspace.numel(), _ptr(status), _stream()),
-           "slim_linear_fwd_q")
-    return Y
+    return (_native or native()).linear_fwd_q(X, vals, meta, s, Lq, Ls, Rq, Rs, Y, workspace, status)
 
 
 def slim_quant(W: torch.Tensor, status=None):

@@ -1,0 +1,217 @@
+// Call path of the forward entry points from Python: argument checks, the output tensor, the current stream and
+// the call into libslim, without interpreted code in between.  A small-batch call takes the GPU about as long as
+// one launch takes the host, so the path from the interpreter to the launch is part of its time: through ctypes and
+// per-argument Python checks a call took the host 22-23 us, this way 4-8 (three to four of them the launch).
+#include <torch/csrc/autograd/python_variable.h>
+#include <ATen/ATen.h>
+#include <ATen/cuda/EmptyTensor.h>
+#include <c10/cuda/CUDAStream.h>
+#include <cstdint>
+
+namespace {
+
+using FwdFn = int (*)(const void*, int, const uint8_t*, const uint8_t*, float, const void*, const void*, int, int, int, void*, void*,
+                      size_t, uint32_t*, void*, int);
+using TiledFn = int (*)(const void*, int, const void*, int, float, const void*, const void*, int, int, int, void*, void*, size_t,
+                        uint32_t*, void*);
+using QFn = int (*)(const void*, int, const uint8_t*, const uint8_t*, float, const uint8_t*, const void*, const uint8_t*, const void*,
+                    int, int, int, void*, void*, size_t, uint32_t*, void*);
+using BytesFn = size_t (*)(int, int, int);
+using TextFn = const char* (*)(int);
+
+FwdFn g_fwd = nullptr;
+TiledFn g_tiled = nullptr;
+QFn g_q = nullptr;
+BytesFn g_tiled_bytes = nullptr;
+TextFn g_text = nullptr;
+PyObject* g_error = nullptr;            // SlimError(code, where, text)
+
+// A contiguous CUDA tensor of the given type, or a TypeError.
+const at::Tensor* device_tensor(PyObject* o, at::ScalarType type, const char* name, const char* type_name) {
+    if (THPVariable_Check(o)) {
+        const at::Tensor& t = THPVariable_Unpack(o);
+        if (t.is_cuda() && t.scalar_type() == type && t.is_contiguous()) return &t;
+    }
+    PyErr_Format(PyExc_TypeError, "%s: expected a contiguous CUDA tensor of %s", name, type_name);
+    return nullptr;
+}
+const at::Tensor* bf16_tensor(PyObject* o, const char* name) { return device_tensor(o, at::kBFloat16, name, "torch.bfloat16"); }
+const at::Tensor* u8_tensor(PyObject* o, const char* name) { return device_tensor(o, at::kByte, name, "torch.uint8"); }
+
+// Any tensor's address, NULL for None (outputs, workspace and status).
+bool address(PyObject* o, const char* name, void** p, size_t* bytes = nullptr) {
+    *p = nullptr;
+    if (o == Py_None) return true;
+    if (!THPVariable_Check(o)) { PyErr_Format(PyExc_TypeError, "%s: expected a tensor", name); return false; }
+    const at::Tensor& t = THPVariable_Unpack(o);
+    *p = t.data_ptr();
+    if (bytes) *bytes = (size_t)t.numel();
+    return true;
+}
+
+bool rank2(const at::Tensor* t, const char* name) {
+    if (t->dim() == 2) return true;
+    PyErr_Format(PyExc_ValueError, "%s: expected a matrix", name);
+    return false;
+}
+
+PyObject* output(PyObject* given, int64_t b, int64_t d_out, const at::Tensor& like, void** p) {
+    if (given != Py_None) {
+        if (!address(given, "Y", p)) return nullptr;
+        Py_INCREF(given);
+        return given;
+    }
+    at::Tensor made = at::detail::empty_cuda({b, d_out}, at::kBFloat16, like.device(), std::nullopt);
+    *p = made.data_ptr();
+    return THPVariable_Wrap(std::move(made));
+}
+
+PyObject* finish(int code, PyObject* y, const char* where) {
+    if (code == 0) return y;
+    Py_DECREF(y);
+    PyObject* e = PyObject_CallFunction(g_error, "iss", code, where, g_text(code));
+    if (e) { PyErr_SetObject(g_error, e); Py_DECREF(e); }
+    return nullptr;
+}
+
+bool bound(Py_ssize_t given, Py_ssize_t wanted) {
+    if (!g_fwd) { PyErr_SetString(PyExc_RuntimeError, "bind() has not been called"); return false; }
+    if (given == wanted) return true;
+    PyErr_SetString(PyExc_TypeError, "wrong number of arguments");
+    return false;
+}
+
+// bf16 adapters L [d_out, r], R [r, d_in]; None: r = 0.
+bool adapters(PyObject* oL, PyObject* oR, int64_t d_out, int64_t d_in, void** L, void** R, int64_t* r) {
+    *L = *R = nullptr; *r = 0;
+    if (oL == Py_None) return true;
+    if (!THPVariable_Check(oL)) return bf16_tensor(oL, "L") != nullptr;
+    const at::Tensor& l = THPVariable_Unpack(oL);
+    if (!rank2(&l, "L")) return false;
+    *r = l.size(1);
+    if (*r == 0) return true;
+    const at::Tensor *pl = bf16_tensor(oL, "L"), *pr = pl ? bf16_tensor(oR, "R") : nullptr;
+    if (!pr) return false;
+    if (pl->size(0) != d_out || pr->dim() != 2 || pr->size(0) != *r || pr->size(1) != d_in) {
+        PyErr_SetString(PyExc_ValueError, "adapter shapes do not match the weight");
+        return false;
+    }
+    *L = pl->data_ptr(); *R = pr->data_ptr();
+    return true;
+}
+
+// linear_fwd(X, vals, meta, s, L, R, Y, workspace, status, kernel)
+PyObject* linear_fwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
+    if (!bound(n, 10)) return nullptr;
+    const at::Tensor *X = bf16_tensor(a[0], "X"), *v = X ? u8_tensor(a[1], "vals") : nullptr, *m = v ? u8_tensor(a[2], "meta") : nullptr;
+    if (!m || !rank2(X, "X") || !rank2(v, "vals") || !rank2(m, "meta")) return nullptr;
+    const double s = PyFloat_AsDouble(a[3]);
+    const long kernel = PyLong_AsLong(a[9]);
+    if (PyErr_Occurred()) return nullptr;
+    const int64_t b = X->size(0), d_in = X->size(1), d_out = v->size(0);
+    void *L, *R, *Y, *ws, *status;
+    int64_t r;
+    if (!adapters(a[4], a[5], d_out, d_in, &L, &R, &r)) return nullptr;
+    if (v->size(1) * 4 != d_in || m->size(0) != d_out || m->size(1) != d_in / 8) {
+        PyErr_SetString(PyExc_ValueError, "packed weight does not match X");
+        return nullptr;
+    }
+    size_t ws_bytes = 0;
+    if (!address(a[7], "workspace", &ws, &ws_bytes) || !address(a[8], "status", &status)) return nullptr;
+    PyObject* y = output(a[6], b, d_out, *X, &Y);
+    if (!y) return nullptr;
+    void* stream = c10::cuda::getCurrentCUDAStream().stream();
+    const void *xp = X->data_ptr(), *vp = v->data_ptr(), *mp = m->data_ptr();
+    int rc;
+    Py_BEGIN_ALLOW_THREADS
+    rc = g_fwd(xp, (int)b, (const uint8_t*)vp, (const uint8_t*)mp, (float)s, L, R, (int)r, (int)d_out, (int)d_in, Y, ws, ws_bytes,
+               (uint32_t*)status, stream, (int)kernel);
+    Py_END_ALLOW_THREADS
+    return finish(rc, y, "slim_linear_fwd");
+}
+
+// linear_fwd_tiled(X, tiled, d_out, s, L, R, Y, workspace, status, layout)
+PyObject* linear_fwd_tiled(PyObject*, PyObject* const* a, Py_ssize_t n) {
+    if (!bound(n, 10)) return nullptr;
+    const at::Tensor *X = bf16_tensor(a[0], "X"), *t = X ? u8_tensor(a[1], "tiled") : nullptr;
+    if (!t || !rank2(X, "X")) return nullptr;
+    const long d_out = PyLong_AsLong(a[2]);
+    const double s = PyFloat_AsDouble(a[3]);
+    const long layout = PyLong_AsLong(a[9]);
+    if (PyErr_Occurred()) return nullptr;
+    const int64_t b = X->size(0), d_in = X->size(1);
+    void *L, *R, *Y, *ws, *status;
+    int64_t r;
+    if (!adapters(a[4], a[5], d_out, d_in, &L, &R, &r)) return nullptr;
+    if ((size_t)t->numel() != g_tiled_bytes((int)d_out, (int)d_in, (int)layout)) {
+        PyErr_SetString(PyExc_ValueError, "tiled weight does not match the shape");
+        return nullptr;
+    }
+    size_t ws_bytes = 0;
+    if (!address(a[7], "workspace", &ws, &ws_bytes) || !address(a[8], "status", &status)) return nullptr;
+    PyObject* y = output(a[6], b, d_out, *X, &Y);
+    if (!y) return nullptr;
+    void* stream = c10::cuda::getCurrentCUDAStream().stream();
+    const void *xp = X->data_ptr(), *tp = t->data_ptr();
+    int rc;
+    Py_BEGIN_ALLOW_THREADS
+    rc = g_tiled(xp, (int)b, tp, (int)layout, (float)s, L, R, (int)r, (int)d_out, (int)d_in, Y, ws, ws_bytes, (uint32_t*)status, stream);
+    Py_END_ALLOW_THREADS
+    return finish(rc, y, "slim_linear_fwd_tiled");
+}
+
+// linear_fwd_q(X, vals, meta, s, Lq, Ls, Rq, Rs, Y, workspace, status)
+PyObject* linear_fwd_q(PyObject*, PyObject* const* a, Py_ssize_t n) {
+    if (!bound(n, 11)) return nullptr;
+    const at::Tensor *X = bf16_tensor(a[0], "X"), *v = X ? u8_tensor(a[1], "vals") : nullptr, *m = v ? u8_tensor(a[2], "meta") : nullptr;
+    const at::Tensor *Lq = m ? u8_tensor(a[4], "Lq") : nullptr, *Ls = Lq ? bf16_tensor(a[5], "Ls") : nullptr;
+    const at::Tensor *Rq = Ls ? u8_tensor(a[6], "Rq") : nullptr, *Rs = Rq ? bf16_tensor(a[7], "Rs") : nullptr;
+    if (!Rs || !rank2(X, "X") || !rank2(v, "vals") || !rank2(Lq, "Lq") || !rank2(Rq, "Rq")) return nullptr;
+    const double s = PyFloat_AsDouble(a[3]);
+    if (PyErr_Occurred()) return nullptr;
+    const int64_t b = X->size(0), d_in = X->size(1), d_out = v->size(0), r = Lq->size(1) * 2;
+    if (Lq->size(0) != d_out || Rq->size(0) != r || Rq->size(1) != d_in / 2) {
+        PyErr_SetString(PyExc_ValueError, "adapter code shapes do not match the weight");
+        return nullptr;
+    }
+    void *Y, *ws, *status;
+    size_t ws_bytes = 0;
+    if (!address(a[9], "workspace", &ws, &ws_bytes) || !address(a[10], "status", &status)) return nullptr;
+    PyObject* y = output(a[8], b, d_out, *X, &Y);
+    if (!y) return nullptr;
+    void* stream = c10::cuda::getCurrentCUDAStream().stream();
+    const void *xp = X->data_ptr(), *vp = v->data_ptr(), *mp = m->data_ptr(), *lqp = Lq->data_ptr(), *lsp = Ls->data_ptr(),
+               *rqp = Rq->data_ptr(), *rsp = Rs->data_ptr();
+    int rc;
+    Py_BEGIN_ALLOW_THREADS
+    rc = g_q(xp, (int)b, (const uint8_t*)vp, (const uint8_t*)mp, (float)s, (const uint8_t*)lqp, lsp, (const uint8_t*)rqp, rsp, (int)r,
+             (int)d_out, (int)d_in, Y, ws, ws_bytes, (uint32_t*)status, stream);
+    Py_END_ALLOW_THREADS
+    return finish(rc, y, "slim_linear_fwd_q");
+}
+
+// bind(SlimError, fwd_ex, fwd_tiled, fwd_q, tiled_bytes, strerror): addresses in the loaded libslim
+PyObject* bind(PyObject*, PyObject* args) {
+    PyObject* err;
+    unsigned long long f, t, q, by, tx;
+    if (!PyArg_ParseTuple(args, "OKKKKK", &err, &f, &t, &q, &by, &tx)) return nullptr;
+    Py_INCREF(err);
+    Py_XDECREF(g_error);
+    g_error = err;
+    g_fwd = reinterpret_cast<FwdFn>(f); g_tiled = reinterpret_cast<TiledFn>(t); g_q = reinterpret_cast<QFn>(q);
+    g_tiled_bytes = reinterpret_cast<BytesFn>(by); g_text = reinterpret_cast<TextFn>(tx);
+    Py_RETURN_NONE;
+}
+
+PyMethodDef methods[] = {
+    {"bind", bind, METH_VARARGS, nullptr},
+    {"linear_fwd", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)(void)>(linear_fwd)), METH_FASTCALL, nullptr},
+    {"linear_fwd_tiled", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)(void)>(linear_fwd_tiled)), METH_FASTCALL, nullptr},
+    {"linear_fwd_q", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)(void)>(linear_fwd_q)), METH_FASTCALL, nullptr},
+    {nullptr, nullptr, 0, nullptr}};
+
+PyModuleDef module = {PyModuleDef_HEAD_INIT, "_slim_native", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
+
+}  // namespace
+
+PyMODINIT_FUNC PyInit__slim_native() { return PyModule_Create(&module); }
