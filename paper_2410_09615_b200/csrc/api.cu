@@ -73,7 +73,7 @@ static bool runs_small(int b, int d_out, int d_in, int r) {
 
 static slim_kernel_t select_kernel(int b, int d_out, int d_in, int r) {
     if (b <= 16 && runs_small(b, d_out, d_in, r)) return SLIM_KERNEL_DECODE;
-    if (b > 16 && (runs_small(b, d_out, d_in, r) || prefill_supports(b, d_out, d_in, r))) return SLIM_KERNEL_PREFILL;
+    if (b > 16 && prefill_supports(b, d_out, d_in, r) && !small_and_ragged(b, d_out, d_in)) return SLIM_KERNEL_PREFILL;
     return SLIM_KERNEL_SIMPLE;
 }
 

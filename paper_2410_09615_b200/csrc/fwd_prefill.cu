@@ -100,6 +100,10 @@ struct PrefillParams {
     // writes its fp32 partial tile to part[z][token][ldo] (part == nullptr: one slice, bf16 to out)
     float* part;
     int k_per;
+    // Index bytes by cp.async where a tensor map cannot describe their rows (d_in / 8 bytes, no 16-byte
+    // multiple): the array and its row pitch; nullptr: by TMA.
+    const uint8_t* meta;
+    int meta_pitch;
 };
 
 // Optional timeline: built with -DSLIM_PREFILL_TRACE, one thread per warp role of the first
@@ -362,7 +366,7 @@ prefill_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap tmV,
             mbar_init(&b_full[i], 1);
             mbar_init(&conv_done[i], TWO ? kConvWarps : kConvWarps / 2); mbar_init(&empty[i], 1); mbar_init(&peer_ready[i], 1);
         }
-        for (int i = 0; i < kPkSlots; ++i) { mbar_init(&pk_full[i], 1); mbar_init(&pk_empty[i], kConvWarps); }
+        for (int i = 0; i < kPkSlots; ++i) { mbar_init(&pk_full[i], p.meta ? 33 : 1); mbar_init(&pk_empty[i], kConvWarps); }
         mbar_init(acc_full, 1);
         *abort_flag = 0u;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -421,9 +425,22 @@ prefill_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap tmV,
             const int slot = gi % kPkSlots;
             const int g = gi + rot_g < n_groups ? gi + rot_g : gi + rot_g - n_groups;
             if (gi >= kPkSlots) ok = mbar_wait(&pk_empty[slot], ((gi / kPkSlots) & 1) ^ 1, abort_flag) && ok;
-            if (lane == 0) mbar_expect_tx(&pk_full[slot], (uint32_t)kPkSlotBytes);
+            if (lane == 0) mbar_expect_tx(&pk_full[slot], (uint32_t)(p.meta ? kValsTile : kPkSlotBytes));
             unsigned char* dst = packed + slot * kPkSlotBytes + (lane == 0 ? 0 : kValsTile);
-            if (lane < 2) tma_tile(dst, lane == 0 ? &tmV : &tmM, g * (lane == 0 ? 64 : 32), m0, &pk_full[slot]);
+            if (lane < (p.meta ? 1 : 2)) tma_tile(dst, lane == 0 ? &tmV : &tmM, g * (lane == 0 ? 64 : 32), m0, &pk_full[slot]);
+            if (p.meta) {
+                // 128 rows x four 8-byte pieces (64 columns each), stored as the TMA's 32-byte swizzle would
+                const int q = lane & 3;
+                const bool col_in = g * 32 + q * 8 < p.meta_pitch;
+#pragma unroll 4
+                for (int r = lane >> 2; r < kPM; r += 8) {
+                    const bool in = col_in && m0 + r < p.m_total;
+                    const uint8_t* src = p.meta + (in ? (size_t)(m0 + r) * p.meta_pitch + g * 32 + q * 8 : 0);
+                    const uint32_t d = s32(packed + slot * kPkSlotBytes + kValsTile) + r * 32 + ((((q >> 1) ^ (r >> 2)) & 1) << 4) + (q & 1) * 8;
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" :: "r"(d), "l"(src), "r"(in ? 8 : 0) : "memory");
+                }
+                asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" :: "r"(s32(&pk_full[slot])) : "memory");
+            }
         }
     } else if (warp == kWarpMma) {
         // ============================ MMA issuer ============================
@@ -516,7 +533,8 @@ prefill_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap tmV,
             // the packed tiles are stored with the 64-byte (values) and 32-byte (indices) TMA swizzles so
             // that a warp's row-strided reads spread over the banks
             const uint4 v = *reinterpret_cast<const uint4*>(pk + row * 64 + (((q ^ (row >> 1)) & 3) << 4));
-            const uint2 mw2 = *reinterpret_cast<const uint2*>(pk + kValsTile + row * 32 + ((((q >> 1) ^ (row >> 2)) & 1) << 4) + (q & 1) * 8);
+            uint2 mw2 = *reinterpret_cast<const uint2*>(pk + kValsTile + row * 32 + ((((q >> 1) ^ (row >> 2)) & 1) << 4) + (q & 1) * 8);
+            if (m0 + row >= p.m_total) mw2 = make_uint2(0x44444444u, 0x44444444u);      // rows past the last: a legal pair of positions
             unsigned char* arow = stages + (size_t)st * kStageBytes + kBTile + row * 64;
             const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
@@ -649,8 +667,8 @@ static bool pf_map(CUtensorMap* map, const void* base, CUtensorMapDataType type,
 }
 
 bool prefill_supports(int b, int d_out, int d_in, int r) {
-    // d_in % 128: the rows of the index-byte array (d_in / 8 bytes) must be a multiple of 16 bytes for TMA
-    return b >= 1 && d_out % kPM == 0 && d_in % 128 == 0 && r % 16 == 0 && r >= 0;
+    // (when the rows of the index-byte array, d_in / 8 bytes, are no 16-byte multiples they come by cp.async)
+    return b >= 1 && d_out % 16 == 0 && d_in % kPBK == 0 && r % 16 == 0 && r >= 0;
 }
 
 size_t prefill_workspace_bytes(int b, int d_out, int d_in, int r) {
@@ -708,21 +726,22 @@ slim_status_t launch_prefill(const __nv_bfloat16* X, int b, const uint8_t* vals,
     const float s_eff = s != 0.f ? s : 1.f;       // with s == 0 only the adapter term remains
     // token tile: 256 when that gives a quarter of the SMs or more a tile, else 64 (measured: with 64 tiles of
     // 128 x 256 on 148 SMs the wide variant is a third faster than 256 tiles of 128 x 64; with 32 it is slower)
-    const bool wide = force_pair || (long long)(d_out / kPM) * ceil_div(b, 256) * 4 >= (long long)di->sm_count;
+    const bool wide = force_pair || (long long)ceil_div(d_out, kPM) * ceil_div(b, 256) * 4 >= (long long)di->sm_count;
     const int n_pre = 64;                         // the T' product has few row tiles: narrow token tiles fill the machine
     // The CTA-pair kernel (prefill_kernel<256, true>) measures 3-8 % faster than one CTA per tile on
     // problems with adapters and a thousand tiles or more (the 70B layers at 4096 tokens) and the same or
     // a little slower below that: it runs for those, or when asked for by name.
-    if (force_pair && (d_out / kPM) % 2 != 0) return SLIM_ERR_UNSUPPORTED_SHAPE;
-    const bool pair = force_pair || (wide && r > 0 && (d_out / kPM) % 2 == 0 &&
-                                     (long long)(d_out / kPM) * ceil_div(b, 256) >= 1024);
+    if (force_pair && ceil_div(d_out, kPM) % 2 != 0) return SLIM_ERR_UNSUPPORTED_SHAPE;
+    const bool pair = force_pair || (wide && r > 0 && ceil_div(d_out, kPM) % 2 == 0 &&
+                                     (long long)ceil_div(d_out, kPM) * ceil_div(b, 256) >= 1024);
     const int xbox = wide ? (pair ? 128 : 256) : 64;      // token rows one CTA loads per stage = one TMA box
     const int dk = PfCfg<256, false>::kDK;                // columns of a dense stage of the main kernels
     CUtensorMap tmV, tmM, tmX, tmXpre, tmA2, tmB2;
     bool ok = pf_map(&tmV, vals, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)d_in / 4, (uint64_t)d_out, kPkStages * kPBK / 4, kPM, 64) &&
-              pf_map(&tmM, meta, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)d_in / 8, (uint64_t)d_out, kPkStages * kPBK / 8, kPM, 32) &&
+              (d_in % 128 != 0 || pf_map(&tmM, meta, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)d_in / 8, (uint64_t)d_out, kPkStages * kPBK / 8, kPM, 32)) &&
               pf_map(&tmX, X, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (uint64_t)d_in, (uint64_t)b, 64, xbox, 128);
     if (!ok) return SLIM_ERR_CUDA;
+    if (d_in % 128 != 0) tmM = tmV;              // not used
     if (r > 0) {
         // T' = (X R^T) / s : dense phase only, output rows = adapter index
         const PrePlan pl = pre_plan(b, d_in, r, di->sm_count, s != 0.f);
@@ -731,7 +750,7 @@ slim_status_t launch_prefill(const __nv_bfloat16* X, int b, const uint8_t* vals,
         if (!ok) return SLIM_ERR_CUDA;
         PrefillParams q;
         q.out = Tq; q.ldo = r; q.m_total = r; q.b = b; q.n1 = 0; q.n2 = d_in / kPBK; q.scale = 1.f / s_eff; q.status = status_dev;
-        q.k_per = pl.k_per;
+        q.k_per = pl.k_per; q.meta = nullptr; q.meta_pitch = 0;
         // partial tiles of the K slices follow T' in the workspace
         q.part = pl.slices > 1 ? reinterpret_cast<float*>(reinterpret_cast<char*>(Tq) + ((size_t)b * r * sizeof(__nv_bfloat16) + 255) / 256 * 256) : nullptr;
         slim_status_t rc = pl.n_tok == 256 ? launch_tile_kernel<256, false, true>(q, r, tmV, tmM, tmXpre, tmA2, tmXpre, st, pl.slices)
@@ -763,6 +782,7 @@ slim_status_t launch_prefill(const __nv_bfloat16* X, int b, const uint8_t* vals,
     p.n1 = s != 0.f ? d_in / kPBK : 0;
     p.n2 = r > 0 ? ceil_div(r, dk) : 0;
     p.scale = s_eff; p.status = status_dev; p.part = nullptr; p.k_per = 0;
+    p.meta = d_in % 128 != 0 ? meta : nullptr; p.meta_pitch = d_in / 8;
     if (p.n1 + p.n2 == 0)             // s == 0 and no adapters: the result is zero
         return cudaMemsetAsync(Y, 0, (size_t)b * d_out * 2, st) == cudaSuccess ? SLIM_OK : SLIM_ERR_CUDA;
     note_token_tile(wide ? 256 : 64);
