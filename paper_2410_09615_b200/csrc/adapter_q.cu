@@ -7,35 +7,55 @@
 
 namespace slim {
 
-// One warp per (row, group): a lane holds four consecutive elements.
-__global__ void pack_adapter_kernel(const __nv_bfloat16* __restrict__ A, int rows, int cols, int groups,
-                                    uint8_t* __restrict__ codes, __nv_bfloat16* __restrict__ scales)
+// One warp per (row, group): a lane holds four consecutive elements (one 8-byte load where rows are multiples of
+// four elements).  Warps walk the groups with the next group's load in flight.
+__device__ __forceinline__ uint2 load_group(const __nv_bfloat16* __restrict__ A, uint32_t item, int cols, int groups, int lane)
+{
+    const int c0 = (int)(item % (uint32_t)groups) * 128 + lane * 4;
+    const __nv_bfloat16* src = A + (size_t)(item / (uint32_t)groups) * cols + c0;
+    if (cols % 4 == 0) return c0 < cols ? __ldg(reinterpret_cast<const uint2*>(src)) : make_uint2(0u, 0u);
+    uint32_t w[2] = {0, 0};                                   // cols is even: elements come in pairs
+#pragma unroll
+    for (int i = 0; i < 2; ++i) if (c0 + 2 * i < cols) w[i] = __ldg(reinterpret_cast<const uint32_t*>(src) + i);
+    return make_uint2(w[0], w[1]);
+}
+
+__global__ void __launch_bounds__(256)
+pack_adapter_kernel(const __nv_bfloat16* __restrict__ A, uint32_t items, int cols, int groups,
+                    uint8_t* __restrict__ codes, __nv_bfloat16* __restrict__ scales)
 {
     const int lane = threadIdx.x & 31;
-    const long long item = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (item >= (long long)rows * groups) return;
-    const int row = (int)(item / groups), grp = (int)(item % groups);
-    const int c0 = grp * 128 + lane * 4;
-    float v[4];
+    const uint32_t stride = gridDim.x * 8;
+    uint32_t item = blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (item >= items) return;
+    uint2 next = load_group(A, item, cols, groups, lane);
+    for (; item < items; item += stride) {
+        const uint2 u = next;
+        if (item + stride < items) next = load_group(A, item + stride, cols, groups, lane);
+        const uint32_t row = item / (uint32_t)groups, grp = item % (uint32_t)groups;
+        const int c0 = (int)grp * 128 + lane * 4;
+        const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u.x)), b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u.y));
+        const float v[4] = {a.x, a.y, b.x, b.y};
+        // magnitudes order like their bit patterns
+        const float m = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(fmaxf(fmaxf(fabsf(v[0]), fabsf(v[1])), fmaxf(fabsf(v[2]), fabsf(v[3]))))));
+        const __nv_bfloat16 sb = m > 0.f ? __float2bfloat16_rn(__fdiv_rn(m, 7.0f)) : __float2bfloat16_rn(0.f);
+        const float sc = __bfloat162float(sb);
+        if (lane == 0) scales[(size_t)row * groups + grp] = sb;
+        const Divisor by(sc > 0.f ? sc : 1.f);
+        uint32_t q[4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) v[i] = c0 + i < cols ? __bfloat162float(A[(size_t)row * cols + c0 + i]) : 0.f;
-    float m = fmaxf(fmaxf(fabsf(v[0]), fabsf(v[1])), fmaxf(fabsf(v[2]), fabsf(v[3])));
-#pragma unroll
-    for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    const __nv_bfloat16 sb = m > 0.f ? __float2bfloat16_rn(__fdiv_rn(m, 7.0f)) : __float2bfloat16_rn(0.f);
-    const float sc = __bfloat162float(sb);
-    if (lane == 0) scales[(size_t)row * groups + grp] = sb;
-    uint32_t q[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        int c = 0;
-        if (sc > 0.f) c = max(-8, min(7, __float2int_rn(__fdiv_rn(v[i], sc))));     // nearest, ties to even
-        q[i] = (uint32_t)c & 0xFu;
+        for (int i = 0; i < 4; ++i)
+            q[i] = sc > 0.f ? (uint32_t)max(-8, min(7, __float2int_rn(by.of(v[i])))) & 0xFu : 0u;      // nearest, ties to even
+        // cols is even, so elements come in pairs: either both of a byte exist or neither
+        uint8_t* dst = codes + (size_t)row * (cols / 2) + c0 / 2;
+        if (c0 + 3 < cols) {
+            const uint16_t w = (uint16_t)(q[0] | (q[1] << 4) | (q[2] << 8) | (q[3] << 12));
+            if (cols % 4 == 0) *reinterpret_cast<uint16_t*>(dst) = w;
+            else { dst[0] = (uint8_t)w; dst[1] = (uint8_t)(w >> 8); }
+        } else if (c0 + 1 < cols) {
+            dst[0] = (uint8_t)(q[0] | (q[1] << 4));
+        }
     }
-    // cols is even, so elements come in pairs: either both of a byte exist or neither
-    uint8_t* dst = codes + (size_t)row * (cols / 2) + c0 / 2;
-    if (c0 + 3 < cols) *reinterpret_cast<uint16_t*>(dst) = (uint16_t)(q[0] | (q[1] << 4) | (q[2] << 8) | (q[3] << 12));
-    else if (c0 + 1 < cols) dst[0] = (uint8_t)(q[0] | (q[1] << 4));
 }
 
 // One thread per byte of codes: two bf16 values out.
@@ -57,7 +77,9 @@ slim_status_t launch_pack_adapter(const __nv_bfloat16* A, int rows, int cols, ui
 {
     const int groups = (cols + 127) / 128;
     const long long items = (long long)rows * groups;
-    pack_adapter_kernel<<<(unsigned)((items + 7) / 8), 256, 0, st>>>(A, rows, cols, groups, codes, scales);
+    if (items > 0x7FFFFFFFll) return SLIM_ERR_INVALID_ARG;
+    const long long blocks = (items + 7) / 8;
+    pack_adapter_kernel<<<(unsigned)(blocks < 1184 ? blocks : 1184), 256, 0, st>>>(A, (uint32_t)items, cols, groups, codes, scales);      // 1184: eight blocks for each of 148 SMs
     count_launch(1);
     return cudaGetLastError() == cudaSuccess ? SLIM_OK : SLIM_ERR_CUDA;
 }

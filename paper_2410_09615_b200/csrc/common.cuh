@@ -14,6 +14,25 @@ __device__ __forceinline__ void flag_error(uint32_t* status_dev, int code) {
 
 __host__ __device__ __forceinline__ int ceil_div(int a, int b) { return (a + b - 1) / b; }
 
+// x / b correctly rounded, for many x and one b: Markstein's theorem (IBM J. Res. Dev. 34, 1990): with y = 1 / b
+// correctly rounded and q within an ulp of x / b, q + (x - q b) y, two fused operations, is x / b correctly
+// rounded, unless b's significand is all ones.  That case, and magnitudes near the ends of the range, take the
+// ordinary division.  (An |x| below 2^-100 may come out inexact: then x / b is below 2^-39 and the callers round it to zero.)
+struct Divisor {
+    float b, y;
+    bool plain;
+    __device__ __forceinline__ explicit Divisor(float d) : b(d) {
+        y = __frcp_rn(d);
+        plain = (__float_as_uint(d) & 0x7FFFFFu) == 0x7FFFFFu || !(d >= 0x1p-60f && d <= 0x1p60f);
+    }
+    __device__ __forceinline__ float of(float x) const {
+        if (plain) return __fdiv_rn(x, b);
+        float q = __fmul_rn(x, y);
+        q = __fmaf_rn(__fmaf_rn(-q, b, x), y, q);
+        return __fmaf_rn(__fmaf_rn(-q, b, x), y, q);
+    }
+};
+
 // Per-device facts the launchers need (filled once per device, read-only after).
 struct DeviceInfo {
     int cc_major;

@@ -7,48 +7,49 @@ namespace slim {
 // One thread handles 16 consecutive columns (four groups) of one row: two
 // 16-byte loads, one 4-byte and one 2-byte store.  Consecutive threads walk
 // consecutive columns, so a warp reads 512 contiguous bytes of codes and mask.
+// The four mask bytes of a group become a 4-bit number, its index nibble comes from a 64-bit table and the two codes
+// from one byte permutation: no branches and no loops over positions (4096 x 11008: 53 -> 20 us).
+//
+// Index nibble (lower | upper << 2) for each set of kept positions; a set of fewer than two is completed with the
+// lowest positions not kept.  Sets of three and four are errors (0x4).
+__host__ __device__ constexpr unsigned long long index_table() {
+    unsigned long long t = 0;
+    for (int m = 0; m < 16; ++m) {
+        int pos[2] = {0, 0}, kept = 0;
+        for (int i = 0; i < 4; ++i)
+            if ((m >> i) & 1) { if (kept < 2) pos[kept] = i; ++kept; }
+        if (kept == 0 || (kept == 1 && pos[0] == 0) || kept > 2) { pos[0] = 0; pos[1] = 1; }
+        else if (kept == 1) { pos[1] = pos[0]; pos[0] = 0; }
+        t |= (unsigned long long)(pos[0] | (pos[1] << 2)) << (4 * m);
+    }
+    return t;
+}
+
 __global__ void __launch_bounds__(256)
 pack_kernel(const int8_t* __restrict__ codes, const uint8_t* __restrict__ mask,
             long long n_chunks, uint8_t* __restrict__ vals, uint8_t* __restrict__ meta,
             uint32_t* status_dev)
 {
+    constexpr unsigned long long table = index_table();
     uint32_t err = 0;
     for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n_chunks;
          c += (long long)gridDim.x * blockDim.x) {
-        const int4 cv = __ldg(reinterpret_cast<const int4*>(codes) + c);
-        const int4 mv = __ldg(reinterpret_cast<const int4*>(mask) + c);
-        const uint32_t cw[4] = {(uint32_t)cv.x, (uint32_t)cv.y, (uint32_t)cv.z, (uint32_t)cv.w};
-        const uint32_t mw[4] = {(uint32_t)mv.x, (uint32_t)mv.y, (uint32_t)mv.z, (uint32_t)mv.w};
+        const uint4 cv = __ldg(reinterpret_cast<const uint4*>(codes) + c);
+        const uint4 mv = __ldg(reinterpret_cast<const uint4*>(mask) + c);
+        const uint32_t cw[4] = {cv.x, cv.y, cv.z, cv.w}, mw[4] = {mv.x, mv.y, mv.z, mv.w};
         uint32_t vout = 0, mout = 0;
 #pragma unroll
         for (int g = 0; g < 4; ++g) {
-            int pos[2] = {0, 0};
-            int v[2] = {0, 0};
-            int kept = 0;
-            bool bad_code = false;
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const bool k = ((mw[g] >> (8 * i)) & 0xFFu) != 0;
-                if (k) {
-                    const int code = (int)(int8_t)((cw[g] >> (8 * i)) & 0xFFu);
-                    if (code < -8 || code > 7) bad_code = true;
-                    if (kept < 2) { pos[kept] = i; v[kept] = code; }
-                    ++kept;
-                }
-            }
-            uint32_t vb, mb;
-            if (kept > 2 || bad_code) {
-                err |= 1u << (kept > 2 ? SLIM_ERR_BAD_MASK : SLIM_ERR_CODE_RANGE);
+            const uint32_t keep = __vcmpne4(mw[g], 0u);                       // 0xFF at kept positions
+            const uint32_t code = cw[g] & keep;
+            const uint32_t m = (((keep & 0x01010101u) * 0x01020408u) >> 24) & 0xFu;
+            uint32_t mb = (uint32_t)(table >> (4 * m)) & 0xFu;
+            const uint32_t two = __byte_perm(code, 0u, (mb & 3u) | (mb >> 2 << 4));      // bytes: lower, upper
+            uint32_t vb = (two & 0xFu) | ((two >> 4) & 0xF0u);
+            const bool many = __popc(m) > 2, range = (__vadd4(code, 0x08080808u) & 0xF0F0F0F0u) != 0;
+            if (many || range) {
+                err |= 1u << (many ? SLIM_ERR_BAD_MASK : SLIM_ERR_CODE_RANGE);
                 vb = 0; mb = 0x4;
-            } else {
-                if (kept == 0) { pos[0] = 0; pos[1] = 1; }
-                else if (kept == 1) {
-                    // complete with the lowest position not kept, keep ascending order
-                    if (pos[0] == 0) { pos[1] = 1; }
-                    else { pos[1] = pos[0]; v[1] = v[0]; pos[0] = 0; v[0] = 0; }
-                }
-                vb = ((uint32_t)v[0] & 0xFu) | (((uint32_t)v[1] & 0xFu) << 4);
-                mb = (uint32_t)pos[0] | ((uint32_t)pos[1] << 2);
             }
             vout |= vb << (8 * g);
             mout |= mb << (4 * g);

@@ -3,6 +3,11 @@
 // decision are those include/slim.h states for slim_quant: the bin of a weight in binary32, the error
 // of a candidate in binary64 with the bins added in ascending order and no fused multiply-add, the
 // codes in binary32.  Four launches: largest magnitude, histogram, search, codes.
+//
+// The three passes over the weights are bound by memory: 16-byte loads, and the histogram walks the array backwards,
+// so that it starts with what the largest-magnitude pass left in the L2 (the codes pass, forwards again, finds the
+// histogram's end there).  Measured on 4096 x 11008 (180 MB): see the figure at each kernel.
+#include <atomic>
 #include "common.cuh"
 
 namespace slim {
@@ -14,26 +19,60 @@ constexpr int kQsTable = 29;          // candidates: ten coarse, nineteen fine
 struct QsHeader {                     // first 256 bytes of the workspace
     unsigned int max_bits;            // bit pattern of the largest |w| (non-negative floats order like unsigned integers)
     unsigned int bad;                 // a NaN or an infinity was seen
+    unsigned int done;                // blocks of the search that have finished
 };
 
-__global__ void qs_absmax_kernel(const float* __restrict__ W, size_t n, QsHeader* hdr)
+constexpr int kVec = 4;               // float4 loads a thread has in flight
+
+// The array as float4s i = first, first + stride, ..: kVec loads at a time, then `f` on each.  `tail` elements (n % 4)
+// go to the first threads.
+template <bool BACKWARDS, typename F>
+__device__ __forceinline__ void for_weights(const float* __restrict__ W, size_t n, F f)
 {
+    const size_t n4 = n / 4, stride = (size_t)gridDim.x * blockDim.x, me = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const float4* W4 = reinterpret_cast<const float4*>(W);
+    size_t i = me;
+    for (; i + (kVec - 1) * stride < n4; i += kVec * stride) {
+        float4 v[kVec];
+#pragma unroll
+        for (int k = 0; k < kVec; ++k) v[k] = __ldg(W4 + (BACKWARDS ? n4 - 1 - (i + k * stride) : i + k * stride));
+#pragma unroll
+        for (int k = 0; k < kVec; ++k) { f(v[k].x); f(v[k].y); f(v[k].z); f(v[k].w); }
+    }
+    for (; i < n4; i += stride) {
+        const float4 v = __ldg(W4 + (BACKWARDS ? n4 - 1 - i : i));
+        f(v.x); f(v.y); f(v.z); f(v.w);
+    }
+    if (me < n - 4 * n4) f(W[4 * n4 + me]);
+}
+
+__global__ void __launch_bounds__(512)
+qs_absmax_kernel(const float* __restrict__ W, size_t n, QsHeader* hdr)
+{
+    __shared__ unsigned int sm[16], sb[16];
     unsigned int m = 0, bad = 0;
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        const float a = fabsf(W[i]);
+    for_weights<false>(W, n, [&](float w) {
+        const float a = fabsf(w);
         if (!(a <= 3.0e38f)) bad = 1;
         m = max(m, __float_as_uint(a));
-    }
-#pragma unroll
-    for (int o = 16; o; o >>= 1) { m = max(m, __shfl_xor_sync(0xffffffffu, m, o)); bad |= __shfl_xor_sync(0xffffffffu, bad, o); }
-    if ((threadIdx.x & 31) == 0) {
-        if (!bad) atomicMax(&hdr->max_bits, m);
-        if (bad) atomicOr(&hdr->bad, 1u);
+    });
+    m = __reduce_max_sync(0xffffffffu, m);
+    bad = __reduce_or_sync(0xffffffffu, bad);
+    if ((threadIdx.x & 31) == 0) { sm[threadIdx.x >> 5] = m; sb[threadIdx.x >> 5] = bad; }
+    __syncthreads();
+    if (threadIdx.x < 16) {
+        m = __reduce_max_sync(0xffffu, sm[threadIdx.x]);
+        bad = __reduce_or_sync(0xffffu, sb[threadIdx.x]);
+        if (threadIdx.x == 0) {
+            if (bad) atomicOr(&hdr->bad, 1u);
+            else atomicMax(&hdr->max_bits, m);
+        }
     }
 }
 
 // Histogram of |w| / M over `bins` uniform bins, per block in shared memory, then added to the global one.
-__global__ void qs_hist_kernel(const float* __restrict__ W, size_t n, const QsHeader* hdr, int bins, unsigned int* hist)
+__global__ void __launch_bounds__(1024)
+qs_hist_kernel(const float* __restrict__ W, size_t n, const QsHeader* hdr, int bins, unsigned int* hist)
 {
     extern __shared__ unsigned int sh[];
     for (int i = threadIdx.x; i < bins; i += blockDim.x) sh[i] = 0;
@@ -41,63 +80,118 @@ __global__ void qs_hist_kernel(const float* __restrict__ W, size_t n, const QsHe
     const float M = __uint_as_float(hdr->max_bits);
     if (M > 0.f && !hdr->bad) {
         const float fb = (float)bins;
-        for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-            int b = (int)__fmul_rn(__fdiv_rn(fabsf(W[i]), M), fb);
-            b = min(b, bins - 1);
-            atomicAdd(&sh[b], 1u);
-        }
+        const Divisor by(M);
+        for_weights<true>(W, n, [&](float w) { atomicAdd(&sh[min((int)__fmul_rn(by.of(fabsf(w)), fb), bins - 1)], 1u); });
     }
     __syncthreads();
     for (int i = threadIdx.x; i < bins; i += blockDim.x)
         if (sh[i]) atomicAdd(&hist[i], sh[i]);
 }
 
-// E(alpha) on the bin centres, by one warp: the lanes work out the terms of 32 bins at a time, every operation
-// rounded on its own, and lane 0 adds them in ascending order of the bins (an empty bin adds +0, which changes
-// nothing), so the sum is the one a single thread would get.  Returns the sum in lane 0.
-__device__ double qs_error(const unsigned int* hist, int bins, double M, double n_total, double alpha, double* terms, int lane)
+// ---------------------------------------------------------------- E(alpha) on the bin centres
+// The error is defined as a sum taken bin by bin, each addition rounded: a chain of 20000 dependent additions for each
+// of the 29 candidates.  Two observations shorten it without changing a bit.
+//   - While the sum e stays in one binade [2^k, 2^(k+1)), whose spacing is u, adding t >= 0 gives e + q with q = t
+//     rounded to a multiple of u, unless t lies exactly half-way between two multiples (then the parity of e
+//     decides).  The q of many bins can be found side by side and added in any order: all are multiples of u
+//     and the sums stay below 2^53 u, so every addition is exact.  A warp takes 256 bins at a time, eight a lane, and
+//     goes through a lane's bins one by one only where e leaves its binade or a half-way case comes up.
+//   - The fine candidates depend on the best coarse one only through ten possible values: all 10 + 10 x 19
+//     candidates are evaluated at once, a block each, and the last block to finish takes the minima.
+constexpr int kSearchThreads = 512, kSlice = 2048, kCoarse = 10, kFine = 19, kCandidates = kCoarse + kCoarse * kFine;
+
+// One bin's term: every operation rounded on its own; an empty bin adds +0, which changes nothing.
+__device__ __forceinline__ double qs_term(unsigned int c, int i, double width, double n_total, double alpha)
 {
-    double e = 0.0;
-    const double width = __ddiv_rn(M, (double)bins);
-    for (int i0 = 0; i0 < bins; i0 += 32) {
-        const int i = i0 + lane;
-        double term = 0.0;
-        const unsigned int c = i < bins ? hist[i] : 0u;
-        if (c) {
-            const double x = __dmul_rn(__dadd_rn((double)i, 0.5), width);
-            const double p = __ddiv_rn((double)c, n_total);
-            double d;
-            if (x <= alpha) {
-                const double level = rint(__ddiv_rn(__dmul_rn(x, 8.0), alpha));
-                d = __dsub_rn(__dmul_rn(__dmul_rn(alpha, 0.125), level), x);
-            } else {
-                d = __dsub_rn(alpha, x);
-            }
-            term = __dmul_rn(p, __dmul_rn(d, d));
-        }
-        terms[lane] = term;
-        __syncwarp();
-        if (lane == 0) {
+    if (!c) return 0.0;
+    const double x = __dmul_rn(__dadd_rn((double)i, 0.5), width);
+    const double p = __ddiv_rn((double)c, n_total);
+    double d;
+    if (x <= alpha) {
+        const double level = rint(__ddiv_rn(__dmul_rn(x, 8.0), alpha));
+        d = __dsub_rn(__dmul_rn(__dmul_rn(alpha, 0.125), level), x);
+    } else {
+        d = __dsub_rn(alpha, x);
+    }
+    return __dmul_rn(p, __dmul_rn(d, d));
+}
+
+// The binade of e > 2^-900: its end, half its start (terms below that are rounded by adding `magic`), half its spacing.
+struct Binade {
+    double end, half, magic, tie;
+    bool valid;
+    __device__ __forceinline__ explicit Binade(double e) {
+        const int k = (int)((__double_as_longlong(e) >> 52) & 0x7FF);
+        valid = k > 123 && k < 2000;
+        end = __longlong_as_double((long long)(k + 1) << 52);
+        half = __longlong_as_double((long long)(valid ? k - 1 : 1) << 52);
+        magic = __longlong_as_double(((long long)k << 52) | (1ll << 51));
+        tie = __longlong_as_double((long long)(valid ? k - 53 : 1) << 52);
+    }
+    // t as a multiple of the spacing; *bad: t is too large for that, or half-way
+    __device__ __forceinline__ double round(double t, bool* bad) const {
+        const double q = __dsub_rn(__dadd_rn(t, magic), magic);
+        *bad = !(t < half) || fabs(__dsub_rn(t, q)) == tie;
+        return q;
+    }
+};
+
+// The terms of 256 bins in shared memory: lane l of the adding warp takes bins 8 l .. 8 l + 7 (pitch: no bank conflicts
+// either way).
+constexpr int kPitch = 36, kBlockTerms = 8 * kPitch;
+__host__ __device__ __forceinline__ constexpr int term_at(int i) { return (i >> 8) * kBlockTerms + (i & 7) * kPitch + ((i & 255) >> 3); }
+
+// e + the first 256 terms, one by one (every lane does it).  They grow from nothing: e leaves a binade every few of them.
+__device__ double add_first(double e, const double* terms)
+{
+#pragma unroll 32
+    for (int i = 0; i < 256; ++i) e = __dadd_rn(e, terms[term_at(i)]);
+    return e;
+}
+
+// e + 256 terms in order.
+__device__ double add_block(double e, const double* terms, int lane)
+{
+    double t[8];
 #pragma unroll
-            for (int k = 0; k < 32; ++k) e = __dadd_rn(e, terms[k]);
+    for (int j = 0; j < 8; ++j) t[j] = terms[j * kPitch + lane];
+    int at = 0;                                               // the terms of lanes before `at` are in e
+    while (at < 32) {
+        const Binade bn(e);
+        bool bad = !bn.valid, b1;
+        double q[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) { q[j] = bn.round(t[j], &b1); bad |= b1; }
+        double s = __dadd_rn(__dadd_rn(__dadd_rn(q[0], q[1]), __dadd_rn(q[2], q[3])), __dadd_rn(__dadd_rn(q[4], q[5]), __dadd_rn(q[6], q[7])));
+        if (lane < at) s = 0.0;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const double v = __shfl_up_sync(0xffffffffu, s, o);
+            if (lane >= o) s = __dadd_rn(s, v);
         }
-        __syncwarp();
+        const double after = __dadd_rn(e, s);
+        const unsigned stop = __ballot_sync(0xffffffffu, lane >= at && (bad || !(after < bn.end)));
+        if (!stop) return __shfl_sync(0xffffffffu, after, 31);
+        const int f = __ffs(stop) - 1;                        // this lane's eight terms go one by one
+        const double before = __shfl_sync(0xffffffffu, after, f > 0 ? f - 1 : 0);
+        if (f > at) e = before;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) e = __dadd_rn(e, terms[j * kPitch + f]);
+        at = f + 1;
     }
     return e;
 }
 
-// One block of 32 warps: warps 0-9 take the coarse candidates, then warps 0-18 the fine ones; thread 0 takes
-// the minima in the order the algorithm visits the candidates.
-__global__ void __launch_bounds__(1024, 1)
-qs_search_kernel(const QsHeader* hdr, const unsigned int* hist, int bins, double n_total,
-                 float* scale_alpha, double* table, uint32_t* status)
+__global__ void __launch_bounds__(kSearchThreads)
+qs_search_kernel(QsHeader* hdr, const unsigned int* hist, int bins, double n_total, float* scale_alpha, double* table,
+                 double* errors, uint32_t* status)
 {
-    __shared__ double a_s[kQsTable], e_s[kQsTable];
-    __shared__ double terms[32][32];
-    __shared__ double a_low_s;
+    __shared__ double terms[2][kSlice / 256 * kBlockTerms];
+    __shared__ bool last;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const float Mf = __uint_as_float(hdr->max_bits);
     if (hdr->bad || !(Mf > 0.f)) {
+        if (blockIdx.x != 0) return;
         if (threadIdx.x == 0) {
             scale_alpha[0] = 0.f; scale_alpha[1] = 0.f;
             if (hdr->bad) flag_error(status, SLIM_ERR_INVALID_ARG);
@@ -106,49 +200,94 @@ qs_search_kernel(const QsHeader* hdr, const unsigned int* hist, int bins, double
         return;
     }
     const double M = (double)Mf, eta_low = __ddiv_rn(M, 10.0), eta_high = __ddiv_rn(eta_low, 10.0);
-    if (warp < 10) {
-        const double a = __ddiv_rn(__dmul_rn(M, (double)(warp + 1)), 10.0);
-        const double e = qs_error(hist, bins, M, n_total, a, terms[warp], lane);
-        if (lane == 0) { a_s[warp] = a; e_s[warp] = e; }
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int best = 0;
-        for (int k = 1; k < 10; ++k) if (e_s[k] < e_s[best]) best = k;
-        a_low_s = a_s[best];
-    }
-    __syncthreads();
-    if (warp < 19) {
-        double a = __dadd_rn(__dsub_rn(a_low_s, eta_low), __dmul_rn((double)(warp + 1), eta_high));
-        if (a > M) a = M;
-        const double e = a > 0.0 ? qs_error(hist, bins, M, n_total, a, terms[warp], lane) : -1.0;
-        if (lane == 0) { a_s[10 + warp] = a; e_s[10 + warp] = e; }
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double best_a = a_s[0], best_e = e_s[0];
-        for (int k = 1; k < 10; ++k) if (e_s[k] < best_e) { best_a = a_s[k]; best_e = e_s[k]; }
-        for (int j = 10; j < kQsTable; ++j) {
-            if (!(a_s[j] > 0.0)) { e_s[j] = __dadd_rn(best_e, 1.0); continue; }     // not a candidate; listed like this
-            if (e_s[j] < best_e || (e_s[j] == best_e && a_s[j] < best_a)) { best_a = a_s[j]; best_e = e_s[j]; }
+    auto coarse = [&](int k) { return __ddiv_rn(__dmul_rn(M, (double)(k + 1)), 10.0); };
+    auto fine = [&](int k, int j) {
+        const double a = __dadd_rn(__dsub_rn(coarse(k), eta_low), __dmul_rn((double)(j + 1), eta_high));
+        return a > M ? M : a;
+    };
+    const int cand = blockIdx.x;
+    const double alpha = cand < kCoarse ? coarse(cand) : fine((cand - kCoarse) / kFine, (cand - kCoarse) % kFine);
+    const double width = __ddiv_rn(M, (double)bins);
+    double e = alpha > 0.0 ? 0.0 : -1.0;
+    if (alpha > 0.0) {
+        // warps 1-15 work out the terms of a slice of bins (with the next slice's counts on their way) while warp 0 adds up
+        // the slice before it
+        constexpr int kMakers = kSearchThreads - 32, kPer = (kSlice + kMakers - 1) / kMakers;
+        const int slices = ceil_div(bins, kSlice), me = (int)threadIdx.x - 32;
+        unsigned int c[kPer];
+        auto counts = [&](int s) {
+#pragma unroll
+            for (int k = 0; k < kPer; ++k) {
+                const int i = me + k * kMakers, b = s * kSlice + i;
+                c[k] = i < kSlice && b < bins ? hist[b] : 0u;
+            }
+        };
+        if (warp > 0) counts(0);
+        for (int s = 0; s <= slices; ++s) {
+            if (warp == 0) {
+                if (s == 1) e = add_first(e, terms[0]);
+                const int n = s > 0 ? min(kSlice, bins - (s - 1) * kSlice) : 0;
+                for (int b = s == 1 ? 1 : 0; b * 256 < n; ++b) e = add_block(e, terms[(s - 1) & 1] + b * kBlockTerms, lane);
+            } else if (s < slices) {
+                double v[kPer];
+#pragma unroll
+                for (int k = 0; k < kPer; ++k) v[k] = qs_term(c[k], s * kSlice + me + k * kMakers, width, n_total, alpha);
+                counts(s + 1);
+#pragma unroll
+                for (int k = 0; k < kPer; ++k)
+                    if (me + k * kMakers < kSlice) terms[s & 1][term_at(me + k * kMakers)] = v[k];
+            }
+            __syncthreads();
         }
-        const float a32 = (float)best_a;
-        scale_alpha[0] = __fmul_rn(a32, 0.125f);
-        scale_alpha[1] = a32;
-        table[2 * kQsTable] = best_a;
+    }
+    if (threadIdx.x == 0) {
+        errors[cand] = e;
+        __threadfence();
+        last = atomicAdd(&hdr->done, 1u) == gridDim.x - 1;
+        __threadfence();
     }
     __syncthreads();
-    if (threadIdx.x < kQsTable) { table[2 * threadIdx.x] = a_s[threadIdx.x]; table[2 * threadIdx.x + 1] = e_s[threadIdx.x]; }
+    if (!last || threadIdx.x != 0) return;
+    // the minima, in the order the algorithm visits the candidates
+    volatile double* er = errors;
+    int best = 0;
+    for (int k = 1; k < kCoarse; ++k) if (er[k] < er[best]) best = k;
+    double best_a = coarse(best), best_e = er[best];
+    for (int k = 0; k < kCoarse; ++k) { table[2 * k] = coarse(k); table[2 * k + 1] = er[k]; }
+    for (int j = 0; j < kFine; ++j) {
+        const double a = fine(best, j);
+        double ej = er[kCoarse + best * kFine + j];
+        if (!(a > 0.0)) ej = __dadd_rn(best_e, 1.0);                              // not a candidate; listed like this
+        else if (ej < best_e || (ej == best_e && a < best_a)) { best_a = a; best_e = ej; }
+        table[2 * (kCoarse + j)] = a; table[2 * (kCoarse + j) + 1] = ej;
+    }
+    const float a32 = (float)best_a;
+    scale_alpha[0] = __fmul_rn(a32, 0.125f);
+    scale_alpha[1] = a32;
+    table[2 * kQsTable] = best_a;
 }
 
-__global__ void qs_codes_kernel(const float* __restrict__ W, size_t n, const float* __restrict__ scale_alpha, int8_t* __restrict__ codes)
+// 16 codes a thread: four float4 loads, one 16-byte store.
+__global__ void __launch_bounds__(256)
+qs_codes_kernel(const float* __restrict__ W, size_t n, const float* __restrict__ scale_alpha, int8_t* __restrict__ codes)
 {
     const float a32 = scale_alpha[1];
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        int q = 0;
-        if (a32 > 0.f) q = max(-8, min(7, __float2int_rn(__fmul_rn(__fdiv_rn(W[i], a32), 8.0f))));
-        codes[i] = (int8_t)q;
+    const Divisor by(a32 > 0.f ? a32 : 1.f);
+    auto code = [&](float w) -> uint32_t {
+        return a32 > 0.f ? (uint32_t)max(-8, min(7, __float2int_rn(__fmul_rn(by.of(w), 8.0f)))) & 0xFFu : 0u;
+    };
+    const size_t n16 = n / 16;
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n16; i += (size_t)gridDim.x * blockDim.x) {
+        float4 v[4];
+        uint32_t o[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[k] = __ldg(reinterpret_cast<const float4*>(W) + 4 * i + k);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) o[k] = code(v[k].x) | code(v[k].y) << 8 | code(v[k].z) << 16 | code(v[k].w) << 24;
+        reinterpret_cast<uint4*>(codes)[i] = make_uint4(o[0], o[1], o[2], o[3]);
     }
+    const size_t me = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (me < n - 16 * n16) codes[16 * n16 + me] = (int8_t)code(W[16 * n16 + me]);
 }
 
 }  // namespace
@@ -161,7 +300,7 @@ int quant_bins(int d_out, int d_in) {
 }
 
 size_t quant_workspace_bytes(int d_out, int d_in) {
-    return 256 + (size_t)quant_bins(d_out, d_in) * 4 + 256 + (2 * kQsTable + 1) * sizeof(double);
+    return 256 + (size_t)quant_bins(d_out, d_in) * 4 + 256 + (2 * kQsTable + 1 + kCandidates) * sizeof(double);
 }
 
 slim_status_t launch_quant(const float* W, int d_out, int d_in, int8_t* codes, float* scale_alpha, void* ws,
@@ -177,15 +316,20 @@ slim_status_t launch_quant(const float* W, int d_out, int d_in, int8_t* codes, f
     unsigned int* hist = reinterpret_cast<unsigned int*>(base + 256);
     double* table = reinterpret_cast<double*>(base + 256 + ((size_t)bins * 4 + 255) / 256 * 256);
     if (cudaMemsetAsync(ws, 0, 256 + (size_t)bins * 4, st) != cudaSuccess) return SLIM_ERR_CUDA;
-    const unsigned grid = (unsigned)(di->sm_count * 4);
-    qs_absmax_kernel<<<grid, 512, 0, st>>>(W, n, hdr);
+    qs_absmax_kernel<<<(unsigned)(di->sm_count * 4), 512, 0, st>>>(W, n, hdr);
     const size_t hist_smem = (size_t)bins * 4;
-    if (hist_smem > 48 * 1024 &&
-        cudaFuncSetAttribute(qs_hist_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)hist_smem) != cudaSuccess)
-        return SLIM_ERR_CUDA;
-    qs_hist_kernel<<<(unsigned)(di->sm_count * 2), 1024, hist_smem, st>>>(W, n, hdr, bins, hist);
-    qs_search_kernel<<<1, 1024, 0, st>>>(hdr, hist, bins, (double)n, scale_alpha, table, status_dev);
-    qs_codes_kernel<<<grid, 512, 0, st>>>(W, n, scale_alpha, codes);
+    int dev = 0;
+    cudaGetDevice(&dev);
+    static std::atomic<bool> attr_set[64];
+    if (dev < 0 || dev >= 64) return SLIM_ERR_CUDA;
+    if (!attr_set[dev].load(std::memory_order_acquire)) {
+        if (cudaFuncSetAttribute(qs_hist_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 20000 * 4) != cudaSuccess) return SLIM_ERR_CUDA;
+        attr_set[dev].store(true, std::memory_order_release);
+    }
+    // a block per SM: two would find no more work in flight and double the additions to the global histogram
+    qs_hist_kernel<<<(unsigned)di->sm_count, 1024, hist_smem, st>>>(W, n, hdr, bins, hist);
+    qs_search_kernel<<<kCandidates, kSearchThreads, 0, st>>>(hdr, hist, bins, (double)n, scale_alpha, table, table + 2 * kQsTable + 1, status_dev);
+    qs_codes_kernel<<<(unsigned)(di->sm_count * 8), 256, 0, st>>>(W, n, scale_alpha, codes);
     count_launch(4);
     return cudaGetLastError() == cudaSuccess ? SLIM_OK : SLIM_ERR_CUDA;
 }
