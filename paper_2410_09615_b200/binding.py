@@ -2,8 +2,8 @@
 
 Argument marshalling only: tensors are torch CUDA tensors (torch supplies device
 memory and streams), every step of the computation runs in the library's
-kernels.  The forward entry points go through the compiled call path of
-``csrc/native.cpp``, everything else through ctypes.  If a library is missing or a
+kernels.  The entry points that a layer's compression and forward call go through the
+compiled call path of ``csrc/native.cpp``, everything else through ctypes.  If a library is missing or a
 call fails, a :class:`SlimError` is raised; there is no fallback path.
 """
 from __future__ import annotations
@@ -97,7 +97,8 @@ def native():
         m = importlib.util.module_from_spec(spec)
         spec.loader.exec_module(m)
         m.bind(SlimError, *[ctypes.cast(getattr(lib(), name), ctypes.c_void_p).value for name in
-                            ("slim_linear_fwd_ex", "slim_linear_fwd_tiled", "slim_linear_fwd_q", "slim_tiled_bytes", "slim_strerror")])
+                            ("slim_linear_fwd_ex", "slim_linear_fwd_tiled", "slim_linear_fwd_q", "slim_tiled_bytes", "slim_strerror",
+                             "slim_pack", "slim_quant", "slim_quant_workspace_bytes", "slim_mask_top2", "slim_pack_adapter")])
         _native = m
     return _native
 
@@ -145,21 +146,9 @@ def raise_on_status(bits: int, where: str):
 
 
 def slim_pack(codes: torch.Tensor, mask: torch.Tensor, vals=None, meta=None, status=None, check=True):
-    """codes int8 [d_out, d_in], mask uint8 [d_out, d_in] -> (vals, meta) uint8 tensors."""
-    _dev(codes, torch.int8, "codes"), _dev(mask, torch.uint8, "mask")
-    d_out, d_in = codes.shape
-    if vals is None:
-        vals = torch.empty((d_out, d_in // 4), dtype=torch.uint8, device=codes.device)
-    if meta is None:
-        meta = torch.empty((d_out, d_in // 8), dtype=torch.uint8, device=codes.device)
-    own_status = status is None and check
-    if own_status:
-        status = torch.zeros(1, dtype=torch.int32, device=codes.device)
-    _check(lib().slim_pack(_ptr(codes), _ptr(mask), d_out, d_in, _ptr(vals), _ptr(meta), _ptr(status), _stream()),
-           "slim_pack")
-    if own_status:
-        raise_on_status(read_status(status), "slim_pack")
-    return vals, meta
+    """codes int8 [d_out, d_in], mask uint8 [d_out, d_in] -> (vals, meta) uint8 tensors.  With ``check`` and no
+    ``status`` the call waits for the GPU and raises on a bad group; else errors are in the caller's ``status``."""
+    return (_native or native()).pack(codes, mask, vals, meta, status, check)
 
 
 def slim_unpack(vals: torch.Tensor, meta: torch.Tensor, want_mask=True):
@@ -295,14 +284,7 @@ def slim_linear_fwd_noalloc(X, vals, meta, s: float, L, R, Y, status=None):
 
 def slim_pack_adapter(A: torch.Tensor):
     """bf16 adapter [rows, cols] -> (codes uint8 [rows, cols / 2], scales bf16 [rows, ceil(cols / 128)])."""
-    _dev(A, torch.bfloat16, "A")
-    rows, cols = A.shape
-    if lib().slim_adapter_code_bytes(rows, cols) == 0:
-        raise SlimError(SLIM_ERR_INVALID_ARG, "slim_pack_adapter", "illegal adapter shape")
-    codes = torch.empty((rows, cols // 2), dtype=torch.uint8, device=A.device)
-    scales = torch.empty((rows, (cols + 127) // 128), dtype=torch.bfloat16, device=A.device)
-    _check(lib().slim_pack_adapter(_ptr(A), rows, cols, _ptr(codes), _ptr(scales), _stream()), "slim_pack_adapter")
-    return codes, scales
+    return (_native or native()).pack_adapter(A)
 
 
 def slim_unpack_adapter(codes: torch.Tensor, scales: torch.Tensor) -> torch.Tensor:
@@ -334,25 +316,9 @@ def slim_linear_fwd_q(X, vals, meta, s: float, Lq, Ls, Rq, Rs, Y=None, workspace
 def slim_quant(W: torch.Tensor, status=None):
     """SLiM-Quant on a float32 matrix: (codes int8 like W, scale_alpha float32[2] on the device = (s, alpha*),
     table float64 [29, 2] of the candidates tried, alpha* as float64)."""
-    _dev(W, torch.float32, "W")
-    d_out, d_in = W.shape
-    n = int(lib().slim_quant_workspace_bytes(d_out, d_in))
-    ws = torch.empty(n, dtype=torch.uint8, device=W.device)
-    codes = torch.empty((d_out, d_in), dtype=torch.int8, device=W.device)
-    sa = torch.empty(4, dtype=torch.float32, device=W.device)
-    _check(lib().slim_quant(_ptr(W), d_out, d_in, _ptr(codes), _ptr(sa), _ptr(ws), n, _ptr(status), _stream()), "slim_quant")
-    bins = max(512, min(d_out * d_in // 1000, 20000))
-    off = 256 + (bins * 4 + 255) // 256 * 256
-    tab = ws[off:off + 59 * 8].view(torch.float64)
-    return codes, sa[:2], tab[:58].view(29, 2), tab[58]
+    return (_native or native()).quant(W, status)
 
 
 def slim_mask_top2(codes: torch.Tensor, xbar=None, status=None) -> torch.Tensor:
     """2:4 mask (uint8, like codes) of int8 codes; xbar: float32 [d_in] average input magnitudes, or None."""
-    _dev(codes, torch.int8, "codes")
-    d_out, d_in = codes.shape
-    if xbar is not None:
-        _dev(xbar, torch.float32, "xbar")
-    mask = torch.empty((d_out, d_in), dtype=torch.uint8, device=codes.device)
-    _check(lib().slim_mask_top2(_ptr(codes), _ptr(xbar), d_out, d_in, _ptr(mask), _ptr(status), _stream()), "slim_mask_top2")
-    return mask
+    return (_native or native()).mask_top2(codes, xbar, status)

@@ -23,6 +23,14 @@ def _stale() -> bool:
     return _older(LIB, [os.path.join(CSRC, f) for f in os.listdir(CSRC) if not f.endswith(".cpp")] + [os.path.join(INCLUDE, "slim.h")])
 
 
+def _cudart(torch_root: str):
+    """The CUDA runtime that torch itself has loaded, by its file name (the module shares its context and streams)."""
+    import glob
+    near = glob.glob(os.path.join(os.path.dirname(torch_root), "nvidia", "cuda_runtime", "lib", "libcudart.so*"))
+    lib = near[0] if near else "/usr/local/cuda/lib64/libcudart.so"
+    return ["-L" + os.path.dirname(lib), "-l:" + os.path.basename(lib)]
+
+
 def build_native(force: bool = False) -> str:
     """Compile ``csrc/native.cpp`` into ``_slim_native.so`` (for the interpreter and the torch that run this)."""
     src = os.path.join(CSRC, "native.cpp")
@@ -36,7 +44,7 @@ def build_native(force: bool = False) -> str:
     tmp = NATIVE + f".tmp{os.getpid()}"
     subprocess.check_call(["g++", "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
                            *[f"-I{d}" for d in dirs], src, "-o", tmp, "-L" + os.path.join(root, "lib"), "-ltorch_python", "-ltorch",
-                           "-ltorch_cpu", "-ltorch_cuda", "-lc10", "-lc10_cuda"])
+                           "-ltorch_cpu", "-ltorch_cuda", "-lc10", "-lc10_cuda", *_cudart(root)])
     os.replace(tmp, NATIVE)
     return NATIVE
 

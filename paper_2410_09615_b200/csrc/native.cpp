@@ -1,12 +1,16 @@
-// Call path of the forward entry points from Python: argument checks, the output tensor, the current stream and
+// Call path of the entry points from Python: argument checks, the output tensors, the current stream and
 // the call into libslim, without interpreted code in between.  A small-batch call takes the GPU about as long as
 // one launch takes the host, so the path from the interpreter to the launch is part of its time: through ctypes and
 // per-argument Python checks a call took the host 22-23 us, this way 4-8 (three to four of them the launch).
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 #include <ATen/ATen.h>
 #include <ATen/cuda/EmptyTensor.h>
 #include <c10/cuda/CUDAStream.h>
+#include <cuda_runtime.h>
+#include <algorithm>
 #include <cstdint>
+#include <mutex>
 
 namespace {
 
@@ -17,12 +21,22 @@ using TiledFn = int (*)(const void*, int, const void*, int, float, const void*, 
 using QFn = int (*)(const void*, int, const uint8_t*, const uint8_t*, float, const uint8_t*, const void*, const uint8_t*, const void*,
                     int, int, int, void*, void*, size_t, uint32_t*, void*);
 using BytesFn = size_t (*)(int, int, int);
+using PackFn = int (*)(const int8_t*, const uint8_t*, int, int, uint8_t*, uint8_t*, uint32_t*, void*);
+using QuantFn = int (*)(const float*, int, int, int8_t*, float*, void*, size_t, uint32_t*, void*);
+using QuantBytesFn = size_t (*)(int, int);
+using MaskFn = int (*)(const int8_t*, const float*, int, int, uint8_t*, uint32_t*, void*);
+using AdapterFn = int (*)(const void*, int, int, uint8_t*, void*, void*);
 using TextFn = const char* (*)(int);
 
 FwdFn g_fwd = nullptr;
 TiledFn g_tiled = nullptr;
 QFn g_q = nullptr;
 BytesFn g_tiled_bytes = nullptr;
+PackFn g_pack = nullptr;
+QuantFn g_quant = nullptr;
+QuantBytesFn g_quant_bytes = nullptr;
+MaskFn g_mask = nullptr;
+AdapterFn g_pack_adapter = nullptr;
 TextFn g_text = nullptr;
 PyObject* g_error = nullptr;            // SlimError(code, where, text)
 
@@ -68,7 +82,7 @@ PyObject* output(PyObject* given, int64_t b, int64_t d_out, const at::Tensor& li
 
 PyObject* finish(int code, PyObject* y, const char* where) {
     if (code == 0) return y;
-    Py_DECREF(y);
+    Py_XDECREF(y);
     PyObject* e = PyObject_CallFunction(g_error, "iss", code, where, g_text(code));
     if (e) { PyErr_SetObject(g_error, e); Py_DECREF(e); }
     return nullptr;
@@ -102,6 +116,7 @@ bool adapters(PyObject* oL, PyObject* oR, int64_t d_out, int64_t d_in, void** L,
 
 // linear_fwd(X, vals, meta, s, L, R, Y, workspace, status, kernel)
 PyObject* linear_fwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
+    HANDLE_TH_ERRORS
     if (!bound(n, 10)) return nullptr;
     const at::Tensor *X = bf16_tensor(a[0], "X"), *v = X ? u8_tensor(a[1], "vals") : nullptr, *m = v ? u8_tensor(a[2], "meta") : nullptr;
     if (!m || !rank2(X, "X") || !rank2(v, "vals") || !rank2(m, "meta")) return nullptr;
@@ -128,10 +143,12 @@ PyObject* linear_fwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
                (uint32_t*)status, stream, (int)kernel);
     Py_END_ALLOW_THREADS
     return finish(rc, y, "slim_linear_fwd");
+    END_HANDLE_TH_ERRORS
 }
 
 // linear_fwd_tiled(X, tiled, d_out, s, L, R, Y, workspace, status, layout)
 PyObject* linear_fwd_tiled(PyObject*, PyObject* const* a, Py_ssize_t n) {
+    HANDLE_TH_ERRORS
     if (!bound(n, 10)) return nullptr;
     const at::Tensor *X = bf16_tensor(a[0], "X"), *t = X ? u8_tensor(a[1], "tiled") : nullptr;
     if (!t || !rank2(X, "X")) return nullptr;
@@ -158,10 +175,12 @@ PyObject* linear_fwd_tiled(PyObject*, PyObject* const* a, Py_ssize_t n) {
     rc = g_tiled(xp, (int)b, tp, (int)layout, (float)s, L, R, (int)r, (int)d_out, (int)d_in, Y, ws, ws_bytes, (uint32_t*)status, stream);
     Py_END_ALLOW_THREADS
     return finish(rc, y, "slim_linear_fwd_tiled");
+    END_HANDLE_TH_ERRORS
 }
 
 // linear_fwd_q(X, vals, meta, s, Lq, Ls, Rq, Rs, Y, workspace, status)
 PyObject* linear_fwd_q(PyObject*, PyObject* const* a, Py_ssize_t n) {
+    HANDLE_TH_ERRORS
     if (!bound(n, 11)) return nullptr;
     const at::Tensor *X = bf16_tensor(a[0], "X"), *v = X ? u8_tensor(a[1], "vals") : nullptr, *m = v ? u8_tensor(a[2], "meta") : nullptr;
     const at::Tensor *Lq = m ? u8_tensor(a[4], "Lq") : nullptr, *Ls = Lq ? bf16_tensor(a[5], "Ls") : nullptr;
@@ -188,18 +207,148 @@ PyObject* linear_fwd_q(PyObject*, PyObject* const* a, Py_ssize_t n) {
              (int)d_out, (int)d_in, Y, ws, ws_bytes, (uint32_t*)status, stream);
     Py_END_ALLOW_THREADS
     return finish(rc, y, "slim_linear_fwd_q");
+    END_HANDLE_TH_ERRORS
 }
 
-// bind(SlimError, fwd_ex, fwd_tiled, fwd_q, tiled_bytes, strerror): addresses in the loaded libslim
+// ---- producers of the packed weight
+at::Tensor fresh(at::IntArrayRef shape, at::ScalarType type, const at::Tensor& like) {
+    return at::detail::empty_cuda(shape, type, like.device(), std::nullopt);
+}
+
+// Words the kernels can set a status bit in and the host can read without a copy: pinned memory, handed out one to a
+// call and given back.  A kernel touches its word only when it has an error to report.
+class StatusWords {
+    static constexpr int kWords = 64, kStride = 16;            // a word per 64 bytes
+    uint32_t* page_ = nullptr;
+    uint64_t used_ = 0;
+    std::mutex m_;
+public:
+    uint32_t* take() {
+        std::lock_guard<std::mutex> lock(m_);
+        if (!page_ && cudaHostAlloc(reinterpret_cast<void**>(&page_), kWords * kStride * 4, cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
+            cudaGetLastError();
+            page_ = nullptr;
+        }
+        if (!page_ || used_ == ~0ull) return nullptr;
+        const int i = __builtin_ctzll(~used_);
+        used_ |= 1ull << i;
+        page_[i * kStride] = 0;
+        return page_ + i * kStride;
+    }
+    void give(uint32_t* w) {
+        std::lock_guard<std::mutex> lock(m_);
+        used_ &= ~(1ull << ((w - page_) / kStride));
+    }
+};
+StatusWords g_words;
+
+// pack(codes, mask, vals, meta, status, check) -> (vals, meta)
+PyObject* pack(PyObject*, PyObject* const* a, Py_ssize_t n) {
+    HANDLE_TH_ERRORS
+    if (!bound(n, 6)) return nullptr;
+    const at::Tensor *c = device_tensor(a[0], at::kChar, "codes", "torch.int8"), *m = c ? u8_tensor(a[1], "mask") : nullptr;
+    if (!m || !rank2(c, "codes")) return nullptr;
+    const int64_t d_out = c->size(0), d_in = c->size(1);
+    const int check = PyObject_IsTrue(a[5]);
+    if (check < 0) return nullptr;
+    void *vp, *mp, *status;
+    if (!address(a[2], "vals", &vp) || !address(a[3], "meta", &mp) || !address(a[4], "status", &status)) return nullptr;
+    at::Tensor vals, meta, own;
+    if (!vp) { vals = fresh({d_out, d_in / 4}, at::kByte, *c); vp = vals.data_ptr(); } else vals = THPVariable_Unpack(a[2]);
+    if (!mp) { meta = fresh({d_out, d_in / 8}, at::kByte, *c); mp = meta.data_ptr(); } else meta = THPVariable_Unpack(a[3]);
+    const auto stream = c10::cuda::getCurrentCUDAStream();
+    uint32_t* word = nullptr;
+    const bool look = check && !status;
+    if (look) {
+        word = g_words.take();
+        if (!word) { own = at::zeros({1}, c->options().dtype(at::kInt)); }
+        status = word ? word : own.data_ptr();
+    }
+    const void *cp = c->data_ptr(), *kp = m->data_ptr();
+    int rc;
+    uint32_t bits = 0;
+    Py_BEGIN_ALLOW_THREADS
+    rc = g_pack((const int8_t*)cp, (const uint8_t*)kp, (int)d_out, (int)d_in, (uint8_t*)vp, (uint8_t*)mp, (uint32_t*)status, stream.stream());
+    if (word) {
+        if (rc == 0 && cudaStreamSynchronize(stream.stream()) != cudaSuccess) rc = 6;          // SLIM_ERR_CUDA
+        bits = *static_cast<volatile uint32_t*>(word);
+        g_words.give(word);
+    }
+    Py_END_ALLOW_THREADS
+    if (look && !word && rc == 0) bits = (uint32_t)own.item<int>();
+    for (int code : {3, 4})                                    // SLIM_ERR_BAD_MASK, SLIM_ERR_CODE_RANGE
+        if (rc == 0 && (bits & (1u << code))) rc = code;
+    if (rc != 0) return finish(rc, nullptr, "slim_pack");
+    return Py_BuildValue("(NN)", THPVariable_Wrap(std::move(vals)), THPVariable_Wrap(std::move(meta)));
+    END_HANDLE_TH_ERRORS
+}
+
+// mask_top2(codes, xbar, status) -> mask
+PyObject* mask_top2(PyObject*, PyObject* const* a, Py_ssize_t n) {
+    HANDLE_TH_ERRORS
+    if (!bound(n, 3)) return nullptr;
+    const at::Tensor* c = device_tensor(a[0], at::kChar, "codes", "torch.int8");
+    if (!c || !rank2(c, "codes")) return nullptr;
+    const at::Tensor* x = a[1] == Py_None ? nullptr : device_tensor(a[1], at::kFloat, "xbar", "torch.float32");
+    if (a[1] != Py_None && !x) return nullptr;
+    void* status;
+    if (!address(a[2], "status", &status)) return nullptr;
+    at::Tensor mask = fresh(c->sizes(), at::kByte, *c);
+    const int rc = g_mask((const int8_t*)c->data_ptr(), x ? (const float*)x->data_ptr() : nullptr, (int)c->size(0), (int)c->size(1),
+                          (uint8_t*)mask.data_ptr(), (uint32_t*)status, c10::cuda::getCurrentCUDAStream().stream());
+    return rc == 0 ? THPVariable_Wrap(std::move(mask)) : finish(rc, nullptr, "slim_mask_top2");
+    END_HANDLE_TH_ERRORS
+}
+
+// pack_adapter(A) -> (codes, scales)
+PyObject* pack_adapter(PyObject*, PyObject* const* a, Py_ssize_t n) {
+    HANDLE_TH_ERRORS
+    if (!bound(n, 1)) return nullptr;
+    const at::Tensor* A = bf16_tensor(a[0], "A");
+    if (!A || !rank2(A, "A")) return nullptr;
+    const int64_t rows = A->size(0), cols = A->size(1);
+    if (rows < 1 || cols < 2 || cols % 2 != 0) return finish(1, nullptr, "slim_pack_adapter");      // SLIM_ERR_INVALID_ARG
+    at::Tensor codes = fresh({rows, cols / 2}, at::kByte, *A), scales = fresh({rows, (cols + 127) / 128}, at::kBFloat16, *A);
+    const int rc = g_pack_adapter(A->data_ptr(), (int)rows, (int)cols, (uint8_t*)codes.data_ptr(), scales.data_ptr(),
+                                  c10::cuda::getCurrentCUDAStream().stream());
+    if (rc != 0) return finish(rc, nullptr, "slim_pack_adapter");
+    return Py_BuildValue("(NN)", THPVariable_Wrap(std::move(codes)), THPVariable_Wrap(std::move(scales)));
+    END_HANDLE_TH_ERRORS
+}
+
+// quant(W, status) -> (codes, scale_alpha, table, alpha)
+PyObject* quant(PyObject*, PyObject* const* a, Py_ssize_t n) {
+    HANDLE_TH_ERRORS
+    if (!bound(n, 2)) return nullptr;
+    const at::Tensor* W = device_tensor(a[0], at::kFloat, "W", "torch.float32");
+    if (!W || !rank2(W, "W")) return nullptr;
+    void* status;
+    if (!address(a[1], "status", &status)) return nullptr;
+    const int64_t d_out = W->size(0), d_in = W->size(1);
+    const size_t bytes = g_quant_bytes((int)d_out, (int)d_in);
+    at::Tensor ws = fresh({(int64_t)bytes}, at::kByte, *W), codes = fresh({d_out, d_in}, at::kChar, *W), sa = fresh({4}, at::kFloat, *W);
+    const int rc = g_quant((const float*)W->data_ptr(), (int)d_out, (int)d_in, (int8_t*)codes.data_ptr(), (float*)sa.data_ptr(),
+                           ws.data_ptr(), bytes, (uint32_t*)status, c10::cuda::getCurrentCUDAStream().stream());
+    if (rc != 0) return finish(rc, nullptr, "slim_quant");
+    const int64_t bins = std::max<int64_t>(512, std::min<int64_t>(d_out * d_in / 1000, 20000)), at_ = 256 + (bins * 4 + 255) / 256 * 256;
+    at::Tensor tab = ws.slice(0, at_, at_ + 59 * 8).view(at::kDouble);
+    return Py_BuildValue("(NNNN)", THPVariable_Wrap(std::move(codes)), THPVariable_Wrap(sa.slice(0, 0, 2)),
+                         THPVariable_Wrap(tab.slice(0, 0, 58).view({29, 2})), THPVariable_Wrap(tab.select(0, 58)));
+    END_HANDLE_TH_ERRORS
+}
+
+// bind(SlimError, addresses of the functions in the loaded libslim)
 PyObject* bind(PyObject*, PyObject* args) {
     PyObject* err;
-    unsigned long long f, t, q, by, tx;
-    if (!PyArg_ParseTuple(args, "OKKKKK", &err, &f, &t, &q, &by, &tx)) return nullptr;
+    unsigned long long f, t, q, by, tx, pk, qu, qb, mk, pa;
+    if (!PyArg_ParseTuple(args, "OKKKKKKKKKK", &err, &f, &t, &q, &by, &tx, &pk, &qu, &qb, &mk, &pa)) return nullptr;
     Py_INCREF(err);
     Py_XDECREF(g_error);
     g_error = err;
     g_fwd = reinterpret_cast<FwdFn>(f); g_tiled = reinterpret_cast<TiledFn>(t); g_q = reinterpret_cast<QFn>(q);
     g_tiled_bytes = reinterpret_cast<BytesFn>(by); g_text = reinterpret_cast<TextFn>(tx);
+    g_pack = reinterpret_cast<PackFn>(pk); g_quant = reinterpret_cast<QuantFn>(qu); g_quant_bytes = reinterpret_cast<QuantBytesFn>(qb);
+    g_mask = reinterpret_cast<MaskFn>(mk); g_pack_adapter = reinterpret_cast<AdapterFn>(pa);
     Py_RETURN_NONE;
 }
 
@@ -208,6 +357,10 @@ PyMethodDef methods[] = {
     {"linear_fwd", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)(void)>(linear_fwd)), METH_FASTCALL, nullptr},
     {"linear_fwd_tiled", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)(void)>(linear_fwd_tiled)), METH_FASTCALL, nullptr},
     {"linear_fwd_q", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)(void)>(linear_fwd_q)), METH_FASTCALL, nullptr},
+    {"pack", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)(void)>(pack)), METH_FASTCALL, nullptr},
+    {"mask_top2", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)(void)>(mask_top2)), METH_FASTCALL, nullptr},
+    {"pack_adapter", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)(void)>(pack_adapter)), METH_FASTCALL, nullptr},
+    {"quant", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)(void)>(quant)), METH_FASTCALL, nullptr},
     {nullptr, nullptr, 0, nullptr}};
 
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_slim_native", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
