@@ -54,34 +54,36 @@
 namespace slim {
 
 constexpr int kPM = 128;            // output rows per CTA (MMA M)
-constexpr int kPBK = 64;            // columns per stage, both phases
-constexpr int kPkStages = 4;        // stages covered by one packed tile (256 weight columns)
+constexpr int kPBK = 64;            // columns of a TMA box of bf16 (128 bytes)
+constexpr int kPkCols = 256;        // weight columns of one packed tile
 constexpr int kConvWarps = 8;       // warps 0-7 converters / epilogue
 constexpr int kWarpXEven = 8, kWarpMma = 9, kWarpXOdd = 10, kWarpPk = 11;
 constexpr int kPThreads = 32 * 12;
 constexpr int kATile = kPM * 128;               // 16 KB: 128 rows x 128 bytes (dense phase)
-constexpr int kValsTile = kPM * (kPkStages * kPBK / 4);     // 8 KB: 64 value bytes per row
-constexpr int kMetaTile = kPM * (kPkStages * kPBK / 8);     // 4 KB: 32 index bytes per row
+constexpr int kValsTile = kPM * (kPkCols / 4);  // 8 KB: 64 value bytes per row
+constexpr int kMetaTile = kPM * (kPkCols / 8);  // 4 KB: 32 index bytes per row
 constexpr int kPkSlotBytes = kValsTile + kMetaTile;
 constexpr uint32_t kPSpinLimit = 1u << 21;
 
 // TWO = a pair of CTAs (cluster of 2 along the row tiles) shares one token tile: each CTA
 // loads half of it and one cta_group::2 MMA of shape 256 x N, issued by the even CTA,
-// drives both tensor cores.  Halves the token-tile traffic per CTA and leaves room for
-// more stages.
+// drives both tensor cores.  Halves the shared-memory traffic of the token tile per CTA, and its
+// stages are twice as long (128 weight columns, four MMAs per commit): a commit per pair of MMAs cost a
+// pair as much time as the MMAs.
 // PRE = the dense-only launch (T' product): no packed tiles, so the room goes to more stages.
 template <int N, bool TWO, bool PRE = false> struct PfCfg {
     static constexpr int kBRows = TWO ? N / 2 : N;                          // token rows this CTA loads
-    static constexpr int kBTile = kBRows * 128;
-    // A region of a stage: the expanded weight tile needs 8 KB.  The main kernels' dense stages are
+    static constexpr int kSK = TWO ? 128 : 64;                              // weight columns of a sparse stage
+    static constexpr int kPkStages = kPkCols / kSK;                         // stages covered by one packed tile
+    static constexpr int kBTile = kBRows * kSK * 2;
+    // A region of a stage: the expanded weight tile, 128 rows x kSK bytes.  The one-CTA kernel's dense stages are
     // 32 columns wide so that their A2 tile fits there too: a smaller stage means more stages in
-    // flight, and the loop is bound by the latency of the token tile.  The dense-only launch
-    // has no expanded tiles and keeps 64-column stages.
-    static constexpr int kARegion = PRE ? kATile : kATile / 2;
-    static constexpr int kDK = PRE ? 64 : 32;                               // columns of a dense stage
-    static constexpr int kStages = PRE ? (N >= 256 ? 4 : 8) : (TWO ? 7 : (N >= 256 ? 5 : 8));
+    // flight.  The dense-only launch has no expanded tiles; it and the pair have 64-column dense stages.
+    static constexpr int kARegion = PRE ? kATile : kPM * kSK;
+    static constexpr int kDK = PRE || TWO ? 64 : 32;                        // columns of a dense stage
+    static constexpr int kStages = PRE ? (N >= 256 ? 4 : 8) : (TWO ? 4 : (N >= 256 ? 5 : 8));
     // Packed tiles come from HBM (latency of a microsecond or two): the ring holds what fits.
-    static constexpr int kPkSlots = PRE ? 1 : (TWO ? 4 : (N >= 256 ? 2 : 7));
+    static constexpr int kPkSlots = PRE ? 1 : (TWO ? 2 : (N >= 256 ? 2 : 7));
     static constexpr int kStageBytes = kBTile + kARegion;
     static constexpr int kECol = N;                                         // index words: N + 4 * stage + mma
     static constexpr int kTmemCols = N >= 256 ? 512 : (N >= 128 ? 256 : 128);
@@ -104,6 +106,7 @@ struct PrefillParams {
     // multiple): the array and its row pitch; nullptr: by TMA.
     const uint8_t* meta;
     int meta_pitch;
+    int d_in;
 };
 
 // Optional timeline: built with -DSLIM_PREFILL_TRACE, one thread per warp role of the first
@@ -205,37 +208,25 @@ __device__ __forceinline__ void mma_sparse2(uint32_t d_tmem, uint64_t a_desc, ui
         "tcgen05.mma.sp.cta_group::2.kind::f16 [%0], %1, %2, [%3], %4, p;\n\t}"
         :: "r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(e_tmem), "r"(idesc), "r"(accumulate) : "memory");
 }
+// The same for a pair's loads: the bytes are counted on the even CTA's barrier.
+__device__ __forceinline__ void tma_tile_pair(void* dst, const CUtensorMap* tmap, int x, int y, uint32_t cluster_bar_addr) {
+    asm volatile("cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
+                 :: "r"(s32(dst)), "l"(tmap), "r"(x), "r"(y), "r"(cluster_bar_addr) : "memory");
+}
 // Address of the same shared-memory object in CTA `rank` of the cluster.
 __device__ __forceinline__ uint32_t peer_addr(const void* p, uint32_t rank) {
     uint32_t r;
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(s32(p)), "r"(rank));
     return r;
 }
-// Completion of this thread's earlier MMAs arrives on a barrier given by cluster address.
-__device__ __forceinline__ void mma_commit2(uint32_t cluster_bar_addr) {
-    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" :: "r"(cluster_bar_addr) : "memory");
+// Completion of this thread's earlier MMAs arrives on the same barrier of both CTAs of the pair.
+__device__ __forceinline__ void mma_commit2(uint64_t* bar) {
+    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
+                 :: "r"(s32(bar)), "h"((uint16_t)3) : "memory");
 }
 // Arrival on a barrier of another CTA of the cluster, ordered like a CTA-local arrival.
 __device__ __forceinline__ void mbar_arrive_remote(uint32_t cluster_bar_addr) {
     asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" :: "r"(cluster_bar_addr) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_bar_addr) {
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" :: "r"(cluster_bar_addr) : "memory");
-}
-__device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity, volatile uint32_t* abort_flag) {
-    const uint32_t addr = s32(bar);
-    for (uint32_t it = 0; it < kPSpinLimit; ++it) {
-        uint32_t done;
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}"
-            : "=r"(done) : "r"(addr), "r"(parity) : "memory");
-        if (done) return true;
-        if (*abort_flag) return false;
-    }
-    *abort_flag = 1u;
-    return false;
 }
 // One try_wait, no loop.  `cluster`: acquire at cluster scope (arrivals came from the other CTA).
 __device__ __forceinline__ uint32_t mbar_try(uint64_t* bar, uint32_t parity, bool cluster) {
@@ -331,7 +322,7 @@ prefill_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap tmV,
     // request of a T' tile.
     if (PRE) asm volatile("griddepcontrol.launch_dependents;");
     constexpr int kBTile = Cfg::kBTile, kStageBytes = Cfg::kStageBytes, kECol = Cfg::kECol, kPStages = Cfg::kStages;
-    constexpr int kPkSlots = Cfg::kPkSlots, kDK = Cfg::kDK;
+    constexpr int kPkSlots = Cfg::kPkSlots, kDK = Cfg::kDK, kSK = Cfg::kSK, kPkStages = Cfg::kPkStages;
     extern __shared__ unsigned char smem_raw[];
     // layout: stages {B | A} | packed slots {value bytes | index bytes} | barriers
     unsigned char* stages = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -343,8 +334,7 @@ prefill_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap tmV,
     uint64_t* pk_full = bars + 3 * kPStages;         // [kPkSlots]
     uint64_t* pk_empty = pk_full + kPkSlots;         // [kPkSlots]
     uint64_t* acc_full = pk_empty + kPkSlots;        // [1]
-    uint64_t* peer_ready = acc_full + 1;             // [kPStages] pair only: the odd CTA's stage is ready
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(peer_ready + kPStages);
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_full + 1);
     volatile uint32_t* abort_flag = tmem_slot + 1;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -357,14 +347,14 @@ prefill_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap tmV,
     // so that at any moment they ask the L2 for different lines of X rather than all for the same
     // ones.  The walk is rotated by whole 256-column groups (a pair of CTAs rotates together).
     const int n_groups = ceil_div(p.n1, kPkStages);
-    const int rot_g = (p.n1 % kPkStages == 0 && n_groups > 0)
+    const int rot_g = (p.d_in % kPkCols == 0 && n_groups > 0)
                           ? (int)(((blockIdx.x >> (TWO ? 1 : 0)) + 3u * blockIdx.y) % (unsigned)n_groups) : 0;
 
     if (threadIdx.x == 0) PSTAMP(5, 44);
     if (threadIdx.x == 0) {
         for (int i = 0; i < kPStages; ++i) {
             mbar_init(&b_full[i], 1);
-            mbar_init(&conv_done[i], TWO ? kConvWarps : kConvWarps / 2); mbar_init(&empty[i], 1); mbar_init(&peer_ready[i], 1);
+            mbar_init(&conv_done[i], TWO ? kConvWarps : kConvWarps / 2); mbar_init(&empty[i], 1);
         }
         for (int i = 0; i < kPkSlots; ++i) { mbar_init(&pk_full[i], p.meta ? 33 : 1); mbar_init(&pk_empty[i], kConvWarps); }
         mbar_init(acc_full, 1);
@@ -407,15 +397,21 @@ prefill_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap tmV,
             // spins: that costs some hundred nanoseconds per stage); lane 0 arms the barrier.
             if (it >= kPStages) ok = mbar_wait(&empty[st], ((it / kPStages) & 1) ^ 1, abort_flag) && ok;
             // dense stage: kDK columns of the token rows and of the A2 rows
-            if (lane == 0) mbar_expect_tx(&b_full[st], (uint32_t)(sparse ? kBTile : (Cfg::kBRows + kPM) * kDK * 2));
+            // a pair's bytes, both CTAs', are counted on the even CTA's barrier
+            if (lane == 0 && rank == 0)
+                mbar_expect_tx(&b_full[st], (uint32_t)((TWO ? 2 : 1) * (sparse ? kBTile : (Cfg::kBRows + kPM) * kDK * 2)));
             unsigned char* sbase = stages + (size_t)st * kStageBytes;
             int kb = sparse ? it + rot_g * kPkStages : it - p.n1 + k_first;
             if (sparse && kb >= p.n1) kb -= p.n1;
-            const int k = sparse ? kb * kPBK : kb * kDK;
-            // lane 0: the token tile (one box); lane 1, dense stages only: the A2 tile
-            if (lane == 0 || (lane == 1 && !sparse))
-                tma_tile(lane == 0 ? sbase : sbase + kBTile, lane == 1 ? &tmA2 : (sparse ? &tmX : &tmB2), k,
-                         lane == 0 ? nb0 : m0, &b_full[st]);
+            const int k = sparse ? kb * kSK : kb * kDK;
+            // sparse stage: the token tile, a box per 64 columns; dense stage: lane 0 the token tile, lane 1 the A2 tile
+            if (lane < (sparse ? kSK / kPBK : 2)) {
+                const CUtensorMap* map = sparse ? &tmX : lane == 0 ? &tmB2 : &tmA2;
+                unsigned char* dst = sbase + (lane == 0 ? 0 : sparse ? Cfg::kBRows * 128 : kBTile);
+                const int x = sparse ? k + lane * kPBK : k, y = !sparse && lane == 1 ? m0 : nb0;
+                if (TWO) tma_tile_pair(dst, map, x, y, peer_addr(&b_full[st], 0));
+                else tma_tile(dst, map, x, y, &b_full[st]);
+            }
             if (lane == 0) PSTAMP(0, it);
         }
     } else if (warp == kWarpPk) {
@@ -446,18 +442,7 @@ prefill_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap tmV,
         // ============================ MMA issuer ============================
         // One elected lane walks the stages and issues.
         if (TWO && rank != 0) {
-            // Odd CTA of a pair: tell the even CTA when this CTA's token rows (and A2 rows) of a
-            // stage have landed.  The data stay in this CTA's shared memory and are read by this
-            // SM's tensor core, so an arrival ordered after the landing within this CTA is enough;
-            // a cluster-scope release costs some 300 cycles per stage.
-            if (lane == 0) {
-                for (int it = 0; it < n_total; ++it) {
-                    const int st = it % kPStages;
-                    ok = mbar_wait(&b_full[st], (it / kPStages) & 1, abort_flag) && ok;
-                    mbar_arrive_remote(peer_addr(&peer_ready[st], 0));
-                    PSTAMP(5, it);
-                }
-            }
+            // the even CTA issues the pair's MMAs
         } else if (elect_one()) {
             constexpr uint32_t idesc = idesc_bf16(TWO ? 2 * kPM : kPM, N);
             uint32_t pre = 0;       // the coming stage was found ready by an early test
@@ -465,10 +450,10 @@ prefill_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap tmV,
                 const int st = it % kPStages;
                 const uint32_t parity = (it / kPStages) & 1;
                 const bool sparse = it < p.n1;
-                // token tile landed; converters done (in a pair: both CTAs', reported here); the other CTA's loads landed
+                // token tile landed; converters done (in a pair: both CTAs', reported here)
                 if (!pre)
-                    ok = mbar_wait_all(&b_full[st], parity, false, sparse ? &conv_done[st] : nullptr, parity, TWO,
-                                       TWO ? &peer_ready[st] : nullptr, parity, true, abort_flag) && ok;
+                    ok = mbar_wait_all(&b_full[st], parity, TWO, sparse ? &conv_done[st] : nullptr, parity, TWO,
+                                       nullptr, 0, false, abort_flag) && ok;
                 fence_after_sync();
                 // ask about the next stage now, without waiting: the answer comes back while this stage's
                 // MMAs are issued, and in steady state it is yes
@@ -476,39 +461,38 @@ prefill_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap tmV,
                 if (it + 1 < n_total) {
                     const int st1 = (it + 1) % kPStages;
                     const uint32_t par1 = ((it + 1) / kPStages) & 1;
-                    pre = mbar_test(&b_full[st1], par1, false);
+                    pre = mbar_test(&b_full[st1], par1, TWO);
                     if (it + 1 < p.n1) pre &= mbar_test(&conv_done[st1], par1, TWO);
-                    if (TWO) pre &= mbar_test(&peer_ready[st1], par1, true);
                 }
                 const uint32_t b_addr = s32(stages + (size_t)st * kStageBytes);
                 const uint32_t a_addr = b_addr + kBTile;
                 PSTAMP(3, it);
                 if (sparse) {
-                    // per MMA: A 16 stored bf16 (32 bytes of a 64-byte row), B 32 columns (64 bytes)
+                    // per MMA: A 16 stored bf16 (32 bytes of a row of kSK bytes), B 32 columns (64 bytes)
 #pragma unroll
-                    for (int j = 0; j < 2; ++j) {
+                    for (int j = 0; j < kSK / 32; ++j) {
                         const uint32_t acc = (it > 0 || j > 0) ? 1u : 0u;
-                        if (TWO) mma_sparse2(tmem_base, smem_desc64(a_addr + 32 * j), smem_desc(b_addr + 64 * j),
-                                             tmem_base + kECol + 4 * st, idesc | (1u << 2) | (uint32_t)j, acc);
-                        else     mma_sparse(tmem_base, smem_desc64(a_addr + 32 * j), smem_desc(b_addr + 64 * j),
-                                            tmem_base + kECol + 4 * st, idesc | (1u << 2) | (uint32_t)j, acc);
+                        const uint32_t e_col = tmem_base + kECol + 4 * st + 2 * (j >> 1);
+                        const uint64_t bd = smem_desc(b_addr + (j >> 1) * (Cfg::kBRows * 128) + 64 * (j & 1));
+                        if (TWO) mma_sparse2(tmem_base, smem_desc(a_addr + 32 * j), bd, e_col, idesc | (1u << 2) | (uint32_t)(j & 1), acc);
+                        else     mma_sparse(tmem_base, smem_desc64(a_addr + 32 * j), bd, e_col, idesc | (1u << 2) | (uint32_t)(j & 1), acc);
                     }
                 } else {
 #pragma unroll
                     for (int j = 0; j < kDK / 16; ++j) {
                         const uint32_t acc = (it > 0 || j > 0) ? 1u : 0u;
                         // 32-column stages: 64-byte rows with the 64-byte swizzle; 64-column stages: 128-byte rows
-                        if (TWO)            mma_dense2(tmem_base, smem_desc64(a_addr + 32 * j), smem_desc64(b_addr + 32 * j), idesc, acc);
+                        if (TWO)            mma_dense2(tmem_base, smem_desc(a_addr + 32 * j), smem_desc(b_addr + 32 * j), idesc, acc);
                         else if (kDK == 32) mma_dense(tmem_base, smem_desc64(a_addr + 32 * j), smem_desc64(b_addr + 32 * j), idesc, acc);
                         else                mma_dense(tmem_base, smem_desc(a_addr + 32 * j), smem_desc(b_addr + 32 * j), idesc, acc);
                     }
                 }
                 // the stage is free (in both CTAs of a pair) once these MMAs have read it
-                if (TWO) { mma_commit2(peer_addr(&empty[st], 0)); mma_commit2(peer_addr(&empty[st], 1)); }
+                if (TWO) mma_commit2(&empty[st]);
                 else mma_commit(&empty[st]);
                 PSTAMP(4, it);
             }
-            if (TWO) { mma_commit2(peer_addr(acc_full, 0)); mma_commit2(peer_addr(acc_full, 1)); }
+            if (TWO) mma_commit2(acc_full);
             else mma_commit(acc_full);
         }
     } else {
@@ -529,33 +513,46 @@ prefill_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap tmV,
             ok = mbar_wait_all(&pk_full[slot], (gi / kPkSlots) & 1, false, it >= kPStages ? &empty[st] : nullptr,
                                ((it / kPStages) & 1) ^ 1, false, nullptr, 0, false, abort_flag) && ok;
             if ((threadIdx.x & 127) == 0) PSTAMP(1, it);
-            // ---- 16 value bytes -> 32 bf16: the row's four 16-byte chunks (64-byte rows, 64-byte swizzle)
-            // the packed tiles are stored with the 64-byte (values) and 32-byte (indices) TMA swizzles so
-            // that a warp's row-strided reads spread over the banks
-            const uint4 v = *reinterpret_cast<const uint4*>(pk + row * 64 + (((q ^ (row >> 1)) & 3) << 4));
-            uint2 mw2 = *reinterpret_cast<const uint2*>(pk + kValsTile + row * 32 + ((((q >> 1) ^ (row >> 2)) & 1) << 4) + (q & 1) * 8);
-            if (m0 + row >= p.m_total) mw2 = make_uint2(0x44444444u, 0x44444444u);      // rows past the last: a legal pair of positions
-            unsigned char* arow = stages + (size_t)st * kStageBytes + kBTile + row * 64;
-            const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+            // ---- 16 value bytes -> 32 bf16 per 64 columns; the packed tiles are stored with the 64-byte (values) and 32-byte
+            // (indices) TMA swizzles so that a warp's row-strided reads spread over the banks
+            unsigned char* arow = stages + (size_t)st * kStageBytes + kBTile + row * kSK;
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                const uint32_t ws = w[c] >> 4;
-                uint4 o;
-                o.x = nib2bf16<0>(w[c], ws); o.y = nib2bf16<1>(w[c], ws);
-                o.z = nib2bf16<2>(w[c], ws); o.w = nib2bf16<3>(w[c], ws);
-                *reinterpret_cast<uint4*>(arow + (((c ^ (row >> 1)) & 3) << 4)) = o;
-            }
-            // ---- index words of the stage's two MMAs (layout in the file header)
-            uint32_t e[2];
+            for (int hh = 0; hh < kSK / 64; ++hh) {
+                const int qq = q * (kSK / 64) + hh;          // which 64 columns of the packed tile
+                const uint4 v = *reinterpret_cast<const uint4*>(pk + row * 64 + (((qq ^ (row >> 1)) & 3) << 4));
+                const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const uint32_t mw = h ? mw2.y : mw2.x;
-                const uint32_t send = x ? (mw & 0xFFFFu) : (mw >> 16);
-                const uint32_t recv = __shfl_xor_sync(0xffffffffu, send, 8);
-                e[h] = x ? ((mw & 0xFFFF0000u) | recv) : ((mw & 0xFFFFu) | (recv << 16));
+                for (int c = 0; c < 4; ++c) {
+                    const uint32_t ws = w[c] >> 4;
+                    uint4 o;
+                    o.x = nib2bf16<0>(w[c], ws); o.y = nib2bf16<1>(w[c], ws);
+                    o.z = nib2bf16<2>(w[c], ws); o.w = nib2bf16<3>(w[c], ws);
+                    const int chunk = TWO ? ((hh * 4 + c) ^ row) & 7 : (c ^ (row >> 1)) & 3;      // 128- or 64-byte rows and swizzle
+                    *reinterpret_cast<uint4*>(arow + (chunk << 4)) = o;
+                }
             }
-            asm volatile("tcgen05.st.sync.aligned.32x32b.x2.b32 [%0], {%1, %2};"
-                         :: "r"(tmem_base + lane_base + kECol + 4 * st), "r"(e[0]), "r"(e[1]) : "memory");
+            // ---- index words of the stage's MMAs (layout in the file header)
+            uint32_t e[kSK / 32];
+#pragma unroll
+            for (int hh = 0; hh < kSK / 64; ++hh) {
+                const int qq = q * (kSK / 64) + hh;
+                uint2 mw2 = *reinterpret_cast<const uint2*>(pk + kValsTile + row * 32 + ((((qq >> 1) ^ (row >> 2)) & 1) << 4) + (qq & 1) * 8);
+                // past the last row or column: a legal pair of positions
+                if (m0 + row >= p.m_total || (TWO && it * kSK + hh * 64 >= p.d_in)) mw2 = make_uint2(0x44444444u, 0x44444444u);
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const uint32_t mw = h ? mw2.y : mw2.x;
+                    const uint32_t send = x ? (mw & 0xFFFFu) : (mw >> 16);
+                    const uint32_t recv = __shfl_xor_sync(0xffffffffu, send, 8);
+                    e[hh * 2 + h] = x ? ((mw & 0xFFFF0000u) | recv) : ((mw & 0xFFFFu) | (recv << 16));
+                }
+            }
+            if constexpr (TWO)
+                asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};"
+                             :: "r"(tmem_base + lane_base + kECol + 4 * st), "r"(e[0]), "r"(e[1]), "r"(e[kSK / 32 - 2]), "r"(e[kSK / 32 - 1]) : "memory");
+            else
+                asm volatile("tcgen05.st.sync.aligned.32x32b.x2.b32 [%0], {%1, %2};"
+                             :: "r"(tmem_base + lane_base + kECol + 4 * st), "r"(e[0]), "r"(e[1]) : "memory");
             asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // A is read by the tensor core
             fence_before_sync();
@@ -566,7 +563,7 @@ prefill_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap tmV,
                 if (TWO && rank != 0) mbar_arrive_remote(peer_addr(&conv_done[st], 0));
                 else mbar_arrive(&conv_done[st]);
                 // this group's last stage of the packed tile
-                if (q >= 2 || it + 2 >= p.n1) mbar_arrive(&pk_empty[slot]);
+                if (q + 2 >= kPkStages || it + 2 >= p.n1) mbar_arrive(&pk_empty[slot]);
             }
             if ((threadIdx.x & 127) == 0) PSTAMP(2, it);
         }
@@ -686,7 +683,7 @@ static slim_status_t launch_tile_kernel(const PrefillParams& q, int m_rows, cons
                                         const CUtensorMap& tmX, const CUtensorMap& tmA2, const CUtensorMap& tmB2,
                                         cudaStream_t st, int slices = 1, bool after_dense_only = false) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(ceil_div(m_rows, kPM), ceil_div(q.b, N), slices);
+    cfg.gridDim = dim3(TWO ? 2 * ceil_div(m_rows, 2 * kPM) : ceil_div(m_rows, kPM), ceil_div(q.b, N), slices);
     cfg.blockDim = dim3(kPThreads);
     cfg.dynamicSmemBytes = PfCfg<N, TWO, PRE>::kSmem;
     cfg.stream = st;
@@ -727,18 +724,16 @@ slim_status_t launch_prefill(const __nv_bfloat16* X, int b, const uint8_t* vals,
     // token tile: 256 when that gives a quarter of the SMs or more a tile, else 64 (measured: with 64 tiles of
     // 128 x 256 on 148 SMs the wide variant is a third faster than 256 tiles of 128 x 64; with 32 it is slower)
     const bool wide = force_pair || (long long)ceil_div(d_out, kPM) * ceil_div(b, 256) * 4 >= (long long)di->sm_count;
-    const int n_pre = 64;                         // the T' product has few row tiles: narrow token tiles fill the machine
     // The CTA-pair kernel (prefill_kernel<256, true>) measures 3-8 % faster than one CTA per tile on
     // problems with adapters and a thousand tiles or more (the 70B layers at 4096 tokens) and the same or
     // a little slower below that: it runs for those, or when asked for by name.
     if (force_pair && ceil_div(d_out, kPM) % 2 != 0) return SLIM_ERR_UNSUPPORTED_SHAPE;
-    const bool pair = force_pair || (wide && r > 0 && ceil_div(d_out, kPM) % 2 == 0 &&
-                                     (long long)ceil_div(d_out, kPM) * ceil_div(b, 256) >= 1024);
+    const bool pair = force_pair || wide;
     const int xbox = wide ? (pair ? 128 : 256) : 64;      // token rows one CTA loads per stage = one TMA box
-    const int dk = PfCfg<256, false>::kDK;                // columns of a dense stage of the main kernels
+    const int dk = pair ? PfCfg<256, true>::kDK : PfCfg<256, false>::kDK;      // columns of a dense stage of the main kernel
     CUtensorMap tmV, tmM, tmX, tmXpre, tmA2, tmB2;
-    bool ok = pf_map(&tmV, vals, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)d_in / 4, (uint64_t)d_out, kPkStages * kPBK / 4, kPM, 64) &&
-              (d_in % 128 != 0 || pf_map(&tmM, meta, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)d_in / 8, (uint64_t)d_out, kPkStages * kPBK / 8, kPM, 32)) &&
+    bool ok = pf_map(&tmV, vals, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)d_in / 4, (uint64_t)d_out, kPkCols / 4, kPM, 64) &&
+              (d_in % 128 != 0 || pf_map(&tmM, meta, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)d_in / 8, (uint64_t)d_out, kPkCols / 8, kPM, 32)) &&
               pf_map(&tmX, X, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (uint64_t)d_in, (uint64_t)b, 64, xbox, 128);
     if (!ok) return SLIM_ERR_CUDA;
     if (d_in % 128 != 0) tmM = tmV;              // not used
@@ -750,7 +745,7 @@ slim_status_t launch_prefill(const __nv_bfloat16* X, int b, const uint8_t* vals,
         if (!ok) return SLIM_ERR_CUDA;
         PrefillParams q;
         q.out = Tq; q.ldo = r; q.m_total = r; q.b = b; q.n1 = 0; q.n2 = d_in / kPBK; q.scale = 1.f / s_eff; q.status = status_dev;
-        q.k_per = pl.k_per; q.meta = nullptr; q.meta_pitch = 0;
+        q.k_per = pl.k_per; q.meta = nullptr; q.meta_pitch = 0; q.d_in = d_in;
         // partial tiles of the K slices follow T' in the workspace
         q.part = pl.slices > 1 ? reinterpret_cast<float*>(reinterpret_cast<char*>(Tq) + ((size_t)b * r * sizeof(__nv_bfloat16) + 255) / 256 * 256) : nullptr;
         slim_status_t rc = pl.n_tok == 256 ? launch_tile_kernel<256, false, true>(q, r, tmV, tmM, tmXpre, tmA2, tmXpre, st, pl.slices)
@@ -779,10 +774,10 @@ slim_status_t launch_prefill(const __nv_bfloat16* X, int b, const uint8_t* vals,
     }
     PrefillParams p;
     p.out = Y; p.ldo = d_out; p.m_total = d_out; p.b = b;
-    p.n1 = s != 0.f ? d_in / kPBK : 0;
+    p.n1 = s != 0.f ? ceil_div(d_in, pair ? PfCfg<256, true>::kSK : PfCfg<256, false>::kSK) : 0;
     p.n2 = r > 0 ? ceil_div(r, dk) : 0;
     p.scale = s_eff; p.status = status_dev; p.part = nullptr; p.k_per = 0;
-    p.meta = d_in % 128 != 0 ? meta : nullptr; p.meta_pitch = d_in / 8;
+    p.meta = d_in % 128 != 0 ? meta : nullptr; p.meta_pitch = d_in / 8; p.d_in = d_in;
     if (p.n1 + p.n2 == 0)             // s == 0 and no adapters: the result is zero
         return cudaMemsetAsync(Y, 0, (size_t)b * d_out * 2, st) == cudaSuccess ? SLIM_OK : SLIM_ERR_CUDA;
     note_token_tile(wide ? 256 : 64);
