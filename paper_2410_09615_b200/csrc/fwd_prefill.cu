@@ -65,28 +65,21 @@ constexpr int kMetaTile = kPM * (kPkCols / 8);  // 4 KB: 32 index bytes per row
 constexpr int kPkSlotBytes = kValsTile + kMetaTile;
 constexpr uint32_t kPSpinLimit = 1u << 21;
 
-// TWO = a pair of CTAs (cluster of 2 along the row tiles) shares one token tile: each CTA
-// loads half of it and one cta_group::2 MMA of shape 256 x N, issued by the even CTA,
-// drives both tensor cores.  Halves the shared-memory traffic of the token tile per CTA, and its
-// stages are twice as long (128 weight columns, four MMAs per commit): a commit per pair of MMAs cost a
-// pair as much time as the MMAs.
-// PRE = the dense-only launch (T' product): no packed tiles, so the room goes to more stages.
-template <int N, bool TWO, bool PRE = false> struct PfCfg {
-    static constexpr int kBRows = TWO ? N / 2 : N;                          // token rows this CTA loads
-    static constexpr int kSK = TWO ? 128 : 64;                              // weight columns of a sparse stage
+// The one-CTA kernel.  PRE = the dense-only launch (T' product): no packed tiles, so the room goes to more stages.
+template <int N, bool PRE = false> struct PfCfg {
+    static constexpr int kSK = 64;                                          // weight columns of a sparse stage
     static constexpr int kPkStages = kPkCols / kSK;                         // stages covered by one packed tile
-    static constexpr int kBTile = kBRows * kSK * 2;
-    // A region of a stage: the expanded weight tile, 128 rows x kSK bytes.  The one-CTA kernel's dense stages are
-    // 32 columns wide so that their A2 tile fits there too: a smaller stage means more stages in
-    // flight.  The dense-only launch has no expanded tiles; it and the pair have 64-column dense stages.
+    static constexpr int kBTile = N * 128;
+    // A region of a stage: the expanded weight tile needs 8 KB.  The main launch's dense stages are 32 columns wide so
+    // that their A2 tile fits there too: a smaller stage means more stages in flight, and the loop is bound by the
+    // latency of the token tile.  The dense-only launch has no expanded tiles and keeps 64-column stages.
     static constexpr int kARegion = PRE ? kATile : kPM * kSK;
-    static constexpr int kDK = PRE || TWO ? 64 : 32;                        // columns of a dense stage
-    static constexpr int kStages = PRE ? (N >= 256 ? 4 : 8) : (TWO ? 4 : (N >= 256 ? 5 : 8));
-    // Packed tiles come from HBM (latency of a microsecond or two): the ring holds what fits.
-    static constexpr int kPkSlots = PRE ? 1 : (TWO ? 2 : (N >= 256 ? 2 : 7));
+    static constexpr int kDK = PRE ? 64 : 32;                               // columns of a dense stage
+    static constexpr int kStages = PRE && N >= 256 ? 4 : 8;
+    static constexpr int kPkSlots = PRE ? 1 : 7;                            // packed tiles come from HBM: the ring holds what fits
     static constexpr int kStageBytes = kBTile + kARegion;
     static constexpr int kECol = N;                                         // index words: N + 4 * stage + mma
-    static constexpr int kTmemCols = N >= 256 ? 512 : (N >= 128 ? 256 : 128);
+    static constexpr int kTmemCols = N >= 256 ? 512 : 128;
     static constexpr size_t kSmem = 1024 + (size_t)kStages * kStageBytes + kPkSlots * kPkSlotBytes + 1024;
 };
 
@@ -107,6 +100,7 @@ struct PrefillParams {
     const uint8_t* meta;
     int meta_pitch;
     int d_in;
+    int row_pairs, tiles;   // pair kernel: pairs of 128-row tiles; tiles of 256 x 256 in all
 };
 
 // Optional timeline: built with -DSLIM_PREFILL_TRACE, one thread per warp role of the first
@@ -228,6 +222,9 @@ __device__ __forceinline__ void mma_commit2(uint64_t* bar) {
 __device__ __forceinline__ void mbar_arrive_remote(uint32_t cluster_bar_addr) {
     asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" :: "r"(cluster_bar_addr) : "memory");
 }
+__device__ __forceinline__ void mbar_arrive_remote_release(uint32_t cluster_bar_addr) {
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" :: "r"(cluster_bar_addr) : "memory");
+}
 // One try_wait, no loop.  `cluster`: acquire at cluster scope (arrivals came from the other CTA).
 __device__ __forceinline__ uint32_t mbar_try(uint64_t* bar, uint32_t parity, bool cluster) {
     uint32_t done;
@@ -309,14 +306,73 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
 
 }  // namespace pf
 
-template <int N, bool TWO, bool PRE = false>
+// One packed tile (128 rows x 256 weight columns, group `kg` along them) into a slot; called by a whole warp.
+__device__ __forceinline__ void load_packed(const PrefillParams& p, const CUtensorMap* tmV, const CUtensorMap* tmM, unsigned char* slot,
+                                            uint64_t* full, int kg, int m0, int lane)
+{
+    using namespace pf;
+    if (lane == 0) mbar_expect_tx(full, (uint32_t)(p.meta ? kValsTile : kPkSlotBytes));
+    // lanes 0 and 1 request the value-byte and the index-byte tile with one instruction
+    if (lane < (p.meta ? 1 : 2)) tma_tile(slot + (lane == 0 ? 0 : kValsTile), lane == 0 ? tmV : tmM, kg * (lane == 0 ? 64 : 32), m0, full);
+    if (p.meta) {
+        // 128 rows x four 8-byte pieces (64 columns each), stored as the TMA's 32-byte swizzle would
+        const int q = lane & 3;
+        const bool col_in = kg * 32 + q * 8 < p.meta_pitch;
+#pragma unroll 4
+        for (int r = lane >> 2; r < kPM; r += 8) {
+            const bool in = col_in && m0 + r < p.m_total;
+            const uint8_t* src = p.meta + (in ? (size_t)(m0 + r) * p.meta_pitch + kg * 32 + q * 8 : 0);
+            const uint32_t d = s32(slot + kValsTile) + r * 32 + ((((q >> 1) ^ (r >> 2)) & 1) << 4) + (q & 1) * 8;
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" :: "r"(d), "l"(src), "r"(in ? 8 : 0) : "memory");
+        }
+        asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" :: "r"(s32(full)) : "memory");
+    }
+}
+
+// One weight row of a stage of SK (64 or 128) columns, the q-th of its packed tile: 16 value bytes -> 32 bf16 per 64
+// columns into the K-major A tile (rows of SK bytes, swizzle of that width), and the row's part of the index words of
+// the stage's MMAs (layout in the file header).  The packed tiles are stored with the 64-byte (values) and 32-byte
+// (indices) TMA swizzles so that a warp's row-strided reads spread over the banks.  Rows past the last (!row_in) and columns
+// past it (cols_left) get a legal pair of positions.
+template <int SK>
+__device__ __forceinline__ void expand_row(const unsigned char* pk, unsigned char* a_tile, int row, int q, int x, bool row_in, int cols_left,
+                                           uint32_t (&e)[SK / 32])
+{
+    unsigned char* arow = a_tile + row * SK;
+#pragma unroll
+    for (int hh = 0; hh < SK / 64; ++hh) {
+        const int qq = q * (SK / 64) + hh;                   // which 64 columns of the packed tile
+        const uint4 v = *reinterpret_cast<const uint4*>(pk + row * 64 + (((qq ^ (row >> 1)) & 3) << 4));
+        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const uint32_t ws = w[c] >> 4;
+            uint4 o;
+            o.x = pf::nib2bf16<0>(w[c], ws); o.y = pf::nib2bf16<1>(w[c], ws);
+            o.z = pf::nib2bf16<2>(w[c], ws); o.w = pf::nib2bf16<3>(w[c], ws);
+            const int chunk = SK == 128 ? ((hh * 4 + c) ^ row) & 7 : (c ^ (row >> 1)) & 3;
+            *reinterpret_cast<uint4*>(arow + (chunk << 4)) = o;
+        }
+        uint2 mw2 = *reinterpret_cast<const uint2*>(pk + kValsTile + row * 32 + ((((qq >> 1) ^ (row >> 2)) & 1) << 4) + (qq & 1) * 8);
+        if (!row_in || hh * 64 >= cols_left) mw2 = make_uint2(0x44444444u, 0x44444444u);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const uint32_t mw = h ? mw2.y : mw2.x;
+            const uint32_t send = x ? (mw & 0xFFFFu) : (mw >> 16);
+            const uint32_t recv = __shfl_xor_sync(0xffffffffu, send, 8);
+            e[hh * 2 + h] = x ? ((mw & 0xFFFF0000u) | recv) : ((mw & 0xFFFFu) | (recv << 16));
+        }
+    }
+}
+
+template <int N, bool PRE = false>
 __global__ void __launch_bounds__(kPThreads, 1)
 prefill_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap tmV,
                const __grid_constant__ CUtensorMap tmM, const __grid_constant__ CUtensorMap tmX,
                const __grid_constant__ CUtensorMap tmA2, const __grid_constant__ CUtensorMap tmB2)
 {
     using namespace pf;
-    using Cfg = PfCfg<N, TWO, PRE>;
+    using Cfg = PfCfg<N, PRE>;
     // The dense-only launch lets the launches behind it start at once (programmatic dependent launch): the
     // main launch's sparse stages do not need T', and it waits (griddepcontrol.wait) just before its first
     // request of a T' tile.
@@ -338,38 +394,30 @@ prefill_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap tmV,
     volatile uint32_t* abort_flag = tmem_slot + 1;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t rank = TWO ? cluster_rank() : 0u;           // 0 = the CTA that issues the pair's MMAs
     const int m0 = blockIdx.x * kPM, n0 = blockIdx.y * N;
-    const int nb0 = n0 + (int)rank * Cfg::kBRows;                // first token row this CTA loads
     const int k_first = PRE && p.part ? (int)blockIdx.z * p.k_per : 0;      // first dense stage of this K slice
     const int n_total = PRE && p.part ? min(p.k_per, p.n2 - k_first) : p.n1 + p.n2;
     // CTAs that share token rows start their walk over the weight columns at different places,
     // so that at any moment they ask the L2 for different lines of X rather than all for the same
-    // ones.  The walk is rotated by whole 256-column groups (a pair of CTAs rotates together).
+    // ones.  The walk is rotated by whole 256-column groups.
     const int n_groups = ceil_div(p.n1, kPkStages);
     const int rot_g = (p.d_in % kPkCols == 0 && n_groups > 0)
-                          ? (int)(((blockIdx.x >> (TWO ? 1 : 0)) + 3u * blockIdx.y) % (unsigned)n_groups) : 0;
+                          ? (int)((blockIdx.x + 3u * blockIdx.y) % (unsigned)n_groups) : 0;
 
     if (threadIdx.x == 0) PSTAMP(5, 44);
     if (threadIdx.x == 0) {
         for (int i = 0; i < kPStages; ++i) {
             mbar_init(&b_full[i], 1);
-            mbar_init(&conv_done[i], TWO ? kConvWarps : kConvWarps / 2); mbar_init(&empty[i], 1);
+            mbar_init(&conv_done[i], kConvWarps / 2); mbar_init(&empty[i], 1);
         }
         for (int i = 0; i < kPkSlots; ++i) { mbar_init(&pk_full[i], p.meta ? 33 : 1); mbar_init(&pk_empty[i], kConvWarps); }
         mbar_init(acc_full, 1);
         *abort_flag = 0u;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (TWO) cluster_sync_all();                    // both CTAs' barriers exist before anything crosses
     if (warp == kWarpMma) {
-        if (TWO) {
-            asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" :: "r"(s32(tmem_slot)), "r"(Cfg::kTmemCols) : "memory");
-            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
-        } else {
-            asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" :: "r"(s32(tmem_slot)), "r"(Cfg::kTmemCols) : "memory");
-            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-        }
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" :: "r"(s32(tmem_slot)), "r"(Cfg::kTmemCols) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     fence_before_sync();
     __syncthreads();
@@ -397,62 +445,38 @@ prefill_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap tmV,
             // spins: that costs some hundred nanoseconds per stage); lane 0 arms the barrier.
             if (it >= kPStages) ok = mbar_wait(&empty[st], ((it / kPStages) & 1) ^ 1, abort_flag) && ok;
             // dense stage: kDK columns of the token rows and of the A2 rows
-            // a pair's bytes, both CTAs', are counted on the even CTA's barrier
-            if (lane == 0 && rank == 0)
-                mbar_expect_tx(&b_full[st], (uint32_t)((TWO ? 2 : 1) * (sparse ? kBTile : (Cfg::kBRows + kPM) * kDK * 2)));
+            // dense stage: kDK columns of the token rows and of the A2 rows
+            if (lane == 0) mbar_expect_tx(&b_full[st], (uint32_t)(sparse ? kBTile : (N + kPM) * kDK * 2));
             unsigned char* sbase = stages + (size_t)st * kStageBytes;
             int kb = sparse ? it + rot_g * kPkStages : it - p.n1 + k_first;
             if (sparse && kb >= p.n1) kb -= p.n1;
-            const int k = sparse ? kb * kSK : kb * kDK;
-            // sparse stage: the token tile, a box per 64 columns; dense stage: lane 0 the token tile, lane 1 the A2 tile
-            if (lane < (sparse ? kSK / kPBK : 2)) {
-                const CUtensorMap* map = sparse ? &tmX : lane == 0 ? &tmB2 : &tmA2;
-                unsigned char* dst = sbase + (lane == 0 ? 0 : sparse ? Cfg::kBRows * 128 : kBTile);
-                const int x = sparse ? k + lane * kPBK : k, y = !sparse && lane == 1 ? m0 : nb0;
-                if (TWO) tma_tile_pair(dst, map, x, y, peer_addr(&b_full[st], 0));
-                else tma_tile(dst, map, x, y, &b_full[st]);
-            }
+            const int k = kb * (sparse ? kSK : kDK);
+            // lane 0: the token tile (one box); lane 1, dense stages only: the A2 tile
+            if (lane == 0 || (lane == 1 && !sparse))
+                tma_tile(lane == 0 ? sbase : sbase + kBTile, lane == 1 ? &tmA2 : (sparse ? &tmX : &tmB2), k, lane == 0 ? n0 : m0, &b_full[st]);
             if (lane == 0) PSTAMP(0, it);
         }
     } else if (warp == kWarpPk) {
         // ============================ packed-tile producer ============================
-        // lanes 0 and 1 request the value-byte and the index-byte tile with one instruction
         for (int gi = 0; gi < n_groups; ++gi) {
             const int slot = gi % kPkSlots;
             const int g = gi + rot_g < n_groups ? gi + rot_g : gi + rot_g - n_groups;
             if (gi >= kPkSlots) ok = mbar_wait(&pk_empty[slot], ((gi / kPkSlots) & 1) ^ 1, abort_flag) && ok;
-            if (lane == 0) mbar_expect_tx(&pk_full[slot], (uint32_t)(p.meta ? kValsTile : kPkSlotBytes));
-            unsigned char* dst = packed + slot * kPkSlotBytes + (lane == 0 ? 0 : kValsTile);
-            if (lane < (p.meta ? 1 : 2)) tma_tile(dst, lane == 0 ? &tmV : &tmM, g * (lane == 0 ? 64 : 32), m0, &pk_full[slot]);
-            if (p.meta) {
-                // 128 rows x four 8-byte pieces (64 columns each), stored as the TMA's 32-byte swizzle would
-                const int q = lane & 3;
-                const bool col_in = g * 32 + q * 8 < p.meta_pitch;
-#pragma unroll 4
-                for (int r = lane >> 2; r < kPM; r += 8) {
-                    const bool in = col_in && m0 + r < p.m_total;
-                    const uint8_t* src = p.meta + (in ? (size_t)(m0 + r) * p.meta_pitch + g * 32 + q * 8 : 0);
-                    const uint32_t d = s32(packed + slot * kPkSlotBytes + kValsTile) + r * 32 + ((((q >> 1) ^ (r >> 2)) & 1) << 4) + (q & 1) * 8;
-                    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" :: "r"(d), "l"(src), "r"(in ? 8 : 0) : "memory");
-                }
-                asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" :: "r"(s32(&pk_full[slot])) : "memory");
-            }
+            load_packed(p, &tmV, &tmM, packed + slot * kPkSlotBytes, &pk_full[slot], g, m0, lane);
         }
     } else if (warp == kWarpMma) {
         // ============================ MMA issuer ============================
         // One elected lane walks the stages and issues.
-        if (TWO && rank != 0) {
-            // the even CTA issues the pair's MMAs
-        } else if (elect_one()) {
-            constexpr uint32_t idesc = idesc_bf16(TWO ? 2 * kPM : kPM, N);
+        if (elect_one()) {
+            constexpr uint32_t idesc = idesc_bf16(kPM, N);
             uint32_t pre = 0;       // the coming stage was found ready by an early test
             for (int it = 0; it < n_total; ++it) {
                 const int st = it % kPStages;
                 const uint32_t parity = (it / kPStages) & 1;
                 const bool sparse = it < p.n1;
-                // token tile landed; converters done (in a pair: both CTAs', reported here)
+                // token tile landed; converters done
                 if (!pre)
-                    ok = mbar_wait_all(&b_full[st], parity, TWO, sparse ? &conv_done[st] : nullptr, parity, TWO,
+                    ok = mbar_wait_all(&b_full[st], parity, false, sparse ? &conv_done[st] : nullptr, parity, false,
                                        nullptr, 0, false, abort_flag) && ok;
                 fence_after_sync();
                 // ask about the next stage now, without waiting: the answer comes back while this stage's
@@ -461,8 +485,8 @@ prefill_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap tmV,
                 if (it + 1 < n_total) {
                     const int st1 = (it + 1) % kPStages;
                     const uint32_t par1 = ((it + 1) / kPStages) & 1;
-                    pre = mbar_test(&b_full[st1], par1, TWO);
-                    if (it + 1 < p.n1) pre &= mbar_test(&conv_done[st1], par1, TWO);
+                    pre = mbar_test(&b_full[st1], par1, false);
+                    if (it + 1 < p.n1) pre &= mbar_test(&conv_done[st1], par1, false);
                 }
                 const uint32_t b_addr = s32(stages + (size_t)st * kStageBytes);
                 const uint32_t a_addr = b_addr + kBTile;
@@ -472,28 +496,22 @@ prefill_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap tmV,
 #pragma unroll
                     for (int j = 0; j < kSK / 32; ++j) {
                         const uint32_t acc = (it > 0 || j > 0) ? 1u : 0u;
-                        const uint32_t e_col = tmem_base + kECol + 4 * st + 2 * (j >> 1);
-                        const uint64_t bd = smem_desc(b_addr + (j >> 1) * (Cfg::kBRows * 128) + 64 * (j & 1));
-                        if (TWO) mma_sparse2(tmem_base, smem_desc(a_addr + 32 * j), bd, e_col, idesc | (1u << 2) | (uint32_t)(j & 1), acc);
-                        else     mma_sparse(tmem_base, smem_desc64(a_addr + 32 * j), bd, e_col, idesc | (1u << 2) | (uint32_t)(j & 1), acc);
+                        const uint32_t e_col = tmem_base + kECol + 4 * st;
+                        mma_sparse(tmem_base, smem_desc64(a_addr + 32 * j), smem_desc(b_addr + 64 * j), e_col, idesc | (1u << 2) | (uint32_t)j, acc);
                     }
                 } else {
 #pragma unroll
                     for (int j = 0; j < kDK / 16; ++j) {
                         const uint32_t acc = (it > 0 || j > 0) ? 1u : 0u;
                         // 32-column stages: 64-byte rows with the 64-byte swizzle; 64-column stages: 128-byte rows
-                        if (TWO)            mma_dense2(tmem_base, smem_desc(a_addr + 32 * j), smem_desc(b_addr + 32 * j), idesc, acc);
-                        else if (kDK == 32) mma_dense(tmem_base, smem_desc64(a_addr + 32 * j), smem_desc64(b_addr + 32 * j), idesc, acc);
-                        else                mma_dense(tmem_base, smem_desc(a_addr + 32 * j), smem_desc(b_addr + 32 * j), idesc, acc);
+                        if (kDK == 32) mma_dense(tmem_base, smem_desc64(a_addr + 32 * j), smem_desc64(b_addr + 32 * j), idesc, acc);
+                        else           mma_dense(tmem_base, smem_desc(a_addr + 32 * j), smem_desc(b_addr + 32 * j), idesc, acc);
                     }
                 }
-                // the stage is free (in both CTAs of a pair) once these MMAs have read it
-                if (TWO) mma_commit2(&empty[st]);
-                else mma_commit(&empty[st]);
+                mma_commit(&empty[st]);             // the stage is free once these MMAs have read it
                 PSTAMP(4, it);
             }
-            if (TWO) mma_commit2(acc_full);
-            else mma_commit(acc_full);
+            mma_commit(acc_full);
         }
     } else {
         // ============================ converters, then epilogue ============================
@@ -513,55 +531,17 @@ prefill_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap tmV,
             ok = mbar_wait_all(&pk_full[slot], (gi / kPkSlots) & 1, false, it >= kPStages ? &empty[st] : nullptr,
                                ((it / kPStages) & 1) ^ 1, false, nullptr, 0, false, abort_flag) && ok;
             if ((threadIdx.x & 127) == 0) PSTAMP(1, it);
-            // ---- 16 value bytes -> 32 bf16 per 64 columns; the packed tiles are stored with the 64-byte (values) and 32-byte
-            // (indices) TMA swizzles so that a warp's row-strided reads spread over the banks
-            unsigned char* arow = stages + (size_t)st * kStageBytes + kBTile + row * kSK;
-#pragma unroll
-            for (int hh = 0; hh < kSK / 64; ++hh) {
-                const int qq = q * (kSK / 64) + hh;          // which 64 columns of the packed tile
-                const uint4 v = *reinterpret_cast<const uint4*>(pk + row * 64 + (((qq ^ (row >> 1)) & 3) << 4));
-                const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    const uint32_t ws = w[c] >> 4;
-                    uint4 o;
-                    o.x = nib2bf16<0>(w[c], ws); o.y = nib2bf16<1>(w[c], ws);
-                    o.z = nib2bf16<2>(w[c], ws); o.w = nib2bf16<3>(w[c], ws);
-                    const int chunk = TWO ? ((hh * 4 + c) ^ row) & 7 : (c ^ (row >> 1)) & 3;      // 128- or 64-byte rows and swizzle
-                    *reinterpret_cast<uint4*>(arow + (chunk << 4)) = o;
-                }
-            }
-            // ---- index words of the stage's MMAs (layout in the file header)
-            uint32_t e[kSK / 32];
-#pragma unroll
-            for (int hh = 0; hh < kSK / 64; ++hh) {
-                const int qq = q * (kSK / 64) + hh;
-                uint2 mw2 = *reinterpret_cast<const uint2*>(pk + kValsTile + row * 32 + ((((qq >> 1) ^ (row >> 2)) & 1) << 4) + (qq & 1) * 8);
-                // past the last row or column: a legal pair of positions
-                if (m0 + row >= p.m_total || (TWO && it * kSK + hh * 64 >= p.d_in)) mw2 = make_uint2(0x44444444u, 0x44444444u);
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const uint32_t mw = h ? mw2.y : mw2.x;
-                    const uint32_t send = x ? (mw & 0xFFFFu) : (mw >> 16);
-                    const uint32_t recv = __shfl_xor_sync(0xffffffffu, send, 8);
-                    e[hh * 2 + h] = x ? ((mw & 0xFFFF0000u) | recv) : ((mw & 0xFFFFu) | (recv << 16));
-                }
-            }
-            if constexpr (TWO)
-                asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};"
-                             :: "r"(tmem_base + lane_base + kECol + 4 * st), "r"(e[0]), "r"(e[1]), "r"(e[kSK / 32 - 2]), "r"(e[kSK / 32 - 1]) : "memory");
-            else
-                asm volatile("tcgen05.st.sync.aligned.32x32b.x2.b32 [%0], {%1, %2};"
-                             :: "r"(tmem_base + lane_base + kECol + 4 * st), "r"(e[0]), "r"(e[1]) : "memory");
+            uint32_t e[2];
+            expand_row<64>(pk, stages + (size_t)st * kStageBytes + kBTile, row, q, x, m0 + row < p.m_total, 64, e);
+            asm volatile("tcgen05.st.sync.aligned.32x32b.x2.b32 [%0], {%1, %2};"
+                         :: "r"(tmem_base + lane_base + kECol + 4 * st), "r"(e[0]), "r"(e[1]) : "memory");
             asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // A is read by the tensor core
             fence_before_sync();
             // one arrival per warp: arrivals on one barrier are served one after another
             __syncwarp();
             if (lane == 0) {
-                // a pair's MMAs are issued by the even CTA: both CTAs' converters report there
-                if (TWO && rank != 0) mbar_arrive_remote(peer_addr(&conv_done[st], 0));
-                else mbar_arrive(&conv_done[st]);
+                mbar_arrive(&conv_done[st]);
                 // this group's last stage of the packed tile
                 if (q + 2 >= kPkStages || it + 2 >= p.n1) mbar_arrive(&pk_empty[slot]);
             }
@@ -593,11 +573,253 @@ prefill_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap tmV,
     if (!ok && lane == 0) flag_error(p.status, SLIM_ERR_TIMEOUT);
     fence_before_sync();
     __syncthreads();
-    if (TWO) cluster_sync_all();                    // neither CTA leaves while the other may still read its shared memory
     if (warp == kWarpMma) {
         fence_after_sync();
-        if (TWO) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" :: "r"(tmem_base), "r"(Cfg::kTmemCols) : "memory");
-        else     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem_base), "r"(Cfg::kTmemCols) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem_base), "r"(Cfg::kTmemCols) : "memory");
+    }
+}
+
+// ---------------------------------------------------------------- the wide kernel: persistent CTA pairs
+// A cluster of two CTAs computes tiles of 256 output rows x 256 tokens with cta_group::2 MMAs issued by the even CTA: each
+// CTA loads and expands its own 128 rows of the weight and loads half of the token tile.  Stages are 128 weight
+// columns (four MMAs of K = 32 per commit; 64 columns of the adapters in phase 2).
+// The pairs are persistent: pair c takes tiles c, c + pairs, ..., and all rings run on across tiles, so that the next
+// tile's operands are loaded and expanded while this tile ends.  Eight warps of their own read the accumulator out:
+// 128 tokens a thread; the next tile's MMAs may start as soon as it is in registers, the stores follow beside
+// them.  A CTA per tile spent 4.4 us on start-up and 2.3 us on the epilogue of every tile, with the tensor
+// core idle.
+// Warps: 0-7 converters (two groups on alternate stages), 8-15 epilogue, 16 token tiles (and A2 / B2), 17 MMA issue,
+// 18 packed tiles.
+struct PairCfg {
+    static constexpr int kN = 256, kThreads = 19 * 32;
+    static constexpr int kWarpX = 16, kWarpMma = 17, kWarpPk = 18;
+    static constexpr int kSK = 128, kDK = 64, kStages = 4, kPkSlots = 2, kPkStages = kPkCols / kSK;
+    static constexpr int kHalfTok = kN / 2;                                 // token rows this CTA loads
+    static constexpr int kBTile = kHalfTok * kSK * 2, kStageBytes = kBTile + kPM * kSK;
+    static constexpr int kECol = kN;                                        // index words: kN + 4 * stage + mma
+    static constexpr size_t kSmem = 1024 + (size_t)kStages * kStageBytes + kPkSlots * kPkSlotBytes + 512;
+};
+
+__global__ void __launch_bounds__(PairCfg::kThreads, 1)
+prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmM,
+                    const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmA2, const __grid_constant__ CUtensorMap tmB2)
+{
+    using namespace pf;
+    using Cfg = PairCfg;
+    constexpr int kStages = Cfg::kStages, kPkSlots = Cfg::kPkSlots, kPkStages = Cfg::kPkStages, kSK = Cfg::kSK, kDK = Cfg::kDK;
+    constexpr int kBTile = Cfg::kBTile, kStageBytes = Cfg::kStageBytes, kECol = Cfg::kECol, kHalfTok = Cfg::kHalfTok;
+    extern __shared__ unsigned char smem_raw[];
+    // layout: stages {B | A} | packed slots {value bytes | index bytes} | barriers
+    unsigned char* stages = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    unsigned char* packed = stages + (size_t)kStages * kStageBytes;
+    uint64_t* b_full = reinterpret_cast<uint64_t*>(packed + kPkSlots * kPkSlotBytes);   // [kStages] even CTA: both CTAs' tiles landed
+    uint64_t* conv_done = b_full + kStages;          // [kStages] even CTA: both CTAs' converters are done with the stage
+    uint64_t* empty = conv_done + kStages;           // [kStages] the MMAs that read the stage are complete
+    uint64_t* pk_full = empty + kStages;             // [kPkSlots]
+    uint64_t* pk_empty = pk_full + kPkSlots;         // [kPkSlots]
+    uint64_t* acc_full = pk_empty + kPkSlots;        // a tile's MMAs are complete
+    uint64_t* acc_empty = acc_full + 1;              // even CTA: both CTAs have read the accumulator
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 1);
+    volatile uint32_t* abort_flag = tmem_slot + 1;
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t rank = cluster_rank();
+    const int pairs = gridDim.x >> 1, first_tile = blockIdx.x >> 1;
+    const int n_total = p.n1 + p.n2, n_groups = ceil_div(p.n1, kPkStages);
+
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < kStages; ++i) { mbar_init(&b_full[i], 1); mbar_init(&conv_done[i], kConvWarps); mbar_init(&empty[i], 1); }
+        for (int i = 0; i < kPkSlots; ++i) { mbar_init(&pk_full[i], p.meta ? 33 : 1); mbar_init(&pk_empty[i], kConvWarps); }
+        mbar_init(acc_full, 1);
+        mbar_init(acc_empty, 16);
+        *abort_flag = 0u;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    cluster_sync_all();                              // both CTAs' barriers exist before anything crosses
+    if (warp == Cfg::kWarpMma) {
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" :: "r"(s32(tmem_slot)), "r"(512) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    }
+    fence_before_sync();
+    __syncthreads();
+    fence_after_sync();
+    const uint32_t tmem_base = *reinterpret_cast<volatile uint32_t*>(tmem_slot);
+    bool ok = true;
+    // Tile -> its first row in this CTA, its first token, and where its walk over the weight columns starts: pairs that share
+    // token rows start at different places, so that at any moment they ask the L2 for different lines of X.
+    struct Tile { int m0, n0, rot; };
+    auto tile_of = [&](int t) {
+        const int rp = t % p.row_pairs, tt = t / p.row_pairs;
+        Tile ti;
+        ti.m0 = (2 * rp + (int)rank) * kPM; ti.n0 = tt * Cfg::kN;
+        ti.rot = p.d_in % kPkCols == 0 && n_groups > 0 ? (rp + 3 * tt) % n_groups : 0;       // whole packed tiles
+        return ti;
+    };
+
+    if (warp == Cfg::kWarpX) {
+        // ============================ token tiles, A2, B2 ============================
+        bool t_ready = false;                               // T' (and everything before it) is complete
+        int g = 0;                                          // stages so far
+        for (int t = first_tile; t < p.tiles; t += pairs) {
+            const Tile ti = tile_of(t);
+            for (int it = 0; it < n_total; ++it, ++g) {
+                const int st = g % kStages;
+                const bool sparse = it < p.n1;
+                if (!sparse && !t_ready) {
+                    asm volatile("griddepcontrol.wait;" ::: "memory");
+                    asm volatile("fence.proxy.async;" ::: "memory");   // the tiles are read by the async proxy
+                    t_ready = true;
+                }
+                if (g >= kStages) ok = mbar_wait(&empty[st], ((g / kStages) & 1) ^ 1, abort_flag) && ok;
+                // both CTAs' bytes are counted on the even CTA's barrier
+                if (lane == 0 && rank == 0) mbar_expect_tx(&b_full[st], (uint32_t)(2 * (sparse ? kBTile : (kHalfTok + kPM) * kDK * 2)));
+                unsigned char* sbase = stages + (size_t)st * kStageBytes;
+                int kb = sparse ? it + ti.rot * kPkStages : it - p.n1;
+                if (sparse && kb >= p.n1) kb -= p.n1;
+                const int k = kb * (sparse ? kSK : kDK);
+                // sparse stage: the token tile, two boxes of 64 columns; dense stage: lane 0 the token tile, lane 1 the A2 tile
+                if (lane < 2) {
+                    const CUtensorMap* map = sparse ? &tmX : lane == 0 ? &tmB2 : &tmA2;
+                    unsigned char* dst = sbase + (lane == 0 ? 0 : sparse ? kHalfTok * 128 : kBTile);
+                    tma_tile_pair(dst, map, sparse ? k + lane * kPBK : k, !sparse && lane == 1 ? ti.m0 : ti.n0 + (int)rank * kHalfTok, peer_addr(&b_full[st], 0));
+                }
+            }
+        }
+    } else if (warp == Cfg::kWarpPk) {
+        // ============================ packed tiles ============================
+        int g = 0;
+        for (int t = first_tile; t < p.tiles; t += pairs) {
+            const Tile ti = tile_of(t);
+            for (int i = 0; i < n_groups; ++i, ++g) {
+                const int slot = g % kPkSlots;
+                const int kg = i + ti.rot < n_groups ? i + ti.rot : i + ti.rot - n_groups;
+                if (g >= kPkSlots) ok = mbar_wait(&pk_empty[slot], ((g / kPkSlots) & 1) ^ 1, abort_flag) && ok;
+                load_packed(p, &tmV, &tmM, packed + slot * kPkSlotBytes, &pk_full[slot], kg, ti.m0, lane);
+            }
+        }
+    } else if (warp == Cfg::kWarpMma) {
+        // ============================ MMA issue: one thread of the even CTA ============================
+        if (rank == 0 && elect_one()) {
+            constexpr uint32_t idesc = idesc_bf16(2 * kPM, Cfg::kN);
+            uint32_t pre = 0;       // the coming stage was found ready by an early test
+            int g = 0, nth = 0;
+            for (int t = first_tile; t < p.tiles; t += pairs, ++nth) {
+                if (nth > 0) ok = mbar_wait_all(acc_empty, (nth & 1) ^ 1, true, nullptr, 0, false, nullptr, 0, false, abort_flag) && ok;
+                for (int it = 0; it < n_total; ++it, ++g) {
+                    const int st = g % kStages;
+                    const uint32_t parity = (g / kStages) & 1;
+                    const bool sparse = it < p.n1;
+                    if (!pre)
+                        ok = mbar_wait_all(&b_full[st], parity, true, &conv_done[st], parity, true, nullptr, 0, false, abort_flag) && ok;
+                    fence_after_sync();
+                    // ask about the next stage now, without waiting: the answer comes back while this stage's MMAs are issued
+                    const int st1 = (g + 1) % kStages;
+                    const uint32_t par1 = ((g + 1) / kStages) & 1;
+                    pre = mbar_test(&b_full[st1], par1, true) & mbar_test(&conv_done[st1], par1, true);
+                    const uint32_t b_addr = s32(stages + (size_t)st * kStageBytes), a_addr = b_addr + kBTile;
+                    if (sparse) {
+                        // per MMA: A 16 stored bf16 (32 bytes of a 128-byte row), B 32 columns (64 bytes)
+#pragma unroll
+                        for (int j = 0; j < kSK / 32; ++j)
+                            mma_sparse2(tmem_base, smem_desc(a_addr + 32 * j), smem_desc(b_addr + (j >> 1) * (kHalfTok * 128) + 64 * (j & 1)),
+                                        tmem_base + kECol + 4 * st + 2 * (j >> 1), idesc | (1u << 2) | (uint32_t)(j & 1), it > 0 || j > 0 ? 1u : 0u);
+                    } else {
+#pragma unroll
+                        for (int j = 0; j < kDK / 16; ++j)
+                            mma_dense2(tmem_base, smem_desc(a_addr + 32 * j), smem_desc(b_addr + 32 * j), idesc, it > 0 || j > 0 ? 1u : 0u);
+                    }
+                    mma_commit2(&empty[st]);            // the stage is free, in both CTAs, once these MMAs have read it
+                }
+                mma_commit2(acc_full);
+            }
+        }
+    } else if (warp < kConvWarps) {
+        // ============================ converters ============================
+        // Within a group of four warps a thread owns one weight row of the tile.
+        const int row = threadIdx.x & 127;           // weight row inside the tile = TMEM lane
+        const int half = threadIdx.x >> 7;
+        const int x = (row >> 3) & 1;
+        const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
+        int base = 0, nth = 0;                       // stages before this tile
+        for (int t = first_tile; t < p.tiles; t += pairs, base += n_total, ++nth) {
+            const bool row_in = tile_of(t).m0 + row < p.m_total;
+            for (int it = (base ^ half) & 1; it < n_total; it += 2) {
+                const int g = base + it, st = g % kStages;
+                uint64_t* free_bar = g >= kStages ? &empty[st] : nullptr;        // the MMAs of the stage's previous use
+                const uint32_t free_par = ((g / kStages) & 1) ^ 1;
+                if (it < p.n1) {
+                    const int gi = nth * n_groups + it / kPkStages, q = it % kPkStages, slot = gi % kPkSlots;
+                    ok = mbar_wait_all(&pk_full[slot], (gi / kPkSlots) & 1, false, free_bar, free_par, false, nullptr, 0, false, abort_flag) && ok;
+                    uint32_t e[4];
+                    expand_row<128>(packed + slot * kPkSlotBytes, stages + (size_t)st * kStageBytes + kBTile, row, q, x, row_in, p.d_in - it * kSK, e);
+                    asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};"
+                                 :: "r"(tmem_base + lane_base + kECol + 4 * st), "r"(e[0]), "r"(e[1]), "r"(e[2]), "r"(e[3]) : "memory");
+                    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // A is read by the tensor core
+                    fence_before_sync();
+                    __syncwarp();
+                    if (lane == 0) {
+                        mbar_arrive_remote(peer_addr(&conv_done[st], 0));
+                        // a packed tile's last stage alone: in place of the other group too
+                        mbar_arrive(&pk_empty[slot]);
+                        if (q == 0 && it + 1 == p.n1) mbar_arrive(&pk_empty[slot]);
+                    }
+                } else {
+                    // nothing to expand in phase 2: the arrival keeps the barrier's phases in step with the stages
+                    if (free_bar) ok = mbar_wait(free_bar, free_par, abort_flag) && ok;
+                    if (lane == 0) mbar_arrive_remote(peer_addr(&conv_done[st], 0));
+                    __syncwarp();
+                }
+            }
+        }
+    } else {
+        // ============================ epilogue: thread = output row, half of the tokens ============================
+        const int half = (warp - kConvWarps) >> 2;
+        const int row = (warp & 3) * 32 + lane;
+        const uint32_t taddr = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + half * kHalfTok;
+        int nth = 0;
+        for (int t = first_tile; t < p.tiles; t += pairs, ++nth) {
+            const Tile ti = tile_of(t);
+            ok = mbar_wait(acc_full, nth & 1, abort_flag) && ok;
+            fence_after_sync();
+            const int orow = ti.m0 + row, tok0 = ti.n0 + half * kHalfTok;
+            __nv_bfloat16* out = p.out + (size_t)tok0 * p.ldo + orow;
+            const int n_tok = orow < p.m_total ? min(kHalfTok, p.b - tok0) : 0;
+            // two passes of 64 tokens (what fits in registers); the accumulator is free before the second pass's stores
+#pragma unroll
+            for (int c0 = 0; c0 < kHalfTok; c0 += 64) {
+                uint32_t y[32];                                              // bf16 pairs of neighbouring tokens
+#pragma unroll
+                for (int c1 = 0; c1 < 64; c1 += 32) {
+                    uint32_t r[32];
+                    tmem_ld32(taddr + c0 + c1, r);
+#pragma unroll
+                    for (int c = 0; c < 32; c += 2) {
+                        __nv_bfloat162 v = __floats2bfloat162_rn(p.scale * __uint_as_float(r[c]), p.scale * __uint_as_float(r[c + 1]));
+                        y[(c1 + c) / 2] = *reinterpret_cast<uint32_t*>(&v);
+                    }
+                }
+                if (c0 + 64 == kHalfTok) {
+                    fence_before_sync();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive_remote_release(peer_addr(acc_empty, 0));
+                }
+#pragma unroll
+                for (int c = 0; c < 64; ++c) {
+                    if (c0 + c < n_tok) *out = __ushort_as_bfloat16((unsigned short)(c & 1 ? y[c / 2] >> 16 : y[c / 2] & 0xFFFFu));
+                    out += p.ldo;
+                }
+            }
+        }
+    }
+
+    if (!ok && lane == 0) flag_error(p.status, SLIM_ERR_TIMEOUT);
+    fence_before_sync();
+    __syncthreads();
+    cluster_sync_all();                              // neither CTA leaves while the other may still use its shared memory
+    if (warp == Cfg::kWarpMma) {
+        fence_after_sync();
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" :: "r"(tmem_base), "r"(512) : "memory");
     }
 }
 
@@ -678,25 +900,27 @@ size_t prefill_workspace_bytes(int b, int d_out, int d_in, int r) {
 
 static std::atomic<bool> g_prefill_attr_set[64];   // attributes set once per device (setting them twice is harmless)
 
-template <int N, bool TWO, bool PRE = false>
-static slim_status_t launch_tile_kernel(const PrefillParams& q, int m_rows, const CUtensorMap& tmV, const CUtensorMap& tmM,
-                                        const CUtensorMap& tmX, const CUtensorMap& tmA2, const CUtensorMap& tmB2,
-                                        cudaStream_t st, int slices = 1, bool after_dense_only = false) {
+// `after_dense_only`: may start while the launch before it (the dense-only launch or its reduction) still runs.
+template <typename K>
+static slim_status_t launch_chained(K kernel, dim3 grid, int threads, size_t smem, int cluster, bool after_dense_only, cudaStream_t st, const PrefillParams& q,
+                                    const CUtensorMap& tmV, const CUtensorMap& tmM, const CUtensorMap& tmX, const CUtensorMap& tmA2, const CUtensorMap& tmB2) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(TWO ? 2 * ceil_div(m_rows, 2 * kPM) : ceil_div(m_rows, kPM), ceil_div(q.b, N), slices);
-    cfg.blockDim = dim3(kPThreads);
-    cfg.dynamicSmemBytes = PfCfg<N, TWO, PRE>::kSmem;
-    cfg.stream = st;
+    cfg.gridDim = grid; cfg.blockDim = dim3(threads); cfg.dynamicSmemBytes = smem; cfg.stream = st;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = TWO ? 2 : 1; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-    // may start while the launch before it (the dense-only launch or its reduction) still runs
+    attr[0].val.clusterDim.x = cluster; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr; cfg.numAttrs = after_dense_only ? 2 : 1;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, prefill_kernel<N, TWO, PRE>, q, tmV, tmM, tmX, tmA2, tmB2);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, q, tmV, tmM, tmX, tmA2, tmB2);
     count_launch(1);
     return e == cudaSuccess ? SLIM_OK : SLIM_ERR_CUDA;
+}
+template <int N, bool PRE>
+static slim_status_t launch_tile_kernel(const PrefillParams& q, int m_rows, const CUtensorMap& tmV, const CUtensorMap& tmM, const CUtensorMap& tmX,
+                                        const CUtensorMap& tmA2, const CUtensorMap& tmB2, cudaStream_t st, int slices = 1, bool after_dense_only = false) {
+    return launch_chained(prefill_kernel<N, PRE>, dim3(ceil_div(m_rows, kPM), ceil_div(q.b, N), slices), kPThreads, PfCfg<N, PRE>::kSmem, 1, after_dense_only, st,
+                          q, tmV, tmM, tmX, tmA2, tmB2);
 }
 
 slim_status_t launch_prefill(const __nv_bfloat16* X, int b, const uint8_t* vals, const uint8_t* meta,
@@ -711,11 +935,10 @@ slim_status_t launch_prefill(const __nv_bfloat16* X, int b, const uint8_t* vals,
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev >= 0 && dev < 64 && !g_prefill_attr_set[dev].load(std::memory_order_acquire)) {
-        if (cudaFuncSetAttribute(prefill_kernel<256, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PfCfg<256, true>::kSmem) != cudaSuccess ||
-            cudaFuncSetAttribute(prefill_kernel<256, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PfCfg<256, false>::kSmem) != cudaSuccess ||
+        if (cudaFuncSetAttribute(prefill_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PairCfg::kSmem) != cudaSuccess ||
             cudaFuncSetAttribute(prefill_kernel<64, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PfCfg<64, false>::kSmem) != cudaSuccess ||
-            cudaFuncSetAttribute(prefill_kernel<64, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PfCfg<64, false, true>::kSmem) != cudaSuccess ||
-            cudaFuncSetAttribute(prefill_kernel<256, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PfCfg<256, false, true>::kSmem) != cudaSuccess)
+            cudaFuncSetAttribute(prefill_kernel<64, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PfCfg<64, true>::kSmem) != cudaSuccess ||
+            cudaFuncSetAttribute(prefill_kernel<256, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PfCfg<256, true>::kSmem) != cudaSuccess)
             return SLIM_ERR_CUDA;
         g_prefill_attr_set[dev].store(true, std::memory_order_release);
     }
@@ -724,13 +947,9 @@ slim_status_t launch_prefill(const __nv_bfloat16* X, int b, const uint8_t* vals,
     // token tile: 256 when that gives a quarter of the SMs or more a tile, else 64 (measured: with 64 tiles of
     // 128 x 256 on 148 SMs the wide variant is a third faster than 256 tiles of 128 x 64; with 32 it is slower)
     const bool wide = force_pair || (long long)ceil_div(d_out, kPM) * ceil_div(b, 256) * 4 >= (long long)di->sm_count;
-    // The CTA-pair kernel (prefill_kernel<256, true>) measures 3-8 % faster than one CTA per tile on
-    // problems with adapters and a thousand tiles or more (the 70B layers at 4096 tokens) and the same or
-    // a little slower below that: it runs for those, or when asked for by name.
     if (force_pair && ceil_div(d_out, kPM) % 2 != 0) return SLIM_ERR_UNSUPPORTED_SHAPE;
-    const bool pair = force_pair || wide;
-    const int xbox = wide ? (pair ? 128 : 256) : 64;      // token rows one CTA loads per stage = one TMA box
-    const int dk = pair ? PfCfg<256, true>::kDK : PfCfg<256, false>::kDK;      // columns of a dense stage of the main kernel
+    const int xbox = wide ? PairCfg::kHalfTok : 64;       // token rows one CTA loads per stage = one TMA box
+    const int dk = wide ? PairCfg::kDK : PfCfg<64>::kDK;  // columns of a dense stage of the main kernel
     CUtensorMap tmV, tmM, tmX, tmXpre, tmA2, tmB2;
     bool ok = pf_map(&tmV, vals, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)d_in / 4, (uint64_t)d_out, kPkCols / 4, kPM, 64) &&
               (d_in % 128 != 0 || pf_map(&tmM, meta, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)d_in / 8, (uint64_t)d_out, kPkCols / 8, kPM, 32)) &&
@@ -748,8 +967,8 @@ slim_status_t launch_prefill(const __nv_bfloat16* X, int b, const uint8_t* vals,
         q.k_per = pl.k_per; q.meta = nullptr; q.meta_pitch = 0; q.d_in = d_in;
         // partial tiles of the K slices follow T' in the workspace
         q.part = pl.slices > 1 ? reinterpret_cast<float*>(reinterpret_cast<char*>(Tq) + ((size_t)b * r * sizeof(__nv_bfloat16) + 255) / 256 * 256) : nullptr;
-        slim_status_t rc = pl.n_tok == 256 ? launch_tile_kernel<256, false, true>(q, r, tmV, tmM, tmXpre, tmA2, tmXpre, st, pl.slices)
-                                           : launch_tile_kernel<64, false, true>(q, r, tmV, tmM, tmXpre, tmA2, tmXpre, st, pl.slices);
+        slim_status_t rc = pl.n_tok == 256 ? launch_tile_kernel<256, true>(q, r, tmV, tmM, tmXpre, tmA2, tmXpre, st, pl.slices)
+                                           : launch_tile_kernel<64, true>(q, r, tmV, tmM, tmXpre, tmA2, tmXpre, st, pl.slices);
         if (rc != SLIM_OK) return rc;
         if (q.part) {
             const size_t n = (size_t)b * r;
@@ -765,7 +984,7 @@ slim_status_t launch_prefill(const __nv_bfloat16* X, int b, const uint8_t* vals,
             count_launch(1);
             if (re != cudaSuccess) return SLIM_ERR_CUDA;
         }
-        // dense stages of the main kernel: 64 columns (128-byte rows), or 32 (64-byte rows) in the pair kernel
+        // dense stages of the main kernel: 64 columns (128-byte rows) in the pair kernel, else 32 (64-byte rows)
         ok = pf_map(&tmA2, L, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (uint64_t)r, (uint64_t)d_out, dk, kPM, dk == 64 ? 128 : 64) &&
              pf_map(&tmB2, Tq, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (uint64_t)r, (uint64_t)b, dk, xbox, dk == 64 ? 128 : 64);
         if (!ok) return SLIM_ERR_CUDA;
@@ -774,7 +993,7 @@ slim_status_t launch_prefill(const __nv_bfloat16* X, int b, const uint8_t* vals,
     }
     PrefillParams p;
     p.out = Y; p.ldo = d_out; p.m_total = d_out; p.b = b;
-    p.n1 = s != 0.f ? ceil_div(d_in, pair ? PfCfg<256, true>::kSK : PfCfg<256, false>::kSK) : 0;
+    p.n1 = s != 0.f ? ceil_div(d_in, wide ? PairCfg::kSK : PfCfg<64>::kSK) : 0;
     p.n2 = r > 0 ? ceil_div(r, dk) : 0;
     p.scale = s_eff; p.status = status_dev; p.part = nullptr; p.k_per = 0;
     p.meta = d_in % 128 != 0 ? meta : nullptr; p.meta_pitch = d_in / 8; p.d_in = d_in;
@@ -783,9 +1002,14 @@ slim_status_t launch_prefill(const __nv_bfloat16* X, int b, const uint8_t* vals,
     note_token_tile(wide ? 256 : 64);
     slim_status_t rc;
     const bool dep = r > 0 && p.n1 > 0;               // sparse stages to run while T' is being made
-    if (!wide) rc = launch_tile_kernel<64, false>(p, d_out, tmV, tmM, tmX, tmA2, tmB2, st, 1, dep);
-    else rc = pair ? launch_tile_kernel<256, true>(p, d_out, tmV, tmM, tmX, tmA2, tmB2, st, 1, dep)
-                   : launch_tile_kernel<256, false>(p, d_out, tmV, tmM, tmX, tmA2, tmB2, st, 1, dep);
+    p.row_pairs = ceil_div(d_out, 2 * kPM); p.tiles = p.row_pairs * ceil_div(b, PairCfg::kN);
+    if (!wide) {
+        rc = launch_tile_kernel<64, false>(p, d_out, tmV, tmM, tmX, tmA2, tmB2, st, 1, dep);
+    } else {
+        const int pairs = di->sm_count / 2;
+        rc = launch_chained(prefill_pair_kernel, dim3(2 * (p.tiles < pairs ? p.tiles : pairs)), PairCfg::kThreads, PairCfg::kSmem, 2, dep, st, p, tmV, tmM, tmX,
+                            tmA2, tmB2);
+    }
     if (rc != SLIM_OK) return rc;
     return SLIM_OK;
 }
