@@ -100,7 +100,16 @@ struct PrefillParams {
     const uint8_t* meta;
     int meta_pitch;
     int d_in;
-    int row_pairs, tiles;   // pair kernel: pairs of 128-row tiles; tiles of 256 x 256 in all
+    // pair kernel: pairs of 128-row tiles; tiles of 256 x 256 in all
+    int row_pairs, tiles;
+    // T' inside the pair kernel: chunks of t_n columns (of r), tiles of 256 tokens x t_n, 64-column stages of one, pairs that
+    // share the work; 1 / s; T' itself, partial tiles, and per (tile, CTA) {arrivals, ready} words that carry the call number
+    int r, t_n, t_chunks, t_tiles, t_stages, t_pairs;
+    float t_scale;
+    __nv_bfloat16* t_out;
+    float4* t_part;
+    unsigned long long* t_sync;
+    unsigned long long* departures;
 };
 
 // Optional timeline: built with -DSLIM_PREFILL_TRACE, one thread per warp role of the first
@@ -303,6 +312,15 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
         : "r"(taddr) : "memory");
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
+
+// 16 consecutive 32-bit columns of this thread's TMEM lane.
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float4 (&v)[4]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+                 : "=f"(v[0].x), "=f"(v[0].y), "=f"(v[0].z), "=f"(v[0].w), "=f"(v[1].x), "=f"(v[1].y), "=f"(v[1].z), "=f"(v[1].w),
+                   "=f"(v[2].x), "=f"(v[2].y), "=f"(v[2].z), "=f"(v[2].w), "=f"(v[3].x), "=f"(v[3].y), "=f"(v[3].z), "=f"(v[3].w) : "r"(taddr) : "memory");
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void epilogue_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
 
 }  // namespace pf
 
@@ -590,6 +608,12 @@ prefill_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap tmV,
 // core idle.
 // Warps: 0-7 converters (two groups on alternate stages), 8-15 epilogue, 16 token tiles (and A2 / B2), 17 MMA issue,
 // 18 packed tiles.
+//
+// T' = (X R^T) / s is made by the same pairs first: tiles of 256 tokens x t_n columns of r (the tokens are the MMA's rows),
+// whose 64-column stages are dealt out evenly in one list, so that every pair gets the same share whatever the number
+// of tiles.  Pairs that share a tile leave their parts as fp32 in the workspace; when all are there, each of them adds up a
+// share of the columns, in list order, and rounds to bf16.  The main tiles wait for the T' they read just before their
+// first adapter stage.  As a launch of its own (and a reduction behind it) T' took 12 us and more of most calls.
 struct PairCfg {
     static constexpr int kN = 256, kThreads = 19 * 32;
     static constexpr int kWarpX = 16, kWarpMma = 17, kWarpPk = 18;
@@ -597,12 +621,49 @@ struct PairCfg {
     static constexpr int kHalfTok = kN / 2;                                 // token rows this CTA loads
     static constexpr int kBTile = kHalfTok * kSK * 2, kStageBytes = kBTile + kPM * kSK;
     static constexpr int kECol = kN;                                        // index words: kN + 4 * stage + mma
-    static constexpr size_t kSmem = 1024 + (size_t)kStages * kStageBytes + kPkSlots * kPkSlotBytes + 512;
+    static constexpr size_t kSmem = 1024 + (size_t)kStages * kStageBytes + kPkSlots * kPkSlotBytes + 256 + 8 * 1024;     // .. barriers, epilogue
 };
+constexpr size_t kSyncTiles = kSmallTBytes / 16 - 1024;     // T' tiles whose words fit the region beside those of the pairs
+
+// The list of T' stages (tile after tile) dealt out to the pairs.
+__host__ __device__ __forceinline__ int share_begin(int q, int units, int pairs) { return (int)((long long)q * units / pairs); }
+__host__ __device__ __forceinline__ int share_owner(int unit, int units, int pairs) { return (int)(((long long)(unit + 1) * pairs - 1) / units); }
+// A share's run inside one tile, from `unit` on.
+struct Run { int tile, k0, len; };
+__device__ __forceinline__ Run run_at(int unit, int end, int stages) {
+    Run r;
+    r.tile = unit / stages; r.k0 = unit - r.tile * stages; r.len = min(stages - r.k0, end - unit);
+    return r;
+}
+__device__ __forceinline__ unsigned long long ld_acquire64(const unsigned long long* p) {
+    unsigned long long v;
+    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
+// Hand-over words: a word's high half is the number of the call that set it, so nothing is cleared between calls.  A
+// pair's part of a tile has two (part written; its share of the sums written), for each of its CTAs; so has a tile made whole (the second alone).
+__device__ __forceinline__ size_t part_word(int q, bool starts, uint32_t rank) { return ((size_t)(2 * q + (starts ? 1 : 0)) * 2 + rank) * 2; }
+__device__ __forceinline__ size_t tile_word(const PrefillParams& p, int tile, uint32_t rank) { return (size_t)p.t_pairs * 8 + (size_t)tile * 2 + rank; }
+// Waits (bounded in time) until every lane's word (nullptr: none) is this call's; called by a whole warp.
+__device__ __forceinline__ bool wait_words(const unsigned long long* w, uint32_t call, volatile uint32_t* abort_flag) {
+    unsigned long long t0 = 0;
+    for (uint32_t it = 0;; ++it) {
+        const bool there = !w || (uint32_t)(ld_acquire64(w) >> 32) == call;
+        if (__all_sync(0xffffffffu, there)) return true;
+        if (__any_sync(0xffffffffu, *abort_flag != 0)) return false;
+        if ((it & 63u) == 63u) {
+            unsigned long long now;
+            asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
+            if (t0 == 0) t0 = now;
+            else if (__any_sync(0xffffffffu, now - t0 > 2000000000ull)) { *abort_flag = 1u; return false; }
+        }
+    }
+}
 
 __global__ void __launch_bounds__(PairCfg::kThreads, 1)
 prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmM,
-                    const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmA2, const __grid_constant__ CUtensorMap tmB2)
+                    const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmA2, const __grid_constant__ CUtensorMap tmB2,
+                    const __grid_constant__ CUtensorMap tmR)
 {
     using namespace pf;
     using Cfg = PairCfg;
@@ -626,6 +687,10 @@ prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap t
     const uint32_t rank = cluster_rank();
     const int pairs = gridDim.x >> 1, first_tile = blockIdx.x >> 1;
     const int n_total = p.n1 + p.n2, n_groups = ceil_div(p.n1, kPkStages);
+    // this pair's share of T': the last pairs, which have the fewest tiles, come first
+    const int t_units = p.t_tiles * p.t_stages, tq = pairs - 1 - first_tile;
+    const int t_begin = tq < p.t_pairs ? share_begin(tq, t_units, p.t_pairs) : 0, t_end = tq < p.t_pairs ? share_begin(tq + 1, t_units, p.t_pairs) : 0;
+    const uint32_t call = p.r > 0 ? (uint32_t)(*(volatile unsigned long long*)p.departures >> 16) + 1u : 0u;
 
     if (threadIdx.x == 0) {
         for (int i = 0; i < kStages; ++i) { mbar_init(&b_full[i], 1); mbar_init(&conv_done[i], kConvWarps); mbar_init(&empty[i], 1); }
@@ -658,17 +723,47 @@ prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap t
 
     if (warp == Cfg::kWarpX) {
         // ============================ token tiles, A2, B2 ============================
-        bool t_ready = false;                               // T' (and everything before it) is complete
         int g = 0;                                          // stages so far
+        int t_checked = -1;                                 // the token tile whose T' was found complete
+        for (int u = t_begin; u < t_end;) {
+            // T': 128 tokens x 64 columns of X as A, half of the chunk's rows of R as B
+            const Run run = run_at(u, t_end, p.t_stages);
+            const int tok = (run.tile / p.t_chunks) * Cfg::kN + (int)rank * kPM, col = (run.tile % p.t_chunks) * p.t_n;
+            for (int it = 0; it < run.len; ++it, ++g) {
+                const int st = g % kStages;
+                if (g >= kStages) ok = mbar_wait(&empty[st], ((g / kStages) & 1) ^ 1, abort_flag) && ok;
+                if (lane == 0 && rank == 0) mbar_expect_tx(&b_full[st], (uint32_t)(2 * (kPM + p.t_n / 2) * kDK * 2));
+                unsigned char* sbase = stages + (size_t)st * kStageBytes;
+                if (lane < 2)
+                    tma_tile_pair(lane == 0 ? sbase + kBTile : sbase, lane == 0 ? &tmX : &tmR, (run.k0 + it) * kDK,
+                                  lane == 0 ? tok : col + (int)rank * (p.t_n / 2), peer_addr(&b_full[st], 0));
+            }
+            u += run.len;
+        }
         for (int t = first_tile; t < p.tiles; t += pairs) {
             const Tile ti = tile_of(t);
             for (int it = 0; it < n_total; ++it, ++g) {
                 const int st = g % kStages;
                 const bool sparse = it < p.n1;
-                if (!sparse && !t_ready) {
-                    asm volatile("griddepcontrol.wait;" ::: "memory");
+                if (it == p.n1) {
+                    // the T' of this CTA's half of the tokens is complete (a word per part of its chunks, 32 at a time)
+                    if (ti.n0 != t_checked) {
+                        const int tile0 = (ti.n0 / Cfg::kN) * p.t_chunks;
+                        for (int first = 0, left = 1; left > 0; first += 32) {
+                            int i = first + lane;
+                            const unsigned long long* w = nullptr;
+                            left = -first - 32;
+                            for (int c = 0; c < p.t_chunks; ++c) {
+                                const int q0 = share_owner((tile0 + c) * p.t_stages, t_units, p.t_pairs), q1 = share_owner((tile0 + c + 1) * p.t_stages - 1, t_units, p.t_pairs);
+                                if (i >= 0 && i <= q1 - q0) w = p.t_sync + (q0 == q1 ? tile_word(p, tile0 + c, rank) : part_word(q0 + i, i == 0, rank) + 1);
+                                i -= q1 - q0 + 1; left += q1 - q0 + 1;
+                            }
+                            ok = wait_words(w, call, abort_flag) && ok;
+                        }
+                        t_checked = ti.n0;
+                    }
+                    __syncwarp();
                     asm volatile("fence.proxy.async;" ::: "memory");   // the tiles are read by the async proxy
-                    t_ready = true;
                 }
                 if (g >= kStages) ok = mbar_wait(&empty[st], ((g / kStages) & 1) ^ 1, abort_flag) && ok;
                 // both CTAs' bytes are counted on the even CTA's barrier
@@ -703,6 +798,24 @@ prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap t
             constexpr uint32_t idesc = idesc_bf16(2 * kPM, Cfg::kN);
             uint32_t pre = 0;       // the coming stage was found ready by an early test
             int g = 0, nth = 0;
+            for (int u = t_begin; u < t_end; ++nth) {
+                const uint32_t idesc_t = idesc_bf16(2 * kPM, 16) + ((uint32_t)((p.t_n - 16) >> 3) << 17);
+                const Run run = run_at(u, t_end, p.t_stages);
+                if (nth > 0) ok = mbar_wait_all(acc_empty, (nth & 1) ^ 1, true, nullptr, 0, false, nullptr, 0, false, abort_flag) && ok;
+                for (int it = 0; it < run.len; ++it, ++g) {
+                    const int st = g % kStages;
+                    const uint32_t parity = (g / kStages) & 1;
+                    ok = mbar_wait_all(&b_full[st], parity, true, &conv_done[st], parity, true, nullptr, 0, false, abort_flag) && ok;
+                    fence_after_sync();
+                    const uint32_t b_addr = s32(stages + (size_t)st * kStageBytes), a_addr = b_addr + kBTile;
+#pragma unroll
+                    for (int j = 0; j < kDK / 16; ++j)
+                        mma_dense2(tmem_base, smem_desc(a_addr + 32 * j), smem_desc(b_addr + 32 * j), idesc_t, it > 0 || j > 0 ? 1u : 0u);
+                    mma_commit2(&empty[st]);
+                }
+                mma_commit2(acc_full);
+                u += run.len;
+            }
             for (int t = first_tile; t < p.tiles; t += pairs, ++nth) {
                 if (nth > 0) ok = mbar_wait_all(acc_empty, (nth & 1) ^ 1, true, nullptr, 0, false, nullptr, 0, false, abort_flag) && ok;
                 for (int it = 0; it < n_total; ++it, ++g) {
@@ -740,7 +853,15 @@ prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap t
         const int half = threadIdx.x >> 7;
         const int x = (row >> 3) & 1;
         const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
-        int base = 0, nth = 0;                       // stages before this tile
+        // nothing to expand for T' and in phase 2: the arrival keeps the barrier's phases in step with the stages
+        auto pass = [&](int g) {
+            const int st = g % kStages;
+            if (g >= kStages) ok = mbar_wait(&empty[st], ((g / kStages) & 1) ^ 1, abort_flag) && ok;
+            if (lane == 0) mbar_arrive_remote(peer_addr(&conv_done[st], 0));
+            __syncwarp();
+        };
+        int base = t_end - t_begin, nth = 0;         // stages before this tile
+        for (int g = half; g < base; g += 2) pass(g);
         for (int t = first_tile; t < p.tiles; t += pairs, base += n_total, ++nth) {
             const bool row_in = tile_of(t).m0 + row < p.m_total;
             for (int it = (base ^ half) & 1; it < n_total; it += 2) {
@@ -765,10 +886,7 @@ prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap t
                         if (q == 0 && it + 1 == p.n1) mbar_arrive(&pk_empty[slot]);
                     }
                 } else {
-                    // nothing to expand in phase 2: the arrival keeps the barrier's phases in step with the stages
-                    if (free_bar) ok = mbar_wait(free_bar, free_par, abort_flag) && ok;
-                    if (lane == 0) mbar_arrive_remote(peer_addr(&conv_done[st], 0));
-                    __syncwarp();
+                    pass(g);
                 }
             }
         }
@@ -777,15 +895,94 @@ prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap t
         const int half = (warp - kConvWarps) >> 2;
         const int row = (warp & 3) * 32 + lane;
         const uint32_t taddr = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + half * kHalfTok;
+        const uint32_t buf = s32(b_full) + 256 + (warp - kConvWarps) * 1024;
         int nth = 0;
+        // ---- T': thread = token.  Part of pair q: [c / 4][128 tokens] float4; a pair has at most one that starts with its tile and
+        // one that does not.
+        auto part = [&](int q, bool starts) { return p.t_part + ((size_t)(2 * q + (starts ? 1 : 0)) * 2 + rank) * ((size_t)kPM * p.t_n / 4) + row; };
+        auto store4 = [&](int tile, int c, float4 v) {
+            const int token = (tile / p.t_chunks) * Cfg::kN + (int)rank * kPM + row, col = (tile % p.t_chunks) * p.t_n + c;
+            if (token >= p.b || col >= p.r) return;
+            __nv_bfloat162 lo = __floats2bfloat162_rn(p.t_scale * v.x, p.t_scale * v.y), hi = __floats2bfloat162_rn(p.t_scale * v.z, p.t_scale * v.w);
+            *reinterpret_cast<uint2*>(p.t_out + (size_t)token * p.r + col) = make_uint2(*reinterpret_cast<uint32_t*>(&lo), *reinterpret_cast<uint32_t*>(&hi));
+        };
+        auto publish = [&](size_t word) {                                    // the writes of the eight warps, then the word
+            epilogue_sync();
+            if (threadIdx.x == kConvWarps * 32) {
+                __threadfence();
+                *(volatile unsigned long long*)(p.t_sync + word) = (unsigned long long)call << 32;
+            }
+        };
+        // all of this pair's runs first (nothing here waits for another pair), every second group of 16 columns a thread
+        for (int u = t_begin; u < t_end; ++nth) {
+            const Run run = run_at(u, t_end, p.t_stages);
+            u += run.len;
+            const bool whole = run.len == p.t_stages;
+            ok = mbar_wait(acc_full, nth & 1, abort_flag) && ok;
+            fence_after_sync();
+            float4* mine = part(tq, run.k0 == 0);
+            const uint32_t t_addr = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
+            for (int c = half * 16; c < p.t_n; c += 32) {
+                float4 v[4];
+                tmem_ld16(t_addr + c, v);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    if (whole) store4(run.tile, c + 4 * i, v[i]);
+                    else __stcg(mine + (size_t)(c / 4 + i) * kPM, v[i]);
+                }
+            }
+            fence_before_sync();
+            __syncwarp();
+            if (lane == 0) mbar_arrive_remote_release(peer_addr(acc_empty, 0));
+            publish(whole ? tile_word(p, run.tile, rank) : part_word(tq, run.k0 == 0, rank));
+        }
+        // then its share of the sums: when every part of a tile is there, columns c4 = .. (mod 2 n) for each of its n pairs
+        for (int u = t_begin; u < t_end;) {
+            const Run run = run_at(u, t_end, p.t_stages);
+            u += run.len;
+            if (run.len == p.t_stages) continue;
+            const int q0 = share_owner(run.tile * p.t_stages, t_units, p.t_pairs), q1 = share_owner((run.tile + 1) * p.t_stages - 1, t_units, p.t_pairs);
+            const int n = q1 - q0 + 1;
+            for (int q = q0; q <= q1; q += 32)
+                ok = wait_words(q + lane <= q1 ? p.t_sync + part_word(q + lane, q + lane == q0, rank) : nullptr, call, abort_flag) && ok;
+            if (n == 2) {                                                    // two parts: four columns' loads in flight
+                const float4 *f0 = part(q0, true), *f1 = part(q1, false);
+                for (int c4 = 2 * (tq - q0) + half; c4 < p.t_n / 4; c4 += 16) {
+                    float4 x[4], y[4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const size_t at = (size_t)min(c4 + 4 * i, p.t_n / 4 - 1) * kPM;
+                        x[i] = __ldcg(f0 + at); y[i] = __ldcg(f1 + at);
+                    }
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+                        if (c4 + 4 * i < p.t_n / 4) store4(run.tile, 4 * (c4 + 4 * i), make_float4(x[i].x + y[i].x, x[i].y + y[i].y, x[i].z + y[i].z, x[i].w + y[i].w));
+                }
+            } else {
+                for (int c4 = 2 * (tq - q0) + half; c4 < p.t_n / 4; c4 += 2 * n) {
+                    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+                    for (int qb = q0; qb <= q1; qb += 12) {
+                        float4 v[12];
+#pragma unroll
+                        for (int i = 0; i < 12; ++i) v[i] = qb + i <= q1 ? __ldcg(part(qb + i, qb + i == q0) + (size_t)c4 * kPM) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                        for (int i = 0; i < 12; ++i) { s.x += v[i].x; s.y += v[i].y; s.z += v[i].z; s.w += v[i].w; }
+                    }
+                    store4(run.tile, 4 * c4, s);
+                }
+            }
+            publish(part_word(tq, run.k0 == 0, rank) + 1);
+        }
         for (int t = first_tile; t < p.tiles; t += pairs, ++nth) {
             const Tile ti = tile_of(t);
             ok = mbar_wait(acc_full, nth & 1, abort_flag) && ok;
             fence_after_sync();
-            const int orow = ti.m0 + row, tok0 = ti.n0 + half * kHalfTok;
-            __nv_bfloat16* out = p.out + (size_t)tok0 * p.ldo + orow;
-            const int n_tok = orow < p.m_total ? min(kHalfTok, p.b - tok0) : 0;
-            // two passes of 64 tokens (what fits in registers); the accumulator is free before the second pass's stores
+            // 16 tokens at a time, through the warp's kilobyte of shared memory, [token][32 rows] bf16: a thread then stores 16 bytes,
+            // eight rows of a token (direct two-byte stores took 5.6 us a tile).  Two passes of 64 tokens (what fits in
+            // registers): the accumulator is free before the second pass's stores.
+            const int tok0 = ti.n0 + half * kHalfTok, row8 = ti.m0 + (warp & 3) * 32 + (lane & 3) * 8;
+            const int n_tok = row8 < p.m_total ? p.b - tok0 : 0;
+            __nv_bfloat16* out = p.out + (size_t)(tok0 + (lane >> 2)) * p.ldo + row8;
 #pragma unroll
             for (int c0 = 0; c0 < kHalfTok; c0 += 64) {
                 uint32_t y[32];                                              // bf16 pairs of neighbouring tokens
@@ -805,9 +1002,19 @@ prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap t
                     if (lane == 0) mbar_arrive_remote_release(peer_addr(acc_empty, 0));
                 }
 #pragma unroll
-                for (int c = 0; c < 64; ++c) {
-                    if (c0 + c < n_tok) *out = __ushort_as_bfloat16((unsigned short)(c & 1 ? y[c / 2] >> 16 : y[c / 2] & 0xFFFFu));
-                    out += p.ldo;
+                for (int c1 = 0; c1 < 64; c1 += 16) {
+                    if (c0 + c1 >= p.b - tok0) break;
+#pragma unroll
+                    for (int c = 0; c < 16; ++c)
+                        asm volatile("st.shared.u16 [%0], %1;" :: "r"(buf + c * 64 + lane * 2), "h"((unsigned short)(c & 1 ? y[(c1 + c) / 2] >> 16 : y[(c1 + c) / 2] & 0xFFFFu)) : "memory");
+                    __syncwarp();
+#pragma unroll
+                    for (int i = 0; i < 2; ++i) {                            // tokens 8 i + lane / 4
+                        uint4 v;
+                        asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(buf + i * 512 + lane * 16) : "memory");
+                        if (c0 + c1 + i * 8 + (lane >> 2) < n_tok) *reinterpret_cast<uint4*>(out + (size_t)(c0 + c1 + i * 8) * p.ldo) = v;
+                    }
+                    __syncwarp();
                 }
             }
         }
@@ -821,6 +1028,8 @@ prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap t
         fence_after_sync();
         asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" :: "r"(tmem_base), "r"(512) : "memory");
     }
+    // a call adds 1 << 16 to the counter in all
+    if (threadIdx.x == 0) atomicAdd(p.departures, blockIdx.x == 0 ? 65536ull - (gridDim.x - 1) : 1ull);
 }
 
 // Sum of the K slices' partial tiles, scaled and rounded to bf16 (fixed order: deterministic).
@@ -890,37 +1099,72 @@ bool prefill_supports(int b, int d_out, int d_in, int r) {
     return b >= 1 && d_out % 16 == 0 && d_in % kPBK == 0 && r % 16 == 0 && r >= 0;
 }
 
+// The pair kernel's T' tiles: chunks of the columns of r.
+static int t_chunks(int r) { return ceil_div(r, 256); }
+static int t_width(int r) { return r > 0 ? ceil_div(ceil_div(r, t_chunks(r)), 16) * 16 : 16; }
+static size_t pair_part_bytes(int r, int sm_count) { return (size_t)(sm_count / 2) * 2 * 256 * t_width(r) * sizeof(float); }
+
+// Pairs that share the work of T'.  Each tile in equal parts, one a pair, where that uses four fifths of the pairs or more
+// (a pair then has one part to write, and the pairs that read the same X walk it together); else an even share each.
+// Four stages (a microsecond and a half) or more for a part: below that its start and end dominate.
+static int t_share(int tiles, int stages, int pairs) {
+    const int most = stages < 4 ? 1 : stages / 4;
+    int parts = pairs / tiles < most ? pairs / tiles : most;
+    if (parts >= 1 && (parts == most || tiles * parts * 5 >= pairs * 4)) return tiles * parts;
+    return (long long)tiles * most < pairs ? tiles * most : pairs;
+}
+
+// Wide token tiles (pair kernel) when they give a quarter of the SMs or more a 128-row tile, else narrow ones (measured: with 64
+// tiles of 128 x 256 on 148 SMs the wide variant is a third faster than 256 tiles of 128 x 64; with 32 it is
+// slower), and when the words of its T' tiles fit their region.
+static bool runs_wide(int b, int d_out, int r, int sm_count) {
+    return (long long)ceil_div(d_out, kPM) * ceil_div(b, 256) * 4 >= (long long)sm_count &&
+           (size_t)ceil_div(b, 256) * t_chunks(r) <= kSyncTiles;
+}
+
 size_t prefill_workspace_bytes(int b, int d_out, int d_in, int r) {
     if (!prefill_supports(b, d_out, d_in, r)) return 0;
     const size_t tq = ((size_t)b * (size_t)r * sizeof(__nv_bfloat16) + 255) / 256 * 256;
     if (r == 0) return tq;
     const PrePlan pl = pre_plan(b, d_in, r, pre_sm_count());
-    return tq + (pl.slices > 1 ? (size_t)pl.slices * b * r * sizeof(float) : 0);
+    const size_t narrow = pl.slices > 1 ? (size_t)pl.slices * b * r * sizeof(float) : 0, wide = pair_part_bytes(r, pre_sm_count());
+    return tq + (runs_wide(b, d_out, r, pre_sm_count()) || wide > narrow ? wide : narrow);     // (the pair kernel may be asked for by name)
 }
 
+static std::atomic<int> g_pairs[64];               // pairs resident at once
 static std::atomic<bool> g_prefill_attr_set[64];   // attributes set once per device (setting them twice is harmless)
 
 // `after_dense_only`: may start while the launch before it (the dense-only launch or its reduction) still runs.
-template <typename K>
-static slim_status_t launch_chained(K kernel, dim3 grid, int threads, size_t smem, int cluster, bool after_dense_only, cudaStream_t st, const PrefillParams& q,
-                                    const CUtensorMap& tmV, const CUtensorMap& tmM, const CUtensorMap& tmX, const CUtensorMap& tmA2, const CUtensorMap& tmB2) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid; cfg.blockDim = dim3(threads); cfg.dynamicSmemBytes = smem; cfg.stream = st;
-    cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = cluster; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr; cfg.numAttrs = after_dense_only ? 2 : 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, q, tmV, tmM, tmX, tmA2, tmB2);
-    count_launch(1);
-    return e == cudaSuccess ? SLIM_OK : SLIM_ERR_CUDA;
-}
 template <int N, bool PRE>
 static slim_status_t launch_tile_kernel(const PrefillParams& q, int m_rows, const CUtensorMap& tmV, const CUtensorMap& tmM, const CUtensorMap& tmX,
                                         const CUtensorMap& tmA2, const CUtensorMap& tmB2, cudaStream_t st, int slices = 1, bool after_dense_only = false) {
-    return launch_chained(prefill_kernel<N, PRE>, dim3(ceil_div(m_rows, kPM), ceil_div(q.b, N), slices), kPThreads, PfCfg<N, PRE>::kSmem, 1, after_dense_only, st,
-                          q, tmV, tmM, tmX, tmA2, tmB2);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(ceil_div(m_rows, kPM), ceil_div(q.b, N), slices); cfg.blockDim = dim3(kPThreads);
+    cfg.dynamicSmemBytes = PfCfg<N, PRE>::kSmem; cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr; cfg.numAttrs = after_dense_only ? 1 : 0;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, prefill_kernel<N, PRE>, q, tmV, tmM, tmX, tmA2, tmB2);
+    count_launch(1);
+    return e == cudaSuccess ? SLIM_OK : SLIM_ERR_CUDA;
+}
+
+static slim_status_t launch_pair(const PrefillParams& p, const CUtensorMap& tmV, const CUtensorMap& tmM, const CUtensorMap& tmX, const CUtensorMap& tmA2,
+                                 const CUtensorMap& tmB2, const CUtensorMap& tmR, int pairs, cudaStream_t st) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(2 * pairs); cfg.blockDim = dim3(PairCfg::kThreads); cfg.dynamicSmemBytes = PairCfg::kSmem; cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    // the pairs wait for one another's T': all of them are resident together (two such calls on different streams could
+    // otherwise each hold half of the SMs and wait for their other half)
+    attr[1].id = cudaLaunchAttributeCooperative;
+    attr[1].val.cooperative = 1;
+    cfg.attrs = attr; cfg.numAttrs = p.t_pairs > 0 ? 2 : 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, prefill_pair_kernel, p, tmV, tmM, tmX, tmA2, tmB2, tmR);
+    count_launch(1);
+    return e == cudaSuccess ? SLIM_OK : SLIM_ERR_CUDA;
 }
 
 slim_status_t launch_prefill(const __nv_bfloat16* X, int b, const uint8_t* vals, const uint8_t* meta,
@@ -934,35 +1178,47 @@ slim_status_t launch_prefill(const __nv_bfloat16* X, int b, const uint8_t* vals,
     if (!prefill_supports(b, d_out, d_in, r)) return SLIM_ERR_UNSUPPORTED_SHAPE;
     int dev = 0;
     cudaGetDevice(&dev);
-    if (dev >= 0 && dev < 64 && !g_prefill_attr_set[dev].load(std::memory_order_acquire)) {
+    if (dev < 0 || dev >= 64) return SLIM_ERR_CUDA;
+    if (!g_prefill_attr_set[dev].load(std::memory_order_acquire)) {
         if (cudaFuncSetAttribute(prefill_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PairCfg::kSmem) != cudaSuccess ||
             cudaFuncSetAttribute(prefill_kernel<64, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PfCfg<64, false>::kSmem) != cudaSuccess ||
             cudaFuncSetAttribute(prefill_kernel<64, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PfCfg<64, true>::kSmem) != cudaSuccess ||
             cudaFuncSetAttribute(prefill_kernel<256, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PfCfg<256, true>::kSmem) != cudaSuccess)
             return SLIM_ERR_CUDA;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(2); cfg.blockDim = dim3(PairCfg::kThreads); cfg.dynamicSmemBytes = PairCfg::kSmem;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr; cfg.numAttrs = 1;
+        int n = 0;
+        if (cudaOccupancyMaxActiveClusters(&n, prefill_pair_kernel, &cfg) != cudaSuccess || n < 1) return SLIM_ERR_CUDA;
+        g_pairs[dev].store(n < di->sm_count / 2 ? n : di->sm_count / 2, std::memory_order_relaxed);
         g_prefill_attr_set[dev].store(true, std::memory_order_release);
     }
     __nv_bfloat16* Tq = reinterpret_cast<__nv_bfloat16*>(reinterpret_cast<char*>(ws) + SLIM_WORKSPACE_SYNC_BYTES + kSmallTBytes);
     const float s_eff = s != 0.f ? s : 1.f;       // with s == 0 only the adapter term remains
-    // token tile: 256 when that gives a quarter of the SMs or more a tile, else 64 (measured: with 64 tiles of
-    // 128 x 256 on 148 SMs the wide variant is a third faster than 256 tiles of 128 x 64; with 32 it is slower)
-    const bool wide = force_pair || (long long)ceil_div(d_out, kPM) * ceil_div(b, 256) * 4 >= (long long)di->sm_count;
+    const bool wide = force_pair || runs_wide(b, d_out, r, di->sm_count);
     if (force_pair && ceil_div(d_out, kPM) % 2 != 0) return SLIM_ERR_UNSUPPORTED_SHAPE;
     const int xbox = wide ? PairCfg::kHalfTok : 64;       // token rows one CTA loads per stage = one TMA box
     const int dk = wide ? PairCfg::kDK : PfCfg<64>::kDK;  // columns of a dense stage of the main kernel
-    CUtensorMap tmV, tmM, tmX, tmXpre, tmA2, tmB2;
+    CUtensorMap tmV, tmM, tmX, tmXpre, tmA2, tmB2, tmR;
     bool ok = pf_map(&tmV, vals, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)d_in / 4, (uint64_t)d_out, kPkCols / 4, kPM, 64) &&
               (d_in % 128 != 0 || pf_map(&tmM, meta, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)d_in / 8, (uint64_t)d_out, kPkCols / 8, kPM, 32)) &&
               pf_map(&tmX, X, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (uint64_t)d_in, (uint64_t)b, 64, xbox, 128);
     if (!ok) return SLIM_ERR_CUDA;
     if (d_in % 128 != 0) tmM = tmV;              // not used
-    if (r > 0) {
+    tmA2 = tmX; tmB2 = tmX; tmR = tmX;    // not used when r == 0
+    if (r > 0 && wide) {
+        ok = pf_map(&tmR, R, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (uint64_t)d_in, (uint64_t)r, 64, t_width(r) / 2, 128);
+        if (!ok) return SLIM_ERR_CUDA;
+    } else if (r > 0) {
         // T' = (X R^T) / s : dense phase only, output rows = adapter index
         const PrePlan pl = pre_plan(b, d_in, r, di->sm_count, s != 0.f);
         ok = pf_map(&tmA2, R, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (uint64_t)d_in, (uint64_t)r, 64, kPM, 128) &&
              pf_map(&tmXpre, X, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (uint64_t)d_in, (uint64_t)b, 64, pl.n_tok, 128);
         if (!ok) return SLIM_ERR_CUDA;
-        PrefillParams q;
+        PrefillParams q = {};
         q.out = Tq; q.ldo = r; q.m_total = r; q.b = b; q.n1 = 0; q.n2 = d_in / kPBK; q.scale = 1.f / s_eff; q.status = status_dev;
         q.k_per = pl.k_per; q.meta = nullptr; q.meta_pitch = 0; q.d_in = d_in;
         // partial tiles of the K slices follow T' in the workspace
@@ -984,14 +1240,14 @@ slim_status_t launch_prefill(const __nv_bfloat16* X, int b, const uint8_t* vals,
             count_launch(1);
             if (re != cudaSuccess) return SLIM_ERR_CUDA;
         }
+    }
+    if (r > 0) {
         // dense stages of the main kernel: 64 columns (128-byte rows) in the pair kernel, else 32 (64-byte rows)
         ok = pf_map(&tmA2, L, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (uint64_t)r, (uint64_t)d_out, dk, kPM, dk == 64 ? 128 : 64) &&
              pf_map(&tmB2, Tq, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (uint64_t)r, (uint64_t)b, dk, xbox, dk == 64 ? 128 : 64);
         if (!ok) return SLIM_ERR_CUDA;
-    } else {
-        tmA2 = tmX; tmB2 = tmX;       // never used when r == 0
     }
-    PrefillParams p;
+    PrefillParams p = {};
     p.out = Y; p.ldo = d_out; p.m_total = d_out; p.b = b;
     p.n1 = s != 0.f ? ceil_div(d_in, wide ? PairCfg::kSK : PfCfg<64>::kSK) : 0;
     p.n2 = r > 0 ? ceil_div(r, dk) : 0;
@@ -1006,9 +1262,19 @@ slim_status_t launch_prefill(const __nv_bfloat16* X, int b, const uint8_t* vals,
     if (!wide) {
         rc = launch_tile_kernel<64, false>(p, d_out, tmV, tmM, tmX, tmA2, tmB2, st, 1, dep);
     } else {
-        const int pairs = di->sm_count / 2;
-        rc = launch_chained(prefill_pair_kernel, dim3(2 * (p.tiles < pairs ? p.tiles : pairs)), PairCfg::kThreads, PairCfg::kSmem, 2, dep, st, p, tmV, tmM, tmX,
-                            tmA2, tmB2);
+        const int pairs = g_pairs[dev].load(std::memory_order_relaxed);
+        p.departures = reinterpret_cast<unsigned long long*>(ws);
+        p.t_sync = reinterpret_cast<unsigned long long*>(reinterpret_cast<char*>(ws) + SLIM_WORKSPACE_SYNC_BYTES);
+        p.r = r;
+        int grid = p.tiles < pairs ? p.tiles : pairs;
+        if (r > 0) {
+            p.t_n = t_width(r); p.t_chunks = t_chunks(r); p.t_tiles = ceil_div(b, PairCfg::kN) * p.t_chunks; p.t_stages = d_in / PairCfg::kDK;
+            p.t_scale = 1.f / s_eff; p.t_out = Tq;
+            p.t_part = reinterpret_cast<float4*>(reinterpret_cast<char*>(Tq) + ((size_t)b * r * sizeof(__nv_bfloat16) + 255) / 256 * 256);
+            p.t_pairs = t_share(p.t_tiles, p.t_stages, pairs);
+            if (grid < p.t_pairs) grid = p.t_pairs;
+        }
+        rc = launch_pair(p, tmV, tmM, tmX, tmA2, tmB2, tmR, grid, st);
     }
     if (rc != SLIM_OK) return rc;
     return SLIM_OK;
