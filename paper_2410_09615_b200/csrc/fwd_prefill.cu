@@ -195,7 +195,7 @@ __device__ __forceinline__ void mma_sparse(uint32_t d_tmem, uint64_t a_desc, uin
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" :: "r"(s32(bar)) : "memory");
 }
-// ---- CTA-pair variants
+// ---- CTA-pair variants.  The sparse one reads A from tensor memory: lane = row, two stored bf16 per column.
 __device__ __forceinline__ void mma_dense2(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
@@ -203,13 +203,13 @@ __device__ __forceinline__ void mma_dense2(uint32_t d_tmem, uint64_t a_desc, uin
         "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
         :: "r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
 }
-__device__ __forceinline__ void mma_sparse2(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t e_tmem,
+__device__ __forceinline__ void mma_sparse2(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t e_tmem,
                                             uint32_t idesc, uint32_t accumulate) {
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
         "setp.ne.b32 p, %5, 0;\n\t"
-        "tcgen05.mma.sp.cta_group::2.kind::f16 [%0], %1, %2, [%3], %4, p;\n\t}"
-        :: "r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(e_tmem), "r"(idesc), "r"(accumulate) : "memory");
+        "tcgen05.mma.sp.cta_group::2.kind::f16 [%0], [%1], %2, [%3], %4, p;\n\t}"
+        :: "r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(e_tmem), "r"(idesc), "r"(accumulate) : "memory");
 }
 // The same for a pair's loads: the bytes are counted on the even CTA's barrier.
 __device__ __forceinline__ void tma_tile_pair(void* dst, const CUtensorMap* tmap, int x, int y, uint32_t cluster_bar_addr) {
@@ -320,6 +320,14 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float4 (&v)[4]) {
                    "=f"(v[2].x), "=f"(v[2].y), "=f"(v[2].z), "=f"(v[2].w), "=f"(v[3].x), "=f"(v[3].y), "=f"(v[3].z), "=f"(v[3].w) : "r"(taddr) : "memory");
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
+__device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint4 (&a)[8]) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, "
+                 "%17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};"
+                 :: "r"(taddr), "r"(a[0].x), "r"(a[0].y), "r"(a[0].z), "r"(a[0].w), "r"(a[1].x), "r"(a[1].y), "r"(a[1].z), "r"(a[1].w),
+                    "r"(a[2].x), "r"(a[2].y), "r"(a[2].z), "r"(a[2].w), "r"(a[3].x), "r"(a[3].y), "r"(a[3].z), "r"(a[3].w),
+                    "r"(a[4].x), "r"(a[4].y), "r"(a[4].z), "r"(a[4].w), "r"(a[5].x), "r"(a[5].y), "r"(a[5].z), "r"(a[5].w),
+                    "r"(a[6].x), "r"(a[6].y), "r"(a[6].z), "r"(a[6].w), "r"(a[7].x), "r"(a[7].y), "r"(a[7].z), "r"(a[7].w) : "memory");
+}
 __device__ __forceinline__ void epilogue_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
 
 }  // namespace pf
@@ -348,15 +356,13 @@ __device__ __forceinline__ void load_packed(const PrefillParams& p, const CUtens
 }
 
 // One weight row of a stage of SK (64 or 128) columns, the q-th of its packed tile: 16 value bytes -> 32 bf16 per 64
-// columns into the K-major A tile (rows of SK bytes, swizzle of that width), and the row's part of the index words of
+// columns, and the row's part of the index words of
 // the stage's MMAs (layout in the file header).  The packed tiles are stored with the 64-byte (values) and 32-byte
 // (indices) TMA swizzles so that a warp's row-strided reads spread over the banks.  Rows past the last (!row_in) and columns
 // past it (cols_left) get a legal pair of positions.
 template <int SK>
-__device__ __forceinline__ void expand_row(const unsigned char* pk, unsigned char* a_tile, int row, int q, int x, bool row_in, int cols_left,
-                                           uint32_t (&e)[SK / 32])
+__device__ __forceinline__ void expand_row(const unsigned char* pk, int row, int q, int x, bool row_in, int cols_left, uint4 (&a)[SK / 16], uint32_t (&e)[SK / 32])
 {
-    unsigned char* arow = a_tile + row * SK;
 #pragma unroll
     for (int hh = 0; hh < SK / 64; ++hh) {
         const int qq = q * (SK / 64) + hh;                   // which 64 columns of the packed tile
@@ -365,11 +371,7 @@ __device__ __forceinline__ void expand_row(const unsigned char* pk, unsigned cha
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
             const uint32_t ws = w[c] >> 4;
-            uint4 o;
-            o.x = pf::nib2bf16<0>(w[c], ws); o.y = pf::nib2bf16<1>(w[c], ws);
-            o.z = pf::nib2bf16<2>(w[c], ws); o.w = pf::nib2bf16<3>(w[c], ws);
-            const int chunk = SK == 128 ? ((hh * 4 + c) ^ row) & 7 : (c ^ (row >> 1)) & 3;
-            *reinterpret_cast<uint4*>(arow + (chunk << 4)) = o;
+            a[hh * 4 + c] = make_uint4(pf::nib2bf16<0>(w[c], ws), pf::nib2bf16<1>(w[c], ws), pf::nib2bf16<2>(w[c], ws), pf::nib2bf16<3>(w[c], ws));
         }
         uint2 mw2 = *reinterpret_cast<const uint2*>(pk + kValsTile + row * 32 + ((((qq >> 1) ^ (row >> 2)) & 1) << 4) + (qq & 1) * 8);
         if (!row_in || hh * 64 >= cols_left) mw2 = make_uint2(0x44444444u, 0x44444444u);
@@ -381,6 +383,12 @@ __device__ __forceinline__ void expand_row(const unsigned char* pk, unsigned cha
             e[hh * 2 + h] = x ? ((mw & 0xFFFF0000u) | recv) : ((mw & 0xFFFFu) | (recv << 16));
         }
     }
+}
+// The expanded row of a 64-column stage into the K-major A tile: 64-byte rows, 64-byte swizzle.
+__device__ __forceinline__ void store_row(unsigned char* a_tile, int row, const uint4 (&a)[4])
+{
+#pragma unroll
+    for (int c = 0; c < 4; ++c) *reinterpret_cast<uint4*>(a_tile + row * 64 + (((c ^ (row >> 1)) & 3) << 4)) = a[c];
 }
 
 template <int N, bool PRE = false>
@@ -549,8 +557,10 @@ prefill_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap tmV,
             ok = mbar_wait_all(&pk_full[slot], (gi / kPkSlots) & 1, false, it >= kPStages ? &empty[st] : nullptr,
                                ((it / kPStages) & 1) ^ 1, false, nullptr, 0, false, abort_flag) && ok;
             if ((threadIdx.x & 127) == 0) PSTAMP(1, it);
+            uint4 a[4];
             uint32_t e[2];
-            expand_row<64>(pk, stages + (size_t)st * kStageBytes + kBTile, row, q, x, m0 + row < p.m_total, 64, e);
+            expand_row<64>(pk, row, q, x, m0 + row < p.m_total, 64, a, e);
+            store_row(stages + (size_t)st * kStageBytes + kBTile, row, a);
             asm volatile("tcgen05.st.sync.aligned.32x32b.x2.b32 [%0], {%1, %2};"
                          :: "r"(tmem_base + lane_base + kECol + 4 * st), "r"(e[0]), "r"(e[1]) : "memory");
             asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
@@ -601,6 +611,9 @@ prefill_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap tmV,
 // A cluster of two CTAs computes tiles of 256 output rows x 256 tokens with cta_group::2 MMAs issued by the even CTA: each
 // CTA loads and expands its own 128 rows of the weight and loads half of the token tile.  Stages are 128 weight
 // columns (four MMAs of K = 32 per commit; 64 columns of the adapters in phase 2).
+// The expanded weight goes to tensor memory, not to shared memory: per stage an SM's shared memory carries 76 KB (TMA
+// writes 38, converters read 6, tensor core reads 32: 0.31 us at 128 bytes a cycle, as long as the MMAs take) where with
+// A in shared memory it was 108 KB and 0.46 us a stage.
 // The pairs are persistent: pair c takes tiles c, c + pairs, ..., and all rings run on across tiles, so that the next
 // tile's operands are loaded and expanded while this tile ends.  Eight warps of their own read the accumulator out:
 // 128 tokens a thread; the next tile's MMAs may start as soon as it is in registers, the stores follow beside
@@ -617,10 +630,11 @@ prefill_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap tmV,
 struct PairCfg {
     static constexpr int kN = 256, kThreads = 19 * 32;
     static constexpr int kWarpX = 16, kWarpMma = 17, kWarpPk = 18;
-    static constexpr int kSK = 128, kDK = 64, kStages = 4, kPkSlots = 2, kPkStages = kPkCols / kSK;
+    static constexpr int kSK = 128, kDK = 64, kStages = 6, kPkSlots = 2, kPkStages = kPkCols / kSK;
     static constexpr int kHalfTok = kN / 2;                                 // token rows this CTA loads
-    static constexpr int kBTile = kHalfTok * kSK * 2, kStageBytes = kBTile + kPM * kSK;
-    static constexpr int kECol = kN;                                        // index words: kN + 4 * stage + mma
+    static constexpr int kStageBytes = kHalfTok * kSK * 2, kBTile = kStageBytes, kATileAt = kStageBytes / 2;     // dense stages and T': B, then A
+    // tensor memory: the accumulator, index words (4 columns a stage), expanded weights (32 columns a stage)
+    static constexpr int kECol = kN, kACol = kN + 32;
     static constexpr size_t kSmem = 1024 + (size_t)kStages * kStageBytes + kPkSlots * kPkSlotBytes + 256 + 8 * 1024;     // .. barriers, epilogue
 };
 constexpr size_t kSyncTiles = kSmallTBytes / 16 - 1024;     // T' tiles whose words fit the region beside those of the pairs
@@ -670,7 +684,7 @@ prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap t
     constexpr int kStages = Cfg::kStages, kPkSlots = Cfg::kPkSlots, kPkStages = Cfg::kPkStages, kSK = Cfg::kSK, kDK = Cfg::kDK;
     constexpr int kBTile = Cfg::kBTile, kStageBytes = Cfg::kStageBytes, kECol = Cfg::kECol, kHalfTok = Cfg::kHalfTok;
     extern __shared__ unsigned char smem_raw[];
-    // layout: stages {B | A} | packed slots {value bytes | index bytes} | barriers
+    // layout: stages | packed slots {value bytes | index bytes} | barriers
     unsigned char* stages = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     unsigned char* packed = stages + (size_t)kStages * kStageBytes;
     uint64_t* b_full = reinterpret_cast<uint64_t*>(packed + kPkSlots * kPkSlotBytes);   // [kStages] even CTA: both CTAs' tiles landed
@@ -735,7 +749,7 @@ prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap t
                 if (lane == 0 && rank == 0) mbar_expect_tx(&b_full[st], (uint32_t)(2 * (kPM + p.t_n / 2) * kDK * 2));
                 unsigned char* sbase = stages + (size_t)st * kStageBytes;
                 if (lane < 2)
-                    tma_tile_pair(lane == 0 ? sbase + kBTile : sbase, lane == 0 ? &tmX : &tmR, (run.k0 + it) * kDK,
+                    tma_tile_pair(lane == 0 ? sbase + Cfg::kATileAt : sbase, lane == 0 ? &tmX : &tmR, (run.k0 + it) * kDK,
                                   lane == 0 ? tok : col + (int)rank * (p.t_n / 2), peer_addr(&b_full[st], 0));
             }
             u += run.len;
@@ -775,7 +789,7 @@ prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap t
                 // sparse stage: the token tile, two boxes of 64 columns; dense stage: lane 0 the token tile, lane 1 the A2 tile
                 if (lane < 2) {
                     const CUtensorMap* map = sparse ? &tmX : lane == 0 ? &tmB2 : &tmA2;
-                    unsigned char* dst = sbase + (lane == 0 ? 0 : sparse ? kHalfTok * 128 : kBTile);
+                    unsigned char* dst = sbase + (lane == 0 ? 0 : Cfg::kATileAt);          // (half a token tile and an A2 tile are the same size)
                     tma_tile_pair(dst, map, sparse ? k + lane * kPBK : k, !sparse && lane == 1 ? ti.m0 : ti.n0 + (int)rank * kHalfTok, peer_addr(&b_full[st], 0));
                 }
             }
@@ -807,7 +821,7 @@ prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap t
                     const uint32_t parity = (g / kStages) & 1;
                     ok = mbar_wait_all(&b_full[st], parity, true, &conv_done[st], parity, true, nullptr, 0, false, abort_flag) && ok;
                     fence_after_sync();
-                    const uint32_t b_addr = s32(stages + (size_t)st * kStageBytes), a_addr = b_addr + kBTile;
+                    const uint32_t b_addr = s32(stages + (size_t)st * kStageBytes), a_addr = b_addr + Cfg::kATileAt;
 #pragma unroll
                     for (int j = 0; j < kDK / 16; ++j)
                         mma_dense2(tmem_base, smem_desc(a_addr + 32 * j), smem_desc(b_addr + 32 * j), idesc_t, it > 0 || j > 0 ? 1u : 0u);
@@ -829,12 +843,12 @@ prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap t
                     const int st1 = (g + 1) % kStages;
                     const uint32_t par1 = ((g + 1) / kStages) & 1;
                     pre = mbar_test(&b_full[st1], par1, true) & mbar_test(&conv_done[st1], par1, true);
-                    const uint32_t b_addr = s32(stages + (size_t)st * kStageBytes), a_addr = b_addr + kBTile;
+                    const uint32_t b_addr = s32(stages + (size_t)st * kStageBytes), a_addr = b_addr + Cfg::kATileAt;
                     if (sparse) {
-                        // per MMA: A 16 stored bf16 (32 bytes of a 128-byte row), B 32 columns (64 bytes)
+                        // per MMA: A 16 stored bf16 (8 columns of tensor memory), B 32 columns (64 bytes)
 #pragma unroll
                         for (int j = 0; j < kSK / 32; ++j)
-                            mma_sparse2(tmem_base, smem_desc(a_addr + 32 * j), smem_desc(b_addr + (j >> 1) * (kHalfTok * 128) + 64 * (j & 1)),
+                            mma_sparse2(tmem_base, tmem_base + Cfg::kACol + 32 * st + 8 * j, smem_desc(b_addr + (j >> 1) * (kHalfTok * 128) + 64 * (j & 1)),
                                         tmem_base + kECol + 4 * st + 2 * (j >> 1), idesc | (1u << 2) | (uint32_t)(j & 1), it > 0 || j > 0 ? 1u : 0u);
                     } else {
 #pragma unroll
@@ -866,25 +880,29 @@ prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap t
             const bool row_in = tile_of(t).m0 + row < p.m_total;
             for (int it = (base ^ half) & 1; it < n_total; it += 2) {
                 const int g = base + it, st = g % kStages;
-                uint64_t* free_bar = g >= kStages ? &empty[st] : nullptr;        // the MMAs of the stage's previous use
-                const uint32_t free_par = ((g / kStages) & 1) ^ 1;
                 if (it < p.n1) {
+                    // expand into registers as soon as the packed tile is there (and give its slot back), store when the MMAs of
+                    // the stage's previous use are done: only the stores are between that and the next MMAs
                     const int gi = nth * n_groups + it / kPkStages, q = it % kPkStages, slot = gi % kPkSlots;
-                    ok = mbar_wait_all(&pk_full[slot], (gi / kPkSlots) & 1, false, free_bar, free_par, false, nullptr, 0, false, abort_flag) && ok;
+                    ok = mbar_wait(&pk_full[slot], (gi / kPkSlots) & 1, abort_flag) && ok;
+                    uint4 a[8];
                     uint32_t e[4];
-                    expand_row<128>(packed + slot * kPkSlotBytes, stages + (size_t)st * kStageBytes + kBTile, row, q, x, row_in, p.d_in - it * kSK, e);
-                    asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};"
-                                 :: "r"(tmem_base + lane_base + kECol + 4 * st), "r"(e[0]), "r"(e[1]), "r"(e[2]), "r"(e[3]) : "memory");
-                    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // A is read by the tensor core
-                    fence_before_sync();
+                    expand_row<128>(packed + slot * kPkSlotBytes, row, q, x, row_in, p.d_in - it * kSK, a, e);
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) asm volatile("" : "+r"(a[i].x), "+r"(a[i].y), "+r"(a[i].z), "+r"(a[i].w));     // here, not after the wait
                     __syncwarp();
                     if (lane == 0) {
-                        mbar_arrive_remote(peer_addr(&conv_done[st], 0));
-                        // a packed tile's last stage alone: in place of the other group too
                         mbar_arrive(&pk_empty[slot]);
-                        if (q == 0 && it + 1 == p.n1) mbar_arrive(&pk_empty[slot]);
+                        if (q == 0 && it + 1 == p.n1) mbar_arrive(&pk_empty[slot]);      // a packed tile's last stage alone: in place of the other group too
                     }
+                    if (g >= kStages) ok = mbar_wait(&empty[st], ((g / kStages) & 1) ^ 1, abort_flag) && ok;
+                    asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};"
+                                 :: "r"(tmem_base + lane_base + kECol + 4 * st), "r"(e[0]), "r"(e[1]), "r"(e[2]), "r"(e[3]) : "memory");
+                    tmem_st32(tmem_base + lane_base + Cfg::kACol + 32 * st, a);
+                    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+                    fence_before_sync();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive_remote(peer_addr(&conv_done[st], 0));
                 } else {
                     pass(g);
                 }
