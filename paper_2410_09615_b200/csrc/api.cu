@@ -289,8 +289,8 @@ slim_status_t slim_linear_fwd_q(const void* X, int b, const uint8_t* vals, const
     char* w = static_cast<char*>(workspace);
     __nv_bfloat16* Ld = reinterpret_cast<__nv_bfloat16*>(w + base);
     __nv_bfloat16* Rd = reinterpret_cast<__nv_bfloat16*>(w + base + align256((size_t)d_out * r * 2));
-    slim_status_t rc = launch_unpack_adapter(Lq, static_cast<const __nv_bfloat16*>(Ls), d_out, r, Ld, st);
-    if (rc == SLIM_OK) rc = launch_unpack_adapter(Rq, static_cast<const __nv_bfloat16*>(Rs), r, d_in, Rd, st);
+    slim_status_t rc = launch_unpack_adapters(Lq, static_cast<const __nv_bfloat16*>(Ls), Rq, static_cast<const __nv_bfloat16*>(Rs), d_out, r, d_in,
+                                              Ld, Rd, st);
     if (rc != SLIM_OK) return rc;
     const int dequant_launches = slim_last_launch_count();
     rc = slim_linear_fwd_ex(X, b, vals, meta, s, Ld, Rd, r, d_out, d_in, Y, workspace, base, status_dev, cuda_stream,

@@ -79,6 +79,9 @@ slim_status_t launch_pack_adapter(const __nv_bfloat16* A, int rows, int cols, ui
 slim_status_t launch_unpack_adapter(const uint8_t* codes, const __nv_bfloat16* scales, int rows, int cols, __nv_bfloat16* out,
                                     cudaStream_t st);
 
+slim_status_t launch_unpack_adapters(const uint8_t* Lq, const __nv_bfloat16* Ls, const uint8_t* Rq, const __nv_bfloat16* Rs, int d_out, int r,
+                                     int d_in, __nv_bfloat16* L, __nv_bfloat16* R, cudaStream_t st);
+
 slim_status_t launch_mask_top2(const int8_t* codes, const float* xbar, int d_out, int d_in, uint8_t* mask, uint32_t* status_dev,
                                cudaStream_t st);
 size_t quant_workspace_bytes(int d_out, int d_in);
