@@ -181,7 +181,7 @@ slim_status_t slim_linear_fwd_ex(const void* X, int b, const uint8_t* vals, cons
         if (automatic && runs_small(b, d_out, d_in, r))            // up to 64 tokens: the small-batch kernel
             return launch_small(Xb, b, vals, meta, nullptr, s, Lb, Rb, nullptr, nullptr, r, d_out, d_in, Yb, workspace, status_dev, stream);
         if (!prefill_supports(b, d_out, d_in, r)) return SLIM_ERR_UNSUPPORTED_SHAPE;
-        return launch_prefill(Xb, b, vals, meta, s, Lb, Rb, r, d_out, d_in, Yb, workspace, status_dev, stream);
+        return launch_prefill(Xb, b, vals, meta, s, Lb, Rb, r, d_out, d_in, Yb, workspace, status_dev, stream, false, automatic);
     case SLIM_KERNEL_PREFILL_PAIR:
         if (!prefill_supports(b, d_out, d_in, r)) return SLIM_ERR_UNSUPPORTED_SHAPE;
         return launch_prefill(Xb, b, vals, meta, s, Lb, Rb, r, d_out, d_in, Yb, workspace, status_dev, stream, true);

@@ -216,6 +216,10 @@ __device__ __forceinline__ void tma_tile_pair(void* dst, const CUtensorMap* tmap
     asm volatile("cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
                  :: "r"(s32(dst)), "l"(tmap), "r"(x), "r"(y), "r"(cluster_bar_addr) : "memory");
 }
+__device__ __forceinline__ void tma_tile_pair3(void* dst, const CUtensorMap* tmap, int y, int z, uint32_t cluster_bar_addr) {
+    asm volatile("cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
+                 :: "r"(s32(dst)), "l"(tmap), "r"(0), "r"(y), "r"(z), "r"(cluster_bar_addr) : "memory");
+}
 // Address of the same shared-memory object in CTA `rank` of the cluster.
 __device__ __forceinline__ uint32_t peer_addr(const void* p, uint32_t rank) {
     uint32_t r;
@@ -619,23 +623,35 @@ prefill_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap tmV,
 // 128 tokens a thread; the next tile's MMAs may start as soon as it is in registers, the stores follow beside
 // them.  A CTA per tile spent 4.4 us on start-up and 2.3 us on the epilogue of every tile, with the tensor
 // core idle.
-// Warps: 0-7 converters (two groups on alternate stages), 8-15 epilogue, 16 token tiles (and A2 / B2), 17 MMA issue,
-// 18 packed tiles.
+// Warps: 0-7 converters (two groups on alternate stages), 8-15 epilogue, 16 and 17 token tiles (and A2 / B2) of even and odd
+// stages, 18 MMA issue, 19 packed tiles.
 //
 // T' = (X R^T) / s is made by the same pairs first: tiles of 256 tokens x t_n columns of r (the tokens are the MMA's rows),
 // whose 64-column stages are dealt out evenly in one list, so that every pair gets the same share whatever the number
 // of tiles.  Pairs that share a tile leave their parts as fp32 in the workspace; when all are there, each of them adds up a
 // share of the columns, in list order, and rounds to bf16.  The main tiles wait for the T' they read just before their
 // first adapter stage.  As a launch of its own (and a reduction behind it) T' took 12 us and more of most calls.
-struct PairCfg {
-    static constexpr int kN = 256, kThreads = 19 * 32;
-    static constexpr int kWarpX = 16, kWarpMma = 17, kWarpPk = 18;
-    static constexpr int kSK = 128, kDK = 64, kStages = 6, kPkSlots = 2, kPkStages = kPkCols / kSK;
-    static constexpr int kHalfTok = kN / 2;                                 // token rows this CTA loads
-    static constexpr int kStageBytes = kHalfTok * kSK * 2, kBTile = kStageBytes, kATileAt = kStageBytes / 2;     // dense stages and T': B, then A
-    // tensor memory: the accumulator, index words (4 columns a stage), expanded weights (32 columns a stage)
-    static constexpr int kECol = kN, kACol = kN + 32;
-    static constexpr size_t kSmem = 1024 + (size_t)kStages * kStageBytes + kPkSlots * kPkSlotBytes + 256 + 8 * 1024;     // .. barriers, epilogue
+//
+// N = tokens of a tile: 256, 128 or 64.  A stage takes the same 0.36 us for each of them (the MMAs' 256 weight rows cost what
+// they cost), so a narrower tile only saves epilogue and token traffic.  A stage is 32 KB for every N (what T' needs).
+// Five stages and four packed tiles in flight: 33.2 -> 32.0 us on 8192 x 8192, 333 tokens, 91 -> 83 us on 28672 -> 8192, 64
+// tokens, against six and two.
+// Stages alternate between two converter groups and two token-tile warps while their number is odd, so each of them sees
+// every second phase of an `empty` barrier.  Waiting by parity is still right: before its stage g such a warp has waited
+// for the MMAs of stage g - 7, so the phase it did not see (stage g - 10) is over.  For the packed tiles' barriers the same holds
+// with four slots: a group that has no stage of a packed tile (the second of a last, half tile) next looks at that slot
+// seven stages later or more.
+constexpr int kTTok = 256;              // tokens of a T' tile (the rows of its MMA)
+constexpr int kPairThreads = 20 * 32;
+template <int N> struct PairCfg {
+    static constexpr int kWarpX = 16, kWarpMma = 18, kWarpPk = 19;
+    static constexpr int kSK = 128, kDK = 64, kStages = 5, kPkSlots = 4, kPkStages = kPkCols / kSK;
+    static constexpr int kHalfTok = N / 2;                                  // token rows this CTA loads
+    static constexpr int kBTile = kHalfTok * kSK * 2, kStageBytes = 32768, kATileAt = kStageBytes / 2;     // dense stages and T': B, then A
+    // tensor memory: the accumulator (a T' tile's is 256 columns too), index words (4 columns a stage), expanded weights (32
+    // columns a stage)
+    static constexpr int kECol = 256, kACol = 256 + 32;
+    static constexpr size_t kSmem = 1024 + (size_t)kStages * kStageBytes + kPkSlots * kPkSlotBytes + 384 + 8 * 1024;     // .. barriers, epilogue
 };
 constexpr size_t kSyncTiles = kSmallTBytes / 16 - 1024;     // T' tiles whose words fit the region beside those of the pairs
 
@@ -674,13 +690,14 @@ __device__ __forceinline__ bool wait_words(const unsigned long long* w, uint32_t
     }
 }
 
-__global__ void __launch_bounds__(PairCfg::kThreads, 1)
+template <int N>
+__global__ void __launch_bounds__(kPairThreads, 1)
 prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmM,
                     const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmA2, const __grid_constant__ CUtensorMap tmB2,
-                    const __grid_constant__ CUtensorMap tmR)
+                    const __grid_constant__ CUtensorMap tmR, const __grid_constant__ CUtensorMap tmXt)
 {
     using namespace pf;
-    using Cfg = PairCfg;
+    using Cfg = PairCfg<N>;
     constexpr int kStages = Cfg::kStages, kPkSlots = Cfg::kPkSlots, kPkStages = Cfg::kPkStages, kSK = Cfg::kSK, kDK = Cfg::kDK;
     constexpr int kBTile = Cfg::kBTile, kStageBytes = Cfg::kStageBytes, kECol = Cfg::kECol, kHalfTok = Cfg::kHalfTok;
     extern __shared__ unsigned char smem_raw[];
@@ -730,69 +747,75 @@ prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap t
     auto tile_of = [&](int t) {
         const int rp = t % p.row_pairs, tt = t / p.row_pairs;
         Tile ti;
-        ti.m0 = (2 * rp + (int)rank) * kPM; ti.n0 = tt * Cfg::kN;
+        ti.m0 = (2 * rp + (int)rank) * kPM; ti.n0 = tt * N;
         ti.rot = p.d_in % kPkCols == 0 && n_groups > 0 ? (rp + 3 * tt) % n_groups : 0;       // whole packed tiles
         return ti;
     };
 
-    if (warp == Cfg::kWarpX) {
+    if (warp == Cfg::kWarpX || warp == Cfg::kWarpX + 1) {
         // ============================ token tiles, A2, B2 ============================
+        // Each of the two warps takes every second stage: a wait, an expectation and a request take one warp 400 ns, more than the
+        // MMAs of a stage.
+        const int odd = warp - Cfg::kWarpX;
         int g = 0;                                          // stages so far
         int t_checked = -1;                                 // the token tile whose T' was found complete
         for (int u = t_begin; u < t_end;) {
             // T': 128 tokens x 64 columns of X as A, half of the chunk's rows of R as B
             const Run run = run_at(u, t_end, p.t_stages);
-            const int tok = (run.tile / p.t_chunks) * Cfg::kN + (int)rank * kPM, col = (run.tile % p.t_chunks) * p.t_n;
-            for (int it = 0; it < run.len; ++it, ++g) {
-                const int st = g % kStages;
-                if (g >= kStages) ok = mbar_wait(&empty[st], ((g / kStages) & 1) ^ 1, abort_flag) && ok;
+            const int tok = (run.tile / p.t_chunks) * kTTok + (int)rank * kPM, col = (run.tile % p.t_chunks) * p.t_n;
+            for (int it = (g ^ odd) & 1; it < run.len; it += 2) {
+                const int st = (g + it) % kStages;
+                if (g + it >= kStages) ok = mbar_wait(&empty[st], (((g + it) / kStages) & 1) ^ 1, abort_flag) && ok;
                 if (lane == 0 && rank == 0) mbar_expect_tx(&b_full[st], (uint32_t)(2 * (kPM + p.t_n / 2) * kDK * 2));
                 unsigned char* sbase = stages + (size_t)st * kStageBytes;
                 if (lane < 2)
-                    tma_tile_pair(lane == 0 ? sbase + Cfg::kATileAt : sbase, lane == 0 ? &tmX : &tmR, (run.k0 + it) * kDK,
+                    tma_tile_pair(lane == 0 ? sbase + Cfg::kATileAt : sbase, lane == 0 ? &tmXt : &tmR, (run.k0 + it) * kDK,
                                   lane == 0 ? tok : col + (int)rank * (p.t_n / 2), peer_addr(&b_full[st], 0));
             }
-            u += run.len;
+            u += run.len; g += run.len;
         }
         for (int t = first_tile; t < p.tiles; t += pairs) {
             const Tile ti = tile_of(t);
-            for (int it = 0; it < n_total; ++it, ++g) {
-                const int st = g % kStages;
+            for (int it = (g ^ odd) & 1; it < n_total; it += 2) {
+                const int st = (g + it) % kStages;
                 const bool sparse = it < p.n1;
-                if (it == p.n1) {
+                if (!sparse) {
                     // the T' of this CTA's half of the tokens is complete (a word per part of its chunks, 32 at a time)
                     if (ti.n0 != t_checked) {
-                        const int tile0 = (ti.n0 / Cfg::kN) * p.t_chunks;
+                        const int tile0 = (ti.n0 / kTTok) * p.t_chunks;
+                        const uint32_t t_half = (uint32_t)(ti.n0 % kTTok + (int)rank * kHalfTok) / kPM;
                         for (int first = 0, left = 1; left > 0; first += 32) {
                             int i = first + lane;
                             const unsigned long long* w = nullptr;
                             left = -first - 32;
                             for (int c = 0; c < p.t_chunks; ++c) {
                                 const int q0 = share_owner((tile0 + c) * p.t_stages, t_units, p.t_pairs), q1 = share_owner((tile0 + c + 1) * p.t_stages - 1, t_units, p.t_pairs);
-                                if (i >= 0 && i <= q1 - q0) w = p.t_sync + (q0 == q1 ? tile_word(p, tile0 + c, rank) : part_word(q0 + i, i == 0, rank) + 1);
+                                if (i >= 0 && i <= q1 - q0) w = p.t_sync + (q0 == q1 ? tile_word(p, tile0 + c, t_half) : part_word(q0 + i, i == 0, t_half) + 1);
                                 i -= q1 - q0 + 1; left += q1 - q0 + 1;
                             }
                             ok = wait_words(w, call, abort_flag) && ok;
                         }
                         t_checked = ti.n0;
+                        __syncwarp();
+                        asm volatile("fence.proxy.async;" ::: "memory");   // the tiles are read by the async proxy
                     }
-                    __syncwarp();
-                    asm volatile("fence.proxy.async;" ::: "memory");   // the tiles are read by the async proxy
                 }
-                if (g >= kStages) ok = mbar_wait(&empty[st], ((g / kStages) & 1) ^ 1, abort_flag) && ok;
+                if (g + it >= kStages) ok = mbar_wait(&empty[st], (((g + it) / kStages) & 1) ^ 1, abort_flag) && ok;
                 // both CTAs' bytes are counted on the even CTA's barrier
                 if (lane == 0 && rank == 0) mbar_expect_tx(&b_full[st], (uint32_t)(2 * (sparse ? kBTile : (kHalfTok + kPM) * kDK * 2)));
                 unsigned char* sbase = stages + (size_t)st * kStageBytes;
                 int kb = sparse ? it + ti.rot * kPkStages : it - p.n1;
                 if (sparse && kb >= p.n1) kb -= p.n1;
                 const int k = kb * (sparse ? kSK : kDK);
-                // sparse stage: the token tile, two boxes of 64 columns; dense stage: lane 0 the token tile, lane 1 the A2 tile
-                if (lane < 2) {
-                    const CUtensorMap* map = sparse ? &tmX : lane == 0 ? &tmB2 : &tmA2;
-                    unsigned char* dst = sbase + (lane == 0 ? 0 : Cfg::kATileAt);          // (half a token tile and an A2 tile are the same size)
-                    tma_tile_pair(dst, map, sparse ? k + lane * kPBK : k, !sparse && lane == 1 ? ti.m0 : ti.n0 + (int)rank * kHalfTok, peer_addr(&b_full[st], 0));
+                // sparse stage: the token tile, two sub-tiles of 64 columns in one box; dense stage: lane 0 the token tile, lane 1 the A2 tile
+                const int y = ti.n0 + (int)rank * kHalfTok;
+                if (sparse) {
+                    if (lane == 0) tma_tile_pair3(sbase, &tmX, y, k / kPBK, peer_addr(&b_full[st], 0));
+                } else if (lane < 2) {
+                    tma_tile_pair(sbase + (lane == 0 ? 0 : Cfg::kATileAt), lane == 0 ? &tmB2 : &tmA2, k, lane == 0 ? y : ti.m0, peer_addr(&b_full[st], 0));
                 }
             }
+            g += n_total;
         }
     } else if (warp == Cfg::kWarpPk) {
         // ============================ packed tiles ============================
@@ -809,7 +832,7 @@ prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap t
     } else if (warp == Cfg::kWarpMma) {
         // ============================ MMA issue: one thread of the even CTA ============================
         if (rank == 0 && elect_one()) {
-            constexpr uint32_t idesc = idesc_bf16(2 * kPM, Cfg::kN);
+            constexpr uint32_t idesc = idesc_bf16(2 * kPM, N);
             uint32_t pre = 0;       // the coming stage was found ready by an early test
             int g = 0, nth = 0;
             for (int u = t_begin; u < t_end; ++nth) {
@@ -913,13 +936,13 @@ prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap t
         const int half = (warp - kConvWarps) >> 2;
         const int row = (warp & 3) * 32 + lane;
         const uint32_t taddr = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + half * kHalfTok;
-        const uint32_t buf = s32(b_full) + 256 + (warp - kConvWarps) * 1024;
+        const uint32_t buf = s32(b_full) + 384 + (warp - kConvWarps) * 1024;
         int nth = 0;
         // ---- T': thread = token.  Part of pair q: [c / 4][128 tokens] float4; a pair has at most one that starts with its tile and
         // one that does not.
         auto part = [&](int q, bool starts) { return p.t_part + ((size_t)(2 * q + (starts ? 1 : 0)) * 2 + rank) * ((size_t)kPM * p.t_n / 4) + row; };
         auto store4 = [&](int tile, int c, float4 v) {
-            const int token = (tile / p.t_chunks) * Cfg::kN + (int)rank * kPM + row, col = (tile % p.t_chunks) * p.t_n + c;
+            const int token = (tile / p.t_chunks) * kTTok + (int)rank * kPM + row, col = (tile % p.t_chunks) * p.t_n + c;
             if (token >= p.b || col >= p.r) return;
             __nv_bfloat162 lo = __floats2bfloat162_rn(p.t_scale * v.x, p.t_scale * v.y), hi = __floats2bfloat162_rn(p.t_scale * v.z, p.t_scale * v.w);
             *reinterpret_cast<uint2*>(p.t_out + (size_t)token * p.r + col) = make_uint2(*reinterpret_cast<uint32_t*>(&lo), *reinterpret_cast<uint32_t*>(&hi));
@@ -1001,11 +1024,12 @@ prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap t
             const int tok0 = ti.n0 + half * kHalfTok, row8 = ti.m0 + (warp & 3) * 32 + (lane & 3) * 8;
             const int n_tok = row8 < p.m_total ? p.b - tok0 : 0;
             __nv_bfloat16* out = p.out + (size_t)(tok0 + (lane >> 2)) * p.ldo + row8;
+            constexpr int kPass = kHalfTok < 64 ? kHalfTok : 64;
 #pragma unroll
-            for (int c0 = 0; c0 < kHalfTok; c0 += 64) {
-                uint32_t y[32];                                              // bf16 pairs of neighbouring tokens
+            for (int c0 = 0; c0 < kHalfTok; c0 += kPass) {
+                uint32_t y[kPass / 2];                                       // bf16 pairs of neighbouring tokens
 #pragma unroll
-                for (int c1 = 0; c1 < 64; c1 += 32) {
+                for (int c1 = 0; c1 < kPass; c1 += 32) {
                     uint32_t r[32];
                     tmem_ld32(taddr + c0 + c1, r);
 #pragma unroll
@@ -1014,13 +1038,13 @@ prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap t
                         y[(c1 + c) / 2] = *reinterpret_cast<uint32_t*>(&v);
                     }
                 }
-                if (c0 + 64 == kHalfTok) {
+                if (c0 + kPass == kHalfTok) {
                     fence_before_sync();
                     __syncwarp();
                     if (lane == 0) mbar_arrive_remote_release(peer_addr(acc_empty, 0));
                 }
 #pragma unroll
-                for (int c1 = 0; c1 < 64; c1 += 16) {
+                for (int c1 = 0; c1 < kPass; c1 += 16) {
                     if (c0 + c1 >= p.b - tok0) break;
 #pragma unroll
                     for (int c = 0; c < 16; ++c)
@@ -1112,6 +1136,18 @@ static bool pf_map(CUtensorMap* map, const void* base, CUtensorMapDataType type,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// bf16 rows as 64-column sub-tiles: one box of box_rows rows x 2 sub-tiles of 128 bytes, in that order.
+static bool pf_map3(CUtensorMap* map, const void* base, uint64_t cols, uint64_t rows, int box_rows) {
+    PfEncodeTiledFn fn = reinterpret_cast<PfEncodeTiledFn>(tensor_map_encoder());
+    if (!fn) return false;
+    cuuint64_t dims[3] = {64, rows, cols / 64};
+    cuuint64_t strides[2] = {cols * 2, 128};
+    cuuint32_t box[3] = {64, (cuuint32_t)box_rows, 2};
+    cuuint32_t estr[3] = {1, 1, 1};
+    return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+              CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 bool prefill_supports(int b, int d_out, int d_in, int r) {
     // (when the rows of the index-byte array, d_in / 8 bytes, are no 16-byte multiples they come by cp.async)
     return b >= 1 && d_out % 16 == 0 && d_in % kPBK == 0 && r % 16 == 0 && r >= 0;
@@ -1125,19 +1161,33 @@ static size_t pair_part_bytes(int r, int sm_count) { return (size_t)(sm_count / 
 // Pairs that share the work of T'.  Each tile in equal parts, one a pair, where that uses four fifths of the pairs or more
 // (a pair then has one part to write, and the pairs that read the same X walk it together); else an even share each.
 // Four stages (a microsecond and a half) or more for a part: below that its start and end dominate.
-static int t_share(int tiles, int stages, int pairs) {
+// Where the tiles leave pairs without one and those can make T' in about the time of the others' sparse phase, they do it
+// alone (`spare` pairs, `main_stages` 128-column stages): the others start their tiles at once.
+static int t_share(int tiles, int stages, int pairs, int spare, int main_stages) {
     const int most = stages < 4 ? 1 : stages / 4;
-    int parts = pairs / tiles < most ? pairs / tiles : most;
+    int parts = spare / tiles < most ? spare / tiles : most;
+    if (parts >= 1 && (long long)ceil_div(stages, parts) <= main_stages) return tiles * parts;
+    parts = pairs / tiles < most ? pairs / tiles : most;
     if (parts >= 1 && (parts == most || tiles * parts * 5 >= pairs * 4)) return tiles * parts;
     return (long long)tiles * most < pairs ? tiles * most : pairs;
 }
 
-// Wide token tiles (pair kernel) when they give a quarter of the SMs or more a 128-row tile, else narrow ones (measured: with 64
-// tiles of 128 x 256 on 148 SMs the wide variant is a third faster than 256 tiles of 128 x 64; with 32 it is
-// slower), and when the words of its T' tiles fit their region.
-static bool runs_wide(int b, int d_out, int r, int sm_count) {
-    return (long long)ceil_div(d_out, kPM) * ceil_div(b, 256) * 4 >= (long long)sm_count &&
-           (size_t)ceil_div(b, 256) * t_chunks(r) <= kSyncTiles;
+// Token tile of the pair kernel: the narrowest with which every tile has a pair of its own, else 256 (a tile takes about the
+// same time whatever its width).
+static int pair_tile(int b, int d_out, int sm_count) {
+    for (int n = 64; n < 256; n *= 2)
+        if ((long long)ceil_div(d_out, 2 * kPM) * ceil_div(b, n) <= sm_count / 2) return n;
+    return 256;
+}
+
+// The pair kernel when its 128 x 256 tiles would give a quarter of the SMs or more a tile, and when the words of its T' tiles fit
+// their region.  The dispatcher (`automatic`) also takes it for smaller problems with eight tiles or more (4096 x 4096, 100 tokens
+// 25 -> 22 us, 200 tokens 45 -> 26), unless both the batch and d_in are short (1024 -> 4096, 128 tokens: 17 us against 13);
+// asked for by name the one-CTA kernel keeps those.
+static bool runs_wide(int b, int d_out, int d_in, int r, int sm_count, bool automatic) {
+    if ((size_t)ceil_div(b, kTTok) * t_chunks(r) > kSyncTiles) return false;
+    if ((long long)ceil_div(d_out, kPM) * ceil_div(b, 256) * 4 >= (long long)sm_count) return true;
+    return automatic && (b >= 192 || d_in >= 2048) && (long long)ceil_div(d_out, 2 * kPM) * ceil_div(b, pair_tile(b, d_out, sm_count)) >= 8;
 }
 
 size_t prefill_workspace_bytes(int b, int d_out, int d_in, int r) {
@@ -1146,7 +1196,7 @@ size_t prefill_workspace_bytes(int b, int d_out, int d_in, int r) {
     if (r == 0) return tq;
     const PrePlan pl = pre_plan(b, d_in, r, pre_sm_count());
     const size_t narrow = pl.slices > 1 ? (size_t)pl.slices * b * r * sizeof(float) : 0, wide = pair_part_bytes(r, pre_sm_count());
-    return tq + (runs_wide(b, d_out, r, pre_sm_count()) || wide > narrow ? wide : narrow);     // (the pair kernel may be asked for by name)
+    return tq + (wide > narrow ? wide : narrow);           // (either kernel may be asked for by name)
 }
 
 static std::atomic<int> g_pairs[64];               // pairs resident at once
@@ -1168,10 +1218,11 @@ static slim_status_t launch_tile_kernel(const PrefillParams& q, int m_rows, cons
     return e == cudaSuccess ? SLIM_OK : SLIM_ERR_CUDA;
 }
 
+template <int N>
 static slim_status_t launch_pair(const PrefillParams& p, const CUtensorMap& tmV, const CUtensorMap& tmM, const CUtensorMap& tmX, const CUtensorMap& tmA2,
-                                 const CUtensorMap& tmB2, const CUtensorMap& tmR, int pairs, cudaStream_t st) {
+                                 const CUtensorMap& tmB2, const CUtensorMap& tmR, const CUtensorMap& tmXt, int pairs, cudaStream_t st) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(2 * pairs); cfg.blockDim = dim3(PairCfg::kThreads); cfg.dynamicSmemBytes = PairCfg::kSmem; cfg.stream = st;
+    cfg.gridDim = dim3(2 * pairs); cfg.blockDim = dim3(kPairThreads); cfg.dynamicSmemBytes = PairCfg<N>::kSmem; cfg.stream = st;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
@@ -1180,7 +1231,7 @@ static slim_status_t launch_pair(const PrefillParams& p, const CUtensorMap& tmV,
     attr[1].id = cudaLaunchAttributeCooperative;
     attr[1].val.cooperative = 1;
     cfg.attrs = attr; cfg.numAttrs = p.t_pairs > 0 ? 2 : 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, prefill_pair_kernel, p, tmV, tmM, tmX, tmA2, tmB2, tmR);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, prefill_pair_kernel<N>, p, tmV, tmM, tmX, tmA2, tmB2, tmR, tmXt);
     count_launch(1);
     return e == cudaSuccess ? SLIM_OK : SLIM_ERR_CUDA;
 }
@@ -1188,7 +1239,7 @@ static slim_status_t launch_pair(const PrefillParams& p, const CUtensorMap& tmV,
 slim_status_t launch_prefill(const __nv_bfloat16* X, int b, const uint8_t* vals, const uint8_t* meta,
                              float s, const __nv_bfloat16* L, const __nv_bfloat16* R, int r,
                              int d_out, int d_in, __nv_bfloat16* Y, void* ws, uint32_t* status_dev,
-                             cudaStream_t st, bool force_pair)
+                             cudaStream_t st, bool force_pair, bool automatic)
 {
     slim_status_t err;
     const DeviceInfo* di = device_info(&err);
@@ -1198,37 +1249,42 @@ slim_status_t launch_prefill(const __nv_bfloat16* X, int b, const uint8_t* vals,
     cudaGetDevice(&dev);
     if (dev < 0 || dev >= 64) return SLIM_ERR_CUDA;
     if (!g_prefill_attr_set[dev].load(std::memory_order_acquire)) {
-        if (cudaFuncSetAttribute(prefill_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PairCfg::kSmem) != cudaSuccess ||
+        if (cudaFuncSetAttribute(prefill_pair_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PairCfg<256>::kSmem) != cudaSuccess ||
+            cudaFuncSetAttribute(prefill_pair_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PairCfg<128>::kSmem) != cudaSuccess ||
+            cudaFuncSetAttribute(prefill_pair_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PairCfg<64>::kSmem) != cudaSuccess ||
             cudaFuncSetAttribute(prefill_kernel<64, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PfCfg<64, false>::kSmem) != cudaSuccess ||
             cudaFuncSetAttribute(prefill_kernel<64, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PfCfg<64, true>::kSmem) != cudaSuccess ||
             cudaFuncSetAttribute(prefill_kernel<256, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PfCfg<256, true>::kSmem) != cudaSuccess)
             return SLIM_ERR_CUDA;
         cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(2); cfg.blockDim = dim3(PairCfg::kThreads); cfg.dynamicSmemBytes = PairCfg::kSmem;
+        cfg.gridDim = dim3(2); cfg.blockDim = dim3(kPairThreads); cfg.dynamicSmemBytes = PairCfg<256>::kSmem;
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeClusterDimension;
         attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
         cfg.attrs = attr; cfg.numAttrs = 1;
         int n = 0;
-        if (cudaOccupancyMaxActiveClusters(&n, prefill_pair_kernel, &cfg) != cudaSuccess || n < 1) return SLIM_ERR_CUDA;
+        if (cudaOccupancyMaxActiveClusters(&n, prefill_pair_kernel<256>, &cfg) != cudaSuccess || n < 1) return SLIM_ERR_CUDA;
         g_pairs[dev].store(n < di->sm_count / 2 ? n : di->sm_count / 2, std::memory_order_relaxed);
         g_prefill_attr_set[dev].store(true, std::memory_order_release);
     }
     __nv_bfloat16* Tq = reinterpret_cast<__nv_bfloat16*>(reinterpret_cast<char*>(ws) + SLIM_WORKSPACE_SYNC_BYTES + kSmallTBytes);
     const float s_eff = s != 0.f ? s : 1.f;       // with s == 0 only the adapter term remains
-    const bool wide = force_pair || runs_wide(b, d_out, r, di->sm_count);
+    const bool wide = force_pair || runs_wide(b, d_out, d_in, r, di->sm_count, automatic);
     if (force_pair && ceil_div(d_out, kPM) % 2 != 0) return SLIM_ERR_UNSUPPORTED_SHAPE;
-    const int xbox = wide ? PairCfg::kHalfTok : 64;       // token rows one CTA loads per stage = one TMA box
-    const int dk = wide ? PairCfg::kDK : PfCfg<64>::kDK;  // columns of a dense stage of the main kernel
-    CUtensorMap tmV, tmM, tmX, tmXpre, tmA2, tmB2, tmR;
+    const int tile_n = wide ? pair_tile(b, d_out, di->sm_count) : 64;
+    const int xbox = wide ? tile_n / 2 : 64;              // token rows one CTA loads per stage = one TMA box
+    const int dk = wide ? PairCfg<256>::kDK : PfCfg<64>::kDK;      // columns of a dense stage of the main kernel
+    CUtensorMap tmV, tmM, tmX, tmXpre, tmA2, tmB2, tmR, tmXt;
     bool ok = pf_map(&tmV, vals, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)d_in / 4, (uint64_t)d_out, kPkCols / 4, kPM, 64) &&
               (d_in % 128 != 0 || pf_map(&tmM, meta, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)d_in / 8, (uint64_t)d_out, kPkCols / 8, kPM, 32)) &&
-              pf_map(&tmX, X, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (uint64_t)d_in, (uint64_t)b, 64, xbox, 128);
+              (wide ? pf_map3(&tmX, X, (uint64_t)d_in, (uint64_t)b, xbox)
+                    : pf_map(&tmX, X, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (uint64_t)d_in, (uint64_t)b, 64, xbox, 128));
     if (!ok) return SLIM_ERR_CUDA;
     if (d_in % 128 != 0) tmM = tmV;              // not used
-    tmA2 = tmX; tmB2 = tmX; tmR = tmX;    // not used when r == 0
+    tmA2 = tmX; tmB2 = tmX; tmR = tmX; tmXt = tmX;    // not used when r == 0
     if (r > 0 && wide) {
-        ok = pf_map(&tmR, R, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (uint64_t)d_in, (uint64_t)r, 64, t_width(r) / 2, 128);
+        ok = pf_map(&tmR, R, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (uint64_t)d_in, (uint64_t)r, 64, t_width(r) / 2, 128) &&
+             pf_map(&tmXt, X, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (uint64_t)d_in, (uint64_t)b, 64, kPM, 128);
         if (!ok) return SLIM_ERR_CUDA;
     } else if (r > 0) {
         // T' = (X R^T) / s : dense phase only, output rows = adapter index
@@ -1267,16 +1323,16 @@ slim_status_t launch_prefill(const __nv_bfloat16* X, int b, const uint8_t* vals,
     }
     PrefillParams p = {};
     p.out = Y; p.ldo = d_out; p.m_total = d_out; p.b = b;
-    p.n1 = s != 0.f ? ceil_div(d_in, wide ? PairCfg::kSK : PfCfg<64>::kSK) : 0;
+    p.n1 = s != 0.f ? ceil_div(d_in, wide ? PairCfg<256>::kSK : PfCfg<64>::kSK) : 0;
     p.n2 = r > 0 ? ceil_div(r, dk) : 0;
     p.scale = s_eff; p.status = status_dev; p.part = nullptr; p.k_per = 0;
     p.meta = d_in % 128 != 0 ? meta : nullptr; p.meta_pitch = d_in / 8; p.d_in = d_in;
     if (p.n1 + p.n2 == 0)             // s == 0 and no adapters: the result is zero
         return cudaMemsetAsync(Y, 0, (size_t)b * d_out * 2, st) == cudaSuccess ? SLIM_OK : SLIM_ERR_CUDA;
-    note_token_tile(wide ? 256 : 64);
+    note_token_tile(wide ? tile_n : 64);
     slim_status_t rc;
     const bool dep = r > 0 && p.n1 > 0;               // sparse stages to run while T' is being made
-    p.row_pairs = ceil_div(d_out, 2 * kPM); p.tiles = p.row_pairs * ceil_div(b, PairCfg::kN);
+    p.row_pairs = ceil_div(d_out, 2 * kPM); p.tiles = p.row_pairs * ceil_div(b, tile_n);
     if (!wide) {
         rc = launch_tile_kernel<64, false>(p, d_out, tmV, tmM, tmX, tmA2, tmB2, st, 1, dep);
     } else {
@@ -1286,13 +1342,15 @@ slim_status_t launch_prefill(const __nv_bfloat16* X, int b, const uint8_t* vals,
         p.r = r;
         int grid = p.tiles < pairs ? p.tiles : pairs;
         if (r > 0) {
-            p.t_n = t_width(r); p.t_chunks = t_chunks(r); p.t_tiles = ceil_div(b, PairCfg::kN) * p.t_chunks; p.t_stages = d_in / PairCfg::kDK;
+            p.t_n = t_width(r); p.t_chunks = t_chunks(r); p.t_tiles = ceil_div(b, kTTok) * p.t_chunks; p.t_stages = d_in / PairCfg<256>::kDK;
             p.t_scale = 1.f / s_eff; p.t_out = Tq;
             p.t_part = reinterpret_cast<float4*>(reinterpret_cast<char*>(Tq) + ((size_t)b * r * sizeof(__nv_bfloat16) + 255) / 256 * 256);
-            p.t_pairs = t_share(p.t_tiles, p.t_stages, pairs);
-            if (grid < p.t_pairs) grid = p.t_pairs;
+            p.t_pairs = t_share(p.t_tiles, p.t_stages, pairs, pairs - grid, p.n1);
+            grid = grid + p.t_pairs < pairs ? grid + p.t_pairs : pairs;      // the last pairs make T'
         }
-        rc = launch_pair(p, tmV, tmM, tmX, tmA2, tmB2, tmR, grid, st);
+        rc = tile_n == 256 ? launch_pair<256>(p, tmV, tmM, tmX, tmA2, tmB2, tmR, tmXt, grid, st)
+           : tile_n == 128 ? launch_pair<128>(p, tmV, tmM, tmX, tmA2, tmB2, tmR, tmXt, grid, st)
+                           : launch_pair<64>(p, tmV, tmM, tmX, tmA2, tmB2, tmR, tmXt, grid, st);
     }
     if (rc != SLIM_OK) return rc;
     return SLIM_OK;
