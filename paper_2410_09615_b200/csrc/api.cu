@@ -66,9 +66,11 @@ static bool small_and_ragged(int b, int d_out, int d_in) {
     return (d_in % 128 != 0 || (d_out % 128 != 0 && b > 16)) && d_out < 256 && (long long)b * d_out * d_in < (1 << 24);
 }
 
-// The small-batch kernel's problems: one launch, up to 64 tokens.
+// The small-batch kernel's problems: up to 64 tokens, one launch.  From 33 tokens on its warp-level MMAs take longer than the
+// tensor-memory kernel's (5120 -> 13824, 64 tokens: 38 us against 26), which has the advantage once d_out gives it enough tiles
+// (8192 x 8192: a tie; 11008 -> 4096: 38 us against 41).
 static bool runs_small(int b, int d_out, int d_in, int r) {
-    return small_supports(b, d_out, d_in, r) && !small_and_ragged(b, d_out, d_in);
+    return small_supports(b, d_out, d_in, r) && !small_and_ragged(b, d_out, d_in) && !(b > 32 && d_out >= 8192);
 }
 
 static slim_kernel_t select_kernel(int b, int d_out, int d_in, int r) {

@@ -142,6 +142,7 @@ __device__ __forceinline__ void tma_tile3(uint32_t dst, const CUtensorMap* map, 
     asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
                  :: "r"(dst), "l"(map), "r"(0), "r"(y), "r"(z), "r"(bar) : "memory");
 }
+__device__ __forceinline__ void prefetch_map(const CUtensorMap* map) { asm volatile("prefetch.tensormap [%0];" :: "l"(map) : "memory"); }
 __device__ __forceinline__ void bulk_copy(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                  :: "r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
@@ -464,6 +465,13 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
     }
     __syncthreads();
     cluster_arrive();                                          // waited for before the first access to a peer
+    // Launched while the grid before it in the stream still runs (programmatic dependent launch): everything above needs
+    // no global memory, everything below comes after that grid.  The next grid may be set up as soon as all CTAs are here.
+    if (warp == kProdW && lane == 0) { prefetch_map(FMT == FMT_TILED ? &tmX : &tmV); prefetch_map(&tmR); prefetch_map(&tmL); }
+    if (warp == kProdX && lane == 0) { prefetch_map(&tmX); prefetch_map(&tmM); }
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (warp == kProdW || warp == kProdX) asm volatile("fence.proxy.async;" ::: "memory");      // what that grid wrote is read through TMA
     bool ok = true;
 
     int p_it = 0;                                              // producers: next stage
@@ -1007,10 +1015,12 @@ slim_status_t launch_small(const __nv_bfloat16* X, int b, const uint8_t* vals, c
     if (!ok) return SLIM_ERR_CUDA;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(C * (p.tiles + p.groups))); cfg.blockDim = dim3(threads_of(nt)); cfg.dynamicSmemBytes = smem_bytes(nt); cfg.stream = st;
-    cudaLaunchAttribute a[1];
+    cudaLaunchAttribute a[2];
     a[0].id = cudaLaunchAttributeClusterDimension;
     a[0].val.clusterDim.x = (unsigned)C; a[0].val.clusterDim.y = 1; a[0].val.clusterDim.z = 1;
-    cfg.attrs = a; cfg.numAttrs = 1;
+    a[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    a[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = a; cfg.numAttrs = 2;
     const cudaError_t e = cudaLaunchKernelEx(&cfg, pick(nt, fmt, qa), p, tmV, tmM, tmX, tmR, tmL);
     count_launch(1);
     return e == cudaSuccess ? SLIM_OK : SLIM_ERR_CUDA;
