@@ -14,7 +14,8 @@
 //   A tile's cluster streams the packed weight and the activations through a ring of stages by TMA
 // (256 rows x 64 value bytes, x 32 index bytes, b tokens x 512 bytes; two requesting warps, since one
 // thread starts a request every 220 cycles and the engine takes about one 32-64 byte row a cycle),
-// then the columns of L, waiting for just the words of T it multiplies, then writes
+// then the columns of L (32 of bf16, or 64 int4 codes a row and stage: codes by plain loads of the consumers, one step ahead,
+// cost 8192 -> 28672 with 16 tokens 58.7 us instead of 47.6), waiting for just the words of T it multiplies, then writes
 // Y = s X Q^T + T L^T.
 //
 // Fragments of the sparse MMA.  Inside a 256-column unit the four 64-column regions are q = 2 a + h; step
@@ -147,6 +148,10 @@ __device__ __forceinline__ void bulk_copy(uint32_t dst, const void* src, uint32_
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                  :: "r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
 }
+// Eight bytes, or (not `in`) eight zero bytes.
+__device__ __forceinline__ void cp_async8(uint32_t dst, const void* src, bool in) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" :: "r"(dst), "l"(src), "r"(in ? 8 : 0) : "memory");
+}
 __device__ __forceinline__ void consumer_sync() { asm volatile("bar.sync 1, %0;" :: "n"(kConsumers) : "memory"); }
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
@@ -171,14 +176,12 @@ __device__ __forceinline__ unsigned long long ld_gpu64(const unsigned long long*
     asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
     return v;
 }
+// Two entries, each seen whole (the vector form is two 64-bit accesses).
+__device__ __forceinline__ void ld_gpu64x2(const unsigned long long* p, unsigned long long& x, unsigned long long& y) {
+    asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(x), "=l"(y) : "l"(p) : "memory");
+}
 __device__ __forceinline__ void st_gpu64(unsigned long long* p, unsigned long long v) {
     asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" :: "l"(p), "l"(v) : "memory");
-}
-// Streamed once: keep it out of L1.
-__device__ __forceinline__ uint32_t ldg_stream32(const void* p) {
-    uint32_t v;
-    asm volatile("ld.global.nc.L1::no_allocate.u32 %0, [%1];" : "=r"(v) : "l"(p));
-    return v;
 }
 __device__ __forceinline__ void ldsm4(uint32_t addr, uint4& v) {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
@@ -371,8 +374,8 @@ __device__ __forceinline__ void ask_T(unsigned long long (&v)[NE], const unsigne
 #pragma unroll
     for (int n = 0; n < NE; ++n) v[n] = at[n] ? ld_gpu64(at[n]) : (unsigned long long)call << 32;
 }
-template <int NE>
-__device__ __forceinline__ bool wait_T(unsigned long long (&v)[NE], const unsigned long long* const (&at)[NE], uint32_t call)
+template <int NE, typename F>
+__device__ __forceinline__ bool wait_words(unsigned long long (&v)[NE], uint32_t call, F ask)
 {
     unsigned long long t0 = 0;
     for (uint32_t spin = 0;; ++spin) {
@@ -388,7 +391,34 @@ __device__ __forceinline__ bool wait_T(unsigned long long (&v)[NE], const unsign
             if (__any_sync(0xffffffffu, late)) return false;
         }
         __nanosleep(40);
-        ask_T<NE>(v, at, call);
+        ask();
+    }
+}
+template <int NE>
+__device__ __forceinline__ bool wait_T(unsigned long long (&v)[NE], const unsigned long long* const (&at)[NE], uint32_t call)
+{
+    return wait_words(v, call, [&] { ask_T<NE>(v, at, call); });
+}
+
+// The words of eight codes of rows g and g + 8 of a 16-row tile, step h of a stage of L's codes (32-byte rows, 32-byte
+// swizzle), and their product with T.  Integer products are scaled once.
+__device__ __forceinline__ uint2 l_codes(uint32_t stage, int rb, int m, int h, const Lane& ln) {
+    const uint32_t at = stage + (uint32_t)(rb * 64 + m * 16 + ln.g) * 32 + ((uint32_t)(h ^ (ln.g >> 2)) << 4) + ln.t * 4;
+    return make_uint2(lds32(at), lds32(at + 256));
+}
+template <int NW>
+__device__ __forceinline__ void code_tile(float (&acc)[NW][4], uint2 w, float sc0, float sc1, const uint4 (&tb)[NW])
+{
+    uint32_t a[4], d[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) { a[q] = nibbles_to_bf16x2(w.x >> (4 * q)); d[q] = nibbles_to_bf16x2(w.y >> (4 * q)); }
+#pragma unroll
+    for (int n = 0; n < NW; ++n) {
+        float pt[4] = {0.f, 0.f, 0.f, 0.f};
+        mma_16816(pt, a[0], d[0], a[1], d[1], tb[n].x, tb[n].y);
+        mma_16816(pt, a[2], d[2], a[3], d[3], tb[n].z, tb[n].w);
+        acc[n][0] = fmaf(pt[0], sc0, acc[n][0]); acc[n][1] = fmaf(pt[1], sc0, acc[n][1]);
+        acc[n][2] = fmaf(pt[2], sc1, acc[n][2]); acc[n][3] = fmaf(pt[3], sc1, acc[n][3]);
     }
 }
 
@@ -452,7 +482,7 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
     const int piece = cluster, tile = cluster - p.groups;
     const int u0 = (int)(rank * (unsigned)p.units) >> logC, u1 = (int)((rank + 1) * (unsigned)p.units) >> logC;
     const int u_end = p.s != 0.f ? u1 : u0;                    // s == 0: the adapter term alone
-    const int l_steps = ceil_div(p.r, 32);
+    const int l_steps = ceil_div(p.r, 32), l_chunks = ceil_div(p.r, QA ? 64 : 32);      // steps of 32 columns; stages of L
 
     if (threadIdx.x == 0) {
         // a stage's barrier counts both producers (and, with index bytes by cp.async, the lanes of one of them)
@@ -481,6 +511,22 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
         ++p_it;
         return st;
     };
+    // L's codes where rows of r / 2 bytes are no 16-byte multiples, half of the tile by either producer: 8-byte pieces, stored
+    // as the TMA's 32-byte swizzle would.  Each lane's pieces are one more arrival that the barrier waits for.
+    const bool l_by_lanes = QA && p.r % 32 != 0;
+    auto codes_of_L = [&](int lc, uint32_t dst, uint32_t bar, int first) {
+        const int q = lane & 3, row0 = tile * kRows;
+        const bool col_in = lc * 64 + q * 16 < p.r;
+#pragma unroll 4
+        for (int r = first + (lane >> 2); r < first + kRows / 2; r += 8) {
+            const bool in = col_in && row0 + r < p.d_out;
+            const uint8_t* src = static_cast<const uint8_t*>(p.L) + (in ? (size_t)(row0 + r) * (p.r / 2) + lc * 32 + q * 8 : 0);
+            cp_async8(dst + r * 32 + (((q >> 1) ^ ((r >> 2) & 1)) << 4) + (q & 1) * 8, src, in);
+        }
+        asm volatile("cp.async.mbarrier.arrive.shared::cta.b64 [%0];" :: "r"(bar) : "memory");
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar);
+    };
     if (warp == kProdW) {
         // ============================ the weight, R, L ============================
         const int row0 = tile * kRows;
@@ -507,17 +553,19 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
                     tma_tile(dst, &tmV, u * 64, row0, bar);
                 }
             }
-            if (!QA)
-                for (int ls = (int)rank; ls < l_steps; ls += (int)C) {
-                    const int st = acquire();
-                    const uint32_t bar = full + 8 * st;
-                    if (lane == 0) {
-                        mbar_expect(bar, kRows * 64);
-                        mbar_arrive(bar);                       // in place of the other producer
-                        tma_tile(smem + st * kStage, &tmL, ls * 32, row0, bar);
-                    }
-                    if (FMT == FMT_PACKED_LD) mbar_arrive(bar);
+            // 32 columns of L in bf16, or 64 codes a row
+            for (int lc = (int)rank; lc < l_chunks; lc += (int)C) {
+                const int st = acquire();
+                const uint32_t dst = smem + st * kStage, bar = full + 8 * st;
+                if (l_by_lanes) {
+                    codes_of_L(lc, dst, bar, 0);
+                } else if (lane == 0) {
+                    mbar_expect(bar, kRows * (QA ? 32 : 64));
+                    mbar_arrive(bar);                           // in place of the other producer
+                    tma_tile(dst, &tmL, lc * 32, row0, bar);
                 }
+                if (FMT == FMT_PACKED_LD) mbar_arrive(bar);
+            }
         }
         cluster_wait();
     } else if (warp == kProdX) {
@@ -568,11 +616,16 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
                         const bool in = col_in && row0 + r < p.d_out;
                         const uint8_t* src = p.meta + (in ? (size_t)(row0 + r) * pitch + (size_t)u * 32 + q * 8 : 0);
                         const uint32_t d = dst + kValsBytes + r * 32 + (((q >> 1) ^ ((r >> 2) & 1)) << 4) + (q & 1) * 8;
-                        asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" :: "r"(d), "l"(src), "r"(in ? 8 : 0) : "memory");
+                        cp_async8(d, src, in);
                     }
                     asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" :: "r"(bar) : "memory");
                 }
             }
+            if (l_by_lanes)
+                for (int lc = (int)rank; lc < l_chunks; lc += (int)C) {
+                    const int st = acquire();
+                    codes_of_L(lc, smem + st * kStage, full + 8 * st, kRows / 2);
+                }
         }
         cluster_wait();
     } else if (NT >= 4 && warp >= kFetchT) {
@@ -581,8 +634,9 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
         if (!makes_T && p.r > 0) {
             const uint32_t call = (uint32_t)(ld_gpu64(p.departures) >> 16) + 1u;
             constexpr int kPer = NT * 2;                       // words a lane fetches
-            int it = 0;
-            for (int ls = (int)rank; ls < l_steps; ls += (int)C, ++it) {
+            const int steps = (l_chunks - (int)rank + (int)C - 1) / (int)C * (QA ? 2 : 1);
+            for (int it = 0; it < steps; ++it) {
+                const int ls = QA ? 2 * ((int)rank + (it >> 1) * (int)C) + (it & 1) : (int)rank + it * (int)C;
                 const int st = it % C_::kTSlots, use = it / C_::kTSlots;
                 if (use > 0) ok = mbar_wait(t_empty + 8 * st, (use - 1) & 1) && ok;
                 unsigned long long v[kPer];
@@ -710,51 +764,40 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
                     for (int e = 0; e < 4; ++e) acc[m][n][e] *= p.s;
             // ---------------- T L^T
             if constexpr (NT >= 4) {
-                // T from shared memory.  bf16: with four n-tiles kk picks the step's MMA depth; codes: the row tiles
+                // T from shared memory.  With four n-tiles kk picks the step's MMA depth (bf16)
                 int lt = 0;
-                for (int ls = (int)rank; ls < l_steps; ls += (int)C, ++lt) {
-                    const int ts = lt % C_::kTSlots;
-                    const uint32_t tslot = part + ts * C_::kTSlot;
-                    const int c = ls * 32 + 8 * ln.t;               // codes: r is a multiple of 16, a thread's 8 columns exist or not
-                    uint32_t lc[8];
-                    float sc[8];
-                    uint32_t stage = 0;
-                    if (QA) {
+                for (int lc = (int)rank; lc < l_chunks; lc += (int)C) {
+                    const uint32_t stage = wait_stage();
+                    if constexpr (QA) {
+                        // codes: four n-tiles, kk picks the row tiles of both steps of the stage
+                        float sc[8];
 #pragma unroll
-                        for (int m = 0; m < 8; ++m) {
-                            const bool mine = (m >> 1) < mts && (NT == 8 || (m >> 2) == kk);
-                            const size_t row = (size_t)(row0 + ln.g + 8 * m);
-                            lc[m] = mine && c < p.r ? ldg_stream32(static_cast<const uint8_t*>(p.L) + row * (p.r / 2) + c / 2) : 0u;
-                            sc[m] = mine ? __bfloat162float(p.Ls[row * ((p.r + 127) >> 7) + (ls >> 2)]) : 0.f;
+                        for (int m = 0; m < 8; ++m)
+                            sc[m] = (m >> 1) < mts && (NT == 8 || (m >> 2) == kk) ? __bfloat162float(p.Ls[(size_t)(row0 + ln.g + 8 * m) * ((p.r + 127) >> 7) + (lc >> 1)]) : 0.f;
+#pragma unroll 1
+                        for (int h = 0; h < 2; ++h, ++lt) {
+                            const int ts = lt % C_::kTSlots;
+                            const uint32_t tslot = part + ts * C_::kTSlot;
+                            ok = mbar_wait(t_full + 8 * ts, (lt / C_::kTSlots) & 1) && ok;
+                            if (mts > 0 && 2 * lc + h < l_steps) {
+                                uint4 tb[kNW];
+#pragma unroll
+                                for (int n = 0; n < kNW; ++n)
+                                    tb[n] = pair_four_apart(lds128(tslot + ((n_first + n) * 8 + ln.g) * 64 + ((ln.t ^ ((ln.g >> 1) & 3)) << 4)));
+#pragma unroll
+                                for (int m = 0; m < 4; ++m)
+                                    if (NT == 8 || (m >> 1) == kk) code_tile<kNW>(acc[m], l_codes(stage, rb, m, h, ln), sc[2 * m], sc[2 * m + 1], tb);
+                            }
+                            __syncwarp();
+                            if (lane == 0) mbar_arrive(t_empty + 8 * ts);
                         }
                     } else {
-                        stage = wait_stage();
-                    }
-                    ok = mbar_wait(t_full + 8 * ts, (lt / C_::kTSlots) & 1) && ok;
-                    if (mts > 0) {
-                        const int mat = lane >> 3, r8 = lane & 7;
-                        if (QA) {
-                            uint4 tb[kNW];
-#pragma unroll
-                            for (int n = 0; n < kNW; ++n)
-                                tb[n] = pair_four_apart(lds128(tslot + ((n_first + n) * 8 + ln.g) * 64 + ((ln.t ^ ((ln.g >> 1) & 3)) << 4)));
-#pragma unroll
-                            for (int m = 0; m < 4; ++m) {
-                                if (NT == 8 || (m >> 1) == kk) {
-                                    uint32_t a[4], d[4];
-#pragma unroll
-                                    for (int q = 0; q < 4; ++q) { a[q] = nibbles_to_bf16x2(lc[2 * m] >> (4 * q)); d[q] = nibbles_to_bf16x2(lc[2 * m + 1] >> (4 * q)); }
-#pragma unroll
-                                    for (int n = 0; n < kNW; ++n) {
-                                        float pt[4] = {0.f, 0.f, 0.f, 0.f};
-                                        mma_16816(pt, a[0], d[0], a[1], d[1], tb[n].x, tb[n].y);
-                                        mma_16816(pt, a[2], d[2], a[3], d[3], tb[n].z, tb[n].w);
-                                        acc[m][n][0] = fmaf(pt[0], sc[2 * m], acc[m][n][0]); acc[m][n][1] = fmaf(pt[1], sc[2 * m], acc[m][n][1]);
-                                        acc[m][n][2] = fmaf(pt[2], sc[2 * m + 1], acc[m][n][2]); acc[m][n][3] = fmaf(pt[3], sc[2 * m + 1], acc[m][n][3]);
-                                    }
-                                }
-                            }
-                        } else {
+                        const int ls = lc, ts = lt % C_::kTSlots;
+                        const uint32_t tslot = part + ts * C_::kTSlot;
+                        ++lt;
+                        ok = mbar_wait(t_full + 8 * ts, ((lt - 1) / C_::kTSlots) & 1) && ok;
+                        if (mts > 0) {
+                            const int mat = lane >> 3, r8 = lane & 7;
 #pragma unroll
                             for (int h = 0; h < 2; ++h) {
                                 if ((NT == 8 || h == kk) && ls * 32 + 16 * h < p.r) {
@@ -775,10 +818,10 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
                                 }
                             }
                         }
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(t_empty + 8 * ts);
                     }
-                    if (!QA) release();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(t_empty + 8 * ts);
+                    release();
                 }
             } else if constexpr (!QA) {
                 // kk picks the MMA depth of 16 of a 32-column step; the words of T are asked for one step ahead
@@ -817,54 +860,47 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
                     }
                     release();
                 }
-            } else if (mts > 0) {
-                // codes by plain loads (rows of r / 2 bytes need not be 16-byte multiples), one step ahead
-                const int stride = 2 * (int)C;
-                uint32_t lc[8];
-                auto load = [&](int ls) {
-                    const int c = ls * 32 + 8 * ln.t;               // r is a multiple of 16: a thread's 8 columns exist or not
-#pragma unroll
-                    for (int m = 0; m < 8; ++m)                     // rows g + 8 m of the warp's 64
-                        lc[m] = c < p.r && (m >> 1) < mts ? ldg_stream32(static_cast<const uint8_t*>(p.L) + (size_t)(row0 + ln.g + 8 * m) * (p.r / 2) + c / 2) : 0u;
-                };
-                const int ls0 = (int)rank * 2 + kk;
-                load(ls0);
-                for (int ls = ls0; ls < l_steps; ls += stride) {
-                    const int c = ls * 32 + 8 * ln.t;
-                    float sc[8];
-#pragma unroll
-                    for (int m = 0; m < 8; ++m)
-                        sc[m] = (m >> 1) < mts ? __bfloat162float(p.Ls[(size_t)(row0 + ln.g + 8 * m) * ((p.r + 127) >> 7) + (ls >> 2)]) : 0.f;
-                    uint4 tb[kNW];
+            } else {
+                // codes: kk picks the step of a stage of 64; scales and words of T are asked for one stage ahead
+                const uint32_t per_row = (uint32_t)((p.r + 127) >> 7);
+                __nv_bfloat16 next[8];
+                unsigned long long v[4 * kNW];
+                const unsigned long long* at = p.T + (size_t)ln.g * (p.r / 2) + 4 * ln.t;
+                auto ask = [&](int ls) {
 #pragma unroll
                     for (int n = 0; n < kNW; ++n) {
-                        const int tok = n * 8 + ln.g;
-                        unsigned long long v[4];
-                        const unsigned long long* at[4];
+                        const bool in = ls * 32 + 8 * ln.t < p.r && n * 8 + ln.g < p.b;      // r is a multiple of 16: a thread's 8 columns exist or not
 #pragma unroll
-                        for (int q = 0; q < 4; ++q) at[q] = c < p.r && tok < p.b ? p.T + (size_t)tok * (p.r / 2) + (c >> 1) + q : nullptr;
-                        ask_T<4>(v, at, call);
-                        ok = wait_T<4>(v, at, call) && ok;
-                        tb[n] = pair_four_apart(make_uint4((uint32_t)v[0], (uint32_t)v[1], (uint32_t)v[2], (uint32_t)v[3]));
-                    }
-                    uint32_t now[8];
-#pragma unroll
-                    for (int m = 0; m < 8; ++m) now[m] = lc[m];
-                    load(ls + stride);
-#pragma unroll
-                    for (int m = 0; m < 4; ++m) {
-                        uint32_t a[4], d[4];
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) { a[q] = nibbles_to_bf16x2(now[2 * m] >> (4 * q)); d[q] = nibbles_to_bf16x2(now[2 * m + 1] >> (4 * q)); }
-#pragma unroll
-                        for (int n = 0; n < kNW; ++n) {
-                            float pt[4] = {0.f, 0.f, 0.f, 0.f};
-                            mma_16816(pt, a[0], d[0], a[1], d[1], tb[n].x, tb[n].y);
-                            mma_16816(pt, a[2], d[2], a[3], d[3], tb[n].z, tb[n].w);
-                            acc[m][n][0] = fmaf(pt[0], sc[2 * m], acc[m][n][0]); acc[m][n][1] = fmaf(pt[1], sc[2 * m], acc[m][n][1]);
-                            acc[m][n][2] = fmaf(pt[2], sc[2 * m + 1], acc[m][n][2]); acc[m][n][3] = fmaf(pt[3], sc[2 * m + 1], acc[m][n][3]);
+                        for (int q = 0; q < 4; q += 2) {
+                            v[4 * n + q] = v[4 * n + q + 1] = (unsigned long long)call << 32;
+                            if (in) ld_gpu64x2(at + n * 4 * p.r + 16 * ls + q, v[4 * n + q], v[4 * n + q + 1]);
                         }
                     }
+                };
+                auto scales = [&](int lc) {
+#pragma unroll
+                    for (int m = 0; m < 8; ++m)                     // rows g + 8 m of the warp's 64
+                        next[m] = lc < l_chunks && (m >> 1) < mts ? p.Ls[(size_t)(row0 + ln.g + 8 * m) * per_row + (lc >> 1)] : __ushort_as_bfloat16(0);
+                };
+                scales((int)rank);
+                ask(2 * (int)rank + kk);
+                for (int lc = (int)rank; lc < l_chunks; lc += (int)C) {
+                    const int ls = 2 * lc + kk;
+                    ok = wait_words(v, call, [&] { ask(ls); }) && ok;
+                    uint4 tb[kNW];
+#pragma unroll
+                    for (int n = 0; n < kNW; ++n)
+                        tb[n] = pair_four_apart(make_uint4((uint32_t)v[4 * n], (uint32_t)v[4 * n + 1], (uint32_t)v[4 * n + 2], (uint32_t)v[4 * n + 3]));
+                    ask(ls + 2 * (int)C);
+                    float sc[8];
+#pragma unroll
+                    for (int m = 0; m < 8; ++m) sc[m] = __bfloat162float(next[m]);
+                    scales(lc + (int)C);
+                    const uint32_t stage = wait_stage();
+                    if (ls < l_steps && mts > 0)
+#pragma unroll
+                        for (int m = 0; m < 4; ++m) code_tile<kNW>(acc[m], l_codes(stage, rb, m, kk, ln), sc[2 * m], sc[2 * m + 1], tb);
+                    release();
                 }
             }
             // ---------------- partial tiles -> Y
@@ -1011,6 +1047,7 @@ slim_status_t launch_small(const __nv_bfloat16* X, int b, const uint8_t* vals, c
                               : make_map3(&tmR, R, (uint64_t)d_in, (uint64_t)r, kGroup));
     else tmR = tmX;
     if (r > 0 && !qa) ok = ok && make_map(&tmL, L, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (uint64_t)r, (uint64_t)d_out, 32, kRows, CU_TENSOR_MAP_SWIZZLE_64B);
+    else if (r > 0 && r % 32 == 0) ok = ok && make_map(&tmL, L, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)r / 2, (uint64_t)d_out, 32, kRows, CU_TENSOR_MAP_SWIZZLE_32B);
     else tmL = tmX;
     if (!ok) return SLIM_ERR_CUDA;
     cudaLaunchConfig_t cfg = {};
