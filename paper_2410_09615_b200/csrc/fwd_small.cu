@@ -1,13 +1,13 @@
 // Small-batch forward (b <= 64): one launch of thread-block clusters that streams the weight and the
 // adapters exactly once.
 //
-// Work split.  A tile is 256 output rows; the C CTAs of a cluster (C = 1, 2, 4 or 8) cut d_in into C
-// ranges of whole 256-column units.  In a CTA eight consumer warps are 4 row blocks of 64 rows x 2
-// halves of every unit: a warp keeps the fp32 accumulators of its 64 rows x b tokens in registers
+// Work split.  A tile is 256 output rows (up to 16 tokens of layers with fewer rows: 128 or 64); the C CTAs of a cluster
+// (C = 1, 2, 4 or 8) cut d_in into C ranges of whole 256-column units.  In a CTA eight consumer warps are 4 row blocks x 2
+// halves of every unit: a warp keeps the fp32 accumulators of its 64 (32, 16) rows x b tokens in registers
 // through the whole range (from 33 tokens on the two halves are token halves instead), so nothing is
-// summed across warps inside the stream; the partial tiles meet once, at the end, over distributed
-// shared memory.  C is the largest with which the clusters of all tiles are resident at once (two CTAs
-// per SM up to 16 tokens), so that a tile's stream is spread as widely as it can be.
+// summed across warps inside the stream; the partial tiles meet once, at the end: each CTA sends its own, a share of the
+// rows to every CTA of the cluster, by asynchronous remote stores.  C is the largest with which the clusters of all tiles are
+// resident at once (two CTAs per SM up to 16 tokens), so that a tile's stream is spread as widely as it can be.
 //   The first clusters make T = X R^T instead: 32 rows of R each, the same cut of d_in; their
 // CTAs exchange partial sums with asynchronous remote stores, round to bf16 and publish T as 8-byte words
 // {two columns, call number}.
@@ -51,12 +51,8 @@ constexpr int kCW = 8;                          // consumer warps
 constexpr int kConsumers = kCW * 32;
 constexpr int kProdW = kCW, kProdX = kCW + 1;   // requests of the weight, R and L; of the activations and the index bytes
 constexpr int kFetchT = kCW + 2;                // from 17 tokens on: two warps that bring T into shared memory
-constexpr int kRows = 256;                      // output rows of a tile
 constexpr int kUnit = 256;                      // columns of a stage
-constexpr int kValsBytes = kRows * 64, kMetaBytes = kRows * 32;
-constexpr int kWBytes = kValsBytes + kMetaBytes;   // 24 KB, = four 6144-byte pieces of the tiled copy
 constexpr int kGroup = 32;                      // rows of R in one piece of the T product
-constexpr int kRedPitch = 260;                  // floats per token of a partial tile (conflict-free writes)
 constexpr unsigned long long kWaitNs = 500ull * 1000 * 1000;
 
 enum { FMT_PACKED = 0, FMT_PACKED_LD = 1, FMT_TILED = 2 };   // LD: index bytes by cp.async (rows no 16-byte multiples)
@@ -74,22 +70,30 @@ struct SmallParams {
     int tiles, units, groups;                                 // of 256 rows, 256 columns, 32 rows of R
 };
 
-template <int NT> struct Cfg {
-    static constexpr int kTok = NT * 8;
+// NT tiles of 8 tokens; a warp's MT tiles of 16 rows (four warps: 64 MT rows of the layer).
+template <int NT, int MT> struct Cfg {
+    static constexpr int kTok = NT * 8, kRows = 64 * MT;
     static constexpr int kThreads = (kCW + (NT >= 4 ? 4 : 2)) * 32;
     static constexpr int kNW = NT < 4 ? NT : 4;               // n-tiles of a warp: with eight, two warps share the tokens of a row block
     static constexpr int kTSlots = NT == 8 ? 6 : 8, kTSlot = kTok * 64;        // steps of T in shared memory: 32 columns in bf16
+    static constexpr int kValsBytes = kRows * 64, kMetaBytes = kRows * 32;     // MT = 4: 24 KB, = four 6144-byte pieces of the tiled copy
+    static constexpr int kXOff = MT == 4 ? kValsBytes + kMetaBytes : 16384;    // a stage of R: 16 KB
     static constexpr int kXBytes = kTok * 512;                // activations of a unit
-    static constexpr int kStage = kWBytes + kXBytes;
-    static constexpr int kStages = NT == 4 ? 4 : 3;
+    static constexpr int kStage = kXOff + kXBytes;
+    static constexpr int kStages = NT == 4 || MT < 4 ? 4 : 3;
     static constexpr int kPiece = kTok * kGroup * 4;          // bytes of a piece of T
-    static constexpr int kOffPart = kStages * kStage;         // [4][kNW * 8][kGroup] floats, or the steps of T
-    static constexpr int kPartBytes = 4 * kNW * 8 * kGroup * 4 > (NT >= 4 ? kTSlots * kTSlot : 0) ? 4 * kNW * 8 * kGroup * 4 : kTSlots * kTSlot;
-    static constexpr int kOffRecv = kOffPart + kPartBytes;
-    static constexpr int kOffBars = kOffRecv + kPiece;
+    static constexpr int kPitch = kRows + 4;                  // floats per token of a partial tile (conflict-free writes)
+    static constexpr int kHalves = NT == 8 ? 1 : 2;
+    // after the ring: in the CTAs that make T, [4][kNW * 8][kGroup] floats and the piece as the cluster sends it; in the others,
+    // the steps of T, and the partial tiles that the cluster sends (eight n-tiles: these in the ring, when all CTAs are done with it)
+    static constexpr int kOffPart = kStages * kStage;
+    static constexpr int kOffRecv = kOffPart + 4 * kNW * 8 * kGroup * 4;
+    static constexpr int kOffY = NT == 8 ? 72 * 1024 : kOffPart + (NT >= 4 ? kTSlots * kTSlot : 0), kYBytes = kTok * kRows * 4;
+    static constexpr int kEndT = kOffRecv + kPiece, kEndY = NT == 8 ? kOffPart + kTSlots * kTSlot : kOffY + kYBytes;
+    static constexpr int kOffBars = kEndT > kEndY ? kEndT : kEndY;
     static constexpr int kSmem = kOffBars + 256;
     static constexpr int kCtasPerSm = NT <= 2 ? 2 : 1;
-    static_assert((NT == 8 ? 1 : 2) * kTok * kRedPitch * 4 <= kStages * kStage, "partial tiles do not fit the ring");
+    static_assert(kHalves * kTok * kPitch * 4 <= (NT == 8 ? kOffY : kOffPart) && (NT < 8 || kOffY + kYBytes <= kOffPart), "partial tiles do not fit the ring");
     static_assert(kSmem <= (NT <= 2 ? 113 : 227) * 1024, "shared memory");
 };
 
@@ -155,18 +159,18 @@ __device__ __forceinline__ void cp_async8(uint32_t dst, const void* src, bool in
 __device__ __forceinline__ void consumer_sync() { asm volatile("bar.sync 1, %0;" :: "n"(kConsumers) : "memory"); }
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
-__device__ __forceinline__ float4 ld_peer4(uint32_t addr) {
-    float4 v;
-    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr));
-    return v;
+// Eight or sixteen bytes into a peer's shared memory; its barrier counts them.
+__device__ __forceinline__ void st_peer4(uint32_t addr, float4 v, uint32_t bar) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];"
+                 :: "r"(addr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "r"(bar) : "memory");
 }
-// Eight bytes into a peer's shared memory; its barrier counts them.
 __device__ __forceinline__ void st_peer2(uint32_t addr, float x, float y, uint32_t bar) {
     asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];" :: "r"(addr), "f"(x), "f"(y), "r"(bar) : "memory");
 }
 __device__ __forceinline__ void sts_f(uint32_t addr, float v) { asm volatile("st.shared.f32 [%0], %1;" :: "r"(addr), "f"(v) : "memory"); }
 __device__ __forceinline__ void sts32(uint32_t addr, uint32_t v) { asm volatile("st.shared.u32 [%0], %1;" :: "r"(addr), "r"(v) : "memory"); }
 __device__ __forceinline__ float2 lds_f2(uint32_t addr) { float2 v; asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr)); return v; }
+__device__ __forceinline__ float4 lds_f4(uint32_t addr) { float4 v; asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr)); return v; }
 __device__ __forceinline__ uint2 lds64(uint32_t addr) {
     return *reinterpret_cast<const uint2*>(__cvta_shared_to_generic(addr));
 }
@@ -204,11 +208,12 @@ struct Lane { int lane, g, t; };
 // Rows past d_out and columns past d_in arrive as zero bytes.  Zero values are what they should be, but zero index
 // bits name one position twice: before a ragged stage is multiplied every lane completes the index words it will
 // read itself (0x4: positions 0 and 1).
+template <int MT>
 __device__ __forceinline__ void complete_index(uint32_t stage, int rb, int kk, int mts, int cols_left, const Lane& ln)
 {
     const int h = ln.t & 1, g = ln.g;
-    const uint32_t mrow = stage + kValsBytes + (uint32_t)(rb * 64 + g) * 32 + h * 8 + kk * 4, mx = (uint32_t)(g >> 2) & 1;
-    for (int i = 0; i < 8; ++i)                                   // rows g + 8 i; regions h and 2 + h
+    const uint32_t mrow = stage + MT * 4096 + (uint32_t)(rb * 16 * MT + g) * 32 + h * 8 + kk * 4, mx = (uint32_t)(g >> 2) & 1;
+    for (int i = 0; i < 2 * MT; ++i)                              // rows g + 8 i; regions h and 2 + h
 #pragma unroll
         for (int a = 0; a < 2; ++a)
             if ((i >> 1) >= mts || 64 * (2 * a + h) >= cols_left) sts32(mrow + i * 256 + (((uint32_t)a ^ mx) << 4), 0x44444444u);
@@ -216,21 +221,21 @@ __device__ __forceinline__ void complete_index(uint32_t stage, int rb, int kk, i
     __syncwarp();
 }
 
-// This warp's 64 rows x half a unit (four steps) of a packed-format stage, NB n-tiles from tile n0 on.
+// This warp's 16 MT rows x half a unit (four steps) of a packed-format stage, NB n-tiles from tile n0 on.
 // KS steps' activations are held at a time: four where the registers allow it, else two.
-template <int NT, int NB>
-__device__ __forceinline__ void weight_stage(float (&acc)[4][NB][4], uint32_t stage, int rb, int kk, int n0, const Lane& ln)
+template <int NT, int NB, int MT>
+__device__ __forceinline__ void weight_stage(float (&acc)[MT][NB][4], uint32_t stage, int rb, int kk, int n0, const Lane& ln)
 {
     constexpr int KS = NB <= 2 ? 4 : 2;
     const int a = ln.t >> 1, h = ln.t & 1, g = ln.g;
     // value bytes: 64-byte rows, 64-byte swizzle; index bytes: 32-byte rows, 32-byte swizzle
-    const uint32_t vrow = stage + (uint32_t)(rb * 64 + g) * 64 + kk * 8, vx = (uint32_t)(g >> 1) & 3;
+    const uint32_t vrow = stage + (uint32_t)(rb * 16 * MT + g) * 64 + kk * 8, vx = (uint32_t)(g >> 1) & 3;
     const uint32_t v0 = vrow + (((uint32_t)(2 * a) ^ vx) << 4), v1 = vrow + (((uint32_t)(2 * a + 1) ^ vx) << 4);
-    const uint32_t mrow = stage + kValsBytes + (uint32_t)(rb * 64 + g) * 32 + h * 8 + kk * 4, mx = (uint32_t)(g >> 2) & 1;
+    const uint32_t mrow = stage + MT * 4096 + (uint32_t)(rb * 16 * MT + g) * 32 + h * 8 + kk * 4, mx = (uint32_t)(g >> 2) & 1;
     const uint32_t m0 = mrow + (mx << 4), m1 = mrow + ((mx ^ 1) << 4);
     // activations: 64-column sub-tiles of 128-byte token rows, 128-byte swizzle; lane l addresses row l & 7 of matrix l / 8
     const int mat = ln.lane >> 3, tok = ln.lane & 7, q = 2 * (mat & 1) + (mat >> 1);
-    const uint32_t xrow = stage + kWBytes + (uint32_t)q * (NT * 1024) + (uint32_t)(n0 * 8 + tok) * 128;
+    const uint32_t xrow = stage + Cfg<NT, MT>::kXOff + (uint32_t)q * (NT * 1024) + (uint32_t)(n0 * 8 + tok) * 128;
     const uint32_t sel_e = 0x4400u + (uint32_t)h * 0x1111u, sel_o = sel_e + 0x2222u;     // byte h (+ 2) of w and of w >> 4
 #pragma unroll
     for (int s0 = 0; s0 < 4; s0 += KS) {
@@ -244,7 +249,7 @@ __device__ __forceinline__ void weight_stage(float (&acc)[4][NB][4], uint32_t st
         const uint32_t S = KS == 4 ? (uint32_t)a : (uint32_t)(s0 >> 1);
         const uint32_t msel = (2 * S) | ((4 + 2 * S) << 4) | ((2 * S + 1) << 8) | ((5 + 2 * S) << 12);
 #pragma unroll
-        for (int mt = 0; mt < 4; ++mt) {
+        for (int mt = 0; mt < MT; ++mt) {
             const uint32_t vo = mt * 1024, mo = mt * 512;
             uint32_t w[4][KS / 2];                            // (row g, h 0), (row g + 8, h 0), (row g, h 1), (row g + 8, h 1)
             if (KS == 4) {
@@ -281,7 +286,7 @@ template <int NT>
 __device__ __forceinline__ void weight_stage_tiled(float (&acc)[4][NT][4], uint32_t stage, int rb, int kk, const Lane& ln)
 {
     const int mat = ln.lane >> 3, tok = ln.lane & 7;
-    const uint32_t xrow = stage + kWBytes + (uint32_t)tok * 128;
+    const uint32_t xrow = stage + Cfg<NT, 4>::kXOff + (uint32_t)tok * 128;
     const uint32_t piece0 = stage + (uint32_t)rb * 6144;
     const uint32_t idx_lane = (uint32_t)(ln.g * 4 + 2 * kk + (ln.t & 1));       // the lane that holds this half's index words
 #pragma unroll
@@ -314,12 +319,12 @@ __device__ __forceinline__ void weight_stage_tiled(float (&acc)[4][NT][4], uint3
 
 // ---------------------------------------------------------------- one stage of R
 // 32 rows of R x 256 columns: warp = (16-row tile m, 64-column sub-tile kq).
-template <int NT>
+template <int NT, int MT>
 __device__ __forceinline__ void adapter_stage(float (&acc)[NT][4], uint32_t stage, int m, int kq, const Lane& ln)
 {
     const int mat = ln.lane >> 3, r8 = ln.lane & 7;
     const uint32_t arow = stage + (uint32_t)kq * 4096 + (uint32_t)(m * 16 + (mat & 1) * 8 + r8) * 128;
-    const uint32_t xrow = stage + kWBytes + (uint32_t)kq * (NT * 1024) + (uint32_t)r8 * 128;
+    const uint32_t xrow = stage + Cfg<NT, MT>::kXOff + (uint32_t)kq * (NT * 1024) + (uint32_t)r8 * 128;
 #pragma unroll
     for (int s = 0; s < 2; ++s) {                  // 32 columns
         uint4 a0, a1;
@@ -336,11 +341,11 @@ __device__ __forceinline__ void adapter_stage(float (&acc)[NT][4], uint32_t stag
 }
 // The same on int4 codes.  A word of a row is eight columns; the activations of a step are read as the thread's
 // own eight columns and paired four apart.  The 64 columns lie in one group: the integer products are scaled once.
-template <int NT>
+template <int NT, int MT>
 __device__ __forceinline__ void adapter_stage_q(float (&acc)[NT][4], uint32_t stage, int m, int kq, float sc0, float sc1, const Lane& ln)
 {
     const uint32_t arow = stage + (uint32_t)(m * 16 + ln.g) * 128 + ln.t * 4;
-    const uint32_t xrow = stage + kWBytes + (uint32_t)kq * (NT * 1024) + (uint32_t)ln.g * 128;
+    const uint32_t xrow = stage + Cfg<NT, MT>::kXOff + (uint32_t)kq * (NT * 1024) + (uint32_t)ln.g * 128;
     float part[NT][4];
 #pragma unroll
     for (int n = 0; n < NT; ++n)
@@ -374,36 +379,46 @@ __device__ __forceinline__ void ask_T(unsigned long long (&v)[NE], const unsigne
 #pragma unroll
     for (int n = 0; n < NE; ++n) v[n] = at[n] ? ld_gpu64(at[n]) : (unsigned long long)call << 32;
 }
-template <int NE, typename F>
-__device__ __forceinline__ bool wait_words(unsigned long long (&v)[NE], uint32_t call, F ask)
+// Where words are missing, one lane polls one of them, and all are asked for again when it has come: the tiles of a layer
+// wait for the same words, and with every lane polling its own (1024 warps on a few lines of the L2) the words
+// themselves came 1-3 us later (2048 -> 2048, rank 208, 6 tokens: 6.8 us a call instead of 7.5).
+template <int NE, typename A, typename W>
+__device__ __forceinline__ bool wait_words(unsigned long long (&v)[NE], uint32_t call, A ask, W word)
 {
-    unsigned long long t0 = 0;
-    for (uint32_t spin = 0;; ++spin) {
-        bool all = true;
+    for (int round = 0; round < 64; ++round) {
+        const unsigned long long* w = nullptr;
 #pragma unroll
-        for (int n = 0; n < NE; ++n) all = all && (uint32_t)(v[n] >> 32) == call;
-        if (__all_sync(0xffffffffu, all)) return true;
-        if ((spin & 63u) == 63u) {
-            const unsigned long long now = now_ns();
-            bool late = false;
-            if (t0 == 0) t0 = now;
-            else late = now - t0 > kWaitNs;
-            if (__any_sync(0xffffffffu, late)) return false;
+        for (int n = 0; n < NE; ++n) if (!w && (uint32_t)(v[n] >> 32) != call) w = word(n);
+        const uint32_t missing = __ballot_sync(0xffffffffu, w != nullptr);
+        if (!missing) return true;
+        bool late = false;
+        if ((int)(threadIdx.x & 31) == __ffs(missing) - 1) {
+            unsigned long long t0 = 0;
+            for (uint32_t spin = 0; !late && (uint32_t)(ld_gpu64(w) >> 32) != call; ++spin) {
+                if ((spin & 63u) == 63u) {
+                    const unsigned long long now = now_ns();
+                    if (t0 == 0) t0 = now;
+                    else late = now - t0 > kWaitNs;
+                }
+                __nanosleep(20);
+            }
         }
-        __nanosleep(40);
+        if (__any_sync(0xffffffffu, late)) return false;
         ask();
     }
+    return false;
 }
 template <int NE>
 __device__ __forceinline__ bool wait_T(unsigned long long (&v)[NE], const unsigned long long* const (&at)[NE], uint32_t call)
 {
-    return wait_words(v, call, [&] { ask_T<NE>(v, at, call); });
+    return wait_words(v, call, [&] { ask_T<NE>(v, at, call); }, [&](int n) { return at[n]; });
 }
 
 // The words of eight codes of rows g and g + 8 of a 16-row tile, step h of a stage of L's codes (32-byte rows, 32-byte
 // swizzle), and their product with T.  Integer products are scaled once.
+template <int MT>
 __device__ __forceinline__ uint2 l_codes(uint32_t stage, int rb, int m, int h, const Lane& ln) {
-    const uint32_t at = stage + (uint32_t)(rb * 64 + m * 16 + ln.g) * 32 + ((uint32_t)(h ^ (ln.g >> 2)) << 4) + ln.t * 4;
+    const uint32_t at = stage + (uint32_t)((rb * MT + m) * 16 + ln.g) * 32 + ((uint32_t)(h ^ (ln.g >> 2)) << 4) + ln.t * 4;
     return make_uint2(lds32(at), lds32(at + 256));
 }
 template <int NW>
@@ -422,53 +437,62 @@ __device__ __forceinline__ void code_tile(float (&acc)[NW][4], uint2 w, float sc
     }
 }
 
-// Y of the rows this CTA finishes, 256 / C of the tile: the 2 C (eight n-tiles: C) partial tiles in a fixed order, four
-// rows of a token at a time.
-template <int NT, int C>
-__device__ __forceinline__ void finish(const SmallParams& p, uint32_t smem, int tile, int rank)
+// The tile of a CTA, its two halves (eight n-tiles: one) added up, goes to the CTAs of the cluster, a share of the rows to
+// each: four rows of a token at a time, [sender][token][rows of the share].  (The CTAs reading the partial tiles out of each
+// other's shared memory, both halves, took 2 us longer for 16 tokens and 0.5 us for one.)
+template <int NT, int MT>
+__device__ __forceinline__ void send(const SmallParams& p, uint32_t smem, uint32_t red_full, int logC, int rank)
 {
-    constexpr int kHalves = NT == 8 ? 1 : 2, kQuads = kRows / C / 4;
-    constexpr int kUn = NT == 1 || NT < C ? 1 : NT / C;       // items in flight
-    const uint32_t half = (uint32_t)(NT * 8 * kRedPitch * 4);
-    for (int e0 = threadIdx.x; e0 < p.b * kQuads; e0 += kConsumers * kUn) {
-        float4 v[kUn][C][kHalves];
-#pragma unroll
-        for (int i = 0; i < kUn; ++i) {
-            const int e = min(e0 + i * kConsumers, p.b * kQuads - 1), tok = e / kQuads, row = rank * (kRows / C) + 4 * (e % kQuads);
-            const uint32_t at = smem + (uint32_t)(tok * kRedPitch + row) * 4;
-#pragma unroll
-            for (int c = 0; c < C; ++c)
-#pragma unroll
-                for (int h = 0; h < kHalves; ++h) v[i][c][h] = ld_peer4(peer(at + h * half, c));
+    using C_ = Cfg<NT, MT>;
+    constexpr int kQuads = C_::kRows / 4;
+    const int share = kQuads >> logC;
+    for (int e = threadIdx.x; e < p.b * kQuads; e += kConsumers) {
+        const int tok = e / kQuads, q = e % kQuads, owner = q / share;
+        const uint32_t at = smem + (uint32_t)(tok * C_::kPitch + 4 * q) * 4;
+        float4 v = lds_f4(at);
+        if (C_::kHalves == 2) {
+            const float4 w = lds_f4(at + C_::kTok * C_::kPitch * 4);
+            v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w;
         }
+        st_peer4(peer(smem + C_::kOffY + (uint32_t)((rank * p.b + tok) * share + (q & (share - 1))) * 16, owner), v, peer(red_full, owner));
+    }
+}
+// Y of the rows of this CTA's share: the senders' sums in a fixed order.
+template <int NT, int MT>
+__device__ __forceinline__ void finish(const SmallParams& p, uint32_t smem, int tile, int logC, int rank)
+{
+    using C_ = Cfg<NT, MT>;
+    const int share = (C_::kRows / 4) >> logC, items = p.b * share, C = 1 << logC;
+    for (int e = threadIdx.x; e < items; e += kConsumers) {
+        const uint32_t at = smem + C_::kOffY + (uint32_t)e * 16;
+        float4 v[8];
 #pragma unroll
-        for (int i = 0; i < kUn; ++i) {
-            const int e = e0 + i * kConsumers, tok = e / kQuads, n = tile * kRows + rank * (kRows / C) + 4 * (e % kQuads);
-            if (e < p.b * kQuads && n < p.d_out) {
-                float4 y = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int c = 0; c < 8; ++c) if (c < C) v[c] = lds_f4(at + (uint32_t)(c * items) * 16);
+        float4 y = v[0];
 #pragma unroll
-                for (int c = 0; c < C; ++c)
-#pragma unroll
-                    for (int h = 0; h < kHalves; ++h) { y.x += v[i][c][h].x; y.y += v[i][c][h].y; y.z += v[i][c][h].z; y.w += v[i][c][h].w; }
-                __nv_bfloat162 lo = __floats2bfloat162_rn(y.x, y.y), hi = __floats2bfloat162_rn(y.z, y.w);
-                *reinterpret_cast<uint2*>(p.Y + (size_t)tok * p.d_out + n) = make_uint2(*reinterpret_cast<uint32_t*>(&lo), *reinterpret_cast<uint32_t*>(&hi));
-            }
+        for (int c = 1; c < 8; ++c) if (c < C) { y.x += v[c].x; y.y += v[c].y; y.z += v[c].z; y.w += v[c].w; }
+        const int tok = e / share, n = tile * C_::kRows + 4 * (rank * share + (e & (share - 1)));
+        if (n < p.d_out) {
+            __nv_bfloat162 lo = __floats2bfloat162_rn(y.x, y.y), hi = __floats2bfloat162_rn(y.z, y.w);
+            *reinterpret_cast<uint2*>(p.Y + (size_t)tok * p.d_out + n) = make_uint2(*reinterpret_cast<uint32_t*>(&lo), *reinterpret_cast<uint32_t*>(&hi));
         }
     }
 }
 
 // ---------------------------------------------------------------- the kernel
-template <int NT, int FMT, bool QA>
-__global__ void __launch_bounds__(Cfg<NT>::kThreads, Cfg<NT>::kCtasPerSm)
+template <int NT, int FMT, bool QA, int MT>
+__global__ void __launch_bounds__(Cfg<NT, MT>::kThreads, Cfg<NT, MT>::kCtasPerSm)
 small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmM,
              const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmR, const __grid_constant__ CUtensorMap tmL)
 {
-    using C_ = Cfg<NT>;
-    constexpr int kTok = C_::kTok, kNW = C_::kNW, kStages = C_::kStages, kStage = C_::kStage;
+    using C_ = Cfg<NT, MT>;
+    static_assert(MT == 4 || (NT <= 2 && FMT != FMT_TILED), "narrow tiles: up to 16 tokens, packed format");
+    constexpr int kTok = C_::kTok, kNW = C_::kNW, kStages = C_::kStages, kStage = C_::kStage, kRows = C_::kRows;
+    constexpr int kValsBytes = C_::kValsBytes, kMetaBytes = C_::kMetaBytes, kXOff = C_::kXOff;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     const uint32_t smem = smem_u32(smem_raw);
     const uint32_t part = smem + C_::kOffPart, recv = smem + C_::kOffRecv, bars = smem + C_::kOffBars;
-    const uint32_t full = bars, empty = bars + 32, piece_bar = bars + 64, red_full = bars + 72, t_full = bars + 80, t_empty = bars + 144;
+    const uint32_t full = bars, empty = bars + 32, piece_bar = bars + 64, red_full = bars + 72, t_full = bars + 80, t_empty = bars + 144, gone = bars + 208;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     Lane ln; ln.lane = lane; ln.g = lane >> 2; ln.t = lane & 3;
@@ -487,11 +511,13 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
     if (threadIdx.x == 0) {
         // a stage's barrier counts both producers (and, with index bytes by cp.async, the lanes of one of them)
         for (int i = 0; i < kStages; ++i) { mbar_init(full + 8 * i, FMT == FMT_PACKED_LD ? 34 : 2); mbar_init(empty + 8 * i, kCW); }
-        mbar_init(piece_bar, 1); mbar_init(red_full, C);
+        mbar_init(piece_bar, 1); mbar_init(red_full, 1); mbar_init(gone, C);
         if (NT >= 4) for (int i = 0; i < C_::kTSlots; ++i) { mbar_init(t_full + 8 * i, 2); mbar_init(t_empty + 8 * i, kCW); }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         // every CTA of the cluster sends this one its share of the piece: 16 / C column pairs per token
         mbar_expect(piece_bar, (uint32_t)p.b * 16 * 8);
+        // and its share of the rows of the tile, four bytes per token and row
+        mbar_expect(red_full, (uint32_t)p.b * kRows * 4);
     }
     __syncthreads();
     cluster_arrive();                                          // waited for before the first access to a peer
@@ -577,7 +603,7 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
                 const uint32_t bar = full + 8 * st;
                 if (lane == 0) {
                     mbar_expect(bar, C_::kXBytes);
-                    tma_tile3(smem + st * kStage + kWBytes, &tmX, 0, u * 4, bar);
+                    tma_tile3(smem + st * kStage + kXOff, &tmX, 0, u * 4, bar);
                 }
                 if (FMT == FMT_PACKED_LD) mbar_arrive(bar);
             }
@@ -604,7 +630,7 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
                 const uint32_t dst = smem + st * kStage, bar = full + 8 * st;
                 if (lane == 0) mbar_expect(bar, C_::kXBytes + (FMT == FMT_PACKED ? kMetaBytes : 0));
                 __syncwarp();
-                if (lane == 0) tma_tile3(dst + kWBytes, &tmX, 0, u * 4, bar);
+                if (lane == 0) tma_tile3(dst + kXOff, &tmX, 0, u * 4, bar);
                 if (FMT == FMT_PACKED && lane == 1) tma_tile(dst + kValsBytes, &tmM, u * 32, row0, bar);
                 if (FMT == FMT_PACKED_LD) {
                     // 256 rows x four 8-byte pieces (64 columns), stored as the TMA's 32-byte swizzle would
@@ -690,8 +716,8 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
                 }
                 const uint32_t stage = wait_stage();
                 if (valid) {
-                    if (QA) adapter_stage_q<NT>(acc, stage, m, kq, sc0, sc1, ln);
-                    else adapter_stage<NT>(acc, stage, m, kq, ln);
+                    if (QA) adapter_stage_q<NT, MT>(acc, stage, m, kq, sc0, sc1, ln);
+                    else adapter_stage<NT, MT>(acc, stage, m, kq, ln);
                 }
                 release();
             }
@@ -727,15 +753,16 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
         } else {
             const int rb = warp & 3, kk = warp >> 2;
             const int n_first = NT == 8 ? 4 * kk : 0;           // with eight n-tiles kk picks tokens, not columns
-            const int row0 = tile * kRows + rb * 64;
-            const int mts = max(0, min(4, (p.d_out - row0) / 16));          // valid 16-row tiles of this warp
-            float acc[4][kNW][4];
+            const int row0 = tile * kRows + rb * 16 * MT;
+            const int mts = max(0, min(MT, (p.d_out - row0) / 16));         // valid 16-row tiles of this warp
+            float acc[MT][kNW][4];
 #pragma unroll
-            for (int m = 0; m < 4; ++m)
+            for (int m = 0; m < MT; ++m)
 #pragma unroll
                 for (int n = 0; n < kNW; ++n)
 #pragma unroll
                     for (int e = 0; e < 4; ++e) acc[m][n][e] = 0.f;
+            cluster_wait();                                    // every CTA has started (they all have by the time the first stage arrives)
             // ---------------- the weight
             for (int u = u0; u < u_end; ++u) {
                 const uint32_t stage = wait_stage();
@@ -746,18 +773,18 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
                     } else if constexpr (NT == 8) {
 #pragma unroll 1
                         for (int h = 0; h < 2; ++h) {
-                            if (mts < 4 || left < kUnit) complete_index(stage, rb, h, mts, left, ln);
-                            weight_stage<NT, kNW>(acc, stage, rb, h, n_first, ln);
+                            if (mts < MT || left < kUnit) complete_index<MT>(stage, rb, h, mts, left, ln);
+                            weight_stage<NT, kNW, MT>(acc, stage, rb, h, n_first, ln);
                         }
                     } else {
-                        if (mts < 4 || left < kUnit) complete_index(stage, rb, kk, mts, left, ln);
-                        weight_stage<NT, kNW>(acc, stage, rb, kk, 0, ln);
+                        if (mts < MT || left < kUnit) complete_index<MT>(stage, rb, kk, mts, left, ln);
+                        weight_stage<NT, kNW, MT>(acc, stage, rb, kk, 0, ln);
                     }
                 }
                 release();
             }
 #pragma unroll
-            for (int m = 0; m < 4; ++m)
+            for (int m = 0; m < MT; ++m)
 #pragma unroll
                 for (int n = 0; n < kNW; ++n)
 #pragma unroll
@@ -786,7 +813,7 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
                                     tb[n] = pair_four_apart(lds128(tslot + ((n_first + n) * 8 + ln.g) * 64 + ((ln.t ^ ((ln.g >> 1) & 3)) << 4)));
 #pragma unroll
                                 for (int m = 0; m < 4; ++m)
-                                    if (NT == 8 || (m >> 1) == kk) code_tile<kNW>(acc[m], l_codes(stage, rb, m, h, ln), sc[2 * m], sc[2 * m + 1], tb);
+                                    if (NT == 8 || (m >> 1) == kk) code_tile<kNW>(acc[m], l_codes<MT>(stage, rb, m, h, ln), sc[2 * m], sc[2 * m + 1], tb);
                             }
                             __syncwarp();
                             if (lane == 0) mbar_arrive(t_empty + 8 * ts);
@@ -850,9 +877,9 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
                     const uint32_t stage = wait_stage();
                     if (ls * 32 + 16 * kk < p.r && mts > 0) {
 #pragma unroll
-                        for (int m = 0; m < 4; ++m) {
+                        for (int m = 0; m < MT; ++m) {
                             uint4 a;                                // 64-byte rows, 64-byte swizzle
-                            const int row = rb * 64 + m * 16 + (mat & 1) * 8 + r8;
+                            const int row = (rb * MT + m) * 16 + (mat & 1) * 8 + r8;
                             ldsm4(stage + row * 64 + ((uint32_t)((2 * kk + (mat >> 1)) ^ ((r8 >> 1) & 3)) << 4), a);
 #pragma unroll
                             for (int n = 0; n < kNW; ++n) mma_16816(acc[m][n], a.x, a.y, a.z, a.w, tb[2 * n], tb[2 * n + 1]);
@@ -863,7 +890,7 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
             } else {
                 // codes: kk picks the step of a stage of 64; scales and words of T are asked for one stage ahead
                 const uint32_t per_row = (uint32_t)((p.r + 127) >> 7);
-                __nv_bfloat16 next[8];
+                __nv_bfloat16 next[2 * MT];
                 unsigned long long v[4 * kNW];
                 const unsigned long long* at = p.T + (size_t)ln.g * (p.r / 2) + 4 * ln.t;
                 auto ask = [&](int ls) {
@@ -879,47 +906,47 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
                 };
                 auto scales = [&](int lc) {
 #pragma unroll
-                    for (int m = 0; m < 8; ++m)                     // rows g + 8 m of the warp's 64
+                    for (int m = 0; m < 2 * MT; ++m)                     // rows g + 8 m of the warp's
                         next[m] = lc < l_chunks && (m >> 1) < mts ? p.Ls[(size_t)(row0 + ln.g + 8 * m) * per_row + (lc >> 1)] : __ushort_as_bfloat16(0);
                 };
                 scales((int)rank);
                 ask(2 * (int)rank + kk);
                 for (int lc = (int)rank; lc < l_chunks; lc += (int)C) {
                     const int ls = 2 * lc + kk;
-                    ok = wait_words(v, call, [&] { ask(ls); }) && ok;
+                    ok = wait_words(v, call, [&] { ask(ls); }, [&](int n) { return at + (n >> 2) * 4 * p.r + 16 * ls + (n & 3); }) && ok;
                     uint4 tb[kNW];
 #pragma unroll
                     for (int n = 0; n < kNW; ++n)
                         tb[n] = pair_four_apart(make_uint4((uint32_t)v[4 * n], (uint32_t)v[4 * n + 1], (uint32_t)v[4 * n + 2], (uint32_t)v[4 * n + 3]));
                     ask(ls + 2 * (int)C);
-                    float sc[8];
+                    float sc[2 * MT];
 #pragma unroll
-                    for (int m = 0; m < 8; ++m) sc[m] = __bfloat162float(next[m]);
+                    for (int m = 0; m < 2 * MT; ++m) sc[m] = __bfloat162float(next[m]);
                     scales(lc + (int)C);
                     const uint32_t stage = wait_stage();
                     if (ls < l_steps && mts > 0)
 #pragma unroll
-                        for (int m = 0; m < 4; ++m) code_tile<kNW>(acc[m], l_codes(stage, rb, m, kk, ln), sc[2 * m], sc[2 * m + 1], tb);
+                        for (int m = 0; m < MT; ++m) code_tile<kNW>(acc[m], l_codes<MT>(stage, rb, m, kk, ln), sc[2 * m], sc[2 * m + 1], tb);
                     release();
                 }
             }
             // ---------------- partial tiles -> Y
             consumer_sync();                                   // every warp is done with the ring
 #pragma unroll
-            for (int m = 0; m < 4; ++m)
+            for (int m = 0; m < MT; ++m)
 #pragma unroll
                 for (int n = 0; n < kNW; ++n)
 #pragma unroll
                     for (int e = 0; e < 4; ++e)
-                        sts_f(smem + (uint32_t)(((NT == 8 ? 0 : kk * kTok) + (n_first + n) * 8 + 2 * ln.t + (e & 1)) * kRedPitch + rb * 64 + m * 16 + ln.g + 8 * (e >> 1)) * 4, acc[m][n][e]);
+                        sts_f(smem + (uint32_t)(((NT == 8 ? 0 : kk * kTok) + (n_first + n) * 8 + 2 * ln.t + (e & 1)) * C_::kPitch + (rb * MT + m) * 16 + ln.g + 8 * (e >> 1)) * 4, acc[m][n][e]);
             consumer_sync();
-            cluster_wait();
-            if (warp == 0 && lane < (int)C) mbar_arrive_peer(peer(red_full, lane));
+            if (NT == 8) {                                     // the receivers' ring is free
+                if (warp == 0 && lane < (int)C) mbar_arrive_peer(peer(gone, lane));
+                ok = mbar_wait<true>(gone, 0) && ok;
+            }
+            send<NT, MT>(p, smem, red_full, logC, (int)rank);
             ok = mbar_wait<true>(red_full, 0) && ok;
-            if (logC == 3) finish<NT, 8>(p, smem, tile, (int)rank);
-            else if (logC == 2) finish<NT, 4>(p, smem, tile, (int)rank);
-            else if (logC == 1) finish<NT, 2>(p, smem, tile, (int)rank);
-            else finish<NT, 1>(p, smem, tile, (int)rank);
+            finish<NT, MT>(p, smem, tile, logC, (int)rank);
         }
     }
     if (!ok && lane == 0) flag_error(p.status, SLIM_ERR_TIMEOUT);
@@ -933,33 +960,39 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
 // ------------------------------------------------------------------ host side
 using KernelFn = void (*)(const SmallParams, const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap);
 
-template <int NT, int FMT> KernelFn pick_q(bool qa) { return qa ? small_kernel<NT, FMT, true> : small_kernel<NT, FMT, false>; }
-KernelFn pick(int nt, int fmt, bool qa) {
-    if (fmt == FMT_TILED) return nt == 1 ? small_kernel<1, FMT_TILED, false> : small_kernel<2, FMT_TILED, false>;
-    if (fmt == FMT_PACKED)
-        return nt == 1 ? pick_q<1, FMT_PACKED>(qa) : nt == 2 ? pick_q<2, FMT_PACKED>(qa) : nt == 4 ? pick_q<4, FMT_PACKED>(qa) : pick_q<8, FMT_PACKED>(qa);
-    return nt == 1 ? pick_q<1, FMT_PACKED_LD>(qa) : nt == 2 ? pick_q<2, FMT_PACKED_LD>(qa) : nt == 4 ? pick_q<4, FMT_PACKED_LD>(qa) : pick_q<8, FMT_PACKED_LD>(qa);
+template <int NT, int FMT, int MT> KernelFn pick_q(bool qa) { return qa ? small_kernel<NT, FMT, true, MT> : small_kernel<NT, FMT, false, MT>; }
+template <int NT, int FMT> KernelFn pick_m(int mt, bool qa) { return mt == 1 ? pick_q<NT, FMT, 1>(qa) : mt == 2 ? pick_q<NT, FMT, 2>(qa) : pick_q<NT, FMT, 4>(qa); }
+template <int FMT> KernelFn pick_n(int nt, int mt, bool qa) {
+    return nt == 1 ? pick_m<1, FMT>(mt, qa) : nt == 2 ? pick_m<2, FMT>(mt, qa) : nt == 4 ? pick_q<4, FMT, 4>(qa) : pick_q<8, FMT, 4>(qa);
 }
-int smem_bytes(int nt) { return nt == 1 ? Cfg<1>::kSmem : nt == 2 ? Cfg<2>::kSmem : nt == 4 ? Cfg<4>::kSmem : Cfg<8>::kSmem; }
-int threads_of(int nt) { return nt >= 4 ? Cfg<4>::kThreads : Cfg<1>::kThreads; }
+KernelFn pick(int nt, int fmt, bool qa, int mt) {
+    if (fmt == FMT_TILED) return nt == 1 ? small_kernel<1, FMT_TILED, false, 4> : small_kernel<2, FMT_TILED, false, 4>;
+    return fmt == FMT_PACKED ? pick_n<FMT_PACKED>(nt, mt, qa) : pick_n<FMT_PACKED_LD>(nt, mt, qa);
+}
+int smem_bytes(int nt, int mt) {
+    if (mt == 1) return nt == 1 ? Cfg<1, 1>::kSmem : Cfg<2, 1>::kSmem;
+    if (mt == 2) return nt == 1 ? Cfg<1, 2>::kSmem : Cfg<2, 2>::kSmem;
+    return nt == 1 ? Cfg<1, 4>::kSmem : nt == 2 ? Cfg<2, 4>::kSmem : nt == 4 ? Cfg<4, 4>::kSmem : Cfg<8, 4>::kSmem;
+}
+int threads_of(int nt) { return nt >= 4 ? Cfg<4, 4>::kThreads : Cfg<1, 4>::kThreads; }
 int tiles_of(int b) { return b <= 8 ? 1 : b <= 16 ? 2 : b <= 32 ? 4 : 8; }
 
 // Clusters of 1, 2, 4, 8 CTAs of one kernel that the device holds at once; asked once per device and kernel.
 struct Residency { std::atomic<int> ready{0}; int clusters[4]; };
-Residency g_res[64][4][3][2];
+Residency g_res[64][4][3][2][3];
 std::mutex g_res_mutex;
 
-const int* residency(int dev, int nt, int fmt, bool qa) {
+const int* residency(int dev, int nt, int fmt, bool qa, int mt) {
     const int ni = nt == 1 ? 0 : nt == 2 ? 1 : nt == 4 ? 2 : 3;
-    Residency& rs = g_res[dev][ni][fmt][qa ? 1 : 0];
+    Residency& rs = g_res[dev][ni][fmt][qa ? 1 : 0][mt >> 1];
     if (rs.ready.load(std::memory_order_acquire)) return rs.clusters;
     std::lock_guard<std::mutex> lock(g_res_mutex);
     if (rs.ready.load(std::memory_order_relaxed)) return rs.clusters;
-    const void* fn = (const void*)pick(nt, fmt, qa);
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes(nt)) != cudaSuccess) return nullptr;
+    const void* fn = (const void*)pick(nt, fmt, qa, mt);
+    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes(nt, mt)) != cudaSuccess) return nullptr;
     for (int i = 0; i < 4; ++i) {
         cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(1u << i); cfg.blockDim = dim3(threads_of(nt)); cfg.dynamicSmemBytes = smem_bytes(nt);
+        cfg.gridDim = dim3(1u << i); cfg.blockDim = dim3(threads_of(nt)); cfg.dynamicSmemBytes = smem_bytes(nt, mt);
         cudaLaunchAttribute a[1];
         a[0].id = cudaLaunchAttributeClusterDimension;
         a[0].val.clusterDim.x = 1u << i; a[0].val.clusterDim.y = 1; a[0].val.clusterDim.z = 1;
@@ -1008,13 +1041,33 @@ int cluster_size(const int* res, int tiles, int units) {
     return 1;
 }
 
+// Up to 16 tokens, tiles of 128 rows where all clusters (tiles, and pieces of T) of four CTAs are then resident at once.  They
+// have eight CTAs if there is no more than one CTA per SM even so: the words of T take 1-2 us longer to reach tiles that
+// share their SMs with others and are done with the weight before T is there (2048 -> 2048, rank 208, 6 tokens:
+// 23 clusters of four 4.8 us, of eight 6.8).  Tiles of 64 rows pay without adapters (4096 x 4096, 16 tokens: 5.1 us against 5.9)
+// and for long rows that leave a CTA of a 128-row tile eight stages or more (8192 -> 3584, rank 368, 16 tokens: 9.9 us
+// against 12.5), else not (4096 x 4096, rank 208: 9.1 us against 8.3).  With 256-row tiles only: 8192 -> 1024, rank 112, 16
+// tokens 9.3 us instead of 6.6; 5120 x 5120, rank 512, 8 tokens 11.1 instead of 8.6; larger layers are better off with them
+// (28672 -> 8192, 16 tokens 48 us against 65).
+void narrow_tiles(int dev, int nt, int fmt, bool qa, int sm_count, int d_out, int units, int groups, int* mt, int* C) {
+    auto fits = [&](int m) {
+        const int* res = residency(dev, nt, fmt, qa, m);
+        return res && ceil_div(d_out, 64 * m) + groups <= res[2];
+    };
+    if (!fits(2)) return;
+    const bool spread = 8 * (ceil_div(d_out, 128) + groups) <= sm_count;
+    *mt = fits(1) && (groups == 0 || (!spread && units >= 32)) ? 1 : 2;
+    const int widest = 8 * (ceil_div(d_out, 64 * *mt) + groups) <= sm_count ? 8 : 4;
+    for (*C = widest; *C > units; *C /= 2) {}
+}
+
 }  // namespace
 
 // Limits of the kernel: the region of the workspace that T lives in (and r <= 3072), and the call counter, which
 // takes 65536 CTAs.
 bool small_supports(int b, int d_out, int d_in, int r) {
     return b >= 1 && b <= 64 && d_out >= 16 && d_out % 16 == 0 && d_in >= 64 && d_in % 64 == 0 && r >= 0 && r % 16 == 0 &&
-           r <= kSmallMaxRank && (size_t)b * r * 4 <= kSmallTBytes && ceil_div(d_out, kRows) < 32768;
+           r <= kSmallMaxRank && (size_t)b * r * 4 <= kSmallTBytes && ceil_div(d_out, 256) < 32768;
 }
 
 slim_status_t launch_small(const __nv_bfloat16* X, int b, const uint8_t* vals, const uint8_t* meta, const uint8_t* tiled, float s,
@@ -1022,43 +1075,48 @@ slim_status_t launch_small(const __nv_bfloat16* X, int b, const uint8_t* vals, c
                            __nv_bfloat16* Y, void* ws, uint32_t* status_dev, cudaStream_t st)
 {
     slim_status_t err;
-    if (!device_info(&err)) return err;
+    const DeviceInfo* di = device_info(&err);
+    if (!di) return err;
     if (!small_supports(b, d_out, d_in, r) || (tiled && (b > 16 || d_in % 256 != 0 || Ls))) return SLIM_ERR_UNSUPPORTED_SHAPE;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return SLIM_ERR_CUDA;
     const int nt = tiles_of(b), fmt = tiled ? FMT_TILED : d_in % 128 == 0 ? FMT_PACKED : FMT_PACKED_LD;
     const bool qa = Ls != nullptr;
-    const int* res = residency(dev, nt, fmt, qa);
+    const int units = ceil_div(d_in, kUnit), groups = ceil_div(r, kGroup);
+    int mt = 4, C = 0;
+    if (nt <= 2 && !tiled) narrow_tiles(dev, nt, fmt, qa, di->sm_count, d_out, units, groups, &mt, &C);
+    const int rows = 64 * mt;
+    const int* res = residency(dev, nt, fmt, qa, mt);
     if (!res) return SLIM_ERR_CUDA;
+    if (mt == 4) C = cluster_size(res, ceil_div(d_out, rows), units);
     SmallParams p;
     p.X = X; p.meta = meta; p.tiled = tiled; p.L = L; p.R = R; p.Ls = Ls; p.Rs = Rs; p.Y = Y;
     p.departures = reinterpret_cast<unsigned long long*>(ws);
     p.T = reinterpret_cast<unsigned long long*>(reinterpret_cast<char*>(ws) + SLIM_WORKSPACE_SYNC_BYTES);
     p.status = status_dev; p.s = s; p.b = b; p.r = r; p.d_out = d_out; p.d_in = d_in;
-    p.tiles = ceil_div(d_out, kRows); p.units = ceil_div(d_in, kUnit); p.groups = ceil_div(r, kGroup);
-    const int C = cluster_size(res, p.tiles, p.units);
+    p.tiles = ceil_div(d_out, rows); p.units = units; p.groups = groups;
     CUtensorMap tmV, tmM, tmX, tmR, tmL;
     bool ok = make_map3(&tmX, X, (uint64_t)d_in, (uint64_t)b, nt * 8);
-    if (!tiled) ok = ok && make_map(&tmV, vals, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)d_in / 4, (uint64_t)d_out, 64, kRows, CU_TENSOR_MAP_SWIZZLE_64B);
+    if (!tiled) ok = ok && make_map(&tmV, vals, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)d_in / 4, (uint64_t)d_out, 64, rows, CU_TENSOR_MAP_SWIZZLE_64B);
     else tmV = tmX;
-    if (fmt == FMT_PACKED) ok = ok && make_map(&tmM, meta, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)d_in / 8, (uint64_t)d_out, 32, kRows, CU_TENSOR_MAP_SWIZZLE_32B);
+    if (fmt == FMT_PACKED) ok = ok && make_map(&tmM, meta, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)d_in / 8, (uint64_t)d_out, 32, rows, CU_TENSOR_MAP_SWIZZLE_32B);
     else tmM = tmX;
     if (r > 0) ok = ok && (qa ? make_map(&tmR, R, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)d_in / 2, (uint64_t)r, 128, kGroup, CU_TENSOR_MAP_SWIZZLE_128B)
                               : make_map3(&tmR, R, (uint64_t)d_in, (uint64_t)r, kGroup));
     else tmR = tmX;
-    if (r > 0 && !qa) ok = ok && make_map(&tmL, L, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (uint64_t)r, (uint64_t)d_out, 32, kRows, CU_TENSOR_MAP_SWIZZLE_64B);
-    else if (r > 0 && r % 32 == 0) ok = ok && make_map(&tmL, L, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)r / 2, (uint64_t)d_out, 32, kRows, CU_TENSOR_MAP_SWIZZLE_32B);
+    if (r > 0 && !qa) ok = ok && make_map(&tmL, L, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (uint64_t)r, (uint64_t)d_out, 32, rows, CU_TENSOR_MAP_SWIZZLE_64B);
+    else if (r > 0 && r % 32 == 0) ok = ok && make_map(&tmL, L, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)r / 2, (uint64_t)d_out, 32, rows, CU_TENSOR_MAP_SWIZZLE_32B);
     else tmL = tmX;
     if (!ok) return SLIM_ERR_CUDA;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(C * (p.tiles + p.groups))); cfg.blockDim = dim3(threads_of(nt)); cfg.dynamicSmemBytes = smem_bytes(nt); cfg.stream = st;
+    cfg.gridDim = dim3((unsigned)(C * (p.tiles + p.groups))); cfg.blockDim = dim3(threads_of(nt)); cfg.dynamicSmemBytes = smem_bytes(nt, mt); cfg.stream = st;
     cudaLaunchAttribute a[2];
     a[0].id = cudaLaunchAttributeClusterDimension;
     a[0].val.clusterDim.x = (unsigned)C; a[0].val.clusterDim.y = 1; a[0].val.clusterDim.z = 1;
     a[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     a[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = a; cfg.numAttrs = 2;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, pick(nt, fmt, qa), p, tmV, tmM, tmX, tmR, tmL);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, pick(nt, fmt, qa, mt), p, tmV, tmM, tmX, tmR, tmL);
     count_launch(1);
     return e == cudaSuccess ? SLIM_OK : SLIM_ERR_CUDA;
 }
