@@ -94,21 +94,46 @@ qs_hist_kernel(const float* __restrict__ W, size_t n, const QsHeader* hdr, int b
 //   - While the sum e stays in one binade [2^k, 2^(k+1)), whose spacing is u, adding t >= 0 gives e + q with q = t
 //     rounded to a multiple of u, unless t lies exactly half-way between two multiples (then the parity of e
 //     decides).  The q of many bins can be found side by side and added in any order: all are multiples of u
-//     and the sums stay below 2^53 u, so every addition is exact.  A warp takes 256 bins at a time, eight a lane, and
-//     goes through a lane's bins one by one only where e leaves its binade or a half-way case comes up.
+//     and the sums stay below 2^53 u, so every addition is exact.  Sixteen warps work out the terms of a block of 256 bins
+//     each; a lane guesses from an ordinary sum of the terms before it which binade e will be in at its eight bins, and
+//     adds up their q.  Lanes where e seems to leave its binade, or that hold a half-way case, are "crossings": between them
+//     the warp adds up the lanes' sums.  Then e walks over the blocks: a segment's sum, a crossing's eight terms one by one, and
+//     so on; where a guess proves wrong, the block is gone through by parts (add_block).
 //   - The fine candidates depend on the best coarse one only through ten possible values: all 10 + 10 x 19
 //     candidates are evaluated at once, a block each, and the last block to finish takes the minima.
-constexpr int kSearchThreads = 512, kSlice = 2048, kCoarse = 10, kFine = 19, kCandidates = kCoarse + kCoarse * kFine;
+// Bound by the FP64 operations of the terms and by the chain of the first blocks, where e leaves a binade every few bins.
+// 20000 bins: 400 us with a warp per candidate and the bins in sequence, 54 with one adding warp per candidate that every
+// block of bins passed through, now 38.
+constexpr int kSearchWarps = 16, kSearchThreads = 32 * kSearchWarps, kCoarse = 10, kFine = 19, kCandidates = kCoarse + kCoarse * kFine;
+
+// x / b correctly rounded in binary64, for many x and one b: as Divisor does it in binary32.
+struct Divisor64 {
+    double b, y;
+    bool plain;
+    __device__ __forceinline__ explicit Divisor64(double d) : b(d) {
+        y = __drcp_rn(d);
+        const unsigned long long bits = (unsigned long long)__double_as_longlong(d);
+        plain = (bits & 0xFFFFFFFFFFFFFull) == 0xFFFFFFFFFFFFFull || !(d >= 0x1p-300 && d <= 0x1p300);
+    }
+    __device__ __forceinline__ double of(double x) const {
+        if (plain) return __ddiv_rn(x, b);
+        double q = __dmul_rn(x, y);
+        q = __fma_rn(__fma_rn(-q, b, x), y, q);
+        return __fma_rn(__fma_rn(-q, b, x), y, q);
+    }
+};
 
 // One bin's term: every operation rounded on its own; an empty bin adds +0, which changes nothing.
-__device__ __forceinline__ double qs_term(unsigned int c, int i, double width, double n_total, double alpha)
+__device__ __forceinline__ double qs_term(unsigned int c, int i, double width, const Divisor64& by_n, const Divisor64& by_alpha)
 {
     if (!c) return 0.0;
-    const double x = __dmul_rn(__dadd_rn((double)i, 0.5), width);
-    const double p = __ddiv_rn((double)c, n_total);
+    // i + 1/2 and c as binary64 (2^52 + i and 2^52 + c less 2^52, exact), and below the nearest integer of a number up to 8:
+    // one or two additions each instead of conversions, which have a quarter of the rate
+    const double alpha = by_alpha.b, x = __dmul_rn(__dadd_rn(__hiloint2double(0x43300000, i), -(0x1p52 - 0.5)), width);
+    const double p = by_n.of(__dadd_rn(__hiloint2double(0x43300000, (int)c), -0x1p52));
     double d;
     if (x <= alpha) {
-        const double level = rint(__ddiv_rn(__dmul_rn(x, 8.0), alpha));
+        const double level = __dadd_rn(__dadd_rn(by_alpha.of(__dmul_rn(x, 8.0)), 0x1.8p52), -0x1.8p52);
         d = __dsub_rn(__dmul_rn(__dmul_rn(alpha, 0.125), level), x);
     } else {
         d = __dsub_rn(alpha, x);
@@ -116,12 +141,14 @@ __device__ __forceinline__ double qs_term(unsigned int c, int i, double width, d
     return __dmul_rn(p, __dmul_rn(d, d));
 }
 
+__device__ __forceinline__ int exponent(double e) { return (int)((__double_as_longlong(e) >> 52) & 0x7FF); }
 // The binade of e > 2^-900: its end, half its start (terms below that are rounded by adding `magic`), half its spacing.
 struct Binade {
     double end, half, magic, tie;
+    int k;                                                    // biased exponent
     bool valid;
     __device__ __forceinline__ explicit Binade(double e) {
-        const int k = (int)((__double_as_longlong(e) >> 52) & 0x7FF);
+        k = exponent(e);
         valid = k > 123 && k < 2000;
         end = __longlong_as_double((long long)(k + 1) << 52);
         half = __longlong_as_double((long long)(valid ? k - 1 : 1) << 52);
@@ -136,10 +163,16 @@ struct Binade {
     }
 };
 
-// The terms of 256 bins in shared memory: lane l of the adding warp takes bins 8 l .. 8 l + 7 (pitch: no bank conflicts
-// either way).
+// The terms of 256 bins in shared memory: lane l has bins 8 l .. 8 l + 7 (pitch: no bank conflicts either way).
 constexpr int kPitch = 36, kBlockTerms = 8 * kPitch;
-__host__ __device__ __forceinline__ constexpr int term_at(int i) { return (i >> 8) * kBlockTerms + (i & 7) * kPitch + ((i & 255) >> 3); }
+__host__ __device__ __forceinline__ constexpr int term_at(int i) { return (i & 7) * kPitch + (i >> 3); }
+
+constexpr int kCross = 3;                                     // crossings of a block that are walked one by one
+__device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll
+    for (int o = 16; o; o >>= 1) v = __dadd_rn(v, __shfl_xor_sync(0xffffffffu, v, o));
+    return v;
+}
 
 // e + the first 256 terms, one by one (every lane does it).  They grow from nothing: e leaves a binade every few of them.
 __device__ double add_first(double e, const double* terms)
@@ -182,11 +215,14 @@ __device__ double add_block(double e, const double* terms, int lane)
     return e;
 }
 
-__global__ void __launch_bounds__(kSearchThreads)
+__global__ void __launch_bounds__(kSearchThreads, 2)
 qs_search_kernel(QsHeader* hdr, const unsigned int* hist, int bins, double n_total, float* scale_alpha, double* table,
                  double* errors, uint32_t* status)
 {
-    __shared__ double terms[2][kSlice / 256 * kBlockTerms];
+    __shared__ double terms[kSearchWarps][kBlockTerms];
+    __shared__ double plain_sum[kSearchWarps], seg_sum[kSearchWarps][kCross + 1], e_now;
+    __shared__ int seg_k[kSearchWarps][kCross + 1];           // a segment's binade, -1: it is empty
+    __shared__ uint32_t crossings[kSearchWarps];              // lanes
     __shared__ bool last;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const float Mf = __uint_as_float(hdr->max_bits);
@@ -210,35 +246,97 @@ qs_search_kernel(QsHeader* hdr, const unsigned int* hist, int bins, double n_tot
     const double width = __ddiv_rn(M, (double)bins);
     double e = alpha > 0.0 ? 0.0 : -1.0;
     if (alpha > 0.0) {
-        // warps 1-15 work out the terms of a slice of bins (with the next slice's counts on their way) while warp 0 adds up
-        // the slice before it
-        constexpr int kMakers = kSearchThreads - 32, kPer = (kSlice + kMakers - 1) / kMakers;
-        const int slices = ceil_div(bins, kSlice), me = (int)threadIdx.x - 32;
-        unsigned int c[kPer];
-        auto counts = [&](int s) {
+        const Divisor64 by_n(n_total), by_alpha(alpha);
+        const int blocks = ceil_div(bins, 256);
+        if (threadIdx.x == 0) e_now = 0.0;
+        for (int first = 0; first < blocks; first += kSearchWarps) {
+            const int i0 = (first + warp) * 256 + lane * 8;
+            unsigned int c[8];
+            if (i0 + 8 <= bins) {
+                const uint4 lo = __ldg(reinterpret_cast<const uint4*>(hist + i0)), hi = __ldg(reinterpret_cast<const uint4*>(hist + i0) + 1);
+                c[0] = lo.x; c[1] = lo.y; c[2] = lo.z; c[3] = lo.w; c[4] = hi.x; c[5] = hi.y; c[6] = hi.z; c[7] = hi.w;
+            } else {
 #pragma unroll
-            for (int k = 0; k < kPer; ++k) {
-                const int i = me + k * kMakers, b = s * kSlice + i;
-                c[k] = i < kSlice && b < bins ? hist[b] : 0u;
+                for (int j = 0; j < 8; ++j) c[j] = i0 + j < bins ? hist[i0 + j] : 0u;
             }
-        };
-        if (warp > 0) counts(0);
-        for (int s = 0; s <= slices; ++s) {
+            double v[8], sum = 0.0;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                v[j] = qs_term(c[j], i0 + j, width, by_n, by_alpha);
+                terms[warp][j * kPitch + lane] = v[j];
+                sum = __dadd_rn(sum, v[j]);
+            }
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const double w = __shfl_up_sync(0xffffffffu, sum, o);
+                if (lane >= o) sum = __dadd_rn(sum, w);
+            }
+            if (lane == 31) plain_sum[warp] = sum;
+            __syncthreads();
+            // guesses: e at the first of this lane's bins and after the last (the next lane's first)
+            const double before = __dadd_rn(e_now, warp_sum(lane < warp ? plain_sum[lane] : 0.0)), end = __dadd_rn(before, sum);
+            double start = __shfl_up_sync(0xffffffffu, end, 1);
+            if (lane == 0) start = before;
+            const Binade bn(start);
+            bool bad = !bn.valid || exponent(end) != bn.k, b1;
+            double q = 0.0;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) { q = __dadd_rn(q, bn.round(v[j], &b1)); bad |= b1; }
+            const uint32_t cross = __ballot_sync(0xffffffffu, bad);
+            const int n_cross = __popc(cross), segment = bad ? -1 : __popc(cross & ((1u << lane) - 1));
+            for (int i = 0; i <= min(n_cross, kCross); ++i) {
+                const uint32_t in = __ballot_sync(0xffffffffu, segment == i);
+                const double s = warp_sum(segment == i ? q : 0.0);
+                const int k = __shfl_sync(0xffffffffu, bn.k, in ? __ffs(in) - 1 : 0);
+                if (lane == 0) { seg_sum[warp][i] = s; seg_k[warp][i] = in ? k : -1; }
+            }
+            if (lane == 0) crossings[warp] = cross;
+            __syncthreads();
             if (warp == 0) {
-                if (s == 1) e = add_first(e, terms[0]);
-                const int n = s > 0 ? min(kSlice, bins - (s - 1) * kSlice) : 0;
-                for (int b = s == 1 ? 1 : 0; b * 256 < n; ++b) e = add_block(e, terms[(s - 1) & 1] + b * kBlockTerms, lane);
-            } else if (s < slices) {
-                double v[kPer];
+                const int n = min(kSearchWarps, blocks - first);
+                e = e_now;
+                int b = 0;
+                if (first == 0) { e = add_first(e, terms[0]); b = 1; }
+                const uint32_t cross_l = lane < n ? crossings[lane] : 1u;
+                const double s_l = lane < n ? seg_sum[lane][0] : 0.0;
+                const int k_l = cross_l == 0 ? seg_k[lane][0] : -1;
+                for (; b < n; ++b) {
+                    // blocks from b on without a crossing, as far as e stays in its binade
+                    double after = lane >= b ? s_l : 0.0;
 #pragma unroll
-                for (int k = 0; k < kPer; ++k) v[k] = qs_term(c[k], s * kSlice + me + k * kMakers, width, n_total, alpha);
-                counts(s + 1);
+                    for (int o = 1; o < kSearchWarps; o <<= 1) {
+                        const double w = __shfl_up_sync(0xffffffffu, after, o);
+                        if (lane >= o) after = __dadd_rn(after, w);
+                    }
+                    after = __dadd_rn(e, after);
+                    const uint32_t stop = __ballot_sync(0xffffffffu, lane >= b && !(k_l == exponent(e) && exponent(after) == k_l));
+                    const int upto = __ffs(stop) - 1;         // lane n at the latest
+                    if (upto > b) { e = __shfl_sync(0xffffffffu, after, upto - 1); b = upto; }
+                    if (b >= n) break;
+                    uint32_t left = crossings[b];
+                    const int nc = __popc(left);
+                    bool good = nc <= kCross;
+                    double f = e;
+                    for (int i = 0; good; ++i) {
+                        const int k = seg_k[b][i];
+                        if (k >= 0) {
+                            const double to = __dadd_rn(f, seg_sum[b][i]);
+                            good = exponent(f) == k && exponent(to) == k;
+                            f = to;
+                        }
+                        if (i == nc) break;
+                        const int l = __ffs(left) - 1;
+                        left &= left - 1;
 #pragma unroll
-                for (int k = 0; k < kPer; ++k)
-                    if (me + k * kMakers < kSlice) terms[s & 1][term_at(me + k * kMakers)] = v[k];
+                        for (int j = 0; j < 8; ++j) f = __dadd_rn(f, terms[b][j * kPitch + l]);
+                    }
+                    e = good ? f : add_block(e, terms[b], lane);
+                }
+                if (lane == 0) e_now = e;
             }
             __syncthreads();
         }
+        e = e_now;
     }
     if (threadIdx.x == 0) {
         errors[cand] = e;
@@ -247,9 +345,13 @@ qs_search_kernel(QsHeader* hdr, const unsigned int* hist, int bins, double n_tot
         __threadfence();
     }
     __syncthreads();
-    if (!last || threadIdx.x != 0) return;
-    // the minima, in the order the algorithm visits the candidates
-    volatile double* er = errors;
+    if (!last) return;
+    // the minima, in the order the algorithm visits the candidates (one thread; the errors are fetched by all, since one
+    // after the other they took 15 us)
+    double* er = terms[0];
+    for (int i = threadIdx.x; i < kCandidates; i += kSearchThreads) er[i] = __ldcg(errors + i);
+    __syncthreads();
+    if (threadIdx.x != 0) return;
     int best = 0;
     for (int k = 1; k < kCoarse; ++k) if (er[k] < er[best]) best = k;
     double best_a = coarse(best), best_e = er[best];
