@@ -58,9 +58,9 @@ L2_BYTES = 126e6
 # case per kernel; traffic grows with the bytes streamed, so other cases are scaled by their bytes).
 # Set an entry to None when its kernel changes after the capture.
 NCU_TRAFFIC = {
-    "decode_kernel": {"ratio": 1.007, "case": "8192,8192,832,16"},
-    "decode_tiled_kernel": {"ratio": 1.035, "case": "8192,28672,832,1"},
-    "source": "profiles/decode_kernels_llama2_70b_decode_layer_set.md",
+    "small_kernel": {"ratio": 1.007, "case": "8192,8192,832,16"},
+    "small_kernel_tiled": {"ratio": 1.035, "case": "8192,28672,832,1"},
+    "source": "profiles/small_kernel_llama2_70b_decode_layer_set.md",
 }
 
 
@@ -244,7 +244,7 @@ def run_reference(args):
 
 
 # ------------------------------------------------------------------ GPU arm
-KERNEL_OF = {"slim_linear_fwd": "decode_kernel", "slim_linear_fwd_tiled": "decode_tiled_kernel"}
+KERNEL_OF = {"slim_linear_fwd": "small_kernel", "slim_linear_fwd_tiled": "small_kernel_tiled"}
 
 
 def weight_copy(ly):
@@ -526,7 +526,7 @@ def per_case_table(K, lib, layers, model, ws, ws_bytes, status, stream, peak, ba
             nbytes = algorithmic_bytes(ly["d_in"], ly["d_out"], ly["r"], b)
             gbs = nbytes / (med * 1e-6) / 1e9
             rows.append({"model": model, "layer": ly["name"], "d_in": ly["d_in"], "d_out": ly["d_out"], "r": ly["r"], "b": b,
-                         "kernel": "decode_tiled_kernel" if hint_tiled else "decode_kernel",
+                         "kernel": KERNEL_OF["slim_linear_fwd_tiled" if hint_tiled else "slim_linear_fwd"],
                          "us": round(med, 3), "us_min": round(best, 3), "GBs": round(gbs, 1),
                          "frac_measured": round(gbs / peak, 4), "frac_nominal_8TBs": round(gbs / NOMINAL_HBM_GBS, 4),
                          "roofline_us": round(nbytes / peak / 1e3, 3),

@@ -65,12 +65,13 @@ typedef enum {
 
 /* Kernel families the dispatcher chooses from (slim_linear_fwd_ex). */
 typedef enum {
-    SLIM_KERNEL_AUTO = 0,    /* by batch size: decode for b <= 16, prefill above */
+    SLIM_KERNEL_AUTO = 0,    /* by batch size and shape */
     SLIM_KERNEL_SIMPLE = 1,  /* CUDA-core kernel, any legal shape; correctness anchor */
     SLIM_KERNEL_DECODE = 2,  /* streaming sparse tensor-core kernel for small batches */
-    SLIM_KERNEL_PREFILL = 3, /* tcgen05 sparse tensor-core kernel for many tokens */
-    SLIM_KERNEL_PREFILL_PAIR = 4 /* the same with two CTAs per 256-row tile (cta_group::2); never chosen
-                                    by the dispatcher; needs an even number of 128-row tiles */
+    SLIM_KERNEL_PREFILL = 3, /* tcgen05 sparse tensor-core kernels for many tokens: CTA pairs on 256-row tiles,
+                                or one CTA per 128-row tile where those would be few */
+    SLIM_KERNEL_PREFILL_PAIR = 4 /* the CTA-pair kernel whatever the size; asked for by name it needs an
+                                    even number of 128-row tiles */
 } slim_kernel_t;
 
 /*
@@ -96,11 +97,11 @@ slim_status_t slim_unpack(const uint8_t* vals, const uint8_t* meta, int d_out, i
                           int8_t* codes, uint8_t* mask, void* cuda_stream);
 
 /*
- * Bytes of device scratch slim_linear_fwd needs for this problem (split-K
- * partial sums, the adapter intermediate T = X R^T, and a call counter).
+ * Bytes of device scratch slim_linear_fwd needs for this problem (a call counter, the
+ * adapter intermediate T = X R^T with its hand-over words, partial sums of T).
  * Returns 0 for illegal arguments.  A workspace must be initialised once with
- * slim_workspace_reset before its first use (counter zero, every hand-over slot
- * marked empty); each call, whichever kernel it runs, leaves it ready for the next
+ * slim_workspace_reset before its first use (counter and hand-over words zero: a word
+ * carries the number of the call that wrote it); each call, whichever kernel it runs, leaves it ready for the next
  * one, of any shape the workspace is large enough for, unless it reported
  * SLIM_ERR_TIMEOUT, after which it must be reset again.  Calls that share a
  * workspace must not overlap on the GPU.
@@ -121,11 +122,12 @@ slim_status_t slim_workspace_reset(void* workspace, size_t workspace_bytes, void
  *   L [d_out, r] bf16, R [r, d_in] bf16 (both NULL iff r == 0), Y [b, d_out] bf16 (out).
  * Shape rules: b >= 1, d_in % 64 == 0, d_out % 16 == 0, r % 16 == 0; s must be finite
  * (NaN or infinity: SLIM_ERR_INVALID_ARG).
- * The kernel is chosen from b and the shape: for b <= 16 the streaming decode kernel, which
- * needs d_in % 256 == 0; above, the tcgen05 prefill kernel, which needs d_in % 128 == 0 and
- * d_out % 128 == 0.  Every other legal shape runs on a plain CUDA-core kernel (one warp per
- * output element) that is orders of magnitude slower: it exists for correctness, not speed.
- * For b <= 16 the fast path is slim_linear_fwd_tiled on the decode-tiled copy of the weight.
+ * The kernel is chosen from b and the shape: up to 16 tokens, and up to 64 of layers with
+ * fewer than 8192 rows, the streaming small-batch kernel (r <= 3072); above, the tcgen05 prefill kernels.
+ * All take any legal shape.  Small ragged problems (d_in % 128 or, above 16 tokens, d_out % 128 not zero,
+ * d_out < 256, fewer than 2^24 multiply-adds) and small batches of a larger rank run on a plain CUDA-core
+ * kernel (one warp per output element).
+ * For one to four tokens of a weight of 64 MiB or more slim_linear_fwd_tiled on the decode-tiled copy is faster.
  */
 slim_status_t slim_linear_fwd(const void* X, int b, const uint8_t* vals, const uint8_t* meta,
                               float s, const void* L, const void* R, int r, int d_out, int d_in,
@@ -142,10 +144,10 @@ slim_status_t slim_linear_fwd_ex(const void* X, int b, const uint8_t* vals, cons
  * Decode-tiled copy of a packed weight, and the small-batch forward that reads it.
  *
  * At batch sizes 1-16 the layer is bound by the bytes of the weight it streams (Sec. 4
- * "Speedup": small decode batches; Fig. 3: quantization contributes most of the speed-up),
- * and the kernel then has about one instruction slot per three weight bytes.  The packed
+ * "Speedup": small decode batches; Fig. 3: quantization contributes most of the speed-up)
+ * and by the instructions that expand them.  The packed
  * format above keeps a row's bytes together, which costs the streaming kernel a byte-pick per
- * register and four-fold redundant shared-memory reads; the tiled copy holds the same nibbles
+ * register; the tiled copy holds the same nibbles
  * and position indices (0.375 byte per weight, nothing is computed) in the order the sparse
  * tensor-core instruction consumes them.  Like the packed format it is this library's own
  * layout (the paper leaves storage to a third-party kernel).  Layout SLIM_LAYOUT_DECODE_TILED,
@@ -194,10 +196,8 @@ slim_status_t slim_linear_fwd_tiled(const void* X, int b, const void* tiled, int
 /*
  * Which copy of a weight serves small-batch calls of this shape faster on the current device:
  * 0 = the packed format (slim_linear_fwd), SLIM_LAYOUT_DECODE_TILED = the decode-tiled copy
- * (slim_linear_fwd_tiled).  The tiled kernel streams large weights at a higher rate but has a
- * longer fixed start and end that grows with the batch (activations and T are staged by few warps):
- * the rule is "tiled when the packed weight has 64 MiB or more and b <= 4 (b <= 2 when d_out < d_in)",
- * from timings of both
+ * (slim_linear_fwd_tiled).  The rule is "tiled when the packed weight has 64 MiB or more and
+ * b <= 4 (b <= 2 when d_out < d_in)", from timings of both
  * kernels on the LLaMA-2 layer shapes.  Returns 0 as well for shapes the tiled kernel does not take
  * and for illegal arguments.  (Storage layout is the implementation's choice: Sec. 4 "Speedup"
  * measures the layer, the paper fixes no format.)
@@ -286,8 +286,8 @@ slim_status_t slim_unpack_adapter(const uint8_t* codes, const void* scales, int 
 /*
  * The layer forward with quantized adapters (SLiM-LoRA^Q; Sec. 3.3, with the layer of Sec. 3.2):
  * slim_linear_fwd with L and R given as codes and scales (Lq/Ls for L[d_out][r], Rq/Rs for
- * R[r][d_in]).  r >= 16.  For b <= 16 and shapes the decode kernel takes, the decode kernel reads codes
- * and scales as they are (through tensor maps; L's codes with plain loads when their rows of r / 2 bytes
+ * R[r][d_in]).  r >= 16.  Where the small-batch kernel runs (slim_linear_fwd), it reads codes
+ * and scales as they are (through tensor maps; L's codes with 8-byte copies when their rows of r / 2 bytes
  * are no 16-byte multiples): it multiplies the exact integer codes and scales its accumulator once
  * per group, and a call moves
  * 4.125 bits per adapter element instead of 16 (Sec. 4 "Speedup": quantized adapters cut the
@@ -312,12 +312,12 @@ slim_status_t slim_linear_fwd_q(const void* X, int b, const uint8_t* vals, const
  * a plug-in living inside a runtime that has handed all device memory to its
  * own pool, a process working under a fixed memory budget.  Such a caller
  * cannot provide the workspace slim_linear_fwd asks for, so this variant keeps
- * the decode kernel's scratch (split-K partial sums and barrier counters) in a
+ * the small-batch kernel's scratch (T and the call counter) in a
  * fixed array of SLIM_NOALLOC_SCRATCH_BYTES inside the library's device image.
  * Every GPU that loads the library holds that array until the process exits.
  *
  * Same operation, arguments and rounding as slim_linear_fwd, for b <= 16 and the
- * shapes the decode kernel takes (d_in % 256 == 0); other problems return
+ * shapes with d_in % 256 == 0, d_in <= 32768; other problems return
  * SLIM_ERR_UNSUPPORTED_SHAPE, and a problem whose scratch would exceed the
  * array returns SLIM_ERR_WORKSPACE (all LLaMA-2 7B/13B/70B layer shapes fit).
  * The call makes no cudaMalloc / cudaFree and uses no allocating library
@@ -350,9 +350,9 @@ slim_kernel_t slim_select_kernel(int b, int d_out, int d_in, int r);
 int slim_last_launch_count(void);
 
 /*
- * Token-tile width (64 or 256 tokens) of the prefill kernel the last slim_linear_fwd* call on this host
- * thread launched, 0 if that call ran another kernel.  The prefill kernel has a wide variant for problems
- * with enough 128-row x 256-token tiles for a quarter of the SMs or more and a narrow one for the rest; tests use this query to
+ * Token-tile width (64, 128 or 256 tokens) of the prefill kernel the last slim_linear_fwd* call on this host
+ * thread launched, 0 if that call ran another kernel.  The CTA-pair kernel takes the narrowest width with which
+ * every tile has a pair of its own, else 256; the one-CTA kernel's is 64.  Tests use this query to
  * make sure they exercise the variant they mean to.
  */
 int slim_last_token_tile(void);
