@@ -1,31 +1,38 @@
 // slim_mask_top2: the 2:4 mask of the pipeline's second step (Sec. 3, Fig. 1; metric: Sec. 3.2, the product
 // of weight and input magnitudes).  One thread per group of four along d_in: metric |code| * xbar[k] (one
 // binary32 multiplication; xbar == nullptr: |code|), the two largest kept, equal metrics to the lower
-// index.  HBM-bound: 1 B read + 1 B written per weight.  4096 x 11008: 57 us with one thread per group, now 30 us.
+// index.  1 B read + 1 B written per weight, and the integer pipe: a group costs it 13
+// operations, the six comparisons being subtractions on the other pipe whose sign bits are voted on.  4096 x 11008: 57 us with
+// one thread per group, 30 with four groups a thread and comparisons on the integer pipe (about 30 operations), now 20.
 #include "common.cuh"
 
 namespace slim {
 
-__device__ __forceinline__ uint32_t ge(float a, float b) {           // all ones if a >= b
-    uint32_t r;
-    asm("set.ge.u32.f32 %0, %1, %2;" : "=r"(r) : "f"(a), "f"(b));
-    return r;
+// Bit 31: a < b.  (A difference of two distinct numbers is never zero when nothing is flushed; inf - inf is positive here.)
+__device__ __forceinline__ uint32_t less(float a, float b) {
+    float d;
+    asm("sub.rn.f32 %0, %1, %2;" : "=f"(d) : "f"(a), "f"(b));
+    return __float_as_uint(d);
 }
 __device__ __forceinline__ uint32_t majority(uint32_t a, uint32_t b, uint32_t c) { return (a & b) | (a & c) | (b & c); }
 
 __device__ __forceinline__ uint32_t top2(uint32_t c, const float4* x)
 {
-    // magnitudes (0-128) as floats: the byte in the significand of 2^23, less 2^23
-    const uint32_t mag = __vabs4(c);
+    // codes as floats: code + 128 in the significand of 2^23, less 2^23 + 128; then magnitudes
+    const uint32_t biased = c ^ 0x80808080u;
     float m[4];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) m[k] = __uint_as_float(__byte_perm(mag, 0x4B000000u, 0x7440 + k)) - 8388608.f;
+    for (int k = 0; k < 4; ++k) m[k] = fabsf(__uint_as_float(__byte_perm(biased, 0x4B000000u, 0x7440 + k)) - 8388736.f);
     if (x) { m[0] = __fmul_rn(m[0], x->x); m[1] = __fmul_rn(m[1], x->y); m[2] = __fmul_rn(m[2], x->z); m[3] = __fmul_rn(m[3], x->w); }
-    // c_ij, i < j: entry i beats entry j (equal metrics: the lower index does).  An entry is kept when it beats
-    // at least two of the other three: a majority of three comparisons, one logic operation.
-    const uint32_t c01 = ge(m[0], m[1]), c02 = ge(m[0], m[2]), c03 = ge(m[0], m[3]), c12 = ge(m[1], m[2]), c13 = ge(m[1], m[3]), c23 = ge(m[2], m[3]);
-    return (majority(c01, c02, c03) & 0x1u) | (majority(~c01, c12, c13) & 0x100u) |
-           (majority(~c02, ~c12, c23) & 0x10000u) | (majority(~c03, ~c13, ~c23) & 0x1000000u);
+    // l_ij, i < j, in bit 31: entry i loses to entry j (equal metrics: the lower index wins).  An entry is kept when it beats
+    // at least two of the other three: a majority of three, one logic operation.
+    const uint32_t l01 = less(m[0], m[1]), l02 = less(m[0], m[2]), l03 = less(m[0], m[3]), l12 = less(m[1], m[2]), l13 = less(m[1], m[3]), l23 = less(m[2], m[3]);
+    const uint32_t k0 = majority(~l01, ~l02, ~l03), k1 = majority(l01, ~l12, ~l13), k2 = majority(l02, l12, ~l23), k3 = majority(l03, l13, l23);
+    // prmt with its sign mode: a byte of ones for a set bit 31
+    uint32_t p, q;
+    asm("prmt.b32 %0, %1, %2, 0xFBFB;" : "=r"(p) : "r"(k0), "r"(k1));
+    asm("prmt.b32 %0, %1, %2, 0xFBFB;" : "=r"(q) : "r"(k2), "r"(k3));
+    return __byte_perm(p, q, 0x7610) & 0x01010101u;
 }
 
 // A thread owns V (four, or one where a row is no multiple of four groups) groups of columns and walks rows: its input
