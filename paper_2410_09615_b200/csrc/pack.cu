@@ -7,22 +7,21 @@ namespace slim {
 // One thread handles 16 consecutive columns (four groups) of one row: two
 // 16-byte loads, one 4-byte and one 2-byte store.  Consecutive threads walk
 // consecutive columns, so a warp reads 512 contiguous bytes of codes and mask.
-// The four mask bytes of a group become a 4-bit number, its index nibble comes from a 64-bit table and the two codes
-// from one byte permutation: no branches and no loops over positions (4096 x 11008: 53 -> 20 us).
+// The four mask bytes of a group become a 4-bit number; a 16-entry table in shared memory gives its index nibble and
+// the byte selector that picks the two codes.  Bound by the integer pipe and the L2: 4096 x 11008 53 us with a loop over
+// positions, 26 with the table in a 64-bit number and emulated byte comparisons (about 30 operations a group), now 22.
 //
-// Index nibble (lower | upper << 2) for each set of kept positions; a set of fewer than two is completed with the
-// lowest positions not kept.  Sets of three and four are errors (0x4).
-__host__ __device__ constexpr unsigned long long index_table() {
-    unsigned long long t = 0;
-    for (int m = 0; m < 16; ++m) {
-        int pos[2] = {0, 0}, kept = 0;
-        for (int i = 0; i < 4; ++i)
-            if ((m >> i) & 1) { if (kept < 2) pos[kept] = i; ++kept; }
-        if (kept == 0 || (kept == 1 && pos[0] == 0) || kept > 2) { pos[0] = 0; pos[1] = 1; }
-        else if (kept == 1) { pos[1] = pos[0]; pos[0] = 0; }
-        t |= (unsigned long long)(pos[0] | (pos[1] << 2)) << (4 * m);
+// A table entry: bits 0-15 the selector of the two kept codes, bits 16-19 the index nibble (lower | upper << 2), bit 31 more than
+// two positions are kept.  A set of fewer than two is completed with the lowest positions not kept.
+__device__ __forceinline__ uint32_t index_entry(uint32_t m) {
+    const int kept = __popc(m);
+    int p0 = 0, p1 = 1;
+    if (kept == 1 || kept == 2) {
+        p0 = __ffs(m) - 1;
+        p1 = kept == 2 ? 31 - __clz(m) : p0;
+        if (kept == 1) { if (p0 == 0) p1 = 1; else p0 = 0; }
     }
-    return t;
+    return (uint32_t)(p0 | p1 << 4) | 0x4400u | (uint32_t)(p0 | p1 << 2) << 16 | (kept > 2 ? 1u << 31 : 0u);
 }
 
 __global__ void __launch_bounds__(256)
@@ -30,7 +29,9 @@ pack_kernel(const int8_t* __restrict__ codes, const uint8_t* __restrict__ mask,
             long long n_chunks, uint8_t* __restrict__ vals, uint8_t* __restrict__ meta,
             uint32_t* status_dev)
 {
-    constexpr unsigned long long table = index_table();
+    __shared__ uint32_t table[16];
+    if (threadIdx.x < 16) table[threadIdx.x] = index_entry(threadIdx.x);
+    __syncthreads();
     uint32_t err = 0;
     for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n_chunks;
          c += (long long)gridDim.x * blockDim.x) {
@@ -40,19 +41,19 @@ pack_kernel(const int8_t* __restrict__ codes, const uint8_t* __restrict__ mask,
         uint32_t vout = 0, mout = 0;
 #pragma unroll
         for (int g = 0; g < 4; ++g) {
-            const uint32_t keep = __vcmpne4(mw[g], 0u);                       // 0xFF at kept positions
-            const uint32_t code = cw[g] & keep;
-            const uint32_t m = (((keep & 0x01010101u) * 0x01020408u) >> 24) & 0xFu;
-            uint32_t mb = (uint32_t)(table >> (4 * m)) & 0xFu;
-            const uint32_t two = __byte_perm(code, 0u, (mb & 3u) | (mb >> 2 << 4));      // bytes: lower, upper
-            uint32_t vb = (two & 0xFu) | ((two >> 4) & 0xF0u);
-            const bool many = __popc(m) > 2, range = (__vadd4(code, 0x08080808u) & 0xF0F0F0F0u) != 0;
-            if (many || range) {
-                err |= 1u << (many ? SLIM_ERR_BAD_MASK : SLIM_ERR_CODE_RANGE);
-                vb = 0; mb = 0x4;
+            const uint32_t h = (((mw[g] & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | mw[g]) & 0x80808080u;      // bit 7 of a byte: kept
+            uint32_t keep;                                                    // 0xFF at kept positions
+            asm("prmt.b32 %0, %1, %1, 0xBA98;" : "=r"(keep) : "r"(h));
+            uint32_t e = table[(h * 0x00204081u) >> 28];                      // bits 7, 15, 23, 31 -> 28 .. 31
+            uint32_t two = __byte_perm(cw[g] & keep, 0u, e);                  // bytes: lower, upper
+            const bool range = ((two ^ (two >> 1)) & 0x7878u) != 0;           // bits 3 .. 7 of a code are its sign
+            if ((int)e < 0 || range) {
+                err |= 1u << ((int)e < 0 ? SLIM_ERR_BAD_MASK : SLIM_ERR_CODE_RANGE);
+                two = 0; e = 4u << 16;
             }
+            const uint32_t vb = (two & 0xFu) | ((two >> 4) & 0xF0u);
             vout |= vb << (8 * g);
-            mout |= mb << (4 * g);
+            mout |= ((e >> 16) & 0xFu) << (4 * g);
         }
         reinterpret_cast<uint32_t*>(vals)[c] = vout;
         reinterpret_cast<uint16_t*>(meta)[c] = (uint16_t)mout;
