@@ -1,7 +1,10 @@
 // Prefill-phase forward (many tokens): tcgen05 tensor cores with the accumulator
 // in tensor memory.
 //
-// One CTA computes a 128 (output rows) x N (tokens; N = 256, or 64 for small problems) tile of
+// Two kernels: persistent CTA pairs on 256-row tiles (prefill_pair_kernel, further down, with what it does otherwise), and, where
+// those would be too few, one CTA per 128-row tile.  The text here describes the latter and what they share.
+//
+// One CTA computes a 128 (output rows) x N (64 tokens; up to 256 in the dense-only launch) tile of
 //     out[token][row] = scale * ( sum_k W[row][k] X[token][k]  +  sum_j A2[row][j] B2[token][j] )
 // in two chained phases that accumulate into the same TMEM tile:
 //   phase 1 (sparse): W is the packed int4 2:4 weight.  TMA brings 128 rows of value
@@ -43,9 +46,7 @@
 // 200 cycles even when the phase is long complete, so waits that follow each other are asked
 // together; a lane left at a warp barrier while another lane of its warp spins costs some hundred
 // nanoseconds per iteration; one MMA costs at least the 128 cycles its 128-row A operand takes to
-// load, whatever N.  With one CTA per tile a stage takes about 320 ns: its slot's next token tile
-// is requested ~600 ns after the MMAs that free the slot were issued and lands ~900 ns later, over
-// the 5 stages that fit in shared memory.
+// load, whatever N.
 // Every wait is bounded; an expired one sets SLIM_ERR_TIMEOUT and the kernel runs on.
 #include <atomic>
 #include <cuda.h>
