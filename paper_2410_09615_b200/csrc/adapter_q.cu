@@ -28,6 +28,7 @@ __global__ void __launch_bounds__(256)
 pack_adapter_kernel(const __nv_bfloat16* __restrict__ A, uint32_t items, int cols, int groups,
                     uint8_t* __restrict__ codes, __nv_bfloat16* __restrict__ scales)
 {
+    after_previous_grid();
     constexpr int K = 2;
     const int lane = threadIdx.x & 15;
     const uint32_t first = (blockIdx.x * 16 + (threadIdx.x >> 4)) * K;
@@ -68,6 +69,7 @@ __global__ void __launch_bounds__(256)
 pack_adapter_pairs_kernel(const __nv_bfloat16* __restrict__ A, uint32_t items, int cols, int groups,
                           uint8_t* __restrict__ codes, __nv_bfloat16* __restrict__ scales)
 {
+    after_previous_grid();
     const int lane = threadIdx.x & 31;
     const uint32_t item = blockIdx.x * 8 + (threadIdx.x >> 5);
     if (item >= items) return;
@@ -100,6 +102,7 @@ template <int BYTES>
 __global__ void __launch_bounds__(256)
 unpack_adapter_kernel(const Unpack a, const Unpack b)
 {
+    after_previous_grid();
     uint32_t i = blockIdx.x * 256u + threadIdx.x;
     const bool second = i >= a.items;
     if (second) i -= a.items;
@@ -124,8 +127,8 @@ slim_status_t launch_pack_adapter(const __nv_bfloat16* A, int rows, int cols, ui
     const int groups = (cols + 127) / 128;
     const long long items = (long long)rows * groups;
     if (items > 0x7FFFFFFFll) return SLIM_ERR_INVALID_ARG;
-    if (cols % 8 == 0) pack_adapter_kernel<<<(unsigned)((items + 31) / 32), 256, 0, st>>>(A, (uint32_t)items, cols, groups, codes, scales);
-    else pack_adapter_pairs_kernel<<<(unsigned)((items + 7) / 8), 256, 0, st>>>(A, (uint32_t)items, cols, groups, codes, scales);
+    if (cols % 8 == 0) launch_dependent(pack_adapter_kernel, dim3((unsigned)((items + 31) / 32)), dim3(256), 0, st, A, (uint32_t)items, cols, groups, codes, scales);
+    else launch_dependent(pack_adapter_pairs_kernel, dim3((unsigned)((items + 7) / 8)), dim3(256), 0, st, A, (uint32_t)items, cols, groups, codes, scales);
     count_launch(1);
     return cudaGetLastError() == cudaSuccess ? SLIM_OK : SLIM_ERR_CUDA;
 }
@@ -135,8 +138,7 @@ static Unpack unpack_of(const uint8_t* codes, const __nv_bfloat16* scales, int r
 }
 static slim_status_t launch_unpack(const Unpack& a, const Unpack& b, int bytes, cudaStream_t st) {
     const unsigned grid = (unsigned)(((size_t)a.items + b.items + 255) / 256);
-    if (bytes == 4) unpack_adapter_kernel<4><<<grid, 256, 0, st>>>(a, b);
-    else unpack_adapter_kernel<1><<<grid, 256, 0, st>>>(a, b);
+    launch_dependent(bytes == 4 ? unpack_adapter_kernel<4> : unpack_adapter_kernel<1>, dim3(grid), dim3(256), 0, st, a, b);
     count_launch(1);
     return cudaGetLastError() == cudaSuccess ? SLIM_OK : SLIM_ERR_CUDA;
 }

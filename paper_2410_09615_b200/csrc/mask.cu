@@ -48,6 +48,7 @@ mask_top2_kernel(const typename Words<V>::T* __restrict__ codes, const float* __
 {
     using T = typename Words<V>::T;
     constexpr int kMaskRows = V == 4 ? 4 : 16;
+    after_previous_grid();
     const int g = blockIdx.x * 256 + threadIdx.x;
     if (g >= per_row) return;
     float4 x[V];
@@ -80,8 +81,7 @@ static void launch_mask(const int8_t* codes, const float* xbar, int d_out, int d
     const dim3 grid((unsigned)ceil_div(per_row, 256), (unsigned)(strips < 65535 ? strips : 65535));
     const T* c = reinterpret_cast<const T*>(codes);
     T* m = reinterpret_cast<T*>(mask);
-    if (xbar) mask_top2_kernel<true, V><<<grid, 256, 0, st>>>(c, xbar, per_row, d_out, m, status_dev);
-    else mask_top2_kernel<false, V><<<grid, 256, 0, st>>>(c, xbar, per_row, d_out, m, status_dev);
+    launch_dependent(xbar ? mask_top2_kernel<true, V> : mask_top2_kernel<false, V>, grid, dim3(256), 0, st, c, xbar, per_row, d_out, m, status_dev);
 }
 
 slim_status_t launch_mask_top2(const int8_t* codes, const float* xbar, int d_out, int d_in, uint8_t* mask, uint32_t* status_dev,

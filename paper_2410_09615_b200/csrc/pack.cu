@@ -31,6 +31,7 @@ pack_kernel(const int8_t* __restrict__ codes, const uint8_t* __restrict__ mask,
 {
     __shared__ uint32_t table[16];
     if (threadIdx.x < 16) table[threadIdx.x] = index_entry(threadIdx.x);
+    after_previous_grid();
     __syncthreads();
     uint32_t err = 0;
     for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n_chunks;
@@ -100,7 +101,7 @@ slim_status_t launch_pack(const int8_t* codes, const uint8_t* mask, int d_out, i
     const DeviceInfo* di = device_info(&err);
     if (!di) return err;
     const long long n_chunks = (long long)d_out * d_in / 16;
-    pack_kernel<<<grid_for(n_chunks, di->sm_count), 256, 0, st>>>(codes, mask, n_chunks, vals, meta, status_dev);
+    launch_dependent(pack_kernel, dim3((unsigned)grid_for(n_chunks, di->sm_count)), dim3(256), 0, st, codes, mask, n_chunks, vals, meta, status_dev);
     count_launch(1);
     return cudaGetLastError() == cudaSuccess ? SLIM_OK : SLIM_ERR_CUDA;
 }

@@ -50,6 +50,7 @@ __global__ void __launch_bounds__(512)
 qs_absmax_kernel(const float* __restrict__ W, size_t n, QsHeader* hdr)
 {
     __shared__ unsigned int sm[16], sb[16];
+    after_previous_grid();
     unsigned int m = 0, bad = 0;
     for_weights<false>(W, n, [&](float w) {
         const float a = fabsf(w);
@@ -76,6 +77,7 @@ qs_hist_kernel(const float* __restrict__ W, size_t n, const QsHeader* hdr, int b
 {
     extern __shared__ unsigned int sh[];
     for (int i = threadIdx.x; i < bins; i += blockDim.x) sh[i] = 0;
+    after_previous_grid();
     __syncthreads();
     const float M = __uint_as_float(hdr->max_bits);
     if (M > 0.f && !hdr->bad) {
@@ -224,6 +226,7 @@ qs_search_kernel(QsHeader* hdr, const unsigned int* hist, int bins, double n_tot
     __shared__ int seg_k[kSearchWarps][kCross + 1];           // a segment's binade, -1: it is empty
     __shared__ uint32_t crossings[kSearchWarps];              // lanes
     __shared__ bool last;
+    after_previous_grid();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const float Mf = __uint_as_float(hdr->max_bits);
     if (hdr->bad || !(Mf > 0.f)) {
@@ -373,6 +376,7 @@ qs_search_kernel(QsHeader* hdr, const unsigned int* hist, int bins, double n_tot
 __global__ void __launch_bounds__(256)
 qs_codes_kernel(const float* __restrict__ W, size_t n, const float* __restrict__ scale_alpha, int8_t* __restrict__ codes)
 {
+    after_previous_grid();
     const float a32 = scale_alpha[1];
     const Divisor by(a32 > 0.f ? a32 : 1.f);
     auto code = [&](float w) -> uint32_t {
@@ -429,9 +433,10 @@ slim_status_t launch_quant(const float* W, int d_out, int d_in, int8_t* codes, f
         attr_set[dev].store(true, std::memory_order_release);
     }
     // a block per SM: two would find no more work in flight and double the additions to the global histogram
-    qs_hist_kernel<<<(unsigned)di->sm_count, 1024, hist_smem, st>>>(W, n, hdr, bins, hist);
-    qs_search_kernel<<<kCandidates, kSearchThreads, 0, st>>>(hdr, hist, bins, (double)n, scale_alpha, table, table + 2 * kQsTable + 1, status_dev);
-    qs_codes_kernel<<<(unsigned)(di->sm_count * 8), 256, 0, st>>>(W, n, scale_alpha, codes);
+    launch_dependent(qs_hist_kernel, dim3((unsigned)di->sm_count), dim3(1024), hist_smem, st, W, n, hdr, bins, hist);
+    launch_dependent(qs_search_kernel, dim3(kCandidates), dim3(kSearchThreads), 0, st, hdr, hist, bins, (double)n, scale_alpha, table,
+                     table + 2 * kQsTable + 1, status_dev);
+    launch_dependent(qs_codes_kernel, dim3((unsigned)(di->sm_count * 8)), dim3(256), 0, st, W, n, scale_alpha, codes);
     count_launch(4);
     return cudaGetLastError() == cudaSuccess ? SLIM_OK : SLIM_ERR_CUDA;
 }
