@@ -116,8 +116,10 @@ slim_status_t slim_workspace_reset(void* workspace, size_t workspace_bytes, void
  * The layer forward (Sec. 2 Eq. 1 with W ~ W^C + L R, Sec. 3.2; factored
  * adapter product, App. "Rank Analysis"):
  *     Y[m][n] = s * sum_k X[m][k] Q[n][k]  +  sum_j (sum_k X[m][k] R[j][k]) L[n][j]
- * Products are bf16 x bf16 accumulated in fp32; the intermediate T = X R^T may
- * be rounded once to bf16; Y is rounded to bf16 (nearest even).
+ * Products are bf16 x bf16 accumulated in fp32; the intermediate T = X R^T is rounded once to bf16, except
+ * where rows or columns are no round numbers - up to 16 tokens d_in % 256 != 0 (or d_in > 32768, or from 9
+ * tokens on r > 2560), above d_in % 128 != 0 or d_out % 128 != 0 - and on the CUDA-core kernel: there it keeps
+ * 16 bits or more of its significand; Y is rounded to bf16 (nearest even).
  *   X [b, d_in] bf16, vals/meta as produced by slim_pack, s fp32 scale,
  *   L [d_out, r] bf16, R [r, d_in] bf16 (both NULL iff r == 0), Y [b, d_out] bf16 (out).
  * Shape rules: b >= 1, d_in % 64 == 0, d_out % 16 == 0, r % 16 == 0; s must be finite

@@ -73,7 +73,7 @@ extern "C" slim_status_t slim_linear_fwd_noalloc(const void* X, int b, const uin
     cudaStream_t stream = (cudaStream_t)cuda_stream;
     // the array keeps whatever the previous call left (possibly cut short by a timeout): restart the call counter and
     // the call numbers of T's entries
-    if (cudaMemsetAsync(scratch, 0, SLIM_WORKSPACE_SYNC_BYTES + ((size_t)b * r * 4 + 255) / 256 * 256, stream) != cudaSuccess)
+    if (cudaMemsetAsync(scratch, 0, SLIM_WORKSPACE_SYNC_BYTES + ((size_t)b * r * (keeps_T32(b, d_out, d_in, r) ? 8 : 4) + 255) / 256 * 256, stream) != cudaSuccess)
         return SLIM_ERR_CUDA;
     return launch_small(static_cast<const __nv_bfloat16*>(X), b, vals, meta, nullptr, s, L, R, nullptr, nullptr, r, d_out, d_in,
                         static_cast<__nv_bfloat16*>(Y), scratch, status_dev, stream);

@@ -15,7 +15,8 @@
 //   phase 2 (dense): A2 and B2 are bf16 matrices brought by TMA as they are; the same
 //       thread issues tcgen05.mma into the same accumulator.
 // The layer forward is two or three launches:
-//   T' = (X R^T) / s          phase 2 only (A2 = R, B2 = X, scale 1/s), bf16 into the workspace.
+//   T' = (X R^T) / s          phase 2 only (A2 = R, B2 = X, scale 1/s), bf16 into the workspace, in one or two parts
+//                             (keeps_T32; two: the main launch's dense stages take a column block of either in turn).
 //                             The product has few tiles, so K is split over blockIdx.z; the
 //                             slices write fp32 partial tiles and a small kernel adds them in a
 //                             fixed order (one slice: bf16 directly, no second launch).
@@ -89,6 +90,7 @@ struct PrefillParams {
     int ldo;
     int m_total;            // valid output rows
     int b;                  // valid tokens
+    int t_parts;            // bf16 matrices [b][r], one behind the other, whose sum is T' (keeps_T32): 1 or 2
     int n1, n2;             // stages of the sparse and of the dense phase
     float scale;
     uint32_t* status;
@@ -479,12 +481,13 @@ prefill_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap tmV,
             // dense stage: kDK columns of the token rows and of the A2 rows
             if (lane == 0) mbar_expect_tx(&b_full[st], (uint32_t)(sparse ? kBTile : (N + kPM) * kDK * 2));
             unsigned char* sbase = stages + (size_t)st * kStageBytes;
-            int kb = sparse ? it + rot_g * kPkStages : it - p.n1 + k_first;
+            int kb = sparse ? it + rot_g * kPkStages : it - p.n1 + k_first, y = n0;
+            if (!PRE && !sparse && p.t_parts == 2) { y += (kb & 1) * p.b; kb >>= 1; }    // a column block of either part in turn
             if (sparse && kb >= p.n1) kb -= p.n1;
             const int k = kb * (sparse ? kSK : kDK);
             // lane 0: the token tile (one box); lane 1, dense stages only: the A2 tile
             if (lane == 0 || (lane == 1 && !sparse))
-                tma_tile(lane == 0 ? sbase : sbase + kBTile, lane == 1 ? &tmA2 : (sparse ? &tmX : &tmB2), k, lane == 0 ? n0 : m0, &b_full[st]);
+                tma_tile(lane == 0 ? sbase : sbase + kBTile, lane == 1 ? &tmA2 : (sparse ? &tmX : &tmB2), k, lane == 0 ? y : m0, &b_full[st]);
             if (lane == 0) PSTAMP(0, it);
         }
     } else if (warp == kWarpPk) {
@@ -589,15 +592,23 @@ prefill_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap tmV,
         for (int c0 = half * (N / 2); c0 < (half + 1) * (N / 2); c0 += 32) {
             uint32_t r[32];
             tmem_ld32(tmem_base + lane_base + c0, r);
-            if (orow < p.m_total) {
+            // what differs between the cases is decided outside the unrolled loops: this code runs once, and its size is its time
+            // (the dense-only launch of 512 x 128, 300 tokens, rank 16: 16.7 us with the decisions inside, 10.9 like this)
+            const int n = orow < p.m_total ? p.b - n0 - c0 : 0;
+            size_t step = (size_t)p.ldo;
+            asm volatile("" : "+l"(step));                     // the 32 products of it are not made ahead of the loop over c0
+            auto store = [&](auto* to, auto value) {
 #pragma unroll
-                for (int c = 0; c < 32; ++c) {
-                    const int token = n0 + c0 + c;
-                    if (token < p.b) {
-                        if (PRE && p.part) p.part[((size_t)blockIdx.z * p.b + token) * p.ldo + orow] = __uint_as_float(r[c]);
-                        else p.out[(size_t)token * p.ldo + orow] = __float2bfloat16_rn(p.scale * __uint_as_float(r[c]));
-                    }
-                }
+                for (int c = 0; c < 32; ++c, to += step) if (c < n) *to = value(__uint_as_float(r[c]));
+            };
+            __nv_bfloat16* out = p.out + (size_t)(n0 + c0) * p.ldo + orow;
+            if (PRE && p.part) {
+                store(p.part + ((size_t)blockIdx.z * p.b + n0 + c0) * p.ldo + orow, [](float v) { return v; });
+            } else if (PRE && p.t_parts == 2) {
+                store(out, [&](float v) { return __float2bfloat16_rn(bf16_head(p.scale * v)); });
+                store(out + (size_t)p.b * p.ldo, [&](float v) { return __float2bfloat16_rn(bf16_tail(p.scale * v)); });
+            } else {
+                store(out, [&](float v) { return __float2bfloat16_rn(p.scale * v); });
             }
         }
     }
@@ -689,6 +700,17 @@ __device__ __forceinline__ bool wait_words(const unsigned long long* w, uint32_t
             else if (__any_sync(0xffffffffu, now - t0 > 2000000000ull)) { *abort_flag = 1u; return false; }
         }
     }
+}
+
+// Four neighbouring values of T', in one part or (`tail`: the way to the second) two.
+__device__ __forceinline__ void store_T(__nv_bfloat16* at, size_t tail, float4 v) {
+    auto put = [&](__nv_bfloat16* to, float4 q) {
+        __nv_bfloat162 lo = __floats2bfloat162_rn(q.x, q.y), hi = __floats2bfloat162_rn(q.z, q.w);
+        *reinterpret_cast<uint2*>(to) = make_uint2(*reinterpret_cast<uint32_t*>(&lo), *reinterpret_cast<uint32_t*>(&hi));
+    };
+    if (tail == 0) { put(at, v); return; }
+    put(at, make_float4(bf16_head(v.x), bf16_head(v.y), bf16_head(v.z), bf16_head(v.w)));
+    put(at + tail, make_float4(bf16_tail(v.x), bf16_tail(v.y), bf16_tail(v.z), bf16_tail(v.w)));
 }
 
 template <int N>
@@ -810,11 +832,11 @@ prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap t
                 // both CTAs' bytes are counted on the even CTA's barrier
                 if (lane == 0 && rank == 0) mbar_expect_tx(&b_full[st], (uint32_t)(2 * (sparse ? kBTile : (kHalfTok + kPM) * kDK * 2)));
                 unsigned char* sbase = stages + (size_t)st * kStageBytes;
-                int kb = sparse ? it + ti.rot * kPkStages : it - p.n1;
+                int kb = sparse ? it + ti.rot * kPkStages : it - p.n1, y = ti.n0 + (int)rank * kHalfTok;
                 if (sparse && kb >= p.n1) kb -= p.n1;
+                if (!sparse && p.t_parts == 2) { y += (kb & 1) * p.b; kb >>= 1; }        // a column block of either part in turn
                 const int k = kb * (sparse ? kSK : kDK);
                 // sparse stage: the token tile, two sub-tiles of 64 columns in one box; dense stage: lane 0 the token tile, lane 1 the A2 tile
-                const int y = ti.n0 + (int)rank * kHalfTok;
                 if (sparse) {
                     if (lane == 0) tma_tile_pair3(sbase, &tmX, y, k / kPBK, peer_addr(&b_full[st], 0));
                 } else if (lane < 2) {
@@ -950,8 +972,8 @@ prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap t
         auto store4 = [&](int tile, int c, float4 v) {
             const int token = (tile / p.t_chunks) * kTTok + (int)rank * kPM + row, col = (tile % p.t_chunks) * p.t_n + c;
             if (token >= p.b || col >= p.r) return;
-            __nv_bfloat162 lo = __floats2bfloat162_rn(p.t_scale * v.x, p.t_scale * v.y), hi = __floats2bfloat162_rn(p.t_scale * v.z, p.t_scale * v.w);
-            *reinterpret_cast<uint2*>(p.t_out + (size_t)token * p.r + col) = make_uint2(*reinterpret_cast<uint32_t*>(&lo), *reinterpret_cast<uint32_t*>(&hi));
+            store_T(p.t_out + (size_t)token * p.r + col, p.t_parts == 2 ? (size_t)p.b * p.r : 0,
+                    make_float4(p.t_scale * v.x, p.t_scale * v.y, p.t_scale * v.z, p.t_scale * v.w));
         };
         auto publish = [&](size_t word) {                                    // the writes of the eight warps, then the word
             epilogue_sync();
@@ -1081,7 +1103,7 @@ prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap t
 }
 
 // Sum of the K slices' partial tiles, scaled and rounded to bf16 (fixed order: deterministic).
-__global__ void pre_reduce_kernel(const float* __restrict__ part, int slices, size_t n, float scale, __nv_bfloat16* __restrict__ out)
+__global__ void pre_reduce_kernel(const float* __restrict__ part, int slices, size_t n, float scale, int t_parts, __nv_bfloat16* __restrict__ out)
 {
     // lets the main launch start, then waits for the dense-only launch whose partial tiles it adds
     asm volatile("griddepcontrol.launch_dependents;");
@@ -1092,9 +1114,7 @@ __global__ void pre_reduce_kernel(const float* __restrict__ part, int slices, si
             const float4 v = *reinterpret_cast<const float4*>(part + (size_t)z * n + i);
             acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w;
         }
-        __nv_bfloat162 lo = __floats2bfloat162_rn(scale * acc.x, scale * acc.y), hi = __floats2bfloat162_rn(scale * acc.z, scale * acc.w);
-        uint2 o; o.x = *reinterpret_cast<uint32_t*>(&lo); o.y = *reinterpret_cast<uint32_t*>(&hi);
-        *reinterpret_cast<uint2*>(out + i) = o;
+        store_T(out + i, t_parts == 2 ? n : 0, make_float4(scale * acc.x, scale * acc.y, scale * acc.z, scale * acc.w));
     }
 }
 
@@ -1196,9 +1216,12 @@ static bool runs_wide(int b, int d_out, int d_in, int r, int sm_count, bool auto
     return automatic && (b >= 192 || d_in >= 2048) && (long long)ceil_div(d_out, 2 * kPM) * ceil_div(b, pair_tile(b, d_out, sm_count)) >= 8;
 }
 
+// T' in the workspace; the partial sums follow it.
+static size_t t_bytes(int b, int r, int parts) { return ((size_t)b * (size_t)r * parts * sizeof(__nv_bfloat16) + 255) / 256 * 256; }
+
 size_t prefill_workspace_bytes(int b, int d_out, int d_in, int r) {
     if (!prefill_supports(b, d_out, d_in, r)) return 0;
-    const size_t tq = ((size_t)b * (size_t)r * sizeof(__nv_bfloat16) + 255) / 256 * 256;
+    const size_t tq = t_bytes(b, r, keeps_T32(b, d_out, d_in, r) ? 2 : 1);
     if (r == 0) return tq;
     const PrePlan pl = pre_plan(b, d_in, r, pre_sm_count());
     const size_t narrow = pl.slices > 1 ? (size_t)pl.slices * b * r * sizeof(float) : 0, wide = pair_part_bytes(r, pre_sm_count());
@@ -1281,6 +1304,7 @@ slim_status_t launch_prefill(const __nv_bfloat16* X, int b, const uint8_t* vals,
     }
     __nv_bfloat16* Tq = reinterpret_cast<__nv_bfloat16*>(reinterpret_cast<char*>(ws) + SLIM_WORKSPACE_SYNC_BYTES + kSmallTBytes);
     const float s_eff = s != 0.f ? s : 1.f;       // with s == 0 only the adapter term remains
+    const int t_parts = keeps_T32(b, d_out, d_in, r) ? 2 : 1;
     const bool wide = force_pair || runs_wide(b, d_out, d_in, r, di->sm_count, automatic);
     if (force_pair && ceil_div(d_out, kPM) % 2 != 0) return SLIM_ERR_UNSUPPORTED_SHAPE;
     const int tile_n = wide ? pair_tile(b, d_out, di->sm_count) : 64;
@@ -1305,10 +1329,10 @@ slim_status_t launch_prefill(const __nv_bfloat16* X, int b, const uint8_t* vals,
              pf_map(&tmXpre, X, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (uint64_t)d_in, (uint64_t)b, 64, pl.n_tok, 128);
         if (!ok) return SLIM_ERR_CUDA;
         PrefillParams q = {};
-        q.out = Tq; q.ldo = r; q.m_total = r; q.b = b; q.n1 = 0; q.n2 = d_in / kPBK; q.scale = 1.f / s_eff; q.status = status_dev;
+        q.out = Tq; q.ldo = r; q.m_total = r; q.b = b; q.t_parts = t_parts; q.n1 = 0; q.n2 = d_in / kPBK; q.scale = 1.f / s_eff; q.status = status_dev;
         q.k_per = pl.k_per; q.meta = nullptr; q.meta_pitch = 0; q.d_in = d_in;
         // partial tiles of the K slices follow T' in the workspace
-        q.part = pl.slices > 1 ? reinterpret_cast<float*>(reinterpret_cast<char*>(Tq) + ((size_t)b * r * sizeof(__nv_bfloat16) + 255) / 256 * 256) : nullptr;
+        q.part = pl.slices > 1 ? reinterpret_cast<float*>(reinterpret_cast<char*>(Tq) + t_bytes(b, r, t_parts)) : nullptr;
         slim_status_t rc = pl.n_tok == 256 ? launch_tile_kernel<256, true>(q, r, tmV, tmM, tmXpre, tmA2, tmXpre, st, pl.slices)
                                            : launch_tile_kernel<64, true>(q, r, tmV, tmM, tmXpre, tmA2, tmXpre, st, pl.slices);
         if (rc != SLIM_OK) return rc;
@@ -1322,7 +1346,7 @@ slim_status_t launch_prefill(const __nv_bfloat16* X, int b, const uint8_t* vals,
             rc_attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
             rc_attr[0].val.programmaticStreamSerializationAllowed = 1;
             rc_cfg.attrs = rc_attr; rc_cfg.numAttrs = 1;
-            const cudaError_t re = cudaLaunchKernelEx(&rc_cfg, pre_reduce_kernel, (const float*)q.part, pl.slices, n, q.scale, Tq);
+            const cudaError_t re = cudaLaunchKernelEx(&rc_cfg, pre_reduce_kernel, (const float*)q.part, pl.slices, n, q.scale, t_parts, Tq);
             count_launch(1);
             if (re != cudaSuccess) return SLIM_ERR_CUDA;
         }
@@ -1330,13 +1354,13 @@ slim_status_t launch_prefill(const __nv_bfloat16* X, int b, const uint8_t* vals,
     if (r > 0) {
         // dense stages of the main kernel: 64 columns (128-byte rows) in the pair kernel, else 32 (64-byte rows)
         ok = pf_map(&tmA2, L, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (uint64_t)r, (uint64_t)d_out, dk, kPM, dk == 64 ? 128 : 64) &&
-             pf_map(&tmB2, Tq, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (uint64_t)r, (uint64_t)b, dk, xbox, dk == 64 ? 128 : 64);
+             pf_map(&tmB2, Tq, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (uint64_t)r, (uint64_t)b * t_parts, dk, xbox, dk == 64 ? 128 : 64);
         if (!ok) return SLIM_ERR_CUDA;
     }
     PrefillParams p = {};
-    p.out = Y; p.ldo = d_out; p.m_total = d_out; p.b = b;
+    p.out = Y; p.ldo = d_out; p.m_total = d_out; p.b = b; p.t_parts = t_parts;
     p.n1 = s != 0.f ? ceil_div(d_in, wide ? PairCfg<256>::kSK : PfCfg<64>::kSK) : 0;
-    p.n2 = r > 0 ? ceil_div(r, dk) : 0;
+    p.n2 = r > 0 ? ceil_div(r, dk) * t_parts : 0;
     p.scale = s_eff; p.status = status_dev; p.part = nullptr; p.k_per = 0;
     p.meta = d_in % 128 != 0 ? meta : nullptr; p.meta_pitch = d_in / 8; p.d_in = d_in;
     if (p.n1 + p.n2 == 0)             // s == 0 and no adapters: the result is zero
@@ -1356,7 +1380,7 @@ slim_status_t launch_prefill(const __nv_bfloat16* X, int b, const uint8_t* vals,
         if (r > 0) {
             p.t_n = t_width(r); p.t_chunks = t_chunks(r); p.t_tiles = ceil_div(b, kTTok) * p.t_chunks; p.t_stages = d_in / PairCfg<256>::kDK;
             p.t_scale = 1.f / s_eff; p.t_out = Tq;
-            p.t_part = reinterpret_cast<float4*>(reinterpret_cast<char*>(Tq) + ((size_t)b * r * sizeof(__nv_bfloat16) + 255) / 256 * 256);
+            p.t_part = reinterpret_cast<float4*>(reinterpret_cast<char*>(Tq) + t_bytes(b, r, t_parts));
             p.t_pairs = t_share(p.t_tiles, p.t_stages, pairs, pairs - grid, p.n1);
             grid = grid + p.t_pairs < pairs ? grid + p.t_pairs : pairs;      // the last pairs make T'
         }

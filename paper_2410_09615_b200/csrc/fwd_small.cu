@@ -9,8 +9,8 @@
 // rows to every CTA of the cluster, by asynchronous remote stores.  C is the largest with which the clusters of all tiles are
 // resident at once (two CTAs per SM up to 16 tokens), so that a tile's stream is spread as widely as it can be.
 //   The first clusters make T = X R^T instead: 32 rows of R each, the same cut of d_in; their
-// CTAs exchange partial sums with asynchronous remote stores, round to bf16 and publish T as 8-byte words
-// {two columns, call number}.
+// CTAs exchange partial sums with asynchronous remote stores, round to bf16 (TP = 2: to two bf16 numbers, keeps_T32) and publish T as
+// 8-byte words {two columns, call number}.
 //   A tile's cluster streams the packed weight and the activations through a ring of stages by TMA
 // (256 rows x 64 value bytes, x 32 index bytes, b tokens x 512 bytes; two requesting warps, since one
 // thread starts a request every 220 cycles and the engine takes about one 32-64 byte row a cycle),
@@ -62,7 +62,7 @@ struct SmallParams {
     const void* L; const void* R;                             // bf16, or int4 codes
     const __nv_bfloat16* Ls; const __nv_bfloat16* Rs;         // scales of quantized adapters
     __nv_bfloat16* Y;
-    unsigned long long* T;                                    // [b][r / 2] {bf16 pair, call number}
+    unsigned long long* T;                                    // [TP][b][r / 2] {bf16 pair, call number}
     unsigned long long* departures;
     uint32_t* status;
     float s;
@@ -371,14 +371,8 @@ __device__ __forceinline__ void adapter_stage_q(float (&acc)[NT][4], uint32_t st
     }
 }
 
-// The words of T that B fragments need (two columns each): asked for, then waited for.  No address: a padding token or
-// column, zero.
-template <int NE>
-__device__ __forceinline__ void ask_T(unsigned long long (&v)[NE], const unsigned long long* const (&at)[NE], uint32_t call)
-{
-#pragma unroll
-    for (int n = 0; n < NE; ++n) v[n] = at[n] ? ld_gpu64(at[n]) : (unsigned long long)call << 32;
-}
+// The words of T that B fragments need (two columns each), asked for by `ask` (a padding token or column is there at once, zero)
+// and waited for.
 // Where words are missing, one lane polls one of them, and all are asked for again when it has come: the tiles of a layer
 // wait for the same words, and with every lane polling its own (1024 warps on a few lines of the L2) the words
 // themselves came 1-3 us later (2048 -> 2048, rank 208, 6 tokens: 6.8 us a call instead of 7.5).
@@ -408,12 +402,6 @@ __device__ __forceinline__ bool wait_words(unsigned long long (&v)[NE], uint32_t
     }
     return false;
 }
-template <int NE>
-__device__ __forceinline__ bool wait_T(unsigned long long (&v)[NE], const unsigned long long* const (&at)[NE], uint32_t call)
-{
-    return wait_words(v, call, [&] { ask_T<NE>(v, at, call); }, [&](int n) { return at[n]; });
-}
-
 // The words of eight codes of rows g and g + 8 of a 16-row tile, step h of a stage of L's codes (32-byte rows, 32-byte
 // swizzle), and their product with T.  Integer products are scaled once.
 template <int MT>
@@ -480,13 +468,15 @@ __device__ __forceinline__ void finish(const SmallParams& p, uint32_t smem, int 
 }
 
 // ---------------------------------------------------------------- the kernel
-template <int NT, int FMT, bool QA, int MT>
+template <int NT, int FMT, bool QA, int MT, int TP>
 __global__ void __launch_bounds__(Cfg<NT, MT>::kThreads, Cfg<NT, MT>::kCtasPerSm)
 small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmM,
              const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmR, const __grid_constant__ CUtensorMap tmL)
 {
     using C_ = Cfg<NT, MT>;
     static_assert(MT == 4 || (NT <= 2 && FMT != FMT_TILED), "narrow tiles: up to 16 tokens, packed format");
+    static_assert(TP == 1 || FMT != FMT_TILED, "T in two parts: packed format");
+    const int t_tail = TP == 2 ? p.b * (p.r / 2) : 0;          // from T's first part to the second
     constexpr int kTok = C_::kTok, kNW = C_::kNW, kStages = C_::kStages, kStage = C_::kStage, kRows = C_::kRows;
     constexpr int kValsBytes = C_::kValsBytes, kMetaBytes = C_::kMetaBytes, kXOff = C_::kXOff;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -620,9 +610,14 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
                         const float2 v = lds_f2(recv + (c * p.b * per + e) * 8);
                         s.x += v.x; s.y += v.y;
                     }
-                __nv_bfloat162 pr = __floats2bfloat162_rn(s.x, s.y);
                 if (j < p.r)
-                    st_gpu64(p.T + (size_t)tok * (p.r / 2) + (j >> 1), ((unsigned long long)call << 32) | *reinterpret_cast<uint32_t*>(&pr));
+#pragma unroll
+                    for (int part = 0; part < TP; ++part) {
+                        __nv_bfloat162 pr = TP == 1    ? __floats2bfloat162_rn(s.x, s.y)
+                                            : part == 0 ? __floats2bfloat162_rn(bf16_head(s.x), bf16_head(s.y))
+                                                        : __floats2bfloat162_rn(bf16_tail(s.x), bf16_tail(s.y));
+                        st_gpu64(p.T + part * t_tail + (size_t)tok * (p.r / 2) + (j >> 1), ((unsigned long long)call << 32) | *reinterpret_cast<uint32_t*>(&pr));
+                    }
             }
         } else {
             for (int u = u0; u < u_end; ++u) {
@@ -663,23 +658,31 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
             const int steps = (l_chunks - (int)rank + (int)C - 1) / (int)C * (QA ? 2 : 1);
             for (int it = 0; it < steps; ++it) {
                 const int ls = QA ? 2 * ((int)rank + (it >> 1) * (int)C) + (it & 1) : (int)rank + it * (int)C;
-                const int st = it % C_::kTSlots, use = it / C_::kTSlots;
-                if (use > 0) ok = mbar_wait(t_empty + 8 * st, (use - 1) & 1) && ok;
-                unsigned long long v[kPer];
-                const unsigned long long* at[kPer];
+                unsigned long long v[TP * kPer];               // both parts of T are under way together
                 const int pr = lane & 15, tok0 = (warp - kFetchT) * (kTok / 2) + (lane >> 4);
+                const unsigned long long* at = p.T + (size_t)tok0 * (p.r / 2) + ls * 16 + pr;
+                const int toks = ls * 32 + 2 * pr < p.r ? p.b - tok0 : 0;
+                auto ask = [&] {
 #pragma unroll
-                for (int i = 0; i < kPer; ++i)
-                    at[i] = tok0 + 2 * i < p.b && ls * 32 + 2 * pr < p.r ? p.T + (size_t)(tok0 + 2 * i) * (p.r / 2) + ls * 16 + pr : nullptr;
-                ask_T<kPer>(v, at, call);
-                ok = wait_T<kPer>(v, at, call) && ok;
+                    for (int n = 0; n < TP * kPer; ++n) {
+                        const int i = n % kPer;
+                        v[n] = 2 * i < toks ? ld_gpu64(at + (n / kPer) * t_tail + i * p.r) : (unsigned long long)call << 32;
+                    }
+                };
+                ask();
+                ok = wait_words(v, call, ask, [&](int n) { return at + (n / kPer) * t_tail + (n % kPer) * p.r; }) && ok;
 #pragma unroll
-                for (int i = 0; i < kPer; ++i) {
-                    const int tok = tok0 + 2 * i;
-                    sts32(part + st * C_::kTSlot + tok * 64 + (((pr >> 2) ^ ((tok >> 1) & 3)) << 4) + (pr & 3) * 4, (uint32_t)v[i]);
+                for (int tp = 0; tp < TP; ++tp) {
+                    const int slot = it * TP + tp, st = slot % C_::kTSlots, use = slot / C_::kTSlots;
+                    if (use > 0) ok = mbar_wait(t_empty + 8 * st, (use - 1) & 1) && ok;
+#pragma unroll
+                    for (int i = 0; i < kPer; ++i) {
+                        const int tok = tok0 + 2 * i;
+                        sts32(part + st * C_::kTSlot + tok * 64 + (((pr >> 2) ^ ((tok >> 1) & 3)) << 4) + (pr & 3) * 4, (uint32_t)v[tp * kPer + i]);
+                    }
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(t_full + 8 * st);
                 }
-                __syncwarp();
-                if (lane == 0) mbar_arrive(t_full + 8 * st);
             }
         }
         cluster_wait();
@@ -802,8 +805,8 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
                         for (int m = 0; m < 8; ++m)
                             sc[m] = (m >> 1) < mts && (NT == 8 || (m >> 2) == kk) ? __bfloat162float(p.Ls[(size_t)(row0 + ln.g + 8 * m) * ((p.r + 127) >> 7) + (lc >> 1)]) : 0.f;
 #pragma unroll 1
-                        for (int h = 0; h < 2; ++h, ++lt) {
-                            const int ts = lt % C_::kTSlots;
+                        for (int ht = 0; ht < 2 * TP; ++ht, ++lt) {             // steps, T's parts inside them
+                            const int h = ht / TP, ts = lt % C_::kTSlots;
                             const uint32_t tslot = part + ts * C_::kTSlot;
                             ok = mbar_wait(t_full + 8 * ts, (lt / C_::kTSlots) & 1) && ok;
                             if (mts > 0 && 2 * lc + h < l_steps) {
@@ -818,11 +821,12 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
                             __syncwarp();
                             if (lane == 0) mbar_arrive(t_empty + 8 * ts);
                         }
-                    } else {
+                    } else
+#pragma unroll 1
+                    for (int tp = 0; tp < TP; ++tp, ++lt) {
                         const int ls = lc, ts = lt % C_::kTSlots;
                         const uint32_t tslot = part + ts * C_::kTSlot;
-                        ++lt;
-                        ok = mbar_wait(t_full + 8 * ts, ((lt - 1) / C_::kTSlots) & 1) && ok;
+                        ok = mbar_wait(t_full + 8 * ts, (lt / C_::kTSlots) & 1) && ok;
                         if (mts > 0) {
                             const int mat = lane >> 3, r8 = lane & 7;
 #pragma unroll
@@ -851,28 +855,25 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
                     release();
                 }
             } else if constexpr (!QA) {
-                // kk picks the MMA depth of 16 of a 32-column step; the words of T are asked for one step ahead
+                // kk picks the MMA depth of 16 of a 32-column step; the words of T (of both its parts) are asked for one step ahead
+                constexpr int kWords = 2 * kNW;
                 const int mat = lane >> 3, r8 = lane & 7;
-                unsigned long long v[2 * kNW];
-                const unsigned long long* at[2 * kNW];
+                unsigned long long v[TP * kWords];
+                auto word = [&](int ls, int q) {
+                    const int n = q % kWords;
+                    return p.T + (q / kWords) * t_tail + (size_t)((n >> 1) * 8 + ln.g) * (p.r / 2) + ls * 16 + 8 * kk + ln.t + 4 * (n & 1);
+                };
                 auto ask = [&](int ls) {
-                    const int j = ls * 32 + 16 * kk;
 #pragma unroll
-                    for (int n = 0; n < kNW; ++n) {
-                        const int tok = n * 8 + ln.g;
-                        const unsigned long long* e = p.T + (size_t)tok * (p.r / 2) + (j >> 1) + ln.t;
-                        const bool in = tok < p.b && j < p.r;
-                        at[2 * n] = in ? e : nullptr;
-                        at[2 * n + 1] = in ? e + 4 : nullptr;
-                    }
-                    ask_T<2 * kNW>(v, at, call);
+                    for (int q = 0; q < TP * kWords; ++q)
+                        v[q] = (q % kWords >> 1) * 8 + ln.g < p.b && ls * 32 + 16 * kk < p.r ? ld_gpu64(word(ls, q)) : (unsigned long long)call << 32;
                 };
                 ask((int)rank);
                 for (int ls = (int)rank; ls < l_steps; ls += (int)C) {
-                    ok = wait_T<2 * kNW>(v, at, call) && ok;
-                    uint32_t tb[2 * kNW];
+                    ok = wait_words(v, call, [&] { ask(ls); }, [&](int q) { return word(ls, q); }) && ok;
+                    uint32_t tb[TP * kWords];
 #pragma unroll
-                    for (int q = 0; q < 2 * kNW; ++q) tb[q] = (uint32_t)v[q];
+                    for (int q = 0; q < TP * kWords; ++q) tb[q] = (uint32_t)v[q];
                     ask(ls + (int)C);
                     const uint32_t stage = wait_stage();
                     if (ls * 32 + 16 * kk < p.r && mts > 0) {
@@ -882,26 +883,31 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
                             const int row = (rb * MT + m) * 16 + (mat & 1) * 8 + r8;
                             ldsm4(stage + row * 64 + ((uint32_t)((2 * kk + (mat >> 1)) ^ ((r8 >> 1) & 3)) << 4), a);
 #pragma unroll
-                            for (int n = 0; n < kNW; ++n) mma_16816(acc[m][n], a.x, a.y, a.z, a.w, tb[2 * n], tb[2 * n + 1]);
+                            for (int tp = 0; tp < TP; ++tp)
+#pragma unroll
+                                for (int n = 0; n < kNW; ++n) mma_16816(acc[m][n], a.x, a.y, a.z, a.w, tb[tp * kWords + 2 * n], tb[tp * kWords + 2 * n + 1]);
                         }
                     }
                     release();
                 }
             } else {
-                // codes: kk picks the step of a stage of 64; scales and words of T are asked for one stage ahead
+                // codes: kk picks the step of a stage of 64; scales and words of T are asked for one stage ahead, sixteen words after the
+                // products of this one (with them in registers beside the products these spilled: 1728 -> 20480, 16 tokens 21.9 us, 19.2 so)
+                constexpr int kWords = 4 * kNW;
+                constexpr bool kAhead = TP * kWords <= 8;
                 const uint32_t per_row = (uint32_t)((p.r + 127) >> 7);
                 __nv_bfloat16 next[2 * MT];
-                unsigned long long v[4 * kNW];
-                const unsigned long long* at = p.T + (size_t)ln.g * (p.r / 2) + 4 * ln.t;
+                unsigned long long v[TP * kWords];
+                auto word = [&](int ls, int q) {
+                    const int n = q % kWords;
+                    return p.T + (q / kWords) * t_tail + (size_t)((n >> 2) * 8 + ln.g) * (p.r / 2) + 4 * ln.t + 16 * ls + (n & 3);
+                };
                 auto ask = [&](int ls) {
 #pragma unroll
-                    for (int n = 0; n < kNW; ++n) {
-                        const bool in = ls * 32 + 8 * ln.t < p.r && n * 8 + ln.g < p.b;      // r is a multiple of 16: a thread's 8 columns exist or not
-#pragma unroll
-                        for (int q = 0; q < 4; q += 2) {
-                            v[4 * n + q] = v[4 * n + q + 1] = (unsigned long long)call << 32;
-                            if (in) ld_gpu64x2(at + n * 4 * p.r + 16 * ls + q, v[4 * n + q], v[4 * n + q + 1]);
-                        }
+                    for (int q = 0; q < TP * kWords; q += 2) {
+                        v[q] = v[q + 1] = (unsigned long long)call << 32;
+                        // r is a multiple of 16: a thread's 8 columns exist or not
+                        if (ls * 32 + 8 * ln.t < p.r && (q % kWords >> 2) * 8 + ln.g < p.b) ld_gpu64x2(word(ls, q), v[q], v[q + 1]);
                     }
                 };
                 auto scales = [&](int lc) {
@@ -913,12 +919,12 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
                 ask(2 * (int)rank + kk);
                 for (int lc = (int)rank; lc < l_chunks; lc += (int)C) {
                     const int ls = 2 * lc + kk;
-                    ok = wait_words(v, call, [&] { ask(ls); }, [&](int n) { return at + (n >> 2) * 4 * p.r + 16 * ls + (n & 3); }) && ok;
-                    uint4 tb[kNW];
+                    ok = wait_words(v, call, [&] { ask(ls); }, [&](int q) { return word(ls, q); }) && ok;
+                    uint4 tb[TP][kNW];
 #pragma unroll
-                    for (int n = 0; n < kNW; ++n)
-                        tb[n] = pair_four_apart(make_uint4((uint32_t)v[4 * n], (uint32_t)v[4 * n + 1], (uint32_t)v[4 * n + 2], (uint32_t)v[4 * n + 3]));
-                    ask(ls + 2 * (int)C);
+                    for (int q = 0; q < TP * kNW; ++q)
+                        tb[q / kNW][q % kNW] = pair_four_apart(make_uint4((uint32_t)v[4 * q], (uint32_t)v[4 * q + 1], (uint32_t)v[4 * q + 2], (uint32_t)v[4 * q + 3]));
+                    if (kAhead) ask(ls + 2 * (int)C);
                     float sc[2 * MT];
 #pragma unroll
                     for (int m = 0; m < 2 * MT; ++m) sc[m] = __bfloat162float(next[m]);
@@ -926,8 +932,11 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
                     const uint32_t stage = wait_stage();
                     if (ls < l_steps && mts > 0)
 #pragma unroll
-                        for (int m = 0; m < MT; ++m) code_tile<kNW>(acc[m], l_codes<MT>(stage, rb, m, kk, ln), sc[2 * m], sc[2 * m + 1], tb);
+                        for (int m = 0; m < MT; ++m)
+#pragma unroll
+                            for (int tp = 0; tp < TP; ++tp) code_tile<kNW>(acc[m], l_codes<MT>(stage, rb, m, kk, ln), sc[2 * m], sc[2 * m + 1], tb[tp]);
                     release();
+                    if (!kAhead) ask(ls + 2 * (int)C);
                 }
             }
             // ---------------- partial tiles -> Y
@@ -960,14 +969,17 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
 // ------------------------------------------------------------------ host side
 using KernelFn = void (*)(const SmallParams, const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap);
 
-template <int NT, int FMT, int MT> KernelFn pick_q(bool qa) { return qa ? small_kernel<NT, FMT, true, MT> : small_kernel<NT, FMT, false, MT>; }
-template <int NT, int FMT> KernelFn pick_m(int mt, bool qa) { return mt == 1 ? pick_q<NT, FMT, 1>(qa) : mt == 2 ? pick_q<NT, FMT, 2>(qa) : pick_q<NT, FMT, 4>(qa); }
-template <int FMT> KernelFn pick_n(int nt, int mt, bool qa) {
-    return nt == 1 ? pick_m<1, FMT>(mt, qa) : nt == 2 ? pick_m<2, FMT>(mt, qa) : nt == 4 ? pick_q<4, FMT, 4>(qa) : pick_q<8, FMT, 4>(qa);
+template <int NT, int FMT, int MT, int TP> KernelFn pick_q(bool qa) { return qa ? small_kernel<NT, FMT, true, MT, TP> : small_kernel<NT, FMT, false, MT, TP>; }
+template <int NT, int FMT, int TP> KernelFn pick_m(int mt, bool qa) {
+    return mt == 1 ? pick_q<NT, FMT, 1, TP>(qa) : mt == 2 ? pick_q<NT, FMT, 2, TP>(qa) : pick_q<NT, FMT, 4, TP>(qa);
 }
-KernelFn pick(int nt, int fmt, bool qa, int mt) {
-    if (fmt == FMT_TILED) return nt == 1 ? small_kernel<1, FMT_TILED, false, 4> : small_kernel<2, FMT_TILED, false, 4>;
-    return fmt == FMT_PACKED ? pick_n<FMT_PACKED>(nt, mt, qa) : pick_n<FMT_PACKED_LD>(nt, mt, qa);
+template <int FMT, int TP> KernelFn pick_n(int nt, int mt, bool qa) {
+    return nt == 1 ? pick_m<1, FMT, TP>(mt, qa) : nt == 2 ? pick_m<2, FMT, TP>(mt, qa) : nt == 4 ? pick_q<4, FMT, 4, TP>(qa) : pick_q<8, FMT, 4, TP>(qa);
+}
+// Rows of index bytes that no tensor map describes (FMT_PACKED_LD) belong to shapes whose T has two parts.
+KernelFn pick(int nt, int fmt, bool qa, int mt, int tp) {
+    if (fmt == FMT_TILED) return nt == 1 ? small_kernel<1, FMT_TILED, false, 4, 1> : small_kernel<2, FMT_TILED, false, 4, 1>;
+    return fmt == FMT_PACKED_LD ? pick_n<FMT_PACKED_LD, 2>(nt, mt, qa) : tp == 2 ? pick_n<FMT_PACKED, 2>(nt, mt, qa) : pick_n<FMT_PACKED, 1>(nt, mt, qa);
 }
 int smem_bytes(int nt, int mt) {
     if (mt == 1) return nt == 1 ? Cfg<1, 1>::kSmem : Cfg<2, 1>::kSmem;
@@ -979,16 +991,16 @@ int tiles_of(int b) { return b <= 8 ? 1 : b <= 16 ? 2 : b <= 32 ? 4 : 8; }
 
 // Clusters of 1, 2, 4, 8 CTAs of one kernel that the device holds at once; asked once per device and kernel.
 struct Residency { std::atomic<int> ready{0}; int clusters[4]; };
-Residency g_res[64][4][3][2][3];
+Residency g_res[64][4][3][2][3][2];
 std::mutex g_res_mutex;
 
-const int* residency(int dev, int nt, int fmt, bool qa, int mt) {
+const int* residency(int dev, int nt, int fmt, bool qa, int mt, int tp) {
     const int ni = nt == 1 ? 0 : nt == 2 ? 1 : nt == 4 ? 2 : 3;
-    Residency& rs = g_res[dev][ni][fmt][qa ? 1 : 0][mt >> 1];
+    Residency& rs = g_res[dev][ni][fmt][qa ? 1 : 0][mt >> 1][tp - 1];
     if (rs.ready.load(std::memory_order_acquire)) return rs.clusters;
     std::lock_guard<std::mutex> lock(g_res_mutex);
     if (rs.ready.load(std::memory_order_relaxed)) return rs.clusters;
-    const void* fn = (const void*)pick(nt, fmt, qa, mt);
+    const void* fn = (const void*)pick(nt, fmt, qa, mt, tp);
     if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes(nt, mt)) != cudaSuccess) return nullptr;
     for (int i = 0; i < 4; ++i) {
         cudaLaunchConfig_t cfg = {};
@@ -1049,9 +1061,9 @@ int cluster_size(const int* res, int tiles, int units) {
 // against 12.5), else not (4096 x 4096, rank 208: 9.1 us against 8.3).  With 256-row tiles only: 8192 -> 1024, rank 112, 16
 // tokens 9.3 us instead of 6.6; 5120 x 5120, rank 512, 8 tokens 11.1 instead of 8.6; larger layers are better off with them
 // (28672 -> 8192, 16 tokens 48 us against 65).
-void narrow_tiles(int dev, int nt, int fmt, bool qa, int sm_count, int d_out, int units, int groups, int* mt, int* C) {
+void narrow_tiles(int dev, int nt, int fmt, bool qa, int tp, int sm_count, int d_out, int units, int groups, int* mt, int* C) {
     auto fits = [&](int m) {
-        const int* res = residency(dev, nt, fmt, qa, m);
+        const int* res = residency(dev, nt, fmt, qa, m, tp);
         return res && ceil_div(d_out, 64 * m) + groups <= res[2];
     };
     if (!fits(2)) return;
@@ -1067,7 +1079,7 @@ void narrow_tiles(int dev, int nt, int fmt, bool qa, int sm_count, int d_out, in
 // takes 65536 CTAs.
 bool small_supports(int b, int d_out, int d_in, int r) {
     return b >= 1 && b <= 64 && d_out >= 16 && d_out % 16 == 0 && d_in >= 64 && d_in % 64 == 0 && r >= 0 && r % 16 == 0 &&
-           r <= kSmallMaxRank && (size_t)b * r * 4 <= kSmallTBytes && ceil_div(d_out, 256) < 32768;
+           r <= kSmallMaxRank && (size_t)b * r * (keeps_T32(b, d_out, d_in, r) ? 8 : 4) <= kSmallTBytes && ceil_div(d_out, 256) < 32768;
 }
 
 slim_status_t launch_small(const __nv_bfloat16* X, int b, const uint8_t* vals, const uint8_t* meta, const uint8_t* tiled, float s,
@@ -1082,11 +1094,12 @@ slim_status_t launch_small(const __nv_bfloat16* X, int b, const uint8_t* vals, c
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return SLIM_ERR_CUDA;
     const int nt = tiles_of(b), fmt = tiled ? FMT_TILED : d_in % 128 == 0 ? FMT_PACKED : FMT_PACKED_LD;
     const bool qa = Ls != nullptr;
+    const int tp = !tiled && (fmt == FMT_PACKED_LD || (r > 0 && keeps_T32(b, d_out, d_in, r))) ? 2 : 1;
     const int units = ceil_div(d_in, kUnit), groups = ceil_div(r, kGroup);
     int mt = 4, C = 0;
-    if (nt <= 2 && !tiled) narrow_tiles(dev, nt, fmt, qa, di->sm_count, d_out, units, groups, &mt, &C);
+    if (nt <= 2 && !tiled) narrow_tiles(dev, nt, fmt, qa, tp, di->sm_count, d_out, units, groups, &mt, &C);
     const int rows = 64 * mt;
-    const int* res = residency(dev, nt, fmt, qa, mt);
+    const int* res = residency(dev, nt, fmt, qa, mt, tp);
     if (!res) return SLIM_ERR_CUDA;
     if (mt == 4) C = cluster_size(res, ceil_div(d_out, rows), units);
     SmallParams p;
@@ -1116,7 +1129,7 @@ slim_status_t launch_small(const __nv_bfloat16* X, int b, const uint8_t* vals, c
     a[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     a[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = a; cfg.numAttrs = 2;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, pick(nt, fmt, qa, mt), p, tmV, tmM, tmX, tmR, tmL);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, pick(nt, fmt, qa, mt, tp), p, tmV, tmM, tmX, tmR, tmL);
     count_launch(1);
     return e == cudaSuccess ? SLIM_OK : SLIM_ERR_CUDA;
 }
