@@ -8,7 +8,8 @@
 
 namespace slim {
 
-// Bit 31: a < b.  (A difference of two distinct numbers is never zero when nothing is flushed; inf - inf is positive here.)
+// Bit 31: a < b, for a and b other than -0.  (A difference of two distinct numbers is never zero when nothing is flushed, that of
+// two equal ones +0; inf - inf is positive here.)
 __device__ __forceinline__ uint32_t less(float a, float b) {
     float d;
     asm("sub.rn.f32 %0, %1, %2;" : "=f"(d) : "f"(a), "f"(b));
@@ -23,7 +24,8 @@ __device__ __forceinline__ uint32_t top2(uint32_t c, const float4* x)
     float m[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) m[k] = fabsf(__uint_as_float(__byte_perm(biased, 0x4B000000u, 0x7440 + k)) - 8388736.f);
-    if (x) { m[0] = __fmul_rn(m[0], x->x); m[1] = __fmul_rn(m[1], x->y); m[2] = __fmul_rn(m[2], x->z); m[3] = __fmul_rn(m[3], x->w); }
+    // the product plus zero, in one rounding: the product itself, but +0 for -0 (an input magnitude may be -0)
+    if (x) { m[0] = __fmaf_rn(m[0], x->x, 0.f); m[1] = __fmaf_rn(m[1], x->y, 0.f); m[2] = __fmaf_rn(m[2], x->z, 0.f); m[3] = __fmaf_rn(m[3], x->w, 0.f); }
     // l_ij, i < j, in bit 31: entry i loses to entry j (equal metrics: the lower index wins).  An entry is kept when it beats
     // at least two of the other three: a majority of three, one logic operation.
     const uint32_t l01 = less(m[0], m[1]), l02 = less(m[0], m[2]), l03 = less(m[0], m[3]), l12 = less(m[1], m[2]), l13 = less(m[1], m[3]), l23 = less(m[2], m[3]);

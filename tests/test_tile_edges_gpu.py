@@ -65,6 +65,17 @@ def test_mask_row_widths(rows, d_in):
         assert np.array_equal(got.cpu().numpy(), oracle.mask_top2(codes, x))
 
 
+def test_mask_takes_a_negative_zero_magnitude_for_zero():
+    # -0 is a legal magnitude (not below zero) and ties with +0: the lower index is kept
+    group = np.array([(5, 0, 0, 3), (0, 7, 0, 0), (0, 0, 0, -8), (1, 1, 1, 1), (0, 0, 0, 0), (2, -2, 0, 1)], np.int8)
+    codes = np.tile(group, (1, 16))
+    ones = np.array([[(-0.0 if i >> k & 1 else 1.0) for k in range(4)] for i in range(16)], np.float32).reshape(64)
+    for xbar in (ones, np.copysign(np.float32(0.0), np.where(np.signbit(ones), -1, 1)).astype(np.float32)):
+        got = K.slim_mask_top2(to_dev(codes), to_dev(xbar)).cpu().numpy()
+        assert np.array_equal(got, oracle.mask_top2(codes, xbar))
+    assert np.array_equal(oracle.mask_top2(group[:1], np.array([-0.0, 1, 1, 1], np.float32)), [[1, 0, 0, 1]])
+
+
 @pytest.mark.parametrize("rows,cols", [(3, 130), (9, 1002), (2, 6), (5, 136)])
 def test_adapter_row_widths(rows, cols):
     A = long_tailed(rows, cols, 54)
