@@ -38,20 +38,21 @@ __device__ __forceinline__ uint32_t top2(uint32_t c, const float4* x)
 }
 
 // A thread owns V (four, or one where a row is no multiple of four groups) groups of columns and walks rows: its input
-// magnitudes stay in registers, and it has the loads of kMaskRows rows in flight.
+// magnitudes stay in registers, and it has the loads of ROWS rows in flight.  A block is up to 256 V groups of columns by as many
+// rows as make up 256 threads (100000 x 64: 27.8 us with one row a block); where blocks of several rows a thread would not
+// give every SM two, a thread takes one (64 x 4096: 3.2 us with four).
 template <int V> struct Words;
 template <> struct Words<4> { using T = uint4; };
 template <> struct Words<1> { using T = uint32_t; };
 
-template <bool XBAR, int V>
+template <bool XBAR, int V, int ROWS>
 __global__ void __launch_bounds__(256)
 mask_top2_kernel(const typename Words<V>::T* __restrict__ codes, const float* __restrict__ xbar, int per_row, int d_out,
                  typename Words<V>::T* __restrict__ mask, uint32_t* status)
 {
     using T = typename Words<V>::T;
-    constexpr int kMaskRows = V == 4 ? 4 : 16;
     after_previous_grid();
-    const int g = blockIdx.x * 256 + threadIdx.x;
+    const int g = blockIdx.x * blockDim.x + threadIdx.x, lanes = blockDim.y;
     if (g >= per_row) return;
     float4 x[V];
 #pragma unroll
@@ -60,37 +61,39 @@ mask_top2_kernel(const typename Words<V>::T* __restrict__ codes, const float* __
         if (blockIdx.y == 0 && !(x[v].x >= 0.f && x[v].x <= 3.0e38f && x[v].y >= 0.f && x[v].y <= 3.0e38f && x[v].z >= 0.f && x[v].z <= 3.0e38f && x[v].w >= 0.f && x[v].w <= 3.0e38f))
             flag_error(status, SLIM_ERR_INVALID_ARG);
     }
-    for (int row0 = blockIdx.y * kMaskRows; row0 < d_out; row0 += gridDim.y * kMaskRows) {
-        T c[kMaskRows];
+    for (long long row0 = (long long)blockIdx.y * ROWS * lanes + threadIdx.y; row0 < d_out; row0 += (long long)gridDim.y * ROWS * lanes) {
+        T c[ROWS];
 #pragma unroll
-        for (int i = 0; i < kMaskRows; ++i) c[i] = __ldg(codes + (size_t)min(row0 + i, d_out - 1) * per_row + g);
+        for (int i = 0; i < ROWS; ++i) c[i] = __ldg(codes + (size_t)min(row0 + i * lanes, (long long)d_out - 1) * per_row + g);
 #pragma unroll
-        for (int i = 0; i < kMaskRows; ++i) {
+        for (int i = 0; i < ROWS; ++i) {
             T o;
 #pragma unroll
             for (int v = 0; v < V; ++v)
                 reinterpret_cast<uint32_t*>(&o)[v] = top2(reinterpret_cast<const uint32_t*>(&c[i])[v], XBAR ? &x[v] : nullptr);
-            if (row0 + i < d_out) mask[(size_t)(row0 + i) * per_row + g] = o;
+            if (row0 + i * lanes < d_out) mask[(size_t)(row0 + i * lanes) * per_row + g] = o;
         }
     }
 }
 
-template <int V>
+template <int V, int ROWS>
 static void launch_mask(const int8_t* codes, const float* xbar, int d_out, int d_in, uint8_t* mask, uint32_t* status_dev, cudaStream_t st)
 {
     using T = typename Words<V>::T;
-    const int per_row = d_in / (4 * V), strips = ceil_div(d_out, V == 4 ? 4 : 16);
-    const dim3 grid((unsigned)ceil_div(per_row, 256), (unsigned)(strips < 65535 ? strips : 65535));
+    const int per_row = d_in / (4 * V), cols = per_row < 256 ? per_row : 256, lanes = 256 / cols;
+    const int strips = ceil_div(d_out, ROWS * lanes), blocks = ceil_div(per_row, cols);
+    if (ROWS > 1 && (long long)strips * blocks < 2 * 148) { launch_mask<V, 1>(codes, xbar, d_out, d_in, mask, status_dev, st); return; }
     const T* c = reinterpret_cast<const T*>(codes);
     T* m = reinterpret_cast<T*>(mask);
-    launch_dependent(xbar ? mask_top2_kernel<true, V> : mask_top2_kernel<false, V>, grid, dim3(256), 0, st, c, xbar, per_row, d_out, m, status_dev);
+    launch_dependent(xbar ? mask_top2_kernel<true, V, ROWS> : mask_top2_kernel<false, V, ROWS>, dim3((unsigned)blocks, (unsigned)(strips < 65535 ? strips : 65535)),
+                     dim3((unsigned)cols, (unsigned)lanes), 0, st, c, xbar, per_row, d_out, m, status_dev);
 }
 
 slim_status_t launch_mask_top2(const int8_t* codes, const float* xbar, int d_out, int d_in, uint8_t* mask, uint32_t* status_dev,
                                cudaStream_t st)
 {
-    if (d_in % 16 == 0) launch_mask<4>(codes, xbar, d_out, d_in, mask, status_dev, st);
-    else launch_mask<1>(codes, xbar, d_out, d_in, mask, status_dev, st);
+    if (d_in % 16 == 0) launch_mask<4, 4>(codes, xbar, d_out, d_in, mask, status_dev, st);
+    else launch_mask<1, 16>(codes, xbar, d_out, d_in, mask, status_dev, st);
     count_launch(1);
     return cudaGetLastError() == cudaSuccess ? SLIM_OK : SLIM_ERR_CUDA;
 }

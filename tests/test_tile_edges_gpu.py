@@ -55,7 +55,8 @@ def test_pair_tile_edges(d_in, d_out, r, b, tile):
     assert res["ok"] and res["launches"] == 1 and res["token_tile"] == tile, res
 
 
-@pytest.mark.parametrize("rows,d_in", [(1, 4), (7, 20), (33, 1028), (16, 64), (5, 4112)])
+# (below: rows a block has lanes for, one and several rows a thread, a last block that is not full)
+@pytest.mark.parametrize("rows,d_in", [(1, 4), (7, 20), (33, 1028), (16, 64), (5, 4112), (9475, 64), (1000, 192), (70001, 12), (300, 4100), (1187, 4112), (2500, 1028)])
 def test_mask_row_widths(rows, d_in):
     rng = np.random.default_rng([rows, d_in])
     codes = rng.integers(-8, 8, size=(rows, d_in)).astype(np.int8)
