@@ -96,19 +96,20 @@ pack_adapter_pairs_kernel(const __nv_bfloat16* __restrict__ A, uint32_t items, i
 // Expansion to bf16 of one matrix or of a layer's two: a thread takes four bytes of codes (eight values, one 16-byte
 // store) where rows are multiples of eight elements, else one byte.  (One byte a thread and a launch per matrix took
 // 11 us for the adapters of a 1728 -> 5120 layer, rank 176.)
-struct Unpack { const uint8_t* codes; const __nv_bfloat16* scales; __nv_bfloat16* out; int cols, groups; uint32_t items; };
+struct Unpack { const uint8_t* codes; const __nv_bfloat16* scales; __nv_bfloat16* out; int cols, groups; size_t items; };
 
-template <int BYTES>
+// I: the type of an item's number; TWO: two matrices.
+template <int BYTES, typename I, bool TWO>
 __global__ void __launch_bounds__(256)
 unpack_adapter_kernel(const Unpack a, const Unpack b)
 {
     after_previous_grid();
-    uint32_t i = blockIdx.x * 256u + threadIdx.x;
-    const bool second = i >= a.items;
-    if (second) i -= a.items;
+    I i = (I)blockIdx.x * 256 + threadIdx.x;
+    const bool second = TWO && i >= (I)a.items;
+    if (second) i -= (I)a.items;
     const Unpack& m = second ? b : a;
-    if (i >= m.items) return;
-    const uint32_t per_row = (uint32_t)m.cols / (2 * BYTES), row = i / per_row, c = (i - row * per_row) * (2 * BYTES);
+    if (i >= (I)m.items) return;
+    const uint32_t per_row = (uint32_t)m.cols / (2 * BYTES), row = (uint32_t)(i / per_row), c = (uint32_t)(i - (I)row * per_row) * (2 * BYTES);
     const float sc = __bfloat162float(m.scales[(size_t)row * m.groups + c / 128]);
     const size_t at = (size_t)row * m.cols + c;
     uint32_t w = BYTES == 4 ? __ldg(reinterpret_cast<const uint32_t*>(m.codes + at / 2)) : m.codes[at / 2], o[BYTES];
@@ -134,11 +135,13 @@ slim_status_t launch_pack_adapter(const __nv_bfloat16* A, int rows, int cols, ui
 }
 
 static Unpack unpack_of(const uint8_t* codes, const __nv_bfloat16* scales, int rows, int cols, __nv_bfloat16* out, int bytes) {
-    return Unpack{codes, scales, out, cols, (cols + 127) / 128, (uint32_t)((size_t)rows * (cols / 2) / bytes)};
+    return Unpack{codes, scales, out, cols, (cols + 127) / 128, (size_t)rows * (cols / 2) / bytes};
 }
-static slim_status_t launch_unpack(const Unpack& a, const Unpack& b, int bytes, cudaStream_t st) {
-    const unsigned grid = (unsigned)(((size_t)a.items + b.items + 255) / 256);
-    launch_dependent(bytes == 4 ? unpack_adapter_kernel<4> : unpack_adapter_kernel<1>, dim3(grid), dim3(256), 0, st, a, b);
+template <int BYTES, bool TWO>
+static slim_status_t launch_unpack(const Unpack& a, const Unpack& b, cudaStream_t st) {
+    const size_t items = a.items + b.items;                                   // 2^32 and more: 64-bit numbers
+    launch_dependent(items <= 0xFFFFFF00u ? unpack_adapter_kernel<BYTES, uint32_t, TWO> : unpack_adapter_kernel<BYTES, uint64_t, TWO>,
+                     dim3((unsigned)((items + 255) / 256)), dim3(256), 0, st, a, b);
     count_launch(1);
     return cudaGetLastError() == cudaSuccess ? SLIM_OK : SLIM_ERR_CUDA;
 }
@@ -146,14 +149,15 @@ static slim_status_t launch_unpack(const Unpack& a, const Unpack& b, int bytes, 
 slim_status_t launch_unpack_adapter(const uint8_t* codes, const __nv_bfloat16* scales, int rows, int cols, __nv_bfloat16* out,
                                     cudaStream_t st)
 {
-    const int bytes = cols % 8 == 0 ? 4 : 1;
-    return launch_unpack(unpack_of(codes, scales, rows, cols, out, bytes), Unpack{nullptr, nullptr, nullptr, 2, 1, 0}, bytes, st);
+    const Unpack none = {};
+    return cols % 8 == 0 ? launch_unpack<4, false>(unpack_of(codes, scales, rows, cols, out, 4), none, st)
+                         : launch_unpack<1, false>(unpack_of(codes, scales, rows, cols, out, 1), none, st);
 }
 
 slim_status_t launch_unpack_adapters(const uint8_t* Lq, const __nv_bfloat16* Ls, const uint8_t* Rq, const __nv_bfloat16* Rs, int d_out, int r,
                                      int d_in, __nv_bfloat16* L, __nv_bfloat16* R, cudaStream_t st)
 {
-    return launch_unpack(unpack_of(Lq, Ls, d_out, r, L, 4), unpack_of(Rq, Rs, r, d_in, R, 4), 4, st);     // r % 16 == 0, d_in % 64 == 0
+    return launch_unpack<4, true>(unpack_of(Lq, Ls, d_out, r, L, 4), unpack_of(Rq, Rs, r, d_in, R, 4), st);       // r % 16 == 0, d_in % 64 == 0
 }
 
 }  // namespace slim
