@@ -1206,12 +1206,10 @@ static int pair_tile(int b, int d_out, int sm_count) {
     return 256;
 }
 
-// The pair kernel when its 128 x 256 tiles would give a quarter of the SMs or more a tile, and when the words of its T' tiles fit
-// their region.  The dispatcher (`automatic`) also takes it for smaller problems with eight tiles or more (4096 x 4096, 100 tokens
+// The pair kernel when its 128 x 256 tiles would give a quarter of the SMs or more a tile.  The dispatcher (`automatic`) also takes it for smaller problems with eight tiles or more (4096 x 4096, 100 tokens
 // 25 -> 22 us, 200 tokens 45 -> 26), unless both the batch and d_in are short (1024 -> 4096, 128 tokens: 17 us against 13);
 // asked for by name the one-CTA kernel keeps those.
 static bool runs_wide(int b, int d_out, int d_in, int r, int sm_count, bool automatic) {
-    if ((size_t)ceil_div(b, kTTok) * t_chunks(r) > kSyncTiles) return false;
     if ((long long)ceil_div(d_out, kPM) * ceil_div(b, 256) * 4 >= (long long)sm_count) return true;
     return automatic && (b >= 192 || d_in >= 2048) && (long long)ceil_div(d_out, 2 * kPM) * ceil_div(b, pair_tile(b, d_out, sm_count)) >= 8;
 }
@@ -1280,6 +1278,16 @@ slim_status_t launch_prefill(const __nv_bfloat16* X, int b, const uint8_t* vals,
     const DeviceInfo* di = device_info(&err);
     if (!di) return err;
     if (!prefill_supports(b, d_out, d_in, r)) return SLIM_ERR_UNSUPPORTED_SHAPE;
+    // The words of T' tiles have a region of fixed size (8.1 million tokens of up to 256 ranks): more go in equal parts, one behind
+    // the other on the stream and the workspace.
+    const long long most = r > 0 ? (long long)(kSyncTiles / t_chunks(r)) * kTTok : b;
+    if (b > most) {
+        const int n = ceil_div(ceil_div(b, (int)((b + most - 1) / most)), kTTok) * kTTok;
+        slim_status_t rc = SLIM_OK;
+        for (long long t = 0; t < b && rc == SLIM_OK; t += n)
+            rc = launch_prefill(X + t * d_in, (int)(b - t < n ? b - t : n), vals, meta, s, L, R, r, d_out, d_in, Y + t * d_out, ws, status_dev, st, force_pair, automatic);
+        return rc;
+    }
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev < 0 || dev >= 64) return SLIM_ERR_CUDA;

@@ -2,7 +2,7 @@
 import pytest
 import torch
 
-from paper_2410_09615_b200 import binding as K
+from paper_2410_09615_b200 import binding as K, inputs, parity
 
 pytestmark = pytest.mark.gpu
 
@@ -29,3 +29,21 @@ def test_adapter_expansion_beyond_four_gigabytes_of_codes():
     assert torch.equal(out[-1000:], (want.float() * scales[-1000:].float()).bfloat16())
     for at in (0, rows // 2, rows - 2000):
         assert torch.equal(out[at], torch.tensor([1, 2, 1, 2, 1, 2], dtype=torch.bfloat16, device="cuda"))
+
+
+@pytest.mark.parametrize("kernel", [K.KERNEL_AUTO, K.KERNEL_PREFILL_PAIR])
+def test_more_tokens_than_the_pair_kernel_has_words_for(kernel):
+    d_in, d_out, r, b = 64, 256, 16, 31744 * 256 + 700
+    g = torch.Generator(device="cuda").manual_seed(6)
+    ly = inputs.make_layer(d_in, d_out, r, 1, 6)
+    vals, meta = K.slim_pack(torch.from_numpy(ly.codes).cuda(), torch.from_numpy(ly.mask).cuda())
+    L, R = K.bf16_from_bits(ly.L), K.bf16_from_bits(ly.R)
+    X = torch.randn((b, d_in), device="cuda", generator=g, dtype=torch.bfloat16)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    Y = K.slim_linear_fwd(X, vals, meta, ly.s, L, R, status=status, kernel=kernel)
+    assert K.read_status(status) == 0
+    half = (b // 2 + 255) // 256 * 256
+    for at in (0, half - 150, b - 300):
+        ref = K.slim_linear_fwd(X[at:at + 300], vals, meta, ly.s, L, R, kernel=K.KERNEL_SIMPLE)
+        res = parity.compare(inputs.bf16_bits_to_f64(K.bits_from_bf16(Y[at:at + 300])), inputs.bf16_bits_to_f64(K.bits_from_bf16(ref)))
+        assert res["ok"], (at, res)
