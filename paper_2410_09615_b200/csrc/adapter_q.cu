@@ -25,8 +25,7 @@ __device__ __forceinline__ uint32_t adapter_codes(const float (&v)[VALS], float 
 // store), two groups' loads in flight.  Bound by instructions: four elements a lane took the adapters of a 4096 -> 11008 layer,
 // rank 416, 13.3 + 5.8 us, this 10.3 + 5.4.
 __global__ void __launch_bounds__(256)
-pack_adapter_kernel(const __nv_bfloat16* __restrict__ A, uint32_t items, int cols, int groups,
-                    uint8_t* __restrict__ codes, __nv_bfloat16* __restrict__ scales)
+pack_adapter_kernel(const __nv_bfloat16* A, uint32_t items, int cols, int groups, uint8_t* codes, __nv_bfloat16* scales)
 {
     after_previous_grid();
     constexpr int K = 2;
@@ -40,7 +39,7 @@ pack_adapter_kernel(const __nv_bfloat16* __restrict__ A, uint32_t items, int col
         const uint32_t item = first + k;
         row[k] = item / (uint32_t)groups;
         c[k] = (int)(item - row[k] * (uint32_t)groups) * 128 + lane * 8;
-        u[k] = item < items && c[k] < cols ? __ldg(reinterpret_cast<const uint4*>(A + (size_t)row[k] * cols + c[k])) : make_uint4(0u, 0u, 0u, 0u);
+        u[k] = item < items && c[k] < cols ? *reinterpret_cast<const uint4*>(A + (size_t)row[k] * cols + c[k]) : make_uint4(0u, 0u, 0u, 0u);
     }
 #pragma unroll
     for (int k = 0; k < K; ++k) {
@@ -66,8 +65,7 @@ pack_adapter_kernel(const __nv_bfloat16* __restrict__ A, uint32_t items, int col
 
 // Any even number of columns: a warp per (row, group), four elements (two pairs) a lane.
 __global__ void __launch_bounds__(256)
-pack_adapter_pairs_kernel(const __nv_bfloat16* __restrict__ A, uint32_t items, int cols, int groups,
-                          uint8_t* __restrict__ codes, __nv_bfloat16* __restrict__ scales)
+pack_adapter_pairs_kernel(const __nv_bfloat16* A, uint32_t items, int cols, int groups, uint8_t* codes, __nv_bfloat16* scales)
 {
     after_previous_grid();
     const int lane = threadIdx.x & 31;
@@ -78,7 +76,7 @@ pack_adapter_pairs_kernel(const __nv_bfloat16* __restrict__ A, uint32_t items, i
     float v[4];
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
-        const uint32_t w = c + 2 * i < cols ? __ldg(reinterpret_cast<const uint32_t*>(A + (size_t)row * cols + c + 2 * i)) : 0u;
+        const uint32_t w = c + 2 * i < cols ? *reinterpret_cast<const uint32_t*>(A + (size_t)row * cols + c + 2 * i) : 0u;
         const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w));
         v[2 * i] = f.x; v[2 * i + 1] = f.y;
     }
@@ -112,7 +110,7 @@ unpack_adapter_kernel(const Unpack a, const Unpack b)
     const uint32_t per_row = (uint32_t)m.cols / (2 * BYTES), row = (uint32_t)(i / per_row), c = (uint32_t)(i - (I)row * per_row) * (2 * BYTES);
     const float sc = __bfloat162float(m.scales[(size_t)row * m.groups + c / 128]);
     const size_t at = (size_t)row * m.cols + c;
-    uint32_t w = BYTES == 4 ? __ldg(reinterpret_cast<const uint32_t*>(m.codes + at / 2)) : m.codes[at / 2], o[BYTES];
+    uint32_t w = BYTES == 4 ? *reinterpret_cast<const uint32_t*>(m.codes + at / 2) : m.codes[at / 2], o[BYTES];
 #pragma unroll
     for (int k = 0; k < BYTES; ++k) {
         const int lo = (int)(w << (28 - 8 * k)) >> 28, hi = (int)(w << (24 - 8 * k)) >> 28;

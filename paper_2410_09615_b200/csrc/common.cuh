@@ -36,6 +36,8 @@ struct Divisor {
 // Programmatic dependent launch for the short kernels that follow each other (compressing a 4096 x 11008 layer, 8
 // launches: 238 -> 228 us):
 // a grid is set up while the one before it in the stream ends, and starts to read and write when that one is complete.
+// What that grid may have written is read with ordinary loads behind the wait: __ldg and const __restrict__ promise data that stays
+// the same for the whole life of the grid, which begins before the wait, and such a load may be moved ahead of it.
 __device__ __forceinline__ void after_previous_grid() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

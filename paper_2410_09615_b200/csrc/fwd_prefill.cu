@@ -1103,7 +1103,7 @@ prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap t
 }
 
 // Sum of the K slices' partial tiles, scaled and rounded to bf16 (fixed order: deterministic).
-__global__ void pre_reduce_kernel(const float* __restrict__ part, int slices, size_t n, float scale, int t_parts, __nv_bfloat16* __restrict__ out)
+__global__ void pre_reduce_kernel(const float* part, int slices, size_t n, float scale, int t_parts, __nv_bfloat16* out)
 {
     // lets the main launch start, then waits for the dense-only launch whose partial tiles it adds
     asm volatile("griddepcontrol.launch_dependents;");

@@ -47,8 +47,7 @@ template <> struct Words<1> { using T = uint32_t; };
 
 template <bool XBAR, int V, int ROWS>
 __global__ void __launch_bounds__(256)
-mask_top2_kernel(const typename Words<V>::T* __restrict__ codes, const float* __restrict__ xbar, int per_row, int d_out,
-                 typename Words<V>::T* __restrict__ mask, uint32_t* status)
+mask_top2_kernel(const typename Words<V>::T* codes, const float* xbar, int per_row, int d_out, typename Words<V>::T* mask, uint32_t* status)
 {
     using T = typename Words<V>::T;
     after_previous_grid();
@@ -57,14 +56,14 @@ mask_top2_kernel(const typename Words<V>::T* __restrict__ codes, const float* __
     float4 x[V];
 #pragma unroll
     for (int v = 0; v < V && XBAR; ++v) {
-        x[v] = __ldg(reinterpret_cast<const float4*>(xbar) + (size_t)g * V + v);
+        x[v] = reinterpret_cast<const float4*>(xbar)[(size_t)g * V + v];
         if (blockIdx.y == 0 && !(x[v].x >= 0.f && x[v].x <= 3.0e38f && x[v].y >= 0.f && x[v].y <= 3.0e38f && x[v].z >= 0.f && x[v].z <= 3.0e38f && x[v].w >= 0.f && x[v].w <= 3.0e38f))
             flag_error(status, SLIM_ERR_INVALID_ARG);
     }
     for (long long row0 = (long long)blockIdx.y * ROWS * lanes + threadIdx.y; row0 < d_out; row0 += (long long)gridDim.y * ROWS * lanes) {
         T c[ROWS];
 #pragma unroll
-        for (int i = 0; i < ROWS; ++i) c[i] = __ldg(codes + (size_t)min(row0 + i * lanes, (long long)d_out - 1) * per_row + g);
+        for (int i = 0; i < ROWS; ++i) c[i] = codes[(size_t)min(row0 + i * lanes, (long long)d_out - 1) * per_row + g];
 #pragma unroll
         for (int i = 0; i < ROWS; ++i) {
             T o;

@@ -25,9 +25,7 @@ __device__ __forceinline__ uint32_t index_entry(uint32_t m) {
 }
 
 __global__ void __launch_bounds__(256)
-pack_kernel(const int8_t* __restrict__ codes, const uint8_t* __restrict__ mask,
-            long long n_chunks, uint8_t* __restrict__ vals, uint8_t* __restrict__ meta,
-            uint32_t* status_dev)
+pack_kernel(const int8_t* codes, const uint8_t* mask, long long n_chunks, uint8_t* vals, uint8_t* meta, uint32_t* status_dev)
 {
     __shared__ uint32_t table[16];
     if (threadIdx.x < 16) table[threadIdx.x] = index_entry(threadIdx.x);
@@ -36,8 +34,7 @@ pack_kernel(const int8_t* __restrict__ codes, const uint8_t* __restrict__ mask,
     uint32_t err = 0;
     for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n_chunks;
          c += (long long)gridDim.x * blockDim.x) {
-        const uint4 cv = __ldg(reinterpret_cast<const uint4*>(codes) + c);
-        const uint4 mv = __ldg(reinterpret_cast<const uint4*>(mask) + c);
+        const uint4 cv = reinterpret_cast<const uint4*>(codes)[c], mv = reinterpret_cast<const uint4*>(mask)[c];
         const uint32_t cw[4] = {cv.x, cv.y, cv.z, cv.w}, mw[4] = {mv.x, mv.y, mv.z, mv.w};
         uint32_t vout = 0, mout = 0;
 #pragma unroll

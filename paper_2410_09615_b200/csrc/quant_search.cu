@@ -4,6 +4,9 @@
 // of a candidate in binary64 with the bins added in ascending order and no fused multiply-add, the
 // codes in binary32.  Four launches: largest magnitude, histogram, search, codes.
 //
+// (The weights themselves are complete before the first launch, which is no dependent one: they are read through the read-only path;
+// what the launches hand to one another is not.)
+//
 // The three passes over the weights are bound by memory: 16-byte loads, and the histogram walks the array backwards,
 // so that it starts with what the largest-magnitude pass left in the L2 (the codes pass, forwards again, finds the
 // histogram's end there).  Measured on 4096 x 11008 (180 MB): see the figure at each kernel.
@@ -256,7 +259,7 @@ qs_search_kernel(QsHeader* hdr, const unsigned int* hist, int bins, double n_tot
             const int i0 = (first + warp) * 256 + lane * 8;
             unsigned int c[8];
             if (i0 + 8 <= bins) {
-                const uint4 lo = __ldg(reinterpret_cast<const uint4*>(hist + i0)), hi = __ldg(reinterpret_cast<const uint4*>(hist + i0) + 1);
+                const uint4 lo = reinterpret_cast<const uint4*>(hist + i0)[0], hi = reinterpret_cast<const uint4*>(hist + i0)[1];
                 c[0] = lo.x; c[1] = lo.y; c[2] = lo.z; c[3] = lo.w; c[4] = hi.x; c[5] = hi.y; c[6] = hi.z; c[7] = hi.w;
             } else {
 #pragma unroll
@@ -374,7 +377,7 @@ qs_search_kernel(QsHeader* hdr, const unsigned int* hist, int bins, double n_tot
 
 // 16 codes a thread: four float4 loads, one 16-byte store.
 __global__ void __launch_bounds__(256)
-qs_codes_kernel(const float* __restrict__ W, size_t n, const float* __restrict__ scale_alpha, int8_t* __restrict__ codes)
+qs_codes_kernel(const float* __restrict__ W, size_t n, const float* scale_alpha, int8_t* codes)
 {
     after_previous_grid();
     const float a32 = scale_alpha[1];
