@@ -52,6 +52,7 @@
 #include <atomic>
 #include <cuda.h>
 #include "common.cuh"
+#include "handover.h"
 
 namespace slim {
 
@@ -667,30 +668,16 @@ template <int N> struct PairCfg {
 };
 constexpr size_t kSyncTiles = kSmallTBytes / 16 - 1024;     // T' tiles whose words fit the region beside those of the pairs
 
-// The list of T' stages (tile after tile) dealt out to the pairs.
-__host__ __device__ __forceinline__ int share_begin(int q, int units, int pairs) { return (int)((long long)q * units / pairs); }
-__host__ __device__ __forceinline__ int share_owner(int unit, int units, int pairs) { return (int)(((long long)(unit + 1) * pairs - 1) / units); }
-// A share's run inside one tile, from `unit` on.
-struct Run { int tile, k0, len; };
-__device__ __forceinline__ Run run_at(int unit, int end, int stages) {
-    Run r;
-    r.tile = unit / stages; r.k0 = unit - r.tile * stages; r.len = min(stages - r.k0, end - unit);
-    return r;
-}
 __device__ __forceinline__ unsigned long long ld_acquire64(const unsigned long long* p) {
     unsigned long long v;
     asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
     return v;
 }
-// Hand-over words: a word's high half is the number of the call that set it, so nothing is cleared between calls.  A
-// pair's part of a tile has two (part written; its share of the sums written), for each of its CTAs; so has a tile made whole (the second alone).
-__device__ __forceinline__ size_t part_word(int q, bool starts, uint32_t rank) { return ((size_t)(2 * q + (starts ? 1 : 0)) * 2 + rank) * 2; }
-__device__ __forceinline__ size_t tile_word(const PrefillParams& p, int tile, uint32_t rank) { return (size_t)p.t_pairs * 8 + (size_t)tile * 2 + rank; }
 // Waits (bounded in time) until every lane's word (nullptr: none) is this call's; called by a whole warp.
 __device__ __forceinline__ bool wait_words(const unsigned long long* w, uint32_t call, volatile uint32_t* abort_flag) {
     unsigned long long t0 = 0;
     for (uint32_t it = 0;; ++it) {
-        const bool there = !w || (uint32_t)(ld_acquire64(w) >> 32) == call;
+        const bool there = !w || is_of(ld_acquire64(w), call);
         if (__all_sync(0xffffffffu, there)) return true;
         if (__any_sync(0xffffffffu, *abort_flag != 0)) return false;
         if ((it & 63u) == 63u) {
@@ -767,7 +754,7 @@ prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap t
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("fence.proxy.async;" ::: "memory");            // what that grid wrote is read through TMA
-    const uint32_t call = p.r > 0 ? (uint32_t)(*(volatile unsigned long long*)p.departures >> 16) + 1u : 0u;
+    const uint32_t call = p.r > 0 ? call_number(*(volatile unsigned long long*)p.departures) : 0u;
     bool ok = true;
     // Tile -> its first row in this CTA, its first token, and where its walk over the weight columns starts: pairs that share
     // token rows start at different places, so that at any moment they ask the L2 for different lines of X.
@@ -818,7 +805,7 @@ prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap t
                             left = -first - 32;
                             for (int c = 0; c < p.t_chunks; ++c) {
                                 const int q0 = share_owner((tile0 + c) * p.t_stages, t_units, p.t_pairs), q1 = share_owner((tile0 + c + 1) * p.t_stages - 1, t_units, p.t_pairs);
-                                if (i >= 0 && i <= q1 - q0) w = p.t_sync + (q0 == q1 ? tile_word(p, tile0 + c, t_half) : part_word(q0 + i, i == 0, t_half) + 1);
+                                if (i >= 0 && i <= q1 - q0) w = p.t_sync + (q0 == q1 ? tile_word(p.t_pairs, tile0 + c, t_half) : part_word(q0 + i, i == 0, t_half) + 1);
                                 i -= q1 - q0 + 1; left += q1 - q0 + 1;
                             }
                             ok = wait_words(w, call, abort_flag) && ok;
@@ -979,7 +966,7 @@ prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap t
             epilogue_sync();
             if (threadIdx.x == kConvWarps * 32) {
                 __threadfence();
-                *(volatile unsigned long long*)(p.t_sync + word) = (unsigned long long)call << 32;
+                *(volatile unsigned long long*)(p.t_sync + word) = tagged(call, 0);
             }
         };
         // all of this pair's runs first (nothing here waits for another pair), every second group of 16 columns a thread
@@ -1003,7 +990,7 @@ prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap t
             fence_before_sync();
             __syncwarp();
             if (lane == 0) mbar_arrive_remote_release(peer_addr(acc_empty, 0));
-            publish(whole ? tile_word(p, run.tile, rank) : part_word(tq, run.k0 == 0, rank));
+            publish(whole ? tile_word(p.t_pairs, run.tile, rank) : part_word(tq, run.k0 == 0, rank));
         }
         // then its share of the sums: when every part of a tile is there, columns c4 = .. (mod 2 n) for each of its n pairs
         for (int u = t_begin; u < t_end;) {
@@ -1098,8 +1085,7 @@ prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap t
         fence_after_sync();
         asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" :: "r"(tmem_base), "r"(512) : "memory");
     }
-    // a call adds 1 << 16 to the counter in all
-    if (threadIdx.x == 0) atomicAdd(p.departures, blockIdx.x == 0 ? 65536ull - (gridDim.x - 1) : 1ull);
+    if (threadIdx.x == 0) atomicAdd(p.departures, departure(blockIdx.x, gridDim.x));
 }
 
 // Sum of the K slices' partial tiles, scaled and rounded to bf16 (fixed order: deterministic).

@@ -32,7 +32,7 @@
 //
 // The hand-over of T is the only wait between clusters.  It goes from lower to higher cluster numbers only:
 // clusters that make T wait for nobody and are started first, so the wait ends whether or not the whole grid is
-// resident.  Every poll is bounded in time.  An entry carries the number of the call that wrote it, so
+// resident.  Every poll is bounded in time, and the first to run out ends all others of the call.  An entry carries the number of the call that wrote it, so
 // nothing has to be cleared between calls; the call number is (departures >> 16) + 1, and every call adds
 // 1 << 16 to that counter in all.
 // Reductions have a fixed order: results are bit-identical from run to run.
@@ -40,6 +40,7 @@
 #include <mutex>
 #include <cuda.h>
 #include "decode_tile.cuh"
+#include "handover.h"
 
 namespace slim {
 
@@ -119,9 +120,30 @@ __device__ __forceinline__ unsigned long long now_ns() {
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
     return t;
 }
+// An entry of T is one 64-bit access: value and call number are seen together.
+__device__ __forceinline__ unsigned long long ld_gpu64(const unsigned long long* p) {
+    unsigned long long v;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_gpu64(unsigned long long* p, unsigned long long v) {
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" :: "l"(p), "l"(v) : "memory");
+}
+// Whether a wait that began at *t0 (0: it starts now) is to be given up: it has taken kWaitNs, or another wait of this call, in whatever
+// CTA, has.  The first to expire leaves the call's number in the word behind the departures, so a broken call costs one such
+// time, not one a step and CTA (3072 ranks in one CTA: 96 steps to wait for).
+__device__ __forceinline__ bool give_up(unsigned long long* sync, unsigned long long* t0) {
+    const unsigned long long now = now_ns();
+    if (*t0 == 0) *t0 = now;
+    const uint32_t call = call_number(ld_gpu64(sync));
+    if (is_of(ld_gpu64(sync + 1), call)) return true;
+    if (now - *t0 <= kWaitNs) return false;
+    st_gpu64(sync + 1, tagged(call, 0));
+    return true;
+}
 // Waits for a phase, for kWaitNs at most (a try may suspend the thread, so the bound is on time).
 template <bool CLUSTER = false>
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, unsigned long long* sync) {
     unsigned long long t0 = 0;
     for (uint32_t it = 0;; ++it) {
         uint32_t done;
@@ -132,11 +154,7 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
             asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
                          : "=r"(done) : "r"(bar), "r"(parity) : "memory");
         if (done) return true;
-        if ((it & 63u) == 63u) {
-            const unsigned long long now = now_ns();
-            if (t0 == 0) t0 = now;
-            else if (now - t0 > kWaitNs) return false;
-        }
+        if ((it & 63u) == 63u && give_up(sync, &t0)) return false;
     }
 }
 __device__ __forceinline__ void tma_tile(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar) {
@@ -174,18 +192,9 @@ __device__ __forceinline__ float4 lds_f4(uint32_t addr) { float4 v; asm volatile
 __device__ __forceinline__ uint2 lds64(uint32_t addr) {
     return *reinterpret_cast<const uint2*>(__cvta_shared_to_generic(addr));
 }
-// An entry of T is one 64-bit access: value and call number are seen together.
-__device__ __forceinline__ unsigned long long ld_gpu64(const unsigned long long* p) {
-    unsigned long long v;
-    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-    return v;
-}
 // Two entries, each seen whole (the vector form is two 64-bit accesses).
 __device__ __forceinline__ void ld_gpu64x2(const unsigned long long* p, unsigned long long& x, unsigned long long& y) {
     asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(x), "=l"(y) : "l"(p) : "memory");
-}
-__device__ __forceinline__ void st_gpu64(unsigned long long* p, unsigned long long v) {
-    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" :: "l"(p), "l"(v) : "memory");
 }
 __device__ __forceinline__ void ldsm4(uint32_t addr, uint4& v) {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
@@ -377,23 +386,19 @@ __device__ __forceinline__ void adapter_stage_q(float (&acc)[NT][4], uint32_t st
 // wait for the same words, and with every lane polling its own (1024 warps on a few lines of the L2) the words
 // themselves came 1-3 us later (2048 -> 2048, rank 208, 6 tokens: 6.8 us a call instead of 7.5).
 template <int NE, typename A, typename W>
-__device__ __forceinline__ bool wait_words(unsigned long long (&v)[NE], uint32_t call, A ask, W word)
+__device__ __forceinline__ bool wait_words(unsigned long long (&v)[NE], uint32_t call, unsigned long long* sync, A ask, W word)
 {
     for (int round = 0; round < 64; ++round) {
         const unsigned long long* w = nullptr;
 #pragma unroll
-        for (int n = 0; n < NE; ++n) if (!w && (uint32_t)(v[n] >> 32) != call) w = word(n);
+        for (int n = 0; n < NE; ++n) if (!w && !is_of(v[n], call)) w = word(n);
         const uint32_t missing = __ballot_sync(0xffffffffu, w != nullptr);
         if (!missing) return true;
         bool late = false;
         if ((int)(threadIdx.x & 31) == __ffs(missing) - 1) {
             unsigned long long t0 = 0;
-            for (uint32_t spin = 0; !late && (uint32_t)(ld_gpu64(w) >> 32) != call; ++spin) {
-                if ((spin & 63u) == 63u) {
-                    const unsigned long long now = now_ns();
-                    if (t0 == 0) t0 = now;
-                    else late = now - t0 > kWaitNs;
-                }
+            for (uint32_t spin = 0; !late && !is_of(ld_gpu64(w), call); ++spin) {
+                if ((spin & 63u) == 63u) late = give_up(sync, &t0);
                 __nanosleep(20);
             }
         }
@@ -523,7 +528,7 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
     int p_it = 0;                                              // producers: next stage
     auto acquire = [&]() -> int {
         const int st = p_it % kStages, use = p_it / kStages;
-        if (use > 0) ok = mbar_wait(empty + 8 * st, (use - 1) & 1) && ok;
+        if (use > 0) ok = mbar_wait(empty + 8 * st, (use - 1) & 1, p.departures) && ok;
         ++p_it;
         return st;
     };
@@ -598,9 +603,9 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
                 if (FMT == FMT_PACKED_LD) mbar_arrive(bar);
             }
             // this CTA's share of the piece, once every CTA of the cluster has sent its sums
-            const uint32_t call = (uint32_t)(ld_gpu64(p.departures) >> 16) + 1u;
+            const uint32_t call = call_number(ld_gpu64(p.departures));
             const int per = 16 >> logC;                        // column pairs of a token that this CTA adds up
-            ok = mbar_wait<true>(piece_bar, 0) && ok;
+            ok = mbar_wait<true>(piece_bar, 0, p.departures) && ok;
             for (int e = lane; e < p.b * per; e += 32) {
                 const int tok = e / per, j = piece * kGroup + 2 * ((int)rank * per + e % per);
                 float2 s = lds_f2(recv + e * 8);
@@ -616,7 +621,7 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
                         __nv_bfloat162 pr = TP == 1    ? __floats2bfloat162_rn(s.x, s.y)
                                             : part == 0 ? __floats2bfloat162_rn(bf16_head(s.x), bf16_head(s.y))
                                                         : __floats2bfloat162_rn(bf16_tail(s.x), bf16_tail(s.y));
-                        st_gpu64(p.T + part * t_tail + (size_t)tok * (p.r / 2) + (j >> 1), ((unsigned long long)call << 32) | *reinterpret_cast<uint32_t*>(&pr));
+                        st_gpu64(p.T + part * t_tail + (size_t)tok * (p.r / 2) + (j >> 1), tagged(call, *reinterpret_cast<uint32_t*>(&pr)));
                     }
             }
         } else {
@@ -653,7 +658,7 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
         // ============================ T into shared memory, step by step ============================
         // [token][32 columns] bf16, 64-byte rows stored with the 64-byte swizzle; each of the two warps half of the tokens
         if (!makes_T && p.r > 0) {
-            const uint32_t call = (uint32_t)(ld_gpu64(p.departures) >> 16) + 1u;
+            const uint32_t call = call_number(ld_gpu64(p.departures));
             constexpr int kPer = NT * 2;                       // words a lane fetches
             const int steps = (l_chunks - (int)rank + (int)C - 1) / (int)C * (QA ? 2 : 1);
             for (int it = 0; it < steps; ++it) {
@@ -666,15 +671,15 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
 #pragma unroll
                     for (int n = 0; n < TP * kPer; ++n) {
                         const int i = n % kPer;
-                        v[n] = 2 * i < toks ? ld_gpu64(at + (n / kPer) * t_tail + i * p.r) : (unsigned long long)call << 32;
+                        v[n] = 2 * i < toks ? ld_gpu64(at + (n / kPer) * t_tail + i * p.r) : tagged(call, 0);
                     }
                 };
                 ask();
-                ok = wait_words(v, call, ask, [&](int n) { return at + (n / kPer) * t_tail + (n % kPer) * p.r; }) && ok;
+                ok = wait_words(v, call, p.departures, ask, [&](int n) { return at + (n / kPer) * t_tail + (n % kPer) * p.r; }) && ok;
 #pragma unroll
                 for (int tp = 0; tp < TP; ++tp) {
                     const int slot = it * TP + tp, st = slot % C_::kTSlots, use = slot / C_::kTSlots;
-                    if (use > 0) ok = mbar_wait(t_empty + 8 * st, (use - 1) & 1) && ok;
+                    if (use > 0) ok = mbar_wait(t_empty + 8 * st, (use - 1) & 1, p.departures) && ok;
 #pragma unroll
                     for (int i = 0; i < kPer; ++i) {
                         const int tok = tok0 + 2 * i;
@@ -689,11 +694,11 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
     } else {
         // ============================ consumer warps ============================
         uint32_t call = 0;
-        if (p.r > 0) call = (uint32_t)(ld_gpu64(p.departures) >> 16) + 1u;
+        if (p.r > 0) call = call_number(ld_gpu64(p.departures));
         int it = 0;
         auto wait_stage = [&]() -> uint32_t {
             const int st = it % kStages;
-            ok = mbar_wait(full + 8 * st, (it / kStages) & 1) && ok;
+            ok = mbar_wait(full + 8 * st, (it / kStages) & 1, p.departures) && ok;
             return smem + st * kStage;
         };
         auto release = [&]() {
@@ -808,7 +813,7 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
                         for (int ht = 0; ht < 2 * TP; ++ht, ++lt) {             // steps, T's parts inside them
                             const int h = ht / TP, ts = lt % C_::kTSlots;
                             const uint32_t tslot = part + ts * C_::kTSlot;
-                            ok = mbar_wait(t_full + 8 * ts, (lt / C_::kTSlots) & 1) && ok;
+                            ok = mbar_wait(t_full + 8 * ts, (lt / C_::kTSlots) & 1, p.departures) && ok;
                             if (mts > 0 && 2 * lc + h < l_steps) {
                                 uint4 tb[kNW];
 #pragma unroll
@@ -826,7 +831,7 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
                     for (int tp = 0; tp < TP; ++tp, ++lt) {
                         const int ls = lc, ts = lt % C_::kTSlots;
                         const uint32_t tslot = part + ts * C_::kTSlot;
-                        ok = mbar_wait(t_full + 8 * ts, (lt / C_::kTSlots) & 1) && ok;
+                        ok = mbar_wait(t_full + 8 * ts, (lt / C_::kTSlots) & 1, p.departures) && ok;
                         if (mts > 0) {
                             const int mat = lane >> 3, r8 = lane & 7;
 #pragma unroll
@@ -866,11 +871,11 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
                 auto ask = [&](int ls) {
 #pragma unroll
                     for (int q = 0; q < TP * kWords; ++q)
-                        v[q] = (q % kWords >> 1) * 8 + ln.g < p.b && ls * 32 + 16 * kk < p.r ? ld_gpu64(word(ls, q)) : (unsigned long long)call << 32;
+                        v[q] = (q % kWords >> 1) * 8 + ln.g < p.b && ls * 32 + 16 * kk < p.r ? ld_gpu64(word(ls, q)) : tagged(call, 0);
                 };
                 ask((int)rank);
                 for (int ls = (int)rank; ls < l_steps; ls += (int)C) {
-                    ok = wait_words(v, call, [&] { ask(ls); }, [&](int q) { return word(ls, q); }) && ok;
+                    ok = wait_words(v, call, p.departures, [&] { ask(ls); }, [&](int q) { return word(ls, q); }) && ok;
                     uint32_t tb[TP * kWords];
 #pragma unroll
                     for (int q = 0; q < TP * kWords; ++q) tb[q] = (uint32_t)v[q];
@@ -905,7 +910,7 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
                 auto ask = [&](int ls) {
 #pragma unroll
                     for (int q = 0; q < TP * kWords; q += 2) {
-                        v[q] = v[q + 1] = (unsigned long long)call << 32;
+                        v[q] = v[q + 1] = tagged(call, 0);
                         // r is a multiple of 16: a thread's 8 columns exist or not
                         if (ls * 32 + 8 * ln.t < p.r && (q % kWords >> 2) * 8 + ln.g < p.b) ld_gpu64x2(word(ls, q), v[q], v[q + 1]);
                     }
@@ -919,7 +924,7 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
                 ask(2 * (int)rank + kk);
                 for (int lc = (int)rank; lc < l_chunks; lc += (int)C) {
                     const int ls = 2 * lc + kk;
-                    ok = wait_words(v, call, [&] { ask(ls); }, [&](int q) { return word(ls, q); }) && ok;
+                    ok = wait_words(v, call, p.departures, [&] { ask(ls); }, [&](int q) { return word(ls, q); }) && ok;
                     uint4 tb[TP][kNW];
 #pragma unroll
                     for (int q = 0; q < TP * kNW; ++q)
@@ -951,10 +956,10 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
             consumer_sync();
             if (NT == 8) {                                     // the receivers' ring is free
                 if (warp == 0 && lane < (int)C) mbar_arrive_peer(peer(gone, lane));
-                ok = mbar_wait<true>(gone, 0) && ok;
+                ok = mbar_wait<true>(gone, 0, p.departures) && ok;
             }
             send<NT, MT>(p, smem, red_full, logC, (int)rank);
-            ok = mbar_wait<true>(red_full, 0) && ok;
+            ok = mbar_wait<true>(red_full, 0, p.departures) && ok;
             finish<NT, MT>(p, smem, tile, logC, (int)rank);
         }
     }
@@ -963,7 +968,7 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
     // nobody leaves while a peer may still read its shared memory (the reads are over: no memory ordering is asked for)
     asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
     cluster_wait();
-    if (threadIdx.x == 0) atomicAdd(p.departures, blockIdx.x == 0 ? 65536ull - (gridDim.x - 1) : 1ull);
+    if (threadIdx.x == 0) atomicAdd(p.departures, departure(blockIdx.x, gridDim.x));
 }
 
 // ------------------------------------------------------------------ host side

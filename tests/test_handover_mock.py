@@ -1,10 +1,10 @@
-"""The workspace hand-over protocol of the decode kernels, run by CPU threads (tests/handover_mock.cpp).
+"""The hand-over protocols of the kernels, run by CPU threads (tests/handover_mock.cpp) over the kernels' own word arithmetic
+(csrc/handover.h).
 
-Slots hold 0xFFFFFFFF while empty and their one reader empties them again; T entries carry the call
-number taken from the departure counter; every poll is bounded.  The cases below run the protocol
-over many calls on one workspace, and make a bounded wait expire by withholding one writer: the
-status word gets the time-out bit, every CTA still leaves, the departure counter still advances,
-and after the reset the interface asks for the next call is clean.  Nothing here touches a GPU."""
+Words carry the number of the call that wrote them, taken from a counter to which every call adds 1 << 16 in all, so small batches,
+CTA pairs with adapters and CTA pairs without take turns on one workspace and nothing is cleared.  A bounded wait that runs out
+(one writer is withheld) sets the time-out bit, every CTA still leaves, and the call costs one time-out, not one for every
+word; after the reset the interface asks for the next call is clean.  Nothing here touches a GPU."""
 import os
 import re
 import subprocess
@@ -12,47 +12,72 @@ import subprocess
 import pytest
 
 HERE = os.path.dirname(os.path.abspath(__file__))
+CSRC = os.path.join(os.path.dirname(HERE), "paper_2410_09615_b200", "csrc")
 TIMEOUT_BIT = 1 << 7
-LINE = re.compile(r"call (\d+) status (\d+) departures (\d+) wrong (\d+) left (\d+)")
+LINE = re.compile(r"call (\d+) kind (\d) status (\d+) number (\d+) departures (\d+) wrong (\d+) expired (\d+)")
 
 
 @pytest.fixture(scope="module")
 def mock(tmp_path_factory):
     exe = str(tmp_path_factory.mktemp("mock") / "handover_mock")
-    subprocess.run(["g++", "-O2", "-std=c++17", "-pthread", os.path.join(HERE, "handover_mock.cpp"), "-o", exe], check=True)
+    subprocess.run(["g++", "-O2", "-std=c++17", "-Wall", "-Werror", "-pthread", os.path.join(HERE, "handover_mock.cpp"), "-o", exe], check=True)
     return exe
 
 
-def run(exe, n_ctas, n_units, calls, withhold, poll_limit):
-    out = subprocess.run([exe, str(n_ctas), str(n_units), str(calls), str(withhold), str(poll_limit)],
-                         check=True, capture_output=True, text=True, timeout=120).stdout.splitlines()
-    rows = [tuple(int(x) for x in LINE.match(l).groups()) for l in out if l.startswith("call")]
-    return rows, out
+def run(exe, *args):
+    out = subprocess.run([exe, *[str(a) for a in args]], check=True, capture_output=True, text=True, timeout=120).stdout.splitlines()
+    return [tuple(int(x) for x in LINE.match(l).groups()) for l in out if l.startswith("call")], out
 
 
-@pytest.mark.parametrize("n_ctas,n_units", [(1, 5), (4, 4), (6, 37), (8, 3)])
-def test_many_calls_share_one_workspace(mock, n_ctas, n_units):
-    rows, _ = run(mock, n_ctas, n_units, 25, 0, 1 << 26)
-    assert len(rows) == 25
-    for k, (call, status, departures, wrong, left) in enumerate(rows, 1):
-        assert call == k and status == 0
-        assert departures == k * n_ctas           # every CTA left, once per call
-        assert wrong == 0                         # every fetched entry was this call's sum, added in list order
-        assert left == 0                          # the readers emptied every slot
+def test_shares_cover_the_list_and_their_words_never_meet(mock):
+    _, out = run(mock, "shares")
+    assert out[0].startswith("shares ")
 
 
-def test_a_wait_that_runs_out_sets_the_status_and_nobody_stays_behind(mock):
-    n_ctas, n_units = 5, 11
-    rows, out = run(mock, n_ctas, n_units, 6, 3, 2000)
-    assert len(rows) == 6
-    for call, status, departures, wrong, left in rows[:2]:
-        assert status == 0 and wrong == 0 and left == 0 and departures == call * n_ctas
-    call, status, departures, wrong, left = rows[2]
-    assert status & TIMEOUT_BIT                   # the bounded poll gave up
-    assert (status >> 16) & 64                    # ... and says it was waiting for partials of T
-    assert departures == 3 * n_ctas               # the call still ended: every CTA left
-    assert wrong > 0                              # its result is not to be used
-    assert out[out.index(f"call 3 status {status} departures {departures} wrong {wrong} left {left}") + 1] == "reset"
-    for k, (call, status, departures, wrong, left) in enumerate(rows[3:], 1):
-        assert status == 0 and wrong == 0 and left == 0
-        assert departures == k * n_ctas           # counted from the reset
+@pytest.mark.parametrize("ctas,makers,words,pairs,t_pairs,tiles,stages", [
+    (2, 1, 5, 1, 1, 1, 1),
+    (8, 3, 40, 6, 5, 4, 7),           # parts of tiles and whole tiles in one list
+    (12, 4, 16, 8, 8, 2, 27),         # every tile in four parts
+    (5, 2, 90, 4, 2, 6, 3),           # whole tiles only
+    (9, 1, 33, 7, 7, 3, 5),           # parts that end and start inside tiles
+])
+def test_kernels_take_turns_on_one_workspace(mock, ctas, makers, words, pairs, t_pairs, tiles, stages):
+    rows, _ = run(mock, ctas, makers, words, pairs, t_pairs, tiles, stages, 24, 0, 1 << 26)
+    assert len(rows) == 24
+    for k, (call, kind, status, number, departures, wrong, expired) in enumerate(rows, 1):
+        assert call == k and number == k and status == 0
+        assert departures == k << 16              # whatever the kind and the number of CTAs
+        assert wrong == 0 and expired == 0        # every word and sum fetched was this call's
+
+
+@pytest.mark.parametrize("withhold", [1, 2, 4, 5])
+def test_a_wait_that_runs_out_costs_one_time_out_and_nobody_stays_behind(mock, withhold):
+    ctas, makers, words, pairs = 6, 2, 64, 4
+    rows, out = run(mock, ctas, makers, words, pairs, 4, 3, 5, 9, withhold, 20000)
+    assert len(rows) == 9
+    since = 0
+    for call, kind, status, number, departures, wrong, expired in rows:
+        since += 1
+        assert departures == since << 16 and number == since                # every CTA left, also from the broken call
+        if call == withhold:
+            assert status & TIMEOUT_BIT and wrong > 0
+            # small batches: CTAs that wait at the same time may run out together, but none twice (32 words are missing);
+            # pairs: once a CTA
+            assert 1 <= expired <= (ctas - makers if kind == 0 else 2 * pairs)
+            at = next(i for i, l in enumerate(out) if l.startswith(f"call {call} "))
+            assert out[at + 1] == "reset"
+            since = 0                                                       # counted from the reset
+        else:
+            assert status == 0 and wrong == 0 and expired == 0
+
+
+def test_every_wait_of_the_small_batch_kernel_can_be_ended_by_another():
+    """The loops of its waits ask, now and then, whether the call has been given up (its CTAs would else each wait their full time
+    for every step of a T that never comes)."""
+    text = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, "fwd_small.cu")).read())
+    for wait in ("mbar_wait", "wait_words"):
+        body = text[text.index(f"bool {wait}("):]
+        assert "give_up(" in body[:body.index("\n}\n")], wait
+    give_up = text[text.index("bool give_up("):]
+    give_up = give_up[:give_up.index("\n}\n")]
+    assert "is_of(ld_gpu64(sync + 1), call)" in give_up and "st_gpu64(sync + 1" in give_up
