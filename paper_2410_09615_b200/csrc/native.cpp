@@ -114,6 +114,16 @@ bool adapters(PyObject* oL, PyObject* oR, int64_t d_out, int64_t d_in, void** L,
     return true;
 }
 
+// A call into the library, with the interpreter free for other threads: a launch waits where the stream's queue is full.
+template <typename F, typename... A>
+int unlocked(F f, A... args) {
+    int rc;
+    Py_BEGIN_ALLOW_THREADS
+    rc = f(args...);
+    Py_END_ALLOW_THREADS
+    return rc;
+}
+
 // linear_fwd(X, vals, meta, s, L, R, Y, workspace, status, kernel)
 PyObject* linear_fwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
     HANDLE_TH_ERRORS
@@ -136,12 +146,8 @@ PyObject* linear_fwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
     PyObject* y = output(a[6], b, d_out, *X, &Y);
     if (!y) return nullptr;
     void* stream = c10::cuda::getCurrentCUDAStream().stream();
-    const void *xp = X->data_ptr(), *vp = v->data_ptr(), *mp = m->data_ptr();
-    int rc;
-    Py_BEGIN_ALLOW_THREADS
-    rc = g_fwd(xp, (int)b, (const uint8_t*)vp, (const uint8_t*)mp, (float)s, L, R, (int)r, (int)d_out, (int)d_in, Y, ws, ws_bytes,
-               (uint32_t*)status, stream, (int)kernel);
-    Py_END_ALLOW_THREADS
+    const int rc = unlocked(g_fwd, X->data_ptr(), (int)b, (const uint8_t*)v->data_ptr(), (const uint8_t*)m->data_ptr(), (float)s, L, R, (int)r,
+                            (int)d_out, (int)d_in, Y, ws, ws_bytes, (uint32_t*)status, stream, (int)kernel);
     return finish(rc, y, "slim_linear_fwd");
     END_HANDLE_TH_ERRORS
 }
@@ -169,11 +175,8 @@ PyObject* linear_fwd_tiled(PyObject*, PyObject* const* a, Py_ssize_t n) {
     PyObject* y = output(a[6], b, d_out, *X, &Y);
     if (!y) return nullptr;
     void* stream = c10::cuda::getCurrentCUDAStream().stream();
-    const void *xp = X->data_ptr(), *tp = t->data_ptr();
-    int rc;
-    Py_BEGIN_ALLOW_THREADS
-    rc = g_tiled(xp, (int)b, tp, (int)layout, (float)s, L, R, (int)r, (int)d_out, (int)d_in, Y, ws, ws_bytes, (uint32_t*)status, stream);
-    Py_END_ALLOW_THREADS
+    const int rc = unlocked(g_tiled, X->data_ptr(), (int)b, t->data_ptr(), (int)layout, (float)s, L, R, (int)r, (int)d_out, (int)d_in, Y, ws,
+                            ws_bytes, (uint32_t*)status, stream);
     return finish(rc, y, "slim_linear_fwd_tiled");
     END_HANDLE_TH_ERRORS
 }
@@ -199,13 +202,9 @@ PyObject* linear_fwd_q(PyObject*, PyObject* const* a, Py_ssize_t n) {
     PyObject* y = output(a[8], b, d_out, *X, &Y);
     if (!y) return nullptr;
     void* stream = c10::cuda::getCurrentCUDAStream().stream();
-    const void *xp = X->data_ptr(), *vp = v->data_ptr(), *mp = m->data_ptr(), *lqp = Lq->data_ptr(), *lsp = Ls->data_ptr(),
-               *rqp = Rq->data_ptr(), *rsp = Rs->data_ptr();
-    int rc;
-    Py_BEGIN_ALLOW_THREADS
-    rc = g_q(xp, (int)b, (const uint8_t*)vp, (const uint8_t*)mp, (float)s, (const uint8_t*)lqp, lsp, (const uint8_t*)rqp, rsp, (int)r,
-             (int)d_out, (int)d_in, Y, ws, ws_bytes, (uint32_t*)status, stream);
-    Py_END_ALLOW_THREADS
+    const int rc = unlocked(g_q, X->data_ptr(), (int)b, (const uint8_t*)v->data_ptr(), (const uint8_t*)m->data_ptr(), (float)s,
+                            (const uint8_t*)Lq->data_ptr(), Ls->data_ptr(), (const uint8_t*)Rq->data_ptr(), Rs->data_ptr(), (int)r, (int)d_out,
+                            (int)d_in, Y, ws, ws_bytes, (uint32_t*)status, stream);
     return finish(rc, y, "slim_linear_fwd_q");
     END_HANDLE_TH_ERRORS
 }
@@ -294,8 +293,8 @@ PyObject* mask_top2(PyObject*, PyObject* const* a, Py_ssize_t n) {
     void* status;
     if (!address(a[2], "status", &status)) return nullptr;
     at::Tensor mask = fresh(c->sizes(), at::kByte, *c);
-    const int rc = g_mask((const int8_t*)c->data_ptr(), x ? (const float*)x->data_ptr() : nullptr, (int)c->size(0), (int)c->size(1),
-                          (uint8_t*)mask.data_ptr(), (uint32_t*)status, c10::cuda::getCurrentCUDAStream().stream());
+    const int rc = unlocked(g_mask, (const int8_t*)c->data_ptr(), x ? (const float*)x->data_ptr() : nullptr, (int)c->size(0), (int)c->size(1),
+                            (uint8_t*)mask.data_ptr(), (uint32_t*)status, c10::cuda::getCurrentCUDAStream().stream());
     return rc == 0 ? THPVariable_Wrap(std::move(mask)) : finish(rc, nullptr, "slim_mask_top2");
     END_HANDLE_TH_ERRORS
 }
@@ -309,8 +308,8 @@ PyObject* pack_adapter(PyObject*, PyObject* const* a, Py_ssize_t n) {
     const int64_t rows = A->size(0), cols = A->size(1);
     if (rows < 1 || cols < 2 || cols % 2 != 0) return finish(1, nullptr, "slim_pack_adapter");      // SLIM_ERR_INVALID_ARG
     at::Tensor codes = fresh({rows, cols / 2}, at::kByte, *A), scales = fresh({rows, (cols + 127) / 128}, at::kBFloat16, *A);
-    const int rc = g_pack_adapter(A->data_ptr(), (int)rows, (int)cols, (uint8_t*)codes.data_ptr(), scales.data_ptr(),
-                                  c10::cuda::getCurrentCUDAStream().stream());
+    const int rc = unlocked(g_pack_adapter, A->data_ptr(), (int)rows, (int)cols, (uint8_t*)codes.data_ptr(), scales.data_ptr(),
+                            c10::cuda::getCurrentCUDAStream().stream());
     if (rc != 0) return finish(rc, nullptr, "slim_pack_adapter");
     return Py_BuildValue("(NN)", THPVariable_Wrap(std::move(codes)), THPVariable_Wrap(std::move(scales)));
     END_HANDLE_TH_ERRORS
@@ -327,8 +326,8 @@ PyObject* quant(PyObject*, PyObject* const* a, Py_ssize_t n) {
     const int64_t d_out = W->size(0), d_in = W->size(1);
     const size_t bytes = g_quant_bytes((int)d_out, (int)d_in);
     at::Tensor ws = fresh({(int64_t)bytes}, at::kByte, *W), codes = fresh({d_out, d_in}, at::kChar, *W), sa = fresh({4}, at::kFloat, *W);
-    const int rc = g_quant((const float*)W->data_ptr(), (int)d_out, (int)d_in, (int8_t*)codes.data_ptr(), (float*)sa.data_ptr(),
-                           ws.data_ptr(), bytes, (uint32_t*)status, c10::cuda::getCurrentCUDAStream().stream());
+    const int rc = unlocked(g_quant, (const float*)W->data_ptr(), (int)d_out, (int)d_in, (int8_t*)codes.data_ptr(), (float*)sa.data_ptr(),
+                            ws.data_ptr(), bytes, (uint32_t*)status, c10::cuda::getCurrentCUDAStream().stream());
     if (rc != 0) return finish(rc, nullptr, "slim_quant");
     const int64_t bins = std::max<int64_t>(512, std::min<int64_t>(d_out * d_in / 1000, 20000)), at_ = 256 + (bins * 4 + 255) / 256 * 256;
     at::Tensor tab = ws.slice(0, at_, at_ + 59 * 8).view(at::kDouble);
