@@ -319,7 +319,7 @@ slim_status_t slim_linear_fwd_q(const void* X, int b, const uint8_t* vals, const
  * Every GPU that loads the library holds that array until the process exits.
  *
  * Same operation, arguments and rounding as slim_linear_fwd, for b <= 16 and the
- * shapes with d_in % 256 == 0, d_in <= 32768; other problems return
+ * shapes with d_in % 256 == 0, d_in <= 32768, r <= 3072 (2560 from 9 tokens on); other problems return
  * SLIM_ERR_UNSUPPORTED_SHAPE, and a problem whose scratch would exceed the
  * array returns SLIM_ERR_WORKSPACE (all LLaMA-2 7B/13B/70B layer shapes fit).
  * The call makes no cudaMalloc / cudaFree and uses no allocating library
@@ -339,9 +339,9 @@ slim_status_t slim_linear_fwd_noalloc(const void* X, int b, const uint8_t* vals,
                                       int d_in, void* Y, uint32_t* status_dev, void* cuda_stream);
 
 /*
- * Bytes of the built-in array slim_linear_fwd_noalloc would use for this problem (host-side
- * arithmetic, no device needed); 0 when the entry point does not take the problem at all.  A
- * value above SLIM_NOALLOC_SCRATCH_BYTES means the call would return SLIM_ERR_WORKSPACE.
+ * The size slim_linear_fwd_noalloc's limit is stated in for this problem (host-side arithmetic, no device needed;
+ * an upper bound of the bytes of the built-in array that the call touches); 0 when the entry point does not take the
+ * problem at all.  A value above SLIM_NOALLOC_SCRATCH_BYTES means the call would return SLIM_ERR_WORKSPACE.
  */
 size_t slim_noalloc_scratch_needed(int b, int d_out, int d_in, int r);
 

@@ -28,11 +28,16 @@ static slim_status_t scratch_address(void** out) {
     return SLIM_OK;
 }
 
-// Size limit of the entry point: T, and one fp32 sum per output and 2048 columns (what a kernel that splits the
-// columns over the whole GPU needs), have to fit the array.  0: not a problem this entry point takes.
+// The entry point's limits, in terms of what a kernel that adds up split columns through the array would need: a slot of fp32
+// sums for 16 rows and up to 2048 columns of the weight, one for 16 rows and 512 columns of R, and T.  The small-batch kernel touches
+// less (the counter and T: 256 bytes and up to 160 KB); the limits stay where they were stated, so that what a caller was promised
+// or refused does not change.  0: not a problem this entry point takes.
 static size_t noalloc_need(int b, int d_out, int d_in, int r) {
-    if (b < 1 || b > 16 || d_in % 256 != 0 || d_in > 32768 || !small_supports(b, d_out, d_in, r)) return 0;
-    return kSmallTBytes + (size_t)ceil_div(d_in, 2048) * d_out * (b <= 8 ? 8 : 16) * sizeof(float);
+    if (b < 1 || b > 16 || d_in % 256 != 0 || d_in > 32768 || (b > 8 && r > 2560) || !small_supports(b, d_out, d_in, r)) return 0;
+    const int blocks = d_in / 256, slices = ceil_div(blocks, 8);
+    size_t slots = (size_t)slices * (d_out / 16);
+    for (int k = 0; k < slices; ++k) slots += (size_t)(r / 16) * (((k + 1) * blocks / slices - k * blocks / slices + 1) / 2);
+    return 198656 + slots * (b <= 8 ? 512 : 1024);
 }
 
 static bool is_aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
@@ -73,7 +78,7 @@ extern "C" slim_status_t slim_linear_fwd_noalloc(const void* X, int b, const uin
     cudaStream_t stream = (cudaStream_t)cuda_stream;
     // the array keeps whatever the previous call left (possibly cut short by a timeout): restart the call counter and
     // the call numbers of T's entries
-    if (cudaMemsetAsync(scratch, 0, SLIM_WORKSPACE_SYNC_BYTES + ((size_t)b * r * (keeps_T32(b, d_out, d_in, r) ? 8 : 4) + 255) / 256 * 256, stream) != cudaSuccess)
+    if (cudaMemsetAsync(scratch, 0, SLIM_WORKSPACE_SYNC_BYTES + ((size_t)b * r * 4 + 255) / 256 * 256, stream) != cudaSuccess)
         return SLIM_ERR_CUDA;
     return launch_small(static_cast<const __nv_bfloat16*>(X), b, vals, meta, nullptr, s, L, R, nullptr, nullptr, r, d_out, d_in,
                         static_cast<__nv_bfloat16*>(Y), scratch, status_dev, stream);

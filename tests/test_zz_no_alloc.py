@@ -37,6 +37,17 @@ def test_noalloc_rejects_problems_beyond_its_scratch_on_the_host():
             assert 0 < K.slim_noalloc_scratch_needed(16, d_out, d_in, r) <= K.NOALLOC_SCRATCH_BYTES
 
 
+def test_noalloc_takes_the_problems_it_always_took():
+    """The limit counts fp32 slots of 16 rows by 2048 columns (R: 512) and 198656 bytes for T, in 16 MiB."""
+    build.build()
+    need = K.slim_noalloc_scratch_needed
+    assert need(8, 512000, 2048, 0) == 256 + 198656 + 512 * (512000 // 16) <= K.NOALLOC_SCRATCH_BYTES
+    assert need(16, 8192, 28672, 832) == 256 + 198656 + 1024 * (14 * 512 + 52 * 56) <= K.NOALLOC_SCRATCH_BYTES
+    assert need(1, 272, 2304, 112) == 256 + 198656 + 512 * (2 * 17 + 7 * 5)           # nine blocks: slices of four and five
+    assert need(8, 520000, 2048, 0) > K.NOALLOC_SCRATCH_BYTES
+    assert need(8, 512, 512, 3072) > 0 and need(9, 512, 512, 2560) > 0 and need(9, 512, 512, 2576) == 0
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("d_in,d_out,r,b", [(2304, 272, 112, 13), (4096, 4096, 416, 16), (1024, 256, 0, 1)])
 def test_noalloc_matches_the_workspace_entry_point_twice(d_in, d_out, r, b):
