@@ -92,8 +92,8 @@ pack_adapter_pairs_kernel(const __nv_bfloat16* A, uint32_t items, int cols, int 
 }
 
 // Expansion to bf16 of one matrix or of a layer's two: a thread takes four bytes of codes (eight values, one 16-byte
-// store) where rows are multiples of eight elements, else one byte.  (One byte a thread and a launch per matrix took
-// 11 us for the adapters of a 1728 -> 5120 layer, rank 176.)
+// store) where rows are multiples of eight elements, else four times two bytes or one.  (One byte a thread and a launch per matrix took
+// 11 us for the adapters of a 1728 -> 5120 layer, rank 176; a dependent launch of one byte a thread 11.2 us for 5000 x 1004, UN_A so.)
 struct Unpack { const uint8_t* codes; const __nv_bfloat16* scales; __nv_bfloat16* out; int cols, groups; size_t items; };
 
 // I: the type of an item's number; TWO: two matrices.
@@ -102,23 +102,30 @@ __global__ void __launch_bounds__(256)
 unpack_adapter_kernel(const Unpack a, const Unpack b)
 {
     after_previous_grid();
-    I i = (I)blockIdx.x * 256 + threadIdx.x;
-    const bool second = TWO && i >= (I)a.items;
-    if (second) i -= (I)a.items;
-    const Unpack& m = second ? b : a;
-    if (i >= (I)m.items) return;
-    const uint32_t per_row = (uint32_t)m.cols / (2 * BYTES), row = (uint32_t)(i / per_row), c = (uint32_t)(i - (I)row * per_row) * (2 * BYTES);
-    const float sc = __bfloat162float(m.scales[(size_t)row * m.groups + c / 128]);
-    const size_t at = (size_t)row * m.cols + c;
-    uint32_t w = BYTES == 4 ? *reinterpret_cast<const uint32_t*>(m.codes + at / 2) : m.codes[at / 2], o[BYTES];
+    constexpr int kItems = BYTES == 4 ? 1 : 4;
 #pragma unroll
-    for (int k = 0; k < BYTES; ++k) {
-        const int lo = (int)(w << (28 - 8 * k)) >> 28, hi = (int)(w << (24 - 8 * k)) >> 28;
-        __nv_bfloat162 v = __floats2bfloat162_rn((float)lo * sc, (float)hi * sc);
-        o[k] = *reinterpret_cast<uint32_t*>(&v);
+    for (int n = 0; n < kItems; ++n) {
+        I i = ((I)blockIdx.x * kItems + n) * 256 + threadIdx.x;
+        const bool second = TWO && i >= (I)a.items;
+        if (second) i -= (I)a.items;
+        const Unpack& m = second ? b : a;
+        if (i >= (I)m.items) return;
+        const uint32_t per_row = (uint32_t)m.cols / (2 * BYTES), row = (uint32_t)(i / per_row), c = (uint32_t)(i - (I)row * per_row) * (2 * BYTES);
+        const float sc = __bfloat162float(m.scales[(size_t)row * m.groups + c / 128]);
+        const size_t at = (size_t)row * m.cols + c;
+        const uint8_t* from = m.codes + at / 2;
+        const uint32_t w = BYTES == 4 ? *reinterpret_cast<const uint32_t*>(from) : BYTES == 2 ? *reinterpret_cast<const uint16_t*>(from) : *from;
+        uint32_t o[4];
+#pragma unroll
+        for (int k = 0; k < BYTES; ++k) {
+            const int lo = (int)(w << (28 - 8 * k)) >> 28, hi = (int)(w << (24 - 8 * k)) >> 28;
+            __nv_bfloat162 v = __floats2bfloat162_rn((float)lo * sc, (float)hi * sc);
+            o[k] = *reinterpret_cast<uint32_t*>(&v);
+        }
+        if (BYTES == 4) *reinterpret_cast<uint4*>(m.out + at) = make_uint4(o[0], o[1], o[2], o[3]);
+        else if (BYTES == 2) *reinterpret_cast<uint2*>(m.out + at) = make_uint2(o[0], o[1]);
+        else *reinterpret_cast<uint32_t*>(m.out + at) = o[0];
     }
-    if (BYTES == 4) *reinterpret_cast<uint4*>(m.out + at) = make_uint4(o[0], o[1 % BYTES], o[2 % BYTES], o[3 % BYTES]);
-    else *reinterpret_cast<uint32_t*>(m.out + at) = o[0];
 }
 
 slim_status_t launch_pack_adapter(const __nv_bfloat16* A, int rows, int cols, uint8_t* codes, __nv_bfloat16* scales, cudaStream_t st)
@@ -137,9 +144,9 @@ static Unpack unpack_of(const uint8_t* codes, const __nv_bfloat16* scales, int r
 }
 template <int BYTES, bool TWO>
 static slim_status_t launch_unpack(const Unpack& a, const Unpack& b, cudaStream_t st) {
-    const size_t items = a.items + b.items;                                   // 2^32 and more: 64-bit numbers
-    launch_dependent(items <= 0xFFFFFF00u ? unpack_adapter_kernel<BYTES, uint32_t, TWO> : unpack_adapter_kernel<BYTES, uint64_t, TWO>,
-                     dim3((unsigned)((items + 255) / 256)), dim3(256), 0, st, a, b);
+    const size_t items = a.items + b.items, per_block = BYTES == 4 ? 256 : 1024;      // 2^32 and more: 64-bit numbers
+    launch_dependent(items <= 0xFFFFF000u ? unpack_adapter_kernel<BYTES, uint32_t, TWO> : unpack_adapter_kernel<BYTES, uint64_t, TWO>,
+                     dim3((unsigned)((items + per_block - 1) / per_block)), dim3(256), 0, st, a, b);
     count_launch(1);
     return cudaGetLastError() == cudaSuccess ? SLIM_OK : SLIM_ERR_CUDA;
 }
@@ -148,8 +155,9 @@ slim_status_t launch_unpack_adapter(const uint8_t* codes, const __nv_bfloat16* s
                                     cudaStream_t st)
 {
     const Unpack none = {};
-    return cols % 8 == 0 ? launch_unpack<4, false>(unpack_of(codes, scales, rows, cols, out, 4), none, st)
-                         : launch_unpack<1, false>(unpack_of(codes, scales, rows, cols, out, 1), none, st);
+    return cols % 8 == 0   ? launch_unpack<4, false>(unpack_of(codes, scales, rows, cols, out, 4), none, st)
+           : cols % 4 == 0 ? launch_unpack<2, false>(unpack_of(codes, scales, rows, cols, out, 2), none, st)
+                           : launch_unpack<1, false>(unpack_of(codes, scales, rows, cols, out, 1), none, st);
 }
 
 slim_status_t launch_unpack_adapters(const uint8_t* Lq, const __nv_bfloat16* Ls, const uint8_t* Rq, const __nv_bfloat16* Rs, int d_out, int r,

@@ -77,7 +77,7 @@ def test_mask_takes_a_negative_zero_magnitude_for_zero():
     assert np.array_equal(oracle.mask_top2(group[:1], np.array([-0.0, 1, 1, 1], np.float32)), [[1, 0, 0, 1]])
 
 
-@pytest.mark.parametrize("rows,cols", [(3, 130), (9, 1002), (2, 6), (5, 136)])
+@pytest.mark.parametrize("rows,cols", [(3, 130), (9, 1002), (2, 6), (5, 136), (7, 1004), (601, 12), (1025, 2)])
 def test_adapter_row_widths(rows, cols):
     A = long_tailed(rows, cols, 54)
     codes, scales = K.slim_pack_adapter(K.bf16_from_bits(A))
