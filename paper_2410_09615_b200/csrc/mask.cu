@@ -39,19 +39,31 @@ __device__ __forceinline__ uint32_t top2(uint32_t c, const float4* x)
 
 // A thread owns V (four, or one where a row is no multiple of four groups) groups of columns and walks rows: its input
 // magnitudes stay in registers, and it has the loads of ROWS rows in flight.  A block is up to 256 V groups of columns by as many
-// rows as make up 256 threads (100000 x 64: 27.8 us with one row a block); where blocks of several rows a thread would not
-// give every SM two, a thread takes one (64 x 4096: 3.2 us with four).
+// rows as make up 256 threads and leave two blocks an SM (100000 x 64: 27.8 us with one row a block, MASK_A so); where blocks of
+// several rows a thread would not give every SM one, a thread takes one (64 x 4096: 3.2 us with four, 2.0 so).
 template <int V> struct Words;
 template <> struct Words<4> { using T = uint4; };
 template <> struct Words<1> { using T = uint32_t; };
 
-template <bool XBAR, int V, int ROWS>
+// Codes are read once: past the L1.  (Volatile: not moved ahead of the wait.)
+__device__ __forceinline__ uint4 load_once(const uint4* p) {
+    uint4 v;
+    asm volatile("ld.global.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ uint32_t load_once(const uint32_t* p) {
+    uint32_t v;
+    asm volatile("ld.global.L1::no_allocate.u32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+}
+
+template <bool XBAR, int V, int ROWS, bool LANES>
 __global__ void __launch_bounds__(256)
 mask_top2_kernel(const typename Words<V>::T* codes, const float* xbar, int per_row, int d_out, typename Words<V>::T* mask, uint32_t* status)
 {
     using T = typename Words<V>::T;
     after_previous_grid();
-    const int g = blockIdx.x * blockDim.x + threadIdx.x, lanes = blockDim.y;
+    const int g = blockIdx.x * blockDim.x + threadIdx.x, lanes = LANES ? blockDim.y : 1;
     if (g >= per_row) return;
     float4 x[V];
 #pragma unroll
@@ -60,17 +72,21 @@ mask_top2_kernel(const typename Words<V>::T* codes, const float* xbar, int per_r
         if (blockIdx.y == 0 && !(x[v].x >= 0.f && x[v].x <= 3.0e38f && x[v].y >= 0.f && x[v].y <= 3.0e38f && x[v].z >= 0.f && x[v].z <= 3.0e38f && x[v].w >= 0.f && x[v].w <= 3.0e38f))
             flag_error(status, SLIM_ERR_INVALID_ARG);
     }
-    for (long long row0 = (long long)blockIdx.y * ROWS * lanes + threadIdx.y; row0 < d_out; row0 += (long long)gridDim.y * ROWS * lanes) {
-        T c[ROWS];
+    const size_t step = (size_t)lanes * per_row;
+    for (uint32_t row0 = blockIdx.y * ROWS * lanes + (LANES ? threadIdx.y : 0u); row0 < (uint32_t)d_out; row0 += gridDim.y * ROWS * lanes) {
+        const size_t at = (size_t)row0 * per_row + g;
+        T c[ROWS] = {};
+        const T* from = codes + at;
 #pragma unroll
-        for (int i = 0; i < ROWS; ++i) c[i] = codes[(size_t)min(row0 + i * lanes, (long long)d_out - 1) * per_row + g];
+        for (int i = 0; i < ROWS; ++i, from += step) if (row0 + i * lanes < (uint32_t)d_out) c[i] = load_once(from);
+        T* to = mask + at;
 #pragma unroll
-        for (int i = 0; i < ROWS; ++i) {
+        for (int i = 0; i < ROWS; ++i, to += step) {
             T o;
 #pragma unroll
             for (int v = 0; v < V; ++v)
                 reinterpret_cast<uint32_t*>(&o)[v] = top2(reinterpret_cast<const uint32_t*>(&c[i])[v], XBAR ? &x[v] : nullptr);
-            if (row0 + i * lanes < d_out) mask[(size_t)(row0 + i * lanes) * per_row + g] = o;
+            if (row0 + i * lanes < (uint32_t)d_out) *to = o;
         }
     }
 }
@@ -79,12 +95,15 @@ template <int V, int ROWS>
 static void launch_mask(const int8_t* codes, const float* xbar, int d_out, int d_in, uint8_t* mask, uint32_t* status_dev, cudaStream_t st)
 {
     using T = typename Words<V>::T;
-    const int per_row = d_in / (4 * V), cols = per_row < 256 ? per_row : 256, lanes = 256 / cols;
-    const int strips = ceil_div(d_out, ROWS * lanes), blocks = ceil_div(per_row, cols);
-    if (ROWS > 1 && (long long)strips * blocks < 2 * 148) { launch_mask<V, 1>(codes, xbar, d_out, d_in, mask, status_dev, st); return; }
+    const int per_row = d_in / (4 * V), cols = per_row < 256 ? per_row : 256, blocks = ceil_div(per_row, cols);
+    const int most = 256 / cols, spread = d_out / (ROWS * 2 * 148), lanes = spread < 1 ? 1 : spread < most ? spread : most;
+    const int strips = ceil_div(d_out, ROWS * lanes);
+    if (ROWS > 1 && (long long)strips * blocks < 148) { launch_mask<V, 1>(codes, xbar, d_out, d_in, mask, status_dev, st); return; }
     const T* c = reinterpret_cast<const T*>(codes);
     T* m = reinterpret_cast<T*>(mask);
-    launch_dependent(xbar ? mask_top2_kernel<true, V, ROWS> : mask_top2_kernel<false, V, ROWS>, dim3((unsigned)blocks, (unsigned)(strips < 65535 ? strips : 65535)),
+    auto* kernel = lanes > 1 ? (xbar ? mask_top2_kernel<true, V, ROWS, true> : mask_top2_kernel<false, V, ROWS, true>)
+                             : (xbar ? mask_top2_kernel<true, V, ROWS, false> : mask_top2_kernel<false, V, ROWS, false>);
+    launch_dependent(kernel, dim3((unsigned)blocks, (unsigned)(strips < 65535 ? strips : 65535)),
                      dim3((unsigned)cols, (unsigned)lanes), 0, st, c, xbar, per_row, d_out, m, status_dev);
 }
 
