@@ -60,22 +60,36 @@ static slim_status_t check_weight_shape(int d_out, int d_in) {
     return SLIM_OK;
 }
 
-// Small ragged problems (rows of d_in / 8 index bytes or 128-row tiles that do not come out even, less than one
-// 256-row tile and few multiply-adds) would occupy one cluster: the CUDA-core kernel spreads them.
-static bool small_and_ragged(int b, int d_out, int d_in) {
-    return (d_in % 128 != 0 || (d_out % 128 != 0 && b > 16)) && d_out < 256 && (long long)b * d_out * d_in < (1 << 24);
+// Problems for the CUDA-core kernel (a warp per output, all SMs at once): of the ragged shapes, whose rows or tiles do not come out even
+// for the tensor cores, those with few outputs or few multiply-adds.  Times on the GPU, CUDA cores against the next best:
+//   up to 16 tokens      64 -> 256, 1 token, no adapters 2.5 us, small batches 3.0
+//   fewer than 256 rows  256 -> 48, 17 tokens, no adapters half of the one-CTA kernel's time; the two meet near 2^22 multiply-adds
+//   no adapters          320 -> 512, 17 tokens 5.0, 5.9; 1088 -> 256, 17 tokens 5.2, 8.0; 8192 -> 16, 300 tokens 22, CTA pairs 26
+static bool on_cuda_cores(int b, int d_out, int d_in, int r) {
+    const long long outputs = (long long)b * d_out, work = outputs * d_in;
+    if (b <= 16) return (d_in % 128 != 0 && d_out < 256 && work < (1 << 24)) || (d_in % 256 != 0 && r == 0 && work < (1 << 19));
+    if (d_in % 128 == 0 && d_out % 128 == 0) return false;
+    if (d_out < (r == 0 && b <= 32 ? 257 : 256) && work < (1 << 24)) return true;
+    return r == 0 && ((b > 64 && outputs <= 4800) || (outputs <= 16384 && work < 3 << 20));
 }
 
 // The small-batch kernel's problems: up to 64 tokens, one launch.  From 33 tokens on its warp-level MMAs take longer than the
 // tensor-memory kernel's (5120 -> 13824, 64 tokens: 38 us against 26), which has the advantage once d_out gives it enough tiles
-// (8192 x 8192: a tie; 11008 -> 4096: 38 us against 41).
-static bool runs_small(int b, int d_out, int d_in, int r) {
-    return small_supports(b, d_out, d_in, r) && !small_and_ragged(b, d_out, d_in) && !(b > 32 && d_out >= 8192);
+// (8192 x 8192: a tie; 11008 -> 4096: 38 us against 41).  Rows of few columns are the one-CTA kernel's (launch_prefill) from 17 tokens on:
+// it has no exchange between CTAs at the end (512 -> 4096, 64 tokens, no adapters 6.2 us against 9.2).  The lines, by tokens, adapters
+// and whether rows and tiles come out even, lie where the two meet; int4 adapters, which the others take expanded and rounded to
+// bf16, stay here.
+static bool runs_small(int b, int d_out, int d_in, int r, bool int4 = false) {
+    if (!small_supports(b, d_out, d_in, r) || on_cuda_cores(b, d_out, d_in, r) || (b > 32 && d_out >= 8192)) return false;
+    if (b <= 16 || int4) return true;
+    if (r == 0) return d_in > (b <= 32 ? 320 : d_in % 128 != 0 ? 1536 : 768);
+    if (d_in % 128 != 0 || d_out % 128 != 0) return b <= 32 || d_in > 256;
+    return d_in > (b <= 32 ? 256 : 768);
 }
 
 static slim_kernel_t select_kernel(int b, int d_out, int d_in, int r) {
     if (b <= 16 && runs_small(b, d_out, d_in, r)) return SLIM_KERNEL_DECODE;
-    if (b > 16 && prefill_supports(b, d_out, d_in, r) && !small_and_ragged(b, d_out, d_in)) return SLIM_KERNEL_PREFILL;
+    if (b > 16 && prefill_supports(b, d_out, d_in, r) && !on_cuda_cores(b, d_out, d_in, r)) return SLIM_KERNEL_PREFILL;
     return SLIM_KERNEL_SIMPLE;
 }
 
@@ -279,7 +293,7 @@ slim_status_t slim_linear_fwd_q(const void* X, int b, const uint8_t* vals, const
     const size_t base = align256(slim_workspace_bytes(b, d_out, d_in, r));
     cudaStream_t st = (cudaStream_t)cuda_stream;
     // small batches: the kernel reads the codes and scales as they are
-    if (runs_small(b, d_out, d_in, r)) {
+    if (runs_small(b, d_out, d_in, r, true)) {
         if (!X || !vals || !meta || !Y || !std::isfinite(s)) return SLIM_ERR_INVALID_ARG;
         if (!aligned16(X) || !aligned16(vals) || !aligned16(meta) || !aligned16(Y)) return SLIM_ERR_INVALID_ARG;
         if (status_dev && (reinterpret_cast<uintptr_t>(status_dev) & 3u)) return SLIM_ERR_INVALID_ARG;

@@ -1192,12 +1192,24 @@ static int pair_tile(int b, int d_out, int sm_count) {
     return 256;
 }
 
-// The pair kernel when its 128 x 256 tiles would give a quarter of the SMs or more a tile.  The dispatcher (`automatic`) also takes it for smaller problems with eight tiles or more (4096 x 4096, 100 tokens
-// 25 -> 22 us, 200 tokens 45 -> 26), unless both the batch and d_in are short (1024 -> 4096, 128 tokens: 17 us against 13);
-// asked for by name the one-CTA kernel keeps those.
+// The pair kernel, asked for by the kernel family's name: when its 128 x 256 tiles would give a quarter of the SMs or more a tile.
+// The dispatcher (`automatic`) takes it unless the 128 x 64 tiles of the one-CTA kernel have an SM each and rows are short: the pairs'
+// stage of 128 columns costs less, but they make T' in a cooperative launch that takes 10 us however short it is.  The two meet
+//   without adapters at 768 columns (512 -> 4096, 200 tokens: one CTA 8 % faster; 1024 -> 4096: the same; 1536 columns: 8 % slower);
+//   on shapes that come out even at 2048 columns up to 191 tokens (768 -> 8192, 100 tokens, rank 208 11.0 us against 22.8; 2048 -> 8192 15.4
+//   against 20.7), at 1024 where tiles are up to two an SM and the rank above 128 (1024 -> 8192, 160 tokens, rank 208 20.0 against 22.2,
+//   rank 64 18.3 against 15.6), at 1024 above (1536 -> 2048, 300 tokens, rank 16 18.0 against 13.4; 1024 -> 256, rank 208 16.2 against 20.5);
+//   on others, whose T' has two parts, at 2048 up to 191 tokens and few tiles; above the pairs are always faster (2048 -> 48, 200 tokens,
+//   rank 16 13.6 us against 32).
 static bool runs_wide(int b, int d_out, int d_in, int r, int sm_count, bool automatic) {
-    if ((long long)ceil_div(d_out, kPM) * ceil_div(b, 256) * 4 >= (long long)sm_count) return true;
-    return automatic && (b >= 192 || d_in >= 2048) && (long long)ceil_div(d_out, 2 * kPM) * ceil_div(b, pair_tile(b, d_out, sm_count)) >= 8;
+    const bool many = (long long)ceil_div(d_out, kPM) * ceil_div(b, 256) * 4 >= (long long)sm_count;
+    if (!automatic) return many;
+    const long long tiles = (long long)ceil_div(d_out, kPM) * ceil_div(b, 64);
+    const bool even = d_out % kPM == 0 && d_in % 128 == 0;
+    if (tiles > sm_count) return !(even && r > 128 && b < 192 && d_in <= 1024 && tiles <= 2 * sm_count);
+    if (r == 0) return d_in > 768;
+    if (!even) return many || b >= 192 || d_in >= 2048;
+    return d_in > (b < 192 ? 2048 : 1024);
 }
 
 // T' in the workspace; the partial sums follow it.
