@@ -70,8 +70,9 @@ typedef enum {
     SLIM_KERNEL_DECODE = 2,  /* streaming sparse tensor-core kernel for small batches */
     SLIM_KERNEL_PREFILL = 3, /* tcgen05 sparse tensor-core kernels for many tokens: CTA pairs on 256-row tiles,
                                 or one CTA per 128-row tile where those would be few */
-    SLIM_KERNEL_PREFILL_PAIR = 4 /* the CTA-pair kernel whatever the size; asked for by name it needs an
+    SLIM_KERNEL_PREFILL_PAIR = 4, /* the CTA-pair kernel whatever the size; asked for by name it needs an
                                     even number of 128-row tiles */
+    SLIM_KERNEL_SMALL = 5    /* the kernel of SLIM_KERNEL_DECODE for 17 to 64 tokens */
 } slim_kernel_t;
 
 /*
@@ -124,10 +125,10 @@ slim_status_t slim_workspace_reset(void* workspace, size_t workspace_bytes, void
  *   L [d_out, r] bf16, R [r, d_in] bf16 (both NULL iff r == 0), Y [b, d_out] bf16 (out).
  * Shape rules: b >= 1, d_in % 64 == 0, d_out % 16 == 0, r % 16 == 0; s must be finite
  * (NaN or infinity: SLIM_ERR_INVALID_ARG).
- * The kernel is chosen from b and the shape: up to 16 tokens, and up to 64 of layers with
- * fewer than 8192 rows, the streaming small-batch kernel (r <= 3072); above, the tcgen05 prefill kernels.
- * All take any legal shape.  Small ragged problems (d_in % 128 or, above 16 tokens, d_out % 128 not zero,
- * d_out < 256, fewer than 2^24 multiply-adds) and small batches of a larger rank run on a plain CUDA-core
+ * The kernel is chosen from b and the shape (slim_select_kernel): up to 16 tokens the streaming small-batch kernel
+ * (r <= 3072), and up to 64 unless rows have few columns or, above 32, the layer has 8192 rows or more; else the tcgen05
+ * prefill kernels.  All take any legal shape.  Ragged problems (d_in % 128 or, above 16 tokens, d_out % 128 not
+ * zero) with few outputs or multiply-adds, and up to 16 tokens of a larger rank, run on a plain CUDA-core
  * kernel (one warp per output element).
  * For one to four tokens of a weight of 64 MiB or more slim_linear_fwd_tiled on the decode-tiled copy is faster.
  */
@@ -345,7 +346,10 @@ slim_status_t slim_linear_fwd_noalloc(const void* X, int b, const uint8_t* vals,
  */
 size_t slim_noalloc_scratch_needed(int b, int d_out, int d_in, int r);
 
-/* The kernel family slim_linear_fwd would pick for this problem. */
+/*
+ * The kernel family slim_linear_fwd would pick for this problem.  Asked for by name it runs the same kernel, except that
+ * SLIM_KERNEL_PREFILL by name keeps to one CTA per tile in more cases (slim_last_token_tile tells which ran).
+ */
 slim_kernel_t slim_select_kernel(int b, int d_out, int d_in, int r);
 
 /* Number of kernels the last slim_linear_fwd* call on this host thread launched. */

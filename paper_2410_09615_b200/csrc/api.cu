@@ -88,7 +88,7 @@ static bool runs_small(int b, int d_out, int d_in, int r, bool int4 = false) {
 }
 
 static slim_kernel_t select_kernel(int b, int d_out, int d_in, int r) {
-    if (b <= 16 && runs_small(b, d_out, d_in, r)) return SLIM_KERNEL_DECODE;
+    if (runs_small(b, d_out, d_in, r)) return b <= 16 ? SLIM_KERNEL_DECODE : SLIM_KERNEL_SMALL;
     if (b > 16 && prefill_supports(b, d_out, d_in, r) && !on_cuda_cores(b, d_out, d_in, r)) return SLIM_KERNEL_PREFILL;
     return SLIM_KERNEL_SIMPLE;
 }
@@ -191,11 +191,10 @@ slim_status_t slim_linear_fwd_ex(const void* X, int b, const uint8_t* vals, cons
     case SLIM_KERNEL_SIMPLE:
         return launch_simple(Xb, b, vals, meta, s, Lb, Rb, r, d_out, d_in, Yb, workspace, stream);
     case SLIM_KERNEL_DECODE:
-        if (b > 16) return SLIM_ERR_UNSUPPORTED_SHAPE;
+    case SLIM_KERNEL_SMALL:
+        if (kernel == SLIM_KERNEL_DECODE ? b > 16 : b <= 16) return SLIM_ERR_UNSUPPORTED_SHAPE;
         return launch_small(Xb, b, vals, meta, nullptr, s, Lb, Rb, nullptr, nullptr, r, d_out, d_in, Yb, workspace, status_dev, stream);
     case SLIM_KERNEL_PREFILL:
-        if (automatic && runs_small(b, d_out, d_in, r))            // up to 64 tokens: the small-batch kernel
-            return launch_small(Xb, b, vals, meta, nullptr, s, Lb, Rb, nullptr, nullptr, r, d_out, d_in, Yb, workspace, status_dev, stream);
         if (!prefill_supports(b, d_out, d_in, r)) return SLIM_ERR_UNSUPPORTED_SHAPE;
         return launch_prefill(Xb, b, vals, meta, s, Lb, Rb, r, d_out, d_in, Yb, workspace, status_dev, stream, false, automatic);
     case SLIM_KERNEL_PREFILL_PAIR:

@@ -51,17 +51,35 @@ def test_dispatcher_choices():
     assert K.slim_select_kernel(1, 4096, 4096, 416) == K.KERNEL_DECODE
     assert K.slim_select_kernel(16, 4096, 11008, 416) == K.KERNEL_DECODE
     assert K.slim_select_kernel(8, 512, 512, 64) == K.KERNEL_DECODE
-    assert K.slim_select_kernel(4, 64, 64, 16) != K.KERNEL_DECODE      # d_in not a multiple of 256
-    assert K.slim_select_kernel(17, 4096, 4096, 416) == K.KERNEL_PREFILL
+    assert K.slim_select_kernel(4, 64, 64, 16) != K.KERNEL_DECODE      # ragged rows, few multiply-adds: CUDA cores
+    assert K.slim_select_kernel(17, 4096, 4096, 416) == K.KERNEL_SMALL      # one launch of the small-batch kernel
     assert K.slim_select_kernel(2048, 4096, 11008, 416) == K.KERNEL_PREFILL
-    assert K.slim_select_kernel(64, 48, 4096, 16) == K.KERNEL_SIMPLE        # d_out not a multiple of 128
-    assert K.slim_select_kernel(50, 128, 704, 32) == K.KERNEL_SIMPLE        # d_in not a multiple of 128
+    assert K.slim_select_kernel(64, 48, 4096, 16) == K.KERNEL_SIMPLE        # d_out not a multiple of 128 and below 256
+    assert K.slim_select_kernel(50, 128, 704, 32) == K.KERNEL_SIMPLE        # d_in not a multiple of 128, d_out below 256
+
+
+@pytest.mark.parametrize("d_in,d_out,r,b", [(1024, 256, 32, 3), (512, 512, 64, 17), (1728, 528, 80, 33), (1024, 512, 0, 64), (704, 128, 32, 50), (320, 512, 0, 17),
+                                            (256, 512, 32, 24), (768, 256, 0, 64), (4096, 8192, 64, 40)])
+def test_selected_kernel_is_the_one_that_runs(d_in, d_out, r, b):
+    ly = inputs.make_layer(d_in, d_out, r, b, seed=19)
+    vals, meta = K.slim_pack(to_dev(ly.codes), to_dev(ly.mask))
+    X, L, R = K.bf16_from_bits(ly.X), K.bf16_from_bits(ly.L) if r else None, K.bf16_from_bits(ly.R) if r else None
+    kernel = K.slim_select_kernel(b, d_out, d_in, r)
+    ran = []
+    for k in (K.KERNEL_AUTO, kernel):
+        Y = K.slim_linear_fwd(X, vals, meta, ly.s, L, R, kernel=k)
+        ran.append((K.slim_last_launch_count(), K.slim_last_token_tile(), Y.view(torch.int16).cpu()))
+    if kernel == K.KERNEL_PREFILL:                  # one kernel or the other of the family
+        assert ran[0][1] > 0 and ran[1][1] > 0
+    else:
+        assert ran[0][:2] == ran[1][:2] and torch.equal(ran[0][2], ran[1][2]) and ran[0][1] == 0
+    assert (kernel == K.KERNEL_SIMPLE) == (ran[0][0] == (2 if r else 1) and ran[0][1] == 0 and kernel not in (K.KERNEL_DECODE, K.KERNEL_SMALL))
 
 
 def test_shapes_outside_the_fast_kernels_still_work():
-    assert_ok(run_case(64, 16, 16, 2, seed=31))          # d_in = 64: simple kernel
-    assert_ok(run_case(320, 32, 0, 40, seed=32))         # b > 16, no adapters
-    assert_ok(run_case(704, 128, 32, 50, seed=33))       # b > 16, d_in % 128 != 0: not the prefill kernel
+    assert_ok(run_case(64, 16, 16, 2, seed=31))          # (small and ragged: the CUDA-core kernel)
+    assert_ok(run_case(320, 32, 0, 40, seed=32))
+    assert_ok(run_case(704, 128, 32, 50, seed=33))
 
 
 # ---- tcgen05 prefill kernel, small cases, all elements ----------------------
