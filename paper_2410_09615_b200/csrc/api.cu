@@ -93,8 +93,8 @@ static slim_kernel_t select_kernel(int b, int d_out, int d_in, int r) {
     return SLIM_KERNEL_SIMPLE;
 }
 
-// Sync words, then the region the small-batch kernel publishes T in (entries carry call numbers, so nothing else is
-// ever written there), then the other kernels' scratch.
+// Sync words, then the region of the words that carry call numbers (the small-batch and the pair kernel's: kSmallTBytes), then the
+// kernels' scratch.
 static size_t workspace_bytes(int b, int d_out, int d_in, int r) {
     size_t need = simple_workspace_bytes(b, d_out, d_in, r);
     const size_t pf = prefill_workspace_bytes(b, d_out, d_in, r);

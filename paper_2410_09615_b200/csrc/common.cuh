@@ -64,9 +64,10 @@ const DeviceInfo* device_info(slim_status_t* err);
 // nullptr when the driver does not have it.  Thread-safe.
 void* tensor_map_encoder();
 
-// The small-batch kernel publishes T = X R^T in a region of this fixed size right after the sync words, whatever
-// the problem, and nothing else is kept there: calls of different shapes on one workspace never read one kind of
-// word as another.
+// The words that CTAs hand to one another have a region of this fixed size right after the sync words, whatever the problem: the
+// small-batch kernel's T = X R^T, the pair kernel's {part written, tile ready}.  Each carries the number of the call that wrote it
+// (handover.h), so kernels and shapes may take turns there as long as every one of them that does counts each of its calls,
+// also those that hand nothing over (the pair kernel without adapters), and nothing is written there without a number.
 constexpr size_t kSmallTBytes = 512 << 10;
 constexpr int kSmallMaxRank = 3072;
 

@@ -50,9 +50,5 @@ __device__ __forceinline__ uint32_t nibbles_to_bf16x2(uint32_t x) {
     return *reinterpret_cast<uint32_t*>(&v);
 }
 
-__device__ __forceinline__ uint32_t word_of(const uint4& v, int i) {
-    return i == 0 ? v.x : i == 1 ? v.y : i == 2 ? v.z : v.w;
-}
-
 }  // namespace dt
 }  // namespace slim

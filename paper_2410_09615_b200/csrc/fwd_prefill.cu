@@ -648,7 +648,7 @@ prefill_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap tmV,
 // N = tokens of a tile: 256, 128 or 64.  A stage takes the same 0.36 us for each of them (the MMAs' 256 weight rows cost what
 // they cost), so a narrower tile only saves epilogue and token traffic.  A stage is 32 KB for every N (what T' needs).
 // Five stages and four packed tiles in flight: 33.2 -> 32.0 us on 8192 x 8192, 333 tokens, 91 -> 83 us on 28672 -> 8192, 64
-// tokens, against six and two.
+// tokens, against six and two (calls on one weight, which stays in the L2; with weights in rotation the first takes 36).
 // Stages alternate between two converter groups and two token-tile warps while their number is odd, so each of them sees
 // every second phase of an `empty` barrier.  Waiting by parity is still right: before its stage g such a warp has waited
 // for the MMAs of stage g - 7, so the phase it did not see (stage g - 10) is over.  For the packed tiles' barriers the same holds
@@ -1257,7 +1257,7 @@ static slim_status_t launch_pair(const PrefillParams& p, const CUtensorMap& tmV,
         attr[1].id = cudaLaunchAttributeCooperative;
         attr[1].val.cooperative = 1;
     } else {
-        // set up while the grid before it ends (8192 x 8192, 333 tokens 32.9 -> 31.8 us; no gain beside a cooperative launch)
+        // set up while the grid before it ends (8192 x 8192, 333 tokens, weight in the L2 32.9 -> 31.8 us; no gain beside a cooperative launch)
         attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[1].val.programmaticStreamSerializationAllowed = 1;
     }

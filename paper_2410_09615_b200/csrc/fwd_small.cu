@@ -27,6 +27,8 @@
 //   - the index bits a lane has to supply for a step are byte j of two regions of two rows: two prmt;
 //   - the activations of a step are 16 contiguous bytes per token and region: one ldmatrix.x4.
 // The decode-tiled copy holds registers and index words in the instruction's natural column order instead.
+// Registers: 96 a thread up to 16 tokens (two CTAs an SM), 168 above.  256-row tiles at 9 to 16 tokens spill 32 bytes there (80 with
+// int4 adapters; up to 140 with T in two parts), 33 to 64 tokens 72 (up to 88 with int4).
 // Alone on an SM (16 warps) a 16-row x 32-column step takes a scheduler 33 cycles at 8 tokens, 41 at 16
 // (20 of them the ALU pipe's), and 24 / 33 on the tiled copy.
 //
@@ -1051,7 +1053,9 @@ bool make_map3(CUtensorMap* map, const void* base, uint64_t cols, uint64_t rows,
 }
 
 // CTAs per cluster: the most (up to 8, and no more than there are units) with which the clusters of all tiles fit the
-// device at once, so that the stream of a tile is spread as widely as it can be; with more tiles than that, one.
+// device at once, so that the stream of a tile is spread as widely as it can be; with more tiles than that, one.  (The clusters of T
+// are not counted here, unlike for narrow tiles: they are done first and leave their places; 28672 -> 8192, 16 tokens has 464 CTAs on 296
+// places this way.  Four CTAs a cluster, with which all would be resident, have not been measured.)
 int cluster_size(const int* res, int tiles, int units) {
     for (int i = 3; i > 0; --i)
         if ((1 << i) <= units && tiles <= res[i]) return 1 << i;

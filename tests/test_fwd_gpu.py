@@ -345,9 +345,11 @@ def test_full_size_prefill_configs(d_in, d_out, r, b, seed, wseed):
     assert_ok(res)
 
 
-def test_prefill_chain_replays_from_a_cuda_graph():
-    """The prefill call's launches depend on one another programmatically (the main launch starts before the
-    dense-only launch has ended): captured in a CUDA graph and replayed, the call gives the same bits."""
+@pytest.mark.parametrize("kernel,launches", [(K.KERNEL_PREFILL, (2, 3)), (K.KERNEL_PREFILL_PAIR, (1,))])
+def test_prefill_replays_from_a_cuda_graph(kernel, launches):
+    """Captured in a CUDA graph and replayed, a prefill call gives the same bits: the chain of the one-CTA kernel, whose launches depend
+    on one another programmatically (the main launch starts before the dense-only launch has ended), and the cooperative launch of the
+    CTA pairs."""
     d_in, d_out, r, b = 1024, 512, 64, 600
     s, codes, mask, ovals, ometa = cached_weights(d_out, d_in, 91)
     ly = inputs.make_layer(d_in, d_out, r, b, 91, weights=(s, codes, mask))
@@ -357,14 +359,15 @@ def test_prefill_chain_replays_from_a_cuda_graph():
     status = torch.zeros(1, dtype=torch.int32, device="cuda")
     Y = torch.empty((b, d_out), dtype=torch.bfloat16, device="cuda")
     assert binding.slim_select_kernel(b, d_out, d_in, r) == binding.KERNEL_PREFILL
-    binding.slim_linear_fwd(X, vals, meta, s, L, R, Y=Y, workspace=ws, status=status)
+    binding.slim_linear_fwd(X, vals, meta, s, L, R, Y=Y, workspace=ws, status=status, kernel=kernel)
+    assert binding.slim_last_launch_count() in launches
     torch.cuda.synchronize()
     direct = Y.clone()
     stream = torch.cuda.Stream()
     g = torch.cuda.CUDAGraph()
     with torch.cuda.stream(stream):
         with torch.cuda.graph(g, stream=stream):
-            binding.slim_linear_fwd(X, vals, meta, s, L, R, Y=Y, workspace=ws, status=status)
+            binding.slim_linear_fwd(X, vals, meta, s, L, R, Y=Y, workspace=ws, status=status, kernel=kernel)
         for _ in range(3):
             Y.zero_()
             g.replay()

@@ -152,12 +152,14 @@ def test_tiled_calls_repeat_bit_for_bit(d_in, d_out, r, b):
 
 
 def test_one_workspace_serves_every_kernel_and_shape_in_turn():
-    """Decode calls of different shapes and batch sizes (both tiled and packed-format kernels), a
-    prefill call and a CUDA-core call share one workspace; every result is checked against the
-    oracle.  A kernel that left the hand-over slots of another in a used state would show here."""
+    """Small batches of different shapes (tiled and packed format, up to 16 and up to 64 tokens), CTA pairs with and without
+    adapters, the one-CTA prefill kernel and the CUDA-core kernel share one workspace; every result is checked against the
+    oracle.  Small batches and CTA pairs keep their hand-over words in the same place, told apart by the call's number: a kernel
+    that does not count its call, or writes there without one, would show here."""
     shapes = [(1024, 256, 32, 16), (768, 48, 16, 3), (2304, 272, 112, 13), (512, 512, 0, 1), (4352, 1040, 208, 9)]
     big = max(K.slim_workspace_bytes(b, d_out, d_in, r) for d_in, d_out, r, b in shapes)
-    big = max(big, K.slim_workspace_bytes(300, 256, 512, 112), K.slim_workspace_bytes(50, 128, 704, 32))
+    big = max(big, K.slim_workspace_bytes(300, 256, 512, 112), K.slim_workspace_bytes(50, 128, 704, 32), K.slim_workspace_bytes(400, 1040, 2304, 208),
+              K.slim_workspace_bytes(60, 784, 1728, 208))
     ws = torch.empty(big, dtype=torch.uint8, device="cuda")
     K.slim_workspace_reset(ws)
     status = torch.zeros(1, dtype=torch.int32, device="cuda")
@@ -180,8 +182,14 @@ def test_one_workspace_serves_every_kernel_and_shape_in_turn():
             res = run_tiled(d_in, d_out, r, b, seed=70 + i, ws=ws, check_repack=False)
             assert res["ok"], (rnd, d_in, d_out, r, b, res)
             packed_call(d_in, d_out, r, b, 70 + i, K.KERNEL_DECODE)
-        packed_call(512, 256, 112, 300, 80, K.KERNEL_PREFILL)      # writes T' where the decode slots live
-        packed_call(704, 128, 32, 50, 81, K.KERNEL_SIMPLE)         # writes T (fp32) there
+            packed_call(512, 256, (112, 0)[i % 2], 300, 80, K.KERNEL_PREFILL_PAIR)      # its words (or none: still a call) between theirs
+            assert K.slim_last_launch_count() == 1
+        packed_call(2304, 1040, 208, 400, 82, K.KERNEL_AUTO)       # pairs, parts of T' from several of them
+        assert K.slim_last_token_tile() > 0 and K.slim_last_launch_count() == 1
+        packed_call(1728, 784, 208, 60, 83, K.KERNEL_AUTO)         # small batches, T in two parts
+        assert K.slim_last_token_tile() == 0 and K.slim_last_launch_count() == 1
+        packed_call(512, 256, 112, 300, 80, K.KERNEL_PREFILL)      # T' and partial sums behind the words
+        packed_call(704, 128, 32, 50, 81, K.KERNEL_SIMPLE)         # T in fp32 there
 
 
 def test_tiled_argument_errors():
