@@ -572,7 +572,7 @@ def quantized_adapter_table(K, lib, layers, stream, peak):
             launches = lib.slim_last_launch_count()
             nb, nq = algorithmic_bytes(d_in, d_out, r, b), algorithmic_bytes_q(d_in, d_out, r, b)
             rows.append({"layer": ly["name"], "d_in": d_in, "d_out": d_out, "r": r, "b": b,
-                         "path": "decode kernel on codes and scales" if launches == 1 else "adapters expanded to bf16 first",
+                         "path": "small-batch kernel on codes and scales" if launches == 1 else "adapters expanded to bf16 first",
                          "bytes_bf16_adapters": nb, "bytes_quantized": nq, "bytes_ratio": round(nb / nq, 3),
                          "us_bf16_adapters": round(t_plain, 3), "us_quantized": round(t_q, 3),
                          "speedup": round(t_plain / t_q, 3), "frac_measured_quantized": round(nq / (t_q * 1e-6) / 1e9 / peak, 4)})

@@ -606,8 +606,9 @@ prefill_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap tmV,
             if (PRE && p.part) {
                 store(p.part + ((size_t)blockIdx.z * p.b + n0 + c0) * p.ldo + orow, [](float v) { return v; });
             } else if (PRE && p.t_parts == 2) {
-                store(out, [&](float v) { return __float2bfloat16_rn(bf16_head(p.scale * v)); });
-                store(out + (size_t)p.b * p.ldo, [&](float v) { return __float2bfloat16_rn(bf16_tail(p.scale * v)); });
+#pragma unroll 1
+                for (int tp = 0; tp < 2; ++tp, out += (size_t)p.b * p.ldo)
+                    store(out, [&](float v) { v *= p.scale; return __float2bfloat16_rn(tp ? bf16_tail(v) : bf16_head(v)); });
             } else {
                 store(out, [&](float v) { return __float2bfloat16_rn(p.scale * v); });
             }
@@ -691,13 +692,19 @@ __device__ __forceinline__ bool wait_words(const unsigned long long* w, uint32_t
 
 // Four neighbouring values of T', in one part or (`tail`: the way to the second) two.
 __device__ __forceinline__ void store_T(__nv_bfloat16* at, size_t tail, float4 v) {
-    auto put = [&](__nv_bfloat16* to, float4 q) {
+    auto put = [&](float4 q) {
         __nv_bfloat162 lo = __floats2bfloat162_rn(q.x, q.y), hi = __floats2bfloat162_rn(q.z, q.w);
-        *reinterpret_cast<uint2*>(to) = make_uint2(*reinterpret_cast<uint32_t*>(&lo), *reinterpret_cast<uint32_t*>(&hi));
+        *reinterpret_cast<uint2*>(at) = make_uint2(*reinterpret_cast<uint32_t*>(&lo), *reinterpret_cast<uint32_t*>(&hi));
     };
-    if (tail == 0) { put(at, v); return; }
-    put(at, make_float4(bf16_head(v.x), bf16_head(v.y), bf16_head(v.z), bf16_head(v.w)));
-    put(at + tail, make_float4(bf16_tail(v.x), bf16_tail(v.y), bf16_tail(v.z), bf16_tail(v.w)));
+    if (tail != 0) {
+        const float4 h = make_float4(bf16_head(v.x), bf16_head(v.y), bf16_head(v.z), bf16_head(v.w));
+        put(h);
+        at += tail;
+        v = make_float4(v.x - h.x, v.y - h.y, v.z - h.z, v.w - h.w);
+        if (!(fabsf(v.x) + fabsf(v.y) + fabsf(v.z) + fabsf(v.w) <= 3.4e38f))        // infinities and NaN are in the head
+            v = make_float4(fabsf(v.x) <= 3.4e38f ? v.x : 0.f, fabsf(v.y) <= 3.4e38f ? v.y : 0.f, fabsf(v.z) <= 3.4e38f ? v.z : 0.f, fabsf(v.w) <= 3.4e38f ? v.w : 0.f);
+    }
+    put(v);
 }
 
 template <int N>

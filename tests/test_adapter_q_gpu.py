@@ -79,7 +79,7 @@ def run_q(d_in, d_out, r, b, seed, wseed=None, rows=None):
 
 
 @pytest.mark.parametrize("d_in,d_out,r,b", [
-    # decode kernel reading codes and scales as they are: short last group, two chunk widths, several
+    # small-batch kernel reading codes and scales as they are: short last group, two chunk widths, several
     # k-slices, both token-tile counts; ranks whose rows of L codes are no 16-byte multiples (plain loads)
     (256, 64, 32, 1), (512, 512, 64, 8), (768, 208, 96, 16), (1024, 384, 160, 5), (2304, 128, 416, 16), (4352, 96, 544, 3),
     (1280, 1040, 1056, 9),
@@ -92,7 +92,7 @@ def test_forward_on_quantized_adapters_small(d_in, d_out, r, b):
     res = run_q(d_in, d_out, r, b, seed=300 + r + b)
     assert res["ok"], res
     fused = b <= 16 and d_in % 256 == 0
-    assert res["launches"] == 1 if fused else res["launches"] >= 3      # else two expansions and the forward launches
+    assert res["launches"] == 1 if fused else res["launches"] >= 3      # else the expansion and the forward launches
 
 
 def test_quantized_adapter_codes_reach_the_right_rows_and_columns():

@@ -16,7 +16,7 @@ from paper_2410_09615_b200 import binding as K, build, inputs, parity
 def test_noalloc_rejects_problems_beyond_its_scratch_on_the_host():
     """Host-side checks come before any device work: a problem whose partial
     sums would not fit the built-in array is refused with SLIM_ERR_WORKSPACE,
-    one the decode kernel does not take with SLIM_ERR_UNSUPPORTED_SHAPE."""
+    one outside its shapes with SLIM_ERR_UNSUPPORTED_SHAPE."""
     build.build()
     lib = K.lib()
     fake = 4096          # aligned, never dereferenced: the call must fail before touching it
