@@ -93,7 +93,7 @@ pack_adapter_pairs_kernel(const __nv_bfloat16* A, uint32_t items, int cols, int 
 
 // Expansion to bf16 of one matrix or of a layer's two: a thread takes four bytes of codes (eight values, one 16-byte
 // store) where rows are multiples of eight elements, else four times two bytes or one.  (One byte a thread and a launch per matrix took
-// 11 us for the adapters of a 1728 -> 5120 layer, rank 176; a dependent launch of one byte a thread 11.2 us for 5000 x 1004, UN_A so.)
+// 11 us for the adapters of a 1728 -> 5120 layer, rank 176; a dependent launch of one byte a thread 11.2 us for 5000 x 1004, 4.3 so.)
 struct Unpack { const uint8_t* codes; const __nv_bfloat16* scales; __nv_bfloat16* out; int cols, groups; size_t items; };
 
 // I: the type of an item's number; TWO: two matrices.

@@ -39,7 +39,7 @@ __device__ __forceinline__ uint32_t top2(uint32_t c, const float4* x)
 
 // A thread owns V (four, or one where a row is no multiple of four groups) groups of columns and walks rows: its input
 // magnitudes stay in registers, and it has the loads of ROWS rows in flight.  A block is up to 256 V groups of columns by as many
-// rows as make up 256 threads and leave two blocks an SM (100000 x 64: 27.8 us with one row a block, MASK_A so); where blocks of
+// rows as make up 256 threads and leave two blocks an SM (100000 x 64: 27.8 us with one row a block, 4.8 so); where blocks of
 // several rows a thread would not give every SM one, a thread takes one (64 x 4096: 3.2 us with four, 2.0 so).
 template <int V> struct Words;
 template <> struct Words<4> { using T = uint4; };
