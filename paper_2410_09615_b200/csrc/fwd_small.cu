@@ -12,8 +12,8 @@
 // CTAs exchange partial sums with asynchronous remote stores, round to bf16 (TP = 2: to two bf16 numbers, keeps_T32) and publish T as
 // 8-byte words {two columns, call number}.
 //   A tile's cluster streams the packed weight and the activations through a ring of stages by TMA
-// (256 rows x 64 value bytes, x 32 index bytes, b tokens x 512 bytes; two requesting warps, since one
-// thread starts a request every 220 cycles and the engine takes about one 32-64 byte row a cycle),
+// (256 rows x 64 value bytes, x 32 index bytes, b tokens x 512 bytes; two requesting warps, since the engine takes about
+// one 32-64 byte row a cycle and a request made on a lane's number took its warp 220 cycles),
 // then the columns of L (32 of bf16, or 64 int4 codes a row and stage: codes by plain loads of the consumers, one step ahead,
 // cost 8192 -> 28672 with 16 tokens 58.7 us instead of 47.6), waiting for just the words of T it multiplies, then writes
 // Y = s X Q^T + T L^T.
@@ -166,6 +166,14 @@ __device__ __forceinline__ void tma_tile(uint32_t dst, const CUtensorMap* map, i
 __device__ __forceinline__ void tma_tile3(uint32_t dst, const CUtensorMap* map, int y, int z, uint32_t bar) {
     asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
                  :: "r"(dst), "l"(map), "r"(0), "r"(y), "r"(z), "r"(bar) : "memory");
+}
+// One lane of a warp whose lanes have all come here.  Requests are made in such a branch, from operands that are the same in all lanes: a
+// branch on the lane's number took longer (4096 -> 11008, rank 416, 16 tokens 17.1 us a call, 15.7 so; 28672 -> 8192, 16 tokens 48.9,
+// 46.6; 8192 -> 8192, rank 832, one token 18.6, 18.0).
+__device__ __forceinline__ bool elect_one() {
+    uint32_t pred;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(pred));
+    return pred != 0;
 }
 __device__ __forceinline__ void prefetch_map(const CUtensorMap* map) { asm volatile("prefetch.tensormap [%0];" :: "l"(map) : "memory"); }
 __device__ __forceinline__ void bulk_copy(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
@@ -491,7 +499,7 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
     const uint32_t part = smem + C_::kOffPart, recv = smem + C_::kOffRecv, bars = smem + C_::kOffBars;
     const uint32_t full = bars, empty = bars + 32, piece_bar = bars + 64, red_full = bars + 72, t_full = bars + 80, t_empty = bars + 144, gone = bars + 208;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;      // (a shuffle: the same in all lanes, for the compiler too)
     Lane ln; ln.lane = lane; ln.g = lane >> 2; ln.t = lane & 3;
     uint32_t C, rank;
     asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(C));
@@ -557,7 +565,7 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
             for (int u = u0; u < u1; ++u) {
                 const int st = acquire();
                 const uint32_t bar = full + 8 * st;
-                if (lane == 0) {
+                if (elect_one()) {
                     mbar_expect(bar, QA ? 4096 : 16384);
                     if (QA) tma_tile(smem + st * kStage, &tmR, u * 128, piece * kGroup, bar);
                     else tma_tile3(smem + st * kStage, &tmR, piece * kGroup, u * 4, bar);
@@ -568,12 +576,13 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
             for (int u = u0; u < u_end; ++u) {
                 const int st = acquire();
                 const uint32_t dst = smem + st * kStage, bar = full + 8 * st;
-                if (lane == 0) mbar_expect(bar, FMT == FMT_TILED ? groups * 6144 : kValsBytes);
-                if (FMT == FMT_TILED) {
-                    __syncwarp();
-                    if (lane < groups) bulk_copy(dst + lane * 6144, p.tiled + ((size_t)(tile * 4 + lane) * p.units + u) * 6144, 6144, bar);
-                } else if (lane == 0) {
-                    tma_tile(dst, &tmV, u * 64, row0, bar);
+                if (elect_one()) {
+                    mbar_expect(bar, FMT == FMT_TILED ? groups * 6144 : kValsBytes);
+                    if (FMT == FMT_TILED) {
+                        for (int i = 0; i < groups; ++i) bulk_copy(dst + i * 6144, p.tiled + ((size_t)(tile * 4 + i) * p.units + u) * 6144, 6144, bar);
+                    } else {
+                        tma_tile(dst, &tmV, u * 64, row0, bar);
+                    }
                 }
             }
             // 32 columns of L in bf16, or 64 codes a row
@@ -582,7 +591,7 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
                 const uint32_t dst = smem + st * kStage, bar = full + 8 * st;
                 if (l_by_lanes) {
                     codes_of_L(lc, dst, bar, 0);
-                } else if (lane == 0) {
+                } else if (elect_one()) {
                     mbar_expect(bar, kRows * (QA ? 32 : 64));
                     mbar_arrive(bar);                           // in place of the other producer
                     tma_tile(dst, &tmL, lc * 32, row0, bar);
@@ -598,7 +607,7 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
             for (int u = u0; u < u1; ++u) {
                 const int st = acquire();
                 const uint32_t bar = full + 8 * st;
-                if (lane == 0) {
+                if (elect_one()) {
                     mbar_expect(bar, C_::kXBytes);
                     tma_tile3(smem + st * kStage + kXOff, &tmX, 0, u * 4, bar);
                 }
@@ -630,10 +639,11 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
             for (int u = u0; u < u_end; ++u) {
                 const int st = acquire();
                 const uint32_t dst = smem + st * kStage, bar = full + 8 * st;
-                if (lane == 0) mbar_expect(bar, C_::kXBytes + (FMT == FMT_PACKED ? kMetaBytes : 0));
-                __syncwarp();
-                if (lane == 0) tma_tile3(dst + kXOff, &tmX, 0, u * 4, bar);
-                if (FMT == FMT_PACKED && lane == 1) tma_tile(dst + kValsBytes, &tmM, u * 32, row0, bar);
+                if (elect_one()) {
+                    mbar_expect(bar, C_::kXBytes + (FMT == FMT_PACKED ? kMetaBytes : 0));
+                    if (FMT == FMT_PACKED) tma_tile(dst + kValsBytes, &tmM, u * 32, row0, bar);
+                    tma_tile3(dst + kXOff, &tmX, 0, u * 4, bar);
+                }
                 if (FMT == FMT_PACKED_LD) {
                     // 256 rows x four 8-byte pieces (64 columns), stored as the TMA's 32-byte swizzle would
                     const size_t pitch = (size_t)p.d_in / 8;
