@@ -61,7 +61,7 @@ constexpr unsigned long long kWaitNs = 500ull * 1000 * 1000;
 enum { FMT_PACKED = 0, FMT_PACKED_LD = 1, FMT_TILED = 2 };   // LD: index bytes by cp.async (rows no 16-byte multiples)
 
 struct SmallParams {
-    const __nv_bfloat16* X; const uint8_t* meta; const uint8_t* tiled;
+    const __nv_bfloat16* X; const uint8_t* vals; const uint8_t* meta; const uint8_t* tiled;
     const void* L; const void* R;                             // bf16, or int4 codes
     const __nv_bfloat16* Ls; const __nv_bfloat16* Rs;         // scales of quantized adapters
     __nv_bfloat16* Y;
@@ -70,6 +70,7 @@ struct SmallParams {
     uint32_t* status;
     float s;
     int b, r, d_out, d_in;
+    bool ahead;                                               // ask the first lines into the L2 while the grid before ends
     int tiles, units, groups;                                 // of 256 rows, 256 columns, 32 rows of R
 };
 
@@ -482,6 +483,20 @@ __device__ __forceinline__ void finish(const SmallParams& p, uint32_t smem, int 
     }
 }
 
+// Asks the consumers' first lines of a matrix's rows into the L2: bytes [from, to) of `rows` rows, column by column of lines, up to eight
+// lines a thread.
+__device__ __forceinline__ void lines_ahead(const void* base, size_t pitch, int row0, int rows, size_t from, size_t to)
+{
+    constexpr uint32_t kLine = 128, kMost = 8 * kConsumers;
+    from = from / kLine * kLine;
+    to = to < pitch ? to : pitch;
+    if (from >= to || rows <= 0) return;
+    const uint32_t items = min((uint32_t)(to - from + kLine - 1) / kLine * (uint32_t)rows, kMost);
+    const char* first = static_cast<const char*>(base) + (size_t)row0 * pitch + from;
+    for (uint32_t i = threadIdx.x; i < items; i += kConsumers)
+        asm volatile("prefetch.global.L2 [%0];" :: "l"(first + (size_t)(i % (uint32_t)rows) * pitch + (size_t)(i / (uint32_t)rows) * kLine));
+}
+
 // ---------------------------------------------------------------- the kernel
 template <int NT, int FMT, bool QA, int MT, int TP>
 __global__ void __launch_bounds__(Cfg<NT, MT>::kThreads, Cfg<NT, MT>::kCtasPerSm)
@@ -530,6 +545,18 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
     // no global memory, everything below comes after that grid.  The next grid may be set up as soon as all CTAs are here.
     if (warp == kProdW && lane == 0) { prefetch_map(FMT == FMT_TILED ? &tmX : &tmV); prefetch_map(&tmR); prefetch_map(&tmL); }
     if (warp == kProdX && lane == 0) { prefetch_map(&tmX); prefetch_map(&tmM); }
+    // The first lines of this CTA's part of the weight or of R go into the L2 meanwhile.  Nothing is read by that: what the grid before still
+    // writes is what the loads behind the wait find there.
+    if (p.ahead && NT < 8 && warp < kCW) {
+        if (makes_T) {
+            const size_t unit = QA ? kUnit / 2 : kUnit * 2;
+            lines_ahead(p.R, (size_t)p.d_in * unit / kUnit, piece * kGroup, min(kGroup, p.r - piece * kGroup), u0 * unit, u1 * unit);
+        } else if (FMT != FMT_TILED) {
+            const int row0 = tile * kRows, rows = min(kRows, p.d_out - row0);
+            lines_ahead(p.vals, (size_t)p.d_in / 4, row0, rows, (size_t)u0 * 64, (size_t)u_end * 64);
+            lines_ahead(p.meta, (size_t)p.d_in / 8, row0, rows, (size_t)u0 * 32, (size_t)u_end * 32);
+        }
+    }
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (warp == kProdW || warp == kProdX) asm volatile("fence.proxy.async;" ::: "memory");      // what that grid wrote is read through TMA
@@ -1122,10 +1149,14 @@ slim_status_t launch_small(const __nv_bfloat16* X, int b, const uint8_t* vals, c
     if (!res) return SLIM_ERR_CUDA;
     if (mt == 4) C = cluster_size(res, ceil_div(d_out, rows), units);
     SmallParams p;
-    p.X = X; p.meta = meta; p.tiled = tiled; p.L = L; p.R = R; p.Ls = Ls; p.Rs = Rs; p.Y = Y;
+    p.X = X; p.vals = vals; p.meta = meta; p.tiled = tiled; p.L = L; p.R = R; p.Ls = Ls; p.Rs = Rs; p.Y = Y;
     p.departures = reinterpret_cast<unsigned long long*>(ws);
     p.T = reinterpret_cast<unsigned long long*>(reinterpret_cast<char*>(ws) + SLIM_WORKSPACE_SYNC_BYTES);
     p.status = status_dev; p.s = s; p.b = b; p.r = r; p.d_out = d_out; p.d_in = d_in;
+    // Up to 40 MB of weight the HBM is idle for much of a call (start, hand-over of T, exchange): the lines asked for ahead come for nothing
+    // (4096 x 4096, rank 416, one token 8.2 -> 7.7 us a call, 11008 -> 4096, 4 tokens 13.0 -> 12.2; 33 to 64 tokens gain nothing).  Beyond, it is
+    // busy throughout and they come in the way (28672 -> 8192, 16 tokens 49 -> 53).
+    p.ahead = (size_t)d_out * (size_t)d_in * 3 / 8 <= (size_t)40 << 20;
     p.tiles = ceil_div(d_out, rows); p.units = units; p.groups = groups;
     CUtensorMap tmV, tmM, tmX, tmR, tmL;
     bool ok = make_map3(&tmX, X, (uint64_t)d_in, (uint64_t)b, nt * 8);
