@@ -358,9 +358,9 @@ slim_kernel_t slim_select_kernel(int b, int d_out, int d_in, int r);
 int slim_last_launch_count(void);
 
 /*
- * Token-tile width (64, 128 or 256 tokens) of the prefill kernel the last slim_linear_fwd* call on this host
- * thread launched, 0 if that call ran another kernel.  The CTA-pair kernel takes the narrowest width with which
- * every tile has a pair of its own, else 256; the one-CTA kernel's is 64.  Tests use this query to
+ * Token-tile width (64, 128 or 256 tokens) of the variant of the prefill kernel that the last slim_linear_fwd* call on this host
+ * thread launched, 0 if that call ran another kernel.  The CTA-pair kernel cuts the tokens evenly into tiles of up to 256, or of 128
+ * or 64 where every tile then has a pair of its own and that is faster; the one-CTA kernel's width is 64.  Tests use this query to
  * make sure they exercise the variant they mean to.
  */
 int slim_last_token_tile(void);

@@ -105,10 +105,11 @@ struct PrefillParams {
     int meta_pitch;
     int d_in;
     // pair kernel: pairs of 128-row tiles; tiles of 256 x 256 in all
-    int row_pairs, tiles;
+    int row_pairs, tiles, half;          // half: token rows one CTA loads, half of a tile's tokens
     // T' inside the pair kernel: chunks of t_n columns (of r), tiles of 256 tokens x t_n, 64-column stages of one, pairs that
     // share the work; 1 / s; T' itself, partial tiles, and per (tile, CTA) {arrivals, ready} words that carry the call number
     int r, t_n, t_chunks, t_tiles, t_stages, t_pairs;
+    bool t_ranks;           // the MMA's rows are ranks and its columns tokens, not the other way round
     float t_scale;
     __nv_bfloat16* t_out;
     float4* t_part;
@@ -199,21 +200,32 @@ __device__ __forceinline__ void mma_sparse(uint32_t d_tmem, uint64_t a_desc, uin
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" :: "r"(s32(bar)) : "memory");
 }
-// ---- CTA-pair variants.  The sparse one reads A from tensor memory: lane = row, two stored bf16 per column.
-__device__ __forceinline__ void mma_dense2(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        :: "r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
+__device__ __forceinline__ void prefetch_map(const CUtensorMap* map) { asm volatile("prefetch.tensormap [%0];" :: "l"(map) : "memory"); }
+// A tile into the L2.
+__device__ __forceinline__ void prefetch_tile(const CUtensorMap* tmap, int x, int y) {
+    asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];" :: "l"(tmap), "r"(x), "r"(y) : "memory");
 }
-__device__ __forceinline__ void mma_sparse2(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t e_tmem,
+// ---- CTA-pair variants.  The sparse one reads A from tensor memory: lane = row, two stored bf16 per column.  Shared-memory operands are
+// given by the low word of their descriptor (128-byte rows; the high word is the same for all): the issuing warp shares its scheduler with the
+// converters, and what it spends on a stage is instructions.
+constexpr uint32_t kDescHi = (uint32_t)(1024 >> 4) | (1u << 14) | (2u << 29);
+__device__ __forceinline__ uint32_t desc_lo(uint32_t saddr) { return ((saddr & 0x3FFFFu) >> 4) | (1u << 16); }
+__device__ __forceinline__ void mma_dense2(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t idesc, uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b64 a, b;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "mov.b64 a, {%1, %5};\n\tmov.b64 b, {%2, %5};\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], a, b, %3, p;\n\t}"
+        :: "r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(idesc), "r"(accumulate), "r"(kDescHi) : "memory");
+}
+__device__ __forceinline__ void mma_sparse2(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t e_tmem,
                                             uint32_t idesc, uint32_t accumulate) {
     asm volatile(
-        "{\n\t.reg .pred p;\n\t"
+        "{\n\t.reg .pred p;\n\t.reg .b64 b;\n\t"
         "setp.ne.b32 p, %5, 0;\n\t"
-        "tcgen05.mma.sp.cta_group::2.kind::f16 [%0], [%1], %2, [%3], %4, p;\n\t}"
-        :: "r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(e_tmem), "r"(idesc), "r"(accumulate) : "memory");
+        "mov.b64 b, {%2, %6};\n\t"
+        "tcgen05.mma.sp.cta_group::2.kind::f16 [%0], [%1], b, [%3], %4, p;\n\t}"
+        :: "r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(e_tmem), "r"(idesc), "r"(accumulate), "r"(kDescHi) : "memory");
 }
 // The same for a pair's loads: the bytes are counted on the even CTA's barrier.
 __device__ __forceinline__ void tma_tile_pair(void* dst, const CUtensorMap* tmap, int x, int y, uint32_t cluster_bar_addr) {
@@ -345,20 +357,23 @@ __device__ __forceinline__ void load_packed(const PrefillParams& p, const CUtens
                                             uint64_t* full, int kg, int m0, int lane)
 {
     using namespace pf;
-    if (lane == 0) mbar_expect_tx(full, (uint32_t)(p.meta ? kValsTile : kPkSlotBytes));
-    // lanes 0 and 1 request the value-byte and the index-byte tile with one instruction
-    if (lane < (p.meta ? 1 : 2)) tma_tile(slot + (lane == 0 ? 0 : kValsTile), lane == 0 ? tmV : tmM, kg * (lane == 0 ? 64 : 32), m0, full);
+    if (elect_one()) {
+        mbar_expect_tx(full, (uint32_t)(p.meta ? kValsTile : kPkSlotBytes));
+        tma_tile(slot, tmV, kg * 64, m0, full);
+        if (!p.meta) tma_tile(slot + kValsTile, tmM, kg * 32, m0, full);
+    }
     if (p.meta) {
-        // 128 rows x four 8-byte pieces (64 columns each), stored as the TMA's 32-byte swizzle would
-        const int q = lane & 3;
+        // 128 rows x four 8-byte pieces (64 columns each), stored as the TMA's 32-byte swizzle would: a lane has the rows r0 + 8 i, which all
+        // have the same swizzle
+        const int q = lane & 3, r0 = lane >> 2;
         const bool col_in = kg * 32 + q * 8 < p.meta_pitch;
-#pragma unroll 4
-        for (int r = lane >> 2; r < kPM; r += 8) {
-            const bool in = col_in && m0 + r < p.m_total;
-            const uint8_t* src = p.meta + (in ? (size_t)(m0 + r) * p.meta_pitch + kg * 32 + q * 8 : 0);
-            const uint32_t d = s32(slot + kValsTile) + r * 32 + ((((q >> 1) ^ (r >> 2)) & 1) << 4) + (q & 1) * 8;
-            asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" :: "r"(d), "l"(src), "r"(in ? 8 : 0) : "memory");
-        }
+        const int rows = col_in ? (p.m_total - m0 - r0 + 7) / 8 : 0;
+        const uint8_t* src = p.meta + (rows > 0 ? (size_t)(m0 + r0) * p.meta_pitch + kg * 32 + q * 8 : 0);
+        const size_t step = rows > 0 ? (size_t)8 * p.meta_pitch : 0;
+        const uint32_t d = s32(slot + kValsTile) + r0 * 32 + ((((q >> 1) ^ (r0 >> 2)) & 1) << 4) + (q & 1) * 8;
+#pragma unroll
+        for (int i = 0; i < kPM / 8; ++i, src += i < rows ? step : 0)
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" :: "r"(d + i * 256), "l"(src), "r"(i < rows ? 8 : 0) : "memory");
         asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" :: "r"(s32(full)) : "memory");
     }
 }
@@ -637,35 +652,41 @@ prefill_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap tmV,
 // 128 tokens a thread; the next tile's MMAs may start as soon as it is in registers, the stores follow beside
 // them.  A CTA per tile spent 4.4 us on start-up and 2.3 us on the epilogue of every tile, with the tensor
 // core idle.
-// Warps: 0-7 converters (two groups on alternate stages), 8-15 epilogue, 16 and 17 token tiles (and A2 / B2) of even and odd
-// stages, 18 MMA issue, 19 packed tiles.
+// Warps: 0-15 converters (four groups, stages in turn), 16-23 epilogue, 24 and 25 token tiles (sparse stages in turn; in the others one
+// requests A, one B), 26 MMA issue, 27 packed tiles.
 //
-// T' = (X R^T) / s is made by the same pairs first: tiles of 256 tokens x t_n columns of r (the tokens are the MMA's rows),
+// T' = (X R^T) / s is made by the same pairs first: tiles of 256 tokens x t_n columns of r (the tokens are the MMA's rows), or of 256 ranks x
+// the tokens of a narrow tile (t_ranks),
 // whose 64-column stages are dealt out evenly in one list, so that every pair gets the same share whatever the number
 // of tiles.  Pairs that share a tile leave their parts as fp32 in the workspace; when all are there, each of them adds up a
 // share of the columns, in list order, and rounds to bf16.  The main tiles wait for the T' they read just before their
 // first adapter stage.  As a launch of its own (and a reduction behind it) T' took 12 us and more of most calls.
 //
-// N = tokens of a tile: 256, 128 or 64.  A stage takes the same 0.36 us for each of them (the MMAs' 256 weight rows cost what
-// they cost), so a narrower tile only saves epilogue and token traffic.  A stage is 32 KB for every N (what T' needs).
-// Five stages and four packed tiles in flight: 33.2 -> 32.0 us on 8192 x 8192, 333 tokens, 91 -> 83 us on 28672 -> 8192, 64
-// tokens, against six and two (calls on one weight, which stays in the L2; with weights in rotation the first takes 36).
-// Stages alternate between two converter groups and two token-tile warps while their number is odd, so each of them sees
-// every second phase of an `empty` barrier.  Waiting by parity is still right: before its stage g such a warp has waited
-// for the MMAs of stage g - 7, so the phase it did not see (stage g - 10) is over.  For the packed tiles' barriers the same holds
-// with four slots: a group that has no stage of a packed tile (the second of a last, half tile) next looks at that slot
-// seven stages later or more.
+// N = most tokens of a tile: 256, 128 or 64 (half: half of those that it has).  The sparse MMA of 256 x N x 32 takes N / 2 cycles.  What held
+// a stage at 690 cycles whatever N was what stands around it, each worth little without the others:
+//   - the issuing thread: a lane walking alone needed 120 cycles an MMA and 400 and more for its barriers; a warp that walks together, asks
+//     ahead and adds to the low words of its descriptors 300-400 a stage;
+//   - the converters: a group takes 1400 cycles from packed bytes to the arrival, so four groups instead of two;
+//   - the packed ring: 48 KB an SM, less than the HBM's latency asks for: a pair's first tile is asked into the L2 ahead.
+// With up to 128 tokens a stage is a whole packed tile of 256 columns (the smaller accumulator leaves the tensor memory for it): half the
+// barriers and commits a column.  8192 x 8192 without adapters, weights in rotation: 128 tokens 28.5 -> 22.3 us, 333 tokens 32.3 -> 27.8;
+// 8192 -> 28672, rank 832, 40 tokens 78 -> 61; 13824 -> 5120, rank 512, 900 tokens 115 -> 110.
+// What bounds it now: with 256 tokens 0.36-0.40 us a stage of 128 columns, of which the MMAs take 0.27 (the shared-memory port is busy for 0.31:
+// TMA writes 38 KB, converters read 6, tensor core reads 32); with 128 tokens 0.25.
+// A token-tile warp sees every second phase of an `empty` barrier.  Waiting by parity is still right: before its stage g it has waited
+// for the MMAs of stage g - 7, so the phase it did not see (stage g - 10) is over.
 constexpr int kTTok = 256;              // tokens of a T' tile (the rows of its MMA)
-constexpr int kPairThreads = 20 * 32;
+constexpr int kPairThreads = 28 * 32;
 template <int N> struct PairCfg {
-    static constexpr int kWarpX = 16, kWarpMma = 18, kWarpPk = 19;
-    static constexpr int kSK = 128, kDK = 64, kStages = 5, kPkSlots = 4, kPkStages = kPkCols / kSK;
-    static constexpr int kHalfTok = N / 2;                                  // token rows this CTA loads
-    static constexpr int kBTile = kHalfTok * kSK * 2, kStageBytes = 32768, kATileAt = kStageBytes / 2;     // dense stages and T': B, then A
-    // tensor memory: the accumulator (a T' tile's is 256 columns too), index words (4 columns a stage), expanded weights (32
+    static constexpr int kGroups = 4, kWarpEpi = 4 * kGroups, kWarpX = kWarpEpi + 8, kWarpMma = kWarpX + 2, kWarpPk = kWarpX + 3;
+    static constexpr int kSK = N <= 128 ? 256 : 128, kDK = 64, kStages = 5, kPkSlots = 4, kPkStages = kPkCols / kSK;
+    static constexpr int kStageBytes = 32768, kATileAt = kStageBytes / 2;     // dense stages and T': B, then A
+    // tensor memory: the accumulator (a T' tile's may be as wide), index words (kSK / 32 columns a stage), expanded weights (kSK / 4
     // columns a stage)
-    static constexpr int kECol = 256, kACol = 256 + 32;
+    static constexpr int kECols = kSK / 32, kACols = kSK / 4, kECol = N <= 128 ? 128 : 256, kACol = N <= 128 ? 192 : 288;
+    static constexpr int kTWidth = kECol;                                   // most columns of r in a T' tile
     static constexpr size_t kSmem = 1024 + (size_t)kStages * kStageBytes + kPkSlots * kPkSlotBytes + 384 + 8 * 1024;     // .. barriers, epilogue
+    static_assert(kECol + kStages * kECols <= kACol && kACol + kStages * kACols <= 512, "tensor memory");
 };
 constexpr size_t kSyncTiles = kSmallTBytes / 16 - 1024;     // T' tiles whose words fit the region beside those of the pairs
 
@@ -711,19 +732,19 @@ template <int N>
 __global__ void __launch_bounds__(kPairThreads, 1)
 prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmM,
                     const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmA2, const __grid_constant__ CUtensorMap tmB2,
-                    const __grid_constant__ CUtensorMap tmR, const __grid_constant__ CUtensorMap tmXt)
+                    const __grid_constant__ CUtensorMap tmTA, const __grid_constant__ CUtensorMap tmTB)
 {
     using namespace pf;
     using Cfg = PairCfg<N>;
     constexpr int kStages = Cfg::kStages, kPkSlots = Cfg::kPkSlots, kPkStages = Cfg::kPkStages, kSK = Cfg::kSK, kDK = Cfg::kDK;
-    constexpr int kBTile = Cfg::kBTile, kStageBytes = Cfg::kStageBytes, kECol = Cfg::kECol, kHalfTok = Cfg::kHalfTok;
+    constexpr int kStageBytes = Cfg::kStageBytes, kECol = Cfg::kECol;
+    const int half_tok = p.half;
     extern __shared__ unsigned char smem_raw[];
     // layout: stages | packed slots {value bytes | index bytes} | barriers
     unsigned char* stages = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     unsigned char* packed = stages + (size_t)kStages * kStageBytes;
-    uint64_t* b_full = reinterpret_cast<uint64_t*>(packed + kPkSlots * kPkSlotBytes);   // [kStages] even CTA: both CTAs' tiles landed
-    uint64_t* conv_done = b_full + kStages;          // [kStages] even CTA: both CTAs' converters are done with the stage
-    uint64_t* empty = conv_done + kStages;           // [kStages] the MMAs that read the stage are complete
+    uint64_t* full = reinterpret_cast<uint64_t*>(packed + kPkSlots * kPkSlotBytes);     // [kStages] even CTA: both CTAs' tiles landed, both CTAs' converters are done
+    uint64_t* empty = full + kStages;                // [kStages] the MMAs that read the stage are complete
     uint64_t* pk_full = empty + kStages;             // [kPkSlots]
     uint64_t* pk_empty = pk_full + kPkSlots;         // [kPkSlots]
     uint64_t* acc_full = pk_empty + kPkSlots;        // a tile's MMAs are complete
@@ -731,7 +752,7 @@ prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap t
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 1);
     volatile uint32_t* abort_flag = tmem_slot + 1;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;      // (a shuffle: the same in all lanes, for the compiler too)
     const uint32_t rank = cluster_rank();
     const int pairs = gridDim.x >> 1, first_tile = blockIdx.x >> 1;
     const int n_total = p.n1 + p.n2, n_groups = ceil_div(p.n1, kPkStages);
@@ -740,13 +761,15 @@ prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap t
     const int t_begin = tq < p.t_pairs ? share_begin(tq, t_units, p.t_pairs) : 0, t_end = tq < p.t_pairs ? share_begin(tq + 1, t_units, p.t_pairs) : 0;
 
     if (threadIdx.x == 0) {
-        for (int i = 0; i < kStages; ++i) { mbar_init(&b_full[i], 1); mbar_init(&conv_done[i], kConvWarps); mbar_init(&empty[i], 1); }
-        for (int i = 0; i < kPkSlots; ++i) { mbar_init(&pk_full[i], p.meta ? 33 : 1); mbar_init(&pk_empty[i], kConvWarps); }
+        for (int i = 0; i < kStages; ++i) { mbar_init(&full[i], 8); mbar_init(&empty[i], 1); }
+        for (int i = 0; i < kPkSlots; ++i) { mbar_init(&pk_full[i], p.meta ? 33 : 1); mbar_init(&pk_empty[i], 4 * kPkStages); }
         mbar_init(acc_full, 1);
         mbar_init(acc_empty, 16);
         *abort_flag = 0u;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    if (warp == Cfg::kWarpPk && elect_one()) { prefetch_map(&tmV); prefetch_map(&tmM); prefetch_map(&tmA2); }
+    if (warp == Cfg::kWarpX && elect_one()) { prefetch_map(&tmX); prefetch_map(&tmTA); prefetch_map(&tmTB); prefetch_map(&tmB2); }
     cluster_sync_all();                              // both CTAs' barriers exist before anything crosses
     if (warp == Cfg::kWarpMma) {
         asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" :: "r"(s32(tmem_slot)), "r"(512) : "memory");
@@ -755,7 +778,7 @@ prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap t
     fence_before_sync();
     __syncthreads();
     fence_after_sync();
-    const uint32_t tmem_base = *reinterpret_cast<volatile uint32_t*>(tmem_slot);
+    const uint32_t tmem_base = __shfl_sync(0xffffffffu, *reinterpret_cast<volatile uint32_t*>(tmem_slot), 0);
     // Launched while the grid before it in the stream still runs (programmatic dependent launch): everything above needs no
     // global memory, everything below comes after that grid.
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -763,84 +786,97 @@ prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap t
     asm volatile("fence.proxy.async;" ::: "memory");            // what that grid wrote is read through TMA
     const uint32_t call = p.r > 0 ? call_number(*(volatile unsigned long long*)p.departures) : 0u;
     bool ok = true;
+    // Which 256 rows of its A operand a T' tile is made of, and which t_n rows of its B operand.
+    auto t_part_of = [&](int tile, bool a) { return a != p.t_ranks ? tile / p.t_chunks : tile % p.t_chunks; };
     // Tile -> its first row in this CTA, its first token, and where its walk over the weight columns starts: pairs that share
     // token rows start at different places, so that at any moment they ask the L2 for different lines of X.
     struct Tile { int m0, n0, rot; };
     auto tile_of = [&](int t) {
         const int rp = t % p.row_pairs, tt = t / p.row_pairs;
         Tile ti;
-        ti.m0 = (2 * rp + (int)rank) * kPM; ti.n0 = tt * N;
+        ti.m0 = (2 * rp + (int)rank) * kPM; ti.n0 = tt * 2 * half_tok;
         ti.rot = p.d_in % kPkCols == 0 && n_groups > 0 ? (rp + 3 * tt) % n_groups : 0;       // whole packed tiles
         return ti;
     };
 
     if (warp == Cfg::kWarpX || warp == Cfg::kWarpX + 1) {
         // ============================ token tiles, A2, B2 ============================
-        // Each of the two warps takes every second stage: a wait, an expectation and a request take one warp 400 ns, more than the
-        // MMAs of a stage.
+        // Two warps: they take the sparse stages in turn, and in the stages of T' and of the adapters one requests A and the other B.  (So the
+        // tiles of L are on their way while T' is waited for.)
         const int odd = warp - Cfg::kWarpX;
         int g = 0;                                          // stages so far
         int t_checked = -1;                                 // the token tile whose T' was found complete
+        auto slot_of = [&](int stage) {                     // waits for the stage's place in the ring
+            const int st = stage % kStages;
+            if (stage >= kStages) ok = mbar_wait(&empty[st], ((stage / kStages) & 1) ^ 1, abort_flag) && ok;
+            return st;
+        };
         for (int u = t_begin; u < t_end;) {
-            // T': 128 tokens x 64 columns of X as A, half of the chunk's rows of R as B
+            // T': 128 rows x 64 columns of X (or R) as A, half of the chunk's rows of R (the tile's tokens of X) as B
             const Run run = run_at(u, t_end, p.t_stages);
-            const int tok = (run.tile / p.t_chunks) * kTTok + (int)rank * kPM, col = (run.tile % p.t_chunks) * p.t_n;
-            for (int it = (g ^ odd) & 1; it < run.len; it += 2) {
-                const int st = (g + it) % kStages;
-                if (g + it >= kStages) ok = mbar_wait(&empty[st], (((g + it) / kStages) & 1) ^ 1, abort_flag) && ok;
-                if (lane == 0 && rank == 0) mbar_expect_tx(&b_full[st], (uint32_t)(2 * (kPM + p.t_n / 2) * kDK * 2));
+            const int a_row = t_part_of(run.tile, true) * kTTok + (int)rank * kPM, b_row = t_part_of(run.tile, false) * p.t_n + (int)rank * (p.t_n / 2);
+            for (int it = 0; it < run.len; ++it) {
+                const int st = slot_of(g + it);
                 unsigned char* sbase = stages + (size_t)st * kStageBytes;
-                if (lane < 2)
-                    tma_tile_pair(lane == 0 ? sbase + Cfg::kATileAt : sbase, lane == 0 ? &tmXt : &tmR, (run.k0 + it) * kDK,
-                                  lane == 0 ? tok : col + (int)rank * (p.t_n / 2), peer_addr(&b_full[st], 0));
+                if (elect_one()) {
+                    if (odd) tma_tile_pair(sbase, &tmTB, (run.k0 + it) * kDK, b_row, peer_addr(&full[st], 0));
+                    else     tma_tile_pair(sbase + Cfg::kATileAt, &tmTA, (run.k0 + it) * kDK, a_row, peer_addr(&full[st], 0));
+                }
             }
             u += run.len; g += run.len;
         }
         for (int t = first_tile; t < p.tiles; t += pairs) {
             const Tile ti = tile_of(t);
-            for (int it = (g ^ odd) & 1; it < n_total; it += 2) {
-                const int st = (g + it) % kStages;
-                const bool sparse = it < p.n1;
-                if (!sparse) {
-                    // the T' of this CTA's half of the tokens is complete (a word per part of its chunks, 32 at a time)
+            // a sparse stage's token tile: sub-tiles of 64 columns in one box
+            for (int it = (g ^ odd) & 1; it < p.n1; it += 2) {
+                const int st = slot_of(g + it);
+                int kb = it + ti.rot * kPkStages;
+                if (kb >= p.n1) kb -= p.n1;
+                if (elect_one()) tma_tile_pair3(stages + (size_t)st * kStageBytes, &tmX, ti.n0 + (int)rank * half_tok, kb * (kSK / kPBK), peer_addr(&full[st], 0));
+            }
+            for (int it = p.n1; it < n_total; ++it) {
+                if (odd) {
+                    // the T' of this CTA's half of the tokens is complete (a word per part of its tiles, 32 at a time)
                     if (ti.n0 != t_checked) {
-                        const int tile0 = (ti.n0 / kTTok) * p.t_chunks;
-                        const uint32_t t_half = (uint32_t)(ti.n0 % kTTok + (int)rank * kHalfTok) / kPM;
-                        for (int first = 0, left = 1; left > 0; first += 32) {
-                            int i = first + lane;
-                            const unsigned long long* w = nullptr;
-                            left = -first - 32;
-                            for (int c = 0; c < p.t_chunks; ++c) {
-                                const int q0 = share_owner((tile0 + c) * p.t_stages, t_units, p.t_pairs), q1 = share_owner((tile0 + c + 1) * p.t_stages - 1, t_units, p.t_pairs);
-                                if (i >= 0 && i <= q1 - q0) w = p.t_sync + (q0 == q1 ? tile_word(p.t_pairs, tile0 + c, t_half) : part_word(q0 + i, i == 0, t_half) + 1);
-                                i -= q1 - q0 + 1; left += q1 - q0 + 1;
+                        // T' tiles of 256 tokens: one or two halves of them; T' tiles of this tile's tokens: both halves of the ranks
+                        const int tok = ti.n0 + (int)rank * half_tok;
+                        const int blk0 = p.t_ranks ? ti.n0 / half_tok : tok / kPM, blk1 = p.t_ranks ? blk0 + 2 : ceil_div(min(tok + half_tok, p.b), kPM);
+                        for (int blk = blk0; blk < blk1; ++blk) {
+                            const int tile0 = (blk / 2) * p.t_chunks;
+                            const uint32_t t_half = (uint32_t)blk & 1;
+                            for (int first = 0, left = 1; left > 0; first += 32) {
+                                int i = first + lane;
+                                const unsigned long long* w = nullptr;
+                                left = -first - 32;
+                                for (int c = 0; c < p.t_chunks; ++c) {
+                                    const int q0 = share_owner((tile0 + c) * p.t_stages, t_units, p.t_pairs), q1 = share_owner((tile0 + c + 1) * p.t_stages - 1, t_units, p.t_pairs);
+                                    if (i >= 0 && i <= q1 - q0) w = p.t_sync + (q0 == q1 ? tile_word(p.t_pairs, tile0 + c, t_half) : part_word(q0 + i, i == 0, t_half) + 1);
+                                    i -= q1 - q0 + 1; left += q1 - q0 + 1;
+                                }
+                                ok = wait_words(w, call, abort_flag) && ok;
                             }
-                            ok = wait_words(w, call, abort_flag) && ok;
                         }
                         t_checked = ti.n0;
                         __syncwarp();
                         asm volatile("fence.proxy.async;" ::: "memory");   // the tiles are read by the async proxy
                     }
                 }
-                if (g + it >= kStages) ok = mbar_wait(&empty[st], (((g + it) / kStages) & 1) ^ 1, abort_flag) && ok;
-                // both CTAs' bytes are counted on the even CTA's barrier
-                if (lane == 0 && rank == 0) mbar_expect_tx(&b_full[st], (uint32_t)(2 * (sparse ? kBTile : (kHalfTok + kPM) * kDK * 2)));
+                const int st = slot_of(g + it);
                 unsigned char* sbase = stages + (size_t)st * kStageBytes;
-                int kb = sparse ? it + ti.rot * kPkStages : it - p.n1, y = ti.n0 + (int)rank * kHalfTok;
-                if (sparse && kb >= p.n1) kb -= p.n1;
-                if (!sparse && p.t_parts == 2) { y += (kb & 1) * p.b; kb >>= 1; }        // a column block of either part in turn
-                const int k = kb * (sparse ? kSK : kDK);
-                // sparse stage: the token tile, two sub-tiles of 64 columns in one box; dense stage: lane 0 the token tile, lane 1 the A2 tile
-                if (sparse) {
-                    if (lane == 0) tma_tile_pair3(sbase, &tmX, y, k / kPBK, peer_addr(&b_full[st], 0));
-                } else if (lane < 2) {
-                    tma_tile_pair(sbase + (lane == 0 ? 0 : Cfg::kATileAt), lane == 0 ? &tmB2 : &tmA2, k, lane == 0 ? y : ti.m0, peer_addr(&b_full[st], 0));
+                int kb = it - p.n1, y = ti.n0 + (int)rank * half_tok;
+                if (p.t_parts == 2) { y += (kb & 1) * p.b; kb >>= 1; }       // a column block of either part in turn
+                if (elect_one()) {
+                    if (odd) tma_tile_pair(sbase, &tmB2, kb * kDK, y, peer_addr(&full[st], 0));
+                    else     tma_tile_pair(sbase + Cfg::kATileAt, &tmA2, kb * kDK, ti.m0, peer_addr(&full[st], 0));
                 }
             }
             g += n_total;
         }
     } else if (warp == Cfg::kWarpPk) {
         // ============================ packed tiles ============================
+        // The ring holds 48 KB, less than what is under way from the HBM to an SM at full rate: a pair's first tile asks its packed tiles into
+        // the L2 kAhead before their turn (not where the index bytes keep this warp busy).
+        constexpr int kAhead = 6;
         int g = 0;
         for (int t = first_tile; t < p.tiles; t += pairs) {
             const Tile ti = tile_of(t);
@@ -849,129 +885,185 @@ prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap t
                 const int kg = i + ti.rot < n_groups ? i + ti.rot : i + ti.rot - n_groups;
                 if (g >= kPkSlots) ok = mbar_wait(&pk_empty[slot], ((g / kPkSlots) & 1) ^ 1, abort_flag) && ok;
                 load_packed(p, &tmV, &tmM, packed + slot * kPkSlotBytes, &pk_full[slot], kg, ti.m0, lane);
+                if (!p.meta && t == first_tile && i + kAhead < n_groups && elect_one()) {
+                    const int ka = i + kAhead + ti.rot < n_groups ? i + kAhead + ti.rot : i + kAhead + ti.rot - n_groups;
+                    prefetch_tile(&tmV, ka * 64, ti.m0);
+                    prefetch_tile(&tmM, ka * 32, ti.m0);
+                }
             }
         }
     } else if (warp == Cfg::kWarpMma) {
-        // ============================ MMA issue: one thread of the even CTA ============================
-        if (rank == 0 && elect_one()) {
-            constexpr uint32_t idesc = idesc_bf16(2 * kPM, N);
-            uint32_t pre = 0;       // the coming stage was found ready by an early test
-            int g = 0, nth = 0;
+        // ============================ MMA issue: a warp of the even CTA ============================
+        // The whole warp walks the stages together and one elected lane issues a stage's MMAs: what they are given is then known to be
+        // the same in all lanes.  (One lane walking alone took 120 cycles for each MMA, 700 and more a stage, whatever N.)  The next
+        // stage is asked about before this one's MMAs are issued: the answer of the barrier takes 200 cycles.
+        if (rank == 0) {
+            const uint32_t idesc = idesc_bf16(2 * kPM, 16) + ((uint32_t)((half_tok - 8) >> 2) << 17);
+            int st = 0, nth = 0;
+            uint32_t parity = 0, pre = 0;
+            auto ready = [&] {
+                if (!__all_sync(0xffffffffu, pre)) ok = mbar_wait_all(&full[st], parity, true, nullptr, 0, false, nullptr, 0, false, abort_flag) && ok;
+                fence_after_sync();
+                const bool wraps = st + 1 == kStages;
+                pre = mbar_test(&full[wraps ? 0 : st + 1], wraps ? parity ^ 1 : parity, true);
+            };
+            auto next = [&] { if (++st == kStages) { st = 0; parity ^= 1; } };
+            const uint32_t lo_first = desc_lo(s32(stages)), lo_sub = (uint32_t)half_tok * (128 >> 4);
+            constexpr uint32_t kLoStage = kStageBytes >> 4, kLoA = Cfg::kATileAt >> 4;
+            auto dense_stage = [&](uint32_t idesc_d, bool adds) {
+                const uint32_t lo = lo_first + (uint32_t)st * kLoStage;
+                if (elect_one()) {
+#pragma unroll
+                    for (int j = 0; j < kDK / 16; ++j) mma_dense2(tmem_base, lo + kLoA + 2 * j, lo + 2 * j, idesc_d, j > 0 || adds ? 1u : 0u);
+                    mma_commit2(&empty[st]);            // the stage is free, in both CTAs, once these MMAs have read it
+                }
+            };
             for (int u = t_begin; u < t_end; ++nth) {
                 const uint32_t idesc_t = idesc_bf16(2 * kPM, 16) + ((uint32_t)((p.t_n - 16) >> 3) << 17);
                 const Run run = run_at(u, t_end, p.t_stages);
                 if (nth > 0) ok = mbar_wait_all(acc_empty, (nth & 1) ^ 1, true, nullptr, 0, false, nullptr, 0, false, abort_flag) && ok;
-                for (int it = 0; it < run.len; ++it, ++g) {
-                    const int st = g % kStages;
-                    const uint32_t parity = (g / kStages) & 1;
-                    ok = mbar_wait_all(&b_full[st], parity, true, &conv_done[st], parity, true, nullptr, 0, false, abort_flag) && ok;
-                    fence_after_sync();
-                    const uint32_t b_addr = s32(stages + (size_t)st * kStageBytes), a_addr = b_addr + Cfg::kATileAt;
-#pragma unroll
-                    for (int j = 0; j < kDK / 16; ++j)
-                        mma_dense2(tmem_base, smem_desc(a_addr + 32 * j), smem_desc(b_addr + 32 * j), idesc_t, it > 0 || j > 0 ? 1u : 0u);
-                    mma_commit2(&empty[st]);
-                }
-                mma_commit2(acc_full);
+                for (int it = 0; it < run.len; ++it) { ready(); dense_stage(idesc_t, it > 0); next(); }
+                if (elect_one()) mma_commit2(acc_full);
                 u += run.len;
             }
             for (int t = first_tile; t < p.tiles; t += pairs, ++nth) {
                 if (nth > 0) ok = mbar_wait_all(acc_empty, (nth & 1) ^ 1, true, nullptr, 0, false, nullptr, 0, false, abort_flag) && ok;
-                for (int it = 0; it < n_total; ++it, ++g) {
-                    const int st = g % kStages;
-                    const uint32_t parity = (g / kStages) & 1;
-                    const bool sparse = it < p.n1;
-                    if (!pre)
-                        ok = mbar_wait_all(&b_full[st], parity, true, &conv_done[st], parity, true, nullptr, 0, false, abort_flag) && ok;
-                    fence_after_sync();
-                    // ask about the next stage now, without waiting: the answer comes back while this stage's MMAs are issued
-                    const int st1 = (g + 1) % kStages;
-                    const uint32_t par1 = ((g + 1) / kStages) & 1;
-                    pre = mbar_test(&b_full[st1], par1, true) & mbar_test(&conv_done[st1], par1, true);
-                    const uint32_t b_addr = s32(stages + (size_t)st * kStageBytes), a_addr = b_addr + Cfg::kATileAt;
-                    if (sparse) {
+                for (int it = 0; it < p.n1; ++it) {
+                    ready();
+                    const uint32_t lo = lo_first + (uint32_t)st * kLoStage, a = tmem_base + Cfg::kACol + Cfg::kACols * st, e = tmem_base + kECol + Cfg::kECols * st;
+                    if (elect_one()) {
                         // per MMA: A 16 stored bf16 (8 columns of tensor memory), B 32 columns (64 bytes)
 #pragma unroll
                         for (int j = 0; j < kSK / 32; ++j)
-                            mma_sparse2(tmem_base, tmem_base + Cfg::kACol + 32 * st + 8 * j, smem_desc(b_addr + (j >> 1) * (kHalfTok * 128) + 64 * (j & 1)),
-                                        tmem_base + kECol + 4 * st + 2 * (j >> 1), idesc | (1u << 2) | (uint32_t)(j & 1), it > 0 || j > 0 ? 1u : 0u);
-                    } else {
-#pragma unroll
-                        for (int j = 0; j < kDK / 16; ++j)
-                            mma_dense2(tmem_base, smem_desc(a_addr + 32 * j), smem_desc(b_addr + 32 * j), idesc, it > 0 || j > 0 ? 1u : 0u);
+                            mma_sparse2(tmem_base, a + 8 * j, lo + (j >> 1) * lo_sub + 4 * (j & 1), e + 2 * (j >> 1), idesc | (1u << 2) | (uint32_t)(j & 1), j > 0 || it > 0 ? 1u : 0u);
+                        mma_commit2(&empty[st]);
                     }
-                    mma_commit2(&empty[st]);            // the stage is free, in both CTAs, once these MMAs have read it
+                    next();
                 }
-                mma_commit2(acc_full);
+                for (int it = p.n1; it < n_total; ++it) { ready(); dense_stage(idesc, it > 0); next(); }
+                if (elect_one()) mma_commit2(acc_full);
             }
         }
-    } else if (warp < kConvWarps) {
+    } else if (warp < Cfg::kWarpEpi) {
         // ============================ converters ============================
         // Within a group of four warps a thread owns one weight row of the tile.
         const int row = threadIdx.x & 127;           // weight row inside the tile = TMEM lane
-        const int half = threadIdx.x >> 7;
+        constexpr int kGroups = Cfg::kGroups;
+        const int group = threadIdx.x >> 7;
         const int x = (row >> 3) & 1;
         const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
-        // nothing to expand for T' and in phase 2: the arrival keeps the barrier's phases in step with the stages
-        auto pass = [&](int g) {
+        // A stage is full when both CTAs' converters have arrived and the bytes have landed that one of the warps announces with its
+        // arrival (bytes that land before are counted below zero; the phase cannot end without the arrivals).
+        auto arrive = [&](int st, uint32_t bytes) {
+            __syncwarp();
+            if (lane == 0) {
+                if (rank != 0) mbar_arrive_remote(peer_addr(&full[st], 0));
+                else if ((warp & 3) == 0) mbar_expect_tx(&full[st], bytes);
+                else mbar_arrive(&full[st]);
+            }
+        };
+        // nothing to expand for T' and in phase 2
+        auto pass = [&](int g, uint32_t bytes) {
             const int st = g % kStages;
             if (g >= kStages) ok = mbar_wait(&empty[st], ((g / kStages) & 1) ^ 1, abort_flag) && ok;
-            if (lane == 0) mbar_arrive_remote(peer_addr(&conv_done[st], 0));
-            __syncwarp();
+            arrive(st, bytes);
+        };
+        // Whether a phase has ended, as lane 0 finds it; the answer is looked at later.
+        auto ask = [&](uint64_t* bar, uint32_t phase) { return lane == 0 ? mbar_test(bar, phase, false) : 0u; };
+        auto yes = [&](uint32_t answer) { return __shfl_sync(0xffffffffu, answer, 0) != 0; };
+        // The groups take turns.  A group waits by parity for the MMAs of stage g - 5, which is right when it knows those of stage g - 10 to be
+        // complete and those of g are still to come: with turns of at most five stages.  Where a turn is longer (from T' to the first tile,
+        // from tile to tile) it waits for another group's stage in between.
+        int last = -1;
+        auto turn_at = [&](int g) {
+            while (g - last > kStages) {
+                last += kGroups;
+                if (last >= kStages) ok = mbar_wait(&empty[last % kStages], ((last / kStages) & 1) ^ 1, abort_flag) && ok;
+            }
+            last = g;
         };
         int base = t_end - t_begin, nth = 0;         // stages before this tile
-        for (int g = half; g < base; g += 2) pass(g);
+        for (int g = group; g < base; g += kGroups) { turn_at(g); pass(g, (uint32_t)(2 * (kPM + p.t_n / 2) * kDK * 2)); }
+        uint32_t pk_there = 0;
         for (int t = first_tile; t < p.tiles; t += pairs, base += n_total, ++nth) {
             const bool row_in = tile_of(t).m0 + row < p.m_total;
-            for (int it = (base ^ half) & 1; it < n_total; it += 2) {
+            // (turns go by the packed tiles: a group sees every phase of their barriers that it has a stage of)
+            const int all = max(n_total, n_groups * kPkStages);
+            for (int it = (group - nth * n_groups * kPkStages) & (kGroups - 1); it < all; it += kGroups) {
+                if (it >= p.n1) {
+                    if (it < n_groups * kPkStages) {                         // the second half of a last, half packed tile: seen, and given back
+                        const int gi = (nth + 1) * n_groups - 1, slot = gi % kPkSlots;
+                        if (!yes(pk_there)) ok = mbar_wait(&pk_full[slot], (gi / kPkSlots) & 1, abort_flag) && ok;
+                        pk_there = 0;
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(&pk_empty[slot]);
+                    }
+                    if (it < n_total) { turn_at(base + it); pass(base + it, (uint32_t)(2 * (half_tok + kPM) * kDK * 2)); }
+                    continue;
+                }
+                turn_at(base + it);
                 const int g = base + it, st = g % kStages;
-                if (it < p.n1) {
-                    // expand into registers as soon as the packed tile is there (and give its slot back), store when the MMAs of
-                    // the stage's previous use are done: only the stores are between that and the next MMAs
-                    const int gi = nth * n_groups + it / kPkStages, q = it % kPkStages, slot = gi % kPkSlots;
-                    ok = mbar_wait(&pk_full[slot], (gi / kPkSlots) & 1, abort_flag) && ok;
+                // expand into registers as soon as the packed tile is there (and give its slot back), store when the MMAs of
+                // the stage's previous use are done: only the stores are between that and the next MMAs.  Both barriers are asked ahead.
+                const int gi = nth * n_groups + it / kPkStages, q = it % kPkStages, slot = gi % kPkSlots;
+                if (!yes(pk_there)) ok = mbar_wait(&pk_full[slot], (gi / kPkSlots) & 1, abort_flag) && ok;
+                const uint32_t free = g >= kStages ? ask(&empty[st], ((g / kStages) & 1) ^ 1) : 1u;
+#pragma unroll
+                for (int hh = 0; hh < kSK / 128; ++hh) {
                     uint4 a[8];
                     uint32_t e[4];
-                    expand_row<128>(packed + slot * kPkSlotBytes, row, q, x, row_in, p.d_in - it * kSK, a, e);
+                    expand_row<128>(packed + slot * kPkSlotBytes, row, kPkStages == 1 ? hh : q, x, row_in, p.d_in - it * kSK - hh * 128, a, e);
 #pragma unroll
                     for (int i = 0; i < 8; ++i) asm volatile("" : "+r"(a[i].x), "+r"(a[i].y), "+r"(a[i].z), "+r"(a[i].w));     // here, not after the wait
-                    __syncwarp();
-                    if (lane == 0) {
-                        mbar_arrive(&pk_empty[slot]);
-                        if (q == 0 && it + 1 == p.n1) mbar_arrive(&pk_empty[slot]);      // a packed tile's last stage alone: in place of the other group too
+                    if (hh + 1 == kSK / 128) {
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(&pk_empty[slot]);
+                        // the packed tile of this group's next stage in this tile
+                        const int gn = gi + kGroups / kPkStages;
+                        pk_there = it + kGroups < n_groups * kPkStages ? ask(&pk_full[gn % kPkSlots], (gn / kPkSlots) & 1) : 0u;
                     }
-                    if (g >= kStages) ok = mbar_wait(&empty[st], ((g / kStages) & 1) ^ 1, abort_flag) && ok;
+                    if (hh == 0 && !yes(free)) ok = mbar_wait(&empty[st], ((g / kStages) & 1) ^ 1, abort_flag) && ok;
                     asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};"
-                                 :: "r"(tmem_base + lane_base + kECol + 4 * st), "r"(e[0]), "r"(e[1]), "r"(e[2]), "r"(e[3]) : "memory");
-                    tmem_st32(tmem_base + lane_base + Cfg::kACol + 32 * st, a);
-                    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-                    fence_before_sync();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive_remote(peer_addr(&conv_done[st], 0));
-                } else {
-                    pass(g);
+                                 :: "r"(tmem_base + lane_base + kECol + Cfg::kECols * st + 4 * hh), "r"(e[0]), "r"(e[1]), "r"(e[2]), "r"(e[3]) : "memory");
+                    tmem_st32(tmem_base + lane_base + Cfg::kACol + Cfg::kACols * st + 32 * hh, a);
                 }
+                asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+                fence_before_sync();
+                arrive(st, (uint32_t)(2 * half_tok * kSK * 2));
             }
         }
     } else {
         // ============================ epilogue: thread = output row, half of the tokens ============================
-        const int half = (warp - kConvWarps) >> 2;
+        const int half = (warp - Cfg::kWarpEpi) >> 2;
         const int row = (warp & 3) * 32 + lane;
-        const uint32_t taddr = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + half * kHalfTok;
-        const uint32_t buf = s32(b_full) + 384 + (warp - kConvWarps) * 1024;
+        const uint32_t taddr = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + half * half_tok;
+        const uint32_t buf = s32(full) + 384 + (warp - Cfg::kWarpEpi) * 1024;
         int nth = 0;
-        // ---- T': thread = token.  Part of pair q: [c / 4][128 tokens] float4; a pair has at most one that starts with its tile and
+        // ---- T': thread = token (t_ranks: rank).  Part of pair q: [c / 4][128 tokens] float4; a pair has at most one that starts with its tile and
         // one that does not.
         auto part = [&](int q, bool starts) { return p.t_part + ((size_t)(2 * q + (starts ? 1 : 0)) * 2 + rank) * ((size_t)kPM * p.t_n / 4) + row; };
         auto store4 = [&](int tile, int c, float4 v) {
-            const int token = (tile / p.t_chunks) * kTTok + (int)rank * kPM + row, col = (tile % p.t_chunks) * p.t_n + c;
+            const int a_row = t_part_of(tile, true) * kTTok + (int)rank * kPM + row, b_row = t_part_of(tile, false) * p.t_n + c;
+            if (p.t_ranks) {
+                if (a_row >= p.r) return;
+                __nv_bfloat16* at = p.t_out + (size_t)b_row * p.r + a_row;
+                const float t[4] = {p.t_scale * v.x, p.t_scale * v.y, p.t_scale * v.z, p.t_scale * v.w};
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    if (b_row + i < p.b) {
+                        at[(size_t)i * p.r] = __float2bfloat16_rn(p.t_parts == 2 ? bf16_head(t[i]) : t[i]);
+                        if (p.t_parts == 2) at[(size_t)i * p.r + (size_t)p.b * p.r] = __float2bfloat16_rn(bf16_tail(t[i]));
+                    }
+                return;
+            }
+            const int token = a_row, col = b_row;
             if (token >= p.b || col >= p.r) return;
             store_T(p.t_out + (size_t)token * p.r + col, p.t_parts == 2 ? (size_t)p.b * p.r : 0,
                     make_float4(p.t_scale * v.x, p.t_scale * v.y, p.t_scale * v.z, p.t_scale * v.w));
         };
         auto publish = [&](size_t word) {                                    // the writes of the eight warps, then the word
             epilogue_sync();
-            if (threadIdx.x == kConvWarps * 32) {
+            if (threadIdx.x == Cfg::kWarpEpi * 32) {
                 __threadfence();
                 *(volatile unsigned long long*)(p.t_sync + word) = tagged(call, 0);
             }
@@ -1021,15 +1113,33 @@ prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap t
                     for (int i = 0; i < 4; ++i)
                         if (c4 + 4 * i < p.t_n / 4) store4(run.tile, 4 * (c4 + 4 * i), make_float4(x[i].x + y[i].x, x[i].y + y[i].y, x[i].z + y[i].z, x[i].w + y[i].w));
                 }
+            } else if (n <= 4) {                                             // four parts of two columns
+                for (int c4 = 2 * (tq - q0) + half; c4 < p.t_n / 4; c4 += 4 * n) {
+                    const int c5 = c4 + 2 * n;
+                    float4 x[4], y[4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const float4* from = part(min(q0 + i, q1), i == 0);
+                        x[i] = __ldcg(from + (size_t)c4 * kPM); y[i] = __ldcg(from + (size_t)min(c5, p.t_n / 4 - 1) * kPM);
+                    }
+#pragma unroll
+                    for (int i = 1; i < 4; ++i)
+                        if (i < n) {
+                            x[0].x += x[i].x; x[0].y += x[i].y; x[0].z += x[i].z; x[0].w += x[i].w;
+                            y[0].x += y[i].x; y[0].y += y[i].y; y[0].z += y[i].z; y[0].w += y[i].w;
+                        }
+                    store4(run.tile, 4 * c4, x[0]);
+                    if (c5 < p.t_n / 4) store4(run.tile, 4 * c5, y[0]);
+                }
             } else {
                 for (int c4 = 2 * (tq - q0) + half; c4 < p.t_n / 4; c4 += 2 * n) {
                     float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-                    for (int qb = q0; qb <= q1; qb += 12) {
-                        float4 v[12];
+                    for (int qb = q0; qb <= q1; qb += 8) {
+                        float4 v[8];
 #pragma unroll
-                        for (int i = 0; i < 12; ++i) v[i] = qb + i <= q1 ? __ldcg(part(qb + i, qb + i == q0) + (size_t)c4 * kPM) : make_float4(0.f, 0.f, 0.f, 0.f);
+                        for (int i = 0; i < 8; ++i) v[i] = qb + i <= q1 ? __ldcg(part(qb + i, qb + i == q0) + (size_t)c4 * kPM) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-                        for (int i = 0; i < 12; ++i) { s.x += v[i].x; s.y += v[i].y; s.z += v[i].z; s.w += v[i].w; }
+                        for (int i = 0; i < 8; ++i) { s.x += v[i].x; s.y += v[i].y; s.z += v[i].z; s.w += v[i].w; }
                     }
                     store4(run.tile, 4 * c4, s);
                 }
@@ -1043,31 +1153,35 @@ prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap t
             // 16 tokens at a time, through the warp's kilobyte of shared memory, [token][32 rows] bf16: a thread then stores 16 bytes,
             // eight rows of a token (direct two-byte stores took 5.6 us a tile).  Two passes of 64 tokens (what fits in
             // registers): the accumulator is free before the second pass's stores.
-            const int tok0 = ti.n0 + half * kHalfTok, row8 = ti.m0 + (warp & 3) * 32 + (lane & 3) * 8;
-            const int n_tok = row8 < p.m_total ? p.b - tok0 : 0;
+            const int tok0 = ti.n0 + half * half_tok, row8 = ti.m0 + (warp & 3) * 32 + (lane & 3) * 8;
+            const int toks = min(half_tok, p.b - tok0), n_tok = row8 < p.m_total ? toks : 0;
             __nv_bfloat16* out = p.out + (size_t)(tok0 + (lane >> 2)) * p.ldo + row8;
-            constexpr int kPass = kHalfTok < 64 ? kHalfTok : 64;
+            constexpr int kPass = N < 128 ? N / 2 : 64;
+            bool held = true;                                                // the accumulator, by this warp
 #pragma unroll
-            for (int c0 = 0; c0 < kHalfTok; c0 += kPass) {
+            for (int c0 = 0; c0 < N / 2; c0 += kPass) {
                 uint32_t y[kPass / 2];                                       // bf16 pairs of neighbouring tokens
+                if (c0 < half_tok) {
 #pragma unroll
-                for (int c1 = 0; c1 < kPass; c1 += 32) {
-                    uint32_t r[32];
-                    tmem_ld32(taddr + c0 + c1, r);
+                    for (int c1 = 0; c1 < kPass; c1 += 32) {
+                        uint32_t r[32];
+                        tmem_ld32(taddr + c0 + c1, r);
 #pragma unroll
-                    for (int c = 0; c < 32; c += 2) {
-                        __nv_bfloat162 v = __floats2bfloat162_rn(p.scale * __uint_as_float(r[c]), p.scale * __uint_as_float(r[c + 1]));
-                        y[(c1 + c) / 2] = *reinterpret_cast<uint32_t*>(&v);
+                        for (int c = 0; c < 32; c += 2) {
+                            __nv_bfloat162 v = __floats2bfloat162_rn(p.scale * __uint_as_float(r[c]), p.scale * __uint_as_float(r[c + 1]));
+                            y[(c1 + c) / 2] = *reinterpret_cast<uint32_t*>(&v);
+                        }
                     }
                 }
-                if (c0 + kPass == kHalfTok) {
+                if (held && c0 + kPass >= half_tok) {
+                    held = false;
                     fence_before_sync();
                     __syncwarp();
                     if (lane == 0) mbar_arrive_remote_release(peer_addr(acc_empty, 0));
                 }
 #pragma unroll
                 for (int c1 = 0; c1 < kPass; c1 += 16) {
-                    if (c0 + c1 >= p.b - tok0) break;
+                    if (c0 + c1 >= toks) break;
 #pragma unroll
                     for (int c = 0; c < 16; ++c)
                         asm volatile("st.shared.u16 [%0], %1;" :: "r"(buf + c * 64 + lane * 2), "h"((unsigned short)(c & 1 ? y[(c1 + c) / 2] >> 16 : y[(c1 + c) / 2] & 0xFFFFu)) : "memory");
@@ -1155,13 +1269,13 @@ static bool pf_map(CUtensorMap* map, const void* base, CUtensorMapDataType type,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// bf16 rows as 64-column sub-tiles: one box of box_rows rows x 2 sub-tiles of 128 bytes, in that order.
-static bool pf_map3(CUtensorMap* map, const void* base, uint64_t cols, uint64_t rows, int box_rows) {
+// bf16 rows as 64-column sub-tiles: one box of box_rows rows x sub_tiles of 128 bytes, in that order.
+static bool pf_map3(CUtensorMap* map, const void* base, uint64_t cols, uint64_t rows, int box_rows, int sub_tiles) {
     PfEncodeTiledFn fn = reinterpret_cast<PfEncodeTiledFn>(tensor_map_encoder());
     if (!fn) return false;
     cuuint64_t dims[3] = {64, rows, cols / 64};
     cuuint64_t strides[2] = {cols * 2, 128};
-    cuuint32_t box[3] = {64, (cuuint32_t)box_rows, 2};
+    cuuint32_t box[3] = {64, (cuuint32_t)box_rows, (cuuint32_t)sub_tiles};
     cuuint32_t estr[3] = {1, 1, 1};
     return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
               CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
@@ -1172,10 +1286,17 @@ bool prefill_supports(int b, int d_out, int d_in, int r) {
     return b >= 1 && d_out % 16 == 0 && d_in % kPBK == 0 && r % 16 == 0 && r >= 0;
 }
 
-// The pair kernel's T' tiles: chunks of the columns of r.
-static int t_chunks(int r) { return ceil_div(r, 256); }
-static int t_width(int r) { return r > 0 ? ceil_div(ceil_div(r, t_chunks(r)), 16) * 16 : 16; }
-static size_t pair_part_bytes(int r, int sm_count) { return (size_t)(sm_count / 2) * 2 * 256 * t_width(r) * sizeof(float); }
+// Columns of a T' tile of the pair kernel that cuts r into `chunks`.
+static int t_width(int r, int chunks) { return r > 0 ? ceil_div(ceil_div(r, chunks), 16) * 16 : 16; }
+static size_t pair_part_bytes(int r, int sm_count) { return (size_t)(sm_count / 2) * 2 * 256 * t_width(r, ceil_div(r, 256)) * sizeof(float); }
+// Chunks of r: of up to `most` columns, and as many as leave a tile up to eight of the pairs that have no other work.  (A tile's parts are added up by
+// these pairs, each part of a column asked for by each of them: 4096 -> 11008, rank 416, 256 tokens, two tiles of 15 parts of four stages,
+// the sums took 4 us, of 7 parts 2.)
+static int t_chunks(int r, int most, int token_tiles, int spare) {
+    int chunks = ceil_div(r, most);
+    while (spare / (token_tiles * chunks) > 8 && t_width(r, chunks + 1) >= 48) ++chunks;
+    return chunks;
+}
 
 // Pairs that share the work of T'.  Each tile in equal parts, one a pair, where that uses four fifths of the pairs or more
 // (a pair then has one part to write, and the pairs that read the same X walk it together); else an even share each.
@@ -1191,12 +1312,48 @@ static int t_share(int tiles, int stages, int pairs, int spare, int main_stages)
     return (long long)tiles * most < pairs ? tiles * most : pairs;
 }
 
-// Token tile of the pair kernel: the narrowest with which every tile has a pair of its own, else 256 (a tile takes about the
-// same time whatever its width).
-static int pair_tile(int b, int d_out, int sm_count) {
-    for (int n = 64; n < 256; n *= 2)
-        if ((long long)ceil_div(d_out, 2 * kPM) * ceil_div(b, n) <= sm_count / 2) return n;
-    return 256;
+// How the pair kernel cuts a problem: tokens of a tile (a multiple of 16), tiles, and the tiles of T'.
+struct PairPlan { int tile_n, tiles, t_n, t_chunks, t_tiles; bool t_ranks; };
+static PairPlan plan_tiles(int b, int d_out, int r, int widest, int pairs) {
+    PairPlan pl;
+    pl.tile_n = ceil_div(ceil_div(b, ceil_div(b, widest)), 16) * 16;
+    pl.tiles = ceil_div(d_out, 2 * kPM) * ceil_div(b, pl.tile_n);
+    // T' tiles of narrow token tiles have up to 128 columns of tensor memory: chunks of the ranks, or, where that makes fewer tiles, the
+    // tile's tokens
+    const int most = pl.tile_n <= 128 ? PairCfg<128>::kTWidth : PairCfg<256>::kTWidth;
+    pl.t_ranks = most == 128 && r > most && ceil_div(b, pl.tile_n) * ceil_div(r, 2 * kPM) < ceil_div(b, kTTok) * ceil_div(r, most);
+    const int t_tokens = ceil_div(b, pl.t_ranks ? pl.tile_n : kTTok);
+    pl.t_chunks = pl.t_ranks ? ceil_div(r, 2 * kPM) : r > 0 ? t_chunks(r, most, t_tokens, pairs - pl.tiles) : 1;
+    pl.t_n = pl.t_ranks ? pl.tile_n : t_width(r, pl.t_chunks);
+    pl.t_tiles = r > 0 ? t_tokens * pl.t_chunks : 0;
+    return pl;
+}
+// Tiles of up to 256 tokens, or of 128 or 64 where every tile then has a pair of its own: what takes the least time, in units of 10 ns.  A
+// stage of 128 columns takes 0.40 us with 256 tokens, 0.27 with 128, 0.24 with 64; T' 7 us and 0.28 for each of its stages, on
+// the pairs without a tile beside the others (of the shorter of the two a quarter counts: they share the L2), else before them.
+// (4096 -> 4096, rank 416, 256 tokens in tiles of 256, 128, 64: 28.7, 24.8, 27.1 us; 5696 -> 1392, rank 288, 1024 tokens 34.9, 36.9, -;
+// 8192 -> 1024, rank 112, 512 tokens 34.8, 26.9, 26.7.)
+static PairPlan pair_plan(int b, int d_out, int d_in, int r, int pairs) {
+    PairPlan best = {};
+    long long best_cost = -1;
+    for (int widest = 256; widest >= 64; widest /= 2) {
+        const PairPlan pl = plan_tiles(b, d_out, r, widest, pairs);
+        if (best_cost >= 0 && pl.tiles > pairs) break;
+        const int stage = pl.tile_n > 128 ? 40 : pl.tile_n > 64 ? 27 : 24, t_stages = d_in / PairCfg<256>::kDK;
+        const long long main = (long long)ceil_div(pl.tiles, pairs) * ceil_div(d_in, 128) * stage;
+        long long cost = main;
+        if (r > 0) {
+            const int spare = pairs - pl.tiles, parts = spare < pl.t_tiles ? 0 : spare / pl.t_tiles < t_stages / 4 ? spare / pl.t_tiles : t_stages < 4 ? 1 : t_stages / 4;
+            if (parts > 0) {
+                const long long t = 700 + (long long)ceil_div(t_stages, parts) * 28;
+                cost = main > t ? main + t / 4 : t + main / 4;
+            } else {
+                cost = main + 700 + (long long)pl.t_tiles * t_stages * 28 / pairs;
+            }
+        }
+        if (best_cost < 0 || cost < best_cost) { best = pl; best_cost = cost; }
+    }
+    return best;
 }
 
 // The pair kernel, asked for by the kernel family's name: when its 128 x 256 tiles would give a quarter of the SMs or more a tile.
@@ -1252,7 +1409,7 @@ static slim_status_t launch_tile_kernel(const PrefillParams& q, int m_rows, cons
 
 template <int N>
 static slim_status_t launch_pair(const PrefillParams& p, const CUtensorMap& tmV, const CUtensorMap& tmM, const CUtensorMap& tmX, const CUtensorMap& tmA2,
-                                 const CUtensorMap& tmB2, const CUtensorMap& tmR, const CUtensorMap& tmXt, int pairs, cudaStream_t st) {
+                                 const CUtensorMap& tmB2, const CUtensorMap& tmTA, const CUtensorMap& tmTB, int pairs, cudaStream_t st) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(2 * pairs); cfg.blockDim = dim3(kPairThreads); cfg.dynamicSmemBytes = PairCfg<N>::kSmem; cfg.stream = st;
     cudaLaunchAttribute attr[2];
@@ -1269,7 +1426,7 @@ static slim_status_t launch_pair(const PrefillParams& p, const CUtensorMap& tmV,
         attr[1].val.programmaticStreamSerializationAllowed = 1;
     }
     cfg.attrs = attr; cfg.numAttrs = 2;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, prefill_pair_kernel<N>, p, tmV, tmM, tmX, tmA2, tmB2, tmR, tmXt);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, prefill_pair_kernel<N>, p, tmV, tmM, tmX, tmA2, tmB2, tmTA, tmTB);
     count_launch(1);
     return e == cudaSuccess ? SLIM_OK : SLIM_ERR_CUDA;
 }
@@ -1285,7 +1442,7 @@ slim_status_t launch_prefill(const __nv_bfloat16* X, int b, const uint8_t* vals,
     if (!prefill_supports(b, d_out, d_in, r)) return SLIM_ERR_UNSUPPORTED_SHAPE;
     // The words of T' tiles have a region of fixed size (8.1 million tokens of up to 256 ranks): more go in equal parts, one behind
     // the other on the stream and the workspace.
-    const long long most = r > 0 ? (long long)(kSyncTiles / t_chunks(r)) * kTTok : b;
+    const long long most = r > 0 ? (long long)(kSyncTiles / ceil_div(r, 256)) * kTTok : b;
     if (b > most) {
         const int n = ceil_div(ceil_div(b, (int)((b + most - 1) / most)), kTTok) * kTTok;
         slim_status_t rc = SLIM_OK;
@@ -1320,20 +1477,23 @@ slim_status_t launch_prefill(const __nv_bfloat16* X, int b, const uint8_t* vals,
     const int t_parts = keeps_T32(b, d_out, d_in, r) ? 2 : 1;
     const bool wide = force_pair || runs_wide(b, d_out, d_in, r, di->sm_count, automatic);
     if (force_pair && ceil_div(d_out, kPM) % 2 != 0) return SLIM_ERR_UNSUPPORTED_SHAPE;
-    const int tile_n = wide ? pair_tile(b, d_out, di->sm_count) : 64;
+    const int n_pairs = g_pairs[dev].load(std::memory_order_relaxed);
+    const PairPlan plan = wide ? pair_plan(b, d_out, d_in, r, n_pairs) : PairPlan{};
+    const int tile_n = wide ? plan.tile_n : 64;
     const int xbox = wide ? tile_n / 2 : 64;              // token rows one CTA loads per stage = one TMA box
+    const bool narrow = tile_n <= 128;
     const int dk = wide ? PairCfg<256>::kDK : PfCfg<64>::kDK;      // columns of a dense stage of the main kernel
-    CUtensorMap tmV, tmM, tmX, tmXpre, tmA2, tmB2, tmR, tmXt;
+    CUtensorMap tmV, tmM, tmX, tmXpre, tmA2, tmB2, tmTA, tmTB;
     bool ok = pf_map(&tmV, vals, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)d_in / 4, (uint64_t)d_out, kPkCols / 4, kPM, 64) &&
               (d_in % 128 != 0 || pf_map(&tmM, meta, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)d_in / 8, (uint64_t)d_out, kPkCols / 8, kPM, 32)) &&
-              (wide ? pf_map3(&tmX, X, (uint64_t)d_in, (uint64_t)b, xbox)
+              (wide ? pf_map3(&tmX, X, (uint64_t)d_in, (uint64_t)b, xbox, (narrow ? PairCfg<128>::kSK : PairCfg<256>::kSK) / 64)
                     : pf_map(&tmX, X, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (uint64_t)d_in, (uint64_t)b, 64, xbox, 128));
     if (!ok) return SLIM_ERR_CUDA;
     if (d_in % 128 != 0) tmM = tmV;              // not used
-    tmA2 = tmX; tmB2 = tmX; tmR = tmX; tmXt = tmX;    // not used when r == 0
+    tmA2 = tmX; tmB2 = tmX; tmTA = tmX; tmTB = tmX;    // not used when r == 0
     if (r > 0 && wide) {
-        ok = pf_map(&tmR, R, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (uint64_t)d_in, (uint64_t)r, 64, t_width(r) / 2, 128) &&
-             pf_map(&tmXt, X, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (uint64_t)d_in, (uint64_t)b, 64, kPM, 128);
+        ok = pf_map(&tmTA, plan.t_ranks ? R : X, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (uint64_t)d_in, (uint64_t)(plan.t_ranks ? r : b), 64, kPM, 128) &&
+             pf_map(&tmTB, plan.t_ranks ? X : R, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (uint64_t)d_in, (uint64_t)(plan.t_ranks ? b : r), 64, plan.t_n / 2, 128);
         if (!ok) return SLIM_ERR_CUDA;
     } else if (r > 0) {
         // T' = (X R^T) / s : dense phase only, output rows = adapter index
@@ -1372,34 +1532,34 @@ slim_status_t launch_prefill(const __nv_bfloat16* X, int b, const uint8_t* vals,
     }
     PrefillParams p = {};
     p.out = Y; p.ldo = d_out; p.m_total = d_out; p.b = b; p.t_parts = t_parts;
-    p.n1 = s != 0.f ? ceil_div(d_in, wide ? PairCfg<256>::kSK : PfCfg<64>::kSK) : 0;
+    p.n1 = s != 0.f ? ceil_div(d_in, !wide ? PfCfg<64>::kSK : narrow ? PairCfg<128>::kSK : PairCfg<256>::kSK) : 0;
     p.n2 = r > 0 ? ceil_div(r, dk) * t_parts : 0;
     p.scale = s_eff; p.status = status_dev; p.part = nullptr; p.k_per = 0;
     p.meta = d_in % 128 != 0 ? meta : nullptr; p.meta_pitch = d_in / 8; p.d_in = d_in;
     if (p.n1 + p.n2 == 0)             // s == 0 and no adapters: the result is zero
         return cudaMemsetAsync(Y, 0, (size_t)b * d_out * 2, st) == cudaSuccess ? SLIM_OK : SLIM_ERR_CUDA;
-    note_token_tile(wide ? tile_n : 64);
+    note_token_tile(tile_n > 128 ? 256 : tile_n > 64 ? 128 : 64);
     slim_status_t rc;
     const bool dep = r > 0 && p.n1 > 0;               // sparse stages to run while T' is being made
-    p.row_pairs = ceil_div(d_out, 2 * kPM); p.tiles = p.row_pairs * ceil_div(b, tile_n);
+    p.row_pairs = ceil_div(d_out, 2 * kPM); p.tiles = plan.tiles; p.half = tile_n / 2;
     if (!wide) {
         rc = launch_tile_kernel<64, false>(p, d_out, tmV, tmM, tmX, tmA2, tmB2, st, 1, dep);
     } else {
-        const int pairs = g_pairs[dev].load(std::memory_order_relaxed);
+        const int pairs = n_pairs;
         p.departures = reinterpret_cast<unsigned long long*>(ws);
         p.t_sync = reinterpret_cast<unsigned long long*>(reinterpret_cast<char*>(ws) + SLIM_WORKSPACE_SYNC_BYTES);
         p.r = r;
         int grid = p.tiles < pairs ? p.tiles : pairs;
         if (r > 0) {
-            p.t_n = t_width(r); p.t_chunks = t_chunks(r); p.t_tiles = ceil_div(b, kTTok) * p.t_chunks; p.t_stages = d_in / PairCfg<256>::kDK;
+            p.t_ranks = plan.t_ranks; p.t_n = plan.t_n; p.t_chunks = plan.t_chunks; p.t_tiles = plan.t_tiles; p.t_stages = d_in / PairCfg<256>::kDK;
             p.t_scale = 1.f / s_eff; p.t_out = Tq;
             p.t_part = reinterpret_cast<float4*>(reinterpret_cast<char*>(Tq) + t_bytes(b, r, t_parts));
-            p.t_pairs = t_share(p.t_tiles, p.t_stages, pairs, pairs - grid, p.n1);
+            p.t_pairs = t_share(p.t_tiles, p.t_stages, pairs, pairs - grid, s != 0.f ? ceil_div(d_in, 128) : 0);
             grid = grid + p.t_pairs < pairs ? grid + p.t_pairs : pairs;      // the last pairs make T'
         }
-        rc = tile_n == 256 ? launch_pair<256>(p, tmV, tmM, tmX, tmA2, tmB2, tmR, tmXt, grid, st)
-           : tile_n == 128 ? launch_pair<128>(p, tmV, tmM, tmX, tmA2, tmB2, tmR, tmXt, grid, st)
-                           : launch_pair<64>(p, tmV, tmM, tmX, tmA2, tmB2, tmR, tmXt, grid, st);
+        rc = tile_n > 128 ? launch_pair<256>(p, tmV, tmM, tmX, tmA2, tmB2, tmTA, tmTB, grid, st)
+           : tile_n > 64  ? launch_pair<128>(p, tmV, tmM, tmX, tmA2, tmB2, tmTA, tmTB, grid, st)
+                          : launch_pair<64>(p, tmV, tmM, tmX, tmA2, tmB2, tmTA, tmTB, grid, st);
     }
     if (rc != SLIM_OK) return rc;
     return SLIM_OK;
