@@ -1107,16 +1107,23 @@ int cluster_size(const int* res, int tiles, int units) {
 // against 12.5), else not (4096 x 4096, rank 208: 9.1 us against 8.3).  With 256-row tiles only: 8192 -> 1024, rank 112, 16
 // tokens 9.3 us instead of 6.6; 5120 x 5120, rank 512, 8 tokens 11.1 instead of 8.6; larger layers are better off with them
 // (28672 -> 8192, 16 tokens 48 us against 65).
+//   Without adapters clusters of two CTAs do where their parts of a row stay short (they start and exchange less), and with them tiles of 128
+// rows fit more layers (16 tokens: 5120 -> 13824 14.8 us with 256 rows, 12.9; 4096 -> 11008 12.2, 11.0; clusters of four against two:
+// 2048 -> 6400 5.8, 5.2, 4096 x 4096 in tiles of 64 rows 6.0, 5.5, 8192 -> 3584 7.7, 8.1).
 void narrow_tiles(int dev, int nt, int fmt, bool qa, int tp, int sm_count, int d_out, int units, int groups, int* mt, int* C) {
-    auto fits = [&](int m) {
+    auto fits = [&](int m, int c) {
         const int* res = residency(dev, nt, fmt, qa, m, tp);
-        return res && ceil_div(d_out, 64 * m) + groups <= res[2];
+        return res && ceil_div(d_out, 64 * m) + groups <= res[c];
     };
-    if (!fits(2)) return;
+    if (!fits(2, 2)) {
+        if (groups == 0 && units >= 2 && fits(2, 1)) { *mt = 2; *C = 2; }
+        return;
+    }
     const bool spread = 8 * (ceil_div(d_out, 128) + groups) <= sm_count;
-    *mt = fits(1) && (groups == 0 || (!spread && units >= 32)) ? 1 : 2;
+    *mt = fits(1, 2) && (groups == 0 || (!spread && units >= 32)) ? 1 : 2;
     const int widest = 8 * (ceil_div(d_out, 64 * *mt) + groups) <= sm_count ? 8 : 4;
     for (*C = widest; *C > units; *C /= 2) {}
+    if (groups == 0 && *C == 4 && (*mt == 1 ? units <= 24 : units <= 20 && d_out >= 6144)) *C = 2;
 }
 
 }  // namespace
