@@ -27,20 +27,37 @@ struct QsHeader {                     // first 256 bytes of the workspace
 
 constexpr int kVec = 4;               // float4 loads a thread has in flight
 
-// The array as float4s i = first, first + stride, ..: kVec loads at a time, then `f` on each.  `tail` elements (n % 4)
+// The array as float4s i = first, first + stride, ..: kVec loads at a time (AHEAD: asked for while `f` works on those before), then `f` on each.  `tail` elements (n % 4)
 // go to the first threads.
-template <bool BACKWARDS, typename F>
+template <bool BACKWARDS, bool AHEAD, typename F>
 __device__ __forceinline__ void for_weights(const float* __restrict__ W, size_t n, F f)
 {
     const size_t n4 = n / 4, stride = (size_t)gridDim.x * blockDim.x, me = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     const float4* W4 = reinterpret_cast<const float4*>(W);
     size_t i = me;
-    for (; i + (kVec - 1) * stride < n4; i += kVec * stride) {
-        float4 v[kVec];
+    float4 v[kVec];
+    auto load = [&](float4 (&to)[kVec]) {
 #pragma unroll
-        for (int k = 0; k < kVec; ++k) v[k] = __ldg(W4 + (BACKWARDS ? n4 - 1 - (i + k * stride) : i + k * stride));
+        for (int k = 0; k < kVec; ++k) to[k] = __ldg(W4 + (BACKWARDS ? n4 - 1 - (i + k * stride) : i + k * stride));
+    };
+    auto use = [&] {
 #pragma unroll
         for (int k = 0; k < kVec; ++k) { f(v[k].x); f(v[k].y); f(v[k].z); f(v[k].w); }
+    };
+    if constexpr (AHEAD) {
+        float4 w[kVec];
+        bool some = i + (kVec - 1) * stride < n4;
+        if (some) load(v);
+        while (some) {
+            i += kVec * stride;
+            some = i + (kVec - 1) * stride < n4;
+            if (some) load(w);
+            use();
+#pragma unroll
+            for (int k = 0; k < kVec; ++k) v[k] = w[k];
+        }
+    } else {
+        for (; i + (kVec - 1) * stride < n4; i += kVec * stride) { load(v); use(); }
     }
     for (; i < n4; i += stride) {
         const float4 v = __ldg(W4 + (BACKWARDS ? n4 - 1 - i : i));
@@ -55,7 +72,7 @@ qs_absmax_kernel(const float* __restrict__ W, size_t n, QsHeader* hdr)
     __shared__ unsigned int sm[16], sb[16];
     after_previous_grid();
     unsigned int m = 0, bad = 0;
-    for_weights<false>(W, n, [&](float w) {
+    for_weights<false, false>(W, n, [&](float w) {
         const float a = fabsf(w);
         if (!(a <= 3.0e38f)) bad = 1;
         m = max(m, __float_as_uint(a));
@@ -86,7 +103,7 @@ qs_hist_kernel(const float* __restrict__ W, size_t n, const QsHeader* hdr, int b
     if (M > 0.f && !hdr->bad) {
         const float fb = (float)bins;
         const Divisor by(M);
-        for_weights<true>(W, n, [&](float w) { atomicAdd(&sh[min((int)__fmul_rn(by.of(fabsf(w)), fb), bins - 1)], 1u); });
+        for_weights<true, true>(W, n, [&](float w) { atomicAdd(&sh[min((int)__fmul_rn(by.of(fabsf(w)), fb), bins - 1)], 1u); });
     }
     __syncthreads();
     for (int i = threadIdx.x; i < bins; i += blockDim.x)
@@ -106,11 +123,11 @@ qs_hist_kernel(const float* __restrict__ W, size_t n, const QsHeader* hdr, int b
 //     so on; where a guess proves wrong, the block is gone through by parts (add_block).
 //   - The fine candidates depend on the best coarse one only through ten possible values: all 10 + 10 x 19
 //     candidates are evaluated at once, a block each, and the last block to finish takes the minima.
-// Bound by the walk of one warp over the blocks' sums, the first of them a term at a time, while the other fifteen wait: the FP64
-// operations of all terms (200 candidates x 20000 bins x about 30, at 64 a cycle and SM) are 6-7 us of it.
+// Bound by the walk of one warp over the blocks' sums, the first of them a term at a time (41 cycles each). A warp of its own walks
+// over a round of blocks while the other sixteen work out the next: their guesses start from ordinary sums, not from the walk's result.
 // 20000 bins: 400 us with a warp per candidate and the bins in sequence, 54 with one adding warp per candidate that every
-// block of bins passed through, now 38.
-constexpr int kSearchWarps = 16, kSearchThreads = 32 * kSearchWarps, kCoarse = 10, kFine = 19, kCandidates = kCoarse + kCoarse * kFine;
+// block of bins passed through, 39 with one of the sixteen warps walking between the rounds, now 36.
+constexpr int kSearchWarps = 16, kTermThreads = 32 * kSearchWarps, kSearchThreads = kTermThreads + 32, kCoarse = 10, kFine = 19, kCandidates = kCoarse + kCoarse * kFine;
 
 // x / b correctly rounded in binary64, for many x and one b: as Divisor does it in binary32.
 struct Divisor64 {
@@ -173,12 +190,16 @@ struct Binade {
 constexpr int kPitch = 36, kBlockTerms = 8 * kPitch;
 __host__ __device__ __forceinline__ constexpr int term_at(int i) { return (i & 7) * kPitch + (i >> 3); }
 
+constexpr size_t kSearchSmem = 2 * kSearchWarps * kBlockTerms * sizeof(double);
 constexpr int kCross = 3;                                     // crossings of a block that are walked one by one
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
     for (int o = 16; o; o >>= 1) v = __dadd_rn(v, __shfl_xor_sync(0xffffffffu, v, o));
     return v;
 }
+
+__device__ __forceinline__ void named_sync(int id, int threads) { asm volatile("bar.sync %0, %1;" :: "r"(id), "r"(threads) : "memory"); }
+__device__ __forceinline__ void named_arrive(int id, int threads) { asm volatile("bar.arrive %0, %1;" :: "r"(id), "r"(threads) : "memory"); }
 
 // e + the first 256 terms, one by one (every lane does it).  They grow from nothing: e leaves a binade every few of them.
 __device__ double add_first(double e, const double* terms)
@@ -225,10 +246,10 @@ __global__ void __launch_bounds__(kSearchThreads, 2)
 qs_search_kernel(QsHeader* hdr, const unsigned int* hist, int bins, double n_total, float* scale_alpha, double* table,
                  double* errors, uint32_t* status)
 {
-    __shared__ double terms[kSearchWarps][kBlockTerms];
-    __shared__ double plain_sum[kSearchWarps], seg_sum[kSearchWarps][kCross + 1], e_now;
-    __shared__ int seg_k[kSearchWarps][kCross + 1];           // a segment's binade, -1: it is empty
-    __shared__ uint32_t crossings[kSearchWarps];              // lanes
+    extern __shared__ double all_terms[];                     // of two rounds: [2][kSearchWarps][kBlockTerms]
+    __shared__ double plain_sum[2][kSearchWarps], seg_sum[2][kSearchWarps][kCross + 1];
+    __shared__ int seg_k[2][kSearchWarps][kCross + 1];        // a segment's binade, -1: it is empty
+    __shared__ uint32_t crossings[2][kSearchWarps];           // lanes
     __shared__ bool last;
     after_previous_grid();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -252,11 +273,14 @@ qs_search_kernel(QsHeader* hdr, const unsigned int* hist, int bins, double n_tot
     const double alpha = cand < kCoarse ? coarse(cand) : fine((cand - kCoarse) / kFine, (cand - kCoarse) % kFine);
     const double width = __ddiv_rn(M, (double)bins);
     double e = alpha > 0.0 ? 0.0 : -1.0;
-    if (alpha > 0.0) {
+    const int blocks = ceil_div(bins, 256), rounds = alpha > 0.0 ? ceil_div(blocks, kSearchWarps) : 0;
+    auto round_terms = [&](int buf, int w) { return all_terms + (buf * kSearchWarps + w) * kBlockTerms; };
+    if (warp < kSearchWarps) {
         const Divisor64 by_n(n_total), by_alpha(alpha);
-        const int blocks = ceil_div(bins, 256);
-        if (threadIdx.x == 0) e_now = 0.0;
-        for (int first = 0; first < blocks; first += kSearchWarps) {
+        double sum_before = 0.0;                              // of the rounds before, an ordinary sum: for the guesses
+        for (int r = 0; r < rounds; ++r) {
+            const int buf = r & 1, first = r * kSearchWarps;
+            double* terms = round_terms(buf, warp);
             const int i0 = (first + warp) * 256 + lane * 8;
             unsigned int c[8];
             if (i0 + 8 <= bins) {
@@ -266,11 +290,12 @@ qs_search_kernel(QsHeader* hdr, const unsigned int* hist, int bins, double n_tot
 #pragma unroll
                 for (int j = 0; j < 8; ++j) c[j] = i0 + j < bins ? hist[i0 + j] : 0u;
             }
+            if (r >= 2) named_sync(4 + buf, kSearchThreads);  // the walk is done with this half of the buffers
             double v[8], sum = 0.0;
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
                 v[j] = qs_term(c[j], i0 + j, width, by_n, by_alpha);
-                terms[warp][j * kPitch + lane] = v[j];
+                terms[j * kPitch + lane] = v[j];
                 sum = __dadd_rn(sum, v[j]);
             }
 #pragma unroll
@@ -278,10 +303,12 @@ qs_search_kernel(QsHeader* hdr, const unsigned int* hist, int bins, double n_tot
                 const double w = __shfl_up_sync(0xffffffffu, sum, o);
                 if (lane >= o) sum = __dadd_rn(sum, w);
             }
-            if (lane == 31) plain_sum[warp] = sum;
-            __syncthreads();
+            if (lane == 31) plain_sum[buf][warp] = sum;
+            named_sync(1, kTermThreads);
             // guesses: e at the first of this lane's bins and after the last (the next lane's first)
-            const double before = __dadd_rn(e_now, warp_sum(lane < warp ? plain_sum[lane] : 0.0)), end = __dadd_rn(before, sum);
+            const double plain = lane < kSearchWarps ? plain_sum[buf][lane] : 0.0;
+            const double before = __dadd_rn(sum_before, warp_sum(lane < warp ? plain : 0.0)), end = __dadd_rn(before, sum);
+            sum_before = __dadd_rn(sum_before, warp_sum(plain));
             double start = __shfl_up_sync(0xffffffffu, end, 1);
             if (lane == 0) start = before;
             const Binade bn(start);
@@ -295,57 +322,57 @@ qs_search_kernel(QsHeader* hdr, const unsigned int* hist, int bins, double n_tot
                 const uint32_t in = __ballot_sync(0xffffffffu, segment == i);
                 const double s = warp_sum(segment == i ? q : 0.0);
                 const int k = __shfl_sync(0xffffffffu, bn.k, in ? __ffs(in) - 1 : 0);
-                if (lane == 0) { seg_sum[warp][i] = s; seg_k[warp][i] = in ? k : -1; }
+                if (lane == 0) { seg_sum[buf][warp][i] = s; seg_k[buf][warp][i] = in ? k : -1; }
             }
-            if (lane == 0) crossings[warp] = cross;
-            __syncthreads();
-            if (warp == 0) {
-                const int n = min(kSearchWarps, blocks - first);
-                e = e_now;
-                int b = 0;
-                if (first == 0) { e = add_first(e, terms[0]); b = 1; }
-                const uint32_t cross_l = lane < n ? crossings[lane] : 1u;
-                const double s_l = lane < n ? seg_sum[lane][0] : 0.0;
-                const int k_l = cross_l == 0 ? seg_k[lane][0] : -1;
-                for (; b < n; ++b) {
-                    // blocks from b on without a crossing, as far as e stays in its binade
-                    double after = lane >= b ? s_l : 0.0;
-#pragma unroll
-                    for (int o = 1; o < kSearchWarps; o <<= 1) {
-                        const double w = __shfl_up_sync(0xffffffffu, after, o);
-                        if (lane >= o) after = __dadd_rn(after, w);
-                    }
-                    after = __dadd_rn(e, after);
-                    const uint32_t stop = __ballot_sync(0xffffffffu, lane >= b && !(k_l == exponent(e) && exponent(after) == k_l));
-                    const int upto = __ffs(stop) - 1;         // lane n at the latest
-                    if (upto > b) { e = __shfl_sync(0xffffffffu, after, upto - 1); b = upto; }
-                    if (b >= n) break;
-                    uint32_t left = crossings[b];
-                    const int nc = __popc(left);
-                    bool good = nc <= kCross;
-                    double f = e;
-                    for (int i = 0; good; ++i) {
-                        const int k = seg_k[b][i];
-                        if (k >= 0) {
-                            const double to = __dadd_rn(f, seg_sum[b][i]);
-                            good = exponent(f) == k && exponent(to) == k;
-                            f = to;
-                        }
-                        if (i == nc) break;
-                        const int l = __ffs(left) - 1;
-                        left &= left - 1;
-#pragma unroll
-                        for (int j = 0; j < 8; ++j) f = __dadd_rn(f, terms[b][j * kPitch + l]);
-                    }
-                    e = good ? f : add_block(e, terms[b], lane);
-                }
-                if (lane == 0) e_now = e;
-            }
-            __syncthreads();
+            if (lane == 0) crossings[buf][warp] = cross;
+            named_arrive(2 + buf, kSearchThreads);
         }
-        e = e_now;
+    } else {
+        for (int r = 0; r < rounds; ++r) {
+            const int buf = r & 1, first = r * kSearchWarps, n = min(kSearchWarps, blocks - first);
+            named_sync(2 + buf, kSearchThreads);
+            int b = 0;
+            if (first == 0) { e = add_first(e, round_terms(0, 0)); b = 1; }
+            const uint32_t cross_l = lane < n ? crossings[buf][lane] : 1u;
+            const double s_l = lane < n ? seg_sum[buf][lane][0] : 0.0;
+            const int k_l = cross_l == 0 ? seg_k[buf][lane][0] : -1;
+            for (; b < n; ++b) {
+                // blocks from b on without a crossing, as far as e stays in its binade
+                double after = lane >= b ? s_l : 0.0;
+#pragma unroll
+                for (int o = 1; o < kSearchWarps; o <<= 1) {
+                    const double w = __shfl_up_sync(0xffffffffu, after, o);
+                    if (lane >= o) after = __dadd_rn(after, w);
+                }
+                after = __dadd_rn(e, after);
+                const uint32_t stop = __ballot_sync(0xffffffffu, lane >= b && !(k_l == exponent(e) && exponent(after) == k_l));
+                const int upto = __ffs(stop) - 1;             // lane n at the latest
+                if (upto > b) { e = __shfl_sync(0xffffffffu, after, upto - 1); b = upto; }
+                if (b >= n) break;
+                const double* terms = round_terms(buf, b);
+                uint32_t left = crossings[buf][b];
+                const int nc = __popc(left);
+                bool good = nc <= kCross;
+                double f = e;
+                for (int i = 0; good; ++i) {
+                    const int k = seg_k[buf][b][i];
+                    if (k >= 0) {
+                        const double to = __dadd_rn(f, seg_sum[buf][b][i]);
+                        good = exponent(f) == k && exponent(to) == k;
+                        f = to;
+                    }
+                    if (i == nc) break;
+                    const int l = __ffs(left) - 1;
+                    left &= left - 1;
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) f = __dadd_rn(f, terms[j * kPitch + l]);
+                }
+                e = good ? f : add_block(e, terms, lane);
+            }
+            if (r + 2 < rounds) named_arrive(4 + buf, kSearchThreads);
+        }
     }
-    if (threadIdx.x == 0) {
+    if (threadIdx.x == kTermThreads) {
         errors[cand] = e;
         __threadfence();
         last = atomicAdd(&hdr->done, 1u) == gridDim.x - 1;
@@ -355,7 +382,7 @@ qs_search_kernel(QsHeader* hdr, const unsigned int* hist, int bins, double n_tot
     if (!last) return;
     // the minima, in the order the algorithm visits the candidates (one thread; the errors are fetched by all, since one
     // after the other they took 15 us)
-    double* er = terms[0];
+    double* er = all_terms;
     for (int i = threadIdx.x; i < kCandidates; i += kSearchThreads) er[i] = __ldcg(errors + i);
     __syncthreads();
     if (threadIdx.x != 0) return;
@@ -376,7 +403,8 @@ qs_search_kernel(QsHeader* hdr, const unsigned int* hist, int bins, double n_tot
     table[2 * kQsTable] = best_a;
 }
 
-// 16 codes a thread: four float4 loads, one 16-byte store.
+// Four float4 loads of a thread under way, a warp's side by side (512 bytes; four neighbouring ones a thread, for a 16-byte store, touch
+// sixteen lines a load), four codes stored together.
 __global__ void __launch_bounds__(256)
 qs_codes_kernel(const float* __restrict__ W, size_t n, const float* scale_alpha, int8_t* codes)
 {
@@ -386,18 +414,17 @@ qs_codes_kernel(const float* __restrict__ W, size_t n, const float* scale_alpha,
     auto code = [&](float w) -> uint32_t {
         return a32 > 0.f ? (uint32_t)max(-8, min(7, __float2int_rn(__fmul_rn(by.of(w), 8.0f)))) & 0xFFu : 0u;
     };
-    const size_t n16 = n / 16;
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n16; i += (size_t)gridDim.x * blockDim.x) {
+    const size_t n4 = n / 4;
+    for (size_t i = (size_t)blockIdx.x * 1024 + threadIdx.x; i < n4; i += (size_t)gridDim.x * 1024) {
         float4 v[4];
-        uint32_t o[4];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) v[k] = __ldg(reinterpret_cast<const float4*>(W) + 4 * i + k);
+        for (int k = 0; k < 4; ++k) if (i + k * 256 < n4) v[k] = __ldg(reinterpret_cast<const float4*>(W) + i + k * 256);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) o[k] = code(v[k].x) | code(v[k].y) << 8 | code(v[k].z) << 16 | code(v[k].w) << 24;
-        reinterpret_cast<uint4*>(codes)[i] = make_uint4(o[0], o[1], o[2], o[3]);
+        for (int k = 0; k < 4; ++k)
+            if (i + k * 256 < n4) reinterpret_cast<uint32_t*>(codes)[i + k * 256] = code(v[k].x) | code(v[k].y) << 8 | code(v[k].z) << 16 | code(v[k].w) << 24;
     }
     const size_t me = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (me < n - 16 * n16) codes[16 * n16 + me] = (int8_t)code(W[16 * n16 + me]);
+    if (me < n - 4 * n4) codes[4 * n4 + me] = (int8_t)code(W[4 * n4 + me]);
 }
 
 }  // namespace
@@ -433,12 +460,13 @@ slim_status_t launch_quant(const float* W, int d_out, int d_in, int8_t* codes, f
     static std::atomic<bool> attr_set[64];
     if (dev < 0 || dev >= 64) return SLIM_ERR_CUDA;
     if (!attr_set[dev].load(std::memory_order_acquire)) {
-        if (cudaFuncSetAttribute(qs_hist_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 20000 * 4) != cudaSuccess) return SLIM_ERR_CUDA;
+        if (cudaFuncSetAttribute(qs_hist_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 20000 * 4) != cudaSuccess ||
+            cudaFuncSetAttribute(qs_search_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSearchSmem) != cudaSuccess) return SLIM_ERR_CUDA;
         attr_set[dev].store(true, std::memory_order_release);
     }
     // a block per SM: two would find no more work in flight and double the additions to the global histogram
     launch_dependent(qs_hist_kernel, dim3((unsigned)di->sm_count), dim3(1024), hist_smem, st, W, n, hdr, bins, hist);
-    launch_dependent(qs_search_kernel, dim3(kCandidates), dim3(kSearchThreads), 0, st, hdr, hist, bins, (double)n, scale_alpha, table,
+    launch_dependent(qs_search_kernel, dim3(kCandidates), dim3(kSearchThreads), kSearchSmem, st, hdr, hist, bins, (double)n, scale_alpha, table,
                      table + 2 * kQsTable + 1, status_dev);
     launch_dependent(qs_codes_kernel, dim3((unsigned)(di->sm_count * 8)), dim3(256), 0, st, W, n, scale_alpha, codes);
     count_launch(4);
