@@ -46,8 +46,7 @@
 // (a warp-wide try_wait or 32 arrivals cost 32 times one); the answer of a try_wait takes about
 // 200 cycles even when the phase is long complete, so waits that follow each other are asked
 // together; a lane left at a warp barrier while another lane of its warp spins costs some hundred
-// nanoseconds per iteration; one MMA costs at least the 128 cycles its 128-row A operand takes to
-// load, whatever N.
+// nanoseconds per iteration; a lane that walks alone takes 120 cycles to issue an MMA.
 // Every wait is bounded; an expired one sets SLIM_ERR_TIMEOUT and the kernel runs on.
 #include <atomic>
 #include <cuda.h>
@@ -86,7 +85,7 @@ template <int N, bool PRE = false> struct PfCfg {
     static constexpr size_t kSmem = 1024 + (size_t)kStages * kStageBytes + kPkSlots * kPkSlotBytes + 1024;
 };
 
-struct PrefillParams {
+struct alignas(128) PrefillParams {      // (so are the tensor maps behind it in the parameters: none lies across two lines)
     __nv_bfloat16* out;     // [tokens][ldo]
     int ldo;
     int m_total;            // valid output rows
@@ -728,6 +727,26 @@ __device__ __forceinline__ void store_T(__nv_bfloat16* at, size_t tail, float4 v
     put(v);
 }
 
+// Four neighbouring values of a row of a T' tile: ranks of a token, or (how & 1) tokens of a rank; in two parts: how & 2.  (As a function that is
+// called a first pass on cold instructions took 2 us less, every other 0.7-1 us more where T' is what a call waits for.)
+__device__ __forceinline__ void put_T(__nv_bfloat16* out, int a_row, int b_row, int b, int r, int how, float4 v)
+{
+    const size_t tail = how & 2 ? (size_t)b * r : 0;
+    if (how & 1) {
+        if (a_row >= r) return;
+        const float t[4] = {v.x, v.y, v.z, v.w};
+        __nv_bfloat16* at = out + (size_t)b_row * r + a_row;
+#pragma unroll
+        for (int i = 0; i < 4; ++i, at += r)
+            if (b_row + i < b) {
+                *at = __float2bfloat16_rn(tail ? bf16_head(t[i]) : t[i]);
+                if (tail) at[tail] = __float2bfloat16_rn(bf16_tail(t[i]));
+            }
+    } else if (a_row < b && b_row < r) {
+        store_T(out + (size_t)a_row * r + b_row, tail, v);
+    }
+}
+
 template <int N>
 __global__ void __launch_bounds__(kPairThreads, 1)
 prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmM,
@@ -1044,22 +1063,8 @@ prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap t
         auto part = [&](int q, bool starts) { return p.t_part + ((size_t)(2 * q + (starts ? 1 : 0)) * 2 + rank) * ((size_t)kPM * p.t_n / 4) + row; };
         auto store4 = [&](int tile, int c, float4 v) {
             const int a_row = t_part_of(tile, true) * kTTok + (int)rank * kPM + row, b_row = t_part_of(tile, false) * p.t_n + c;
-            if (p.t_ranks) {
-                if (a_row >= p.r) return;
-                __nv_bfloat16* at = p.t_out + (size_t)b_row * p.r + a_row;
-                const float t[4] = {p.t_scale * v.x, p.t_scale * v.y, p.t_scale * v.z, p.t_scale * v.w};
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-                    if (b_row + i < p.b) {
-                        at[(size_t)i * p.r] = __float2bfloat16_rn(p.t_parts == 2 ? bf16_head(t[i]) : t[i]);
-                        if (p.t_parts == 2) at[(size_t)i * p.r + (size_t)p.b * p.r] = __float2bfloat16_rn(bf16_tail(t[i]));
-                    }
-                return;
-            }
-            const int token = a_row, col = b_row;
-            if (token >= p.b || col >= p.r) return;
-            store_T(p.t_out + (size_t)token * p.r + col, p.t_parts == 2 ? (size_t)p.b * p.r : 0,
-                    make_float4(p.t_scale * v.x, p.t_scale * v.y, p.t_scale * v.z, p.t_scale * v.w));
+            put_T(p.t_out, a_row, b_row, p.b, p.r, (p.t_ranks ? 1 : 0) | (p.t_parts == 2 ? 2 : 0),
+                  make_float4(p.t_scale * v.x, p.t_scale * v.y, p.t_scale * v.z, p.t_scale * v.w));
         };
         auto publish = [&](size_t word) {                                    // the writes of the eight warps, then the word
             epilogue_sync();

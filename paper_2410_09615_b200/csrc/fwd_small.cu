@@ -60,7 +60,9 @@ constexpr unsigned long long kWaitNs = 500ull * 1000 * 1000;
 
 enum { FMT_PACKED = 0, FMT_PACKED_LD = 1, FMT_TILED = 2 };   // LD: index bytes by cp.async (rows no 16-byte multiples)
 
-struct SmallParams {
+// (A multiple of 128 bytes, as the tensor maps behind it in the parameters are: a map across two lines of 128 takes two fetches.  8192 -> 1024,
+// int4 adapters, 16 tokens 8.4 us a call, with the maps 64 bytes further 8.8.)
+struct alignas(128) SmallParams {
     const __nv_bfloat16* X; const uint8_t* vals; const uint8_t* meta; const uint8_t* tiled;
     const void* L; const void* R;                             // bf16, or int4 codes
     const __nv_bfloat16* Ls; const __nv_bfloat16* Rs;         // scales of quantized adapters
@@ -70,8 +72,8 @@ struct SmallParams {
     uint32_t* status;
     float s;
     int b, r, d_out, d_in;
-    bool ahead;                                               // ask the first lines into the L2 while the grid before ends
-    int tiles, units, groups;                                 // of 256 rows, 256 columns, 32 rows of R
+    int units, groups;                                        // of 256 columns, 32 rows of R
+    int ahead;                                                // ask the first lines into the L2 while the grid before ends
 };
 
 // NT tiles of 8 tokens; a warp's MT tiles of 16 rows (four warps: 64 MT rows of the layer).
@@ -221,6 +223,8 @@ __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
 __device__ __forceinline__ uint4 pair_four_apart(const uint4& v) {
     return make_uint4(prmt(v.x, v.z, 0x5410), prmt(v.x, v.z, 0x7632), prmt(v.y, v.w, 0x5410), prmt(v.y, v.w, 0x7632));
 }
+
+static_assert(sizeof(SmallParams) == 128, "the tensor maps' place in the parameters");
 
 // ---------------------------------------------------------------- one stage of the weight
 struct Lane { int lane, g, t; };
@@ -514,7 +518,11 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
     const uint32_t part = smem + C_::kOffPart, recv = smem + C_::kOffRecv, bars = smem + C_::kOffBars;
     const uint32_t full = bars, empty = bars + 32, piece_bar = bars + 64, red_full = bars + 72, t_full = bars + 80, t_empty = bars + 144, gone = bars + 208;
 
-    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;      // (a shuffle: the same in all lanes, for the compiler too)
+    const int lane = threadIdx.x & 31;
+    const int warp = QA ? threadIdx.x >> 5 : __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0);       // (a shuffle: the same in all lanes, for the compiler too)
+    // The lane that requests.  (Beside int4 adapters the branch on the lane's number, two lanes' requests with one instruction, is the faster one:
+    // 5120 x 5120, rank 512, 7 tokens 8.1 us against 8.5, 4096 x 4096, rank 208, 6 tokens 6.5 against 7.1, weights in the L2.)
+    auto asks = [&] { return QA ? lane == 0 : elect_one(); };
     Lane ln; ln.lane = lane; ln.g = lane >> 2; ln.t = lane & 3;
     uint32_t C, rank;
     asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(C));
@@ -547,11 +555,12 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
     if (warp == kProdX && lane == 0) { prefetch_map(&tmX); prefetch_map(&tmM); }
     // The first lines of this CTA's part of the weight or of R go into the L2 meanwhile.  Nothing is read by that: what the grid before still
     // writes is what the loads behind the wait find there.
-    if (p.ahead && NT < 8 && warp < kCW) {
+    constexpr bool kAsksAhead = NT < 8 && FMT != FMT_TILED && !(QA && MT < 4);      // (see p.ahead: beside int4 adapters only layers of the tall tiles)
+    if (kAsksAhead && p.ahead && warp < kCW) {
         if (makes_T) {
             const size_t unit = QA ? kUnit / 2 : kUnit * 2;
             lines_ahead(p.R, (size_t)p.d_in * unit / kUnit, piece * kGroup, min(kGroup, p.r - piece * kGroup), u0 * unit, u1 * unit);
-        } else if (FMT != FMT_TILED) {
+        } else {
             const int row0 = tile * kRows, rows = min(kRows, p.d_out - row0);
             lines_ahead(p.vals, (size_t)p.d_in / 4, row0, rows, (size_t)u0 * 64, (size_t)u_end * 64);
             lines_ahead(p.meta, (size_t)p.d_in / 8, row0, rows, (size_t)u0 * 32, (size_t)u_end * 32);
@@ -592,7 +601,7 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
             for (int u = u0; u < u1; ++u) {
                 const int st = acquire();
                 const uint32_t bar = full + 8 * st;
-                if (elect_one()) {
+                if (asks()) {
                     mbar_expect(bar, QA ? 4096 : 16384);
                     if (QA) tma_tile(smem + st * kStage, &tmR, u * 128, piece * kGroup, bar);
                     else tma_tile3(smem + st * kStage, &tmR, piece * kGroup, u * 4, bar);
@@ -603,7 +612,7 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
             for (int u = u0; u < u_end; ++u) {
                 const int st = acquire();
                 const uint32_t dst = smem + st * kStage, bar = full + 8 * st;
-                if (elect_one()) {
+                if (asks()) {
                     mbar_expect(bar, FMT == FMT_TILED ? groups * 6144 : kValsBytes);
                     if (FMT == FMT_TILED) {
                         for (int i = 0; i < groups; ++i) bulk_copy(dst + i * 6144, p.tiled + ((size_t)(tile * 4 + i) * p.units + u) * 6144, 6144, bar);
@@ -618,7 +627,7 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
                 const uint32_t dst = smem + st * kStage, bar = full + 8 * st;
                 if (l_by_lanes) {
                     codes_of_L(lc, dst, bar, 0);
-                } else if (elect_one()) {
+                } else if (asks()) {
                     mbar_expect(bar, kRows * (QA ? 32 : 64));
                     mbar_arrive(bar);                           // in place of the other producer
                     tma_tile(dst, &tmL, lc * 32, row0, bar);
@@ -634,7 +643,7 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
             for (int u = u0; u < u1; ++u) {
                 const int st = acquire();
                 const uint32_t bar = full + 8 * st;
-                if (elect_one()) {
+                if (asks()) {
                     mbar_expect(bar, C_::kXBytes);
                     tma_tile3(smem + st * kStage + kXOff, &tmX, 0, u * 4, bar);
                 }
@@ -666,7 +675,12 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
             for (int u = u0; u < u_end; ++u) {
                 const int st = acquire();
                 const uint32_t dst = smem + st * kStage, bar = full + 8 * st;
-                if (elect_one()) {
+                if (QA) {                                       // (both requests with one instruction)
+                    if (lane == 0) mbar_expect(bar, C_::kXBytes + (FMT == FMT_PACKED ? kMetaBytes : 0));
+                    __syncwarp();
+                    if (lane == 0) tma_tile3(dst + kXOff, &tmX, 0, u * 4, bar);
+                    if (FMT == FMT_PACKED && lane == 1) tma_tile(dst + kValsBytes, &tmM, u * 32, row0, bar);
+                } else if (elect_one()) {
                     mbar_expect(bar, C_::kXBytes + (FMT == FMT_PACKED ? kMetaBytes : 0));
                     if (FMT == FMT_PACKED) tma_tile(dst + kValsBytes, &tmM, u * 32, row0, bar);
                     tma_tile3(dst + kXOff, &tmX, 0, u * 4, bar);
@@ -1162,9 +1176,13 @@ slim_status_t launch_small(const __nv_bfloat16* X, int b, const uint8_t* vals, c
     p.status = status_dev; p.s = s; p.b = b; p.r = r; p.d_out = d_out; p.d_in = d_in;
     // Up to 40 MB of weight the HBM is idle for much of a call (start, hand-over of T, exchange): the lines asked for ahead come for nothing
     // (4096 x 4096, rank 416, one token 8.2 -> 7.7 us a call, 11008 -> 4096, 4 tokens 13.0 -> 12.2; 33 to 64 tokens gain nothing).  Beyond, it is
-    // busy throughout and they come in the way (28672 -> 8192, 16 tokens 49 -> 53).
-    p.ahead = (size_t)d_out * (size_t)d_in * 3 / 8 <= (size_t)40 << 20;
-    p.tiles = ceil_div(d_out, rows); p.units = units; p.groups = groups;
+    // busy throughout and they come in the way (28672 -> 8192, 16 tokens 49 -> 53).  Where the weight is in the L2 already they cost some
+    // instructions, which shows where a call is short: without adapters they are asked up to 16 MB (5120 -> 6912, one token, from the HBM 7.2 ->
+    // 6.75, from the L2 6.3 -> 6.4; 8192 x 8192 9.8 -> 9.8, 8.6 -> 9.4), beside int4 adapters from 12 MB on (4096 -> 11008, rank 416 12.65 ->
+    // 11.85; 5120 x 5120, rank 512 9.3 -> 9.15, 8.1 -> 8.6).
+    const size_t weight = (size_t)d_out * (size_t)d_in * 3 / 8;
+    p.ahead = weight <= (size_t)(r > 0 ? 40 : 16) << 20 && (!qa || (mt == 4 && weight >= (size_t)12 << 20));
+    p.units = units; p.groups = groups;
     CUtensorMap tmV, tmM, tmX, tmR, tmL;
     bool ok = make_map3(&tmX, X, (uint64_t)d_in, (uint64_t)b, nt * 8);
     if (!tiled) ok = ok && make_map(&tmV, vals, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)d_in / 4, (uint64_t)d_out, 64, rows, CU_TENSOR_MAP_SWIZZLE_64B);
@@ -1179,7 +1197,7 @@ slim_status_t launch_small(const __nv_bfloat16* X, int b, const uint8_t* vals, c
     else tmL = tmX;
     if (!ok) return SLIM_ERR_CUDA;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(C * (p.tiles + p.groups))); cfg.blockDim = dim3(threads_of(nt)); cfg.dynamicSmemBytes = smem_bytes(nt, mt); cfg.stream = st;
+    cfg.gridDim = dim3((unsigned)(C * (ceil_div(d_out, rows) + groups))); cfg.blockDim = dim3(threads_of(nt)); cfg.dynamicSmemBytes = smem_bytes(nt, mt); cfg.stream = st;
     cudaLaunchAttribute a[2];
     a[0].id = cudaLaunchAttributeClusterDimension;
     a[0].val.clusterDim.x = (unsigned)C; a[0].val.clusterDim.y = 1; a[0].val.clusterDim.z = 1;
