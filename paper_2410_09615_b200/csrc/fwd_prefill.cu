@@ -584,6 +584,7 @@ prefill_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap tmV,
             uint32_t e[2];
             expand_row<64>(pk, row, q, x, m0 + row < p.m_total, 64, a, e);
             store_row(stages + (size_t)st * kStageBytes + kBTile, row, a);
+            fence_after_sync();                              // the MMAs have read what is stored over
             asm volatile("tcgen05.st.sync.aligned.32x32b.x2.b32 [%0], {%1, %2};"
                          :: "r"(tmem_base + lane_base + kECol + 4 * st), "r"(e[0]), "r"(e[1]) : "memory");
             asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
@@ -987,9 +988,14 @@ prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap t
             if (g >= kStages) ok = mbar_wait(&empty[st], ((g / kStages) & 1) ^ 1, abort_flag) && ok;
             arrive(st, bytes);
         };
-        // Whether a phase has ended, as lane 0 finds it; the answer is looked at later.
+        // Whether a phase has ended, as lane 0 finds it; the answer is looked at later.  (The shuffle hands the answer over, the barrier behind
+        // it what lane 0 has acquired with it.)
         auto ask = [&](uint64_t* bar, uint32_t phase) { return lane == 0 ? mbar_test(bar, phase, false) : 0u; };
-        auto yes = [&](uint32_t answer) { return __shfl_sync(0xffffffffu, answer, 0) != 0; };
+        auto yes = [&](uint32_t answer) {
+            const bool there = __shfl_sync(0xffffffffu, answer, 0) != 0;
+            __syncwarp();
+            return there;
+        };
         // The groups take turns.  A group waits by parity for the MMAs of stage g - 5, which is right when it knows those of stage g - 10 to be
         // complete and those of g are still to come: with turns of at most five stages.  Where a turn is longer (from T' to the first tile,
         // from tile to tile) it waits for another group's stage in between.
@@ -1041,7 +1047,10 @@ prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap t
                         const int gn = gi + kGroups / kPkStages;
                         pk_there = it + kGroups < n_groups * kPkStages ? ask(&pk_full[gn % kPkSlots], (gn / kPkSlots) & 1) : 0u;
                     }
-                    if (hh == 0 && !yes(free)) ok = mbar_wait(&empty[st], ((g / kStages) & 1) ^ 1, abort_flag) && ok;
+                    if (hh == 0) {
+                        if (!yes(free)) ok = mbar_wait(&empty[st], ((g / kStages) & 1) ^ 1, abort_flag) && ok;
+                        fence_after_sync();                                  // the MMAs have read what is stored over
+                    }
                     asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};"
                                  :: "r"(tmem_base + lane_base + kECol + Cfg::kECols * st + 4 * hh), "r"(e[0]), "r"(e[1]), "r"(e[2]), "r"(e[3]) : "memory");
                     tmem_st32(tmem_base + lane_base + Cfg::kACol + Cfg::kACols * st + 32 * hh, a);
