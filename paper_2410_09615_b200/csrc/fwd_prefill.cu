@@ -52,6 +52,7 @@
 #include <cuda.h>
 #include "common.cuh"
 #include "handover.h"
+#include "turns.h"
 
 namespace slim {
 
@@ -687,6 +688,7 @@ template <int N> struct PairCfg {
     static constexpr int kTWidth = kECol;                                   // most columns of r in a T' tile
     static constexpr size_t kSmem = 1024 + (size_t)kStages * kStageBytes + kPkSlots * kPkSlotBytes + 384 + 8 * 1024;     // .. barriers, epilogue
     static_assert(kECol + kStages * kECols <= kACol && kACol + kStages * kACols <= 512, "tensor memory");
+    static_assert(kGroups == kTurnGroups && kStages == kTurnPlaces && kPkSlots == kTurnSlots, "the turns' rings");
 };
 constexpr size_t kSyncTiles = kSmallTBytes / 16 - 1024;     // T' tiles whose words fit the region beside those of the pairs
 
@@ -996,43 +998,22 @@ prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap t
             __syncwarp();
             return there;
         };
-        // The groups take turns.  A group waits by parity for the MMAs of stage g - 5, which is right when it knows those of stage g - 10 to be
-        // complete and those of g are still to come: with turns of at most five stages.  Where a turn is longer (from T' to the first tile,
-        // from tile to tile) it waits for another group's stage in between.
-        int last = -1;
-        auto turn_at = [&](int g) {
-            while (g - last > kStages) {
-                last += kGroups;
-                if (last >= kStages) ok = mbar_wait(&empty[last % kStages], ((last / kStages) & 1) ^ 1, abort_flag) && ok;
-            }
-            last = g;
-        };
+        // The groups take the stages in turn (turns.h: why the waits by parity are right).
         int base = t_end - t_begin, nth = 0;         // stages before this tile
-        for (int g = group; g < base; g += kGroups) { turn_at(g); pass(g, (uint32_t)(2 * (kPM + p.t_n / 2) * kDK * 2)); }
-        uint32_t pk_there = 0;
+        for (int g = first_turn(group, 0); g < base; g += kGroups) pass(g, (uint32_t)(2 * (kPM + p.t_n / 2) * kDK * 2));
         for (int t = first_tile; t < p.tiles; t += pairs, base += n_total, ++nth) {
             const bool row_in = tile_of(t).m0 + row < p.m_total;
-            // (turns go by the packed tiles: a group sees every phase of their barriers that it has a stage of)
-            const int all = max(n_total, n_groups * kPkStages);
-            for (int it = (group - nth * n_groups * kPkStages) & (kGroups - 1); it < all; it += kGroups) {
-                if (it >= p.n1) {
-                    if (it < n_groups * kPkStages) {                         // the second half of a last, half packed tile: seen, and given back
-                        const int gi = (nth + 1) * n_groups - 1, slot = gi % kPkSlots;
-                        if (!yes(pk_there)) ok = mbar_wait(&pk_full[slot], (gi / kPkSlots) & 1, abort_flag) && ok;
-                        pk_there = 0;
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(&pk_empty[slot]);
-                    }
-                    if (it < n_total) { turn_at(base + it); pass(base + it, (uint32_t)(2 * (half_tok + kPM) * kDK * 2)); }
-                    continue;
-                }
-                turn_at(base + it);
+            uint32_t pk_there = 0;
+            const int seen = seen_from(nth, p.n1, p.n2, kPkStages);
+            int it = first_turn(group, base);
+            for (; it < p.n1; it += kGroups) {
                 const int g = base + it, st = g % kStages;
                 // expand into registers as soon as the packed tile is there (and give its slot back), store when the MMAs of
                 // the stage's previous use are done: only the stores are between that and the next MMAs.  Both barriers are asked ahead.
                 const int gi = nth * n_groups + it / kPkStages, q = it % kPkStages, slot = gi % kPkSlots;
+                if (it < seen && g >= kStages) ok = mbar_wait(&empty[st], ((g / kStages) & 1) ^ 1, abort_flag) && ok;
                 if (!yes(pk_there)) ok = mbar_wait(&pk_full[slot], (gi / kPkSlots) & 1, abort_flag) && ok;
-                const uint32_t free = g >= kStages ? ask(&empty[st], ((g / kStages) & 1) ^ 1) : 1u;
+                const uint32_t free = it >= seen && g >= kStages ? ask(&empty[st], ((g / kStages) & 1) ^ 1) : 1u;
 #pragma unroll
                 for (int hh = 0; hh < kSK / 128; ++hh) {
                     uint4 a[8];
@@ -1042,10 +1023,11 @@ prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap t
                     for (int i = 0; i < 8; ++i) asm volatile("" : "+r"(a[i].x), "+r"(a[i].y), "+r"(a[i].z), "+r"(a[i].w));     // here, not after the wait
                     if (hh + 1 == kSK / 128) {
                         __syncwarp();
-                        if (lane == 0) mbar_arrive(&pk_empty[slot]);
+                        // (half a packed tile at the end: for the other half too)
+                        if (lane <= (q + 1 < kPkStages && it + 1 == p.n1 ? 1 : 0)) mbar_arrive(&pk_empty[slot]);
                         // the packed tile of this group's next stage in this tile
-                        const int gn = gi + kGroups / kPkStages;
-                        pk_there = it + kGroups < n_groups * kPkStages ? ask(&pk_full[gn % kPkSlots], (gn / kPkSlots) & 1) : 0u;
+                        constexpr int kNext = kGroups / kPkStages;
+                        pk_there = it + kGroups < p.n1 && it + kGroups >= seen ? ask(&pk_full[(gi + kNext) % kPkSlots], ((gi + kNext) / kPkSlots) & 1) : 0u;
                     }
                     if (hh == 0) {
                         if (!yes(free)) ok = mbar_wait(&empty[st], ((g / kStages) & 1) ^ 1, abort_flag) && ok;
@@ -1059,6 +1041,7 @@ prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap t
                 fence_before_sync();
                 arrive(st, (uint32_t)(2 * half_tok * kSK * 2));
             }
+            for (; it < n_total; it += kGroups) pass(base + it, (uint32_t)(2 * (half_tok + kPM) * kDK * 2));
         }
     } else {
         // ============================ epilogue: thread = output row, half of the tokens ============================
