@@ -109,7 +109,6 @@ struct alignas(128) PrefillParams {      // (so are the tensor maps behind it in
     // T' inside the pair kernel: chunks of t_n columns (of r), tiles of 256 tokens x t_n, 64-column stages of one, pairs that
     // share the work; 1 / s; T' itself, partial tiles, and per (tile, CTA) {arrivals, ready} words that carry the call number
     int r, t_n, t_chunks, t_tiles, t_stages, t_pairs;
-    bool t_ranks;           // the MMA's rows are ranks and its columns tokens, not the other way round
     float t_scale;
     __nv_bfloat16* t_out;
     float4* t_part;
@@ -730,12 +729,14 @@ __device__ __forceinline__ void store_T(__nv_bfloat16* at, size_t tail, float4 v
     put(v);
 }
 
-// Four neighbouring values of a row of a T' tile: ranks of a token, or (how & 1) tokens of a rank; in two parts: how & 2.  (As a function that is
-// called a first pass on cold instructions took 2 us less, every other 0.7-1 us more where T' is what a call waits for.)
-__device__ __forceinline__ void put_T(__nv_bfloat16* out, int a_row, int b_row, int b, int r, int how, float4 v)
+// Four neighbouring values of a row of a T' tile: ranks of a token, or (RANKS) tokens of a rank; in two parts where `tail` is not 0.  (Which of the
+// two is known when the kernel is compiled: with the question asked at every store, and the rows worked out there, the first pass over the
+// longer code made the sums 1-3 us longer: 5120 x 5120, rank 512, 720 tokens 39.6 us a call, 43.0 so; 2304 -> 1568, rank 160, 300 tokens 20.8,
+// 22.3.  As a function that is called a first pass took 2 us less, every other 0.7-1 us more where T' is what a call waits for.)
+template <bool RANKS>
+__device__ __forceinline__ void put_T(__nv_bfloat16* out, int a_row, int b_row, int b, int r, size_t tail, float4 v)
 {
-    const size_t tail = how & 2 ? (size_t)b * r : 0;
-    if (how & 1) {
+    if constexpr (RANKS) {
         if (a_row >= r) return;
         const float t[4] = {v.x, v.y, v.z, v.w};
         __nv_bfloat16* at = out + (size_t)b_row * r + a_row;
@@ -750,7 +751,7 @@ __device__ __forceinline__ void put_T(__nv_bfloat16* out, int a_row, int b_row, 
     }
 }
 
-template <int N>
+template <int N, bool RANKS>
 __global__ void __launch_bounds__(kPairThreads, 1)
 prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmM,
                     const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmA2, const __grid_constant__ CUtensorMap tmB2,
@@ -809,7 +810,7 @@ prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap t
     const uint32_t call = p.r > 0 ? call_number(*(volatile unsigned long long*)p.departures) : 0u;
     bool ok = true;
     // Which 256 rows of its A operand a T' tile is made of, and which t_n rows of its B operand.
-    auto t_part_of = [&](int tile, bool a) { return a != p.t_ranks ? tile / p.t_chunks : tile % p.t_chunks; };
+    auto t_part_of = [&](int tile, bool a) { return a != RANKS ? tile / p.t_chunks : tile % p.t_chunks; };
     // Tile -> its first row in this CTA, its first token, and where its walk over the weight columns starts: pairs that share
     // token rows start at different places, so that at any moment they ask the L2 for different lines of X.
     struct Tile { int m0, n0, rot; };
@@ -862,7 +863,7 @@ prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap t
                     if (ti.n0 != t_checked) {
                         // T' tiles of 256 tokens: one or two halves of them; T' tiles of this tile's tokens: both halves of the ranks
                         const int tok = ti.n0 + (int)rank * half_tok;
-                        const int blk0 = p.t_ranks ? ti.n0 / half_tok : tok / kPM, blk1 = p.t_ranks ? blk0 + 2 : ceil_div(min(tok + half_tok, p.b), kPM);
+                        const int blk0 = RANKS ? ti.n0 / half_tok : tok / kPM, blk1 = RANKS ? blk0 + 2 : ceil_div(min(tok + half_tok, p.b), kPM);
                         for (int blk = blk0; blk < blk1; ++blk) {
                             const int tile0 = (blk / 2) * p.t_chunks;
                             const uint32_t t_half = (uint32_t)blk & 1;
@@ -1053,10 +1054,11 @@ prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap t
         // ---- T': thread = token (t_ranks: rank).  Part of pair q: [c / 4][128 tokens] float4; a pair has at most one that starts with its tile and
         // one that does not.
         auto part = [&](int q, bool starts) { return p.t_part + ((size_t)(2 * q + (starts ? 1 : 0)) * 2 + rank) * ((size_t)kPM * p.t_n / 4) + row; };
-        auto store4 = [&](int tile, int c, float4 v) {
-            const int a_row = t_part_of(tile, true) * kTTok + (int)rank * kPM + row, b_row = t_part_of(tile, false) * p.t_n + c;
-            put_T(p.t_out, a_row, b_row, p.b, p.r, (p.t_ranks ? 1 : 0) | (p.t_parts == 2 ? 2 : 0),
-                  make_float4(p.t_scale * v.x, p.t_scale * v.y, p.t_scale * v.z, p.t_scale * v.w));
+        const size_t t_tail = p.t_parts == 2 ? (size_t)p.b * p.r : 0;
+        int a_row = 0, b_row = 0;                                            // of the run's tile
+        auto rows_of = [&](int tile) { a_row = t_part_of(tile, true) * kTTok + (int)rank * kPM + row; b_row = t_part_of(tile, false) * p.t_n; };
+        auto store4 = [&](int c, float4 v) {
+            put_T<RANKS>(p.t_out, a_row, b_row + c, p.b, p.r, t_tail, make_float4(p.t_scale * v.x, p.t_scale * v.y, p.t_scale * v.z, p.t_scale * v.w));
         };
         auto publish = [&](size_t word) {                                    // the writes of the eight warps, then the word
             epilogue_sync();
@@ -1070,6 +1072,7 @@ prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap t
             const Run run = run_at(u, t_end, p.t_stages);
             u += run.len;
             const bool whole = run.len == p.t_stages;
+            rows_of(run.tile);
             ok = mbar_wait(acc_full, nth & 1, abort_flag) && ok;
             fence_after_sync();
             float4* mine = part(tq, run.k0 == 0);
@@ -1079,7 +1082,7 @@ prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap t
                 tmem_ld16(t_addr + c, v);
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
-                    if (whole) store4(run.tile, c + 4 * i, v[i]);
+                    if (whole) store4(c + 4 * i, v[i]);
                     else __stcg(mine + (size_t)(c / 4 + i) * kPM, v[i]);
                 }
             }
@@ -1095,6 +1098,7 @@ prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap t
             if (run.len == p.t_stages) continue;
             const int q0 = share_owner(run.tile * p.t_stages, t_units, p.t_pairs), q1 = share_owner((run.tile + 1) * p.t_stages - 1, t_units, p.t_pairs);
             const int n = q1 - q0 + 1;
+            rows_of(run.tile);
             for (int q = q0; q <= q1; q += 32)
                 ok = wait_words(q + lane <= q1 ? p.t_sync + part_word(q + lane, q + lane == q0, rank) : nullptr, call, abort_flag) && ok;
             if (n == 2) {                                                    // two parts: four columns' loads in flight
@@ -1108,7 +1112,7 @@ prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap t
                     }
 #pragma unroll
                     for (int i = 0; i < 4; ++i)
-                        if (c4 + 4 * i < p.t_n / 4) store4(run.tile, 4 * (c4 + 4 * i), make_float4(x[i].x + y[i].x, x[i].y + y[i].y, x[i].z + y[i].z, x[i].w + y[i].w));
+                        if (c4 + 4 * i < p.t_n / 4) store4(4 * (c4 + 4 * i), make_float4(x[i].x + y[i].x, x[i].y + y[i].y, x[i].z + y[i].z, x[i].w + y[i].w));
                 }
             } else if (n <= 4) {                                             // four parts of two columns
                 for (int c4 = 2 * (tq - q0) + half; c4 < p.t_n / 4; c4 += 4 * n) {
@@ -1125,8 +1129,8 @@ prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap t
                             x[0].x += x[i].x; x[0].y += x[i].y; x[0].z += x[i].z; x[0].w += x[i].w;
                             y[0].x += y[i].x; y[0].y += y[i].y; y[0].z += y[i].z; y[0].w += y[i].w;
                         }
-                    store4(run.tile, 4 * c4, x[0]);
-                    if (c5 < p.t_n / 4) store4(run.tile, 4 * c5, y[0]);
+                    store4(4 * c4, x[0]);
+                    if (c5 < p.t_n / 4) store4(4 * c5, y[0]);
                 }
             } else {
                 for (int c4 = 2 * (tq - q0) + half; c4 < p.t_n / 4; c4 += 2 * n) {
@@ -1138,7 +1142,7 @@ prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap t
 #pragma unroll
                         for (int i = 0; i < 8; ++i) { s.x += v[i].x; s.y += v[i].y; s.z += v[i].z; s.w += v[i].w; }
                     }
-                    store4(run.tile, 4 * c4, s);
+                    store4(4 * c4, s);
                 }
             }
             publish(part_word(tq, run.k0 == 0, rank) + 1);
@@ -1404,7 +1408,7 @@ static slim_status_t launch_tile_kernel(const PrefillParams& q, int m_rows, cons
     return e == cudaSuccess ? SLIM_OK : SLIM_ERR_CUDA;
 }
 
-template <int N>
+template <int N, bool RANKS>
 static slim_status_t launch_pair(const PrefillParams& p, const CUtensorMap& tmV, const CUtensorMap& tmM, const CUtensorMap& tmX, const CUtensorMap& tmA2,
                                  const CUtensorMap& tmB2, const CUtensorMap& tmTA, const CUtensorMap& tmTB, int pairs, cudaStream_t st) {
     cudaLaunchConfig_t cfg = {};
@@ -1423,7 +1427,7 @@ static slim_status_t launch_pair(const PrefillParams& p, const CUtensorMap& tmV,
         attr[1].val.programmaticStreamSerializationAllowed = 1;
     }
     cfg.attrs = attr; cfg.numAttrs = 2;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, prefill_pair_kernel<N>, p, tmV, tmM, tmX, tmA2, tmB2, tmTA, tmTB);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, prefill_pair_kernel<N, RANKS>, p, tmV, tmM, tmX, tmA2, tmB2, tmTA, tmTB);
     count_launch(1);
     return e == cudaSuccess ? SLIM_OK : SLIM_ERR_CUDA;
 }
@@ -1451,9 +1455,11 @@ slim_status_t launch_prefill(const __nv_bfloat16* X, int b, const uint8_t* vals,
     cudaGetDevice(&dev);
     if (dev < 0 || dev >= 64) return SLIM_ERR_CUDA;
     if (!g_prefill_attr_set[dev].load(std::memory_order_acquire)) {
-        if (cudaFuncSetAttribute(prefill_pair_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PairCfg<256>::kSmem) != cudaSuccess ||
-            cudaFuncSetAttribute(prefill_pair_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PairCfg<128>::kSmem) != cudaSuccess ||
-            cudaFuncSetAttribute(prefill_pair_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PairCfg<64>::kSmem) != cudaSuccess ||
+        if (cudaFuncSetAttribute(prefill_pair_kernel<256, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PairCfg<256>::kSmem) != cudaSuccess ||
+            cudaFuncSetAttribute(prefill_pair_kernel<128, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PairCfg<128>::kSmem) != cudaSuccess ||
+            cudaFuncSetAttribute(prefill_pair_kernel<128, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PairCfg<128>::kSmem) != cudaSuccess ||
+            cudaFuncSetAttribute(prefill_pair_kernel<64, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PairCfg<64>::kSmem) != cudaSuccess ||
+            cudaFuncSetAttribute(prefill_pair_kernel<64, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PairCfg<64>::kSmem) != cudaSuccess ||
             cudaFuncSetAttribute(prefill_kernel<64, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PfCfg<64, false>::kSmem) != cudaSuccess ||
             cudaFuncSetAttribute(prefill_kernel<64, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PfCfg<64, true>::kSmem) != cudaSuccess ||
             cudaFuncSetAttribute(prefill_kernel<256, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PfCfg<256, true>::kSmem) != cudaSuccess)
@@ -1465,7 +1471,7 @@ slim_status_t launch_prefill(const __nv_bfloat16* X, int b, const uint8_t* vals,
         attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
         cfg.attrs = attr; cfg.numAttrs = 1;
         int n = 0;
-        if (cudaOccupancyMaxActiveClusters(&n, prefill_pair_kernel<256>, &cfg) != cudaSuccess || n < 1) return SLIM_ERR_CUDA;
+        if (cudaOccupancyMaxActiveClusters(&n, prefill_pair_kernel<256, false>, &cfg) != cudaSuccess || n < 1) return SLIM_ERR_CUDA;
         g_pairs[dev].store(n < di->sm_count / 2 ? n : di->sm_count / 2, std::memory_order_relaxed);
         g_prefill_attr_set[dev].store(true, std::memory_order_release);
     }
@@ -1548,15 +1554,16 @@ slim_status_t launch_prefill(const __nv_bfloat16* X, int b, const uint8_t* vals,
         p.r = r;
         int grid = p.tiles < pairs ? p.tiles : pairs;
         if (r > 0) {
-            p.t_ranks = plan.t_ranks; p.t_n = plan.t_n; p.t_chunks = plan.t_chunks; p.t_tiles = plan.t_tiles; p.t_stages = d_in / PairCfg<256>::kDK;
+            p.t_n = plan.t_n; p.t_chunks = plan.t_chunks; p.t_tiles = plan.t_tiles; p.t_stages = d_in / PairCfg<256>::kDK;
             p.t_scale = 1.f / s_eff; p.t_out = Tq;
             p.t_part = reinterpret_cast<float4*>(reinterpret_cast<char*>(Tq) + t_bytes(b, r, t_parts));
             p.t_pairs = t_share(p.t_tiles, p.t_stages, pairs, pairs - grid, s != 0.f ? ceil_div(d_in, 128) : 0);
             grid = grid + p.t_pairs < pairs ? grid + p.t_pairs : pairs;      // the last pairs make T'
         }
-        rc = tile_n > 128 ? launch_pair<256>(p, tmV, tmM, tmX, tmA2, tmB2, tmTA, tmTB, grid, st)
-           : tile_n > 64  ? launch_pair<128>(p, tmV, tmM, tmX, tmA2, tmB2, tmTA, tmTB, grid, st)
-                          : launch_pair<64>(p, tmV, tmM, tmX, tmA2, tmB2, tmTA, tmTB, grid, st);
+        auto* launch = tile_n > 128 ? launch_pair<256, false>
+                     : tile_n > 64  ? (plan.t_ranks ? launch_pair<128, true> : launch_pair<128, false>)
+                                    : (plan.t_ranks ? launch_pair<64, true> : launch_pair<64, false>);
+        rc = launch(p, tmV, tmM, tmX, tmA2, tmB2, tmTA, tmTB, grid, st);
     }
     if (rc != SLIM_OK) return rc;
     return SLIM_OK;
