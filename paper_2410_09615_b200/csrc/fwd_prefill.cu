@@ -52,6 +52,7 @@
 #include <cuda.h>
 #include "common.cuh"
 #include "handover.h"
+#include "pair_plan.h"
 #include "turns.h"
 
 namespace slim {
@@ -675,7 +676,7 @@ prefill_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap tmV,
 // TMA writes 38 KB, converters read 6, tensor core reads 32); with 128 tokens 0.25.
 // A token-tile warp sees every second phase of an `empty` barrier.  Waiting by parity is still right: before its stage g it has waited
 // for the MMAs of stage g - 7, so the phase it did not see (stage g - 10) is over.
-constexpr int kTTok = 256;              // tokens of a T' tile (the rows of its MMA)
+constexpr int kTTok = kPairTTok;        // tokens of a T' tile (the rows of its MMA)
 constexpr int kPairThreads = 28 * 32;
 template <int N> struct PairCfg {
     static constexpr int kGroups = 4, kWarpEpi = 4 * kGroups, kWarpX = kWarpEpi + 8, kWarpMma = kWarpX + 2, kWarpPk = kWarpX + 3;
@@ -684,7 +685,7 @@ template <int N> struct PairCfg {
     // tensor memory: the accumulator (a T' tile's may be as wide), index words (kSK / 32 columns a stage), expanded weights (kSK / 4
     // columns a stage)
     static constexpr int kECols = kSK / 32, kACols = kSK / 4, kECol = N <= 128 ? 128 : 256, kACol = N <= 128 ? 192 : 288;
-    static constexpr int kTWidth = kECol;                                   // most columns of r in a T' tile
+    static_assert(kDK == kPairDK && 2 * kPM == kPairRows, "the plan's tiles");      // (a T' tile has up to kECol columns)
     static constexpr size_t kSmem = 1024 + (size_t)kStages * kStageBytes + kPkSlots * kPkSlotBytes + 384 + 8 * 1024;     // .. barriers, epilogue
     static_assert(kECol + kStages * kECols <= kACol && kACol + kStages * kACols <= 512, "tensor memory");
     static_assert(kGroups == kTurnGroups && kStages == kTurnPlaces && kPkSlots == kTurnSlots, "the turns' rings");
@@ -1287,75 +1288,7 @@ bool prefill_supports(int b, int d_out, int d_in, int r) {
     return b >= 1 && d_out % 16 == 0 && d_in % kPBK == 0 && r % 16 == 0 && r >= 0;
 }
 
-// Columns of a T' tile of the pair kernel that cuts r into `chunks`.
-static int t_width(int r, int chunks) { return r > 0 ? ceil_div(ceil_div(r, chunks), 16) * 16 : 16; }
-static size_t pair_part_bytes(int r, int sm_count) { return (size_t)(sm_count / 2) * 2 * 256 * t_width(r, ceil_div(r, 256)) * sizeof(float); }
-// Chunks of r: of up to `most` columns, and as many as leave a tile up to eight of the pairs that have no other work.  (A tile's parts are added up by
-// these pairs, each part of a column asked for by each of them: 4096 -> 11008, rank 416, 256 tokens, two tiles of 15 parts of four stages,
-// the sums took 4 us, of 7 parts 2.)
-static int t_chunks(int r, int most, int token_tiles, int spare) {
-    int chunks = ceil_div(r, most);
-    while (spare / (token_tiles * chunks) > 8 && t_width(r, chunks + 1) >= 48) ++chunks;
-    return chunks;
-}
-
-// Pairs that share the work of T'.  Each tile in equal parts, one a pair, where that uses four fifths of the pairs or more
-// (a pair then has one part to write, and the pairs that read the same X walk it together); else an even share each.
-// Four stages (a microsecond and a half) or more for a part: below that its start and end dominate.
-// Where the tiles leave pairs without one and those can make T' in about the time of the others' sparse phase, they do it
-// alone (`spare` pairs, `main_stages` 128-column stages): the others start their tiles at once.
-static int t_share(int tiles, int stages, int pairs, int spare, int main_stages) {
-    const int most = stages < 4 ? 1 : stages / 4;
-    int parts = spare / tiles < most ? spare / tiles : most;
-    if (parts >= 1 && (long long)ceil_div(stages, parts) <= main_stages) return tiles * parts;
-    parts = pairs / tiles < most ? pairs / tiles : most;
-    if (parts >= 1 && (parts == most || tiles * parts * 5 >= pairs * 4)) return tiles * parts;
-    return (long long)tiles * most < pairs ? tiles * most : pairs;
-}
-
-// How the pair kernel cuts a problem: tokens of a tile (a multiple of 16), tiles, and the tiles of T'.
-struct PairPlan { int tile_n, tiles, t_n, t_chunks, t_tiles; bool t_ranks; };
-static PairPlan plan_tiles(int b, int d_out, int r, int widest, int pairs) {
-    PairPlan pl;
-    pl.tile_n = ceil_div(ceil_div(b, ceil_div(b, widest)), 16) * 16;
-    pl.tiles = ceil_div(d_out, 2 * kPM) * ceil_div(b, pl.tile_n);
-    // T' tiles of narrow token tiles have up to 128 columns of tensor memory: chunks of the ranks, or, where that makes fewer tiles, the
-    // tile's tokens
-    const int most = pl.tile_n <= 128 ? PairCfg<128>::kTWidth : PairCfg<256>::kTWidth;
-    pl.t_ranks = most == 128 && r > most && ceil_div(b, pl.tile_n) * ceil_div(r, 2 * kPM) < ceil_div(b, kTTok) * ceil_div(r, most);
-    const int t_tokens = ceil_div(b, pl.t_ranks ? pl.tile_n : kTTok);
-    pl.t_chunks = pl.t_ranks ? ceil_div(r, 2 * kPM) : r > 0 ? t_chunks(r, most, t_tokens, pairs - pl.tiles) : 1;
-    pl.t_n = pl.t_ranks ? pl.tile_n : t_width(r, pl.t_chunks);
-    pl.t_tiles = r > 0 ? t_tokens * pl.t_chunks : 0;
-    return pl;
-}
-// Tiles of up to 256 tokens, or of 128 or 64 where every tile then has a pair of its own: what takes the least time, in units of 10 ns.  A
-// stage of 128 columns takes 0.40 us with 256 tokens, 0.27 with 128, 0.24 with 64; T' 7 us and 0.28 for each of its stages, on
-// the pairs without a tile beside the others (of the shorter of the two a quarter counts: they share the L2), else before them.
-// (4096 -> 4096, rank 416, 256 tokens in tiles of 256, 128, 64: 28.7, 24.8, 27.1 us; 5696 -> 1392, rank 288, 1024 tokens 34.9, 36.9, -;
-// 8192 -> 1024, rank 112, 512 tokens 34.8, 26.9, 26.7.)
-static PairPlan pair_plan(int b, int d_out, int d_in, int r, int pairs) {
-    PairPlan best = {};
-    long long best_cost = -1;
-    for (int widest = 256; widest >= 64; widest /= 2) {
-        const PairPlan pl = plan_tiles(b, d_out, r, widest, pairs);
-        if (best_cost >= 0 && pl.tiles > pairs) break;
-        const int stage = pl.tile_n > 128 ? 40 : pl.tile_n > 64 ? 27 : 24, t_stages = d_in / PairCfg<256>::kDK;
-        const long long main = (long long)ceil_div(pl.tiles, pairs) * ceil_div(d_in, 128) * stage;
-        long long cost = main;
-        if (r > 0) {
-            const int spare = pairs - pl.tiles, parts = spare < pl.t_tiles ? 0 : spare / pl.t_tiles < t_stages / 4 ? spare / pl.t_tiles : t_stages < 4 ? 1 : t_stages / 4;
-            if (parts > 0) {
-                const long long t = 700 + (long long)ceil_div(t_stages, parts) * 28;
-                cost = main > t ? main + t / 4 : t + main / 4;
-            } else {
-                cost = main + 700 + (long long)pl.t_tiles * t_stages * 28 / pairs;
-            }
-        }
-        if (best_cost < 0 || cost < best_cost) { best = pl; best_cost = cost; }
-    }
-    return best;
-}
+static size_t pair_part_bytes(int r, int sm_count) { return (size_t)(sm_count / 2) * 2 * kPairTTok * t_width(r, ceil_div(r, 256)) * sizeof(float); }
 
 // The pair kernel, asked for by the kernel family's name: when its 128 x 256 tiles would give a quarter of the SMs or more a tile.
 // The dispatcher (`automatic`) takes it unless the 128 x 64 tiles of the one-CTA kernel have an SM each and rows are short: the pairs'
