@@ -110,6 +110,7 @@ struct alignas(128) PrefillParams {      // (so are the tensor maps behind it in
     // T' inside the pair kernel: chunks of t_n columns (of r), tiles of 256 tokens x t_n, 64-column stages of one, pairs that
     // share the work; 1 / s; T' itself, partial tiles, and per (tile, CTA) {arrivals, ready} words that carry the call number
     int r, t_n, t_chunks, t_tiles, t_stages, t_pairs;
+    int t_even;             // parts of a T' tile where all have as many, else 0
     float t_scale;
     __nv_bfloat16* t_out;
     float4* t_part;
@@ -810,7 +811,9 @@ prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap t
     asm volatile("fence.proxy.async;" ::: "memory");            // what that grid wrote is read through TMA
     const uint32_t call = p.r > 0 ? call_number(*(volatile unsigned long long*)p.departures) : 0u;
     bool ok = true;
-    // Which 256 rows of its A operand a T' tile is made of, and which t_n rows of its B operand.
+    // The pairs that share a T' tile.  Which 256 rows of its A operand it is made of, and which t_n rows of its B operand.
+    auto first_owner = [&](int tile) { return p.t_even > 0 ? tile * p.t_even : share_owner(tile * p.t_stages, t_units, p.t_pairs); };
+    auto last_owner = [&](int tile) { return p.t_even > 0 ? (tile + 1) * p.t_even - 1 : share_owner((tile + 1) * p.t_stages - 1, t_units, p.t_pairs); };
     auto t_part_of = [&](int tile, bool a) { return a != RANKS ? tile / p.t_chunks : tile % p.t_chunks; };
     // Tile -> its first row in this CTA, its first token, and where its walk over the weight columns starts: pairs that share
     // token rows start at different places, so that at any moment they ask the L2 for different lines of X.
@@ -865,6 +868,16 @@ prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap t
                         // T' tiles of 256 tokens: one or two halves of them; T' tiles of this tile's tokens: both halves of the ranks
                         const int tok = ti.n0 + (int)rank * half_tok;
                         const int blk0 = RANKS ? ti.n0 / half_tok : tok / kPM, blk1 = RANKS ? blk0 + 2 : ceil_div(min(tok + half_tok, p.b), kPM);
+                        const int per = p.t_chunks * p.t_even;
+                        if (per > 0) {                                       // equal parts: the words of a block's chunks follow each other
+                            for (int first = 0; first < (blk1 - blk0) * per; first += 32) {
+                                const bool in = first + lane < (blk1 - blk0) * per, next = first + lane >= per;
+                                const int blk = blk0 + (next ? 1 : 0), i = first + lane - (next ? per : 0), tile0 = (blk / 2) * p.t_chunks;
+                                const size_t word = p.t_even == 1 ? tile_word(p.t_pairs, tile0 + i, (uint32_t)blk & 1)
+                                                                  : part_word(tile0 * p.t_even + i, i % p.t_even == 0, (uint32_t)blk & 1) + 1;
+                                ok = wait_words(in ? p.t_sync + word : nullptr, call, abort_flag) && ok;
+                            }
+                        } else
                         for (int blk = blk0; blk < blk1; ++blk) {
                             const int tile0 = (blk / 2) * p.t_chunks;
                             const uint32_t t_half = (uint32_t)blk & 1;
@@ -873,7 +886,7 @@ prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap t
                                 const unsigned long long* w = nullptr;
                                 left = -first - 32;
                                 for (int c = 0; c < p.t_chunks; ++c) {
-                                    const int q0 = share_owner((tile0 + c) * p.t_stages, t_units, p.t_pairs), q1 = share_owner((tile0 + c + 1) * p.t_stages - 1, t_units, p.t_pairs);
+                                    const int q0 = first_owner(tile0 + c), q1 = last_owner(tile0 + c);
                                     if (i >= 0 && i <= q1 - q0) w = p.t_sync + (q0 == q1 ? tile_word(p.t_pairs, tile0 + c, t_half) : part_word(q0 + i, i == 0, t_half) + 1);
                                     i -= q1 - q0 + 1; left += q1 - q0 + 1;
                                 }
@@ -1097,7 +1110,7 @@ prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap t
             const Run run = run_at(u, t_end, p.t_stages);
             u += run.len;
             if (run.len == p.t_stages) continue;
-            const int q0 = share_owner(run.tile * p.t_stages, t_units, p.t_pairs), q1 = share_owner((run.tile + 1) * p.t_stages - 1, t_units, p.t_pairs);
+            const int q0 = first_owner(run.tile), q1 = last_owner(run.tile);
             const int n = q1 - q0 + 1;
             rows_of(run.tile);
             for (int q = q0; q <= q1; q += 32)
@@ -1134,14 +1147,15 @@ prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap t
                     if (c5 < p.t_n / 4) store4(4 * c5, y[0]);
                 }
             } else {
+                constexpr int kParts = 9;
                 for (int c4 = 2 * (tq - q0) + half; c4 < p.t_n / 4; c4 += 2 * n) {
                     float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-                    for (int qb = q0; qb <= q1; qb += 8) {
-                        float4 v[8];
+                    for (int qb = q0; qb <= q1; qb += kParts) {
+                        float4 v[kParts];
 #pragma unroll
-                        for (int i = 0; i < 8; ++i) v[i] = qb + i <= q1 ? __ldcg(part(qb + i, qb + i == q0) + (size_t)c4 * kPM) : make_float4(0.f, 0.f, 0.f, 0.f);
+                        for (int i = 0; i < kParts; ++i) v[i] = qb + i <= q1 ? __ldcg(part(qb + i, qb + i == q0) + (size_t)c4 * kPM) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-                        for (int i = 0; i < 8; ++i) { s.x += v[i].x; s.y += v[i].y; s.z += v[i].z; s.w += v[i].w; }
+                        for (int i = 0; i < kParts; ++i) { s.x += v[i].x; s.y += v[i].y; s.z += v[i].z; s.w += v[i].w; }
                     }
                     store4(4 * c4, s);
                 }
@@ -1491,6 +1505,7 @@ slim_status_t launch_prefill(const __nv_bfloat16* X, int b, const uint8_t* vals,
             p.t_scale = 1.f / s_eff; p.t_out = Tq;
             p.t_part = reinterpret_cast<float4*>(reinterpret_cast<char*>(Tq) + t_bytes(b, r, t_parts));
             p.t_pairs = t_share(p.t_tiles, p.t_stages, pairs, pairs - grid, s != 0.f ? ceil_div(d_in, 128) : 0);
+            p.t_even = p.t_pairs % p.t_tiles == 0 ? p.t_pairs / p.t_tiles : 0;
             grid = grid + p.t_pairs < pairs ? grid + p.t_pairs : pairs;      // the last pairs make T'
         }
         auto* launch = tile_n > 128 ? launch_pair<256, false>

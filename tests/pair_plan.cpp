@@ -2,6 +2,7 @@
 #include <cstdio>
 #include <initializer_list>
 
+#include "../paper_2410_09615_b200/csrc/handover.h"
 #include "../paper_2410_09615_b200/csrc/pair_plan.h"
 
 using namespace slim;
@@ -37,6 +38,11 @@ int main() {
                         const int stages = d_in / kPairDK, grid = pl.tiles < pairs ? pl.tiles : pairs;
                         const int shares = t_share(pl.t_tiles, stages, pairs, pairs - grid, ceil_div(d_in, 128));
                         if (shares < 1 || shares > pairs || shares > pl.t_tiles * stages) return bad("shares of T'", b, d_out, d_in, r, pairs);
+                        // where the shares divide the tiles, tile t is made by pairs t * parts to t * parts + parts - 1
+                        const int parts = shares % pl.t_tiles == 0 ? shares / pl.t_tiles : 0, units = pl.t_tiles * stages;
+                        for (int t = 0; parts > 0 && t < pl.t_tiles; ++t)
+                            if (share_owner(t * stages, units, shares) != t * parts || share_owner((t + 1) * stages - 1, units, shares) != (t + 1) * parts - 1)
+                                return bad("owners of T'", b, d_out, d_in, r, pairs);
                     }
     printf("ok\n");
     return 0;
