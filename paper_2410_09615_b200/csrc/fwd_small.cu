@@ -6,8 +6,9 @@
 // halves of every unit: a warp keeps the fp32 accumulators of its 64 (32, 16) rows x b tokens in registers
 // through the whole range (from 33 tokens on the two halves are token halves instead), so nothing is
 // summed across warps inside the stream; the partial tiles meet once, at the end: each CTA sends its own, a share of the
-// rows to every CTA of the cluster, by asynchronous remote stores.  C is the largest with which the clusters of all tiles are
-// resident at once (two CTAs per SM up to 16 tokens), so that a tile's stream is spread as widely as it can be.
+// rows to every CTA of the cluster, by asynchronous remote stores.  With 256-row tiles C is the largest with which the clusters of
+// all tiles are resident at once (two CTAs per SM up to 16 tokens), so that a tile's stream is spread as widely as it can be; with
+// lower ones see narrow_tiles.
 //   The first clusters make T = X R^T instead: 32 rows of R each, the same cut of d_in; their
 // CTAs exchange partial sums with asynchronous remote stores, round to bf16 (TP = 2: to two bf16 numbers, keeps_T32) and publish T as
 // 8-byte words {two columns, call number}.
@@ -1121,9 +1122,12 @@ int cluster_size(const int* res, int tiles, int units) {
 // against 12.5), else not (4096 x 4096, rank 208: 9.1 us against 8.3).  With 256-row tiles only: 8192 -> 1024, rank 112, 16
 // tokens 9.3 us instead of 6.6; 5120 x 5120, rank 512, 8 tokens 11.1 instead of 8.6; larger layers are better off with them
 // (28672 -> 8192, 16 tokens 48 us against 65).
-//   Without adapters clusters of two CTAs do where their parts of a row stay short (they start and exchange less), and with them tiles of 128
-// rows fit more layers (16 tokens: 5120 -> 13824 14.8 us with 256 rows, 12.9; 4096 -> 11008 12.2, 11.0; clusters of four against two:
-// 2048 -> 6400 5.8, 5.2, 4096 x 4096 in tiles of 64 rows 6.0, 5.5, 8192 -> 3584 7.7, 8.1).
+//   Without adapters clusters of two CTAs do (they start and exchange less) where rows are short and four would put more than a CTA on every SM.
+// Clusters of four against two, us a call in a graph, weights in the L2 / from the HBM: tiles of 64 rows up to 8 units (1024 -> 4096, 16 tokens
+// 3.07 / 3.08, 2.77 / 2.81; 2048 -> 4096 3.52 / 3.80, 3.37 / 3.72; but 4096 -> 4096, one token 3.89 / 4.75, 4.15 / 4.93; 2048 -> 2048, a CTA an SM
+// either way, 2.62 / 2.65, 2.86 / 2.90), of 128 rows up to 20 (2304 -> 6784, 2 tokens 4.71 / 5.47, 4.11 / 5.06; 3072 -> 8192, one token 4.81 / 5.98,
+// 4.63 / 5.62; 5120 -> 8192 6.05 / 7.63, 6.15 / 7.22).  And with them tiles of 128 rows fit more layers (16 tokens, 256 rows against 128: 5120 ->
+// 13824 13.52 / 14.72, 12.23 / 13.14; 4096 -> 11008 10.69 / 12.20, 10.06 / 11.10; one token 7.64 / 9.16, 7.78 / 8.80).
 void narrow_tiles(int dev, int nt, int fmt, bool qa, int tp, int sm_count, int d_out, int units, int groups, int* mt, int* C) {
     auto fits = [&](int m, int c) {
         const int* res = residency(dev, nt, fmt, qa, m, tp);
@@ -1137,7 +1141,7 @@ void narrow_tiles(int dev, int nt, int fmt, bool qa, int tp, int sm_count, int d
     *mt = fits(1, 2) && (groups == 0 || (!spread && units >= 32)) ? 1 : 2;
     const int widest = 8 * (ceil_div(d_out, 64 * *mt) + groups) <= sm_count ? 8 : 4;
     for (*C = widest; *C > units; *C /= 2) {}
-    if (groups == 0 && *C == 4 && (*mt == 1 ? units <= 24 : units <= 20 && d_out >= 6144)) *C = 2;
+    if (groups == 0 && *C == 4 && (*mt == 1 ? units <= 8 && 4 * ceil_div(d_out, 64) > sm_count : units <= 20 && d_out >= 6144)) *C = 2;
 }
 
 }  // namespace
