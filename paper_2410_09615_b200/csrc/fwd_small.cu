@@ -74,7 +74,7 @@ struct alignas(128) SmallParams {
     float s;
     int b, r, d_out, d_in;
     int units, groups;                                        // of 256 columns, 32 rows of R
-    int ahead;                                                // ask the first lines into the L2 while the grid before ends
+    int ahead;                                                // so many CTAs ask their first lines into the L2 while the grid before ends
 };
 
 // NT tiles of 8 tokens; a warp's MT tiles of 16 rows (four warps: 64 MT rows of the layer).
@@ -488,18 +488,19 @@ __device__ __forceinline__ void finish(const SmallParams& p, uint32_t smem, int 
     }
 }
 
-// Asks the consumers' first lines of a matrix's rows into the L2: bytes [from, to) of `rows` rows, column by column of lines, up to eight
-// lines a thread.
+// Asks bytes [from, to) of `rows` rows from row0 on into the L2, up to eight lines a consumer: ROWS rows side by side, then the next lines
+// of each.  (A line that begins before `from` is asked for with the bytes that it begins with.)
+template <int ROWS>
 __device__ __forceinline__ void lines_ahead(const void* base, size_t pitch, int row0, int rows, size_t from, size_t to)
 {
-    constexpr uint32_t kLine = 128, kMost = 8 * kConsumers;
-    from = from / kLine * kLine;
-    to = to < pitch ? to : pitch;
-    if (from >= to || rows <= 0) return;
-    const uint32_t items = min((uint32_t)(to - from + kLine - 1) / kLine * (uint32_t)rows, kMost);
-    const char* first = static_cast<const char*>(base) + (size_t)row0 * pitch + from;
-    for (uint32_t i = threadIdx.x; i < items; i += kConsumers)
-        asm volatile("prefetch.global.L2 [%0];" :: "l"(first + (size_t)(i % (uint32_t)rows) * pitch + (size_t)(i / (uint32_t)rows) * kLine));
+    constexpr size_t kLine = 128, kBeside = kConsumers / ROWS;
+    const int row = threadIdx.x % ROWS;
+    if (row >= rows) return;
+    const char* at_row = static_cast<const char*>(base) + (size_t)(row0 + row) * pitch;
+    size_t at = (from + (from > 0 ? kLine - 1 : 0)) / kLine * kLine + threadIdx.x / ROWS * kLine;
+#pragma unroll 1
+    for (int i = 0; i < 8 && at < to; ++i, at += kBeside * kLine)
+        asm volatile("prefetch.global.L2 [%0];" :: "l"(at_row + at));
 }
 
 // ---------------------------------------------------------------- the kernel
@@ -556,15 +557,14 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
     if (warp == kProdX && lane == 0) { prefetch_map(&tmX); prefetch_map(&tmM); }
     // The first lines of this CTA's part of the weight or of R go into the L2 meanwhile.  Nothing is read by that: what the grid before still
     // writes is what the loads behind the wait find there.
-    constexpr bool kAsksAhead = NT < 8 && FMT != FMT_TILED && !(QA && MT < 4);      // (see p.ahead: beside int4 adapters only layers of the tall tiles)
-    if (kAsksAhead && p.ahead && warp < kCW) {
+    if (NT <= 2 && FMT != FMT_TILED && !QA && (int)blockIdx.x < p.ahead && warp < kCW) {
+        const size_t c0 = (size_t)u0 * kUnit, c1 = min((size_t)(makes_T ? u1 : u_end) * kUnit, (size_t)p.d_in);
         if (makes_T) {
-            const size_t unit = QA ? kUnit / 2 : kUnit * 2;
-            lines_ahead(p.R, (size_t)p.d_in * unit / kUnit, piece * kGroup, min(kGroup, p.r - piece * kGroup), u0 * unit, u1 * unit);
+            lines_ahead<kGroup>(p.R, (size_t)p.d_in * 2, piece * kGroup, min(kGroup, p.r - piece * kGroup), c0 * 2, c1 * 2);
         } else {
             const int row0 = tile * kRows, rows = min(kRows, p.d_out - row0);
-            lines_ahead(p.vals, (size_t)p.d_in / 4, row0, rows, (size_t)u0 * 64, (size_t)u_end * 64);
-            lines_ahead(p.meta, (size_t)p.d_in / 8, row0, rows, (size_t)u0 * 32, (size_t)u_end * 32);
+            lines_ahead<kRows>(p.vals, (size_t)p.d_in / 4, row0, rows, c0 / 4, c1 / 4);
+            lines_ahead<kRows>(p.meta, (size_t)p.d_in / 8, row0, rows, c0 / 8, c1 / 8);
         }
     }
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -1178,14 +1178,17 @@ slim_status_t launch_small(const __nv_bfloat16* X, int b, const uint8_t* vals, c
     p.departures = reinterpret_cast<unsigned long long*>(ws);
     p.T = reinterpret_cast<unsigned long long*>(reinterpret_cast<char*>(ws) + SLIM_WORKSPACE_SYNC_BYTES);
     p.status = status_dev; p.s = s; p.b = b; p.r = r; p.d_out = d_out; p.d_in = d_in;
-    // Up to 40 MB of weight the HBM is idle for much of a call (start, hand-over of T, exchange): the lines asked for ahead come for nothing
-    // (4096 x 4096, rank 416, one token 8.2 -> 7.7 us a call, 11008 -> 4096, 4 tokens 13.0 -> 12.2; 33 to 64 tokens gain nothing).  Beyond, it is
-    // busy throughout and they come in the way (28672 -> 8192, 16 tokens 49 -> 53).  Where the weight is in the L2 already they cost some
-    // instructions, which shows where a call is short: without adapters they are asked up to 16 MB (5120 -> 6912, one token, from the HBM 7.2 ->
-    // 6.75, from the L2 6.3 -> 6.4; 8192 x 8192 9.8 -> 9.8, 8.6 -> 9.4), beside int4 adapters from 12 MB on (4096 -> 11008, rank 416 12.65 ->
-    // 11.85; 5120 x 5120, rank 512 9.3 -> 9.15, 8.1 -> 8.6).
+    // With adapters the HBM is idle for much of a call (start, hand-over of T, exchange), and the lines asked for ahead come for little: us a call
+    // in a graph, weights in the L2 / from the HBM, without and with them: 4096 x 4096, rank 416, one token 6.82 / 7.92, 6.81 / 7.37; 4096 ->
+    // 11008, rank 416 10.23 / 11.79, 10.38 / 11.14; 3584 -> 8192, rank 368, 4 tokens 10.95 / 12.68, 11.08 / 12.09; over 200 such calls 0.7 % more from
+    // the L2, 3-4 % less from the HBM.  Not where that is not so: without adapters (4096 x 4096, one token 3.83 / 4.75, 4.46 / 4.81; 3072 -> 13824,
+    // 16 tokens 8.14 / 9.44, 8.89 / 9.35), beside int4 adapters (4096 -> 11008, rank 416 10.54 / 12.36, 11.30 / 11.85), from 17 tokens on (8192 x 8192,
+    // rank 832, 25 tokens 23.9, 25.3), under 2 MB of weight, beyond 40 MB (the HBM is busy throughout: 28672 -> 8192, 16 tokens 49, 53), and in CTAs
+    // that find no place at first: those start in the middle of the call (3584 -> 8192 11.08 / 12.09 without them, 12.16 / 12.70).
     const size_t weight = (size_t)d_out * (size_t)d_in * 3 / 8;
-    p.ahead = weight <= (size_t)(r > 0 ? 40 : 16) << 20 && (!qa || (mt == 4 && weight >= (size_t)12 << 20));
+    int log_c = 0;
+    while ((2 << log_c) <= C) ++log_c;
+    p.ahead = r > 0 && !qa && b <= 16 && weight >= (size_t)2 << 20 && weight <= (size_t)40 << 20 ? res[log_c] * C : 0;
     p.units = units; p.groups = groups;
     CUtensorMap tmV, tmM, tmX, tmR, tmL;
     bool ok = make_map3(&tmX, X, (uint64_t)d_in, (uint64_t)b, nt * 8);
