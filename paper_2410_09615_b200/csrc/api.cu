@@ -76,14 +76,16 @@ static bool on_cuda_cores(int b, int d_out, int d_in, int r) {
 // The small-batch kernel's problems: up to 64 tokens, one launch.  From 33 tokens on its warp-level MMAs take longer than the
 // tensor-memory kernel's, which has the advantage once d_out gives it enough tiles: without adapters from 4096 rows on (small against pairs,
 // 33 tokens: 4096 -> 4096 15.4 us, 12.8; 5504 -> 4096 20.5, 15.7; 13824 -> 5120 40.2, 31.0; 8192 -> 3584 16.4, 20.4), with them from 5120 where
-// rows are long enough to hide T' (13824 -> 5120, rank 512 51.0, 41.3; 5120 x 5120 25.7, 24.7; 5504 -> 4096, rank 416 22.7, 24.8; 1728 ->
-// 5120, rank 176 13.6, 18.5), else from 8192.  Rows of few columns are the one-CTA kernel's (launch_prefill) from 17 tokens on:
+// rows are long enough to hide T' (34 tokens: 5504 -> 5120, rank 256 21.6, 20.6; 4096 -> 7168, rank 208 20.4, 17.8; 1728 -> 5120, rank 176 13.6,
+// 18.5), else from 8192.  With 4096 to 5119 columns the two meet where the small kernel's clusters (256 rows, 32 ranks of T) are all there at once,
+// 33 of four CTAs (4096 -> 5120, rank 416, 33 of them 17.6, 18.8; 4160 -> 6160, rank 208, 32 20.7, 22.6; 4096 -> 6160, rank 416, 38 23.5, 21.0).  Rows of few columns are the one-CTA kernel's (launch_prefill) from 17 tokens on:
 // it has no exchange between CTAs at the end (512 -> 4096, 64 tokens, no adapters 6.2 us against 9.2).  The lines, by tokens, adapters
 // and whether rows and tiles come out even, lie where the two meet; int4 adapters, which the others take expanded and rounded to
 // bf16, stay here.
 static bool runs_small(int b, int d_out, int d_in, int r, bool int4 = false) {
     if (!small_supports(b, d_out, d_in, r) || on_cuda_cores(b, d_out, d_in, r)) return false;
-    if (b > 32 && d_out >= (int4 || (r > 0 && d_in < 4096) ? 8192 : r > 0 ? 5120 : 4096)) return false;
+    if (b > 32 && d_out >= (int4 || (r > 0 && d_in < 4096) ? 8192 : r > 0 ? 5120 : 4096) &&
+        (int4 || r == 0 || d_out >= 8192 || d_in >= 5120 || ceil_div(d_out, 256) + ceil_div(r, 32) > 33)) return false;
     if (b <= 16 || int4) return true;
     if (r == 0) return d_in > (b <= 32 ? 320 : d_in % 128 != 0 ? 1536 : 768);
     if (d_in % 128 != 0 || d_out % 128 != 0) return b <= 32 || d_in > 256;

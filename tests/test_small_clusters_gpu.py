@@ -22,7 +22,8 @@ def test_small_batches_without_adapters(d_in, d_out, b):
 
 @pytest.mark.parametrize("d_in,d_out,r,b,kernel", [
     (2048, 4080, 0, 33, K.KERNEL_SMALL), (2048, 4096, 0, 33, K.KERNEL_PREFILL), (2048, 4096, 0, 64, K.KERNEL_PREFILL), (2048, 4096, 0, 32, K.KERNEL_SMALL),
-    (4096, 5104, 32, 40, K.KERNEL_SMALL), (4096, 5120, 32, 64, K.KERNEL_PREFILL), (4032, 5120, 32, 64, K.KERNEL_SMALL),
+    (5120, 5104, 32, 40, K.KERNEL_SMALL), (5120, 5120, 32, 64, K.KERNEL_PREFILL), (4032, 5120, 32, 64, K.KERNEL_SMALL),
+    (4096, 5120, 416, 33, K.KERNEL_SMALL), (4096, 5120, 432, 33, K.KERNEL_PREFILL), (4160, 6160, 256, 64, K.KERNEL_SMALL),
 ])
 def test_lines_from_33_tokens_on(d_in, d_out, r, b, kernel):
     assert K.slim_select_kernel(b, d_out, d_in, r) == kernel
