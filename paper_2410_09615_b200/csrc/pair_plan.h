@@ -20,6 +20,15 @@ inline int t_chunks(int r, int most, int token_tiles, int spare) {
     return ceil_div(r, t_width(r, chunks));      // (widths are multiples of 16: the last of the chunks counted may hold no rank)
 }
 
+// Parts of a T' tile, of up to `parts` that it may have: fewer where they are then added up in fewer rounds of loads (nine parts each) and the longest
+// part grows by no more than two stages.  (us a call before and with this: 3584 -> 8192, rank 352, 600 tokens, twelve parts of up to 5 stages or
+// eight of 7: 43.4, 41.1; rank 720, 300 tokens 34.6, 32.2; 8192 x 8192, rank 816, 40 tokens, ten of 13 or nine of 15: 30.0, 29.3.)
+inline int t_parts(int stages, int parts) {
+    int fewer = parts > 9 && parts <= 12 && ceil_div(stages, 9) <= ceil_div(stages, parts) + 2 ? 9 : parts;
+    fewer = ceil_div(stages, ceil_div(stages, fewer));
+    return ceil_div(fewer, 9) < ceil_div(parts, 9) ? fewer : parts;
+}
+
 // Pairs that share the work of T'.  Each tile in equal parts, one a pair, where that uses four fifths of the pairs or more
 // (a pair then has one part to write, and the pairs that read the same X walk it together); else an even share each.
 // Four stages (a microsecond and a half) or more for a part: below that its start and end dominate.
@@ -28,9 +37,9 @@ inline int t_chunks(int r, int most, int token_tiles, int spare) {
 inline int t_share(int tiles, int stages, int pairs, int spare, int main_stages) {
     const int most = stages < 4 ? 1 : stages / 4;
     int parts = spare / tiles < most ? spare / tiles : most;
-    if (parts >= 1 && (long long)ceil_div(stages, parts) <= main_stages) return tiles * parts;
+    if (parts >= 1 && (long long)ceil_div(stages, parts) <= main_stages) return tiles * t_parts(stages, parts);
     parts = pairs / tiles < most ? pairs / tiles : most;
-    if (parts >= 1 && (parts == most || tiles * parts * 5 >= pairs * 4)) return tiles * parts;
+    if (parts >= 1 && (parts == most || tiles * parts * 5 >= pairs * 4)) return tiles * t_parts(stages, parts);
     return (long long)tiles * most < pairs ? tiles * most : pairs;
 }
 
