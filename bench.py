@@ -12,10 +12,10 @@ through slim_linear_fwd, or the decode-tiled copy through slim_linear_fwd_tiled;
 outside the timed region).
 Every linear has its own copy of weight and adapters; the set is 563 MB, so each call reads its
 operands from HBM (the L2 holds 126 MB).  The step is captured in a CUDA graph and replayed; time
-is taken with CUDA events on the launching stream, max over ranks.  Prints one JSON line, which
-also carries per-case tables for the 7B / 13B / 70B shapes, prefill tables (2048 and 4096 tokens,
-rank sweep on the 70B shapes), an end-to-end figure through the host-buffer entry point and the CPU
-oracle timed on the host's cores.
+is taken with CUDA events on the launching stream, max over ranks.  Prints one JSON line, with
+an end-to-end figure through the host-buffer entry point and the CPU oracle timed on the host's cores;
+per-case tables for the 7B / 13B / 70B shapes and prefill tables (2048 and 4096 tokens, rank sweep on
+the 70B shapes) go to stderr, a JSON line each.
 
 With N > 1 every rank runs the same step on its own GPU (independent replicas, no collective on
 the data path).
@@ -463,7 +463,10 @@ def run_ours(args):
     if rank == 0 and world == 1 and not args.skip_cpu:
         line["cpu_baseline"] = time_cpu_baseline(layers)
     if rank == 0:
-        print(json.dumps(line))
+        short, details = split_details(line)
+        for name, table in details.items():
+            print(json.dumps({name: table}), file=sys.stderr)
+        print(json.dumps(short))
     if world > 1:
         dist.destroy_process_group()
     return 0
@@ -765,6 +768,21 @@ def time_cpu_baseline(layers, repeats=2):
     except Exception as e:
         out["single_thread"] = {"error": str(e)[:100]}
     return out
+
+
+# The tables beside the result, 17 KB of them: a line each on stderr, so that the result line stays short enough to be kept whole
+# wherever output is cut.
+DETAILS = ("per_case", "per_case_batch_sweep", "prefill", "pack", "quantized_adapters", "roofline_prefill")
+
+
+def split_details(line):
+    """(result line, tables) of everything that was measured."""
+    short = {k: v for k, v in line.items() if k not in DETAILS}
+    details = {k: line[k] for k in DETAILS if k in line}
+    if "cpu_baseline" in short:
+        short["cpu_baseline"] = {k: v for k, v in short["cpu_baseline"].items() if k != "single_thread"}
+        details["cpu_baseline"] = line["cpu_baseline"]
+    return short, details
 
 
 def run_single_case(args):
