@@ -793,8 +793,8 @@ prefill_pair_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap t
         *abort_flag = 0u;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == Cfg::kWarpPk && elect_one()) { prefetch_map(&tmV); prefetch_map(&tmM); prefetch_map(&tmA2); }
-    if (warp == Cfg::kWarpX && elect_one()) { prefetch_map(&tmX); prefetch_map(&tmTA); prefetch_map(&tmTB); prefetch_map(&tmB2); }
+    if (warp == Cfg::kWarpPk && elect_one()) { prefetch_map(&tmV); if (!p.meta) prefetch_map(&tmM); if (p.r > 0) prefetch_map(&tmA2); }
+    if (warp == Cfg::kWarpX && elect_one()) { prefetch_map(&tmX); if (p.r > 0) { prefetch_map(&tmTA); prefetch_map(&tmTB); prefetch_map(&tmB2); } }
     cluster_sync_all();                              // both CTAs' barriers exist before anything crosses
     if (warp == Cfg::kWarpMma) {
         asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" :: "r"(s32(tmem_slot)), "r"(512) : "memory");
