@@ -489,7 +489,8 @@ __device__ __forceinline__ void finish(const SmallParams& p, uint32_t smem, int 
 }
 
 // Asks bytes [from, to) of `rows` rows from row0 on into the L2, up to eight lines a consumer: ROWS rows side by side, then the next lines
-// of each.  (A line that begins before `from` is asked for with the bytes that it begins with.)
+// of each.  (Where rows are whole lines, one that begins before `from` is asked for with the bytes that it begins with; where they are not, bytes
+// of two CTAs share lines that neither need see whole, and both ask: 5504 -> 4096, rank 416, 4 tokens 8.95 us, 8.83 so.)
 template <int ROWS>
 __device__ __forceinline__ void lines_ahead(const void* base, size_t pitch, int row0, int rows, size_t from, size_t to)
 {
@@ -497,10 +498,10 @@ __device__ __forceinline__ void lines_ahead(const void* base, size_t pitch, int 
     const int row = threadIdx.x % ROWS;
     if (row >= rows) return;
     const char* at_row = static_cast<const char*>(base) + (size_t)(row0 + row) * pitch;
-    size_t at = (from + (from > 0 ? kLine - 1 : 0)) / kLine * kLine + threadIdx.x / ROWS * kLine;
-#pragma unroll 1
-    for (int i = 0; i < 8 && at < to; ++i, at += kBeside * kLine)
-        asm volatile("prefetch.global.L2 [%0];" :: "l"(at_row + at));
+    size_t at = (from + (from > 0 && pitch % kLine == 0 ? kLine - 1 : 0)) / kLine * kLine + threadIdx.x / ROWS * kLine;
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+        if (at + i * (kBeside * kLine) < to) asm volatile("prefetch.global.L2 [%0];" :: "l"(at_row + at + i * (kBeside * kLine)));
 }
 
 // ---------------------------------------------------------------- the kernel
