@@ -359,8 +359,9 @@ int slim_last_launch_count(void);
 
 /*
  * Token-tile width (64, 128 or 256 tokens) of the variant of the prefill kernel that the last slim_linear_fwd* call on this host
- * thread launched, 0 if that call ran another kernel.  The CTA-pair kernel cuts the tokens evenly into tiles of up to 256, or of 128
- * or 64 where every tile then has a pair of its own and that is faster; the one-CTA kernel's width is 64.  Tests use this query to
+ * thread launched, 0 if that call ran another kernel.  The CTA-pair kernel cuts the tokens evenly into tiles of up to 256 (so up to 128
+ * tokens are one tile of the 128 or 64 variant, however many tiles the rows make), or more finely, into tiles of up to 128 or 64, where every
+ * tile then has a pair of its own and that is faster; the one-CTA kernel's width is 64.  Tests use this query to
  * make sure they exercise the variant they mean to.
  */
 int slim_last_token_tile(void);

@@ -671,10 +671,10 @@ prefill_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap tmV,
 //   - the converters: a group takes 1400 cycles from packed bytes to the arrival, so four groups instead of two;
 //   - the packed ring: 48 KB an SM, less than the HBM's latency asks for: a pair's first tile is asked into the L2 ahead.
 // With up to 128 tokens a stage is a whole packed tile of 256 columns (the smaller accumulator leaves the tensor memory for it): half the
-// barriers and commits a column.  8192 x 8192 without adapters, weights in rotation: 128 tokens 28.5 -> 22.3 us, 333 tokens 32.3 -> 27.8;
+// barriers and commits a column.  8192 x 8192 without adapters, weights in rotation: 128 tokens 28.5 -> 22.4 us, 333 tokens 32.3 -> 28.3;
 // 8192 -> 28672, rank 832, 40 tokens 78 -> 61; 13824 -> 5120, rank 512, 900 tokens 115 -> 110.
 // What bounds it now: with 256 tokens 0.36-0.40 us a stage of 128 columns, of which the MMAs take 0.27 (the shared-memory port is busy for 0.31:
-// TMA writes 38 KB, converters read 6, tensor core reads 32); with 128 tokens 0.25.
+// TMA writes 38 KB, converters read 6, tensor core reads 32); with 128 tokens 0.25.  Whose turn a stage is, and why waits by parity are right: turns.h.
 // A token-tile warp sees every second phase of an `empty` barrier.  Waiting by parity is still right: before its stage g it has waited
 // for the MMAs of stage g - 7, so the phase it did not see (stage g - 10) is over.
 constexpr int kTTok = kPairTTok;        // tokens of a T' tile (the rows of its MMA)

@@ -12,8 +12,8 @@ inline int ceil_div(int a, int b) { return (a + b - 1) / b; }
 // Columns of a T' tile of the pair kernel that cuts r into `chunks`.
 inline int t_width(int r, int chunks) { return r > 0 ? ceil_div(ceil_div(r, chunks), 16) * 16 : 16; }
 // Chunks of r: of up to `most` columns, and as many as leave a tile up to eight of the pairs that have no other work.  (A tile's parts are added up by
-// these pairs, each part of a column asked for by each of them: 4096 -> 11008, rank 416, 256 tokens, two tiles of 15 parts of four stages,
-// the sums took 4 us, of 7 parts 2.)
+// these pairs, each part of a column asked for by each of them.  us a call with as few chunks as can be and so: 4096 -> 11008, rank 416, 256
+// tokens 27.3, 26.5; 8192 -> 1024, rank 112, 512 tokens 25.9, 24.7.)
 inline int t_chunks(int r, int most, int token_tiles, int spare) {
     int chunks = ceil_div(r, most);
     while (spare / (token_tiles * chunks) > 8 && t_width(r, chunks + 1) >= 48) ++chunks;
@@ -59,11 +59,11 @@ inline PairPlan plan_tiles(int b, int d_out, int r, int widest, int pairs) {
     pl.t_tiles = r > 0 ? t_tokens * pl.t_chunks : 0;
     return pl;
 }
-// Tiles of up to 256 tokens, or of 128 or 64 where every tile then has a pair of its own: what takes the least time, in units of 10 ns.  A
-// stage of 128 columns takes 0.40 us with 256 tokens, 0.27 with 128, 0.24 with 64; T' 7 us and 0.28 for each of its stages, on
+// The tokens cut evenly into tiles of up to 256 (so that up to 128 tokens are one narrow tile, however many tiles the rows make), or of up to 128 or 64
+// where every tile then has a pair of its own: what takes the least time, in units of 10 ns.  A stage of 128 columns takes 0.40 us with 256 tokens, 0.27 with 128, 0.24 with 64; T' 7 us and 0.28 for each of its stages, on
 // the pairs without a tile beside the others (of the shorter of the two a quarter counts: they share the L2), else before them.
-// (4096 -> 4096, rank 416, 256 tokens in tiles of 256, 128, 64: 28.7, 24.8, 27.1 us; 5696 -> 1392, rank 288, 1024 tokens 34.9, 36.9, -;
-// 8192 -> 1024, rank 112, 512 tokens 34.8, 26.9, 26.7.)
+// (4096 -> 4096, rank 416, 256 tokens in tiles of 256, 128, 64: 24.6, 22.7, 27.7 us; 5696 -> 1392, rank 288, 1024 tokens 31.1, 32.8, 49.4;
+// 8192 -> 1024, rank 112, 512 tokens 32.8, 26.6, 24.7.)
 inline PairPlan pair_plan(int b, int d_out, int d_in, int r, int pairs) {
     PairPlan best = {};
     long long best_cost = -1;
