@@ -522,7 +522,8 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
     const uint32_t full = bars, empty = bars + 32, piece_bar = bars + 64, red_full = bars + 72, t_full = bars + 80, t_empty = bars + 144, gone = bars + 208;
 
     const int lane = threadIdx.x & 31;
-    const int warp = QA ? threadIdx.x >> 5 : __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0);       // (a shuffle: the same in all lanes, for the compiler too)
+    // (role, a shuffle: the same in all lanes, for the compiler too.  Not so the consumers' warp: see `release`.)
+    const int warp = threadIdx.x >> 5, role = QA ? warp : __shfl_sync(0xffffffffu, warp, 0);
     // The lane that requests.  (Beside int4 adapters the branch on the lane's number, two lanes' requests with one instruction, is the faster one:
     // 5120 x 5120, rank 512, 7 tokens 8.1 us against 8.5, 4096 x 4096, rank 208, 6 tokens 6.5 against 7.1, weights in the L2.)
     auto asks = [&] { return QA ? lane == 0 : elect_one(); };
@@ -554,8 +555,8 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
     cluster_arrive();                                          // waited for before the first access to a peer
     // Launched while the grid before it in the stream still runs (programmatic dependent launch): everything above needs
     // no global memory, everything below comes after that grid.  The next grid may be set up as soon as all CTAs are here.
-    if (warp == kProdW && lane == 0) { prefetch_map(FMT == FMT_TILED ? &tmX : &tmV); prefetch_map(&tmR); prefetch_map(&tmL); }
-    if (warp == kProdX && lane == 0) { prefetch_map(&tmX); prefetch_map(&tmM); }
+    if (role == kProdW && lane == 0) { prefetch_map(FMT == FMT_TILED ? &tmX : &tmV); prefetch_map(&tmR); prefetch_map(&tmL); }
+    if (role == kProdX && lane == 0) { prefetch_map(&tmX); prefetch_map(&tmM); }
     // The first lines of this CTA's part of the weight or of R go into the L2 meanwhile.  Nothing is read by that: what the grid before still
     // writes is what the loads behind the wait find there.
     if (NT <= 2 && FMT != FMT_TILED && !QA && (int)blockIdx.x < p.ahead && warp < kCW) {
@@ -570,7 +571,7 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
     }
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    if (warp == kProdW || warp == kProdX) asm volatile("fence.proxy.async;" ::: "memory");      // what that grid wrote is read through TMA
+    if (role == kProdW || role == kProdX) asm volatile("fence.proxy.async;" ::: "memory");      // what that grid wrote is read through TMA
     bool ok = true;
 
     int p_it = 0;                                              // producers: next stage
@@ -596,7 +597,7 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
         __syncwarp();
         if (lane == 0) mbar_arrive(bar);
     };
-    if (warp == kProdW) {
+    if (role == kProdW) {
         // ============================ the weight, R, L ============================
         const int row0 = tile * kRows;
         if (makes_T) {
@@ -638,7 +639,7 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
             }
         }
         cluster_wait();
-    } else if (warp == kProdX) {
+    } else if (role == kProdX) {
         // ============================ activations, index bytes ============================
         const int row0 = tile * kRows;
         if (makes_T) {
@@ -754,11 +755,17 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
         auto wait_stage = [&]() -> uint32_t {
             const int st = it % kStages;
             ok = mbar_wait(full + 8 * st, (it / kStages) & 1, p.departures) && ok;
+            __syncwarp();                                      // lanes find the phase ended one by one, and what follows takes the whole warp (ldmatrix, mma)
             return smem + st * kStage;
         };
+        // The stage's reads are over before TMA, another proxy, writes it again: an arrival does not say so by itself.  (With addresses that the compiler
+        // knew to be the same in all lanes arrivals overtook ldmatrix: with more steps of L than places in the ring rows came out wrong.)
         auto release = [&]() {
             __syncwarp();
-            if (lane == 0) mbar_arrive(empty + 8 * (it % kStages));
+            if (lane == 0) {
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                mbar_arrive(empty + 8 * (it % kStages));
+            }
             ++it;
         };
         if (makes_T) {
@@ -869,6 +876,7 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
                             const int h = ht / TP, ts = lt % C_::kTSlots;
                             const uint32_t tslot = part + ts * C_::kTSlot;
                             ok = mbar_wait(t_full + 8 * ts, (lt / C_::kTSlots) & 1, p.departures) && ok;
+                            __syncwarp();
                             if (mts > 0 && 2 * lc + h < l_steps) {
                                 uint4 tb[kNW];
 #pragma unroll
@@ -887,6 +895,7 @@ small_kernel(const SmallParams p, const __grid_constant__ CUtensorMap tmV, const
                         const int ls = lc, ts = lt % C_::kTSlots;
                         const uint32_t tslot = part + ts * C_::kTSlot;
                         ok = mbar_wait(t_full + 8 * ts, (lt / C_::kTSlots) & 1, p.departures) && ok;
+                        __syncwarp();
                         if (mts > 0) {
                             const int mat = lane >> 3, r8 = lane & 7;
 #pragma unroll
